@@ -287,3 +287,168 @@ def tolerance(case):
     if k == "heads":
         return {"rel": 5e-4, "max": 5e-3}
     return {"rel": 1e-5, "differ": 2e-3}
+
+
+# ------------------------------------------------------------------------------------------------------- in 64 bits
+def _ridge(R, G, ridge=None):
+    """R (G + rho tr(G)/dim I)^-1."""
+    ridge = RHO * G.diagonal().mean() if ridge is None else ridge
+    L = torch.linalg.cholesky(G + ridge * torch.eye(G.shape[0], dtype=G.dtype, device=G.device))
+    return torch.cholesky_solve(R.T, L).T
+
+
+def _refit(R, G, keep):
+    W = torch.zeros_like(R)
+    W[:, keep] = _ridge(R[:, keep], G[keep][:, keep], RHO * G.diagonal().mean())
+    return W
+
+
+def _top(s, k):
+    return torch.sort(torch.sort(s, descending=True, stable=True).indices[:k]).values
+
+
+def _exact_ffn(c, seed):
+    g, d, n, N, f64 = _gen(seed), c["d"], c["n"], c["N"], torch.float64
+    iters = c["iters"] if c["kind"] == "layer" else 5 if c["select"] else 3
+    if (iters + 1) * N * (2.0 * n * n + 8.0 * n * d) > 2.5e14:
+        return None
+    X = _activations(g, N, d, torch.float32 if c["dtype"] == "f32" else torch.bfloat16, c["out_share"], c["out_factor"],
+                     c["laplace"])
+    W1, W2 = _weight(g, n, d, c["sigma"]), _weight(g, d, n, c["sigma"])
+    Wg = _weight(g, n, d, c["sigma"]).to(f64) if c["act"] == "swiglu" else None
+    fixed = _top(W1.double().square().sum(1) * W2.double().square().sum(0), _keep(c))
+    stored, X, W1, W2 = X.dtype, X.to(f64), W1.to(f64), W2.to(f64)
+    chunks = [slice(t, min(N, t + 16384)) for t in range(0, N, 16384)]
+    Z, U = torch.empty(N, n, dtype=f64, device=DEV), None
+    Y = torch.empty(N, d, dtype=f64, device=DEV)
+    if c["dual"]:
+        U = torch.zeros_like(Z)
+    G_X, out = X.T @ X, {}
+
+    def sums(t, A, first):
+        for name, v in (("G_A", A.T @ A), ("R1", Z[t].T @ X[t]), ("R2", Y[t].T @ A), ("absA", A.abs().sum(0))):
+            out[name] = v if first else out[name].add_(v)
+
+    def phi(t):
+        return Z[t].clamp_min(0) if Wg is None else torch.nn.functional.silu(X[t] @ Wg.T) * Z[t]
+
+    for t in chunks:
+        Z[t] = X[t] @ W1.T
+        A = phi(t)
+        Y[t] = (A @ W2.T).to(stored).to(f64)       # the target is held in the storage type
+        sums(t, A, t.start == 0)
+    for i in range(iters):
+        select = c["select"] and (c["kind"] == "layer" or i == iters - 1)
+        keep = fixed
+        if select:
+            out["scores"] = (_ridge(out["R2"], out["G_A"]).square().sum(0) * out["G_A"].diagonal()).sqrt()
+            out["importance"] = out["scores"].mean().reshape(1)
+            keep = _top(out["scores"], _keep(c))
+        out["W1"] = torch.zeros_like(W1)
+        out["W1"][keep] = _ridge(out["R1"][keep], G_X)
+        out["W2"] = _refit(out["R2"], out["G_A"], keep)
+        w1, w2 = out["W1"], out["W2"]
+        inner = torch.linalg.inv(torch.eye(d, dtype=f64, device=DEV) + w2 @ w2.T) @ w2
+        for t in chunks:
+            h = phi(t) if U is None else phi(t) - U[t]
+            A = h + (Y[t] - h @ w2.T) @ inner
+            Au, z1 = A if U is None else A + U[t], X[t] @ w1.T
+            if Wg is not None:
+                gate = torch.nn.functional.silu(X[t] @ Wg.T)
+                Z[t] = (gate * Au + z1) / (gate * gate + 1)
+            elif c["exact"]:
+                zn, zp = z1.clamp_max(0), ((Au + z1) / 2).clamp_min(0)
+                lower = Au.square() + (zn - z1).square() < (Au - zp).square() + (zp - z1).square()
+                Z[t] = torch.where(lower, zn, zp)
+            else:
+                Z[t] = torch.where(Z[t] < 0, z1, (Au + z1) / 2)
+            if U is not None:
+                U[t] += A - phi(t)
+            sums(t, A, t.start == 0)
+    res = dict(W1=out["W1"], W2=out["W2"], Z=Z, mask=None, G_A=out["G_A"], R1=out["R1"], R2=out["R2"], absA=out["absA"],
+               report=None)
+    if c["kind"] == "layer":
+        res.update(Ypre=Y, G_X=G_X)
+    if c["select"]:
+        res.update(scores=out["scores"], importance=out["importance"])
+    if U is not None:
+        res["U"] = U
+    return res
+
+
+def _exact_heads(c, seed):
+    g, d, H = _gen(seed), c["d"], c["heads"]
+    X = _activations(g, c["N"], d, torch.bfloat16, 0.005, 8.0)
+    W = _weight(g, d, d, 0.02).float()
+    Y, X, W = (X.float() @ W.T).bfloat16().double(), X.double(), W.double()
+    G, R = X.T @ X, Y.T @ X
+    scores = (W.square().sum(0) * G.diagonal()).view(H, -1).sum(1).sqrt()
+    dh = d // H
+    keep = (_top(scores, c["keep_heads"])[:, None] * dh + torch.arange(dh, device=DEV)).flatten()
+    return dict(mask=None, W=_refit(R, G, keep), scores=scores)
+
+
+def _exact_mha(c, seed):
+    g, d, H, T, S = _gen(seed), c["d"], c["heads"], c["T"], c["seqs"]
+    dh = d // H
+    X = _activations(g, S * T, d, torch.bfloat16, 0.005, 5.0).double()
+    Wq, Wk, Wv, Wo = (_weight(g, d, d, 1.0 / math.sqrt(d)).double() for _ in range(4))
+    kept = torch.sort(torch.randperm(H, generator=g, device=DEV)[:c["keep_heads"]]).values
+    keep = (kept[:, None] * dh + torch.arange(dh, device=DEV)).flatten()
+    future = torch.ones(T, T, dtype=torch.bool, device=DEV).triu(1)
+
+    def heads(v):                                  # [S T, d] -> [S, H, T, dh]
+        return v.view(S, T, H, dh).transpose(1, 2)
+
+    def flat(v):
+        return v.transpose(1, 2).reshape(S * T, d)
+
+    def probs(zq, zk):
+        return (heads(zq) @ heads(zk).transpose(2, 3) / math.sqrt(dh)).masked_fill(future, float("-inf")).softmax(3)
+
+    def rows(w):
+        out = torch.zeros_like(w)
+        out[keep] = w[keep]
+        return out
+
+    zq, zk, v = X @ Wq.T, X @ Wk.T, X @ Wv.T
+    P = probs(zq, zk)
+    A = flat(P @ heads(v))
+    Y = (A @ Wo.T).bfloat16().double()
+    G_X = X.T @ X
+    Wq, Wk, Wo = rows(_ridge(zq.T @ X, G_X)), rows(_ridge(zk.T @ X, G_X)), _refit(Y.T @ A, A.T @ A, keep)
+    Wv = torch.zeros_like(Wv)
+    for h in kept.tolist():
+        r, cols = (P[:, h] @ X.view(S, T, d)).reshape(S * T, d), slice(h * dh, (h + 1) * dh)
+        Wv[cols] = _ridge(A[:, cols].T @ r, r.T @ r)
+    v, target_q, target_k, F = X @ Wv.T, X @ Wq.T, X @ Wk.T, probs(zq, zk)
+    step = 1.0 / (2.0 * (heads(v).square().sum((2, 3), keepdim=True) + 1.0))
+    for _ in range(c["a_steps"]):
+        P = P - step * (2.0 * (P @ heads(v) - heads(A)) @ heads(v).transpose(2, 3) + 2.0 * (P - F))
+    A = (flat(P @ heads(v)) + Y @ Wo) @ torch.linalg.inv(Wo.T @ Wo + torch.eye(d, dtype=X.dtype, device=DEV))
+    for _ in range(c["z_steps"]):
+        F = probs(zq, zk)
+        E = F - P
+        dS = 2.0 * F * (E - (E * F).sum(3, keepdim=True)) / math.sqrt(dh)
+        q, k = heads(zq), heads(zk)
+        eta = 1.0 / (2.0 + (q.square().sum((2, 3), keepdim=True) + k.square().sum((2, 3), keepdim=True)) / dh)
+        zq, zk = (flat(q - eta * (dS @ k + 2.0 * (q - heads(target_q)))),
+                  flat(k - eta * (dS.transpose(2, 3) @ q + 2.0 * (k - heads(target_k)))))
+    return dict(Wq=Wq, Wk=Wk, Wv=Wv, Wo=Wo, Zq=zq, Zk=zk, P=P, Aattn=A, R_Q=zq.T @ X, R_K=zk.T @ X, G_attn=A.T @ A,
+                R_O=Y.T @ A)
+
+
+def exact(case, seed):
+    """What run() returns for these inputs, in 64 bits throughout (integer and report outputs left out)."""
+    kind = case["kind"]
+    if kind != "plan":
+        return {"heads": _exact_heads, "mha": _exact_mha}.get(kind, _exact_ffn)(case, seed)
+    g, L, d, n = _gen(seed), case["layers"], case["d"], case["n"]
+    sq = torch.stack([(_weight(g, d, n, 0.02).float() * (1.0 + 0.03 * l)).double().square().sum(0) for l in range(L)])
+    scores = (sq * (torch.rand(L, n, generator=g, device=DEV) + 0.5)).sqrt()
+    I = scores.mean(1)
+    raw = (1.0 - case["keep"]) * L * torch.softmax(-I / I.abs().mean(), 0)
+    r = raw.clamp(0, 0.95)
+    if not bool((raw > 0.95).any()):
+        r = (r * ((1.0 - case["keep"]) / r.mean())).clamp(0, 0.95)
+    return dict(importance=I, r=r[None], k_keep=None, scores=scores, mask=None, tau=None)
