@@ -101,9 +101,10 @@ struct OutOperand {
 
 // C[M,N] (row-major) = alpha * sum_k A(i,k) B(k,j) + beta * Cin[i,j].  Cin may alias C or be another matrix of
 // another dtype; beta == 0 never reads Cin.  lower_only skips tiles that lie strictly above the diagonal.
-// acc64: accumulate in fp64 (else fp32).
+// acc64: accumulate in fp64 (else fp32).  k_tri: A(i, k) = 0 for k < i and B(k, j) = 0 for k < j, so that a tile may
+// start its sum there (honoured where it pays; the stored zeros are read otherwise).
 cudaError_t gemm_simt(int64_t M, int64_t N, int64_t K, double alpha, Operand A, Operand B, double beta,
-                      Operand Cin, OutOperand C, bool lower_only, bool acc64, cudaStream_t stream);
+                      Operand Cin, OutOperand C, bool lower_only, bool acc64, cudaStream_t stream, bool k_tri = false);
 
 // tcgen05 path: bf16 operands, fp32 accumulation in tensor memory.
 //   a_kmajor: A is stored [M, K] row-major (K contiguous) ; else [K, M] row-major (M contiguous).
@@ -147,18 +148,18 @@ sp_status gemm_tc(int64_t M, int64_t N, int64_t K, float alpha, TcOperand A, TcO
                   const TcBatch* batch = nullptr);
 bool gemm_tc_supported(int64_t M, int64_t N, int64_t K, TcOperand A, TcOperand B);
 
-// Dense symmetric positive definite solve in precision T (float or double), all on `stream`.
-//   potrf: in-place lower Cholesky of the n x n matrix A (ld lda); the strict upper triangle is not referenced.
-//   inv diag blocks are kept in `dinv` (n x NB row-major slabs) for the triangular solves.
-struct CholWork {
-  void* dinv;  // [ceil(n/NB) * NB * NB] elements of T
-};
-template <typename T>
-cudaError_t potrf_lower(T* A, int64_t n, int64_t lda, T* dinv, int32_t* status_dev, cudaStream_t stream);
-// X[m,n] <- X L^-T L^-1 (right solves with the factor of potrf_lower), i.e. X (L L^T)^-1.
-template <typename T>
-cudaError_t potrs_right(T* X, int64_t m, int64_t n, int64_t ldx, const T* L, int64_t ldl, const T* dinv,
-                        cudaStream_t stream);
+struct SolveAssist;
+// fp64 factorisation and solves (sp_linalg.cu), block columns of kCholNB.
+//   potrf_lower_f64: in-place lower Cholesky of the n x n matrix A (ld lda); the strict upper triangle and the diagonal
+//   blocks of the factor are not written; dinv: ceil(n / kCholNB) inverse diagonal blocks [kCholNB, kCholNB].
+//   m_extra > 0: A has m_extra more rows below row n, right-hand sides B of X L^T = B that ride along and hold X on
+//   return.  extra_is_identity: B is the identity (m_extra == n), so that X is upper triangular and a step touches
+//   only the rows that are no longer zero.
+cudaError_t potrf_lower_f64(double* A, int64_t n, int64_t lda, double* dinv, int32_t* status_dev, cudaStream_t stream,
+                            const SolveAssist* assist, int64_t m_extra, bool extra_is_identity = false);
+// X[m,n] <- X L^-1 (backward sweep with the factor of potrf_lower_f64).
+cudaError_t potrs_backward_f64(double* X, int64_t m, int64_t n, int64_t ldx, const double* L, int64_t ldl,
+                               const double* dinv, cudaStream_t stream, const SolveAssist* assist);
 constexpr int kCholNB = 64;
 
 // fp32 factorisation / solves with tensor-core trailing updates (sp_linalg_tc.cu).  Panels are kCholTcNB wide.
@@ -343,7 +344,8 @@ cudaError_t mha_z_update(float* Zq, float* Zk, const float* Gq, const float* Gk,
                          const float* eta, int64_t tokens, int d, int T, int d_h, double alpha, void* Zqs, void* Zks,
                          int64_t plane, cudaStream_t stream);
 // A[n, n] (ld) = identity
-cudaError_t set_identity(float* A, int64_t n, int64_t ld, cudaStream_t stream);
+template <typename T>
+cudaError_t set_identity(T* A, int64_t n, int64_t ld, cudaStream_t stream);
 // dst[e] = bf16(x[e]), dst[plane + e] = bf16(x[e] - hi) (plane == 0: hi only)
 cudaError_t split_planes(const float* x, int64_t total, void* dst, int64_t plane, cudaStream_t stream);
 

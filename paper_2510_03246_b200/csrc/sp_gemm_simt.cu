@@ -1,6 +1,8 @@
-// Strided CUDA-core GEMM: the fp32-mode contraction kernel (fp32 storage, fp64 accumulation) and the workhorse of
-// the blocked Cholesky / triangular solves.  Operand element types are chosen at run time; the accumulator type and
-// the tile shape are compile-time.
+// GEMMs outside the bf16 tensor-core path.
+//   gemm_dmma_kernel: fp64 accumulation of two fp32 or two fp64 operands on the fp64 matrix instruction; the fp32-mode
+//                     contraction kernel and the workhorse of the blocked fp64 Cholesky / triangular solves.
+//   gemm_simt_kernel: strided CUDA-core form for everything else (bf16 or mixed operands, two non-unit strides, fp32
+//                     accumulation).  Operand element types are chosen at run time.
 #include "sp_common.cuh"
 
 namespace sp {
@@ -123,14 +125,212 @@ gemm_simt_kernel(int64_t M, int64_t N, int64_t K, Acc alpha, Operand A, Operand 
   }
 }
 
+
+// ---- fp64 accumulation on the fp64 matrix instruction (tcgen05 has no fp64 kind, so this is mma.sync)
+//
+// A 64 x 64 (or 32 x 64) tile per block of four warps, each 32 x 32 (16 x 32): per 8 values of K a warp issues eight
+// m16n8k8 instructions on fragments of 16 eight-byte shared-memory reads, so the fp64 pipe (64 fused multiply-adds per
+// SM and cycle) is the bound and not shared memory, as it was for the scalar kernel (16 fused multiply-adds per 8 reads and a
+// conversion of every element on its way in).  Operands stay in their stored orientation in shared memory; a pitch of 4
+// doubles beyond a multiple of 16 makes every fragment read conflict-free in both orientations.  The next K slab travels
+// through registers (16-byte loads, fp32 widened there) while the current one is multiplied; small blocks let three
+// of them share an SM, which hides the prologue and the read-modify-write of C in the K = 64 updates of the factorisation.
+// Measured: token contractions of fp32 operands (3072 x 3072 lower, K = 2048) 29 TFLOP/s; the scalar kernel made 12.
+constexpr int DM_BN = 64, DM_BK = 16, DM_THREADS = 128, DM_PAD = 4;
+
+__device__ __forceinline__ void dmma_16x8x8(double (&d)[4], const double (&a)[4], const double (&b)[2]) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k8.row.col.f64.f64.f64.f64 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+      : "+d"(d[0]), "+d"(d[1]), "+d"(d[2]), "+d"(d[3])
+      : "d"(a[0]), "d"(a[1]), "d"(a[2]), "d"(a[3]), "d"(b[0]), "d"(b[1]));
+}
+
+// One DIM x DM_BK slab of an operand: rows of FAST contiguous elements (K when KFAST, else the M / N index).
+template <typename T, bool KFAST, int DIM>
+struct DmmaSlab {
+  static constexpr int V = 16 / sizeof(T);
+  static constexpr int FAST = KFAST ? DM_BK : DIM, OUTER = KFAST ? DIM : DM_BK;
+  static constexpr int PITCH = FAST + DM_PAD, VPR = FAST / V, CNT = OUTER * VPR / DM_THREADS;
+  static constexpr int ELEMS = OUTER * PITCH;
+  static_assert(OUTER * VPR % DM_THREADS == 0, "slab / thread mismatch");
+  T r[CNT][V];
+
+  // d0: first index of the tile along M / N, k0: first K index, dim / kend: extents
+  __device__ __forceinline__ void fetch(const T* p, int64_t ld, bool vec, int64_t d0, int64_t k0, int64_t dim,
+                                        int64_t kend) {
+    const int64_t o0 = KFAST ? d0 : k0, f0 = KFAST ? k0 : d0, olim = KFAST ? dim : kend, flim = KFAST ? kend : dim;
+#pragma unroll
+    for (int q = 0; q < CNT; ++q) {
+      const int e = (int)threadIdx.x + q * DM_THREADS;
+      const int64_t o = o0 + e / VPR, f = f0 + (e % VPR) * V;
+      const T* src = p + o * ld + f;
+      if (vec && o < olim && f + V <= flim) {
+        *reinterpret_cast<int4*>(r[q]) = *reinterpret_cast<const int4*>(src);
+      } else {
+#pragma unroll
+        for (int v = 0; v < V; ++v) r[q][v] = (o < olim && f + v < flim) ? src[v] : (T)0;
+      }
+    }
+  }
+  __device__ __forceinline__ void store(double* sm) const {
+#pragma unroll
+    for (int q = 0; q < CNT; ++q) {
+      const int e = (int)threadIdx.x + q * DM_THREADS;
+      double* dst = sm + (e / VPR) * PITCH + (e % VPR) * V;
+#pragma unroll
+      for (int v = 0; v < V; v += 2) *reinterpret_cast<double2*>(dst + v) = make_double2((double)r[q][v], (double)r[q][v + 1]);
+    }
+  }
+  static __device__ __forceinline__ double at(const double* sm, int dim, int k) {
+    return KFAST ? sm[dim * PITCH + k] : sm[k * PITCH + dim];
+  }
+};
+
+template <typename T, bool A_KFAST, bool B_KFAST, int BM>
+__global__ void __launch_bounds__(DM_THREADS, 3)
+gemm_dmma_kernel(int64_t M, int64_t N, int64_t K, double alpha, const T* A, int64_t lda,
+                 const T* B, int64_t ldb, double beta, Operand Cin, OutOperand C, int lower_only, int k_tri) {
+  using SlabA = DmmaSlab<T, A_KFAST, BM>;
+  using SlabB = DmmaSlab<T, B_KFAST, DM_BN>;
+  constexpr int WM = BM / 2, MT = WM / 16;      // rows of a warp, its 16-row tiles
+  const int64_t row0 = (int64_t)blockIdx.y * BM, col0 = (int64_t)blockIdx.x * DM_BN;
+  if (lower_only && row0 + BM - 1 < col0) return;
+  __shared__ __align__(16) double sa[2][SlabA::ELEMS];
+  __shared__ __align__(16) double sb[2][SlabB::ELEMS];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int g = lane >> 2, t = lane & 3;
+  const int wm = (warp & 1) * WM, wn = (warp >> 1) * 32;
+  constexpr int V = 16 / sizeof(T);
+  const bool va = lda % V == 0 && (reinterpret_cast<uintptr_t>(A) & 15u) == 0;
+  const bool vb = ldb % V == 0 && (reinterpret_cast<uintptr_t>(B) & 15u) == 0;
+
+  double acc[MT][4][4];
+#pragma unroll
+  for (int i = 0; i < MT; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[i][j][q] = 0.0;
+
+  // k_tri: both operands are zero for K indices below their own M / N index (upper-triangular rows)
+  int64_t k0 = 0;
+  if (k_tri) k0 = (row0 > col0 ? row0 : col0) / DM_BK * DM_BK;
+  SlabA fa;
+  SlabB fb;
+  fa.fetch(A, lda, va, row0, k0, M, K);
+  fb.fetch(B, ldb, vb, col0, k0, N, K);
+  fa.store(sa[0]);
+  fb.store(sb[0]);
+  __syncthreads();
+  for (int buf = 0; k0 < K; k0 += DM_BK, buf ^= 1) {
+    const bool more = k0 + DM_BK < K;
+    if (more) {
+      fa.fetch(A, lda, va, row0, k0 + DM_BK, M, K);
+      fb.fetch(B, ldb, vb, col0, k0 + DM_BK, N, K);
+    }
+#pragma unroll
+    for (int kk = 0; kk < DM_BK; kk += 8) {
+      double a[MT][4], b[4][2];
+#pragma unroll
+      for (int i = 0; i < MT; ++i) {
+        const int m = wm + 16 * i + g;
+        a[i][0] = SlabA::at(sa[buf], m, kk + t);
+        a[i][1] = SlabA::at(sa[buf], m + 8, kk + t);
+        a[i][2] = SlabA::at(sa[buf], m, kk + t + 4);
+        a[i][3] = SlabA::at(sa[buf], m + 8, kk + t + 4);
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        b[j][0] = SlabB::at(sb[buf], wn + 8 * j + g, kk + t);
+        b[j][1] = SlabB::at(sb[buf], wn + 8 * j + g, kk + t + 4);
+      }
+#pragma unroll
+      for (int i = 0; i < MT; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) dmma_16x8x8(acc[i][j], a[i], b[j]);
+    }
+    if (more) {      // the other buffer was last read before the previous barrier
+      fa.store(sa[buf ^ 1]);
+      fb.store(sb[buf ^ 1]);
+      __syncthreads();
+    }
+  }
+
+  // a thread holds columns 2t, 2t + 1 of rows g and g + 8 of every 16 x 8 tile
+  const bool c64 = C.dtype == SP_F64;
+  const bool vc = C.ld % 2 == 0 && (reinterpret_cast<uintptr_t>(C.ptr) & (c64 ? 15u : 7u)) == 0;
+#pragma unroll
+  for (int i = 0; i < MT; ++i)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int64_t gi = row0 + wm + 16 * i + 8 * h + g;
+      if (gi >= M) continue;
+      double v[4][2];
+      if (beta != 0.0) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            const int64_t gj = col0 + wn + 8 * j + 2 * t + q;
+            v[j][q] = gj < N ? load_elem<double>(Cin.ptr, Cin.dtype, gi * Cin.s0 + gj * Cin.s1) : 0.0;
+          }
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int64_t gj = col0 + wn + 8 * j + 2 * t;
+        double o[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          o[q] = alpha * acc[i][j][2 * h + q];
+          if (beta != 0.0) o[q] += beta * v[j][q];
+        }
+        if (vc && gj + 2 <= N && C.dtype != SP_BF16) {
+          if (c64) *reinterpret_cast<double2*>(reinterpret_cast<double*>(C.ptr) + gi * C.ld + gj) = make_double2(o[0], o[1]);
+          else *reinterpret_cast<float2*>(reinterpret_cast<float*>(C.ptr) + gi * C.ld + gj) = make_float2((float)o[0], (float)o[1]);
+        } else {
+#pragma unroll
+          for (int q = 0; q < 2; ++q)
+            if (gj + q < N) store_elem<double>(C.ptr, C.dtype, gi * C.ld + gj + q, o[q]);
+        }
+      }
+    }
+}
+
+template <typename T, int BM>
+void launch_dmma(int64_t M, int64_t N, int64_t K, double alpha, const Operand& A, const Operand& B, double beta,
+                 const Operand& Cin, const OutOperand& C, bool lower_only, bool k_tri, cudaStream_t stream) {
+  const dim3 grid((unsigned)ceil_div(N, DM_BN), (unsigned)ceil_div(M, BM));
+  const bool ak = A.s1 == 1, bk = B.s0 == 1;
+  const int64_t lda = ak ? A.s0 : A.s1, ldb = bk ? B.s1 : B.s0;
+  const T* a = reinterpret_cast<const T*>(A.ptr);
+  const T* b = reinterpret_cast<const T*>(B.ptr);
+  const int lo = lower_only ? 1 : 0, tri = k_tri ? 1 : 0;
+  if (ak && bk) gemm_dmma_kernel<T, true, true, BM><<<grid, DM_THREADS, 0, stream>>>(M, N, K, alpha, a, lda, b, ldb, beta, Cin, C, lo, tri);
+  else if (ak) gemm_dmma_kernel<T, true, false, BM><<<grid, DM_THREADS, 0, stream>>>(M, N, K, alpha, a, lda, b, ldb, beta, Cin, C, lo, tri);
+  else if (bk) gemm_dmma_kernel<T, false, true, BM><<<grid, DM_THREADS, 0, stream>>>(M, N, K, alpha, a, lda, b, ldb, beta, Cin, C, lo, tri);
+  else gemm_dmma_kernel<T, false, false, BM><<<grid, DM_THREADS, 0, stream>>>(M, N, K, alpha, a, lda, b, ldb, beta, Cin, C, lo, tri);
+}
+
 }  // namespace
 
 cudaError_t gemm_simt(int64_t M, int64_t N, int64_t K, double alpha, Operand A, Operand B, double beta, Operand Cin,
-                      OutOperand C, bool lower_only, bool acc64, cudaStream_t stream) {
+                      OutOperand C, bool lower_only, bool acc64, cudaStream_t stream, bool k_tri) {
   if (M <= 0 || N <= 0) return cudaSuccess;
   count_launch();
   ProfScope prof(PK_GEMM_SIMT, (lower_only ? 1.0 : 2.0) * (double)M * (double)N * (double)K, 0.0, stream);
-  if (acc64) {
+  const bool dmma = acc64 && A.dtype == B.dtype && (A.dtype == SP_F32 || A.dtype == SP_F64) &&
+                    (A.s0 == 1 || A.s1 == 1) && (B.s0 == 1 || B.s1 == 1) && K > 0;
+  if (dmma) {
+    // 32-row tiles while 64-row ones would leave SMs idle (the block columns of a solve: one tile wide)
+    const bool small = ceil_div(M, 64) * ceil_div(N, (int64_t)DM_BN) < sm_count();
+    if (A.dtype == SP_F64) {
+      if (small) launch_dmma<double, 32>(M, N, K, alpha, A, B, beta, Cin, C, lower_only, k_tri, stream);
+      else launch_dmma<double, 64>(M, N, K, alpha, A, B, beta, Cin, C, lower_only, k_tri, stream);
+    } else {
+      if (small) launch_dmma<float, 32>(M, N, K, alpha, A, B, beta, Cin, C, lower_only, k_tri, stream);
+      else launch_dmma<float, 64>(M, N, K, alpha, A, B, beta, Cin, C, lower_only, k_tri, stream);
+    }
+  } else if (acc64) {
     constexpr int BM = 64, BN = 64;
     dim3 grid((unsigned)ceil_div(N, BN), (unsigned)ceil_div(M, BM));
     gemm_simt_kernel<double, BM, BN, 4, 4><<<grid, 256, 0, stream>>>(M, N, K, alpha, A, B, beta, Cin, C,

@@ -183,7 +183,8 @@ __global__ void __launch_bounds__(256) split_planes_kernel(const float* __restri
   }
 }
 
-__global__ void set_identity_kernel(float* A, int64_t n, int64_t ld) {
+template <typename T>
+__global__ void set_identity_kernel(T* A, int64_t n, int64_t ld) {
   const int64_t total = n * n;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = e / n, j = e % n;
@@ -258,12 +259,15 @@ cudaError_t mha_z_update(float* Zq, float* Zk, const float* Gq, const float* Gk,
   return cudaGetLastError();
 }
 
-cudaError_t set_identity(float* A, int64_t n, int64_t ld, cudaStream_t stream) {
+template <typename T>
+cudaError_t set_identity(T* A, int64_t n, int64_t ld, cudaStream_t stream) {
   if (n == 0) return cudaSuccess;
   count_launch();
   set_identity_kernel<<<grid_1d(n * n, 256), 256, 0, stream>>>(A, n, ld);
   return cudaGetLastError();
 }
+template cudaError_t set_identity<float>(float*, int64_t, int64_t, cudaStream_t);
+template cudaError_t set_identity<double>(double*, int64_t, int64_t, cudaStream_t);
 
 cudaError_t split_planes(const float* x, int64_t total, void* dst, int64_t plane, cudaStream_t stream) {
   if (total == 0) return cudaSuccess;

@@ -1,0 +1,77 @@
+"""The fp64 contraction kernel and the fp64 factorisation / solves at the edges of their tiles (64 x 64 and 32 x 64 tiles,
+K slabs of 16, block columns of 64), against plain fp64 torch."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+def _api():
+    from paper_2510_03246_b200 import api
+    return api
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+@pytest.mark.parametrize("transA", [False, True])
+@pytest.mark.parametrize("transB", [False, True])
+@pytest.mark.parametrize("M,N,K,pad", [(1, 1, 1, 0), (33, 65, 17, 1), (64, 64, 16, 0), (130, 70, 250, 3), (1027, 769, 131, 2),
+                                       (2048, 832, 64, 4)])
+def test_gemm_fp64_accumulation(dtype, transA, transB, M, N, K, pad):
+    """Every stored orientation, aligned and unaligned pitches, accumulation into C and the lower triangle alone."""
+    api = _api()
+    g = torch.Generator(device="cuda").manual_seed(M + 7 * N + 13 * K)
+
+    def stored(r, c):
+        buf = torch.randn(r, c + pad, generator=g, device="cuda", dtype=torch.float64).to(dtype)
+        return buf[:, :c]
+
+    A, B = stored(*((K, M) if transA else (M, K))), stored(*((N, K) if transB else (K, N)))
+    C0 = stored(M, N)
+    a, b = (A.T if transA else A).double(), (B.T if transB else B).double()
+    want = 0.75 * (a @ b) - 0.5 * C0.double()
+    # one rounding to the stored type, and K + 2 roundings of the fp64 sum on either side
+    unit = 2.0 ** -24 if dtype == torch.float32 else 2.0 ** -53
+    bound = unit * want.abs() + 2 * (K + 4) * 2.0 ** -53 * (a.abs() @ b.abs() + C0.double().abs())
+    got = C0.clone()
+    api.sp_gemm(A, B, got, transA, transB, alpha=0.75, beta=-0.5)
+    assert bool(((got.double() - want).abs() <= bound).all())
+    low = C0.clone()
+    api.sp_gemm(A, B, low, transA, transB, alpha=0.75, beta=-0.5, lower_only=True)
+    tri = torch.ones(M, N, device="cuda", dtype=torch.bool).tril()
+    assert torch.equal(low[tri], got[tri])
+
+
+def _spd(n, seed):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    X = torch.randn(2 * n + 3, n, generator=g, device="cuda") * torch.logspace(0, 1.5, n, device="cuda")
+    G = (X.T @ X).float()
+    return torch.tril(G) + torch.tril(G, -1).T
+
+
+@pytest.mark.parametrize("n,m", [(1, 1), (3, 70), (63, 5), (64, 64), (65, 33), (127, 129), (200, 1), (321, 500), (1030, 259)])
+def test_precise_ridge_solve_at_block_edges(n, m):
+    api = _api()
+    G = _spd(n, n)
+    R = torch.randn(m, n, generator=torch.Generator(device="cuda").manual_seed(m), device="cuda")
+    got = api.sp_ridge_solve(R, G, 0.01, True, precise=True)
+    H = G.double() + 0.01 * G.double().diagonal().mean() * torch.eye(n, device="cuda", dtype=torch.float64)
+    want = torch.linalg.solve(H, R.double().T).T
+    # fp64 throughout (condition number below 1e5: 1e-10 of the largest entry), stored as fp32 (2^-24)
+    assert float((got.double() - want).abs().max() / want.abs().max()) < 1.2e-7
+    again = api.sp_ridge_solve(R, G, 0.01, True, precise=True)
+    assert torch.equal(got, again)      # no result depends on the order of the two streams
+
+
+@pytest.mark.parametrize("d", [8, 64, 72, 136, 520, 1096])
+def test_cached_input_inverse_at_block_edges(d):
+    api = _api()
+    g = torch.Generator(device="cuda").manual_seed(d)
+    X = torch.randn(2 * d, d, generator=g, device="cuda").bfloat16()
+    mod = api.FfnModule(X, torch.randn(16, d, generator=g, device="cuda"), torch.randn(d, 16, generator=g, device="cuda"))
+    mod.sp_ffn_init()
+    mod.sp_ffn_cache_input_inverse(0.1)
+    G = mod.G_X.double()
+    want = torch.linalg.inv(G + 0.1 * G.diagonal().mean() * torch.eye(d, device="cuda", dtype=torch.float64))
+    assert float((mod.G_X_inv.double() - want).abs().max() / want.abs().max()) < 1.2e-7
+    assert torch.equal(mod.G_X_inv, mod.G_X_inv.T)
+    mod.check_status()
