@@ -1,0 +1,237 @@
+// Factorisation of one NB x NB diagonal block by one thread block, and the inverse of its factor: the serial link of the
+// blocked Cholesky factorisations (fp32: NB = 128, fp64: NB = 64).
+#pragma once
+#include "sp_common.cuh"
+
+namespace sp {
+
+// 1 / sqrt(x) to about 1 ulp, x > 0: hardware approximation and a step of Newton's iteration (fp32) or of the third-order
+// iteration y (1 + e / 2 + 3 e^2 / 8), e = 1 - x y^2 (fp64: the approximation's 20 bits become 58).  No branches, so that
+// the steps of consecutive columns interleave.
+__device__ __forceinline__ float rsqrt_refined(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r * fmaf(-0.5f * x, r * r, 1.5f);
+}
+__device__ __forceinline__ double rsqrt_refined(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x * y, y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
+// acc += a b on pairs of neighbouring values (fp32: one packed instruction)
+__device__ __forceinline__ void fma_pair(float2& acc, const float* a, const float* b) {
+  asm("{\n\t.reg .b64 a, b, c;\n\t"
+      "mov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tmov.b64 c, {%0, %1};\n\t"
+      "fma.rn.f32x2 c, a, b, c;\n\tmov.b64 {%0, %1}, c;\n\t}"
+      : "+f"(acc.x), "+f"(acc.y)
+      : "f"(a[0]), "f"(a[1]), "f"(b[0]), "f"(b[1]));
+}
+__device__ __forceinline__ void fma_pair(double& acc, const double* a, const double* b) {
+  acc = fma(a[0], b[0], acc);
+  acc = fma(a[1], b[1], acc);
+}
+__device__ __forceinline__ float pair_sum(const float2& v) { return v.x + v.y; }
+__device__ __forceinline__ double pair_sum(double v) { return v; }
+template <typename T> struct PairAcc { using type = double; };
+template <> struct PairAcc<float> { using type = float2; };
+
+// The block is eliminated in sub-blocks of 32 columns.  Rows to carry along are the rows of the matrix below the
+// sub-block and the rows of an identity appended under the matrix (X L^T = I, so X = L^-T): together always NB rows.  Per sub-block
+//   A  one warp factorises the 32 x 32 diagonal sub-block, one row per lane, columns handed round by shuffles;
+//   B  one thread per row solves x L11^T = row for its 32 entries (L11 read as broadcasts);
+//   C  the columns to the right receive the rank-32 update in 32 x 32 pieces, one warp each.  The next diagonal
+//      sub-block comes first, by all warps; the other pieces run beside the next phase A.
+// What bounds it is latency: A (about 120 cycles per column: shuffle, reciprocal root, product, update), B and the first
+// piece of C; for 128 columns the other pieces take as long as A.  Measured inside a factorisation: 25 us for 128 columns
+// in fp32, 14 us for 64 in fp64.  The form before this one eliminated four columns per step in registers of one thread
+// per 4 x 4 block; two block barriers and all warps' shared update stood between a pivot and the next (37 and 20 us).
+template <typename T, int NB>
+struct DiagBlock {
+  static constexpr int SB = 32, NS = NB / SB;
+  static constexpr int V = 16 / (int)sizeof(T);              // elements per 16-byte access
+  static constexpr int P = NB + V;                           // pitch: rows 16 bytes off a multiple of 128
+  static constexpr int PL = SB + V;
+  static constexpr int THREADS = 256;                        // seven warps for C, one for A
+  static constexpr size_t SMEM = ((size_t)2 * NB * P + (size_t)SB * PL + SB) * sizeof(T);
+  static_assert(NB % SB == 0 && NB <= 256, "rows map to threads");
+
+  struct __align__(16) Vec { T v[V]; };
+
+  // phase A on the sub-block at D (pitch P): LT[k][j] = L[j][k] below the diagonal, rds[j] = 1 / L[j][j]
+  static __device__ __forceinline__ void factor(const T* D, T* LT, T* rds, int lane, int64_t row0, int32_t* status) {
+    T a[SB];
+#pragma unroll
+    for (int c = 0; c < SB; c += V) {
+      const Vec q = *reinterpret_cast<const Vec*>(D + lane * P + c);
+#pragma unroll
+      for (int v = 0; v < V; ++v) a[c + v] = q.v[v];
+    }
+    T dg = D[lane * P + lane];                               // this lane's diagonal entry, updated on its own
+    int bad = SB;
+    T lp = (T)0;                                             // l of the previous column
+#pragma unroll
+    for (int j = 0; j < SB; ++j) {
+      // critical chain: diagonal entry -> reciprocal root -> l of this column
+      T d = __shfl_sync(0xffffffffu, dg, j);
+      if (j > 0) a[j] = fma(-lp, __shfl_sync(0xffffffffu, lp, j), a[j]);
+      bad = (d > (T)0 || bad < SB) ? bad : j;
+      d = d > (T)0 ? d : (T)1;
+      const T rd = rsqrt_refined(d);
+      const T l = lane > j ? a[j] * rd : (T)0;
+      dg = fma(-l, l, dg);
+      LT[j * PL + lane] = l;
+      if (lane == j) rds[j] = rd;
+      // the rest of the previous column's update fills the chain's latencies
+      if (j > 0) {
+#pragma unroll
+        for (int c0 = (j + 1) / V * V; c0 < SB; c0 += V) {
+          const Vec q = *reinterpret_cast<const Vec*>(LT + (j - 1) * PL + c0);
+#pragma unroll
+          for (int v = 0; v < V; ++v)
+            if (c0 + v > j) a[c0 + v] = fma(-lp, q.v[v], a[c0 + v]);
+        }
+      }
+      __syncwarp();
+      lp = l;
+    }
+    if (bad < SB && lane == 0) report_status(status, SP_ERR_NOT_SPD, (int32_t)(row0 + bad), 0);
+  }
+
+  // phase B: x <- x L11^-T
+  static __device__ __forceinline__ void solve_row(T* row, const T* LT, const T* rds) {
+    T x[SB];
+#pragma unroll
+    for (int c = 0; c < SB; c += V) {
+      const Vec q = *reinterpret_cast<const Vec*>(row + c);
+#pragma unroll
+      for (int v = 0; v < V; ++v) x[c + v] = q.v[v];
+    }
+#pragma unroll
+    for (int k = 0; k < SB; ++k) {
+      x[k] *= rds[k];
+#pragma unroll
+      for (int j0 = (k + 1) / V * V; j0 < SB; j0 += V) {
+        const Vec q = *reinterpret_cast<const Vec*>(LT + k * PL + j0);
+#pragma unroll
+        for (int v = 0; v < V; ++v)
+          if (j0 + v > k) x[j0 + v] = fma(-x[k], q.v[v], x[j0 + v]);
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < SB; c += V) {
+      Vec q;
+#pragma unroll
+      for (int v = 0; v < V; ++v) q.v[v] = x[c + v];
+      *reinterpret_cast<Vec*>(row + c) = q;
+    }
+  }
+
+  // dst -= Y L^T over 32 values of K for one warp: 32 rows (from `row` on) x 4 C columns; dcol / ycol: first column of dst
+  // and Y, L: offset of L's first element.  A lane has rows (lane >> 2) + 8 i and columns (lane & 3) + 4 j: no bank conflicts.
+  template <int C>
+  static __device__ __forceinline__ void rank32(T* sm, int row, int dcol, int ycol, int L, int lane) {
+    typename PairAcc<T>::type acc[4][C];
+    const int lr = lane >> 2, lc = lane & 3;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < C; ++j) acc[i][j] = {};
+#pragma unroll 4
+    for (int k = 0; k < SB; k += V) {
+      Vec a[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        a[i] = *reinterpret_cast<const Vec*>(sm + (row + lr + i * 8) * P + ycol + k);
+#pragma unroll
+      for (int j = 0; j < C; ++j) {
+        const Vec l = *reinterpret_cast<const Vec*>(sm + L + (lc + j * 4) * P + k);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int v = 0; v < V; v += 2) fma_pair(acc[i][j], a[i].v + v, l.v + v);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < C; ++j) sm[(row + lr + i * 8) * P + dcol + lc + j * 4] -= pair_sum(acc[i][j]);
+  }
+
+  // A: the nb x nb block (lower triangle; rows and columns beyond nb are those of an identity).  inv [NB, NB] receives
+  // inv(L), inv_t (nullptr: not wanted) its transpose; both dense, zero outside their triangle.
+  static __device__ void run(const T* A, int64_t lda, int nb, T* inv, T* inv_t, int64_t row0, int32_t* status) {
+    extern __shared__ __align__(16) unsigned char diag_smem[];
+    T* M = reinterpret_cast<T*>(diag_smem);                  // matrix rows
+    T* X = M + NB * P;                                       // identity rows
+    T* LT = X + NB * P;
+    T* rds = LT + SB * PL;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    constexpr int NW = THREADS / 32;
+    // load: one warp per row and 32 V columns, 16 bytes per lane where the rows allow it
+    const bool vec = lda % V == 0 && (reinterpret_cast<uintptr_t>(A) & 15u) == 0;
+    constexpr int VPR = NB / V;
+#pragma unroll
+    for (int e = t; e < NB * VPR; e += THREADS) {
+      const int i = e / VPR, c = (e % VPR) * V;
+      Vec q;
+      if (vec && i < nb && c + V <= nb) {
+        q = *reinterpret_cast<const Vec*>(A + (int64_t)i * lda + c);
+      } else {
+#pragma unroll
+        for (int v = 0; v < V; ++v) q.v[v] = (i < nb && c + v <= i) ? A[(int64_t)i * lda + c + v] : (T)0;
+      }
+#pragma unroll
+      for (int v = 0; v < V; ++v) q.v[v] = c + v > i ? (T)0 : (i >= nb && c + v == i) ? (T)1 : q.v[v];
+      *reinterpret_cast<Vec*>(M + i * P + c) = q;
+#pragma unroll
+      for (int v = 0; v < V; ++v) q.v[v] = c + v == i ? (T)1 : (T)0;
+      *reinterpret_cast<Vec*>(X + i * P + c) = q;
+    }
+    __syncthreads();
+    // columns cs .. cs + 31 of X: rows of inv(L) (lanes along a row) and columns of its transpose, by the NB threads from
+    // STORE0 on
+    constexpr int STORE0 = 96;
+    auto store_inv = [&](int cs) {
+      const int t = (int)threadIdx.x - STORE0;
+      if (t >= NB) return;
+#pragma unroll
+      for (int c = 0; c < SB; c += V) {
+        const Vec q = *reinterpret_cast<const Vec*>(X + t * P + cs + c);
+        if (inv_t != nullptr) *reinterpret_cast<Vec*>(inv_t + t * NB + cs + c) = q;
+#pragma unroll
+        for (int v = 0; v < V; ++v) inv[(cs + c + v) * NB + t] = q.v[v];
+      }
+    };
+    for (int s = 0; s < NS; ++s) {
+      const int cs = s * SB, ce = cs + SB;
+      if (warp == NW - 1) {
+        factor(M + cs * P + cs, LT, rds, lane, row0 + cs, status);
+      } else if (s > 0) {
+        // rest of the update of sub-block s - 1: matrix rows, then identity rows (X follows M: its row r is row NB + r).
+        // The factorising warp shares its scheduler with warp 3, which comes last; warps 3 to 6 also store.
+        const int ps = cs - SB;
+        int turn = 0;
+        for (int cb = s; cb < NS; ++cb)
+          for (int rb = cb == s ? s + 1 : cb; rb < NS + s; ++rb) {             // ((s, s) is done before)
+            const int w = turn++ % (NW - 1);
+            if (warp == (w < 3 ? w : w < 6 ? w + 1 : 3))
+              rank32<8>(M, (rb < NS ? rb : NB / SB + rb - NS) * SB, cb * SB, ps, cb * SB * P + ps, lane);
+          }
+        if (t >= STORE0) store_inv(ps);
+      }
+      __syncthreads();
+      if (t < NB) solve_row((t >= ce ? M : X) + t * P + cs, LT, rds);
+      __syncthreads();
+      if (ce < NB) {
+        // next diagonal sub-block, 32 x 4 entries per warp
+        rank32<1>(M, ce, ce + warp * 4, cs, (ce + warp * 4) * P + cs, lane);
+        __syncthreads();
+      }
+    }
+    if (t >= STORE0) store_inv(NB - SB);
+  }
+};
+
+}  // namespace sp

@@ -7,234 +7,29 @@
 // mid.mid), each a K segment of one tcgen05 GEMM with fp32 accumulation.  The dropped terms are below 2^-23.
 //
 // Blocked right-looking algorithm with 128-wide panels:
-//   diagonal block : one CTA factorises it in registers (4 x 4 elements per thread, four columns per step) and forms
-//                    inv(L11) in the same sweep (the row operations of the elimination applied to an identity block);
+//   diagonal block : one CTA factorises it and forms inv(L11) in the same sweep (sp_chol_block.cuh);
 //   panel          : L21 = A21 inv(L11)^T on the CUDA cores (K = 128), written as fp32 and as the three bf16 parts;
 //   trailing update: A22 -= L21 L21^T (lower triangle) as one six-segment tensor-core GEMM.
 // The triangular solves X L^T = R, W L = X use the same two kernels block column by block column.
+#include "sp_chol_block.cuh"
 #include "sp_common.cuh"
 
 namespace sp {
 namespace {
 
 constexpr int TB = kCholTcNB;          // 128
-constexpr int DIAG_BLOCKS = (TB / 4) * (TB / 4 + 1) / 2;   // 528 lower-triangular 4 x 4 blocks
-constexpr int DIAG_THREADS = 544;      // 17 warps
 
-// 1 / sqrt(x) to about 1 ulp: hardware approximation plus one Newton step.
-__device__ __forceinline__ float rsqrt_refined(float x) {
-  float r;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r * fmaf(-0.5f * x, r * r, 1.5f);
-}
+using Diag = DiagBlock<float, TB>;
 
-constexpr int DIAG_TPAD = TB + 1;
-constexpr size_t DIAG_SMEM = (size_t)TB * DIAG_TPAD * sizeof(float);
-
-// Factorise the nb x nb diagonal block at A (lower triangle, left as it is) and write inv(L) and its transpose to
-// dinv[0 : TB*TB] and dinv[TB*TB : 2*TB*TB] (row-major TB x TB, zero above / below the diagonal respectively,
-// identity on the padding rows nb..TB-1).  A non-positive pivot is reported once through `status` and replaced by 1.
-//
-// One thread owns one 4 x 4 block (bi, bj), bj <= bi, of the lower triangle in registers.  Blocked right-looking
-// elimination, four columns per step jb, that carries inv(L) along (the row operations of the elimination applied to
-// an identity block B).  Register block m holds the trailing matrix on block columns > jb and B on block columns
-// <= jb; a block column of the trailing matrix is final when its step comes and moves to lcol.  Per step:
-//   1. the owner of the diagonal block factorises it, D = C C^T, and inverts C (sequential, one thread; it runs while
-//      the other threads still finish step jb - 1);
-//   2. owners of block column jb:  L_i = A_i C^-T (final);  owners of block row jb:  B_jb <- C^-1 B_jb (final rows of
-//      inv(L)).  Both go to the shared array W (4 values per index): W[:, i] = L[i, j0:j0+4] for rows below the
-//      block, W[:, c] = inv(L)[j0:j0+4, c] for columns up to the block;
-//   3. every block below block row jb:  m -= W[:, rows]^T W[:, cols]  — the trailing update where the block still
-//      holds the matrix, the update of B where it holds B (a block of block column jb starts its life as B from 0).
-// Global input and output go through a padded shared tile so that every global access is a full coalesced row.
-__global__ void __launch_bounds__(DIAG_THREADS) chol_diag128_kernel(float* A, int64_t lda, int nb, float* dinv,
-                                                                    int64_t row0, int32_t* status,
-                                                                    const int32_t* skip, int64_t a_bs, int64_t d_bs) {
+// Diagonal block: inv(L) and its transpose to dinv[0 : TB*TB] and dinv[TB*TB : 2*TB*TB].  L itself is not written back:
+// the solves use inv(L) of the diagonal blocks and the blocks of L below them only.
+__global__ void __launch_bounds__(Diag::THREADS) chol_diag128_kernel(const float* A, int64_t lda, int nb, float* dinv,
+                                                                     int64_t row0, int32_t* status,
+                                                                     const int32_t* skip, int64_t a_bs, int64_t d_bs) {
   if (skip != nullptr && *skip != 0) return;                  // conditional launch (see SkipScope)
   A += (int64_t)blockIdx.x * a_bs;                            // batched launch: one CTA per system
   dinv += (int64_t)blockIdx.x * d_bs;
-  extern __shared__ __align__(16) float diag_tile[];          // T[TB][TB + 1]
-  float (*T)[DIAG_TPAD] = reinterpret_cast<float (*)[DIAG_TPAD]>(diag_tile);
-  __shared__ __align__(16) float W[2][4][TB];   // W[k][index]: conflict-free 16-byte accesses along the index
-  __shared__ __align__(16) float Ci_s[2][16];   // inverse of the diagonal factor, row-major 4 x 4 (lower)
-  const int t = threadIdx.x;
-  const int lane = t & 31, warp = t >> 5;
-  constexpr int NWARP = DIAG_THREADS / 32;
-  const bool active = t < DIAG_BLOCKS;
-  // t = bi (bi + 1) / 2 + bj with bj <= bi
-  int bi = (int)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
-  while ((bi + 1) * (bi + 2) / 2 <= t) ++bi;
-  while (bi * (bi + 1) / 2 > t) --bi;
-  const int bj = t - bi * (bi + 1) / 2;
-
-  // ---- load: one warp per row, lanes along the columns; identity on the padding
-  for (int i = warp; i < TB; i += NWARP)
-    for (int c = lane; c < TB; c += 32) {
-      float v = 0.f;
-      if (i < nb && c <= i) v = A[(int64_t)i * lda + c];
-      if (i >= nb && i == c) v = 1.f;
-      T[i][c] = v;
-    }
-  __syncthreads();
-  float m[4][4], lcol[4][4];
-#pragma unroll
-  for (int r = 0; r < 4; ++r)
-#pragma unroll
-    for (int s = 0; s < 4; ++s) {
-      m[r][s] = active ? T[4 * bi + r][4 * bj + s] : 0.f;
-      lcol[r][s] = 0.f;
-    }
-
-  // step 1 for block jb by its diagonal owner: C -> lcol, C^-1 -> m, shared copies of C^-1
-  auto factor_diag = [&](int jb) {
-    float c[4][4], ci[4][4];
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-      for (int s = 0; s < 4; ++s) { c[r][s] = 0.f; ci[r][s] = 0.f; }
-    float rd[4];   // reciprocals of the diagonal of C
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      float p = m[k][k];
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (q < k) p = fmaf(-c[k][q], c[k][q], p);
-      if (!(p > 0.f)) {
-        report_status(status, SP_ERR_NOT_SPD, (int32_t)(row0 + 4 * jb + k), 0);
-        p = 1.f;
-      }
-      rd[k] = rsqrt_refined(p);
-      c[k][k] = p * rd[k];
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        if (r > k) {
-          float v = m[r][k];
-#pragma unroll
-          for (int q = 0; q < 4; ++q)
-            if (q < k) v = fmaf(-c[r][q], c[k][q], v);
-          c[r][k] = v * rd[k];
-        }
-      }
-    }
-    // inverse of the lower-triangular C by forward substitution, column by column
-#pragma unroll
-    for (int s = 0; s < 4; ++s) {
-      ci[s][s] = rd[s];
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        if (r > s) {
-          float v = 0.f;
-#pragma unroll
-          for (int q = 0; q < 4; ++q)
-            if (q >= s && q < r) v = fmaf(c[r][q], ci[q][s], v);
-          ci[r][s] = -v * rd[r];
-        }
-      }
-    }
-    float* cs = Ci_s[jb & 1];
-    float (*w)[TB] = W[jb & 1];
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-      for (int s = 0; s < 4; ++s) {
-        lcol[r][s] = c[r][s];
-        m[r][s] = ci[r][s];
-        cs[r * 4 + s] = ci[r][s];
-        w[r][4 * jb + s] = ci[r][s];          // W[k][c] = inv(L)[j0 + k][c]
-      }
-  };
-
-  if (active && bi == 0) factor_diag(0);
-  const int nsteps = (nb + 3) / 4;
-  for (int jb = 0; jb < nsteps; ++jb) {
-    float (*w)[TB] = W[jb & 1];
-    __syncthreads();
-    if (active && bj == jb && bi > jb) {
-      // L_i = A_i C^-T : L_i[r][k] = sum_{s <= k} A_i[r][s] Ci[k][s]
-      const float* cs = Ci_s[jb & 1];
-      float l[4][4];
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          float v = 0.f;
-#pragma unroll
-          for (int s2 = 0; s2 < 4; ++s2)
-            if (s2 <= k) v = fmaf(m[r][s2], cs[k * 4 + s2], v);
-          l[r][k] = v;
-        }
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-        *reinterpret_cast<float4*>(&w[k][4 * bi]) = make_float4(l[0][k], l[1][k], l[2][k], l[3][k]);
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) { lcol[r][k] = l[r][k]; m[r][k] = 0.f; }
-    }
-    if (active && bi == jb && bj < jb) {
-      // B_jb <- C^-1 B_jb : Bn[k][s] = sum_{r <= k} Ci[k][r] B[r][s]
-      const float* cs = Ci_s[jb & 1];
-      float bn[4][4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-#pragma unroll
-        for (int s2 = 0; s2 < 4; ++s2) {
-          float v = 0.f;
-#pragma unroll
-          for (int r = 0; r < 4; ++r)
-            if (r <= k) v = fmaf(cs[k * 4 + r], m[r][s2], v);
-          bn[k][s2] = v;
-        }
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        *reinterpret_cast<float4*>(&w[k][4 * bj]) = make_float4(bn[k][0], bn[k][1], bn[k][2], bn[k][3]);
-#pragma unroll
-        for (int s2 = 0; s2 < 4; ++s2) m[k][s2] = bn[k][s2];
-      }
-    }
-    __syncthreads();
-    if (active && bi > jb) {
-      float wr[4][4], wc[4][4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const float4 v = *reinterpret_cast<const float4*>(&w[k][4 * bi]);
-        wr[0][k] = v.x; wr[1][k] = v.y; wr[2][k] = v.z; wr[3][k] = v.w;
-        const float4 u = *reinterpret_cast<const float4*>(&w[k][4 * bj]);
-        wc[0][k] = u.x; wc[1][k] = u.y; wc[2][k] = u.z; wc[3][k] = u.w;
-      }
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int s2 = 0; s2 < 4; ++s2) {
-          float v = m[r][s2];
-#pragma unroll
-          for (int k = 0; k < 4; ++k) v = fmaf(-wr[r][k], wc[s2][k], v);
-          m[r][s2] = v;
-        }
-      // the owner of the next diagonal block goes straight on to factorise it
-      if (bi == jb + 1 && bj == jb + 1 && jb + 1 < nsteps) factor_diag(jb + 1);
-    }
-  }
-
-  // ---- store inv(L) and its transpose through the tile
-  __syncthreads();
-  for (int e = t; e < TB * TB; e += DIAG_THREADS) T[e / TB][e % TB] = 0.f;
-  __syncthreads();
-  if (active) {
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-      for (int s = 0; s < 4; ++s)
-        if (4 * bj + s <= 4 * bi + r) T[4 * bi + r][4 * bj + s] = m[r][s];
-  }
-  __syncthreads();
-  for (int i = warp; i < TB; i += NWARP)
-    for (int c = lane; c < TB; c += 32) {
-      dinv[i * TB + c] = T[i][c];
-      dinv[TB * TB + i * TB + c] = T[c][i];      // row i of the transpose = column i of inv(L)
-    }
-  // L itself is not written back: the solves use inv(L) of the diagonal blocks and the blocks of L below them only.
-  (void)lcol;
+  Diag::run(A, lda, nb, dinv, dinv + TB * TB, row0, status);
 }
 
 __device__ __forceinline__ void split3(float v, __nv_bfloat16& hi, __nv_bfloat16& mid, __nv_bfloat16& lo) {
@@ -647,7 +442,7 @@ sp_status potrf_lower_tc(float* A, int64_t n, int64_t lda, float* dinv, void* Pv
   static PerDeviceOnce attr_once;
   if (attr_once.run([] {
         cudaError_t e = cudaFuncSetAttribute(chol_diag128_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)DIAG_SMEM);
+                                             (int)Diag::SMEM);
         if (e == cudaSuccess)
           e = cudaFuncSetAttribute(chol_next_diag_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)NM_SMEM);
         if (e == cudaSuccess)
@@ -697,7 +492,7 @@ sp_status potrf_lower_tc(float* A, int64_t n, int64_t lda, float* dinv, void* Pv
       if (assist && inner_first && kb > 0) SP_CUDA_OK(cudaStreamWaitEvent(stream, assist->near_done, 0));
       count_launch();
       ProfScope prof(PK_CHOL_DIAG, (double)nb * nb * nb * (2.0 / 3.0), 0.0, stream);
-      chol_diag128_kernel<<<1, DIAG_THREADS, DIAG_SMEM, stream>>>(from_scratch ? S : A + k0 * lda + k0,
+      chol_diag128_kernel<<<1, Diag::THREADS, Diag::SMEM, stream>>>(from_scratch ? S : A + k0 * lda + k0,
                                                                   from_scratch ? (int64_t)TB : lda, nb, dk, k0,
                                                                   status_dev, skip, 0, 0);
       if (cudaGetLastError() != cudaSuccess) return SP_ERR_CUDA;
@@ -980,7 +775,7 @@ sp_status potrf_potrs_tc_batched(float* A, int64_t n, int64_t m, int batch, int6
   const int32_t* skip = skip_flag();
   static PerDeviceOnce attr_once;
   if (attr_once.run([] {
-        return cudaFuncSetAttribute(chol_diag128_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DIAG_SMEM);
+        return cudaFuncSetAttribute(chol_diag128_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Diag::SMEM);
       }) != cudaSuccess)
     return SP_ERR_CUDA;
   TcBatch bt;
@@ -993,7 +788,7 @@ sp_status potrf_potrs_tc_batched(float* A, int64_t n, int64_t m, int batch, int6
     const int64_t k0 = kb * TB;
     float* dk = dinv + kb * 2 * TB * TB;
     count_launch();
-    chol_diag128_kernel<<<batch, DIAG_THREADS, DIAG_SMEM, stream>>>(A + k0 * lda + k0, lda, TB, dk, k0, status_dev, skip,
+    chol_diag128_kernel<<<batch, Diag::THREADS, Diag::SMEM, stream>>>(A + k0 * lda + k0, lda, TB, dk, k0, status_dev, skip,
                                                                   a_bs, d_bs);
     if (cudaGetLastError() != cudaSuccess) return SP_ERR_CUDA;
     const int64_t rem = n - k0 - TB, prow = rem + m;

@@ -1,5 +1,5 @@
-"""The fp64 contraction kernel and the fp64 factorisation / solves at the edges of their tiles (64 x 64 and 32 x 64 tiles,
-K slabs of 16, block columns of 64), against plain fp64 torch."""
+"""The fp64 contraction kernel and the factorisations / solves of both precisions at the edges of their tiles (fp64: 64 x 64
+and 32 x 64 tiles, K slabs of 16, block columns of 64; fp32: block columns of 128), against plain fp64 torch."""
 import pytest
 import torch
 
@@ -60,6 +60,26 @@ def test_precise_ridge_solve_at_block_edges(n, m):
     assert float((got.double() - want).abs().max() / want.abs().max()) < 1.2e-7
     again = api.sp_ridge_solve(R, G, 0.01, True, precise=True)
     assert torch.equal(got, again)      # no result depends on the order of the two streams
+
+
+@pytest.mark.parametrize("n,m", [(1, 3), (31, 40), (33, 8), (96, 129), (127, 64), (128, 200), (129, 7), (385, 96), (1000, 300)])
+def test_tensor_core_ridge_solve_at_block_edges(n, m):
+    """Diagonal blocks of 128 eliminated in sub-blocks of 32, panels of a few rows."""
+    api = _api()
+    G = _spd(n, n + 1)
+    R = torch.randn(m, n, generator=torch.Generator(device="cuda").manual_seed(m), device="cuda")
+    status = api.new_status(G.device)
+    got = api.sp_ridge_solve(R, G, 0.1, True, status=status)
+    H = G.double() + 0.1 * G.double().diagonal().mean() * torch.eye(n, device="cuda", dtype=torch.float64)
+    want = torch.linalg.solve(H, R.double().T).T
+    # backward stable fp32 solve: a few roundings of 2^-24 times the condition number (the ridge bounds it by 10 n)
+    assert float((got.double() - want).abs().max() / want.abs().max()) < 4 * 2.0 ** -24 * 10 * max(n, 10)
+    assert int(status[0]) == 0
+    bad = G.clone()
+    i = n // 2
+    bad[i, i] = -bad[i, i].abs() * 100
+    api.sp_ridge_solve(R, bad, 1e-6, False, status=status)
+    assert status[:2].tolist() == [6, i]      # SP_ERR_NOT_SPD and the pivot
 
 
 @pytest.mark.parametrize("d", [8, 64, 72, 136, 520, 1096])
