@@ -20,33 +20,17 @@ __device__ __forceinline__ double rsqrt_refined(double x) {
   return fma(y * e, fma(0.375, e, 0.5), y);
 }
 
-// acc += a b on pairs of neighbouring values (fp32: one packed instruction)
-__device__ __forceinline__ void fma_pair(float2& acc, const float* a, const float* b) {
-  asm("{\n\t.reg .b64 a, b, c;\n\t"
-      "mov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tmov.b64 c, {%0, %1};\n\t"
-      "fma.rn.f32x2 c, a, b, c;\n\tmov.b64 {%0, %1}, c;\n\t}"
-      : "+f"(acc.x), "+f"(acc.y)
-      : "f"(a[0]), "f"(a[1]), "f"(b[0]), "f"(b[1]));
-}
-__device__ __forceinline__ void fma_pair(double& acc, const double* a, const double* b) {
-  acc = fma(a[0], b[0], acc);
-  acc = fma(a[1], b[1], acc);
-}
-__device__ __forceinline__ float pair_sum(const float2& v) { return v.x + v.y; }
-__device__ __forceinline__ double pair_sum(double v) { return v; }
-template <typename T> struct PairAcc { using type = double; };
-template <> struct PairAcc<float> { using type = float2; };
-
 // The block is eliminated in sub-blocks of 32 columns.  Rows to carry along are the rows of the matrix below the
 // sub-block and the rows of an identity appended under the matrix (X L^T = I, so X = L^-T): together always NB rows.  Per sub-block
 //   A  one warp factorises the 32 x 32 diagonal sub-block, one row per lane, columns handed round by shuffles;
 //   B  one thread per row solves x L11^T = row for its 32 entries (L11 read as broadcasts);
 //   C  the columns to the right receive the rank-32 update in 32 x 32 pieces, one warp each.  The next diagonal
 //      sub-block comes first, by all warps; the other pieces run beside the next phase A.
-// What bounds it is latency: A (about 120 cycles per column: shuffle, reciprocal root, product, update), B and the first
-// piece of C; for 128 columns the other pieces take as long as A.  Measured inside a factorisation: 25 us for 128 columns
-// in fp32, 14 us for 64 in fp64.  The form before this one eliminated four columns per step in registers of one thread
-// per 4 x 4 block; two block barriers and all warps' shared update stood between a pivot and the next (37 and 20 us).
+// Every entry receives its updates column by column in ascending order, whatever the blocking.  What bounds the kernel is
+// latency: A (about 120 cycles per column), B and the first piece of C; for 128 columns the other pieces take as long as
+// A.  Measured inside a factorisation: 25 us for 128 columns in fp32, 14 us for 64 in fp64.  The form before this one held
+// one 4 x 4 block per thread; two block barriers and all warps' shared update stood between one 4 x 4 pivot block and the
+// next (37 and 20 us, the same operations in the same order).
 template <typename T, int NB>
 struct DiagBlock {
   static constexpr int SB = 32, NS = NB / SB;
@@ -54,13 +38,26 @@ struct DiagBlock {
   static constexpr int P = NB + V;                           // pitch: rows 16 bytes off a multiple of 128
   static constexpr int PL = SB + V;
   static constexpr int THREADS = 256;                        // seven warps for C, one for A
-  static constexpr size_t SMEM = ((size_t)2 * NB * P + (size_t)SB * PL + SB) * sizeof(T);
+  static constexpr size_t SMEM = ((size_t)2 * NB * P + (size_t)SB * PL + 4 * SB) * sizeof(T);
   static_assert(NB % SB == 0 && NB <= 256, "rows map to threads");
 
   struct __align__(16) Vec { T v[V]; };
 
-  // phase A on the sub-block at D (pitch P): LT[k][j] = L[j][k] below the diagonal, rds[j] = 1 / L[j][j]
-  static __device__ __forceinline__ void factor(const T* D, T* LT, T* rds, int lane, int64_t row0, int32_t* status) {
+  // Four columns are eliminated at a time: C C^T = their 4 x 4 diagonal block, and a row's entries m in these columns become
+  // l = m C^-T, with C^-1 (row-major, lower) in ci.
+  static __device__ __forceinline__ void apply_ci(const T (&m)[4], const T* ci, T (&l)[4]) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      T v = (T)0;
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (q <= k) v = fma(m[q], ci[k * 4 + q], v);
+      l[k] = v;
+    }
+  }
+
+  // phase A on the sub-block at D (pitch P): LT[k][j] = L[j][k] below the 4 x 4 diagonal blocks, CI[k / 4] = their C^-1
+  static __device__ __forceinline__ void factor(const T* D, T* LT, T* CI, int lane, int64_t row0, int32_t* status) {
     T a[SB];
 #pragma unroll
     for (int c = 0; c < SB; c += V) {
@@ -68,39 +65,92 @@ struct DiagBlock {
 #pragma unroll
       for (int v = 0; v < V; ++v) a[c + v] = q.v[v];
     }
-    T dg = D[lane * P + lane];                               // this lane's diagonal entry, updated on its own
     int bad = SB;
-    T lp = (T)0;                                             // l of the previous column
+    T lp[4] = {(T)0, (T)0, (T)0, (T)0};            // this lane's L entries of the previous four columns
+    // a[c .. c + 3] -= lp L[c .. c + 3]^T of the previous four columns (from k0 on)
+    auto update = [&](int k0, int c) {
 #pragma unroll
-    for (int j = 0; j < SB; ++j) {
-      // critical chain: diagonal entry -> reciprocal root -> l of this column
-      T d = __shfl_sync(0xffffffffu, dg, j);
-      if (j > 0) a[j] = fma(-lp, __shfl_sync(0xffffffffu, lp, j), a[j]);
-      bad = (d > (T)0 || bad < SB) ? bad : j;
-      d = d > (T)0 ? d : (T)1;
-      const T rd = rsqrt_refined(d);
-      const T l = lane > j ? a[j] * rd : (T)0;
-      dg = fma(-l, l, dg);
-      LT[j * PL + lane] = l;
-      if (lane == j) rds[j] = rd;
-      // the rest of the previous column's update fills the chain's latencies
+      for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int h = 0; h < 4; h += V) {
+          const Vec q = *reinterpret_cast<const Vec*>(LT + (k0 + k) * PL + c + h);
+#pragma unroll
+          for (int v = 0; v < V; ++v) a[c + h + v] = fma(-lp[k], q.v[v], a[c + h + v]);
+        }
+    };
+#pragma unroll
+    for (int j = 0; j < SB; j += 4) {
+      // critical chain: next four columns -> their diagonal block in every lane -> C, C^-1 -> l of these columns
+      if (j > 0) update(j - 4, j);
+      T m[4][4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (q <= r) m[r][q] = __shfl_sync(0xffffffffu, a[j + q], j + r);
+      // the rest of the previous columns' update fills the chain's latencies
       if (j > 0) {
 #pragma unroll
-        for (int c0 = (j + 1) / V * V; c0 < SB; c0 += V) {
-          const Vec q = *reinterpret_cast<const Vec*>(LT + (j - 1) * PL + c0);
+        for (int c = j + 4; c < SB; c += 4) update(j - 4, c);
+      }
+      T c[4][4], rd[4], ci[16];
 #pragma unroll
-          for (int v = 0; v < V; ++v)
-            if (c0 + v > j) a[c0 + v] = fma(-lp, q.v[v], a[c0 + v]);
+      for (int k = 0; k < 4; ++k) {
+        T p = m[k][k];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (q < k) p = fma(-c[k][q], c[k][q], p);
+        bad = (p > (T)0 || bad < SB) ? bad : j + k;
+        p = p > (T)0 ? p : (T)1;
+        rd[k] = rsqrt_refined(p);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+          if (r > k) {
+            T v = m[r][k];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+              if (q < k) v = fma(-c[r][q], c[k][q], v);
+            c[r][k] = v * rd[k];
+          }
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        ci[q * 4 + q] = rd[q];
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+          if (r > q) {
+            T v = (T)0;
+#pragma unroll
+            for (int z = 0; z < 4; ++z)
+              if (z >= q && z < r) v = fma(c[r][z], ci[z * 4 + q], v);
+            ci[r * 4 + q] = -v * rd[r];
+          } else if (r < q) {
+            ci[r * 4 + q] = (T)0;
+          }
+      }
+      const T mine[4] = {a[j], a[j + 1], a[j + 2], a[j + 3]};
+      apply_ci(mine, ci, lp);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (lane < j + 4) lp[k] = (T)0;
+        LT[(j + k) * PL + lane] = lp[k];
+      }
+      if (lane == 0) {
+#pragma unroll
+        for (int q = 0; q < 16; q += V) {
+          Vec u;
+#pragma unroll
+          for (int v = 0; v < V; ++v) u.v[v] = ci[q + v];
+          *reinterpret_cast<Vec*>(CI + j * 4 + q) = u;
         }
       }
       __syncwarp();
-      lp = l;
     }
     if (bad < SB && lane == 0) report_status(status, SP_ERR_NOT_SPD, (int32_t)(row0 + bad), 0);
   }
 
   // phase B: x <- x L11^-T
-  static __device__ __forceinline__ void solve_row(T* row, const T* LT, const T* rds) {
+  static __device__ __forceinline__ void solve_row(T* row, const T* LT, const T* CI) {
     T x[SB];
 #pragma unroll
     for (int c = 0; c < SB; c += V) {
@@ -109,14 +159,25 @@ struct DiagBlock {
       for (int v = 0; v < V; ++v) x[c + v] = q.v[v];
     }
 #pragma unroll
-    for (int k = 0; k < SB; ++k) {
-      x[k] *= rds[k];
+    for (int j = 0; j < SB; j += 4) {
+      T ci[16], l[4];
 #pragma unroll
-      for (int j0 = (k + 1) / V * V; j0 < SB; j0 += V) {
-        const Vec q = *reinterpret_cast<const Vec*>(LT + k * PL + j0);
+      for (int q = 0; q < 16; q += V) {
+        const Vec u = *reinterpret_cast<const Vec*>(CI + j * 4 + q);
 #pragma unroll
-        for (int v = 0; v < V; ++v)
-          if (j0 + v > k) x[j0 + v] = fma(-x[k], q.v[v], x[j0 + v]);
+        for (int v = 0; v < V; ++v) ci[q + v] = u.v[v];
+      }
+      const T mine[4] = {x[j], x[j + 1], x[j + 2], x[j + 3]};
+      apply_ci(mine, ci, l);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        x[j + k] = l[k];
+#pragma unroll
+        for (int c = j + 4; c < SB; c += V) {
+          const Vec q = *reinterpret_cast<const Vec*>(LT + (j + k) * PL + c);
+#pragma unroll
+          for (int v = 0; v < V; ++v) x[c + v] = fma(-l[k], q.v[v], x[c + v]);
+        }
       }
     }
 #pragma unroll
@@ -132,12 +193,12 @@ struct DiagBlock {
   // and Y, L: offset of L's first element.  A lane has rows (lane >> 2) + 8 i and columns (lane & 3) + 4 j: no bank conflicts.
   template <int C>
   static __device__ __forceinline__ void rank32(T* sm, int row, int dcol, int ycol, int L, int lane) {
-    typename PairAcc<T>::type acc[4][C];
+    T acc[4][C];
     const int lr = lane >> 2, lc = lane & 3;
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int j = 0; j < C; ++j) acc[i][j] = {};
+      for (int j = 0; j < C; ++j) acc[i][j] = sm[(row + lr + i * 8) * P + dcol + lc + j * 4];
 #pragma unroll 4
     for (int k = 0; k < SB; k += V) {
       Vec a[4];
@@ -148,15 +209,15 @@ struct DiagBlock {
       for (int j = 0; j < C; ++j) {
         const Vec l = *reinterpret_cast<const Vec*>(sm + L + (lc + j * 4) * P + k);
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int v = 0; v < V; ++v)
 #pragma unroll
-          for (int v = 0; v < V; v += 2) fma_pair(acc[i][j], a[i].v + v, l.v + v);
+          for (int i = 0; i < 4; ++i) acc[i][j] = fma(-a[i].v[v], l.v[v], acc[i][j]);
       }
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int j = 0; j < C; ++j) sm[(row + lr + i * 8) * P + dcol + lc + j * 4] -= pair_sum(acc[i][j]);
+      for (int j = 0; j < C; ++j) sm[(row + lr + i * 8) * P + dcol + lc + j * 4] = acc[i][j];
   }
 
   // A: the nb x nb block (lower triangle; rows and columns beyond nb are those of an identity).  inv [NB, NB] receives
@@ -166,7 +227,7 @@ struct DiagBlock {
     T* M = reinterpret_cast<T*>(diag_smem);                  // matrix rows
     T* X = M + NB * P;                                       // identity rows
     T* LT = X + NB * P;
-    T* rds = LT + SB * PL;
+    T* CI = LT + SB * PL;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     constexpr int NW = THREADS / 32;
     // load: one warp per row and 32 V columns, 16 bytes per lane where the rows allow it
@@ -207,7 +268,7 @@ struct DiagBlock {
     for (int s = 0; s < NS; ++s) {
       const int cs = s * SB, ce = cs + SB;
       if (warp == NW - 1) {
-        factor(M + cs * P + cs, LT, rds, lane, row0 + cs, status);
+        factor(M + cs * P + cs, LT, CI, lane, row0 + cs, status);
       } else if (s > 0) {
         // rest of the update of sub-block s - 1: matrix rows, then identity rows (X follows M: its row r is row NB + r).
         // The factorising warp shares its scheduler with warp 3, which comes last; warps 3 to 6 also store.
@@ -222,7 +283,7 @@ struct DiagBlock {
         if (t >= STORE0) store_inv(ps);
       }
       __syncthreads();
-      if (t < NB) solve_row((t >= ce ? M : X) + t * P + cs, LT, rds);
+      if (t < NB) solve_row((t >= ce ? M : X) + t * P + cs, LT, CI);
       __syncthreads();
       if (ce < NB) {
         // next diagonal sub-block, 32 x 4 entries per warp

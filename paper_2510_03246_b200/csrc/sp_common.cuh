@@ -187,8 +187,8 @@ sp_status potrf_lower_tc(float* A, int64_t n, int64_t lda, float* dinv, void* P,
                          bool split_lookahead = false);   // lookahead kernel as two launches without a cluster
 // Xs holds TWO buffers of [m, 3 * kCholTcNB] bf16.
 // forward_done: X already holds the solution of the forward system (it rode along with the factorisation).
-// Lf / ldl (optional): the fp32 factor potrf_lower_tc left in A; with it the backward sweep updates the next block
-// column inside the panel kernel instead of by a GEMM of its own.
+// Lf / ldl (optional): the fp32 factor potrf_lower_tc left in A; with it the backward sweep updates a block column by
+// the one before it inside the panel kernel instead of by a GEMM of its own.
 sp_status potrs_right_tc(float* X, int64_t m, int64_t n, int64_t ldx, const void* P, const float* dinv, void* Xs,
                          int32_t* status_dev, cudaStream_t stream, const SolveAssist* assist = nullptr,
                          bool forward_done = false, const float* Lf = nullptr, int64_t ldl = 0,

@@ -78,137 +78,180 @@ __device__ __forceinline__ bool stage_block_wait(uint64_t* bar, uint32_t parity)
   }
 }
 
-constexpr int PA_ROWS = 32;
-constexpr int PA_THREADS = 256;
-constexpr int PA_APAD = PA_ROWS + 4;
-constexpr size_t PA_SMEM = ((size_t)TB * TB + (size_t)TB * PA_APAD) * sizeof(float) + 128;
-constexpr size_t PA_SMEM_NEAR = PA_SMEM + (size_t)TB * TB * sizeof(float);   // + the block of L of the second product
+// acc += {a, a} * {x, y} in one packed instruction
+__device__ __forceinline__ void fma_dup(float2& acc, float a, float x, float y) {
+  asm("{\n\t.reg .b64 a, b, c;\n\t"
+      "mov.b64 a, {%2, %2};\n\tmov.b64 b, {%3, %4};\n\tmov.b64 c, {%0, %1};\n\t"
+      "fma.rn.f32x2 c, a, b, c;\n\tmov.b64 {%0, %1}, c;\n\t}"
+      : "+f"(acc.x), "+f"(acc.y)
+      : "f"(a), "f"(x), "f"(y));
+}
 
-// Optional second product of the same launch (backward triangular solve, TRANS form only): with W_j the block column
-// just computed, X[:, near columns] -= W_j L[j rows, near columns], the update of the block column the NEXT step
-// needs, so that the chain of a solve is one kernel per block column.  L: fp32 factor, pointer to its element
-// (first row of block j, first near column), leading dimension ldl (a multiple of 4, 16-byte aligned rows); Xn: first
-// near column of X.  The far columns are updated by a tensor-core GEMM on another stream, which may still be adding
-// into the near columns when this kernel runs: both add atomically.
-struct PanelNear {
-  const float* L;    // nullptr: no second product
-  int64_t ldl;
-  float* Xn;
+// Product of an R x 128 tile (At[k][row], pitch R + 4) with a 128 x 128 block (Lt[k][c]), summed over k in ascending order
+// whatever R.  A warp takes RT rows, a lane four columns.  Shared memory delivers one register per lane and cycle and
+// the multiply-adds wait for it, so few rows per block are what makes a block fast.
+template <int R>
+struct RowTile {
+  static constexpr int THREADS = R == 32 ? 256 : 128;
+  static constexpr int AP = R + 4, RT = R / (THREADS / 32);
+  static_assert(R == 8 || R == 16 || R == 32, "tile shapes");
+  struct __align__(RT == 2 ? 8 : 16) Rows { float v[RT]; };
+  // thread t: rows row0(t) .. + RT - 1, columns col(t) .. + 3
+  static __device__ __forceinline__ int row0(int t) { return (t >> 5) * RT; }
+  static __device__ __forceinline__ int col(int t) { return (t & 31) * 4; }
+
+  static __device__ __forceinline__ void product(const float* At, const float* Lt, float4 (&out)[RT]) {
+    const float* ap = At + row0(threadIdx.x);
+    const float* lp = Lt + col(threadIdx.x);
+    float2 acc[RT][2];
+#pragma unroll
+    for (int r = 0; r < RT; ++r) acc[r][0] = acc[r][1] = make_float2(0.f, 0.f);
+#pragma unroll 8
+    for (int k = 0; k < TB; ++k) {
+      const Rows a = *reinterpret_cast<const Rows*>(ap + k * AP);
+      const float4 l = *reinterpret_cast<const float4*>(lp + k * TB);
+#pragma unroll
+      for (int r = 0; r < RT; ++r) {
+        fma_dup(acc[r][0], a.v[r], l.x, l.y);
+        fma_dup(acc[r][1], a.v[r], l.z, l.w);
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < RT; ++r) out[r] = make_float4(acc[r][0].x, acc[r][0].y, acc[r][1].x, acc[r][1].y);
+  }
+  // this thread's entries into At
+  static __device__ __forceinline__ void store(float* At, const float4 (&v)[RT]) { store_transposed(At, AP, v); }
+  static __device__ __forceinline__ void store_transposed(float* base, int pitch, const float4 (&v)[RT]) {
+    float* dst = base + col(threadIdx.x) * pitch + row0(threadIdx.x);
+    Rows u[4];
+#pragma unroll
+    for (int r = 0; r < RT; ++r) { u[0].v[r] = v[r].x; u[1].v[r] = v[r].y; u[2].v[r] = v[r].z; u[3].v[r] = v[r].w; }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) *reinterpret_cast<Rows*>(dst + j * pitch) = u[j];
+  }
 };
+template <int R>
+constexpr size_t pa_smem(bool with_near) {     // inv(L) block, row tile, (near) the block of L, barriers
+  return ((size_t)TB * TB * (with_near ? 2 : 1) + (size_t)TB * RowTile<R>::AP) * sizeof(float) + 16;
+}
+
+// Optional first product of the same launch (backward triangular solve, TRANS form only): the block column W_p that the
+// previous step left (nb_p columns, right of this one) is applied to this block column before it is multiplied by inv(L),
+// X_j -= W_p L[p rows, j columns], so that the chain of a solve is one kernel per block column.  A CTA reads and writes
+// its own rows only, and what the tensor-core updates on the other stream add into X_j is complete before the launch:
+// every entry is summed in a fixed order.  L: fp32 factor, pointer to element (first row of block p, first column of block
+// j), leading dimension ldl (a multiple of 4, 16-byte aligned rows); W: first column of W_p in X.
+struct PanelNear {
+  const float* L;    // nullptr: no such product
+  int64_t ldl;
+  const float* W;
+  int nb_p;
+};
+constexpr PanelNear kNoNear{nullptr, 0, nullptr, 0};
 // Batched launch of the panel kernel (grid.y = systems): element strides between the systems' arrays
 struct PanelBatch {
-  int64_t x = 0, dinv = 0, s = 0, near_l = 0;    // X (and the near columns), dinv, S, near.L
+  int64_t x = 0, dinv = 0, s = 0, near_l = 0;    // X (and near.W), dinv, S, near.L
 };
 
 // X[i, 0:nb] <- X[i, 0:nb] inv(L)^T (TRANS == false) or X[i, 0:nb] inv(L) (TRANS == true), for `rows` rows.
 // dinv is the pair of TB x TB blocks written by chol_diag128_kernel.  The result is written back in fp32 (write_f32)
 // and as three bf16 parts to S[i * lds + part * s_seg + c] for all TB columns (zero beyond nb).
-// One CTA takes 32 rows.  The 64 KiB block of inv(L) comes in by bulk copies while the threads fetch and transpose
-// the rows of X; a thread then computes 4 rows x 4 columns (a warp: 4 rows x 128 columns).
-template <bool TRANS>
-__global__ void __launch_bounds__(PA_THREADS) panel_apply_kernel(float* X, int64_t ldx, int64_t rows, int nb,
+// One CTA takes R rows.  The 64 KiB block of inv(L) comes in by bulk copies while the threads fetch and transpose the
+// rows of X.  The kernel is a link of a serial chain: few rows per CTA shorten it as long as one wave covers all rows
+// (see panel_rows): 768 rows, both products: 10.4 us with 48 CTAs of 16 rows, 15.4 us with 24 of 32.
+template <bool TRANS, int R>
+__global__ void __launch_bounds__(RowTile<R>::THREADS) panel_apply_kernel(float* X, int64_t ldx, int64_t rows, int nb,
                                                                  const float* __restrict__ dinv, __nv_bfloat16* S,
                                                                  int64_t lds, int64_t s_seg, int write_f32,
                                                                  int32_t* status, PanelNear near,
                                                                  const int32_t* skip, PanelBatch pb) {
   if (skip != nullptr && *skip != 0) return;
+  using Tile = RowTile<R>;
+  constexpr int AP = Tile::AP;
   X += (int64_t)blockIdx.y * pb.x;
   dinv += (int64_t)blockIdx.y * pb.dinv;
   if (S) S += (int64_t)blockIdx.y * pb.s;
-  if (near.L) { near.L += (int64_t)blockIdx.y * pb.near_l; near.Xn += (int64_t)blockIdx.y * pb.x; }
-  extern __shared__ __align__(128) float pa_smem[];
-  float (*Lt)[TB] = reinterpret_cast<float (*)[TB]>(pa_smem);                       // Lt[k][c]
-  float (*At)[PA_APAD] = reinterpret_cast<float (*)[PA_APAD]>(pa_smem + TB * TB);   // At[k][row]
-  uint64_t* bar = reinterpret_cast<uint64_t*>(pa_smem + TB * TB + TB * PA_APAD);    // [0]: Lt landed, [1]: Bn landed
-  float (*Bn)[TB] = reinterpret_cast<float (*)[TB]>(pa_smem + TB * TB + TB * PA_APAD + 32);   // Bn[k][c] (near only)
-  const int t = threadIdx.x;
-  const int64_t r0 = (int64_t)blockIdx.x * PA_ROWS;
-  const bool x_al = (ldx % 4 == 0) && ((reinterpret_cast<uintptr_t>(X) & 15u) == 0);
+  if (near.L) { near.L += (int64_t)blockIdx.y * pb.near_l; near.W += (int64_t)blockIdx.y * pb.x; }
+  extern __shared__ __align__(128) float pa_smem_raw[];
   const bool do_near = TRANS && near.L != nullptr;
-  if (t == 0) {
-    stage_bar_init(bar);
-    if (do_near) stage_bar_init(bar + 1);
-  }
+  float* Lt = pa_smem_raw;                                                      // Lt[k][c]
+  float* At = Lt + TB * TB;                                                     // At[k][row]
+  float* Bn = At + TB * AP;                                                     // Bn[k][c] (near only)
+  uint64_t* bar = reinterpret_cast<uint64_t*>(Bn + (do_near ? TB * TB : 0));    // Lt landed
+  const int t = threadIdx.x;
+  const int64_t r0 = (int64_t)blockIdx.x * R;
+  const bool x_al = (ldx % 4 == 0) && ((reinterpret_cast<uintptr_t>(X) & 15u) == 0);
+  if (t == 0) stage_bar_init(bar);
   __syncthreads();
   // Lt[k][c] = inv(L)[c][k] (the transposed copy) or inv(L)[k][c]: a straight copy either way
-  if (t == 0) stage_block_issue(pa_smem, dinv + (TRANS ? 0 : TB * TB), bar);
-  if (do_near && t < 32) {
-    // rows j0 .. j0 + nb - 1 of L, TB columns each (512 bytes per row), one bulk copy per row, four per lane
-    const uint32_t b1 = lin_smem_u32(bar + 1);
-    if (t == 0)
-      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b1), "r"((uint32_t)(nb * TB * 4))
-                   : "memory");
-    __syncwarp();
-    for (int k = t; k < nb; k += 32)
-      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                   ::"r"(lin_smem_u32(&Bn[k][0])), "l"(near.L + (int64_t)k * near.ldl), "r"((uint32_t)(TB * 4)),
-                     "r"(b1)
-                   : "memory");
+  if (t == 0) stage_block_issue(Lt, dinv + (TRANS ? 0 : TB * TB), bar);
+  if (do_near) {
+    // rows p .. p + nb_p - 1 of L, TB columns each; zeros below
+    for (int e = t; e < TB * TB / 4; e += Tile::THREADS) {
+      float* dst = Bn + e * 4;
+      if (e / (TB / 4) < near.nb_p)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(lin_smem_u32(dst)),
+                     "l"(near.L + (int64_t)(e / (TB / 4)) * near.ldl + (e % (TB / 4)) * 4)
+                     : "memory");
+      else
+        *reinterpret_cast<float4*>(dst) = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
   }
-  {
-    float4 xv[PA_ROWS * TB / 4 / PA_THREADS];
+  const int c0 = Tile::col(t), i0 = Tile::row0(t);      // the thread loads and stores columns c0 .. c0 + 3 of RT rows
+  auto load_rows = [&](const float* M, int width, float4 (&v)[Tile::RT]) {
 #pragma unroll
-    for (int q = 0; q < PA_ROWS * TB / 4 / PA_THREADS; ++q) {
-      const int e = t + q * PA_THREADS;
-      const int i = e / (TB / 4), k = (e % (TB / 4)) * 4;
-      const int64_t gi = r0 + i;
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int q = 0; q < Tile::RT; ++q) {
+      const int64_t gi = r0 + i0 + q;
+      v[q] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (gi < rows) {
-        const float* src = X + gi * ldx + k;
-        if (x_al && k + 4 <= nb) {
-          v = *reinterpret_cast<const float4*>(src);
+        const float* src = M + gi * ldx + c0;
+        if (x_al && c0 + 4 <= width) {
+          v[q] = *reinterpret_cast<const float4*>(src);
         } else {
-          if (k < nb) v.x = src[0];
-          if (k + 1 < nb) v.y = src[1];
-          if (k + 2 < nb) v.z = src[2];
-          if (k + 3 < nb) v.w = src[3];
+          if (c0 < width) v[q].x = src[0];
+          if (c0 + 1 < width) v[q].y = src[1];
+          if (c0 + 2 < width) v[q].z = src[2];
+          if (c0 + 3 < width) v[q].w = src[3];
         }
       }
-      xv[q] = v;
     }
+  };
+  float4 xv[Tile::RT], out[Tile::RT];
+  load_rows(X, nb, xv);
+  if (do_near) {
+    load_rows(near.W, near.nb_p, out);
+    Tile::store(At, out);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    Tile::product(At, Bn, out);
 #pragma unroll
-    for (int q = 0; q < PA_ROWS * TB / 4 / PA_THREADS; ++q) {
-      const int e = t + q * PA_THREADS;
-      const int i = e / (TB / 4), k = (e % (TB / 4)) * 4;
-      At[k][i] = xv[q].x; At[k + 1][i] = xv[q].y; At[k + 2][i] = xv[q].z; At[k + 3][i] = xv[q].w;
+    for (int q = 0; q < Tile::RT; ++q) {
+      xv[q].x -= out[q].x; xv[q].y -= out[q].y; xv[q].z -= out[q].z; xv[q].w -= out[q].w;
     }
+    __syncthreads();     // everyone is done reading At
   }
+  Tile::store(At, xv);
   // (the outcome is made uniform over the block: a thread whose wait ran out must not leave while others go on)
   const bool staged = __syncthreads_and(stage_block_wait(bar, 0) ? 1 : 0) != 0;
   if (!staged) {   // the copies did not land in time: report and leave X untouched
     if (t == 0) report_status(status, SP_ERR_TIMEOUT, (int32_t)blockIdx.x, 10);
     return;
   }
-  const int tx = t & 31, ty = t >> 5;   // columns 4 tx .. 4 tx + 3, rows 4 ty .. 4 ty + 3
-  float acc[4][4];
-#pragma unroll
-  for (int r = 0; r < 4; ++r)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[r][j] = 0.f;
-#pragma unroll 8
-  for (int k = 0; k < TB; ++k) {
-    const float4 a0 = *reinterpret_cast<const float4*>(&At[k][4 * ty]);
-    const float4 l0 = *reinterpret_cast<const float4*>(&Lt[k][4 * tx]);
-    const float av[4] = {a0.x, a0.y, a0.z, a0.w};
-    const float lv[4] = {l0.x, l0.y, l0.z, l0.w};
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[r][j] = fmaf(av[r], lv[j], acc[r][j]);
-  }
+  Tile::product(At, Lt, out);
   const bool x_vec = write_f32 && x_al;
-  const int c0 = 4 * tx;
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int64_t gi = r0 + 4 * ty + r;
+  for (int q = 0; q < Tile::RT; ++q) {
+    const int64_t gi = r0 + i0 + q;
+    float v[4] = {out[q].x, out[q].y, out[q].z, out[q].w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (c0 + j >= nb) v[j] = 0.f;
+    out[q] = make_float4(v[0], v[1], v[2], v[3]);
     if (gi >= rows) continue;
-    float v[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) v[j] = (c0 + j < nb) ? acc[r][j] : 0.f;
     if (write_f32) {
       float* dst = X + gi * ldx + c0;
       if (x_vec && c0 + 4 <= nb) {
-        *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
+        *reinterpret_cast<float4*>(dst) = out[q];
       } else {
 #pragma unroll
         for (int j = 0; j < 4; ++j)
@@ -220,73 +263,49 @@ __global__ void __launch_bounds__(PA_THREADS) panel_apply_kernel(float* X, int64
 #pragma unroll
       for (int j = 0; j < 4; ++j) split3(v[j], part[0][j], part[1][j], part[2][j]);
 #pragma unroll
-      for (int q = 0; q < 3; ++q)
-        *reinterpret_cast<uint2*>(S + gi * lds + q * s_seg + c0) = *reinterpret_cast<const uint2*>(part[q]);
+      for (int z = 0; z < 3; ++z)
+        *reinterpret_cast<uint2*>(S + gi * lds + z * s_seg + c0) = *reinterpret_cast<const uint2*>(part[z]);
     }
   }
+}
 
-  if (do_near) {
-    // ---- second product: X[rows, near columns] -= W_j Bn.  W_j goes back to shared memory as the left operand
-    // (At[k][row], k = column of W_j); rows of Bn beyond nb are cleared by hand (no copy wrote them).
-    __syncthreads();     // everyone is done reading At
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) At[c0 + j][4 * ty + r] = (c0 + j < nb) ? acc[r][j] : 0.f;
-    for (int e = t; e < (TB - nb) * TB; e += PA_THREADS) Bn[nb + e / TB][e % TB] = 0.f;
-    const bool staged2 = __syncthreads_and(stage_block_wait(bar + 1, 0) ? 1 : 0) != 0;
-    if (!staged2) {
-      if (t == 0) report_status(status, SP_ERR_TIMEOUT, (int32_t)blockIdx.x, 12);
-      return;
-    }
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[r][j] = 0.f;
-#pragma unroll 8
-    for (int k = 0; k < TB; ++k) {
-      const float4 a0 = *reinterpret_cast<const float4*>(&At[k][4 * ty]);
-      const float4 l0 = *reinterpret_cast<const float4*>(&Bn[k][4 * tx]);
-      const float av[4] = {a0.x, a0.y, a0.z, a0.w};
-      const float lv[4] = {l0.x, l0.y, l0.z, l0.w};
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[r][j] = fmaf(av[r], lv[j], acc[r][j]);
-    }
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int64_t gi = r0 + 4 * ty + r;
-      if (gi >= rows) continue;
-      float* dst = near.Xn + gi * ldx + c0;      // 16-byte aligned: the launcher checks ldx and the base
-      asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst), "f"(-acc[r][0]), "f"(-acc[r][1]),
-                   "f"(-acc[r][2]), "f"(-acc[r][3])
-                   : "memory");
-    }
-  }
+template <bool TRANS, int R>
+cudaError_t launch_panel_rows(float* X, int64_t ldx, int64_t rows, int nb, const float* dinv, __nv_bfloat16* S, int64_t lds,
+                              int64_t s_seg, bool write_f32, int32_t* status, cudaStream_t stream, PanelNear near,
+                              int batch, PanelBatch pb) {
+  static PerDeviceOnce attr_once;      // one per instantiation; the attribute belongs to the device's context
+  cudaError_t e = attr_once.run([] {
+    return cudaFuncSetAttribute(panel_apply_kernel<TRANS, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)pa_smem<R>(true));
+  });
+  if (e != cudaSuccess) return e;
+  const bool with_near = TRANS && near.L != nullptr;
+  panel_apply_kernel<TRANS, R><<<dim3((unsigned)ceil_div(rows, R), (unsigned)batch), RowTile<R>::THREADS,
+                                 pa_smem<R>(with_near), stream>>>(X, ldx, rows, nb, dinv, S, lds, s_seg, write_f32 ? 1 : 0, status, near,
+                                           skip_flag(), pb);
+  return cudaGetLastError();
+}
+
+// Rows per CTA: the fewest (8, 16, 32) for which `ctas` CTAs cover all rows, since every CTA stages the whole block of
+// inv(L) whatever its rows; 32 beyond.
+inline int panel_rows(int64_t rows, int batch, int64_t ctas) {
+  return ceil_div(rows, (int64_t)8) * batch <= ctas ? 8 : ceil_div(rows, (int64_t)16) * batch <= ctas ? 16 : 32;
 }
 
 template <bool TRANS>
 cudaError_t launch_panel_apply(float* X, int64_t ldx, int64_t rows, int nb, const float* dinv, __nv_bfloat16* S,
                                int64_t lds, int64_t s_seg, bool write_f32, int32_t* status, cudaStream_t stream,
-                               PanelNear near = PanelNear{nullptr, 0, nullptr}, int batch = 1,
-                               PanelBatch pb = PanelBatch{}) {
-  static PerDeviceOnce attr_once;      // one per instantiation; the attribute belongs to the device's context
-  {
-    cudaError_t e = attr_once.run([] {
-      return cudaFuncSetAttribute(panel_apply_kernel<TRANS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)PA_SMEM_NEAR);
-    });
-    if (e != cudaSuccess) return e;
-  }
+                               PanelNear near = kNoNear, int batch = 1, PanelBatch pb = PanelBatch{}, int per_cta = 0) {
   if (rows <= 0) return cudaSuccess;
   count_launch();
   const bool with_near = TRANS && near.L != nullptr;
   ProfScope prof(PK_PANEL_APPLY, (with_near ? 4.0 : 2.0) * (double)rows * TB * TB, 0.0, stream);
-  panel_apply_kernel<TRANS><<<dim3((unsigned)ceil_div(rows, PA_ROWS), (unsigned)batch), PA_THREADS,
-                              with_near ? PA_SMEM_NEAR : PA_SMEM, stream>>>(
-      X, ldx, rows, nb, dinv, S, lds, s_seg, write_f32 ? 1 : 0, status, near, skip_flag(), pb);
-  return cudaGetLastError();
+  if (per_cta == 0) per_cta = panel_rows(rows, batch, sm_count());
+  if (per_cta == 8)
+    return launch_panel_rows<TRANS, 8>(X, ldx, rows, nb, dinv, S, lds, s_seg, write_f32, status, stream, near, batch, pb);
+  if (per_cta == 16)
+    return launch_panel_rows<TRANS, 16>(X, ldx, rows, nb, dinv, S, lds, s_seg, write_f32, status, stream, near, batch, pb);
+  return launch_panel_rows<TRANS, 32>(X, ldx, rows, nb, dinv, S, lds, s_seg, write_f32, status, stream, near, batch, pb);
 }
 
 // The six kept part products of two three-part operands: A parts (hi, hi, mid, hi, lo, mid) against B parts
@@ -298,8 +317,8 @@ cudaError_t launch_panel_apply(float* X, int64_t ldx, int64_t rows, int nb, cons
 // with A21 = A[next block rows, block k columns] and A22 = A[next block, next block] as the trailing updates up to
 // step k - 1 left them.  One cluster of 8 CTAs, 16 rows each: every CTA forms its rows of Lm, publishes them
 // (transposed, in global scratch LmT[c][row]), the cluster meets, and every CTA forms its rows of S from all of Lm.
-constexpr int NM_ROWS = 16, NM_THREADS = 256, NM_APAD = NM_ROWS + 4, NM_CTAS = TB / NM_ROWS;
-constexpr size_t NM_SMEM = ((size_t)TB * TB + (size_t)TB * NM_APAD) * sizeof(float) + 16;
+constexpr int NM_ROWS = 16, NM_THREADS = RowTile<NM_ROWS>::THREADS, NM_CTAS = TB / NM_ROWS;
+constexpr size_t NM_SMEM = ((size_t)TB * TB + (size_t)TB * RowTile<NM_ROWS>::AP) * sizeof(float) + 16;
 static_assert(NM_CTAS == 8, "one portable cluster covers the block");
 
 __device__ __forceinline__ void cluster_meet() {
@@ -314,90 +333,76 @@ __device__ __forceinline__ void next_diag_body(const float* __restrict__ A21, co
                                                int64_t lda, int nb2, const float* __restrict__ dinv, float* LmT,
                                                float* S, int32_t* status) {
   extern __shared__ __align__(128) float nm_smem[];
-  float (*Lt)[TB] = reinterpret_cast<float (*)[TB]>(nm_smem);                       // Lt[k][c]
-  float (*At)[NM_APAD] = reinterpret_cast<float (*)[NM_APAD]>(nm_smem + TB * TB);   // At[k][row]
-  uint64_t* bar = reinterpret_cast<uint64_t*>(nm_smem + TB * TB + TB * NM_APAD);
+  using Tile = RowTile<NM_ROWS>;
+  constexpr int AP = Tile::AP;
+  float* Lt = nm_smem;                   // Lt[k][c]
+  float* At = nm_smem + TB * TB;         // At[k][row]
+  uint64_t* bar = reinterpret_cast<uint64_t*>(At + TB * AP);
   const int t = threadIdx.x;
   const int i0 = (int)blockIdx.x * NM_ROWS;
-  const int tx = t & 31, ty = t >> 5;   // columns 4 tx .. 4 tx + 3; rows 2 ty, 2 ty + 1
-  float acc[2][4];
+  const int c0 = Tile::col(t), ir = Tile::row0(t);      // columns c0 .. c0 + 3 of rows i0 + ir .. + RT - 1
+  float4 out[Tile::RT];
   if (MODE != 2) {
     // ---- stage 1: rows i0 .. i0 + 15 of Lm; Lt[k][c] = inv(L)[c][k] comes in by bulk copies
     if (t == 0) stage_bar_init(bar);
     __syncthreads();
-    if (t == 0) stage_block_issue(nm_smem, dinv + TB * TB, bar);
-    for (int e = t; e < NM_ROWS * TB; e += NM_THREADS) {
-      const int i = e / TB, k = e % TB;
-      At[k][i] = (i0 + i < nb2) ? A21[(int64_t)(i0 + i) * lda + k] : 0.f;
+    if (t == 0) stage_block_issue(Lt, dinv + TB * TB, bar);
+#pragma unroll
+    for (int q = 0; q < Tile::RT; ++q) {
+      const int i = i0 + ir + q;
+      float v[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) v[j] = i < nb2 ? A21[(int64_t)i * lda + c0 + j] : 0.f;
+      out[q] = make_float4(v[0], v[1], v[2], v[3]);
     }
+    Tile::store(At, out);
+  }
+  // this thread's entries of A22
+  float4 base[Tile::RT];
+  if (MODE != 1) {
+#pragma unroll
+    for (int q = 0; q < Tile::RT; ++q) {
+      const int i = i0 + ir + q;
+      float v[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) v[j] = (i < nb2 && c0 + j <= i) ? A22[(int64_t)i * lda + c0 + j] : 0.f;
+      base[q] = make_float4(v[0], v[1], v[2], v[3]);
+    }
+  }
+  if (MODE != 2) {
     const bool staged = __syncthreads_and(stage_block_wait(bar, 0) ? 1 : 0) != 0;
     if (!staged && t == 0) report_status(status, SP_ERR_TIMEOUT, (int32_t)blockIdx.x, 11);
     // (a CTA whose copies did not land still goes on to the barrier below; its rows are then wrong and the status
     //  says so)
-#pragma unroll
-    for (int r = 0; r < 2; ++r)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[r][j] = 0.f;
-#pragma unroll 8
-    for (int k = 0; k < TB; ++k) {
-      const float2 a = *reinterpret_cast<const float2*>(&At[k][2 * ty]);
-      const float4 l0 = *reinterpret_cast<const float4*>(&Lt[k][4 * tx]);
-      const float av[2] = {a.x, a.y};
-      const float lv[4] = {l0.x, l0.y, l0.z, l0.w};
-#pragma unroll
-      for (int r = 0; r < 2; ++r)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[r][j] = fmaf(av[r], lv[j], acc[r][j]);
-    }
+    Tile::product(At, Lt, out);
     __syncthreads();   // everyone is done with At and Lt
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int c = 4 * tx + j;
-      const float2 v = make_float2(acc[0][j], acc[1][j]);
-      *reinterpret_cast<float2*>(&At[c][2 * ty]) = v;                              // own rows, left operand of stage 2
-      *reinterpret_cast<float2*>(&LmT[(int64_t)c * TB + i0 + 2 * ty]) = v;         // for the other CTAs
-    }
+    Tile::store(At, out);                          // own rows, left operand of stage 2
+    Tile::store_transposed(LmT + i0, TB, out);     // for the other CTAs
     if (MODE == 1) return;
     cluster_meet();
   }
   // ---- stage 2: rows i0 .. i0 + 15 of S; Lt[c][j] = Lm[j][c]
   {
     const float4* src = reinterpret_cast<const float4*>(LmT);
-    float4* dst = reinterpret_cast<float4*>(nm_smem);
-#pragma unroll
+    float4* dst = reinterpret_cast<float4*>(Lt);
+#pragma unroll 16
     for (int q = 0; q < TB * TB / 4 / NM_THREADS; ++q) dst[t + q * NM_THREADS] = __ldcg(src + t + q * NM_THREADS);
     if (MODE == 2)     // own rows of Lm come from the first launch
       for (int e = t; e < NM_ROWS * TB; e += NM_THREADS) {
         const int c = e / NM_ROWS, i = e % NM_ROWS;
-        At[c][i] = __ldcg(&LmT[(int64_t)c * TB + i0 + i]);
+        At[c * AP + i] = __ldcg(&LmT[(int64_t)c * TB + i0 + i]);
       }
   }
   __syncthreads();
+  Tile::product(At, Lt, out);
 #pragma unroll
-  for (int r = 0; r < 2; ++r)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[r][j] = 0.f;
-#pragma unroll 8
-  for (int k = 0; k < TB; ++k) {
-    const float2 a = *reinterpret_cast<const float2*>(&At[k][2 * ty]);
-    const float4 l0 = *reinterpret_cast<const float4*>(&Lt[k][4 * tx]);
-    const float av[2] = {a.x, a.y};
-    const float lv[4] = {l0.x, l0.y, l0.z, l0.w};
-#pragma unroll
-    for (int r = 0; r < 2; ++r)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[r][j] = fmaf(av[r], lv[j], acc[r][j]);
-  }
-#pragma unroll
-  for (int r = 0; r < 2; ++r) {
-    const int i = i0 + 2 * ty + r;
+  for (int q = 0; q < Tile::RT; ++q) {
+    const int i = i0 + ir + q;
+    const float d[4] = {base[q].x - out[q].x, base[q].y - out[q].y, base[q].z - out[q].z, base[q].w - out[q].w};
     float v[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int c = 4 * tx + j;
-      v[j] = (i < nb2 && c <= i) ? A22[(int64_t)i * lda + c] - acc[r][j] : 0.f;
-    }
-    *reinterpret_cast<float4*>(&S[i * TB + 4 * tx]) = make_float4(v[0], v[1], v[2], v[3]);
+    for (int j = 0; j < 4; ++j) v[j] = (i < nb2 && c0 + j <= i) ? d[j] : 0.f;
+    *reinterpret_cast<float4*>(&S[i * TB + c0]) = make_float4(v[0], v[1], v[2], v[3]);
   }
 }
 
@@ -670,11 +675,23 @@ sp_status potrs_right_tc(float* X, int64_t m, int64_t n, int64_t ldx, const void
   // Reproducible mode: the far update of a step (assisting stream) and the next step's near update would add into the
   // same columns in an order that depends on timing; on one stream every column receives its updates in step order.
   if (reproducible_mode()) assist = nullptr;
-  // Backward sweep: the update of the next block column can ride in the panel kernel (fp32, from the fp32 factor)
+  // Backward sweep: the update by the previous block column can ride in the panel kernel (fp32, from the fp32 factor)
   // when the factor's rows are 16-byte aligned too.
   // (its 144 KB of shared memory allow one CTA per SM: only while all row blocks fit in one wave)
   const bool fuse_near = Lf != nullptr && x_al16 && (ldl % 4 == 0) && ((reinterpret_cast<uintptr_t>(Lf) & 15u) == 0) &&
-                         ceil_div(m, (int64_t)PA_ROWS) <= 148;
+                         ceil_div(m, (int64_t)32) <= 148;
+  // Backward sweep: a panel runs beside the far update of the step before, whose CTAs take a whole SM each; one that has to
+  // wait for SMs lengthens the chain by the update's time.  So the panel gets half of the SMs and the update the rest,
+  // unless the update has so many tiles that the two one after the other, each with all SMs, are shorter.  Measured on the
+  // step's kernels: 8 us and 6.2 us for every round of tiles for the update, 12 us for the panel.
+  const int64_t sms = sm_count();
+  const int rows_beside = panel_rows(m, 1, sms / 2);
+  const int64_t beside_pairs = (sms - ceil_div(m, (int64_t)rows_beside)) / 2;
+  auto tiles_of = [&](int64_t w) { return ceil_div(m, (int64_t)256) * ceil_div(w, (int64_t)256); };
+  auto runs_beside = [&](int64_t w) {
+    if (beside_pairs < 1) return false;
+    return 6.2 * (double)ceil_div(tiles_of(w), beside_pairs) < 12.0 + 6.2 * (double)ceil_div(tiles_of(w), sms / 2);
+  };
   bool rec[2] = {false, false};
   auto run_sweep = [&](bool forward) -> sp_status {
     for (int64_t step = 0; step < nblk; ++step) {
@@ -686,13 +703,17 @@ sp_status potrs_right_tc(float* X, int64_t m, int64_t n, int64_t ldx, const void
       if (assist && rec[step & 1]) SP_CUDA_OK(cudaStreamWaitEvent(stream, assist->rest_done[step & 1], 0));
       // columns still to be updated: [lo, hi)
       const int64_t lo = forward ? j0 + nb : 0, hi = forward ? n : j0;
-      // backward: the near columns are the whole block before j (TB wide)
-      const bool near_in_panel = !forward && fuse_near && hi > lo;
-      PanelNear pn{nullptr, 0, nullptr};
-      if (near_in_panel) pn = PanelNear{Lf + j0 * ldl + (hi - TB), ldl, X + (hi - TB)};
+      // backward: the near columns are the whole block before j (TB wide), which the next panel updates itself
+      const bool near_in_panel = !forward && fuse_near;
+      PanelNear pn = kNoNear;
+      if (near_in_panel && j0 + nb < n) {
+        const int64_t p0 = j0 + nb;
+        pn = PanelNear{Lf + p0 * ldl + j0, ldl, X + p0, (int)((n - p0 < TB) ? n - p0 : TB)};
+      }
       cudaError_t e = forward ? launch_panel_apply<false>(X + j0, ldx, m, nb, dj, Xcur, lds, TB, true, status_dev, stream)
                               : launch_panel_apply<true>(X + j0, ldx, m, nb, dj, Xcur, lds, TB, true, status_dev, stream,
-                                                         pn);
+                                                         pn, 1, PanelBatch{},
+                                                         near_in_panel && assist && runs_beside(j0) ? rows_beside : 0);
       if (e != cudaSuccess) return SP_ERR_CUDA;
       if (hi <= lo) break;
       if (assist) SP_CUDA_OK(cudaEventRecord(assist->panel_done, stream));
@@ -732,7 +753,8 @@ sp_status potrs_right_tc(float* X, int64_t m, int64_t n, int64_t ldx, const void
         }
         float* Xc = X + c0;
         sp_status stt = gemm_tc(m, w, TB, -1.f, ta, tb, 1.f, Operand{Xc, SP_F32, ldx, 1}, OutOperand{Xc, SP_F32, ldx},
-                                false, status_dev, st_run, &sg, 2.0 * (double)m * (double)w * (double)nb);
+                                false, status_dev, st_run, &sg, 2.0 * (double)m * (double)w * (double)nb,
+                                on_assist && near_in_panel && runs_beside(w) && tiles_of(w) > beside_pairs ? (int)beside_pairs : 0);
         if (stt != SP_OK) return stt;
         if (on_assist) {
           SP_CUDA_OK(cudaEventRecord(assist->rest_done[step & 1], st_run));
@@ -795,7 +817,7 @@ sp_status potrf_potrs_tc_batched(float* A, int64_t n, int64_t m, int batch, int6
     PanelBatch pb;
     pb.x = a_bs; pb.dinv = d_bs; pb.s = p_bs;
     if (launch_panel_apply<false>(A + (k0 + TB) * lda + k0, lda, prow, TB, dk, P + (k0 + TB) * ldp + k0, ldp, np, true,
-                                  status_dev, stream, PanelNear{nullptr, 0, nullptr}, batch, pb) != cudaSuccess)
+                                  status_dev, stream, kNoNear, batch, pb) != cudaSuccess)
       return SP_ERR_CUDA;
     if (rem <= 0) break;
     TcOperand ta{P + (k0 + TB) * ldp, ldp, true}, tb{P + (k0 + TB) * ldp, ldp, true};
@@ -817,22 +839,21 @@ sp_status potrf_potrs_tc_batched(float* A, int64_t n, int64_t m, int batch, int6
   // ---- backward sweep W L = Y on the appended rows, block columns right to left
   float* X = A + n * lda;                       // [m, n] per system
   const int64_t lds = 3 * TB, xs_bs = 2 * m * lds;
-  const bool fuse_near = ceil_div(m, (int64_t)PA_ROWS) * batch <= 148;
+  const bool fuse_near = ceil_div(m, (int64_t)32) * batch <= 148;
   TcBatch bs = bt;
   bs.a_s0 = bs.a_s1 = xs_bs;
   for (int64_t step = 0; step < nblk; ++step) {
     const int64_t jb = nblk - 1 - step, j0 = jb * TB;
     const float* dj = dinv + jb * 2 * TB * TB;
     __nv_bfloat16* Xcur = Xs + (step & 1) * m * lds;
-    const bool near_in_panel = fuse_near && j0 > 0;
-    PanelNear pn{nullptr, 0, nullptr};
-    if (near_in_panel) pn = PanelNear{A + j0 * lda + (j0 - TB), lda, X + (j0 - TB)};
+    PanelNear pn = kNoNear;
+    if (fuse_near && step > 0) pn = PanelNear{A + (j0 + TB) * lda + j0, lda, X + j0 + TB, TB};
     PanelBatch pb;
     pb.x = a_bs; pb.dinv = d_bs; pb.s = xs_bs; pb.near_l = a_bs;
     if (launch_panel_apply<true>(X + j0, lda, m, TB, dj, Xcur, lds, TB, true, status_dev, stream, pn, batch, pb) !=
         cudaSuccess)
       return SP_ERR_CUDA;
-    const int64_t w = near_in_panel ? j0 - TB : j0;     // columns still to be updated by a product: [0, w)
+    const int64_t w = fuse_near ? j0 - TB : j0;     // columns still to be updated by a product: [0, w)
     if (w <= 0) continue;
     TcOperand ta{Xcur, lds, true}, tb{P + j0 * ldp, ldp, false};
     ta.kext = lds;
