@@ -1196,7 +1196,7 @@ static sp_status admm_step_impl(const sp_ffn_module* m, sp_ffn_state* st, const 
   }
   if (decay) {
     // the accumulators in channel order for the next step's weight phase and for the caller
-    CU(unpermute_gram(st->G_A_perm, st->decay_tag + 8, n, st->G_A, s));
+    CU(unpermute_gram(st->G_A_perm, st->decay_tag + 8, n, st->G_A, p.perm, s));     // (p.perm is free by now)
     CU(unpermute_cols(st->R2_perm, st->decay_tag + 8, d, n, st->R2, s));
     if (decay_z) CU(unpermute_rows(st->R1_perm, st->decay_tag + 8, n, d, st->R1, s));
   } else {

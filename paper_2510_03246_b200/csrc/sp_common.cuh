@@ -81,6 +81,51 @@ int sm_count();
 __host__ __device__ __forceinline__ int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 __host__ __device__ __forceinline__ size_t align_up(size_t a, size_t b) { return (a + b - 1) / b * b; }
 
+// Shape of the kernels that move whole matrices: blocks of 256 threads, gridDim.x strips of 1024 columns (a thread has
+// four, 256 apart, so that every access of a warp is one line), gridDim.y walks the rows.  No index is divided, and what
+// depends on the column alone is read once per block.
+constexpr int kStripThreads = 256, kStripPer = 4;
+inline dim3 strip_grid(int64_t rows, int64_t cols) {
+  const int64_t gx = ceil_div(cols, (int64_t)kStripThreads * kStripPer);
+  int64_t gy = ceil_div((int64_t)sm_count() * 8, gx);
+  if (gy > rows) gy = rows;
+  return dim3((unsigned)(gx > 0 ? gx : 1), (unsigned)(gy > 0 ? (gy < 65535 ? gy : 65535) : 1));
+}
+inline unsigned lower_tiles(int64_t n, int64_t tile) {
+  const int64_t nt = ceil_div(n, tile);
+  return (unsigned)(nt * (nt + 1) / 2);
+}
+#ifdef __CUDACC__
+// f(i, j, q) for the rows of this block and this thread's columns j, q = 0 .. 3 their number
+template <typename F>
+__device__ __forceinline__ void for_strip(int64_t rows, int64_t cols, F&& f) {
+  const int64_t c0 = (int64_t)blockIdx.x * (kStripThreads * kStripPer) + threadIdx.x;
+#pragma unroll 2
+  for (int64_t i = blockIdx.y; i < rows; i += gridDim.y)
+#pragma unroll
+    for (int q = 0; q < kStripPer; ++q) {
+      const int64_t j = c0 + q * kStripThreads;
+      if (j < cols) f(i, j, q);
+    }
+}
+// tile (row block y, column block x <= y) of a lower triangle of tiles counted row by row
+__device__ __forceinline__ void lower_tile(unsigned t, unsigned& y, unsigned& x) {
+  y = (unsigned)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
+  while ((unsigned long long)(y + 1) * (y + 2) / 2 <= t) ++y;
+  while ((unsigned long long)y * (y + 1) / 2 > t) --y;
+  x = t - (unsigned)((unsigned long long)y * (y + 1) / 2);
+}
+// idx[j] (idx == nullptr: j) of this thread's columns
+__device__ __forceinline__ void strip_index(const int32_t* idx, int64_t cols, int64_t (&at)[kStripPer]) {
+  const int64_t c0 = (int64_t)blockIdx.x * (kStripThreads * kStripPer) + threadIdx.x;
+#pragma unroll
+  for (int q = 0; q < kStripPer; ++q) {
+    const int64_t j = c0 + q * kStripThreads;
+    at[q] = j < cols ? (idx ? (int64_t)idx[j] : j) : 0;
+  }
+}
+#endif
+
 inline size_t dtype_size(int32_t dt) { return dt == SP_BF16 ? 2 : (dt == SP_F64 ? 8 : 4); }
 
 // A strided operand of the SIMT GEMM: element (i, k) lives at ptr[i * s0 + k * s1].
@@ -185,7 +230,6 @@ struct SolveAssist {
 sp_status potrf_lower_tc(float* A, int64_t n, int64_t lda, float* dinv, void* P, int32_t* status_dev,
                          cudaStream_t stream, const SolveAssist* assist = nullptr, int64_t m_extra = 0,
                          bool split_lookahead = false);   // lookahead kernel as two launches without a cluster
-// Xs holds TWO buffers of [m, 3 * kCholTcNB] bf16.
 // forward_done: X already holds the solution of the forward system (it rode along with the factorisation).
 // Lf / ldl (optional): the fp32 factor potrf_lower_tc left in A; with it the backward sweep updates a block column by
 // the one before it inside the panel kernel instead of by a GEMM of its own.
@@ -387,7 +431,8 @@ cudaError_t mask_count_check(const uint8_t* mask, int64_t n, int64_t k, int32_t*
 cudaError_t scale_block(float* C, int64_t ld, int64_t rows, int64_t cols, const int32_t* f_bits, int power,
                         cudaStream_t stream);
 // G[perm[i], perm[j]] = G[perm[j], perm[i]] = Gp[i, j] for i >= j (Gp: lower triangle in permuted order)
-cudaError_t unpermute_gram(const float* Gp, const int32_t* perm, int64_t n, float* G, cudaStream_t stream);
+cudaError_t unpermute_gram(const float* Gp, const int32_t* perm, int64_t n, float* G, int32_t* inv,
+                           cudaStream_t stream);
 // R[r, perm[j]] = Rp[r, j]
 cudaError_t unpermute_cols(const float* Rp, const int32_t* perm, int64_t rows, int64_t n, float* R,
                            cudaStream_t stream);

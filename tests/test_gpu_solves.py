@@ -82,6 +82,30 @@ def test_tensor_core_ridge_solve_at_block_edges(n, m):
     assert status[:2].tolist() == [6, i]      # SP_ERR_NOT_SPD and the pivot
 
 
+@pytest.mark.parametrize("n,rows", [(4, 5), (64, 64), (72, 33), (200, 130), (1096, 70)])
+def test_ordered_accumulators_come_back_in_channel_order(n, rows):
+    """A module whose token pass works with the kept channels first: G_A (both triangles), R1 and R2 in channel order
+    equal the products over the tokens, at the edges of the 32 x 32 tiles and of the 1024-column strips."""
+    api = _api()
+    g = torch.Generator(device="cuda").manual_seed(n)
+    d, N, k = 64, 8 * rows, max(1, n // 3)
+    mod = api.FfnModule(torch.randn(N, d, generator=g, device="cuda").bfloat16(),
+                        torch.randn(n, d, generator=g, device="cuda") * 0.1,
+                        torch.randn(d, n, generator=g, device="cuda") * 0.1, overlap_k=k)
+    mod.sp_ffn_init()
+    mod.mask.zero_()
+    mod.mask[torch.randperm(n, generator=g, device="cuda")[:k]] = 1
+    p = api.AdmmParams(k_keep=k, rho=0.1, reselect_mask=False, skip_scores=True)
+    for _ in range(2):
+        mod.sp_admm_step(p)
+    mod.check_status()
+    assert torch.equal(mod.G_A, mod.G_A.T)
+    want = mod.Z.double().T @ mod.X.double()
+    # (Z enters the product as bf16: one rounding of 2^-9 per term)
+    assert float((mod.R1.double() - want).abs().max()) < 2.0 ** -9 * float((mod.Z.double().abs().T @ mod.X.double().abs()).max())
+    assert torch.allclose(mod.G_A.diagonal(), mod.G_A_perm.diagonal()[torch.argsort(mod.decay_tag[8:8 + n])])
+
+
 @pytest.mark.parametrize("d", [8, 64, 72, 136, 520, 1096])
 def test_cached_input_inverse_at_block_edges(d):
     api = _api()
