@@ -128,7 +128,7 @@ SolveBufs carve_solve(Carver& c, int64_t nmax, int64_t mmax, size_t tsize) {
     const size_t np = (size_t)chol_tc_pad(nmax);
     b.P = c.take_bytes((np + (size_t)mmax) * 3 * np * 2);
     const size_t rows = (size_t)(nmax > mmax ? nmax : mmax);   // either dimension may be the right-hand-side count
-    b.Xs = c.take_bytes(2 * rows * 3 * kCholTcNB * 2);
+    b.Xs = c.take_bytes((size_t)chol_tc_xs_elems(nmax, (int64_t)rows) * 2);
   }
   return b;
 }

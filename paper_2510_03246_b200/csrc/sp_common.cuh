@@ -210,9 +210,17 @@ constexpr int kCholNB = 64;
 // fp32 factorisation / solves with tensor-core trailing updates (sp_linalg_tc.cu).  Panels are kCholTcNB wide.
 //   dinv: ceil(n / kCholTcNB) blocks of 2 * kCholTcNB^2 floats (inverse diagonal blocks and their transposes)
 //   P   : bf16 [chol_tc_pad(n), 3 * chol_tc_pad(n)] — the factor below its diagonal blocks as three bf16 parts
-//   Xs  : 2 x bf16 [m, 3 * kCholTcNB] — the current block column of the right-hand sides as three bf16 parts
+//   Xs  : chol_tc_xs_elems(n, m) bf16 — the current block columns of the right-hand sides as three bf16 parts
 constexpr int kCholTcNB = 128;
+// Two-level blocking of the factorisation and of the backward sweep: systems of at least kOuterMinN unknowns, outer blocks
+// of kOuterBlocks diagonal blocks.
+constexpr int64_t kOuterMinN = 12288;
+constexpr int64_t kOuterBlocks = 4;
 int64_t chol_tc_pad(int64_t n);
+// two buffers of one block column, or one of an outer block
+inline int64_t chol_tc_xs_elems(int64_t n, int64_t m) {
+  return m * 3 * kCholTcNB * (n >= kOuterMinN ? kOuterBlocks : 2);
+}
 // Optional second stream (with three events) that carries the part of each step that the next step's first kernel
 // does not wait for: the far part of a solve step's update; the panel and trailing update of a factorisation step.
 struct SolveAssist {

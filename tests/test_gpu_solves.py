@@ -82,6 +82,27 @@ def test_tensor_core_ridge_solve_at_block_edges(n, m):
     assert status[:2].tolist() == [6, i]      # SP_ERR_NOT_SPD and the pivot
 
 
+@pytest.mark.parametrize("n,m", [(12288, 40), (12300, 200), (12420, 4800)])
+def test_two_level_sweep_of_a_large_system(n, m):
+    """Outer blocks of 512 columns, the last of them ragged; few right-hand sides (a block column pulls the update of the
+    one before it) and more than one wave of panels holds (it does not)."""
+    api = _api()
+    g = torch.Generator(device="cuda").manual_seed(n)
+    X = torch.randn(n + 64, n, generator=g, device="cuda")
+    G = X.T @ X
+    G = torch.tril(G) + torch.tril(G, -1).T
+    del X
+    R = torch.randn(m, n, generator=g, device="cuda")
+    status = api.new_status(G.device)
+    got = api.sp_ridge_solve(R, G, 0.1, True, status=status)
+    assert int(status[0]) == 0
+    # residual of the solution in fp64, relative to its terms: a few roundings of 2^-24 per block column (n / 128)
+    H = G.double()
+    H.diagonal().add_(0.1 * H.diagonal().mean())
+    res = got.double() @ H - R.double()
+    assert float(res.abs().max()) < (n // 128) * 2.0 ** -24 * float((got.double().abs() @ H.abs()).max())
+
+
 @pytest.mark.parametrize("n,rows", [(4, 5), (64, 64), (72, 33), (200, 130), (1096, 70)])
 def test_ordered_accumulators_come_back_in_channel_order(n, rows):
     """A module whose token pass works with the kept channels first: G_A (both triangles), R1 and R2 in channel order
