@@ -384,7 +384,7 @@ cudaError_t mha_softmax_rows(float* S, int64_t pairs, int T, bool causal, void* 
 // P <- P - eta_pair (-2 alpha G1 + 2 beta (P - Phi)); Pb: optional bf16 copy of the new P (hi / lo planes as above)
 cudaError_t mha_p_update(float* P, const float* Phi, const float* G1, const float* eta, int64_t pairs, int T,
                          double alpha, double beta, void* Pb, int64_t plane, cudaStream_t stream);
-// S (logits) <- dS = 2 beta Phi (E - rowsum(E Phi)), Phi = softmax(S), E = Phi - P; dSb: optional bf16 copy
+// dS = 2 beta Phi (E - rowsum(E Phi)), Phi = softmax(S), E = Phi - P, as bf16 to dSb or (dSb == nullptr) in place of S
 cudaError_t mha_softmax_backward_rows(float* S, const float* P, int64_t pairs, int T, bool causal, double beta,
                                       void* dSb, cudaStream_t stream);
 // per-pair step sizes from the squared norms of the [T, d_h] slices of x (and y): mode 0: 1 / (2 (alpha s + beta)),

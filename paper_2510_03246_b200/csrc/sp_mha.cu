@@ -20,8 +20,57 @@ __device__ __forceinline__ float warp_sum(float v) {
 
 constexpr int kRowWarps = 8;
 
+// A row of logits in registers, lane l holding the keys l, l + 32, ...: NV of them cover rows of up to 32 NV keys (NV = 0: any
+// length, the row is read again instead).  The three passes over a row (maximum, sum, values) then cost one read and one
+// exponential per entry (T = 128: 9.5 -> 5.3 us for the backward).  Above 256 keys the registers cost more warps than the
+// rereads, which the L1 answers (T = 1024: 717 us in registers).
+template <int NV>
+struct RowVals {
+  float e[NV > 0 ? NV : 1];      // exp(s - max) once sum() has run
+  float mx;
+  __device__ __forceinline__ float at(const float* row, int lane, int i) const {
+    if constexpr (NV > 0) return e[i];
+    else return __expf(row[lane + 32 * i] - mx);
+  }
+  // loads the row and returns 1 / sum_u exp(s_u - max)
+  __device__ __forceinline__ float prepare(const float* row, int lane, int lim) {
+    mx = -INFINITY;
+    float sum = 0.f;
+    if constexpr (NV > 0) {
+#pragma unroll
+      for (int i = 0; i < NV; ++i) e[i] = lane + 32 * i < lim ? row[lane + 32 * i] : -INFINITY;
+#pragma unroll
+      for (int i = 0; i < NV; ++i) mx = fmaxf(mx, e[i]);
+      mx = warp_max(mx);
+#pragma unroll
+      for (int i = 0; i < NV; ++i)
+        if (lane + 32 * i < lim) {
+          e[i] = __expf(e[i] - mx);
+          sum += e[i];
+        }
+    } else {
+      for (int u = lane; u < lim; u += 32) mx = fmaxf(mx, row[u]);
+      mx = warp_max(mx);
+      for (int u = lane; u < lim; u += 32) sum += __expf(row[u] - mx);
+    }
+    return 1.f / warp_sum(sum);
+  }
+};
+// f(u, i) for the entries u = lane + 32 i < n
+template <int NV, typename F>
+__device__ __forceinline__ void for_row(int lane, int n, F&& f) {
+  if constexpr (NV > 0) {
+#pragma unroll
+    for (int i = 0; i < NV; ++i)
+      if (lane + 32 * i < n) f(lane + 32 * i, i);
+  } else {
+    for (int u = lane, i = 0; u < n; u += 32, ++i) f(u, i);
+  }
+}
+
 // S[row, :] <- softmax over the keys of the row (in place).  rows = pairs * T; row r belongs to query t = r % T; with
 // `causal` keys u > t get probability 0.  Optional bf16 copy.
+template <int NV>
 __global__ void __launch_bounds__(kRowWarps * 32) softmax_rows_kernel(float* __restrict__ S, int64_t rows, int T,
                                                                       int causal, __nv_bfloat16* __restrict__ Sb,
                                                                       int64_t plane) {
@@ -30,46 +79,56 @@ __global__ void __launch_bounds__(kRowWarps * 32) softmax_rows_kernel(float* __r
   if (r >= rows) return;
   float* row = S + r * T;
   const int lim = causal ? (int)(r % T) + 1 : T;
-  float mx = -INFINITY;
-  for (int u = lane; u < lim; u += 32) mx = fmaxf(mx, row[u]);
-  mx = warp_max(mx);
-  float sum = 0.f;
-  for (int u = lane; u < lim; u += 32) sum += __expf(row[u] - mx);
-  sum = warp_sum(sum);
-  const float inv = 1.f / sum;
-  for (int u = lane; u < T; u += 32) {
-    const float v = u < lim ? __expf(row[u] - mx) * inv : 0.f;
-    row[u] = v;
+  RowVals<NV> v;
+  const float inv = v.prepare(row, lane, lim);
+  for_row<NV>(lane, T, [&](int u, int i) {
+    const float p = u < lim ? v.at(row, lane, i) * inv : 0.f;
+    row[u] = p;
     if (Sb) {
-      const __nv_bfloat16 hi = __float2bfloat16_rn(v);
+      const __nv_bfloat16 hi = __float2bfloat16_rn(p);
       Sb[r * T + u] = hi;
-      if (plane > 0) Sb[plane + r * T + u] = __float2bfloat16_rn(v - __bfloat162float(hi));
+      if (plane > 0) Sb[plane + r * T + u] = __float2bfloat16_rn(p - __bfloat162float(hi));
     }
-  }
+  });
 }
 
 // Gradient step of Eq. (85) on the attention probabilities of every (sequence, head) pair:
 //   P <- P - eta_b (-2 alpha G1 + 2 beta (P - Phi)),  G1 = R V^T from the preceding product, eta_b per pair.
+// gridDim.y walks the pairs, a thread takes V neighbouring entries (V = 4: 16-byte accesses).
+template <int V>
 __global__ void __launch_bounds__(256) p_update_kernel(float* __restrict__ P, const float* __restrict__ Phi,
                                                        const float* __restrict__ G1, const float* __restrict__ eta,
-                                                       int64_t per_pair, int64_t total, float alpha, float beta,
+                                                       int64_t per_pair, int64_t pairs, float alpha, float beta,
                                                        __nv_bfloat16* __restrict__ Pb, int64_t plane) {
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    const float et = eta[e / per_pair];
-    const float p = P[e];
-    const float g = -2.f * alpha * G1[e] + 2.f * beta * (p - Phi[e]);
-    const float pn = p - et * g;
-    P[e] = pn;
-    if (Pb) {
-      const __nv_bfloat16 hi = __float2bfloat16_rn(pn);
-      Pb[e] = hi;
-      if (plane > 0) Pb[plane + e] = __float2bfloat16_rn(pn - __bfloat162float(hi));
+  struct __align__(4 * V) F { float v[V]; };
+  struct __align__(2 * V) H { __nv_bfloat16 v[V]; };
+  for (int64_t b = blockIdx.y; b < pairs; b += gridDim.y) {
+    const float et = eta[b];
+    for (int64_t i = ((int64_t)blockIdx.x * 256 + threadIdx.x) * V; i < per_pair; i += (int64_t)gridDim.x * 256 * V) {
+      const int64_t e = b * per_pair + i;
+      const F p = *reinterpret_cast<const F*>(P + e), ph = *reinterpret_cast<const F*>(Phi + e),
+              g1 = *reinterpret_cast<const F*>(G1 + e);
+      F pn;
+      H hi, lo;
+#pragma unroll
+      for (int q = 0; q < V; ++q) {
+        const float g = -2.f * alpha * g1.v[q] + 2.f * beta * (p.v[q] - ph.v[q]);
+        pn.v[q] = p.v[q] - et * g;
+        hi.v[q] = __float2bfloat16_rn(pn.v[q]);
+        lo.v[q] = __float2bfloat16_rn(pn.v[q] - __bfloat162float(hi.v[q]));
+      }
+      *reinterpret_cast<F*>(P + e) = pn;
+      if (Pb) {
+        *reinterpret_cast<H*>(Pb + e) = hi;
+        if (plane > 0) *reinterpret_cast<H*>(Pb + plane + e) = lo;
+      }
     }
   }
 }
 
 // Softmax and its backward for the softmax term of Eq. (87), one warp per row of logits S:
-//   Phi = softmax(S),  E = Phi - P,  dS = 2 beta Phi (E - sum_u E Phi)  -> fp32 in place of S and / or bf16 copy.
+//   Phi = softmax(S),  E = Phi - P,  dS = 2 beta Phi (E - sum_u E Phi)  -> as bf16 to dSb, or (dSb == nullptr) in place.
+template <int NV>
 __global__ void __launch_bounds__(kRowWarps * 32) softmax_backward_rows_kernel(float* __restrict__ S,
                                                                                const float* __restrict__ P,
                                                                                int64_t rows, int T, int causal,
@@ -81,28 +140,25 @@ __global__ void __launch_bounds__(kRowWarps * 32) softmax_backward_rows_kernel(f
   float* row = S + r * T;
   const float* prow = P + r * T;
   const int lim = causal ? (int)(r % T) + 1 : T;
-  float mx = -INFINITY;
-  for (int u = lane; u < lim; u += 32) mx = fmaxf(mx, row[u]);
-  mx = warp_max(mx);
-  float sum = 0.f;
-  for (int u = lane; u < lim; u += 32) sum += __expf(row[u] - mx);
-  sum = warp_sum(sum);
-  const float inv = 1.f / sum;
+  RowVals<NV> v;
+  const float inv = v.prepare(row, lane, lim);
+  float p[NV > 0 ? NV : 1];
   float dot = 0.f;        // sum_u E Phi (Phi = 0 beyond the causal limit)
-  for (int u = lane; u < lim; u += 32) {
-    const float ph = __expf(row[u] - mx) * inv;
-    dot = fmaf(ph - prow[u], ph, dot);
-  }
+  for_row<NV>(lane, lim, [&](int u, int i) {
+    const float ph = v.at(row, lane, i) * inv, pu = prow[u];
+    if constexpr (NV > 0) p[i] = pu;
+    dot = fmaf(ph - pu, ph, dot);
+  });
   dot = warp_sum(dot);
-  for (int u = lane; u < T; u += 32) {
-    float v = 0.f;
+  for_row<NV>(lane, T, [&](int u, int i) {
+    float g = 0.f;
     if (u < lim) {
-      const float ph = __expf(row[u] - mx) * inv;
-      v = 2.f * beta * ph * (ph - prow[u] - dot);
+      const float ph = v.at(row, lane, i) * inv;
+      g = 2.f * beta * ph * (ph - (NV > 0 ? p[NV > 0 ? i : 0] : prow[u]) - dot);
     }
-    row[u] = v;
-    if (dSb) dSb[r * T + u] = __float2bfloat16_rn(v);
-  }
+    if (dSb) dSb[r * T + u] = __float2bfloat16_rn(g);
+    else row[u] = g;
+  });
 }
 
 // Sum of squares of the [T, d_h] slice of every (sequence, head) pair of up to two token-major [tokens, d] tensors;
@@ -114,13 +170,22 @@ __global__ void __launch_bounds__(256) pair_sumsq_kernel(const float* __restrict
   const int64_t base = (int64_t)seq * T * ld + (int64_t)head * d_h;
   double acc = 0.0;
   const int total = T * d_h;
-  for (int e = threadIdx.x; e < total; e += 256) {
-    const int64_t o = base + (int64_t)(e / d_h) * ld + (e % d_h);
-    const float v = x[o];
-    acc += (double)v * v;
-    if (y) {
-      const float w = y[o];
-      acc += (double)w * w;
+  // eight entries in flight, added in order; a head width that divides 256 keeps a thread in its column
+  const bool one_col = 256 % d_h == 0;
+  const int64_t o0 = base + (int64_t)(threadIdx.x / d_h) * ld + threadIdx.x % d_h, step = (int64_t)(256 / d_h) * ld;
+  for (int e0 = threadIdx.x, j = 0; e0 < total; e0 += 8 * 256, j += 8) {
+    float v[8], w[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int e = e0 + q * 256;
+      const int64_t o = one_col ? o0 + (j + q) * step : base + (int64_t)(e / d_h) * ld + (e % d_h);
+      v[q] = e < total ? x[o] : 0.f;
+      w[q] = y && e < total ? y[o] : 0.f;
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      acc += (double)v[q] * v[q];
+      if (y) acc += (double)w[q] * w[q];
     }
   }
   sm[threadIdx.x] = acc;
@@ -144,31 +209,42 @@ __global__ void step_size_kernel(const double* __restrict__ s, int n, int mode, 
 
 // Gradient step of Eq. (87) on the projection outputs, token-major [tokens, d]:
 //   Z <- Z - eta_b (G + 2 alpha (Z - Tg)) for Z in {Zq, Zk}, b = (token / T) * H + column / d_h;
-// optional bf16 hi / lo planes of the new values (operands of the next logits product).
+// optional bf16 hi / lo planes of the new values (operands of the next logits product).  A thread takes V neighbouring
+// columns of one head (V = 4: 16-byte accesses).
+template <int V>
 __global__ void __launch_bounds__(256) z_update_kernel(float* __restrict__ Zq, float* __restrict__ Zk,
                                                        const float* __restrict__ Gq, const float* __restrict__ Gk,
                                                        const float* __restrict__ Tq, const float* __restrict__ Tk,
                                                        const float* __restrict__ eta, int64_t tokens, int d, int T,
                                                        int d_h, float alpha, __nv_bfloat16* __restrict__ Zqs,
                                                        __nv_bfloat16* __restrict__ Zks, int64_t plane) {
-  const int H = d / d_h;
-  const int64_t total = tokens * d;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t tok = e / d;
-    const int c = (int)(e % d);
-    const float et = eta[(tok / T) * H + c / d_h];
-    const float zq = Zq[e], zk = Zk[e];
-    const float nq = zq - et * (Gq[e] + 2.f * alpha * (zq - Tq[e]));
-    const float nk = zk - et * (Gk[e] + 2.f * alpha * (zk - Tk[e]));
-    Zq[e] = nq;
-    Zk[e] = nk;
-    if (Zqs) {
-      const __nv_bfloat16 hq = __float2bfloat16_rn(nq), hk = __float2bfloat16_rn(nk);
-      Zqs[e] = hq;
-      Zqs[plane + e] = __float2bfloat16_rn(nq - __bfloat162float(hq));
-      Zks[e] = hk;
-      Zks[plane + e] = __float2bfloat16_rn(nk - __bfloat162float(hk));
-    }
+  struct __align__(4 * V) F { float v[V]; };
+  struct __align__(2 * V) B { __nv_bfloat16 v[V]; };
+  const int H = d / d_h, c = ((int)blockIdx.x * 256 + (int)threadIdx.x) * V;
+  if (c >= d) return;
+  const int head = c / d_h;
+  for (int64_t tok = blockIdx.y; tok < tokens; tok += gridDim.y) {
+    const int64_t e = tok * d + c;
+    const float et = eta[(tok / T) * H + head];
+    const auto step = [&](float* Z, const float* G, const float* Tg, __nv_bfloat16* S) {
+      const F z = *reinterpret_cast<const F*>(Z + e), g = *reinterpret_cast<const F*>(G + e),
+              t = *reinterpret_cast<const F*>(Tg + e);
+      F n;
+      B hi, lo;
+#pragma unroll
+      for (int q = 0; q < V; ++q) {
+        n.v[q] = z.v[q] - et * (g.v[q] + 2.f * alpha * (z.v[q] - t.v[q]));
+        hi.v[q] = __float2bfloat16_rn(n.v[q]);
+        lo.v[q] = __float2bfloat16_rn(n.v[q] - __bfloat162float(hi.v[q]));
+      }
+      *reinterpret_cast<F*>(Z + e) = n;
+      if (S) {
+        *reinterpret_cast<B*>(S + e) = hi;
+        *reinterpret_cast<B*>(S + plane + e) = lo;
+      }
+    };
+    step(Zq, Gq, Tq, Zqs);
+    step(Zk, Gk, Tk, Zks);
   }
 }
 
@@ -208,8 +284,13 @@ cudaError_t mha_softmax_rows(float* S, int64_t pairs, int T, bool causal, void* 
   if (rows == 0) return cudaSuccess;
   ProfScope prof(PK_ELEMENTWISE, 0.0, (double)rows * T * 8.0, stream);
   count_launch();
-  softmax_rows_kernel<<<(unsigned)ceil_div(rows, (int64_t)kRowWarps), kRowWarps * 32, 0, stream>>>(
-      S, rows, T, causal ? 1 : 0, reinterpret_cast<__nv_bfloat16*>(Sb), plane);
+  const unsigned grid = (unsigned)ceil_div(rows, (int64_t)kRowWarps);
+  const auto run = [&](auto kernel) {
+    kernel<<<grid, kRowWarps * 32, 0, stream>>>(S, rows, T, causal ? 1 : 0, reinterpret_cast<__nv_bfloat16*>(Sb), plane);
+  };
+  if (T <= 128) run(softmax_rows_kernel<4>);
+  else if (T <= 256) run(softmax_rows_kernel<8>);
+  else run(softmax_rows_kernel<0>);
   return cudaGetLastError();
 }
 
@@ -219,8 +300,17 @@ cudaError_t mha_p_update(float* P, const float* Phi, const float* G1, const floa
   if (total == 0) return cudaSuccess;
   ProfScope prof(PK_ELEMENTWISE, 0.0, (double)total * 16.0, stream);
   count_launch();
-  p_update_kernel<<<grid_1d(total, 256), 256, 0, stream>>>(P, Phi, G1, eta, (int64_t)T * T, total, (float)alpha,
-                                                           (float)beta, reinterpret_cast<__nv_bfloat16*>(Pb), plane);
+  const int64_t per_pair = (int64_t)T * T;
+  const auto al = [](const void* p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; };
+  const bool vec = per_pair % 4 == 0 && plane % 4 == 0 && al(P, 16) && al(Phi, 16) && al(G1, 16) && al(Pb, 8);
+  int64_t gx = ceil_div(per_pair, (int64_t)(vec ? 1024 : 256)), gy = pairs < 65535 ? pairs : 65535;
+  const int64_t cap = (int64_t)sm_count() * 16;
+  if (gx > cap) gx = cap;
+  if (gx * gy > cap) gy = cap / gx > 0 ? cap / gx : 1;
+  const dim3 grid((unsigned)gx, (unsigned)gy);
+  __nv_bfloat16* pb = reinterpret_cast<__nv_bfloat16*>(Pb);
+  if (vec) p_update_kernel<4><<<grid, 256, 0, stream>>>(P, Phi, G1, eta, per_pair, pairs, (float)alpha, (float)beta, pb, plane);
+  else p_update_kernel<1><<<grid, 256, 0, stream>>>(P, Phi, G1, eta, per_pair, pairs, (float)alpha, (float)beta, pb, plane);
   return cudaGetLastError();
 }
 
@@ -230,8 +320,14 @@ cudaError_t mha_softmax_backward_rows(float* S, const float* P, int64_t pairs, i
   if (rows == 0) return cudaSuccess;
   ProfScope prof(PK_ELEMENTWISE, 0.0, (double)rows * T * 12.0, stream);
   count_launch();
-  softmax_backward_rows_kernel<<<(unsigned)ceil_div(rows, (int64_t)kRowWarps), kRowWarps * 32, 0, stream>>>(
-      S, P, rows, T, causal ? 1 : 0, (float)beta, reinterpret_cast<__nv_bfloat16*>(dSb));
+  const unsigned grid = (unsigned)ceil_div(rows, (int64_t)kRowWarps);
+  const auto run = [&](auto kernel) {
+    kernel<<<grid, kRowWarps * 32, 0, stream>>>(S, P, rows, T, causal ? 1 : 0, (float)beta,
+                                                reinterpret_cast<__nv_bfloat16*>(dSb));
+  };
+  if (T <= 128) run(softmax_backward_rows_kernel<4>);
+  else if (T <= 256) run(softmax_backward_rows_kernel<8>);
+  else run(softmax_backward_rows_kernel<0>);
   return cudaGetLastError();
 }
 
@@ -253,9 +349,19 @@ cudaError_t mha_z_update(float* Zq, float* Zk, const float* Gq, const float* Gk,
   if (total == 0) return cudaSuccess;
   ProfScope prof(PK_ELEMENTWISE, 0.0, (double)total * 32.0, stream);
   count_launch();
-  z_update_kernel<<<grid_1d(total, 256), 256, 0, stream>>>(Zq, Zk, Gq, Gk, Tq, Tk, eta, tokens, d, T, d_h, (float)alpha,
-                                                           reinterpret_cast<__nv_bfloat16*>(Zqs),
-                                                           reinterpret_cast<__nv_bfloat16*>(Zks), plane);
+  const auto al = [](const void* p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; };
+  const bool vec = d_h % 4 == 0 && plane % 4 == 0 && al(Zq, 16) && al(Zk, 16) && al(Gq, 16) && al(Gk, 16) && al(Tq, 16) &&
+                   al(Tk, 16) && al(Zqs, 8) && al(Zks, 8);
+  const int64_t gx = ceil_div(d, vec ? 1024 : 256);
+  int64_t gy = ceil_div((int64_t)sm_count() * 8, gx);
+  if (gy > tokens) gy = tokens;
+  const auto run = [&](auto kernel) {
+    kernel<<<dim3((unsigned)gx, (unsigned)gy), 256, 0, stream>>>(Zq, Zk, Gq, Gk, Tq, Tk, eta, tokens, d, T, d_h, (float)alpha,
+                                                                 reinterpret_cast<__nv_bfloat16*>(Zqs),
+                                                                 reinterpret_cast<__nv_bfloat16*>(Zks), plane);
+  };
+  if (vec) run(z_update_kernel<4>);
+  else run(z_update_kernel<1>);
   return cudaGetLastError();
 }
 
