@@ -36,6 +36,8 @@ constexpr int BM = 128;            // rows of A (and of the accumulator) per CTA
 constexpr int BNH = 128;           // columns of B loaded per CTA (half of the pair's tile)
 constexpr int TILE_M = 2 * BM;     // tile of the CTA pair
 constexpr int TILE_N = 2 * BNH;
+constexpr int kNarrowN = 128;      // columns of the narrow tile
+constexpr int kMinCutKb = 32;      // a range of K that a tile may be cut into has at least this many k-blocks
 constexpr int BK = 64;
 constexpr int STAGES = 6;
 constexpr int UMMA_K = 16;
@@ -261,15 +263,15 @@ __device__ __forceinline__ uint64_t make_smem_desc(uint32_t addr, bool kmajor, u
   return d;
 }
 
-// Instruction descriptor of the pair's MMA: 256 x 256 x 16, bf16 operands, fp32 accumulator.
-__device__ __forceinline__ uint32_t make_instr_desc(bool a_kmajor, bool b_kmajor) {
+// Instruction descriptor of the pair's MMA: 256 x tile_n x 16, bf16 operands, fp32 accumulator.
+__device__ __forceinline__ uint32_t make_instr_desc(bool a_kmajor, bool b_kmajor, int tile_n) {
   uint32_t d = 0;
   d |= 1u << 4;                          // accumulator format: fp32
   d |= 1u << 7;                          // A format: bf16
   d |= 1u << 10;                         // B format: bf16
   d |= (a_kmajor ? 0u : 1u) << 15;       // A major-ness
   d |= (b_kmajor ? 0u : 1u) << 16;       // B major-ness
-  d |= (uint32_t)(TILE_N >> 3) << 17;    // N
+  d |= (uint32_t)(tile_n >> 3) << 17;    // N
   d |= (uint32_t)(TILE_M >> 4) << 24;    // M
   return d;
 }
@@ -322,11 +324,17 @@ __device__ __forceinline__ void tc_commit_local(uint32_t bar) {
 // BATCHED = false is the plain two-dimensional form (the products of the FFN path); BATCHED = true adds the batch
 // and plane coordinates (five-dimensional tensor maps).  Two instantiations, so that the plain form carries none of
 // the batched form's instructions.
-template <bool BATCHED>
+// TN: columns of the pair's tile, 256 or 128.  The narrow tile is for products that leave SM pairs idle, where a tile's
+// main loop (0.3 us per 64 values of K at 256 columns) and epilogue are the whole time (3072 x 256, K = 768: 11.1 -> 9.9 us;
+// 256 x 256, K = 64: 7.2 -> 5.9), and for products of at most 128 columns, which the wide tile would do twice over with
+// zeros.  The sum over K runs in the same order either way.
+template <bool BATCHED, int TN>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmCin, const TcParams p) {
   if (p.skip != nullptr && *p.skip != 0) return;   // the same answer in every CTA: nothing is allocated yet
+  constexpr int BN_LOAD = TN / 2;                            // columns of B loaded per CTA
+  constexpr uint32_t LOAD_BYTES = A_BYTES + BN_LOAD * BK * 2;
   extern __shared__ uint8_t smem_raw[];
   __shared__ uint32_t s_tmem_base;
   __shared__ int s_abort;
@@ -387,7 +395,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         for (int kb = kb0; kb < kb1; ++kb) {
           if (!mbar_wait(empty_bar(s), ph ^ 1u, abort_flag, p.wait_budget)) { ok = false; break; }
           // the leader's barrier collects the bytes of both CTAs' loads of this stage
-          if (rank == 0) mbar_expect_tx(full_bar(s), 2 * STAGE_BYTES);
+          if (rank == 0) mbar_expect_tx(full_bar(s), 2 * LOAD_BYTES);
           const uint32_t fbar = map_to_cta(full_bar(s), 0);
           const uint32_t a_dst = tiles + s * STAGE_BYTES;
           const uint32_t b_dst = a_dst + A_BYTES;
@@ -395,7 +403,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           const int kk = (kb - sg * p.seg_kb) * BK;
           const int ka = kk + p.seg.a_k[sg], kbb = kk + p.seg.b_k[sg];
           const int am = tm * TILE_M + (int)rank * BM + p.seg.a_mn[sg];
-          const int bn = tn * TILE_N + (int)rank * BNH + p.seg.b_mn[sg];
+          const int bn = tn * TN + (int)rank * BN_LOAD + p.seg.b_mn[sg];
           if constexpr (BATCHED) {
             const int pa = p.seg.a_p[sg], pb = p.seg.b_p[sg];
             if (p.a_kmajor) {
@@ -409,7 +417,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
               tma_load_5d(b_dst, &tmB, make_coord(p.b_ord, kbb, bn, b0, b1, pb), fbar);
             } else {
 #pragma unroll
-              for (int nb = 0; nb < BNH / 64; ++nb)
+              for (int nb = 0; nb < BN_LOAD / 64; ++nb)
                 tma_load_5d(b_dst + nb * (64 * BK * 2), &tmB, make_coord(p.b_ord, bn + nb * 64, kbb, b0, b1, pb), fbar);
             }
           } else {
@@ -423,7 +431,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
               tma_load_2d(b_dst, &tmB, kbb, bn, fbar);
             } else {
 #pragma unroll
-              for (int nb = 0; nb < BNH / 64; ++nb) tma_load_2d(b_dst + nb * (64 * BK * 2), &tmB, bn + nb * 64, kbb, fbar);
+              for (int nb = 0; nb < BN_LOAD / 64; ++nb) tma_load_2d(b_dst + nb * (64 * BK * 2), &tmB, bn + nb * 64, kbb, fbar);
             }
           }
           if (++s == STAGES) { s = 0; ph ^= 1u; }
@@ -439,7 +447,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer (leader CTA only)
     if (lane == 0 && rank == 0) {
-      const uint32_t idesc = make_instr_desc(p.a_kmajor != 0, p.b_kmajor != 0);
+      const uint32_t idesc = make_instr_desc(p.a_kmajor != 0, p.b_kmajor != 0, TN);
       int s = 0;
       uint32_t ph = 0;
       int acc = 0;
@@ -517,15 +525,15 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         // blocks of Cin (loaded one block ahead) and two blocks of C.  64-byte rows, 64-byte swizzle: 16-byte chunk j
         // of row r sits at chunk j ^ ((r >> 1) & 3).
         const bool rows_ok = rows_here > 0;
-        const int nsl = (int)(((p.N - (int64_t)tn * TILE_N < TILE_N) ? (p.N - (int64_t)tn * TILE_N) : TILE_N) + 31) / 32;
+        const int nsl = (int)(((p.N - (int64_t)tn * TN < TN) ? (p.N - (int64_t)tn * TN) : TN) + 31) / 32;
         if (rows_ok && lane == 0 && nsl > 0) {
           fence_async_smem();
           mbar_expect_tx(cin_bar(q, cbuf), 2048);
-          tma_load_2d_local(wstg + cbuf * 2048, &tmCin, (int32_t)((int64_t)tn * TILE_N), (int32_t)row0, cin_bar(q, cbuf));
+          tma_load_2d_local(wstg + cbuf * 2048, &tmCin, (int32_t)((int64_t)tn * TN), (int32_t)row0, cin_bar(q, cbuf));
         }
 #pragma unroll 1
         for (int sl = 0; sl < nsl; ++sl) {
-          const int64_t gj0 = (int64_t)tn * TILE_N + sl * 32;
+          const int64_t gj0 = (int64_t)tn * TN + sl * 32;
           uint32_t r[32];
           tc_ld32(taddr + (uint32_t)(sl * 32), r);
           tc_wait_ld();
@@ -574,8 +582,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         // 32 x 32 fp32 block -> 128-byte-swizzled shared tile (16-byte chunk j of row r sits at chunk j ^ (r & 7))
         // -> one TMA store / add-reduction, which clips at the edges of C.  Two tiles per warp alternate.
 #pragma unroll 1
-        for (int c0 = 0; c0 < TILE_N; c0 += 32) {
-          const int64_t gj0 = (int64_t)tn * TILE_N + c0;
+        for (int c0 = 0; c0 < TN; c0 += 32) {
+          const int64_t gj0 = (int64_t)tn * TN + c0;
           if (gj0 >= p.N) break;                  // uniform over the warp
           uint32_t r[32];
           tc_ld32(taddr + (uint32_t)c0, r);
@@ -610,8 +618,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         // plain path: the block is turned through a padded tile so that global loads and stores see a warp on 32
         // consecutive columns of one row (128-byte lines) instead of 32 different rows
 #pragma unroll 1
-        for (int c0 = 0; c0 < TILE_N; c0 += 32) {
-          const int64_t gj0 = (int64_t)tn * TILE_N + c0;
+        for (int c0 = 0; c0 < TN; c0 += 32) {
+          const int64_t gj0 = (int64_t)tn * TN + c0;
           if (gj0 >= p.N) break;                  // uniform over the warp
           const int64_t gj = gj0 + lane;
           // the 32 rows of Cin for this column are fetched first (independent loads in flight while the accumulator
@@ -697,7 +705,7 @@ EncodeTiledFn encode_fn() {
 }
 
 // Tensor map of a row-major matrix [outer, inner] with leading dimension ld (elements), 128-byte swizzle.
-//   bf16 operand, K-major : inner = K, outer = rows, box = {64, 128}
+//   bf16 operand, K-major : inner = K, outer = rows, box = {64, 128} (B of the narrow tile: {64, 64})
 //   bf16 operand, MN-major: inner = rows, outer = K, box = {64, 64}
 //   fp32 output C         : inner = N, outer = M, box = {32, 32}
 //   bf16 C / Cin          : inner = N, outer = M, box = {32, 32}, 64-byte swizzle
@@ -809,6 +817,17 @@ sp_status gemm_tc(int64_t M, int64_t N, int64_t K, float alpha, TcOperand A, TcO
   if (C.dtype != SP_F32 && C.dtype != SP_BF16) return SP_ERR_DTYPE;
   if (beta != 0.f && Cin.dtype != SP_F32 && Cin.dtype != SP_BF16) return SP_ERR_DTYPE;
 
+  int pairs_max = sm_count() / 2;
+  if (max_pairs > 0 && max_pairs < pairs_max) pairs_max = max_pairs;
+  const int num_kb = (int)ceil_div(K, BK) * sg.nseg;
+  // The narrow tile where both halves of every wide tile run at once, or N fits it; not where K may be cut instead (see
+  // below), and for a lower triangle only where one wide tile covers all columns, so that the same entries are written.
+  const int64_t wide_tiles = ceil_div(M, (int64_t)TILE_M) * ceil_div(N, (int64_t)TILE_N) *
+                             (batched ? (int64_t)batch->nb0 * batch->nb1 : 1);
+  const bool narrow = (batched || num_kb < kMinCutKb * 2) && (!lower_only || N <= TILE_N) &&
+                      (N <= kNarrowN || 2 * wide_tiles <= pairs_max);
+  const int tile_n = narrow ? kNarrowN : TILE_N;
+
   CUtensorMap tmA, tmB, tmC, tmCin;
   memset(&tmC, 0, sizeof(tmC));
   memset(&tmCin, 0, sizeof(tmCin));
@@ -824,7 +843,7 @@ sp_status gemm_tc(int64_t M, int64_t N, int64_t K, float alpha, TcOperand A, TcO
                               bt.a_planes, bt.a_plane, true, p.a_ord)
                   : make_map5(&tmA, false, A.ptr, a_mext, 64, a_kext, A.ld, BK, bt.nb0, bt.a_s0, bt.nb1, bt.a_s1,
                               bt.a_planes, bt.a_plane, true, p.a_ord);
-    ok = ok && (B.kmajor ? make_map5(&tmB, false, B.ptr, b_kext, BK, b_next, B.ld, BNH, bt.nb0, bt.b_s0, bt.nb1,
+    ok = ok && (B.kmajor ? make_map5(&tmB, false, B.ptr, b_kext, BK, b_next, B.ld, tile_n / 2, bt.nb0, bt.b_s0, bt.nb1,
                                      bt.b_s1, bt.b_planes, bt.b_plane, true, p.b_ord)
                          : make_map5(&tmB, false, B.ptr, b_next, 64, b_kext, B.ld, BK, bt.nb0, bt.b_s0, bt.nb1,
                                      bt.b_s1, bt.b_planes, bt.b_plane, true, p.b_ord));
@@ -832,7 +851,7 @@ sp_status gemm_tc(int64_t M, int64_t N, int64_t K, float alpha, TcOperand A, TcO
   } else {
     ok = A.kmajor ? make_map(&tmA, false, A.ptr, a_kext, a_mext, A.ld, BK, BM)
                   : make_map(&tmA, false, A.ptr, a_mext, a_kext, A.ld, 64, BK);
-    ok = ok && (B.kmajor ? make_map(&tmB, false, B.ptr, b_kext, b_next, B.ld, BK, BNH)
+    ok = ok && (B.kmajor ? make_map(&tmB, false, B.ptr, b_kext, b_next, B.ld, BK, tile_n / 2)
                          : make_map(&tmB, false, B.ptr, b_next, b_kext, B.ld, 64, BK));
     if (!ok) return SP_ERR_CUDA;
   }
@@ -850,6 +869,7 @@ sp_status gemm_tc(int64_t M, int64_t N, int64_t K, float alpha, TcOperand A, TcO
   if (C.lo_off < 0 || (C.lo_off > 0 && C.dtype != SP_BF16)) return SP_ERR_INVALID_ARG;
   p.a_kmajor = A.kmajor ? 1 : 0;
   p.b_kmajor = B.kmajor ? 1 : 0;
+  if (narrow) lower_only = false;
   p.lower_only = lower_only ? 1 : 0;
   // fp32 C that a tensor map can describe leaves through TMA: a store when nothing is added, an add-reduction when
   // the call accumulates into C itself (each element of C is touched once per launch, so the result is the same sum)
@@ -884,7 +904,7 @@ sp_status gemm_tc(int64_t M, int64_t N, int64_t K, float alpha, TcOperand A, TcO
   p.seg = sg;
   p.seg_kb = (int32_t)ceil_div(K, BK);
   p.tiles_m = (int32_t)ceil_div(M, TILE_M);
-  p.tiles_n = (int32_t)ceil_div(N, TILE_N);
+  p.tiles_n = (int32_t)ceil_div(N, tile_n);
   // consecutive tiles (which run at the same time on neighbouring SMs) should share the larger operand panel
   p.n_fast = p.tiles_n < p.tiles_m ? 1 : 0;
   if (lower_only) {
@@ -908,9 +928,6 @@ sp_status gemm_tc(int64_t M, int64_t N, int64_t K, float alpha, TcOperand A, TcO
   // the add-reduction epilogue may cut K into a few ranges per tile instead: the partial products add up in C (in an
   // order that is not fixed, so the last bits of such sums can differ between runs).  A plain store into an fp32 C
   // is turned into "clear C, then accumulate" when that pays.
-  int pairs_max = sm_count() / 2;
-  if (max_pairs > 0 && max_pairs < pairs_max) pairs_max = max_pairs;
-  const int num_kb = p.seg_kb * sg.nseg;
   p.ksplit = 1;
   const bool may_cut = !batched && !reproducible_mode();   // partial products of a cut tile add in no fixed order
   if (may_cut && (p.epi_mode == EPI_TMA_STORE || p.epi_mode == EPI_TMA_ADD) && p.num_tiles > 0) {
@@ -920,7 +937,7 @@ sp_status gemm_tc(int64_t M, int64_t N, int64_t K, float alpha, TcOperand A, TcO
     };
     int best = 1;
     for (int ks = 2; ks <= 4; ++ks)
-      if (num_kb / ks >= 32 && eff(ks) > eff(best) + 0.03) best = ks;
+      if (num_kb / ks >= kMinCutKb && eff(ks) > eff(best) + 0.03) best = ks;
     if (best > 1 && p.epi_mode == EPI_TMA_STORE && p.skip != nullptr) best = 1;   // no unconditional clear of C
     if (best > 1) {
       if (p.epi_mode == EPI_TMA_STORE) {
@@ -938,7 +955,7 @@ sp_status gemm_tc(int64_t M, int64_t N, int64_t K, float alpha, TcOperand A, TcO
     const int full = p.num_tiles / pairs_max, rem = p.num_tiles % pairs_max;
     int ways = pairs_max / rem;
     if (ways > 8) ways = 8;
-    while (ways > 1 && num_kb / ways < 32) --ways;
+    while (ways > 1 && num_kb / ways < kMinCutKb) --ways;
     const double t_uniform = ceil((double)p.num_tiles * p.ksplit / pairs_max) / p.ksplit;
     const double t_tail = full + 1.0 / ways;
     if (ways > 1 && t_tail < 0.99 * t_uniform) {
@@ -952,11 +969,12 @@ sp_status gemm_tc(int64_t M, int64_t N, int64_t K, float alpha, TcOperand A, TcO
 
   static PerDeviceOnce attr_once;
   if (attr_once.run([] {
-        cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)SMEM_BYTES);
-        if (e == cudaSuccess)
-          e = cudaFuncSetAttribute(gemm_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
-        return e;
+        for (auto k : {gemm_tc_kernel<false, TILE_N>, gemm_tc_kernel<true, TILE_N>, gemm_tc_kernel<false, kNarrowN>,
+                       gemm_tc_kernel<true, kNarrowN>}) {
+          const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
+          if (e != cudaSuccess) return e;
+        }
+        return cudaSuccess;
       }) != cudaSuccess)
     return SP_ERR_CUDA;
   count_launch();
@@ -967,8 +985,9 @@ sp_status gemm_tc(int64_t M, int64_t N, int64_t K, float alpha, TcOperand A, TcO
   ProfScope prof(p.skip != nullptr ? PK_CONDITIONAL : max_pairs > 0 ? PK_GEMM_TC_SHARED : PK_GEMM_TC,
                  p.skip != nullptr ? 0.0 : flops, 0.0, stream);
   const int pairs = p.num_units < pairs_max ? p.num_units : pairs_max;
-  if (batched) gemm_tc_kernel<true><<<2 * pairs, NUM_THREADS, SMEM_BYTES, stream>>>(tmA, tmB, tmC, tmCin, p);
-  else gemm_tc_kernel<false><<<2 * pairs, NUM_THREADS, SMEM_BYTES, stream>>>(tmA, tmB, tmC, tmCin, p);
+  const auto kernel = batched ? (narrow ? gemm_tc_kernel<true, kNarrowN> : gemm_tc_kernel<true, TILE_N>)
+                              : (narrow ? gemm_tc_kernel<false, kNarrowN> : gemm_tc_kernel<false, TILE_N>);
+  kernel<<<2 * pairs, NUM_THREADS, SMEM_BYTES, stream>>>(tmA, tmB, tmC, tmCin, p);
   return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ERR_CUDA;
 }
 

@@ -749,7 +749,7 @@ sp_status potrs_right_tc(float* X, int64_t m, int64_t n, int64_t ldx, const void
         float* Xc = X + c0;
         sp_status stt = gemm_tc(m, w, TB, -1.f, ta, tb, 1.f, Operand{Xc, SP_F32, ldx, 1}, OutOperand{Xc, SP_F32, ldx},
                                 false, status_dev, st_run, &sg, 2.0 * (double)m * (double)w * (double)nb,
-                                on_assist && near_in_panel && runs_beside(w) && tiles_of(w) > beside_pairs ? (int)beside_pairs : 0);
+                                on_assist && near_in_panel && runs_beside(w) ? (int)beside_pairs : 0);
         if (stt != SP_OK) return stt;
         if (on_assist) {
           SP_CUDA_OK(cudaEventRecord(assist->rest_done[step & 1], st_run));

@@ -41,6 +41,32 @@ def test_gemm_fp64_accumulation(dtype, transA, transB, M, N, K, pad):
     assert torch.equal(low[tri], got[tri])
 
 
+@pytest.mark.parametrize("a_kmajor", [False, True])
+@pytest.mark.parametrize("b_kmajor", [False, True])
+@pytest.mark.parametrize("M,N,K,lower", [(8, 8, 8, False), (256, 128, 64, False), (264, 136, 72, False), (1000, 64, 704, False),
+                                         (1288, 256, 768, True), (520, 520, 128, False), (2304, 1032, 320, False),
+                                         (3000, 256, 192, False)])
+def test_gemm_tensor_core_tiles_of_both_widths(a_kmajor, b_kmajor, M, N, K, lower):
+    """256 x 128 tiles (few tiles, or few columns) and 256 x 256 tiles, stored and accumulated into C."""
+    api = _api()
+    g = torch.Generator(device="cuda").manual_seed(M + N + K)
+    A = torch.randn(*((M, K) if a_kmajor else (K, M)), generator=g, device="cuda").bfloat16()
+    B = torch.randn(*((N, K) if b_kmajor else (K, N)), generator=g, device="cuda").bfloat16()
+    a, b = (A if a_kmajor else A.T).double(), (B.T if b_kmajor else B).double()
+    C0 = torch.randn(M, N, generator=g, device="cuda")
+    # exact products, fp32 sums: at most one rounding of 2^-23 (the unit truncates) of the sum of magnitudes per term
+    bound = (K + 2) * 2.0 ** -23 * (a.abs() @ b.abs() + C0.double().abs())
+    keep = torch.ones(M, N, dtype=torch.bool, device="cuda")
+    if lower:
+        keep = keep.tril()
+    for beta, dtype in ((0.0, torch.float32), (1.0, torch.float32), (0.0, torch.bfloat16)):
+        C = C0.to(dtype)
+        want = a @ b + beta * C.double()
+        api.sp_gemm(A, B, C, not a_kmajor, b_kmajor, beta=beta, lower_only=lower, use_tensor_cores=True)
+        off = (C.double() - want).abs() - bound - (2.0 ** -8 * want.abs() if dtype == torch.bfloat16 else 0)
+        assert float(off[keep].max()) <= 0
+
+
 def _spd(n, seed):
     g = torch.Generator(device="cuda").manual_seed(seed)
     X = torch.randn(2 * n + 3, n, generator=g, device="cuda") * torch.logspace(0, 1.5, n, device="cuda")
