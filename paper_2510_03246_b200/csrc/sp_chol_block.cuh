@@ -5,20 +5,17 @@
 
 namespace sp {
 
-// 1 / sqrt(x) to about 1 ulp, x > 0: hardware approximation and a step of Newton's iteration (fp32) or of the third-order
-// iteration y (1 + e / 2 + 3 e^2 / 8), e = 1 - x y^2 (fp64: the approximation's 20 bits become 58).  No branches, so that
-// the steps of consecutive columns interleave.
-__device__ __forceinline__ float rsqrt_refined(float x) {
+// 1 / sqrt(x), x > 0.
+// fp32: the hardware approximation r (relative error d below 2^-22) and one step of Newton's method for f(r) = r^-2 - x,
+// r - f(r) / f'(r) = r (3 - x r^2) / 2, which leaves 1.5 d^2 and the roundings of r^2 (counted half), of the bracket and of
+// the product: 2.5 x 2^-24 together.  x is a normal number (the approximation takes subnormals for zero).
+// fp64: CUDA's function, which takes subnormal and infinite pivots too (a column with an infinite pivot becomes zero).
+__device__ __forceinline__ float recip_sqrt(float x) {
   float r;
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r * fmaf(-0.5f * x, r * r, 1.5f);
 }
-__device__ __forceinline__ double rsqrt_refined(double x) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-x * y, y, 1.0);
-  return fma(y * e, fma(0.375, e, 0.5), y);
-}
+__device__ __forceinline__ double recip_sqrt(double x) { return rsqrt(x); }
 
 // The block is eliminated in sub-blocks of 32 columns.  Rows to carry along are the rows of the matrix below the
 // sub-block and the rows of an identity appended under the matrix (X L^T = I, so X = L^-T): together always NB rows.  Per sub-block
@@ -102,7 +99,7 @@ struct DiagBlock {
           if (q < k) p = fma(-c[k][q], c[k][q], p);
         bad = (p > (T)0 || bad < SB) ? bad : j + k;
         p = p > (T)0 ? p : (T)1;
-        rd[k] = rsqrt_refined(p);
+        rd[k] = recip_sqrt(p);
 #pragma unroll
         for (int r = 0; r < 4; ++r)
           if (r > k) {

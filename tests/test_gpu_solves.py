@@ -108,6 +108,50 @@ def test_tensor_core_ridge_solve_at_block_edges(n, m):
     assert status[:2].tolist() == [6, i]      # SP_ERR_NOT_SPD and the pivot
 
 
+def _diagonal(lo, hi, n=128):
+    """Diagonal matrix with entries over 2^lo .. 2^hi, mantissas spread."""
+    e = torch.linspace(lo, hi, n, dtype=torch.float64, device="cuda")
+    return torch.diag((2.0 ** e).float())
+
+
+def test_reciprocal_square_roots_of_the_pivots():
+    """A diagonal system solved for its own matrix: every entry of the answer is g y y with y = 1 / sqrt(g)."""
+    api = _api()
+    eye = torch.eye(128, device="cuda")
+    # fp32: y to 2.5 x 2^-24, two products of 2^-24 each; at the upper end y^2 is subnormal (one more 2^-24 in y)
+    for lo, hi, units in ((-100, 100, 7.0), (-125.5, 127.5, 9.0)):
+        G = _diagonal(lo, hi)
+        W = api.sp_ridge_solve(G, G, 0.0, False)
+        assert torch.equal(W != 0, eye != 0)
+        assert float((W.diagonal().double() - 1).abs().max()) <= units * 2.0 ** -24
+    # fp64: a few 2^-53, nothing of which is left in fp32; subnormal fp32 entries among them
+    G = _diagonal(-148.5, 127.5)
+    assert torch.equal(api.sp_ridge_solve(G, G, 0.0, False, precise=True), eye)
+
+
+@pytest.mark.parametrize("n", [5, 64, 130])
+def test_precise_solve_with_extreme_pivots(n):
+    """Pivots that are subnormal in fp64, near the upper end, or infinite (an accumulator that overflowed): the solution is what
+    the square root and the division by it give, a column with an infinite pivot is zero."""
+    api = _api()
+    zero = torch.zeros(n, n, device="cuda")
+    for rho, value in ((1e-310, 0.0), (5e-324, 0.0), (1e300, 3e38), (1.7e308, 3e38)):
+        status = api.new_status(zero.device)
+        W = api.sp_ridge_solve(torch.full_like(zero, value), zero, rho, False, precise=True, status=status)
+        assert torch.equal(W, zero) and int(status[0]) == 0, rho
+    G = _spd(n, n)
+    R = torch.randn(7, n, generator=torch.Generator(device="cuda").manual_seed(n), device="cuda")
+    i = n // 2
+    rest = [j for j in range(n) if j != i]
+    bad = G.clone()
+    bad[i, i] = float("inf")
+    W = api.sp_ridge_solve(R, bad, 0.5, False, precise=True)
+    assert torch.equal(W[:, i], torch.zeros_like(W[:, i]))
+    H = G[rest][:, rest].double() + 0.5 * torch.eye(n - 1, device="cuda", dtype=torch.float64)
+    want = torch.linalg.solve(H, R[:, rest].double().T).T
+    assert float((W[:, rest].double() - want).abs().max() / want.abs().max()) < 1.2e-7
+
+
 @pytest.mark.parametrize("n,m", [(12288, 40), (12300, 200), (12420, 4800)])
 def test_two_level_sweep_of_a_large_system(n, m):
     """Outer blocks of 512 columns, the last of them ragged; few right-hand sides (a block column pulls the update of the
