@@ -24,12 +24,13 @@
  *   - Return value: SP_OK or an error detected on the host before any launch (argument / shape / alignment /
  *     workspace errors).  Numerical failures found on the device (non-positive Cholesky pivot, a bounded wait that
  *     ran out) are written to the caller's `status_dev[4]` = {code, index, aux, 0}; nothing traps or spins forever.
- *   - Streams: a call is ordered on the caller's stream, but sp_admm_step, sp_admm_scores, sp_ridge_solve and
- *     sp_linear_refit also fork independent parts (the two weight recoveries, the panels and trailing updates of a
- *     factorisation, the z^(1) products) onto a few streams and events that the library creates once per device and
- *     joins back to the caller's stream with events before the call's results are used (also when a call returns an
- *     error after the fork).  That set is shared by all calls on a device: issue the calls of one device from one
- *     host thread at a time.  Nothing else persists inside the library.
+ *   - Streams: a call is ordered on the caller's stream, but sp_admm_step, sp_admm_scores, sp_mha_value_refit and
+ *     (precise == 0) sp_ridge_solve and sp_linear_refit also fork independent parts (the two weight recoveries, the
+ *     panels and trailing updates of a factorisation, the z^(1) products) onto a few streams and events that the
+ *     library creates once per device and joins back to the caller's stream with events before the call's results are
+ *     used (also when a call returns an error after the fork).  That set is shared by all these calls on a device: issue
+ *     them from one host thread at a time.  All other calls, sp_ffn_cache_input_inverse and the precise solves among
+ *     them, use the caller's stream alone.  Nothing else persists inside the library.
  *   - Reproducibility: by default a product whose tile count leaves SMs idle is cut along K and its partial
  *     products add up in C in an order that is not fixed, and the backward triangular solve adds updates from two
  *     streams; fp32 results (accumulators, recovered weights, scores) can then differ in their last bits between two

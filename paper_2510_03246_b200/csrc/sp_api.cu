@@ -485,9 +485,9 @@ sp_status sp_ridge_solve(const float* R, int64_t ldr, const float* G, int64_t ld
   Carver c(ws);
   SolveBufs b = carve_solve(c, n, m, precise ? 8 : 4);
   CU(effective_ridge(G, ldg, n, rho, rho_relative, b.rho, s));
+  // (the precise form keeps to the caller's stream: it shares nothing with other streams, threads or captures)
+  if (precise) return ridge_core<double>(R, ldr, G, ldg, m, n, nullptr, n, b.rho, W, ldw, b, status_dev, s);
   SideStream* side = side_stream();
-  if (precise) return ridge_core<double>(R, ldr, G, ldg, m, n, nullptr, n, b.rho, W, ldw, b, status_dev, s,
-                                         side ? &side->assist_main : nullptr);
   return ridge_core<float>(R, ldr, G, ldg, m, n, nullptr, n, b.rho, W, ldw, b, status_dev, s,
                            side ? &side->assist_main : nullptr);
 }
@@ -517,9 +517,8 @@ sp_status sp_linear_refit(const float* R, int64_t ldr, const float* G, int64_t l
     expand_group_index_kernel<<<(unsigned)ceil_div(k, 256), 256, 0, s>>>(unit_idx, k_keep, group, b.idx);
     CU(cudaGetLastError());
   }
+  if (precise) return ridge_core<double>(R, ldr, G, ldg, m, n, b.idx, k, b.rho, W, ldw, b, status_dev, s);
   SideStream* side = side_stream();
-  if (precise) return ridge_core<double>(R, ldr, G, ldg, m, n, b.idx, k, b.rho, W, ldw, b, status_dev, s,
-                                         side ? &side->assist_main : nullptr);
   return ridge_core<float>(R, ldr, G, ldg, m, n, b.idx, k, b.rho, W, ldw, b, status_dev, s,
                            side ? &side->assist_main : nullptr);
 }
@@ -788,11 +787,11 @@ sp_status sp_ffn_cache_input_inverse(const sp_ffn_module* m, sp_ffn_state* st, d
   ProfScope prof(PK_SOLVE, (double)d * d * d, 0.0, s);
   double* Gs = reinterpret_cast<double*>(b.Gs);
   double* X = Gs + (size_t)d * d;
-  SideStream* side = side_stream();
+  // On the caller's stream alone, like the precise solves.  (With far updates on an assisting stream d = 4096 takes 4.6
+  // instead of 5.4 ms, once per module, but two calls on two streams queue there and an open capture may hold it.)
   CU(load_spd<double>(st->G_X, d, d, b.rho, Gs, d, s));
   CU(set_identity(X, d, d, s));
-  CU(potrf_lower_f64(Gs, d, d, reinterpret_cast<double*>(b.dinv), status_dev, s, side ? &side->assist_main : nullptr, d,
-                     true));
+  CU(potrf_lower_f64(Gs, d, d, reinterpret_cast<double*>(b.dinv), status_dev, s, nullptr, d, true));
   CU(gemm_simt(d, d, d, 1.0, Operand{X, SP_F64, d, 1}, Operand{X, SP_F64, 1, d}, 0.0, Operand{st->G_X_inv, SP_F32, d, 1},
                OutOperand{st->G_X_inv, SP_F32, d}, true, true, s, true));
   CU(symmetrize_lower(st->G_X_inv, d, d, s));

@@ -210,3 +210,97 @@ def test_cached_input_inverse_at_block_edges(d):
     assert float((mod.G_X_inv.double() - want).abs().max() / want.abs().max()) < 1.2e-7
     assert torch.equal(mod.G_X_inv, mod.G_X_inv.T)
     mod.check_status()
+
+
+def _own_stream_calls(api, seed):
+    """The calls that use the caller's stream alone, each as (call, its output)."""
+    n, m = 200, 90
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    G, R = _spd(n, seed), torch.randn(m, n, generator=g, device="cuda")
+    mask = torch.zeros(n, dtype=torch.uint8, device="cuda")
+    mask[::2] = 1
+    mod = api.FfnModule(torch.randn(2 * n, n, generator=g, device="cuda").bfloat16(),
+                        torch.randn(16, n, generator=g, device="cuda"), torch.randn(n, 16, generator=g, device="cuda"))
+    mod.sp_ffn_init()
+    mod.G_X_inv = torch.zeros(n, n, device="cuda")
+    ws = [torch.empty(api.workspace_bytes(op, m, n, 0, 0, api.SP_F64), dtype=torch.uint8, device="cuda") for op in (7, 5)]
+    W = [torch.zeros(m, n, device="cuda") for _ in range(2)]
+    return {"solve": (lambda: api.sp_ridge_solve(R, G, 0.1, True, precise=True, W=W[0], ws=ws[0]), W[0]),
+            "refit": (lambda: api.sp_linear_refit(R, G, mask, n // 2, 0.1, precise=True, W=W[1], ws=ws[1]), W[1]),
+            "inverse": (lambda: mod.sp_ffn_cache_input_inverse(0.1), mod.G_X_inv)}
+
+
+@pytest.mark.parametrize("name", ["solve", "refit", "inverse"])
+def test_calls_on_the_callers_stream_alone_beside_a_capture(name):
+    """Issued on a stream of its own while another stream's capture holds the library's assisting streams: neither the call
+    nor the capture fails, and the call itself can be captured."""
+    api = _api()
+    call, out = _own_stream_calls(api, 3)[name]
+    call()
+    torch.cuda.synchronize()
+    want = out.clone()
+    G, R = _spd(600, 5), torch.randn(64, 600, generator=torch.Generator(device="cuda").manual_seed(6), device="cuda")
+    W = torch.zeros_like(R)
+    ws = torch.empty(api.workspace_bytes(7, 64, 600, 0, 0, api.SP_F32), dtype=torch.uint8, device="cuda")
+    forks = lambda: api.sp_ridge_solve(R, G, 0.1, True, W=W, ws=ws)
+    api.sp_set_reproducible(True)
+    try:
+        forks()
+        torch.cuda.synchronize()
+        want_W = W.clone()
+        cap, other = torch.cuda.Stream(), torch.cuda.Stream()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=cap, capture_error_mode="relaxed"):
+            forks()
+            with torch.cuda.stream(other):
+                out.zero_()
+                call()
+        torch.cuda.synchronize()
+        assert torch.equal(out, want)
+        W.zero_()
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(W, want_W)
+    finally:
+        api.sp_set_reproducible(False)
+    own = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(own, stream=cap, capture_error_mode="relaxed"):
+        call()
+    for _ in range(2):
+        out.zero_()
+        own.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(out, want)
+
+
+def test_calls_on_the_callers_stream_alone_from_several_threads():
+    """Three host threads, each on a stream and buffers of its own."""
+    import threading
+    api = _api()
+    jobs = [list(_own_stream_calls(api, seed).values()) for seed in (11, 12, 13)]
+    for job in jobs:
+        for call, _ in job:
+            call()
+    torch.cuda.synchronize()
+    want = [[out.clone() for _, out in job] for job in jobs]
+    got = [[] for _ in jobs]
+    start = threading.Barrier(len(jobs))
+
+    def work(k):
+        with torch.cuda.stream(torch.cuda.Stream()):
+            start.wait()
+            for _ in range(8):
+                for call, out in jobs[k]:
+                    out.zero_()
+                    call()
+                got[k].append([out.clone() for _, out in jobs[k]])
+            torch.cuda.current_stream().synchronize()
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(len(jobs))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    for k in range(len(jobs)):
+        assert len(got[k]) == 8 and all(torch.equal(a, b) for r in got[k] for a, b in zip(r, want[k]))
