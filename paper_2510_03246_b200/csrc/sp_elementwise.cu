@@ -31,9 +31,10 @@ __device__ __forceinline__ T block_sum(T v, T* smem) {
 }
 
 // ------------------------------------------------------------------------------------------------ conversions
+template <int W>
 __global__ void __launch_bounds__(kStripThreads) convert_kernel(const void* src, int32_t sdt, int64_t lds, void* dst, int32_t ddt, int64_t ldd,
                                int64_t rows, int64_t cols) {
-  for_strip(rows, cols, [&](int64_t i, int64_t j, int) {
+  for_strip<W>(rows, cols, [&](int64_t i, int64_t j, int) {
     const int64_t si = i * lds + j, di = i * ldd + j;
     if (sdt == SP_F64) {
       const double v = reinterpret_cast<const double*>(src)[si];
@@ -79,12 +80,13 @@ __device__ __forceinline__ bool pairs_aligned(const float* src, int64_t lds) {
 }
 
 // (kpad is even: a thread takes two columns, so that the bf16 stores are 4 bytes wide)
+template <int W>
 __global__ void __launch_bounds__(kStripThreads) split_bf16_kernel(const float* __restrict__ src, int64_t lds,
                                                                    const int32_t* __restrict__ row_idx, int64_t rows,
                                                                    int64_t cols, int64_t kpad,
                                                                    __nv_bfloat16* __restrict__ dst) {
   const bool vec = pairs_aligned(src, lds);
-  for_strip(rows, kpad / 2, [&](int64_t i, int64_t p, int) {
+  for_strip<W>(rows, kpad / 2, [&](int64_t i, int64_t p, int) {
     const float2 v = load_pair(src + (row_idx ? (int64_t)row_idx[i] : i) * lds, 2 * p, cols, vec);
     const __nv_bfloat162 hi = __floats2bfloat162_rn(v.x, v.y);
     __nv_bfloat162* out = reinterpret_cast<__nv_bfloat162*>(dst + i * 2 * kpad) + p;
@@ -95,11 +97,12 @@ __global__ void __launch_bounds__(kStripThreads) split_bf16_kernel(const float* 
 
 // dst[i, part * kpad + j] = part `part` of the three-part bf16 split of src[i, j] (hi + mid + lo = src exactly up to
 // 2^-24); padding columns are zero.
+template <int W>
 __global__ void __launch_bounds__(kStripThreads) split3_bf16_kernel(const float* __restrict__ src, int64_t lds,
                                                                     int64_t rows, int64_t cols, int64_t kpad,
                                                                     __nv_bfloat16* __restrict__ dst) {
   const bool vec = pairs_aligned(src, lds);
-  for_strip(rows, kpad / 2, [&](int64_t i, int64_t p, int) {
+  for_strip<W>(rows, kpad / 2, [&](int64_t i, int64_t p, int) {
     const float2 v = load_pair(src + i * lds, 2 * p, cols, vec);
     const __nv_bfloat162 hi = __floats2bfloat162_rn(v.x, v.y);
     const float2 r1 = make_float2(v.x - __low2float(hi), v.y - __high2float(hi));
@@ -174,49 +177,52 @@ __global__ void __launch_bounds__(256) load_spd_kernel(const float* __restrict__
   }
 }
 
-template <typename T>
+template <int W, typename T>
 __global__ void __launch_bounds__(kStripThreads) gather_cols_kernel(const float* __restrict__ src, int64_t lds,
                                                                     const int32_t* idx, int64_t rows, int64_t k,
                                                                     T* __restrict__ dst, int64_t ldd,
                                                                     const int32_t* skip) {
   if (skip != nullptr && *skip != 0) return;
   int64_t at[kStripPer];
-  strip_index(idx, k, at);
-  for_strip(rows, k, [&](int64_t i, int64_t a, int q) {
+  strip_index<W>(idx, k, at);
+  for_strip<W>(rows, k, [&](int64_t i, int64_t a, int q) {
     dst[i * ldd + a] = (T)src[i * lds + at[q]];
   });
 }
 
+template <int W>
 __global__ void __launch_bounds__(kStripThreads) gather_rows_kernel(const float* __restrict__ src, int64_t lds, const int32_t* __restrict__ idx,
                                    int64_t rows, int64_t cols, float* __restrict__ dst, int64_t ldd) {
-  for_strip(rows, cols, [&](int64_t i, int64_t j, int) {
+  for_strip<W>(rows, cols, [&](int64_t i, int64_t j, int) {
     dst[i * ldd + j] = src[(int64_t)idx[i] * lds + j];
   });
 }
 
-template <typename T>
+template <int W, typename T>
 __global__ void __launch_bounds__(kStripThreads) scatter_cols_kernel(const T* __restrict__ src, int64_t lds,
                                                                      const int32_t* idx, int64_t rows, int64_t k,
                                                                      float* __restrict__ dst, int64_t ldd,
                                                                      const int32_t* skip) {
   if (skip != nullptr && *skip != 0) return;
   int64_t at[kStripPer];
-  strip_index(idx, k, at);
-  for_strip(rows, k, [&](int64_t i, int64_t a, int q) {
+  strip_index<W>(idx, k, at);
+  for_strip<W>(rows, k, [&](int64_t i, int64_t a, int q) {
     dst[i * ldd + at[q]] = (float)src[i * lds + a];
   });
 }
 
+template <int W>
 __global__ void __launch_bounds__(kStripThreads) fill_zero_kernel(float* dst, int64_t ld, int64_t rows, int64_t cols,
                                                                   const int32_t* skip) {
   if (skip != nullptr && *skip != 0) return;
-  for_strip(rows, cols, [&](int64_t i, int64_t j, int) { dst[i * ld + j] = 0.f; });
+  for_strip<W>(rows, cols, [&](int64_t i, int64_t j, int) { dst[i * ld + j] = 0.f; });
 }
 
 // dst[i, 0:kpad] = src[i, 0:k] followed by zeros
+template <int W>
 __global__ void __launch_bounds__(kStripThreads) copy_cols_padded_kernel(const float* __restrict__ src, int64_t lds, int64_t rows, int64_t k,
                                         int64_t kpad, float* __restrict__ dst) {
-  for_strip(rows, kpad, [&](int64_t i, int64_t a, int) {
+  for_strip<W>(rows, kpad, [&](int64_t i, int64_t a, int) {
     dst[i * kpad + a] = a < k ? src[i * lds + a] : 0.f;
   });
 }
@@ -1091,7 +1097,9 @@ cudaError_t convert_matrix(const void* src, int32_t sdt, int64_t lds, void* dst,
   if (rows * cols == 0) return cudaSuccess;
   ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
   count_launch();
-  convert_kernel<<<strip_grid(rows, cols), kStripThreads, 0, stream>>>(src, sdt, lds, dst, ddt, ldd, rows, cols);
+  strip_launch(rows, cols, [&](auto w, dim3 grid, dim3 block) {
+    convert_kernel<decltype(w)::value><<<grid, block, 0, stream>>>(src, sdt, lds, dst, ddt, ldd, rows, cols);
+  });
   return cudaGetLastError();
 }
 
@@ -1116,8 +1124,10 @@ cudaError_t split3_bf16(const float* src, int64_t lds, int64_t rows, int64_t col
   if (rows * kpad == 0) return cudaSuccess;
   ProfScope prof(PK_ELEMENTWISE, 0.0, (double)rows * cols * 10.0, stream);
   count_launch();
-  split3_bf16_kernel<<<strip_grid(rows, kpad / 2), kStripThreads, 0, stream>>>(src, lds, rows, cols, kpad,
-                                                                     reinterpret_cast<__nv_bfloat16*>(dst));
+  strip_launch(rows, kpad / 2, [&](auto w, dim3 grid, dim3 block) {
+    split3_bf16_kernel<decltype(w)::value><<<grid, block, 0, stream>>>(
+        src, lds, rows, cols, kpad, reinterpret_cast<__nv_bfloat16*>(dst));
+  });
   return cudaGetLastError();
 }
 
@@ -1126,8 +1136,10 @@ cudaError_t split_bf16(const float* src, int64_t lds, const int32_t* row_idx, in
   if (rows * kpad == 0) return cudaSuccess;
   ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
   count_launch();
-  split_bf16_kernel<<<strip_grid(rows, kpad / 2), kStripThreads, 0, stream>>>(src, lds, row_idx, rows, cols, kpad,
-                                                                     reinterpret_cast<__nv_bfloat16*>(dst));
+  strip_launch(rows, kpad / 2, [&](auto w, dim3 grid, dim3 block) {
+    split_bf16_kernel<decltype(w)::value><<<grid, block, 0, stream>>>(
+        src, lds, row_idx, rows, cols, kpad, reinterpret_cast<__nv_bfloat16*>(dst));
+  });
   return cudaGetLastError();
 }
 
@@ -1164,7 +1176,10 @@ cudaError_t gather_cols(const float* src, int64_t lds, const int32_t* idx, int64
   if (rows * k == 0) return cudaSuccess;
   ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
   count_launch();
-  gather_cols_kernel<T><<<strip_grid(rows, k), kStripThreads, 0, stream>>>(src, lds, idx, rows, k, dst, ldd, skip_flag());
+  strip_launch(rows, k, [&](auto w, dim3 grid, dim3 block) {
+    gather_cols_kernel<decltype(w)::value, T><<<grid, block, 0, stream>>>(
+        src, lds, idx, rows, k, dst, ldd, skip_flag());
+  });
   return cudaGetLastError();
 }
 cudaError_t copy_cols_padded(const float* src, int64_t lds, int64_t rows, int64_t k, int64_t kpad, float* dst,
@@ -1172,7 +1187,9 @@ cudaError_t copy_cols_padded(const float* src, int64_t lds, int64_t rows, int64_
   if (rows * kpad == 0) return cudaSuccess;
   ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
   count_launch();
-  copy_cols_padded_kernel<<<strip_grid(rows, kpad), kStripThreads, 0, stream>>>(src, lds, rows, k, kpad, dst);
+  strip_launch(rows, kpad, [&](auto w, dim3 grid, dim3 block) {
+    copy_cols_padded_kernel<decltype(w)::value><<<grid, block, 0, stream>>>(src, lds, rows, k, kpad, dst);
+  });
   return cudaGetLastError();
 }
 cudaError_t gather_rows(const float* src, int64_t lds, const int32_t* idx, int64_t rows, int64_t cols, float* dst,
@@ -1180,7 +1197,9 @@ cudaError_t gather_rows(const float* src, int64_t lds, const int32_t* idx, int64
   if (rows * cols == 0) return cudaSuccess;
   ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
   count_launch();
-  gather_rows_kernel<<<strip_grid(rows, cols), kStripThreads, 0, stream>>>(src, lds, idx, rows, cols, dst, ldd);
+  strip_launch(rows, cols, [&](auto w, dim3 grid, dim3 block) {
+    gather_rows_kernel<decltype(w)::value><<<grid, block, 0, stream>>>(src, lds, idx, rows, cols, dst, ldd);
+  });
   return cudaGetLastError();
 }
 
@@ -1191,12 +1210,16 @@ cudaError_t scatter_cols(const T* src, int64_t lds, const int32_t* idx, int64_t 
   if (idx) {
     ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
     count_launch();
-    fill_zero_kernel<<<strip_grid(rows, n), kStripThreads, 0, stream>>>(dst, ldd, rows, n, skip_flag());
+    strip_launch(rows, n, [&](auto w, dim3 grid, dim3 block) {
+      fill_zero_kernel<decltype(w)::value><<<grid, block, 0, stream>>>(dst, ldd, rows, n, skip_flag());
+    });
   }
   if (rows * k == 0) return cudaGetLastError();
   count_launch();
-  scatter_cols_kernel<T><<<strip_grid(rows, k), kStripThreads, 0, stream>>>(src, lds, idx, rows, k, dst, ldd,
-                                                                      skip_flag());
+  strip_launch(rows, k, [&](auto w, dim3 grid, dim3 block) {
+    scatter_cols_kernel<decltype(w)::value, T><<<grid, block, 0, stream>>>(
+        src, lds, idx, rows, k, dst, ldd, skip_flag());
+  });
   return cudaGetLastError();
 }
 #define SP_INST(T)                                                                                                  \

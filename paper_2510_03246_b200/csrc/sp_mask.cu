@@ -871,9 +871,10 @@ __global__ void zero_cols_kernel(const uint8_t* mask, int group, float* W, int64
   }
 }
 
+template <int W>
 __global__ void __launch_bounds__(kStripThreads) mask_rows_copy_kernel(const uint8_t* mask, const float* src, int64_t lds, float* dst, int64_t ldd,
                                       int64_t rows, int64_t cols) {
-  for_strip(rows, cols, [&](int64_t i, int64_t j, int) {
+  for_strip<W>(rows, cols, [&](int64_t i, int64_t j, int) {
     dst[i * ldd + j] = mask[i] ? src[i * lds + j] : 0.f;
   });
 }
@@ -1338,27 +1339,29 @@ cudaError_t mask_to_index(const uint8_t* mask, int64_t n, int32_t* kept_idx, cud
   return cudaGetLastError();
 }
 
-__global__ void scale_block_kernel(float* C, int64_t ld, int64_t rows, int64_t cols, const int32_t* f_bits, int power,
-                                   const int32_t* skip) {
+template <int W>
+__global__ void __launch_bounds__(kStripThreads) scale_block_kernel(float* C, int64_t ld, int64_t rows, int64_t cols,
+                                                                    const int32_t* f_bits, int power,
+                                                                    const int32_t* skip) {
   if (skip != nullptr && *skip != 0) return;   // conditional launch (see SkipScope)
   const float f = __int_as_float(f_bits[0]);
   const float s = power == 2 ? f * f : f;
   // (all loads of a thread's rows before the stores: the compiler cannot know that they do not overlap)
-  const int64_t c0 = (int64_t)blockIdx.x * (kStripThreads * kStripPer) + threadIdx.x;
-  for (int64_t i = blockIdx.y; i < rows; i += 2 * (int64_t)gridDim.y) {
+  const int64_t c0 = strip_col<W>(), step = strip_rows<W>();
+  for (int64_t i = strip_row<W>(); i < rows; i += 2 * step) {
     float v[2][kStripPer];
 #pragma unroll
     for (int h = 0; h < 2; ++h)
 #pragma unroll
       for (int q = 0; q < kStripPer; ++q) {
-        const int64_t r = i + h * (int64_t)gridDim.y, j = c0 + q * kStripThreads;
+        const int64_t r = i + h * step, j = c0 + q * strip_width<W>();
         v[h][q] = r < rows && j < cols ? C[r * ld + j] : 0.f;
       }
 #pragma unroll
     for (int h = 0; h < 2; ++h)
 #pragma unroll
       for (int q = 0; q < kStripPer; ++q) {
-        const int64_t r = i + h * (int64_t)gridDim.y, j = c0 + q * kStripThreads;
+        const int64_t r = i + h * step, j = c0 + q * strip_width<W>();
         if (r < rows && j < cols) C[r * ld + j] = v[h][q] * s;
       }
   }
@@ -1410,12 +1413,13 @@ __global__ void __launch_bounds__(256) unpermute_gram_kernel(const float* __rest
   }
 }
 
+template <int W>
 __global__ void __launch_bounds__(kStripThreads) unpermute_cols_kernel(const float* __restrict__ Rp,
                                                                        const int32_t* __restrict__ perm, int64_t rows,
                                                                        int64_t n, float* __restrict__ R) {
   int64_t at[kStripPer];
-  strip_index(perm, n, at);
-  for_strip(rows, n, [&](int64_t r, int64_t j, int q) { R[r * n + at[q]] = Rp[r * n + j]; });
+  strip_index<W>(perm, n, at);
+  for_strip<W>(rows, n, [&](int64_t r, int64_t j, int q) { R[r * n + at[q]] = Rp[r * n + j]; });
 }
 
 __global__ void decay_tag_set_kernel(int32_t* tag, int k, float c, int valid, int h_ld, int h_chunk) {
@@ -1430,18 +1434,20 @@ __global__ void h_next_ready_kernel(const int32_t* same, const int32_t* tag, int
   ready[1] = 1 - ready[0];
 }
 
+template <int W>
 __global__ void __launch_bounds__(kStripThreads) unpermute_rows_kernel(const float* __restrict__ Rp,
                                                                        const int32_t* __restrict__ perm, int64_t n,
                                                                        int64_t cols, float* __restrict__ R) {
-  for_strip(n, cols, [&](int64_t i, int64_t j, int) { R[(int64_t)perm[i] * cols + j] = Rp[i * cols + j]; });
+  for_strip<W>(n, cols, [&](int64_t i, int64_t j, int) { R[(int64_t)perm[i] * cols + j] = Rp[i * cols + j]; });
 }
 
 cudaError_t scale_block(float* C, int64_t ld, int64_t rows, int64_t cols, const int32_t* f_bits, int power,
                         cudaStream_t stream) {
   if (rows * cols <= 0) return cudaSuccess;
   count_launch();
-  scale_block_kernel<<<strip_grid(rows, cols), kStripThreads, 0, stream>>>(
-      C, ld, rows, cols, f_bits, power, skip_flag());
+  strip_launch(rows, cols, [&](auto w, dim3 grid, dim3 block) {
+    scale_block_kernel<decltype(w)::value><<<grid, block, 0, stream>>>(C, ld, rows, cols, f_bits, power, skip_flag());
+  });
   return cudaGetLastError();
 }
 
@@ -1459,7 +1465,9 @@ cudaError_t unpermute_cols(const float* Rp, const int32_t* perm, int64_t rows, i
                            cudaStream_t stream) {
   if (rows * n <= 0) return cudaSuccess;
   count_launch();
-  unpermute_cols_kernel<<<strip_grid(rows, n), kStripThreads, 0, stream>>>(Rp, perm, rows, n, R);
+  strip_launch(rows, n, [&](auto w, dim3 grid, dim3 block) {
+    unpermute_cols_kernel<decltype(w)::value><<<grid, block, 0, stream>>>(Rp, perm, rows, n, R);
+  });
   return cudaGetLastError();
 }
 
@@ -1481,7 +1489,9 @@ cudaError_t unpermute_rows(const float* Rp, const int32_t* perm, int64_t n, int6
                            cudaStream_t stream) {
   if (n * cols <= 0) return cudaSuccess;
   count_launch();
-  unpermute_rows_kernel<<<strip_grid(n, cols), kStripThreads, 0, stream>>>(Rp, perm, n, cols, R);
+  strip_launch(n, cols, [&](auto w, dim3 grid, dim3 block) {
+    unpermute_rows_kernel<decltype(w)::value><<<grid, block, 0, stream>>>(Rp, perm, n, cols, R);
+  });
   return cudaGetLastError();
 }
 
@@ -1538,7 +1548,9 @@ cudaError_t mask_rows_copy(const uint8_t* mask, const float* src, int64_t lds, f
   if (rows * cols == 0) return cudaSuccess;
   ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
   count_launch();
-  mask_rows_copy_kernel<<<strip_grid(rows, cols), kStripThreads, 0, stream>>>(mask, src, lds, dst, ldd, rows, cols);
+  strip_launch(rows, cols, [&](auto w, dim3 grid, dim3 block) {
+    mask_rows_copy_kernel<decltype(w)::value><<<grid, block, 0, stream>>>(mask, src, lds, dst, ldd, rows, cols);
+  });
   return cudaGetLastError();
 }
 

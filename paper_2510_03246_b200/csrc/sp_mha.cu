@@ -94,7 +94,7 @@ __global__ void __launch_bounds__(kRowWarps * 32) softmax_rows_kernel(float* __r
 
 // Gradient step of Eq. (85) on the attention probabilities of every (sequence, head) pair:
 //   P <- P - eta_b (-2 alpha G1 + 2 beta (P - Phi)),  G1 = R V^T from the preceding product, eta_b per pair.
-// gridDim.y walks the pairs, a thread takes V neighbouring entries (V = 4: 16-byte accesses).
+// gridDim.y and blockDim.y walk the pairs, a thread takes V neighbouring entries (V = 4: 16-byte accesses).
 template <int V>
 __global__ void __launch_bounds__(256) p_update_kernel(float* __restrict__ P, const float* __restrict__ Phi,
                                                        const float* __restrict__ G1, const float* __restrict__ eta,
@@ -102,9 +102,10 @@ __global__ void __launch_bounds__(256) p_update_kernel(float* __restrict__ P, co
                                                        __nv_bfloat16* __restrict__ Pb, int64_t plane) {
   struct __align__(4 * V) F { float v[V]; };
   struct __align__(2 * V) H { __nv_bfloat16 v[V]; };
-  for (int64_t b = blockIdx.y; b < pairs; b += gridDim.y) {
+  for (int64_t b = strip_row(); b < pairs; b += strip_rows()) {
     const float et = eta[b];
-    for (int64_t i = ((int64_t)blockIdx.x * 256 + threadIdx.x) * V; i < per_pair; i += (int64_t)gridDim.x * 256 * V) {
+    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * V; i < per_pair;
+         i += (int64_t)gridDim.x * blockDim.x * V) {
       const int64_t e = b * per_pair + i;
       const F p = *reinterpret_cast<const F*>(P + e), ph = *reinterpret_cast<const F*>(Phi + e),
               g1 = *reinterpret_cast<const F*>(G1 + e);
@@ -220,10 +221,10 @@ __global__ void __launch_bounds__(256) z_update_kernel(float* __restrict__ Zq, f
                                                        __nv_bfloat16* __restrict__ Zks, int64_t plane) {
   struct __align__(4 * V) F { float v[V]; };
   struct __align__(2 * V) B { __nv_bfloat16 v[V]; };
-  const int H = d / d_h, c = ((int)blockIdx.x * 256 + (int)threadIdx.x) * V;
+  const int H = d / d_h, c = (int)(blockIdx.x * blockDim.x + threadIdx.x) * V;
   if (c >= d) return;
   const int head = c / d_h;
-  for (int64_t tok = blockIdx.y; tok < tokens; tok += gridDim.y) {
+  for (int64_t tok = strip_row(); tok < tokens; tok += strip_rows()) {
     const int64_t e = tok * d + c;
     const float et = eta[(tok / T) * H + head];
     const auto step = [&](float* Z, const float* G, const float* Tg, __nv_bfloat16* S) {
@@ -303,14 +304,17 @@ cudaError_t mha_p_update(float* P, const float* Phi, const float* G1, const floa
   const int64_t per_pair = (int64_t)T * T;
   const auto al = [](const void* p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; };
   const bool vec = per_pair % 4 == 0 && plane % 4 == 0 && al(P, 16) && al(Phi, 16) && al(G1, 16) && al(Pb, 8);
-  int64_t gx = ceil_div(per_pair, (int64_t)(vec ? 1024 : 256)), gy = pairs < 65535 ? pairs : 65535;
+  const int V = vec ? 4 : 1;
+  const dim3 block = strip_block(ceil_div(per_pair, (int64_t)V));
+  int64_t gx = ceil_div(per_pair, (int64_t)block.x * V), gy = ceil_div(pairs, (int64_t)block.y);
+  if (gy > 65535) gy = 65535;
   const int64_t cap = (int64_t)sm_count() * 16;
   if (gx > cap) gx = cap;
   if (gx * gy > cap) gy = cap / gx > 0 ? cap / gx : 1;
   const dim3 grid((unsigned)gx, (unsigned)gy);
   __nv_bfloat16* pb = reinterpret_cast<__nv_bfloat16*>(Pb);
-  if (vec) p_update_kernel<4><<<grid, 256, 0, stream>>>(P, Phi, G1, eta, per_pair, pairs, (float)alpha, (float)beta, pb, plane);
-  else p_update_kernel<1><<<grid, 256, 0, stream>>>(P, Phi, G1, eta, per_pair, pairs, (float)alpha, (float)beta, pb, plane);
+  if (vec) p_update_kernel<4><<<grid, block, 0, stream>>>(P, Phi, G1, eta, per_pair, pairs, (float)alpha, (float)beta, pb, plane);
+  else p_update_kernel<1><<<grid, block, 0, stream>>>(P, Phi, G1, eta, per_pair, pairs, (float)alpha, (float)beta, pb, plane);
   return cudaGetLastError();
 }
 
@@ -352,11 +356,13 @@ cudaError_t mha_z_update(float* Zq, float* Zk, const float* Gq, const float* Gk,
   const auto al = [](const void* p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; };
   const bool vec = d_h % 4 == 0 && plane % 4 == 0 && al(Zq, 16) && al(Zk, 16) && al(Gq, 16) && al(Gk, 16) && al(Tq, 16) &&
                    al(Tk, 16) && al(Zqs, 8) && al(Zks, 8);
-  const int64_t gx = ceil_div(d, vec ? 1024 : 256);
+  const int V = vec ? 4 : 1;
+  const dim3 block = strip_block(ceil_div(d, V));
+  const int64_t gx = ceil_div(d, (int)block.x * V), row_blocks = ceil_div(tokens, (int64_t)block.y);
   int64_t gy = ceil_div((int64_t)sm_count() * 8, gx);
-  if (gy > tokens) gy = tokens;
+  if (gy > row_blocks) gy = row_blocks;
   const auto run = [&](auto kernel) {
-    kernel<<<dim3((unsigned)gx, (unsigned)gy), 256, 0, stream>>>(Zq, Zk, Gq, Gk, Tq, Tk, eta, tokens, d, T, d_h, (float)alpha,
+    kernel<<<dim3((unsigned)gx, (unsigned)gy), block, 0, stream>>>(Zq, Zk, Gq, Gk, Tq, Tk, eta, tokens, d, T, d_h, (float)alpha,
                                                                  reinterpret_cast<__nv_bfloat16*>(Zqs),
                                                                  reinterpret_cast<__nv_bfloat16*>(Zks), plane);
   };

@@ -304,3 +304,25 @@ def test_calls_on_the_callers_stream_alone_from_several_threads():
     torch.cuda.synchronize()
     for k in range(len(jobs)):
         assert len(got[k]) == 8 and all(torch.equal(a, b) for r in got[k] for a, b in zip(r, want[k]))
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 8, 31, 33, 64, 100, 128, 200, 255, 257, 520])
+@pytest.mark.parametrize("precise", [False, True])
+def test_refit_of_narrow_matrices(n, precise):
+    """Right-hand sides of few columns: the kernels that gather, clear and scatter them put several rows into a block."""
+    api = _api()
+    m, k = 1237, (n + 1) // 2
+    g = torch.Generator(device="cuda").manual_seed(n)
+    G, R = _spd(n, n), torch.randn(m, n, generator=g, device="cuda")
+    keep = torch.sort(torch.randperm(n, generator=g, device="cuda")[:k]).values
+    mask = torch.zeros(n, dtype=torch.uint8, device="cuda")
+    mask[keep] = 1
+    W = torch.full((m + 1, n + 3), 7.0, device="cuda")
+    api.sp_linear_refit(R, G, mask, k, 0.1, precise=precise, W=W[:m, :n], rho_relative=True)
+    H = G[keep][:, keep].double() + 0.1 * G.double().diagonal().mean() * torch.eye(k, device="cuda", dtype=torch.float64)
+    want = torch.zeros(m, n, dtype=torch.float64, device="cuda")
+    want[:, keep] = torch.linalg.solve(H, R[:, keep].double().T).T
+    # fp64: rounded to fp32 once; fp32: a few 2^-24 times the condition number (the ridge bounds it by 10 n)
+    bound = 1.2e-7 if precise else 4 * 2.0 ** -24 * 10 * max(n, 10)
+    assert float((W[:m, :n].double() - want).abs().max() / want.abs().max()) < bound
+    assert bool((W[:m, :n][:, mask == 0] == 0).all()) and bool((W[m] == 7).all()) and bool((W[:, n:] == 7).all())
