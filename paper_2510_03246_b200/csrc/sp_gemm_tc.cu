@@ -869,8 +869,8 @@ sp_status gemm_tc(int64_t M, int64_t N, int64_t K, float alpha, TcOperand A, TcO
   if (C.lo_off < 0 || (C.lo_off > 0 && C.dtype != SP_BF16)) return SP_ERR_INVALID_ARG;
   p.a_kmajor = A.kmajor ? 1 : 0;
   p.b_kmajor = B.kmajor ? 1 : 0;
-  if (narrow) lower_only = false;
-  p.lower_only = lower_only ? 1 : 0;
+  const bool skip_tiles = lower_only && !narrow;      // the narrow tile is taken where a wide one would cover all columns
+  p.lower_only = skip_tiles ? 1 : 0;
   // fp32 C that a tensor map can describe leaves through TMA: a store when nothing is added, an add-reduction when
   // the call accumulates into C itself (each element of C is touched once per launch, so the result is the same sum)
   p.epi_mode = EPI_DIRECT;
@@ -907,7 +907,7 @@ sp_status gemm_tc(int64_t M, int64_t N, int64_t K, float alpha, TcOperand A, TcO
   p.tiles_n = (int32_t)ceil_div(N, tile_n);
   // consecutive tiles (which run at the same time on neighbouring SMs) should share the larger operand panel
   p.n_fast = p.tiles_n < p.tiles_m ? 1 : 0;
-  if (lower_only) {
+  if (skip_tiles) {
     int64_t cnt = 0;
     for (int tn = 0; tn < p.tiles_n && tn < p.tiles_m; ++tn) cnt += p.tiles_m - tn;
     p.num_tiles = (int32_t)cnt;

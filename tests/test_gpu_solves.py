@@ -67,6 +67,23 @@ def test_gemm_tensor_core_tiles_of_both_widths(a_kmajor, b_kmajor, M, N, K, lowe
         assert float(off[keep].max()) <= 0
 
 
+@pytest.mark.parametrize("M,N,K,lower", [(256, 256, 64, True), (128, 96, 64, True), (1288, 256, 768, True), (520, 520, 128, True),
+                                         (256, 256, 64, False)])
+def test_profile_counts_the_operations_of_a_lower_triangle(M, N, K, lower):
+    """The triangle of the leading N x N square and the rows below it, whichever tile computes them."""
+    api = _api()
+    A, B = (torch.ones(r, K, device="cuda", dtype=torch.bfloat16) for r in (M, N))
+    C = torch.zeros(M, N, device="cuda")
+    api.sp_profile_begin(1)
+    try:
+        api.sp_gemm(A, B, C, False, True, lower_only=lower, use_tensor_cores=True)
+        torch.cuda.synchronize()
+        got = api.sp_profile_read()["gemm_tc"]
+    finally:
+        api.sp_profile_begin(0)
+    assert got["records"] == 1 and got["flops"] == (K * N * (2 * M - N) if lower else 2 * M * N * K)
+
+
 def _spd(n, seed):
     g = torch.Generator(device="cuda").manual_seed(seed)
     X = torch.randn(2 * n + 3, n, generator=g, device="cuda") * torch.logspace(0, 1.5, n, device="cuda")
