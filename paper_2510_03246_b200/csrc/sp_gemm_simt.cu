@@ -153,7 +153,7 @@ struct DmmaSlab {
   static constexpr int PITCH = FAST + DM_PAD, VPR = FAST / V, CNT = OUTER * VPR / DM_THREADS;
   static constexpr int ELEMS = OUTER * PITCH;
   static_assert(OUTER * VPR % DM_THREADS == 0, "slab / thread mismatch");
-  T r[CNT][V];
+  alignas(16) T r[CNT][V];      // written 16 bytes at a time, wherever the compiler keeps it
 
   // d0: first index of the tile along M / N, k0: first K index, dim / kend: extents
   __device__ __forceinline__ void fetch(const T* p, int64_t ld, bool vec, int64_t d0, int64_t k0, int64_t dim,
@@ -192,6 +192,7 @@ gemm_dmma_kernel(int64_t M, int64_t N, int64_t K, double alpha, const T* A, int6
                  const T* B, int64_t ldb, double beta, Operand Cin, OutOperand C, int lower_only, int k_tri) {
   using SlabA = DmmaSlab<T, A_KFAST, BM>;
   using SlabB = DmmaSlab<T, B_KFAST, DM_BN>;
+  static_assert(alignof(SlabA) % 16 == 0 && alignof(SlabB) % 16 == 0, "16-byte pieces");
   constexpr int WM = BM / 2, MT = WM / 16;      // rows of a warp, its 16-row tiles
   const int64_t row0 = (int64_t)blockIdx.y * BM, col0 = (int64_t)blockIdx.x * DM_BN;
   if (lower_only && row0 + BM - 1 < col0) return;
