@@ -488,8 +488,11 @@ sp_status sp_ridge_solve(const float* R, int64_t ldr, const float* G, int64_t ld
   // (the precise form keeps to the caller's stream: it shares nothing with other streams, threads or captures)
   if (precise) return ridge_core<double>(R, ldr, G, ldg, m, n, nullptr, n, b.rho, W, ldw, b, status_dev, s);
   SideStream* side = side_stream();
-  return ridge_core<float>(R, ldr, G, ldg, m, n, nullptr, n, b.rho, W, ldw, b, status_dev, s,
-                           side ? &side->assist_main : nullptr);
+  JoinOnExit join_guard{side, s};
+  SPCHK(ridge_core<float>(R, ldr, G, ldg, m, n, nullptr, n, b.rho, W, ldw, b, status_dev, s,
+                          side ? &side->assist_main : nullptr));
+  join_guard.armed = false;
+  return SP_OK;
 }
 
 sp_status sp_linear_refit(const float* R, int64_t ldr, const float* G, int64_t ldg, int64_t m, int64_t n_units,
@@ -519,8 +522,11 @@ sp_status sp_linear_refit(const float* R, int64_t ldr, const float* G, int64_t l
   }
   if (precise) return ridge_core<double>(R, ldr, G, ldg, m, n, b.idx, k, b.rho, W, ldw, b, status_dev, s);
   SideStream* side = side_stream();
-  return ridge_core<float>(R, ldr, G, ldg, m, n, b.idx, k, b.rho, W, ldw, b, status_dev, s,
-                           side ? &side->assist_main : nullptr);
+  JoinOnExit join_guard{side, s};
+  SPCHK(ridge_core<float>(R, ldr, G, ldg, m, n, b.idx, k, b.rho, W, ldw, b, status_dev, s,
+                          side ? &side->assist_main : nullptr));
+  join_guard.armed = false;
+  return SP_OK;
 }
 
 sp_status sp_struct_scores(int32_t kind, int32_t group, const sp_score_inputs* in, int64_t n_units, float* scores,
