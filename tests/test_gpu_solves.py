@@ -192,8 +192,9 @@ def test_two_level_sweep_of_a_large_system(n, m):
 
 @pytest.mark.parametrize("n,rows", [(4, 5), (64, 64), (72, 33), (200, 130), (1096, 70)])
 def test_ordered_accumulators_come_back_in_channel_order(n, rows):
-    """A module whose token pass works with the kept channels first: G_A (both triangles), R1 and R2 in channel order
-    equal the products over the tokens, at the edges of the 32 x 32 tiles and of the 1024-column strips."""
+    """A module whose token pass works with the kept channels first: G_A (both triangles, from the lower one), R1 and R2 in
+    channel order hold the entries of the ordered buffers, at the edges of the 32 x 32 tiles and of the 1024-column strips, and
+    R1 is the product over the tokens."""
     api = _api()
     g = torch.Generator(device="cuda").manual_seed(n)
     d, N, k = 64, 8 * rows, max(1, n // 3)
@@ -207,11 +208,13 @@ def test_ordered_accumulators_come_back_in_channel_order(n, rows):
     for _ in range(2):
         mod.sp_admm_step(p)
     mod.check_status()
-    assert torch.equal(mod.G_A, mod.G_A.T)
     want = mod.Z.double().T @ mod.X.double()
     # (Z enters the product as bf16: one rounding of 2^-9 per term)
     assert float((mod.R1.double() - want).abs().max()) < 2.0 ** -9 * float((mod.Z.double().abs().T @ mod.X.double().abs()).max())
-    assert torch.allclose(mod.G_A.diagonal(), mod.G_A_perm.diagonal()[torch.argsort(mod.decay_tag[8:8 + n])])
+    inv = torch.argsort(mod.decay_tag[8:8 + n])
+    ordered = torch.tril(mod.G_A_perm) + torch.tril(mod.G_A_perm, -1).T
+    assert torch.equal(mod.G_A, ordered[inv][:, inv])
+    assert torch.equal(mod.R1, mod.R1_perm[inv]) and torch.equal(mod.R2, mod.R2_perm[:, inv])
 
 
 @pytest.mark.parametrize("d", [8, 64, 72, 136, 520, 1096])
