@@ -32,13 +32,14 @@
  *     them from one host thread at a time.  All other calls, sp_ffn_cache_input_inverse and the precise solves among
  *     them, use the caller's stream alone.  Nothing else persists inside the library.
  *   - Reproducibility: by default a product whose tile count leaves SMs idle is cut along K and its partial
- *     products add up in C in an order that is not fixed, and the backward triangular solve adds updates from two
- *     streams; fp32 results (accumulators, recovered weights, scores) can then differ in their last bits between two
- *     runs on equal inputs, and a mask can differ at scores that tie within that rounding.  sp_set_reproducible(1)
- *     switches both off (process-wide): every sum is then taken in an order fixed by the call's arguments and equal
- *     inputs give bit-identical outputs, at a few per cent of the step time.  The fp32 mode (fp64 accumulation on the
- *     CUDA cores, fp64 factorisation) and the score, statistics, report and selection kernels are reproducible either
- *     way.
+ *     products add up in C in an order that is not fixed, and a factorisation adds updates of its trailing matrix from
+ *     two streams (a backward sweep too, for more right-hand sides than one wave of its panels holds); fp32 results
+ *     (accumulators, recovered weights, scores) can then differ in their last bits between two runs on equal inputs,
+ *     and a mask can differ at scores that tie within that rounding.  sp_set_reproducible(1) switches both off
+ *     (process-wide): every sum is then taken in an order fixed by the call's arguments and equal inputs give
+ *     bit-identical outputs, at a few per cent of the step time.  The fp32 mode (fp64 accumulation on the fp64 matrix
+ *     instruction, fp64 factorisation) and the score, statistics, report and selection kernels are reproducible
+ *     either way.
  *   - Symmetric accumulators (Gram matrices) are stored as full squares; calls that update them keep the LOWER
  *     triangle (including the diagonal) authoritative.  sp_symmetrize() mirrors it to the upper triangle.
  */

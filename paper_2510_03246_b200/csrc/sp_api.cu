@@ -33,8 +33,8 @@ struct MatRef {
 
 // C[M,N] = alpha * sum_k A(i,k) B(k,j) + beta * Cin.
 //   a_kmajor: A stored [M,K] (ld) else [K,M];  b_kmajor: B stored [N,K] (ld) else [K,N].
-// bf16 operands go to the tensor-core kernel when its alignment rules hold; everything else (and the fp32 mode,
-// which accumulates in fp64) runs on the CUDA-core kernel.
+// bf16 operands go to the bf16 tensor-core kernel when its alignment rules hold; the fp32 mode (fp64 accumulation) runs on
+// the fp64 matrix instruction, everything else on the CUDA cores.
 sp_status contract(int64_t M, int64_t N, int64_t K, double alpha, MatRef A, bool a_kmajor, MatRef B, bool b_kmajor,
                    double beta, MatRef Cin, MatRef C, bool lower_only, bool acc64, bool allow_tc, int32_t* status,
                    cudaStream_t stream) {
@@ -1238,7 +1238,7 @@ struct BMat {
 
 // C_b = alpha * sum over segments A_b[plane pa] B_b[plane pb] + beta * Cin_b for all nb0 x nb1 pairs.
 // bf16 operands: one batched tensor-core launch.  fp32 operands (fp32 mode): plane 0 holds the full value, the
-// segments collapse to one product per pair on the CUDA cores with fp64 accumulation.
+// segments collapse to one product per pair with fp64 accumulation.
 sp_status bcontract(int64_t M, int64_t N, int64_t K, double alpha, BMat A, bool a_kmajor, BMat B, bool b_kmajor,
                     int nseg, const int* pa, const int* pb, double beta, BMat Cin, BMat C, int64_t c_lo_off, int nb0,
                     int nb1, int32_t* status, cudaStream_t s) {

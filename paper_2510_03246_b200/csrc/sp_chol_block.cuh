@@ -25,9 +25,8 @@ __device__ __forceinline__ double recip_sqrt(double x) { return rsqrt(x); }
 //      sub-block comes first, by all warps; the other pieces run beside the next phase A.
 // Every entry receives its updates column by column in ascending order, whatever the blocking.  What bounds the kernel is
 // latency: A (about 120 cycles per column), B and the first piece of C; for 128 columns the other pieces take as long as
-// A.  Measured inside a factorisation: 25 us for 128 columns in fp32, 14 us for 64 in fp64.  The form before this one held
-// one 4 x 4 block per thread; two block barriers and all warps' shared update stood between one 4 x 4 pivot block and the
-// next (37 and 20 us, the same operations in the same order).
+// A.  Measured inside a factorisation: 25 us for 128 columns in fp32, 14 us for 64 in fp64.  (One 4 x 4 block per thread,
+// with two block barriers and all warps' shared update between one 4 x 4 pivot block and the next: 37 and 20 us.)
 template <typename T, int NB>
 struct DiagBlock {
   static constexpr int SB = 32, NS = NB / SB;

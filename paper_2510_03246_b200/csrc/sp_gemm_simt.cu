@@ -130,12 +130,12 @@ gemm_simt_kernel(int64_t M, int64_t N, int64_t K, Acc alpha, Operand A, Operand 
 //
 // A 64 x 64 (or 32 x 64) tile per block of four warps, each 32 x 32 (16 x 32): per 8 values of K a warp issues eight
 // m16n8k8 instructions on fragments of 16 eight-byte shared-memory reads, so the fp64 pipe (64 fused multiply-adds per
-// SM and cycle) is the bound and not shared memory, as it was for the scalar kernel (16 fused multiply-adds per 8 reads and a
+// SM and cycle) is the bound and not shared memory, which bounds scalar products (16 fused multiply-adds per 8 reads and a
 // conversion of every element on its way in).  Operands stay in their stored orientation in shared memory; a pitch of 4
 // doubles beyond a multiple of 16 makes every fragment read conflict-free in both orientations.  The next K slab travels
 // through registers (16-byte loads, fp32 widened there) while the current one is multiplied; small blocks let three
 // of them share an SM, which hides the prologue and the read-modify-write of C in the K = 64 updates of the factorisation.
-// Measured: token contractions of fp32 operands (3072 x 3072 lower, K = 2048) 29 TFLOP/s; the scalar kernel made 12.
+// Measured: token contractions of fp32 operands (3072 x 3072 lower, K = 2048) 29 TFLOP/s, scalar 12.
 constexpr int DM_BN = 64, DM_BK = 16, DM_THREADS = 128, DM_PAD = 4;
 
 __device__ __forceinline__ void dmma_16x8x8(double (&d)[4], const double (&a)[4], const double (&b)[2]) {

@@ -2,7 +2,7 @@
 // mode and for the cached inverse of the input system.  The O(n^3) and O(m n^2) work is GEMMs on the diagonal-block
 // inverses; only the 64 x 64 diagonal factorisation runs in a single thread block.  What bounds it: up to n of a few
 // thousand the chain diagonal block -> panel -> next block column (about 33 us per 64 columns), above that the fp64 pipe.
-// The inverse of a 4096-wide input system takes 8 ms (42 ms with scalar fp64 products and a solve for 4096 columns).
+// The inverse of a 4096-wide input system takes 5.4 ms (36 ms with scalar fp64 products and a solve for 4096 columns).
 #include "sp_chol_block.cuh"
 #include "sp_common.cuh"
 

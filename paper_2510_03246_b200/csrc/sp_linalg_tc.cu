@@ -667,14 +667,15 @@ sp_status potrs_right_tc(float* X, int64_t m, int64_t n, int64_t ldx, const void
   // without it everything stays on one stream.
   const bool x_al16 = (ldx % 4 == 0) && ((reinterpret_cast<uintptr_t>(X) & 15u) == 0);
   if (!x_al16) assist = nullptr;
-  // Reproducible mode: the far update of a step (assisting stream) and the next step's near update would add into the
-  // same columns in an order that depends on timing; on one stream every column receives its updates in step order.
+  // Reproducible mode stays on one stream, where every column receives its updates in step order.  With an assisting stream
+  // a far update and the next step's near update add into the same columns in an order that depends on timing, unless the
+  // panel pulls the near update (fuse_near: added last, in either mode).
   if (reproducible_mode()) assist = nullptr;
   // Backward sweep: the update by the previous block column can ride in the panel kernel (fp32, from the fp32 factor)
   // when the factor's rows are 16-byte aligned too.
   // (its 144 KB of shared memory allow one CTA per SM: only while all row blocks fit in one wave)
   const bool fuse_near = Lf != nullptr && x_al16 && (ldl % 4 == 0) && ((reinterpret_cast<uintptr_t>(Lf) & 15u) == 0) &&
-                         ceil_div(m, (int64_t)32) <= 148;
+                         ceil_div(m, (int64_t)32) <= sm_count();
   // Backward sweep: a panel runs beside the far update of the step before, whose CTAs take a whole SM each; one that has to
   // wait for SMs lengthens the chain by the update's time.  So the panel gets half of the SMs and the update the rest,
   // unless the update has so many tiles that the two one after the other, each with all SMs, are shorter.  Measured on the
@@ -875,7 +876,7 @@ sp_status potrf_potrs_tc_batched(float* A, int64_t n, int64_t m, int batch, int6
   // ---- backward sweep W L = Y on the appended rows, block columns right to left
   float* X = A + n * lda;                       // [m, n] per system
   const int64_t lds = 3 * TB, xs_bs = 2 * m * lds;
-  const bool fuse_near = ceil_div(m, (int64_t)32) * batch <= 148;
+  const bool fuse_near = ceil_div(m, (int64_t)32) * batch <= sm_count();
   TcBatch bs = bt;
   bs.a_s0 = bs.a_s1 = xs_bs;
   for (int64_t step = 0; step < nblk; ++step) {
