@@ -261,7 +261,11 @@ struct DiagBlock {
         for (int v = 0; v < V; ++v) inv[(cs + c + v) * NB + t] = q.v[v];
       }
     };
-    for (int s = 0; s < NS; ++s) {
+    // sub-blocks beyond nb are those of an identity: nothing is eliminated there, their columns of X stay as they are (a
+    // solve for 17 unknowns in fp32: 53 us, 65 through all four).  Two sub-blocks (fp64) are always run: a bound known at
+    // compile time is worth more there (1 % of a fp32-mode layer).
+    const int ns = NS > 2 ? (nb + SB - 1) / SB : NS;
+    for (int s = 0; s < ns; ++s) {
       const int cs = s * SB, ce = cs + SB;
       if (warp == NW - 1) {
         factor(M + cs * P + cs, LT, CI, lane, row0 + cs, status);
@@ -270,7 +274,7 @@ struct DiagBlock {
         // The factorising warp shares its scheduler with warp 3, which comes last; warps 3 to 6 also store.
         const int ps = cs - SB;
         int turn = 0;
-        for (int cb = s; cb < NS; ++cb)
+        for (int cb = s; cb < ns; ++cb)
           for (int rb = cb == s ? s + 1 : cb; rb < NS + s; ++rb) {             // ((s, s) is done before)
             const int w = turn++ % (NW - 1);
             if (warp == (w < 3 ? w : w < 6 ? w + 1 : 3))
@@ -281,13 +285,14 @@ struct DiagBlock {
       __syncthreads();
       if (t < NB) solve_row((t >= ce ? M : X) + t * P + cs, LT, CI);
       __syncthreads();
-      if (ce < NB) {
+      if (s + 1 < ns) {
         // next diagonal sub-block, 32 x 4 entries per warp
         rank32<1>(M, ce, ce + warp * 4, cs, (ce + warp * 4) * P + cs, lane);
         __syncthreads();
       }
     }
-    if (t >= STORE0) store_inv(NB - SB);
+    if (t >= STORE0)
+      for (int cs = (ns - 1) * SB; cs < NB; cs += SB) store_inv(cs);
   }
 };
 

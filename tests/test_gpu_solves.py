@@ -125,6 +125,18 @@ def test_tensor_core_ridge_solve_at_block_edges(n, m):
     assert status[:2].tolist() == [6, i]      # SP_ERR_NOT_SPD and the pivot
 
 
+@pytest.mark.parametrize("n", [1, 2, 17, 31, 32, 33, 64, 65, 96, 97, 127])
+def test_partial_diagonal_block_equals_the_whole_one(n):
+    """A system that fills part of a diagonal block is eliminated up to its last sub-block only: the same bits as beside an
+    identity that fills the block."""
+    api = _api()
+    G, R = _spd(n, n), torch.randn(70, n, generator=torch.Generator(device="cuda").manual_seed(n), device="cuda")
+    whole, Rw = torch.eye(128, device="cuda"), torch.zeros(70, 128, device="cuda")
+    whole[:n, :n], Rw[:, :n] = G, R
+    got, want = api.sp_ridge_solve(R, G, 0.5, False), api.sp_ridge_solve(Rw, whole, 0.5, False)
+    assert torch.equal(got, want[:, :n])
+
+
 def _diagonal(lo, hi, n=128):
     """Diagonal matrix with entries over 2^lo .. 2^hi, mantissas spread."""
     e = torch.linspace(lo, hi, n, dtype=torch.float64, device="cuda")
