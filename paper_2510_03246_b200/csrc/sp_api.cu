@@ -2,6 +2,7 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "sp_common.cuh"
@@ -1606,16 +1607,16 @@ struct ValueRefitPlan {
   int64_t dh, sc, cap;
   bool bf16;
   SolveBufs sb, sb2;   // two sets: the systems of the heads are independent and are solved two at a time
-  void* Pb;     // bf16 mode: hi / lo planes of P of one chunk, [2][sc H, T, T]
-  void* Ab;     // bf16 mode: Aattn of one chunk as bf16 hi | lo parts, [cap, 2 pad64(d)]
-  void* R;      // regressors of one head and chunk: bf16 hi | lo [cap, 2 pad64(d)], or fp32 [cap, d]
-  float* G;     // [H][d, d]   sum over sequences of R^T R per head (lower triangle)
-  float* Cv;    // [H][d_h, d] sum over sequences of Aattn_i^T R per head
-  // the heads' systems solved together (bf16 mode, d a multiple of the solver's block): see potrf_potrs_tc_batched
+  int64_t hg, dq;      // bf16 mode: heads whose products are formed together (at most); columns of R's hi part
+  void* Pb;     // bf16 mode: hi / lo planes of P of one chunk and group, [2][sequences, heads, T, T]
+  void* R;      // bf16 mode: per head of the group [cap, 2 dq]: regressors (d columns) beside the head's Aattn (d_h columns),
+                // hi | lo; fp32 mode: regressors of one head, [cap, d]
+  float* G;     // per kept head [d + d_h, d]: sum over sequences of R^T R (lower triangle) and, below it, of Aattn_i^T R
+  // the heads' systems solved together, in place in G (bf16 mode, d a multiple of the solver's block): see
+  // potrf_potrs_tc_batched
   bool batched;
-  float *Gs_all, *dinv_all;
+  float* dinv_all;
   void *P_all, *Xs_all;
-  double* rho_all;
   size_t bytes;
 };
 
@@ -1631,24 +1632,41 @@ ValueRefitPlan plan_value_refit(void* ws, int64_t d, int64_t H, int64_t T, int64
   Carver c(ws);
   p.sb = carve_solve(c, d, p.dh, p.bf16 ? 4 : 8);
   p.sb2 = carve_solve(c, d, p.dh, p.bf16 ? 4 : 8);
-  p.Pb = p.bf16 ? c.take_bytes((size_t)2 * p.sc * H * T * T * 2) : nullptr;
-  p.Ab = p.bf16 ? c.take_bytes((size_t)p.cap * 2 * split_kpad(d) * 2) : nullptr;
-  p.R = c.take_bytes(p.bf16 ? (size_t)p.cap * 2 * split_kpad(d) * 2 : (size_t)p.cap * d * 4);
-  p.G = c.take<float>((size_t)H * d * d);
-  p.Cv = c.take<float>((size_t)d * d);
+  p.dq = split_kpad(d + p.dh);
+  p.Pb = nullptr;
+  p.hg = 1;
+  if (p.bf16) {
+    // half a GB is room for enough heads to fill the SM pairs at every width (d = 2048, 8192 tokens: seven heads)
+    const size_t per_head = (size_t)p.cap * 2 * p.dq * 2 + (size_t)2 * p.sc * T * T * 2;
+    p.hg = (int64_t)((size_t)(512u << 20) / per_head);
+    p.hg = std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(H, kMaxHeadGroup), p.hg));
+    p.Pb = c.take_bytes((size_t)2 * p.sc * p.hg * T * T * 2);
+  }
+  p.R = c.take_bytes(p.bf16 ? (size_t)p.hg * p.cap * 2 * p.dq * 2 : (size_t)p.cap * d * 4);
+  p.G = c.take<float>((size_t)H * (d + p.dh) * d);
   p.batched = p.bf16 && d % kCholTcNB == 0;
-  p.Gs_all = p.dinv_all = nullptr;
+  p.dinv_all = nullptr;
   p.P_all = p.Xs_all = nullptr;
-  p.rho_all = nullptr;
   if (p.batched) {
-    p.rho_all = c.take<double>((size_t)H);
-    p.Gs_all = c.take<float>((size_t)H * (d + p.dh) * d);
     p.dinv_all = c.take<float>((size_t)H * dinv_elems(d));
     p.P_all = c.take_bytes((size_t)H * (d + p.dh) * 3 * d * 2);
     p.Xs_all = c.take_bytes((size_t)H * 2 * p.dh * 3 * kCholTcNB * 2);
   }
   p.bytes = align_up(c.off, 256);
   return p;
+}
+
+// Heads per launch: the Gram products of g heads are g times as many tiles, and whole waves of SM pairs take equal time;
+// the largest group with the fewest waves over all nk heads.
+int64_t value_refit_group(int64_t nk, int64_t max_group, int64_t d, int64_t dh) {
+  const int64_t tm = ceil_div(d + dh, (int64_t)256), tn = ceil_div(d, (int64_t)256), tiles = tn * tm - tn * (tn - 1) / 2;
+  const int64_t pairs = sm_count() / 2;
+  int64_t best = 1, best_waves = -1;
+  for (int64_t g = 1; g <= max_group && g <= nk; ++g) {
+    const int64_t waves = nk / g * ceil_div(g * tiles, pairs) + ceil_div(nk % g * tiles, pairs);
+    if (best_waves < 0 || waves <= best_waves) { best = g; best_waves = waves; }
+  }
+  return best;
 }
 }  // namespace
 
@@ -1672,63 +1690,90 @@ sp_status sp_mha_value_refit(const sp_mha_module* m, const sp_mha_state* st, con
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const bool bf16 = p.bf16;
   const size_t esz = bf16 ? 2 : 4;
-  const int64_t TT = T * T, dp = split_kpad(d);
-  auto kept = [&](int64_t i) { return head_mask_host == nullptr || head_mask_host[i] != 0; };
+  const int64_t TT = T * T;
+  auto is_kept = [&](int64_t i) { return head_mask_host == nullptr || head_mask_host[i] != 0; };
+  int64_t nk = 0;
+  for (int64_t i = 0; i < H; ++i) nk += is_kept(i) ? 1 : 0;
+  const int64_t g_bs = (d + dh) * d;
   CU(cudaMemset2DAsync(Wv_out, (size_t)ldw * sizeof(float), 0, (size_t)d * sizeof(float), (size_t)d, s));
+  if (nk == 0) return SP_OK;
+  const int64_t group = bf16 ? value_refit_group(nk, p.hg, d, dh) : 1;
+  // kept heads i0 .. i0 + g - 1 (in ascending order)
+  auto heads_of = [&](int64_t i0, int64_t g) {
+    HeadList l;
+    for (int64_t i = 0, q = 0; i < H && l.n < g; ++i)
+      if (is_kept(i) && q++ >= i0) l.h[l.n++] = (uint16_t)i;
+    return l;
+  };
 
-  // ---- per head: G_i = sum_s R^T R and C_i = sum_s Aattn_i^T R with the regressors R = P_i X of every sequence
+  // ---- per kept head: G_i = sum_s R^T R and C_i = sum_s Aattn_i^T R with the regressors R = P_i X of every sequence
   // (token-major: row q of R is sum_k P_i[q, k] x_k)
   for (int64_t q0 = 0; q0 < n_seq; q0 += p.sc) {
     const int64_t nq = (n_seq - q0 < p.sc) ? n_seq - q0 : p.sc;
-    const int64_t t0 = q0 * T, Tc = nq * T, pairs = nq * H;
+    const int64_t t0 = q0 * T, Tc = nq * T;
     const double acc = q0 > 0 ? 1.0 : 0.0;
     const uint8_t* xptr = reinterpret_cast<const uint8_t*>(m->X.ptr) + (size_t)t0 * d * esz;
     const float* Aat = st->Aattn + (size_t)t0 * d;
     const float* P = st->P + (size_t)q0 * H * TT;
-    const int64_t pplane = p.sc * H * TT;
-    if (bf16) {
-      CU(split_planes(P, pairs * TT, p.Pb, pplane, s));
-      CU(split_bf16(Aat, d, nullptr, Tc, d, dp, p.Ab, s));
-    }
     const BMat none{nullptr, SP_F32, 0, 0, 0, 1, 0};
-    for (int64_t i = 0; i < H; ++i) {
-      if (!kept(i)) continue;
-      float* Gi = p.G + (size_t)i * d * d;
-      float* Ci = p.Cv + (size_t)i * dh * d;
-      // one launch for the nq sequences of the chunk (the batch index b0 is not used: one head at a time)
-      const BMat Xb{xptr, cdt, d, d, T * d, 1, 0};
+    for (int64_t i0 = 0; i0 < nk; i0 += group) {
+      const int64_t g = std::min<int64_t>(group, nk - i0);
+      float* Gi = p.G + (size_t)i0 * g_bs;
       if (bf16) {
-        const BMat Pi{reinterpret_cast<const __nv_bfloat16*>(p.Pb) + (size_t)i * TT, SP_BF16, T, TT, H * TT, 2, pplane};
-        const BMat Rb{p.R, SP_BF16, 2 * dp, 2 * dp, T * 2 * dp, 1, 0};
-        static const int pa[2] = {0, 1}, pb[2] = {0, 0};     // (P hi + P lo) X
-        SPCHK(bcontract(T, d, T, 1.0, Pi, true, Xb, false, 2, pa, pb, 0.0, none, Rb, dp, 1, (int)nq, status_dev, s));
-        // G_i (+)= R^T R with R = R_hi + R_lo: hi.hi, lo.hi, hi.lo; the token axis is K, both operands MN-major
-        TcOperand ra{p.R, 2 * dp, false}, rb{p.R, 2 * dp, false};
-        ra.kext = rb.kext = Tc;
-        ra.mnext = rb.mnext = 2 * dp;
-        TcSegments sg;
-        sg.nseg = 3;
-        sg.a_mn[1] = (int32_t)dp;
-        sg.b_mn[2] = (int32_t)dp;
-        SPCHK(gemm_tc(d, d, Tc, 1.f, ra, rb, (float)acc, Operand{Gi, SP_F32, d, 1}, OutOperand{Gi, SP_F32, d}, true,
-                      status_dev, s, &sg, (double)d * d * Tc));
-        // C_i (+)= Aattn_i^T R: the head's d_h columns of Aattn (hi | lo) against R (hi | lo): hi.hi, lo.hi, hi.lo
-        TcOperand aa{reinterpret_cast<const __nv_bfloat16*>(p.Ab) + i * dh, 2 * dp, false};
-        aa.kext = Tc;
-        aa.mnext = dp + dh;      // the lo part of the head's columns sits dp columns to the right
-        TcSegments sc2;
-        sc2.nseg = 3;
-        sc2.a_mn[1] = (int32_t)dp;
-        sc2.b_mn[2] = (int32_t)dp;
-        SPCHK(gemm_tc(dh, d, Tc, 1.f, aa, rb, (float)acc, Operand{Ci, SP_F32, d, 1}, OutOperand{Ci, SP_F32, d}, false,
-                      status_dev, s, &sc2, 2.0 * (double)dh * d * Tc));
+        // A head by itself leaves half of the SM pairs idle in its Gram product and most of them in the product with
+        // Aattn: the heads of a group go through each product together, and Aattn's columns ride as further rows of the
+        // Gram product.
+        const HeadList heads = heads_of(i0, g);
+        const int64_t pplane = nq * g * TT, ldr = 2 * p.dq, r_bs = Tc * ldr;
+        CU(mha_split_heads(P, nq, H, TT, heads, p.Pb, pplane, s));
+        CU(mha_split_head_cols(Aat, Tc, d, dh, heads, reinterpret_cast<__nv_bfloat16*>(p.R) + d, ldr, p.dq, s));
+        {
+          // R = (P hi + P lo) X for every (head, sequence)
+          TcOperand ta{p.Pb, T, true}, tb{xptr, d, false};
+          TcSegments sg;
+          sg.nseg = 2;
+          sg.a_p[1] = 1;
+          TcBatch bt;
+          bt.nb0 = (int32_t)g; bt.nb1 = (int32_t)nq;
+          bt.a_s0 = TT; bt.a_s1 = g * TT; bt.a_planes = 2; bt.a_plane = pplane;
+          bt.b_shared0 = true; bt.b_s1 = T * d;
+          bt.c_s0 = r_bs; bt.c_s1 = T * ldr;
+          OutOperand r_out{p.R, SP_BF16, ldr};
+          r_out.lo_off = p.dq;
+          SPCHK(gemm_tc(T, d, T, 1.f, ta, tb, 0.f, Operand{nullptr, SP_F32, 0, 1}, r_out, false, status_dev, s, &sg,
+                        2.0 * (double)T * d * T * g * nq, 0, &bt));
+        }
+        // [R | Aattn_i]^T R with both as hi + lo: hi.hi, lo.hi, hi.lo; the token axis is K, both operands MN-major.  A tensor-core
+        // sum runs over 2048 tokens at most: over 8192 in one go its rounding shows in W_V (the error against 64 bits grows).
+        constexpr int64_t kMaxTokens = 2048;
+        for (int64_t k0 = 0; k0 < Tc; k0 += kMaxTokens) {
+          const int64_t kn = std::min<int64_t>(kMaxTokens, Tc - k0);
+          const __nv_bfloat16* rk = reinterpret_cast<const __nv_bfloat16*>(p.R) + (size_t)k0 * ldr;
+          TcOperand ra{rk, ldr, false}, rb{rk, ldr, false};
+          ra.kext = rb.kext = kn;
+          ra.mnext = rb.mnext = ldr;
+          TcSegments sg;
+          sg.nseg = 3;
+          sg.a_mn[1] = (int32_t)p.dq;
+          sg.b_mn[2] = (int32_t)p.dq;
+          TcBatch bt;
+          bt.nb0 = (int32_t)g; bt.nb1 = 1;
+          bt.a_s0 = bt.b_s0 = r_bs;
+          bt.c_s0 = bt.cin_s0 = g_bs;
+          SPCHK(gemm_tc(d + dh, d, kn, 1.f, ra, rb, k0 > 0 ? 1.f : (float)acc, Operand{Gi, SP_F32, d, 1},
+                        OutOperand{Gi, SP_F32, d}, true, status_dev, s, &sg,
+                        ((double)d * d + 2.0 * (double)dh * d) * kn * g, 0, &bt));
+        }
       } else {
+        const int64_t i = heads_of(i0, 1).h[0];
+        // one launch for the nq sequences of the chunk (the batch index b0 is not used: one head at a time)
+        const BMat Xb{xptr, cdt, d, d, T * d, 1, 0};
         const BMat Pi{P + (size_t)i * TT, SP_F32, T, TT, H * TT, 1, 0};
         const BMat Rb{p.R, SP_F32, d, d, T * d, 1, 0};
         SPCHK(bcontract(T, d, T, 1.0, Pi, true, Xb, false, 1, kSegHH, kSegHH, 0.0, none, Rb, 0, 1, (int)nq, status_dev,
                         s));
-        MatRef r{p.R, SP_F32, d}, g{Gi, SP_F32, d}, c{Ci, SP_F32, d}, a{Aat + i * dh, SP_F32, d};
-        SPCHK(contract(d, d, Tc, 1.0, r, false, r, false, acc, g, g, true, true, false, status_dev, s));
+        MatRef r{p.R, SP_F32, d}, gm{Gi, SP_F32, d}, c{Gi + (size_t)d * d, SP_F32, d}, a{Aat + i * dh, SP_F32, d};
+        SPCHK(contract(d, d, Tc, 1.0, r, false, r, false, acc, gm, gm, true, true, false, status_dev, s));
         SPCHK(contract(dh, d, Tc, 1.0, a, false, r, false, acc, c, c, false, true, false, status_dev, s));
       }
     }
@@ -1736,27 +1781,15 @@ sp_status sp_mha_value_refit(const sp_mha_module* m, const sp_mha_state* st, con
   // ---- W_V,i = C_i (G_i + rho_i I)^-1, one regularised solve per kept head.
   if (p.batched) {
     // all kept heads' systems together: every step of the factorisation and of the sweep is one launch over them
-    const int64_t a_bs = (d + dh) * d, d_bs = (int64_t)dinv_elems(d);
-    int nk = 0;
-    for (int64_t i = 0; i < H; ++i) {
-      if (!kept(i)) continue;
-      float* Gs = p.Gs_all + (size_t)nk * a_bs;
-      CU(effective_ridge(p.G + (size_t)i * d * d, d, d, rho, rho_relative, p.rho_all + nk, s));
-      CU(load_spd<float>(p.G + (size_t)i * d * d, d, d, p.rho_all + nk, Gs, d, s));
-      CU(gather_cols<float>(p.Cv + (size_t)i * dh * d, d, nullptr, dh, d, Gs + (size_t)d * d, d, s));
-      ++nk;
-    }
-    if (nk > 0) {
+    CU(add_ridge_batched(p.G, g_bs, d, (int)nk, rho, rho_relative != 0, s));
+    {
       ProfScope prof(PK_SOLVE, (double)nk * ((double)d * d * d / 3.0 + 2.0 * (double)dh * d * d), 0.0, s);
-      SPCHK(potrf_potrs_tc_batched(p.Gs_all, d, dh, nk, a_bs, p.dinv_all, d_bs, p.P_all, p.Xs_all, status_dev, s));
+      SPCHK(potrf_potrs_tc_batched(p.G, d, dh, (int)nk, g_bs, p.dinv_all, (int64_t)dinv_elems(d), p.P_all, p.Xs_all,
+                                   status_dev, s));
     }
-    nk = 0;
-    for (int64_t i = 0; i < H; ++i) {
-      if (!kept(i)) continue;
-      const float* Xi = p.Gs_all + (size_t)nk * a_bs + (size_t)d * d;
-      CU(scatter_cols<float>(Xi, d, nullptr, dh, d, d, Wv_out + (size_t)i * dh * ldw, ldw, s));
-      ++nk;
-    }
+    for (int64_t i0 = 0; i0 < nk; i0 += kMaxHeadGroup)
+      CU(mha_place_heads(p.G + (size_t)i0 * g_bs + (size_t)d * d, g_bs, dh, d,
+                         heads_of(i0, std::min<int64_t>(kMaxHeadGroup, nk - i0)), Wv_out, ldw, s));
     return SP_OK;
   }
   // Otherwise one system at a time.  A solve is a chain of short kernels that leaves most SMs idle, and the heads'
@@ -1769,11 +1802,10 @@ sp_status sp_mha_value_refit(const sp_mha_module* m, const sp_mha_state* st, con
     CU(cudaStreamWaitEvent(side->stream, side->fork, 0));
   }
   int64_t turn = 0;
-  for (int64_t i = 0; i < H; ++i) {
-    if (!kept(i)) continue;
-    const float* Gi = p.G + (size_t)i * d * d;
-    const float* Ci = p.Cv + (size_t)i * dh * d;
-    float* Wi = Wv_out + (size_t)i * dh * ldw;
+  for (int64_t q = 0; q < nk; ++q) {
+    const float* Gi = p.G + (size_t)q * g_bs;
+    const float* Ci = Gi + (size_t)d * d;
+    float* Wi = Wv_out + (size_t)heads_of(q, 1).h[0] * dh * ldw;
     const bool on_side = side != nullptr && (turn++ & 1) != 0;
     cudaStream_t sq = on_side ? side->stream : s;
     SolveBufs& sb = on_side ? p.sb2 : p.sb;

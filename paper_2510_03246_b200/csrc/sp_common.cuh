@@ -211,6 +211,7 @@ struct TcBatch {
   int64_t a_s0 = 0, a_s1 = 0, b_s0 = 0, b_s1 = 0, c_s0 = 0, c_s1 = 0, cin_s0 = 0, cin_s1 = 0;
   int32_t a_planes = 1, b_planes = 1;
   int64_t a_plane = 0, b_plane = 0;
+  bool b_shared0 = false;       // B is the same for all nb0 products (b_s0 unused)
 };
 // K is the extent of ONE segment.  alg_flops >= 0 overrides the flop count recorded for profiling.  max_pairs > 0
 // limits the launch to that many CTA pairs (SM pairs), leaving the other SMs to kernels of another stream.
@@ -422,6 +423,23 @@ cudaError_t mha_step_sizes(const float* x, const float* y, int64_t ld, int64_t n
 cudaError_t mha_z_update(float* Zq, float* Zk, const float* Gq, const float* Gk, const float* Tq, const float* Tk,
                          const float* eta, int64_t tokens, int d, int T, int d_h, double alpha, void* Zqs, void* Zks,
                          int64_t plane, cudaStream_t stream);
+// Selected heads of a chunk, for the recovery of W_V: dst[plane][seq][slot][per_pair] = bf16 hi / lo parts of
+// P[seq][heads.h[slot]][per_pair] (per_pair a multiple of 4)
+constexpr int kMaxHeadGroup = 256;
+struct HeadList {
+  int32_t n = 0;
+  uint16_t h[kMaxHeadGroup];
+};
+cudaError_t mha_split_heads(const float* P, int64_t n_seq, int64_t H, int64_t per_pair, const HeadList& heads, void* dst,
+                            int64_t plane, cudaStream_t stream);
+// dst[(slot * tokens + t) * ld + c] = bf16 hi part of A[t, heads.h[slot] * d_h + c], lo part lo_off columns to the right
+cudaError_t mha_split_head_cols(const float* A, int64_t tokens, int64_t d, int64_t d_h, const HeadList& heads, void* dst,
+                                int64_t ld, int64_t lo_off, cudaStream_t stream);
+// per system b: G_b[i, i] += rel ? rho tr(G_b) / n : rho (G_b [n, n], dense rows, bs elements apart)
+cudaError_t add_ridge_batched(float* G, int64_t bs, int64_t n, int batch, double rho, bool rel, cudaStream_t stream);
+// W[(heads.h[slot] * d_h + r) * ldw + c] = src[slot * bs + r * d + c]
+cudaError_t mha_place_heads(const float* src, int64_t bs, int64_t d_h, int64_t d, const HeadList& heads, float* W,
+                            int64_t ldw, cudaStream_t stream);
 // A[n, n] (ld) = identity
 template <typename T>
 cudaError_t set_identity(T* A, int64_t n, int64_t ld, cudaStream_t stream);

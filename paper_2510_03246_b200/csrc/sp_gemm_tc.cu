@@ -52,7 +52,7 @@ constexpr size_t SMEM_BYTES = (size_t)STAGES * STAGE_BYTES + 4 * STG_BYTES + 102
 constexpr long long WAIT_BUDGET_CYCLES = 4000000000LL;   // ~2 s
 constexpr long long DRAIN_BUDGET_CYCLES = 200000000LL;   // ~0.1 s
 
-enum EpiMode : int { EPI_DIRECT = 0, EPI_TMA_STORE = 1, EPI_TMA_ADD = 2, EPI_TMA_BF16_CIN = 3 };
+enum EpiMode : int { EPI_DIRECT = 0, EPI_TMA_STORE = 1, EPI_TMA_ADD = 2, EPI_TMA_BF16_CIN = 3, EPI_TMA_BF16 = 4 };
 
 struct TcParams {
   int64_t M, N, K;
@@ -82,6 +82,7 @@ struct TcParams {
   int32_t batched, nb0, nb1, tiles_per_batch;
   int8_t a_ord[4], b_ord[4], c_ord[4];
   int64_t c_s0, c_s1, cin_s0, cin_s1;
+  int32_t b_shared0;       // one B for all b0
   long long wait_budget;   // clock cycles a role may wait on one barrier before it gives up (SP_ERR_TIMEOUT)
   int32_t* status;
   const int32_t* skip;     // conditional launch: every CTA returns at once when *skip != 0 (see SkipScope)
@@ -405,7 +406,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           const int am = tm * TILE_M + (int)rank * BM + p.seg.a_mn[sg];
           const int bn = tn * TN + (int)rank * BN_LOAD + p.seg.b_mn[sg];
           if constexpr (BATCHED) {
-            const int pa = p.seg.a_p[sg], pb = p.seg.b_p[sg];
+            const int pa = p.seg.a_p[sg], pb = p.seg.b_p[sg], bb0 = p.b_shared0 ? 0 : b0;
             if (p.a_kmajor) {
               tma_load_5d(a_dst, &tmA, make_coord(p.a_ord, ka, am, b0, b1, pa), fbar);
             } else {
@@ -414,11 +415,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 tma_load_5d(a_dst + mb * (64 * BK * 2), &tmA, make_coord(p.a_ord, am + mb * 64, ka, b0, b1, pa), fbar);
             }
             if (p.b_kmajor) {
-              tma_load_5d(b_dst, &tmB, make_coord(p.b_ord, kbb, bn, b0, b1, pb), fbar);
+              tma_load_5d(b_dst, &tmB, make_coord(p.b_ord, kbb, bn, bb0, b1, pb), fbar);
             } else {
 #pragma unroll
               for (int nb = 0; nb < BN_LOAD / 64; ++nb)
-                tma_load_5d(b_dst + nb * (64 * BK * 2), &tmB, make_coord(p.b_ord, bn + nb * 64, kbb, b0, b1, pb), fbar);
+                tma_load_5d(b_dst + nb * (64 * BK * 2), &tmB, make_coord(p.b_ord, bn + nb * 64, kbb, bb0, b1, pb), fbar);
             }
           } else {
             if (p.a_kmajor) {
@@ -578,6 +579,54 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           }
         }
         if (!ok) break;
+      } else if (p.epi_mode == EPI_TMA_BF16) {
+        // bf16 C without Cin, one or two (hi, lo) parts: 32 x 32 blocks in 64-byte swizzled rows (as above), tmCin describes
+        // the lo part.  Two-byte stores of a turned tile bounded short products (P X with P as hi + lo, 8 x 1024 x 2048,
+        // K = 2048, results as hi | lo: 113 us).
+#pragma unroll 1
+        for (int c0 = 0; c0 < TN; c0 += 32) {
+          const int64_t gj0 = (int64_t)tn * TN + c0;
+          if (gj0 >= p.N) break;                  // uniform over the warp
+          uint32_t r[32];
+          tc_ld32(taddr + (uint32_t)c0, r);
+          tc_wait_ld();
+          if (lane == 0) bulk_wait_read_1();      // the copies that last read this half (two blocks ago) are done
+          __syncwarp();
+          uint8_t* out_row = wstg_ptr + buf * 4096 + lane * 64;
+          const int sw = (lane >> 1) & 3;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            uint32_t hw[4], lw[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const float v0 = p.alpha * __uint_as_float(r[8 * j + 2 * e]), v1 = p.alpha * __uint_as_float(r[8 * j + 2 * e + 1]);
+              const __nv_bfloat162 h2 = __floats2bfloat162_rn(v0, v1);
+              const __nv_bfloat162 l2 = __floats2bfloat162_rn(v0 - __low2float(h2), v1 - __high2float(h2));
+              hw[e] = *reinterpret_cast<const uint32_t*>(&h2);
+              lw[e] = *reinterpret_cast<const uint32_t*>(&l2);
+            }
+            *reinterpret_cast<uint4*>(out_row + ((j ^ sw) << 4)) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
+            if (p.c_lo_off > 0)
+              *reinterpret_cast<uint4*>(out_row + 2048 + ((j ^ sw) << 4)) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
+          }
+          fence_async_smem();
+          __syncwarp();
+          if (lane == 0) {
+            if (rows_here > 0) {
+              const uint32_t src = wstg + buf * 4096;
+              if constexpr (BATCHED) {
+                const Coord5 cc = make_coord(p.c_ord, (int32_t)gj0, (int32_t)row0, b0, b1, 0);
+                tma_store_5d(&tmC, cc, src);
+                if (p.c_lo_off > 0) tma_store_5d(&tmCin, cc, src + 2048);
+              } else {
+                tma_store_2d(&tmC, (int32_t)gj0, (int32_t)row0, src);
+                if (p.c_lo_off > 0) tma_store_2d(&tmCin, (int32_t)gj0, (int32_t)row0, src + 2048);
+              }
+            }
+            bulk_commit();
+          }
+          buf ^= 1;
+        }
       } else if (p.epi_mode != EPI_DIRECT) {
         // 32 x 32 fp32 block -> 128-byte-swizzled shared tile (16-byte chunk j of row r sits at chunk j ^ (r & 7))
         // -> one TMA store / add-reduction, which clips at the edges of C.  Two tiles per warp alternate.
@@ -732,8 +781,7 @@ namespace {
 // dimensions last); ord[r] receives the slot (1..4) of role r = outer, b0, b1, plane.  Boxes are 1 deep in b0, b1, plane.
 bool make_map5(CUtensorMap* map, bool f32, const void* ptr, int64_t inner, int box_inner, int64_t outer, int64_t ld,
                int box_outer, int64_t nb0, int64_t s0, int64_t nb1, int64_t s1, int64_t planes, int64_t plane_stride,
-               bool swizzle_none_ok, int8_t ord[4]) {
-  (void)swizzle_none_ok;
+               bool swizzle64, int8_t ord[4]) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return false;
   const int64_t es = f32 ? 4 : 2;
@@ -764,7 +812,7 @@ bool make_map5(CUtensorMap* map, bool f32, const void* ptr, int64_t inner, int b
   }
   CUresult r = fn(map, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5,
                   const_cast<void*>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                  CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                  swizzle64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
 }
 }  // namespace
@@ -795,7 +843,7 @@ sp_status gemm_tc(int64_t M, int64_t N, int64_t K, float alpha, TcOperand A, TcO
                   OutOperand C, bool lower_only, int32_t* status_dev, cudaStream_t stream, const TcSegments* segs,
                   double alg_flops, int max_pairs, const TcBatch* batch) {
   const bool batched = batch != nullptr;
-  if (batched && (lower_only || batch->nb0 < 1 || batch->nb1 < 1 || batch->a_planes < 1 || batch->b_planes < 1))
+  if (batched && (batch->nb0 < 1 || batch->nb1 < 1 || batch->a_planes < 1 || batch->b_planes < 1))
     return SP_ERR_INVALID_ARG;
   TcSegments sg;
   if (segs) sg = *segs;
@@ -836,17 +884,19 @@ sp_status gemm_tc(int64_t M, int64_t N, int64_t K, float alpha, TcOperand A, TcO
   bool ok;
   if (batched) {
     const TcBatch& bt = *batch;
+    const int b_nb0 = bt.b_shared0 ? 1 : bt.nb0;
+    p.b_shared0 = bt.b_shared0 ? 1 : 0;
     for (int i = 0; i < sg.nseg; ++i)
       if (sg.a_p[i] < 0 || sg.a_p[i] >= bt.a_planes || sg.b_p[i] < 0 || sg.b_p[i] >= bt.b_planes)
         return SP_ERR_INVALID_ARG;
     ok = A.kmajor ? make_map5(&tmA, false, A.ptr, a_kext, BK, a_mext, A.ld, BM, bt.nb0, bt.a_s0, bt.nb1, bt.a_s1,
-                              bt.a_planes, bt.a_plane, true, p.a_ord)
+                              bt.a_planes, bt.a_plane, false, p.a_ord)
                   : make_map5(&tmA, false, A.ptr, a_mext, 64, a_kext, A.ld, BK, bt.nb0, bt.a_s0, bt.nb1, bt.a_s1,
-                              bt.a_planes, bt.a_plane, true, p.a_ord);
-    ok = ok && (B.kmajor ? make_map5(&tmB, false, B.ptr, b_kext, BK, b_next, B.ld, tile_n / 2, bt.nb0, bt.b_s0, bt.nb1,
-                                     bt.b_s1, bt.b_planes, bt.b_plane, true, p.b_ord)
-                         : make_map5(&tmB, false, B.ptr, b_next, 64, b_kext, B.ld, BK, bt.nb0, bt.b_s0, bt.nb1,
-                                     bt.b_s1, bt.b_planes, bt.b_plane, true, p.b_ord));
+                              bt.a_planes, bt.a_plane, false, p.a_ord);
+    ok = ok && (B.kmajor ? make_map5(&tmB, false, B.ptr, b_kext, BK, b_next, B.ld, tile_n / 2, b_nb0, bt.b_s0, bt.nb1,
+                                     bt.b_s1, bt.b_planes, bt.b_plane, false, p.b_ord)
+                         : make_map5(&tmB, false, B.ptr, b_next, 64, b_kext, B.ld, BK, b_nb0, bt.b_s0, bt.nb1,
+                                     bt.b_s1, bt.b_planes, bt.b_plane, false, p.b_ord));
     if (!ok) return SP_ERR_ALIGNMENT;
   } else {
     ok = A.kmajor ? make_map(&tmA, false, A.ptr, a_kext, a_mext, A.ld, BK, BM)
@@ -885,7 +935,7 @@ sp_status gemm_tc(int64_t M, int64_t N, int64_t K, float alpha, TcOperand A, TcO
   if (p.epi_mode != EPI_DIRECT) {
     if (batched) {
       if (!make_map5(&tmC, true, C.ptr, N, 32, M, C.ld, 32, batch->nb0, batch->c_s0, batch->nb1, batch->c_s1, 1, 0,
-                     true, p.c_ord))
+                     false, p.c_ord))
         return SP_ERR_CUDA;
     } else if (!make_map(&tmC, true, C.ptr, N, M, C.ld, 32, 32)) {
       return SP_ERR_CUDA;
@@ -900,6 +950,19 @@ sp_status gemm_tc(int64_t M, int64_t N, int64_t K, float alpha, TcOperand A, TcO
         !make_map(&tmCin, false, Cin.ptr, N, M, Cin.s0, 32, 32, true))
       return SP_ERR_CUDA;
     p.epi_mode = EPI_TMA_BF16_CIN;
+  }
+  // bf16 C without Cin (one part, or hi and lo parts through a map each)
+  if (p.epi_mode == EPI_DIRECT && C.dtype == SP_BF16 && beta == 0.f && C.ld % 8 == 0 && N % 8 == 0 && C.lo_off % 8 == 0 &&
+      (reinterpret_cast<uintptr_t>(C.ptr) & 15u) == 0 &&
+      (!batched || ((batch->nb0 == 1 || batch->c_s0 % 8 == 0) && (batch->nb1 == 1 || batch->c_s1 % 8 == 0)))) {
+    auto describe = [&](CUtensorMap* map, void* ptr) {
+      return batched ? make_map5(map, false, ptr, N, 32, M, C.ld, 32, batch->nb0, batch->c_s0, batch->nb1, batch->c_s1, 1, 0,
+                                 true, p.c_ord)
+                     : make_map(map, false, ptr, N, M, C.ld, 32, 32, true);
+    };
+    if (describe(&tmC, C.ptr) &&
+        (p.c_lo_off == 0 || describe(&tmCin, reinterpret_cast<__nv_bfloat16*>(C.ptr) + p.c_lo_off)))
+      p.epi_mode = EPI_TMA_BF16;
   }
   p.seg = sg;
   p.seg_kb = (int32_t)ceil_div(K, BK);

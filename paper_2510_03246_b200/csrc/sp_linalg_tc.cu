@@ -869,7 +869,7 @@ sp_status potrf_potrs_tc_batched(float* A, int64_t n, int64_t m, int batch, int6
     }
     float* A22 = A + (k0 + TB) * lda + (k0 + TB);
     sp_status st = gemm_tc(prow, rem, TB, -1.f, ta, tb, 1.f, Operand{A22, SP_F32, lda, 1}, OutOperand{A22, SP_F32, lda},
-                           false, status_dev, stream, &sg,
+                           true, status_dev, stream, &sg,
                            ((double)rem * rem + 2.0 * (double)m * rem) * TB * batch, 0, &bt);
     if (st != SP_OK) return st;
   }

@@ -260,6 +260,73 @@ __global__ void __launch_bounds__(256) split_planes_kernel(const float* __restri
   }
 }
 
+// bf16 hi / lo planes of the selected heads' [T, T] blocks: grid (pieces of a block, slots, sequences), 16-byte reads.
+__global__ void __launch_bounds__(256) split_heads_kernel(const float* __restrict__ P, int64_t n_seq, int64_t H, int64_t per_pair,
+                                                          const __grid_constant__ HeadList heads,
+                                                          __nv_bfloat16* __restrict__ dst, int64_t plane) {
+  struct __align__(8) B { __nv_bfloat162 v[2]; };
+  for (int64_t seq = blockIdx.z; seq < n_seq; seq += gridDim.z) {
+    const float* src = P + (seq * H + heads.h[blockIdx.y]) * per_pair;
+    __nv_bfloat16* out = dst + (seq * gridDim.y + blockIdx.y) * per_pair;
+    for (int64_t e = ((int64_t)blockIdx.x * 256 + threadIdx.x) * 4; e < per_pair; e += (int64_t)gridDim.x * 1024) {
+      const float4 x = *reinterpret_cast<const float4*>(src + e);
+      B hi, lo;
+      hi.v[0] = __floats2bfloat162_rn(x.x, x.y);
+      hi.v[1] = __floats2bfloat162_rn(x.z, x.w);
+      lo.v[0] = __floats2bfloat162_rn(x.x - __low2float(hi.v[0]), x.y - __high2float(hi.v[0]));
+      lo.v[1] = __floats2bfloat162_rn(x.z - __low2float(hi.v[1]), x.w - __high2float(hi.v[1]));
+      *reinterpret_cast<B*>(out + e) = hi;
+      *reinterpret_cast<B*>(out + plane + e) = lo;
+    }
+  }
+}
+
+// The selected heads' columns of a token-major tensor as hi / lo parts: grid (tokens, slots)
+__global__ void split_head_cols_kernel(const float* __restrict__ A, int64_t tokens, int64_t d, int d_h,
+                                       const __grid_constant__ HeadList heads, __nv_bfloat16* __restrict__ dst, int64_t ld,
+                                       int64_t lo_off) {
+  const int per_block = blockDim.x / d_h > 0 ? blockDim.x / d_h : 1;
+  const int64_t t0 = (int64_t)blockIdx.x * per_block;
+  for (int e = threadIdx.x; e < per_block * d_h; e += blockDim.x) {
+    const int64_t t = t0 + e / d_h;
+    const int c = e % d_h;
+    if (t >= tokens) continue;
+    const float v = A[t * d + (int64_t)heads.h[blockIdx.y] * d_h + c];
+    const __nv_bfloat16 hi = __float2bfloat16_rn(v);
+    __nv_bfloat16* out = dst + ((int64_t)blockIdx.y * tokens + t) * ld + c;
+    out[0] = hi;
+    out[lo_off] = __float2bfloat16_rn(v - __bfloat162float(hi));
+  }
+}
+
+__global__ void __launch_bounds__(1024) add_ridge_batched_kernel(float* __restrict__ G, int64_t bs, int64_t n, double rho,
+                                                                 int rel) {
+  __shared__ double sm[32];
+  G += (int64_t)blockIdx.x * bs;
+  double s = 0.0;
+  if (rel)
+    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) s += (double)G[i * n + i];
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += sm[w];
+    sm[0] = rel ? rho * t / (double)n : rho;
+  }
+  __syncthreads();
+  const double r = sm[0];
+  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) G[i * n + i] = (float)((double)G[i * n + i] + r);
+}
+
+__global__ void __launch_bounds__(256) place_heads_kernel(const float* __restrict__ src, int64_t bs, int64_t d,
+                                                          const __grid_constant__ HeadList heads, float* __restrict__ W,
+                                                          int64_t ldw) {
+  const float* in = src + (int64_t)blockIdx.y * bs + (int64_t)blockIdx.x * d;
+  float* out = W + ((int64_t)heads.h[blockIdx.y] * gridDim.x + blockIdx.x) * ldw;
+  for (int64_t c = threadIdx.x; c < d; c += 256) out[c] = in[c];
+}
+
 template <typename T>
 __global__ void set_identity_kernel(T* A, int64_t n, int64_t ld) {
   const int64_t total = n * n;
@@ -386,6 +453,49 @@ cudaError_t split_planes(const float* x, int64_t total, void* dst, int64_t plane
   ProfScope prof(PK_ELEMENTWISE, 0.0, (double)total * 8.0, stream);
   count_launch();
   split_planes_kernel<<<grid_1d(total, 256), 256, 0, stream>>>(x, total, reinterpret_cast<__nv_bfloat16*>(dst), plane);
+  return cudaGetLastError();
+}
+
+cudaError_t mha_split_heads(const float* P, int64_t n_seq, int64_t H, int64_t per_pair, const HeadList& heads, void* dst,
+                            int64_t plane, cudaStream_t stream) {
+  if (n_seq * heads.n * per_pair == 0) return cudaSuccess;
+  if (per_pair % 4 != 0) return cudaErrorInvalidValue;
+  ProfScope prof(PK_ELEMENTWISE, 0.0, (double)n_seq * heads.n * per_pair * 8.0, stream);
+  count_launch();
+  int64_t gx = ceil_div(per_pair, (int64_t)1024);
+  const int64_t cap = ceil_div((int64_t)sm_count() * 32, n_seq * heads.n);
+  if (gx > cap) gx = cap;
+  const unsigned gz = (unsigned)(n_seq < 65535 ? n_seq : 65535);
+  split_heads_kernel<<<dim3((unsigned)gx, (unsigned)heads.n, gz), 256, 0, stream>>>(
+      P, n_seq, H, per_pair, heads, reinterpret_cast<__nv_bfloat16*>(dst), plane);
+  return cudaGetLastError();
+}
+
+cudaError_t mha_split_head_cols(const float* A, int64_t tokens, int64_t d, int64_t d_h, const HeadList& heads, void* dst,
+                                int64_t ld, int64_t lo_off, cudaStream_t stream) {
+  if (tokens * heads.n == 0) return cudaSuccess;
+  ProfScope prof(PK_ELEMENTWISE, 0.0, (double)tokens * heads.n * d_h * 8.0, stream);
+  count_launch();
+  const int64_t per_block = 256 / d_h > 0 ? 256 / d_h : 1;
+  split_head_cols_kernel<<<dim3((unsigned)ceil_div(tokens, per_block), (unsigned)heads.n), 256, 0, stream>>>(
+      A, tokens, d, (int)d_h, heads, reinterpret_cast<__nv_bfloat16*>(dst), ld, lo_off);
+  return cudaGetLastError();
+}
+
+cudaError_t add_ridge_batched(float* G, int64_t bs, int64_t n, int batch, double rho, bool rel, cudaStream_t stream) {
+  if (n == 0 || batch == 0) return cudaSuccess;
+  ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
+  count_launch();
+  add_ridge_batched_kernel<<<(unsigned)batch, 1024, 0, stream>>>(G, bs, n, rho, rel ? 1 : 0);
+  return cudaGetLastError();
+}
+
+cudaError_t mha_place_heads(const float* src, int64_t bs, int64_t d_h, int64_t d, const HeadList& heads, float* W,
+                            int64_t ldw, cudaStream_t stream) {
+  if (heads.n == 0 || d_h == 0) return cudaSuccess;
+  ProfScope prof(PK_ELEMENTWISE, 0.0, (double)heads.n * d_h * d * 8.0, stream);
+  count_launch();
+  place_heads_kernel<<<dim3((unsigned)d_h, (unsigned)heads.n), 256, 0, stream>>>(src, bs, d, heads, W, ldw);
   return cudaGetLastError();
 }
 

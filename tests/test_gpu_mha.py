@@ -222,6 +222,27 @@ def test_mha_value_refit_matches_oracle(dtype, d, H, T, n_seq, chunk, causal):
     assert torch.all(out[:, d:] == -3.0)
 
 
+@pytest.mark.parametrize("d,H,T,n_seq,chunk,kept", [
+    (64, 4, 1032, 2, 2, (0, 1, 3)),      # 2064 tokens in a chunk: the Gram products in two ranges, 16 tokens in the second
+    (128, 16, 16, 5, 2, (1, 2, 7, 15)),  # batched systems, heads not in a row, a last chunk of one sequence
+    (256, 2, 40, 3, 0, (1,)),            # one head, one sequence per chunk
+])
+def test_mha_value_refit_of_some_heads(d, H, T, n_seq, chunk, kept):
+    """The kept heads' products in groups, packed from their places among all heads: against the oracle from the same P, Aattn, X."""
+    X, W = _case(torch.bfloat16, d, H, T, n_seq, seed_layer=5)
+    mod = api.MhaModule(X.to(DEV), *[w.to(DEV) for w in W], n_heads=H, T=T, seq_chunk=chunk)
+    mod.sp_mha_init(True)
+    head_mask = [1 if h in kept else 0 for h in range(H)]
+    Wv = np64(mod.sp_mha_value_refit(head_mask, 0.05, True))
+    mod.check_status()
+    Xo, Ao = np64(X), np64(mod.Aattn)
+    rows = [slice(q * T, (q + 1) * T) for q in range(n_seq)]
+    ref = O.mha_recover_value_weights([Xo[r].T for r in rows], [np64(mod.P[q]) for q in range(n_seq)], [Ao[r].T for r in rows],
+                                      head_mask, d // H, 0.05, True)
+    assert relerr(Wv, ref) < TOL[torch.bfloat16]
+    assert np.all(Wv[~np.repeat(np.asarray(head_mask, bool), d // H)] == 0)
+
+
 def test_mha_value_refit_argument_errors():
     X, W = _case(torch.bfloat16, 96, 4, 40, 2)
     mod = api.MhaModule(X.to(DEV), *[w.to(DEV) for w in W], n_heads=4, T=40)
