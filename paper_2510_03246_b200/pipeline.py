@@ -231,8 +231,9 @@ def mha_outer_iterations(mod: api.MhaModule, head_mask: torch.Tensor, iters: int
     api.sp_apply_mask(unit_scores, k_heads, group=d_head, W_rows=mod.Wv)
     precise = mod.X.dtype == torch.float32          # fp32 mode: fp64 factorisations
     for _ in range(iters):
-        Wq = api.sp_ridge_solve(mod.R_Q, mod.G_X, rho, rho_relative, precise)
-        Wk = api.sp_ridge_solve(mod.R_K, mod.G_X, rho, rho_relative, precise)
+        # W_Q and W_K have one system matrix: one factorisation with the rows of both below it
+        Wqk = api.sp_ridge_solve(torch.cat((mod.R_Q, mod.R_K)), mod.G_X, rho, rho_relative, precise)
+        Wq, Wk = Wqk[:mod.d], Wqk[mod.d:]
         api.sp_apply_mask(unit_scores, k_heads, group=d_head, W_rows=Wq)
         api.sp_apply_mask(unit_scores, k_heads, group=d_head, W_rows=Wk)
         Wo = api.sp_linear_refit(mod.R_O, mod.G_attn, head_mask, k_heads, rho, group=d_head, precise=precise,
