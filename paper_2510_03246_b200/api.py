@@ -7,6 +7,7 @@ missing or a CUDA device is absent the calls raise.
 from __future__ import annotations
 
 import ctypes as C
+import functools
 import os
 from dataclasses import dataclass
 
@@ -175,23 +176,33 @@ def _require_cuda(*tensors):
 
 
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+
+
+_DTYPES = {torch.float32: SP_F32, torch.bfloat16: SP_BF16, torch.float64: SP_F64}
 
 
 def _dt(t: torch.Tensor) -> int:
-    return {torch.float32: SP_F32, torch.bfloat16: SP_BF16, torch.float64: SP_F64}[t.dtype]
+    return _DTYPES[t.dtype]
 
 
 def mat(t: torch.Tensor | None) -> SpMat:
     """Row-major matrix view of a 2-D tensor whose last dimension is contiguous."""
     if t is None:
         return SpMat(None, 0, 0, 0, 0, 0)
-    assert t.dim() == 2 and (t.stride(1) == 1 or t.shape[1] <= 1), "need a row-major 2-D tensor"
-    return SpMat(t.data_ptr(), _dt(t), 0, t.shape[0], t.shape[1], t.stride(0) if t.shape[0] > 1 else max(t.shape[1], t.stride(0)))
+    assert t.dim() == 2, "need a row-major 2-D tensor"
+    (rows, cols), (ld, step) = t.shape, t.stride()
+    assert step == 1 or cols <= 1, "need a row-major 2-D tensor"
+    return SpMat(t.data_ptr(), _DTYPES[t.dtype], 0, rows, cols, ld if rows > 1 else max(cols, ld))
 
 
 def _ptr(t: torch.Tensor | None):
     return None if t is None else t.data_ptr()
+
+
+@functools.lru_cache(maxsize=256)
+def _scores_bytes(cols: int, rows: int, device: int) -> int:      # (a function of the sizes and the device alone)
+    return workspace_bytes(SP_WS_SCORES, cols, 0, rows, 0, SP_F32)
 
 
 def workspace_bytes(op: int, d: int, n: int, N: int, token_chunk: int = 0, dtype: int = SP_F32) -> int:
@@ -292,18 +303,21 @@ def sp_linear_refit(R, G, mask, k_keep, rho, group=1, precise=False, W=None, sta
 def sp_struct_scores(kind, n_units, group=1, W=None, colsq=None, colsq_stride=1, colabs=None, inv_tokens=0.0,
                      b=None, c=None, dd=None, t=None, r_layer=0.0, want_relaxed=False, ws=None):
     """Returns (scores fp32 [n_units], importance fp64 [1], relaxed fp64 [n_units] or None)."""
-    dev = (W if W is not None else b).device
+    src = W if W is not None else b
+    dev = src.device
     _require_cuda(W, colsq, colabs, b, c, dd, t)
-    inp = SpScoreInputs(mat(W), _ptr(colsq), colsq_stride, _ptr(colabs), float(inv_tokens), mat(b), mat(c), mat(dd),
-                        mat(t))
+    # (fields that are not given stay zero: no matrix)
+    inp = SpScoreInputs(colsq=_ptr(colsq), colsq_stride=colsq_stride, colabs=_ptr(colabs), inv_tokens=inv_tokens)
+    for field, m in (("W", W), ("b", b), ("c", c), ("dd", dd), ("t", t)):
+        if m is not None:
+            setattr(inp, field, mat(m))
     scores = torch.empty(n_units, dtype=torch.float32, device=dev)
     imp = torch.empty(1, dtype=torch.float64, device=dev)
     relaxed = torch.empty(n_units, dtype=torch.float64, device=dev) if want_relaxed else None
-    rows = W.shape[0] if W is not None else b.shape[0]
     if ws is None:
-        ws = _ws(workspace_bytes(SP_WS_SCORES, n_units * group, 0, rows, 0, SP_F32), dev)
+        ws = _ws(_scores_bytes(n_units * group, src.shape[0], dev.index), dev)
     _check(lib().sp_struct_scores(kind, group, C.byref(inp), n_units, scores.data_ptr(), imp.data_ptr(),
-                                  _ptr(relaxed), float(r_layer), ws.data_ptr(), ws.numel(), _stream()),
+                                  _ptr(relaxed), r_layer, ws.data_ptr(), ws.numel(), _stream()),
            "sp_struct_scores")
     return scores, imp, relaxed
 
