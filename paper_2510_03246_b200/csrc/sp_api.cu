@@ -172,6 +172,7 @@ sp_status ridge_core(const float* R, int64_t ldr, const float* G, int64_t ldg, i
 }
 
 __global__ void expand_group_index_kernel(const int32_t* unit_idx, int64_t k_units, int group, int32_t* col_idx) {
+  kernel_begin();
   const int64_t total = k_units * group;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x)
     col_idx[e] = unit_idx[e / group] * group + (int32_t)(e % group);
@@ -522,6 +523,7 @@ sp_status sp_ridge_solve(const float* R, int64_t ldr, const float* G, int64_t ld
   if (!ws || ws_bytes < ridge_ws_bytes(m, n, precise != 0)) return SP_ERR_WORKSPACE;
   if (misaligned(ws, 256)) return SP_ERR_ALIGNMENT;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+  const OverlapScope overlap(n <= kOverlapMaxN);
   Carver c(ws);
   SolveBufs b = carve_solve(c, n, m, precise ? 8 : 4);
   CU(effective_ridge(G, ldg, n, rho, rho_relative, b.rho, s));
@@ -549,6 +551,7 @@ sp_status sp_linear_refit(const float* R, int64_t ldr, const float* G, int64_t l
   if (!ws || ws_bytes < need) return SP_ERR_WORKSPACE;
   if (misaligned(ws, 256)) return SP_ERR_ALIGNMENT;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+  const OverlapScope overlap(n <= kOverlapMaxN);
   Carver c(ws);
   SolveBufs b = carve_solve(c, n, m, precise ? 8 : 4);
   int32_t* unit_idx = c.take<int32_t>((size_t)n_units);
@@ -557,7 +560,7 @@ sp_status sp_linear_refit(const float* R, int64_t ldr, const float* G, int64_t l
   const int64_t k = k_keep * group;
   if (k > 0) {
     count_launch();
-    expand_group_index_kernel<<<(unsigned)ceil_div(k, 256), 256, 0, s>>>(unit_idx, k_keep, group, b.idx);
+    launch(expand_group_index_kernel, (unsigned)ceil_div(k, 256), 256, 0, s, unit_idx, k_keep, group, b.idx);
     CU(cudaGetLastError());
   }
   if (precise) return ridge_core<double>(R, ldr, G, ldg, m, n, b.idx, k, b.rho, W, ldw, b, status_dev, s);
@@ -653,6 +656,7 @@ sp_status sp_apply_mask_global(const float* scores, int64_t ld_scores, int64_t n
 }
 
 __global__ void objective_accumulate_kernel(const sp_step_report* rep, double beta, double* loss, int accumulate) {
+  kernel_begin();
   const double v = rep->res_out + beta * rep->res_act + rep->res_in;
   loss[0] = accumulate ? loss[0] + v : v;
 }
@@ -661,7 +665,7 @@ sp_status sp_objective_accumulate(const sp_step_report* rep_dev, double beta, do
                                   void* stream) {
   if (!rep_dev || !loss_dev) return SP_ERR_INVALID_ARG;
   count_launch();
-  objective_accumulate_kernel<<<1, 1, 0, reinterpret_cast<cudaStream_t>(stream)>>>(rep_dev, beta, loss_dev, accumulate);
+  launch(objective_accumulate_kernel, 1, 1, 0, reinterpret_cast<cudaStream_t>(stream), rep_dev, beta, loss_dev, accumulate);
   CU(cudaGetLastError());
   return SP_OK;
 }
@@ -825,6 +829,7 @@ sp_status sp_ffn_cache_input_inverse(const sp_ffn_module* m, sp_ffn_state* st, d
   if (!ws || ws_bytes < sp_workspace_bytes(SP_WS_INPUT_INVERSE, d, 0, 0, 0, 0)) return SP_ERR_WORKSPACE;
   if (misaligned(ws, 256)) return SP_ERR_ALIGNMENT;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+  const OverlapScope overlap(d <= kOverlapMaxN);
   Carver c(ws);
   SolveBufs b = carve_solve(c, d, d, 8);
   CU(effective_ridge(st->G_X, d, d, rho, rho_relative, b.rho, s));
@@ -879,6 +884,7 @@ static sp_status admm_step_impl(const sp_ffn_module* m, sp_ffn_state* st, const 
   // runs on the side stream while the caller's stream carries the W2 chain.
   SideStream* side = side_stream();
   cudaStream_t sa = side ? side->stream : s;
+  const OverlapScope overlap(std::max(n, d) <= kOverlapMaxN);
   JoinOnExit join_guard{side, s};
   // Reuse of the factorisation for the recovery on the kept support (tensor-core path): the unrestricted system is
   // solved with the channels that the mask kept so far in front.  The leading block of that factor is the factor of
@@ -1312,6 +1318,8 @@ sp_status bcontract(int64_t M, int64_t N, int64_t K, double alpha, BMat A, bool 
   return SP_OK;
 }
 
+constexpr int64_t kOverlapMaxPairs = int64_t(1) << 24;     // T x T entries of a chunk up to which its kernels are short
+
 struct MhaPlan {
   int64_t d, H, T, dh, sc, cap;   // cap = tokens of a full chunk
   bool bf16;
@@ -1464,6 +1472,7 @@ static sp_status mha_impl(const sp_mha_module* m, sp_mha_state* st, const sp_mha
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const bool bf16 = p.bf16, causal = prm->causal != 0;
   const int64_t dp = split_kpad(d);
+  const OverlapScope overlap(p.sc * H * T * T <= kOverlapMaxPairs);
   const size_t esz = bf16 ? 2 : 4;
   const double inv_sqrt = 1.0 / sqrt((double)dh);
   const int64_t TT = T * T;
@@ -1744,6 +1753,7 @@ sp_status sp_mha_value_refit(const sp_mha_module* m, const sp_mha_state* st, con
   ValueRefitPlan p = plan_value_refit(ws, d, H, T, n_seq, seq_chunk, cdt);
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const bool bf16 = p.bf16;
+  const OverlapScope overlap(p.sc * H * T * T <= kOverlapMaxPairs);
   const size_t esz = bf16 ? 2 : 4;
   const int64_t TT = T * T;
   auto is_kept = [&](int64_t i) { return head_mask_host == nullptr || head_mask_host[i] != 0; };

@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include <mutex>
+#include <utility>
 #include <type_traits>
 
 #include "../../include/sp.h"
@@ -81,6 +82,54 @@ int sm_count();
 
 __host__ __device__ __forceinline__ int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 __host__ __device__ __forceinline__ size_t align_up(size_t a, size_t b) { return (a + b - 1) / b * b; }
+
+// Programmatic dependent launch.  Every kernel of the library starts with kernel_begin() (the GEMM after setting up its
+// barriers and tensor memory): the next kernel of the stream may be brought onto the SMs from here on, and nothing of the
+// kernels before is touched until they have completed.  Each kernel waits, so the completion of one implies that of all
+// before it, as without the attribute; only launch latency, block start and the set-up ahead of the wait overlap.  Both
+// instructions do nothing in a kernel that was launched plainly.
+// The attribute is given inside an OverlapScope only, which the entry points open for calls whose kernels are short: their
+// time is launches and gaps (attention step 768 wide, 284 kernels: 2.68 -> 2.42 ms; ADMM step 768 x 3072 2.40 -> 2.28).  Long
+// kernels lose: waiting blocks hold SMs that another stream's kernels could use (ADMM step of 2048 x 8192 on 262144 tokens: 49.3
+// -> 51.4 ms).
+__device__ __forceinline__ void dependents_may_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_predecessors() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void kernel_begin() {
+  dependents_may_launch();
+  wait_for_predecessors();
+}
+bool& overlap_flag();                   // of this host thread (sp_profile.cu)
+struct OverlapScope {
+  bool saved;
+  explicit OverlapScope(bool on) : saved(overlap_flag()) { overlap_flag() = on; }
+  ~OverlapScope() { overlap_flag() = saved; }
+  OverlapScope(const OverlapScope&) = delete;
+};
+constexpr int64_t kOverlapMaxN = 4608;        // widest system whose solve is launches and gaps for the most part
+inline bool may_overlap_launches(cudaStream_t stream) {
+  if (!overlap_flag()) return false;
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(stream, &capture) == cudaSuccess) return capture == cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return false;
+}
+template <typename... P, typename... A>
+inline cudaError_t launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A&&... args) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = &attr;
+  // a grid of more than two waves of threads hides its own launch, and its successor's waiting blocks would only hold SMs
+  // that other streams' kernels could use
+  const int64_t threads = (int64_t)grid.x * grid.y * grid.z * block.x * block.y * block.z;
+  cfg.numAttrs = threads <= (int64_t)sm_count() * 4096 && may_overlap_launches(stream) ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
 
 // Shape of the kernels that move whole matrices: blocks of 256 threads, gridDim.x strips of columns (a thread has four of a
 // strip's, blockDim.x apart, so that every access of a warp is one line), blockDim.y and gridDim.y walk the rows.  No

@@ -34,6 +34,7 @@ __device__ __forceinline__ T block_sum(T v, T* smem) {
 template <int W>
 __global__ void __launch_bounds__(kStripThreads) convert_kernel(const void* src, int32_t sdt, int64_t lds, void* dst, int32_t ddt, int64_t ldd,
                                int64_t rows, int64_t cols) {
+  kernel_begin();
   for_strip<W>(rows, cols, [&](int64_t i, int64_t j, int) {
     const int64_t si = i * lds + j, di = i * ldd + j;
     if (sdt == SP_F64) {
@@ -54,6 +55,7 @@ __global__ void __launch_bounds__(kStripThreads) convert_kernel(const void* src,
 template <typename TD>
 __global__ void transpose_convert_kernel(const float* src, int64_t lds, int64_t rows, int64_t cols, TD* dst,
                                          int64_t ldd) {
+  kernel_begin();
   __shared__ float tile[32][33];
   const int64_t c0 = (int64_t)blockIdx.x * 32, r0 = (int64_t)blockIdx.y * 32;
   for (int r = threadIdx.y; r < 32; r += blockDim.y) {
@@ -85,6 +87,7 @@ __global__ void __launch_bounds__(kStripThreads) split_bf16_kernel(const float* 
                                                                    const int32_t* __restrict__ row_idx, int64_t rows,
                                                                    int64_t cols, int64_t kpad,
                                                                    __nv_bfloat16* __restrict__ dst) {
+  kernel_begin();
   const bool vec = pairs_aligned(src, lds);
   for_strip<W>(rows, kpad / 2, [&](int64_t i, int64_t p, int) {
     const float2 v = load_pair(src + (row_idx ? (int64_t)row_idx[i] : i) * lds, 2 * p, cols, vec);
@@ -101,6 +104,7 @@ template <int W>
 __global__ void __launch_bounds__(kStripThreads) split3_bf16_kernel(const float* __restrict__ src, int64_t lds,
                                                                     int64_t rows, int64_t cols, int64_t kpad,
                                                                     __nv_bfloat16* __restrict__ dst) {
+  kernel_begin();
   const bool vec = pairs_aligned(src, lds);
   for_strip<W>(rows, kpad / 2, [&](int64_t i, int64_t p, int) {
     const float2 v = load_pair(src + i * lds, 2 * p, cols, vec);
@@ -115,6 +119,7 @@ __global__ void __launch_bounds__(kStripThreads) split3_bf16_kernel(const float*
 }
 
 __global__ void symmetrize_kernel(float* G, int64_t n, int64_t ld) {
+  kernel_begin();
   __shared__ float tile[32][33];
   // block (bx, by) with bx > by mirrors lower tile (row block bx, col block by) to (by, bx); diagonal blocks in place
   const int64_t bx = blockIdx.x, by = blockIdx.y;
@@ -139,6 +144,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) load_spd_kernel(const float* __restrict__ G, int64_t ldg, const int32_t* idx,
                                                        int64_t n, const double* rho, T* __restrict__ dst, int64_t ldd,
                                                        const int32_t* skip) {
+  kernel_begin();
   if (skip != nullptr && *skip != 0) return;   // conditional launch (see SkipScope)
   constexpr int TS = kSpdTile;
   __shared__ float tile[TS][TS + 1];
@@ -182,6 +188,7 @@ __global__ void __launch_bounds__(kStripThreads) gather_cols_kernel(const float*
                                                                     const int32_t* idx, int64_t rows, int64_t k,
                                                                     T* __restrict__ dst, int64_t ldd,
                                                                     const int32_t* skip) {
+  kernel_begin();
   if (skip != nullptr && *skip != 0) return;
   int64_t at[kStripPer];
   strip_index<W>(idx, k, at);
@@ -193,6 +200,7 @@ __global__ void __launch_bounds__(kStripThreads) gather_cols_kernel(const float*
 template <int W>
 __global__ void __launch_bounds__(kStripThreads) gather_rows_kernel(const float* __restrict__ src, int64_t lds, const int32_t* __restrict__ idx,
                                    int64_t rows, int64_t cols, float* __restrict__ dst, int64_t ldd) {
+  kernel_begin();
   for_strip<W>(rows, cols, [&](int64_t i, int64_t j, int) {
     dst[i * ldd + j] = src[(int64_t)idx[i] * lds + j];
   });
@@ -203,6 +211,7 @@ __global__ void __launch_bounds__(kStripThreads) scatter_cols_kernel(const T* __
                                                                      const int32_t* idx, int64_t rows, int64_t k,
                                                                      float* __restrict__ dst, int64_t ldd,
                                                                      const int32_t* skip) {
+  kernel_begin();
   if (skip != nullptr && *skip != 0) return;
   int64_t at[kStripPer];
   strip_index<W>(idx, k, at);
@@ -214,6 +223,7 @@ __global__ void __launch_bounds__(kStripThreads) scatter_cols_kernel(const T* __
 template <int W>
 __global__ void __launch_bounds__(kStripThreads) fill_zero_kernel(float* dst, int64_t ld, int64_t rows, int64_t cols,
                                                                   const int32_t* skip) {
+  kernel_begin();
   if (skip != nullptr && *skip != 0) return;
   for_strip<W>(rows, cols, [&](int64_t i, int64_t j, int) { dst[i * ld + j] = 0.f; });
 }
@@ -222,12 +232,14 @@ __global__ void __launch_bounds__(kStripThreads) fill_zero_kernel(float* dst, in
 template <int W>
 __global__ void __launch_bounds__(kStripThreads) copy_cols_padded_kernel(const float* __restrict__ src, int64_t lds, int64_t rows, int64_t k,
                                         int64_t kpad, float* __restrict__ dst) {
+  kernel_begin();
   for_strip<W>(rows, kpad, [&](int64_t i, int64_t a, int) {
     dst[i * kpad + a] = a < k ? src[i * lds + a] : 0.f;
   });
 }
 
 __global__ void effective_ridge_kernel(const float* G, int64_t ldg, int64_t n, double rho, int rel, double* out) {
+  kernel_begin();
   __shared__ double sm[32];
   double s = 0.0;
   if (rel)
@@ -244,6 +256,7 @@ __global__ void effective_ridge_kernel(const float* G, int64_t ldg, int64_t n, d
 // grp_base[g], grp_base[g] + 1, ... in channel order.
 __global__ void __launch_bounds__(1024) group_map_kernel(const uint8_t* __restrict__ mask, int64_t n,
                                                          int32_t* grp_base, uint8_t* grp_mask) {
+  kernel_begin();
   __shared__ int warp_tot[32];
   __shared__ int s_before;
   const int64_t groups = ceil_div(n, (int64_t)8);
@@ -302,6 +315,7 @@ __global__ void __launch_bounds__(256) prep_h_kernel(const float* __restrict__ Z
                                                      int64_t ldh, int64_t ncols, int64_t lo_off, int64_t k,
                                                      const int32_t* __restrict__ idx, int32_t rows_per_block,
                                                      const int32_t* skip) {
+  kernel_begin();
   if (skip != nullptr && *skip != 0) return;   // conditional launch (see SkipScope)
   const int64_t p0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 8;
   if (p0 >= ncols) return;
@@ -404,6 +418,7 @@ struct UpdRow {
 
 template <bool HAS_U, int Z_RULE>
 __global__ void __launch_bounds__(256, 2) fused_update_kernel(UpdateArgs g) {
+  kernel_begin();
   __shared__ double sm[32];
   const int64_t grp4 = (int64_t)blockIdx.x * 256 + threadIdx.x;
   const int64_t c0 = grp4 * 4;
@@ -655,6 +670,7 @@ struct NextRow {
 
 template <int Z_RULE>
 __global__ void __launch_bounds__(256, 2) fused_update_next_kernel(UpdateArgs g) {
+  kernel_begin();
   __shared__ double sm[32];
   extern __shared__ __align__(16) __nv_bfloat16 next_tiles[];  // a_tile[512][kAtPitch], then z_tile[512][kAtPitch]
   __shared__ int32_t at_row[512];                              // per warp: row of each of its channels in "kept first" order
@@ -819,6 +835,7 @@ __global__ void __launch_bounds__(256, 3) gather_ht_kernel(const float* __restri
                                                            const uint8_t* __restrict__ grp_mask,
                                                            __nv_bfloat16* __restrict__ Ht, int64_t ldt,
                                                            int32_t row_blocks, const int32_t* __restrict__ skip) {
+  kernel_begin();
   if (skip != nullptr && *skip != 0) return;
   extern __shared__ __align__(16) __nv_bfloat16 zt_tile[];     // [1024][kAtPitch]
   __shared__ int32_t row_of[8][128];                           // per warp: row of each of its channels in Ht, -1: pruned
@@ -899,6 +916,7 @@ __global__ void __launch_bounds__(256, 3) gather_ht_kernel(const float* __restri
 __global__ void __launch_bounds__(256) init_act_kernel(const float* __restrict__ Z, float* gate_io, void* A_out,
                                                        void* Zb_out, int32_t out_dtype, int64_t T, int64_t n,
                                                        double* absA_part, int32_t row_blocks) {
+  kernel_begin();
   const int64_t c0 = ((int64_t)blockIdx.x * 256 + threadIdx.x) * 4;
   if (c0 >= n) return;
   const int64_t rows_per = ceil_div(T, (int64_t)row_blocks);
@@ -980,6 +998,7 @@ __global__ void __launch_bounds__(256) init_act_kernel(const float* __restrict__
 // each), then the 8 partial sums of a column are added in a fixed order.
 __global__ void __launch_bounds__(256) reduce_col_partials_kernel(const double* __restrict__ part, int32_t row_blocks,
                                                                   int64_t n, double* out, int acc) {
+  kernel_begin();
   __shared__ double sm[8][33];
   const int cx = threadIdx.x & 31, ry = threadIdx.x >> 5;
   const int64_t j = (int64_t)blockIdx.x * 32 + cx;
@@ -1004,6 +1023,7 @@ __global__ void __launch_bounds__(256) reduce_col_partials_kernel(const double* 
 }
 
 __global__ void reduce_report_kernel(const double* partial, int nblocks, sp_step_report* rep, int acc, double alpha) {
+  kernel_begin();
   __shared__ double sm[32];
   double s[4] = {0.0, 0.0, 0.0, 0.0};
   for (int i = threadIdx.x; i < nblocks; i += blockDim.x)
@@ -1020,6 +1040,7 @@ __global__ void reduce_report_kernel(const double* partial, int nblocks, sp_step
 // out[0] (+)= scale * sum x^2 over a [rows, cols] fp32 matrix: block partials, then one block adds them in order
 __global__ void __launch_bounds__(256) sumsq_partial_kernel(const float* __restrict__ x, int64_t ld, int64_t rows,
                                                             int64_t cols, double* part) {
+  kernel_begin();
   __shared__ double sm[32];
   double s = 0.0;
   const int64_t total = rows * cols;
@@ -1031,6 +1052,7 @@ __global__ void __launch_bounds__(256) sumsq_partial_kernel(const float* __restr
   if (threadIdx.x == 0) part[blockIdx.x] = r;
 }
 __global__ void sumsq_finish_kernel(const double* part, int nblocks, double scale, double* out, int acc) {
+  kernel_begin();
   __shared__ double sm[32];
   double s = 0.0;
   for (int i = threadIdx.x; i < nblocks; i += blockDim.x) s += part[i];
@@ -1040,6 +1062,7 @@ __global__ void sumsq_finish_kernel(const double* part, int nblocks, double scal
 
 __global__ void init_report_kernel(sp_step_report* rep, const double* rho1, const double* rho2, double kept,
                                    const int32_t* reused, const int32_t* scaled) {
+  kernel_begin();
   rep->res_act = 0.0;
   rep->res_out = nan("");
   rep->res_in = 0.0;
@@ -1055,6 +1078,7 @@ __global__ void init_report_kernel(sp_step_report* rep, const double* rho1, cons
 // per-column sum |x| and sum x^2 of a [T, C] chunk: grid (col blocks of 256, row blocks) -> scratch, then reduced
 __global__ void column_stats_kernel(const void* X, int32_t dt, int64_t ld, int64_t T, int64_t C, double* scratch,
                                     int32_t row_blocks) {
+  kernel_begin();
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= C) return;
   const int64_t rows_per = ceil_div(T, (int64_t)row_blocks);
@@ -1071,6 +1095,7 @@ __global__ void column_stats_kernel(const void* X, int32_t dt, int64_t ld, int64
 }
 
 __global__ void column_stats_reduce_kernel(const double* scratch, int32_t row_blocks, int64_t C, double* rowstats) {
+  kernel_begin();
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= C) return;
   double s1 = rowstats[c * 2 + 0], s2 = rowstats[c * 2 + 1];
@@ -1098,7 +1123,7 @@ cudaError_t convert_matrix(const void* src, int32_t sdt, int64_t lds, void* dst,
   ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
   count_launch();
   strip_launch(rows, cols, [&](auto w, dim3 grid, dim3 block) {
-    convert_kernel<decltype(w)::value><<<grid, block, 0, stream>>>(src, sdt, lds, dst, ddt, ldd, rows, cols);
+    launch(convert_kernel<decltype(w)::value>, grid, block, 0, stream, src, sdt, lds, dst, ddt, ldd, rows, cols);
   });
   return cudaGetLastError();
 }
@@ -1110,7 +1135,7 @@ cudaError_t transpose_convert(const float* src, int64_t lds, int64_t rows, int64
   dim3 grid((unsigned)ceil_div(cols, 32), (unsigned)ceil_div(rows, 32));
   ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
   count_launch();
-  transpose_convert_kernel<TD><<<grid, dim3(32, 8), 0, stream>>>(src, lds, rows, cols, dst, ldd);
+  launch(transpose_convert_kernel<TD>, grid, dim3(32, 8), 0, stream, src, lds, rows, cols, dst, ldd);
   return cudaGetLastError();
 }
 template cudaError_t transpose_convert<float>(const float*, int64_t, int64_t, int64_t, float*, int64_t, cudaStream_t);
@@ -1125,7 +1150,7 @@ cudaError_t split3_bf16(const float* src, int64_t lds, int64_t rows, int64_t col
   ProfScope prof(PK_ELEMENTWISE, 0.0, (double)rows * cols * 10.0, stream);
   count_launch();
   strip_launch(rows, kpad / 2, [&](auto w, dim3 grid, dim3 block) {
-    split3_bf16_kernel<decltype(w)::value><<<grid, block, 0, stream>>>(
+    launch(split3_bf16_kernel<decltype(w)::value>, grid, block, 0, stream, 
         src, lds, rows, cols, kpad, reinterpret_cast<__nv_bfloat16*>(dst));
   });
   return cudaGetLastError();
@@ -1137,7 +1162,7 @@ cudaError_t split_bf16(const float* src, int64_t lds, const int32_t* row_idx, in
   ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
   count_launch();
   strip_launch(rows, kpad / 2, [&](auto w, dim3 grid, dim3 block) {
-    split_bf16_kernel<decltype(w)::value><<<grid, block, 0, stream>>>(
+    launch(split_bf16_kernel<decltype(w)::value>, grid, block, 0, stream, 
         src, lds, row_idx, rows, cols, kpad, reinterpret_cast<__nv_bfloat16*>(dst));
   });
   return cudaGetLastError();
@@ -1148,7 +1173,7 @@ cudaError_t symmetrize_lower(float* G, int64_t n, int64_t ld, cudaStream_t strea
   const unsigned nb = (unsigned)ceil_div(n, 32);
   ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
   count_launch();
-  symmetrize_kernel<<<dim3(nb, nb), dim3(32, 8), 0, stream>>>(G, n, ld);
+  launch(symmetrize_kernel, dim3(nb, nb), dim3(32, 8), 0, stream, G, n, ld);
   return cudaGetLastError();
 }
 
@@ -1158,7 +1183,7 @@ cudaError_t load_spd(const float* G, int64_t ldg, int64_t n, const double* rho_d
   if (n == 0) return cudaSuccess;
   ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
   count_launch();
-  load_spd_kernel<T><<<lower_tiles(n, kSpdTile), 256, 0, stream>>>(G, ldg, nullptr, n, rho_dev, dst, ldd, skip_flag());
+  launch(load_spd_kernel<T>, lower_tiles(n, kSpdTile), 256, 0, stream, G, ldg, nullptr, n, rho_dev, dst, ldd, skip_flag());
   return cudaGetLastError();
 }
 template <typename T>
@@ -1167,7 +1192,7 @@ cudaError_t load_spd_gather(const float* G, int64_t ldg, const int32_t* idx, int
   if (k == 0) return cudaSuccess;
   ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
   count_launch();
-  load_spd_kernel<T><<<lower_tiles(k, kSpdTile), 256, 0, stream>>>(G, ldg, idx, k, rho_dev, dst, ldd, skip_flag());
+  launch(load_spd_kernel<T>, lower_tiles(k, kSpdTile), 256, 0, stream, G, ldg, idx, k, rho_dev, dst, ldd, skip_flag());
   return cudaGetLastError();
 }
 template <typename T>
@@ -1177,7 +1202,7 @@ cudaError_t gather_cols(const float* src, int64_t lds, const int32_t* idx, int64
   ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
   count_launch();
   strip_launch(rows, k, [&](auto w, dim3 grid, dim3 block) {
-    gather_cols_kernel<decltype(w)::value, T><<<grid, block, 0, stream>>>(
+    launch(gather_cols_kernel<decltype(w)::value, T>, grid, block, 0, stream, 
         src, lds, idx, rows, k, dst, ldd, skip_flag());
   });
   return cudaGetLastError();
@@ -1188,7 +1213,7 @@ cudaError_t copy_cols_padded(const float* src, int64_t lds, int64_t rows, int64_
   ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
   count_launch();
   strip_launch(rows, kpad, [&](auto w, dim3 grid, dim3 block) {
-    copy_cols_padded_kernel<decltype(w)::value><<<grid, block, 0, stream>>>(src, lds, rows, k, kpad, dst);
+    launch(copy_cols_padded_kernel<decltype(w)::value>, grid, block, 0, stream, src, lds, rows, k, kpad, dst);
   });
   return cudaGetLastError();
 }
@@ -1198,7 +1223,7 @@ cudaError_t gather_rows(const float* src, int64_t lds, const int32_t* idx, int64
   ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
   count_launch();
   strip_launch(rows, cols, [&](auto w, dim3 grid, dim3 block) {
-    gather_rows_kernel<decltype(w)::value><<<grid, block, 0, stream>>>(src, lds, idx, rows, cols, dst, ldd);
+    launch(gather_rows_kernel<decltype(w)::value>, grid, block, 0, stream, src, lds, idx, rows, cols, dst, ldd);
   });
   return cudaGetLastError();
 }
@@ -1211,13 +1236,13 @@ cudaError_t scatter_cols(const T* src, int64_t lds, const int32_t* idx, int64_t 
     ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
     count_launch();
     strip_launch(rows, n, [&](auto w, dim3 grid, dim3 block) {
-      fill_zero_kernel<decltype(w)::value><<<grid, block, 0, stream>>>(dst, ldd, rows, n, skip_flag());
+      launch(fill_zero_kernel<decltype(w)::value>, grid, block, 0, stream, dst, ldd, rows, n, skip_flag());
     });
   }
   if (rows * k == 0) return cudaGetLastError();
   count_launch();
   strip_launch(rows, k, [&](auto w, dim3 grid, dim3 block) {
-    scatter_cols_kernel<decltype(w)::value, T><<<grid, block, 0, stream>>>(
+    launch(scatter_cols_kernel<decltype(w)::value, T>, grid, block, 0, stream, 
         src, lds, idx, rows, k, dst, ldd, skip_flag());
   });
   return cudaGetLastError();
@@ -1238,7 +1263,7 @@ cudaError_t effective_ridge(const float* G, int64_t ldg, int64_t n, double rho, 
                             cudaStream_t stream) {
   ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
   count_launch();
-  effective_ridge_kernel<<<1, 1024, 0, stream>>>(G, ldg, n, rho, rel, rho_out);
+  launch(effective_ridge_kernel, 1, 1024, 0, stream, G, ldg, n, rho, rel, rho_out);
   return cudaGetLastError();
 }
 
@@ -1246,7 +1271,7 @@ cudaError_t build_group_map(const uint8_t* mask, int64_t n, int32_t* grp_base, u
   if (n == 0) return cudaSuccess;
   ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
   count_launch();
-  group_map_kernel<<<1, 1024, 0, stream>>>(mask, n, grp_base, grp_mask);
+  launch(group_map_kernel, 1, 1024, 0, stream, mask, n, grp_base, grp_mask);
   return cudaGetLastError();
 }
 
@@ -1268,7 +1293,7 @@ cudaError_t launch_prep_h(const float* Z, const float* U, const float* gate, voi
   if (rb > 65535) rb = 65535;
   const int32_t rows_per = (int32_t)ceil_div(T, rb);
   count_launch();
-  prep_h_kernel<<<dim3(gx, (unsigned)ceil_div(T, (int64_t)rows_per)), 256, 0, stream>>>(Z, U, gate, H, hdt, T, n, ldh, ncols, lo_off,
+  launch(prep_h_kernel, dim3(gx, (unsigned)ceil_div(T, (int64_t)rows_per)), 256, 0, stream, Z, U, gate, H, hdt, T, n, ldh, ncols, lo_off,
                                                                                         k, idx, rows_per, skip_flag());
   return cudaGetLastError();
 }
@@ -1324,7 +1349,7 @@ static cudaError_t launch_fused_update_next(const UpdateArgs& a, cudaStream_t st
   cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void*>(fn), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)kNextTileBytes);
   if (e != cudaSuccess) return e;
-  fn<<<grid, 256, kNextTileBytes, stream>>>(a);
+  launch(fn, grid, 256, kNextTileBytes, stream, a);
   return cudaGetLastError();
 }
 
@@ -1350,7 +1375,7 @@ cudaError_t launch_fused_update(const UpdateArgs& a, cudaStream_t stream) {
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  fn<<<grid, 256, smem, stream>>>(a);
+  launch(fn, grid, 256, smem, stream, a);
   return cudaGetLastError();
 }
 
@@ -1368,7 +1393,7 @@ cudaError_t launch_gather_ht(const float* Z, int64_t T, int64_t n, int64_t k, co
   cudaError_t e = cudaFuncSetAttribute(gather_ht_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)kAtTileBytes);
   if (e != cudaSuccess) return e;
-  gather_ht_kernel<<<grid, 256, kAtTileBytes, stream>>>(Z, T, n, k, grp_base, grp_mask,
+  launch(gather_ht_kernel, grid, 256, kAtTileBytes, stream, Z, T, n, k, grp_base, grp_mask,
                                                        reinterpret_cast<__nv_bfloat16*>(Ht), ldt, row_blocks, skip);
   return cudaGetLastError();
 }
@@ -1379,7 +1404,7 @@ cudaError_t launch_init_act(const float* Z, float* gate_io, void* A_out, void* Z
   dim3 grid((unsigned)ceil_div(n, 1024), (unsigned)row_blocks);
   ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
   count_launch();
-  init_act_kernel<<<grid, 256, 0, stream>>>(Z, gate_io, A_out, Zb_out, out_dtype, T, n, absA_part, row_blocks);
+  launch(init_act_kernel, grid, 256, 0, stream, Z, gate_io, A_out, Zb_out, out_dtype, T, n, absA_part, row_blocks);
   return cudaGetLastError();
 }
 
@@ -1388,7 +1413,7 @@ cudaError_t reduce_col_partials(const double* part, int32_t row_blocks, int64_t 
   if (n == 0) return cudaSuccess;
   ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
   count_launch();
-  reduce_col_partials_kernel<<<(unsigned)ceil_div(n, (int64_t)32), 256, 0, stream>>>(part, row_blocks, n, out,
+  launch(reduce_col_partials_kernel, (unsigned)ceil_div(n, (int64_t)32), 256, 0, stream, part, row_blocks, n, out,
                                                                                     accumulate ? 1 : 0);
   return cudaGetLastError();
 }
@@ -1396,7 +1421,7 @@ cudaError_t reduce_col_partials(const double* part, int32_t row_blocks, int64_t 
 cudaError_t reduce_report(const double* partial, int nblocks, sp_step_report* rep, bool accumulate, double alpha,
                           cudaStream_t stream) {
   count_launch();
-  reduce_report_kernel<<<1, 256, 0, stream>>>(partial, nblocks, rep, accumulate ? 1 : 0, alpha);
+  launch(reduce_report_kernel, 1, 256, 0, stream, partial, nblocks, rep, accumulate ? 1 : 0, alpha);
   return cudaGetLastError();
 }
 
@@ -1406,8 +1431,8 @@ cudaError_t sumsq_accumulate(const float* x, int64_t ld, int64_t rows, int64_t c
   ProfScope prof(PK_ELEMENTWISE, 0.0, (double)rows * cols * 4.0, stream);
   const int nb = kSumsqBlocks;
   count_launch(2);
-  sumsq_partial_kernel<<<nb, 256, 0, stream>>>(x, ld, rows, cols, scratch);
-  sumsq_finish_kernel<<<1, 256, 0, stream>>>(scratch, nb, scale, out, accumulate ? 1 : 0);
+  launch(sumsq_partial_kernel, nb, 256, 0, stream, x, ld, rows, cols, scratch);
+  launch(sumsq_finish_kernel, 1, 256, 0, stream, scratch, nb, scale, out, accumulate ? 1 : 0);
   return cudaGetLastError();
 }
 
@@ -1415,7 +1440,7 @@ cudaError_t init_report(sp_step_report* rep, const double* rho1, const double* r
                         const int32_t* reused, const int32_t* scaled, cudaStream_t stream) {
   ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
   count_launch();
-  init_report_kernel<<<1, 1, 0, stream>>>(rep, rho1, rho2, kept, reused, scaled);
+  launch(init_report_kernel, 1, 1, 0, stream, rep, rho1, rho2, kept, reused, scaled);
   return cudaGetLastError();
 }
 
@@ -1426,9 +1451,9 @@ cudaError_t column_stats(const void* X, int32_t dt, int64_t ld, int64_t T, int64
   dim3 grid((unsigned)ceil_div(C, 256), (unsigned)rb);
   ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
   count_launch();
-  column_stats_kernel<<<grid, 256, 0, stream>>>(X, dt, ld, T, C, scratch, rb);
+  launch(column_stats_kernel, grid, 256, 0, stream, X, dt, ld, T, C, scratch, rb);
   count_launch();
-  column_stats_reduce_kernel<<<(unsigned)ceil_div(C, 256), 256, 0, stream>>>(scratch, rb, C, rowstats);
+  launch(column_stats_reduce_kernel, (unsigned)ceil_div(C, 256), 256, 0, stream, scratch, rb, C, rowstats);
   return cudaGetLastError();
 }
 

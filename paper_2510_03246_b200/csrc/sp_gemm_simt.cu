@@ -32,6 +32,7 @@ template <typename Acc, int BM, int BN, int TM, int TN>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN))
 gemm_simt_kernel(int64_t M, int64_t N, int64_t K, Acc alpha, Operand A, Operand B, Acc beta, Operand Cin,
                  OutOperand C, int lower_only) {
+  kernel_begin();
   constexpr int NT = (BM / TM) * (BN / TN);
   constexpr int EA = BM * BK / NT;
   constexpr int EB = BN * BK / NT;
@@ -190,6 +191,7 @@ template <typename T, bool A_KFAST, bool B_KFAST, int BM>
 __global__ void __launch_bounds__(DM_THREADS, 3)
 gemm_dmma_kernel(int64_t M, int64_t N, int64_t K, double alpha, const T* A, int64_t lda,
                  const T* B, int64_t ldb, double beta, Operand Cin, OutOperand C, int lower_only, int k_tri) {
+  kernel_begin();
   using SlabA = DmmaSlab<T, A_KFAST, BM>;
   using SlabB = DmmaSlab<T, B_KFAST, DM_BN>;
   static_assert(alignof(SlabA) % 16 == 0 && alignof(SlabB) % 16 == 0, "16-byte pieces");
@@ -306,10 +308,10 @@ void launch_dmma(int64_t M, int64_t N, int64_t K, double alpha, const Operand& A
   const T* a = reinterpret_cast<const T*>(A.ptr);
   const T* b = reinterpret_cast<const T*>(B.ptr);
   const int lo = lower_only ? 1 : 0, tri = k_tri ? 1 : 0;
-  if (ak && bk) gemm_dmma_kernel<T, true, true, BM><<<grid, DM_THREADS, 0, stream>>>(M, N, K, alpha, a, lda, b, ldb, beta, Cin, C, lo, tri);
-  else if (ak) gemm_dmma_kernel<T, true, false, BM><<<grid, DM_THREADS, 0, stream>>>(M, N, K, alpha, a, lda, b, ldb, beta, Cin, C, lo, tri);
-  else if (bk) gemm_dmma_kernel<T, false, true, BM><<<grid, DM_THREADS, 0, stream>>>(M, N, K, alpha, a, lda, b, ldb, beta, Cin, C, lo, tri);
-  else gemm_dmma_kernel<T, false, false, BM><<<grid, DM_THREADS, 0, stream>>>(M, N, K, alpha, a, lda, b, ldb, beta, Cin, C, lo, tri);
+  if (ak && bk) launch(gemm_dmma_kernel<T, true, true, BM>, grid, DM_THREADS, 0, stream, M, N, K, alpha, a, lda, b, ldb, beta, Cin, C, lo, tri);
+  else if (ak) launch(gemm_dmma_kernel<T, true, false, BM>, grid, DM_THREADS, 0, stream, M, N, K, alpha, a, lda, b, ldb, beta, Cin, C, lo, tri);
+  else if (bk) launch(gemm_dmma_kernel<T, false, true, BM>, grid, DM_THREADS, 0, stream, M, N, K, alpha, a, lda, b, ldb, beta, Cin, C, lo, tri);
+  else launch(gemm_dmma_kernel<T, false, false, BM>, grid, DM_THREADS, 0, stream, M, N, K, alpha, a, lda, b, ldb, beta, Cin, C, lo, tri);
 }
 
 }  // namespace
@@ -334,12 +336,12 @@ cudaError_t gemm_simt(int64_t M, int64_t N, int64_t K, double alpha, Operand A, 
   } else if (acc64) {
     constexpr int BM = 64, BN = 64;
     dim3 grid((unsigned)ceil_div(N, BN), (unsigned)ceil_div(M, BM));
-    gemm_simt_kernel<double, BM, BN, 4, 4><<<grid, 256, 0, stream>>>(M, N, K, alpha, A, B, beta, Cin, C,
+    launch(gemm_simt_kernel<double, BM, BN, 4, 4>, grid, 256, 0, stream, M, N, K, alpha, A, B, beta, Cin, C,
                                                                       lower_only ? 1 : 0);
   } else {
     constexpr int BM = 128, BN = 128;
     dim3 grid((unsigned)ceil_div(N, BN), (unsigned)ceil_div(M, BM));
-    gemm_simt_kernel<float, BM, BN, 8, 8><<<grid, 256, 0, stream>>>(M, N, K, (float)alpha, A, B, (float)beta, Cin, C,
+    launch(gemm_simt_kernel<float, BM, BN, 8, 8>, grid, 256, 0, stream, M, N, K, (float)alpha, A, B, (float)beta, Cin, C,
                                                                      lower_only ? 1 : 0);
   }
   return cudaGetLastError();

@@ -333,7 +333,11 @@ template <bool BATCHED, int TN>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmCin, const TcParams p) {
-  if (p.skip != nullptr && *p.skip != 0) return;   // the same answer in every CTA: nothing is allocated yet
+  dependents_may_launch();
+  if (p.skip != nullptr) {
+    wait_for_predecessors();
+    if (*p.skip != 0) return;      // the same answer in every CTA: nothing is allocated yet
+  }
   constexpr int BN_LOAD = TN / 2;                            // columns of B loaded per CTA
   constexpr uint32_t LOAD_BYTES = A_BYTES + BN_LOAD * BK * 2;
   extern __shared__ uint8_t smem_raw[];
@@ -380,6 +384,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   cluster_sync_all();      // the peer's barriers exist before anything is sent to them
   tc_fence_after();
   const uint32_t tmem_base = s_tmem_base;
+  wait_for_predecessors();
 
   const int num_kb = p.seg_kb * p.seg.nseg;
 
@@ -1050,7 +1055,9 @@ sp_status gemm_tc(int64_t M, int64_t N, int64_t K, float alpha, TcOperand A, TcO
   const int pairs = p.num_units < pairs_max ? p.num_units : pairs_max;
   const auto kernel = batched ? (narrow ? gemm_tc_kernel<true, kNarrowN> : gemm_tc_kernel<true, TILE_N>)
                               : (narrow ? gemm_tc_kernel<false, kNarrowN> : gemm_tc_kernel<false, TILE_N>);
-  kernel<<<2 * pairs, NUM_THREADS, SMEM_BYTES, stream>>>(tmA, tmB, tmC, tmCin, p);
+  // (programmatic launch only for one wave of tiles with the GPU to itself, see launch())
+  if (p.num_units <= pairs && max_pairs == 0) launch(kernel, 2 * pairs, NUM_THREADS, SMEM_BYTES, stream, tmA, tmB, tmC, tmCin, p);
+  else kernel<<<2 * pairs, NUM_THREADS, SMEM_BYTES, stream>>>(tmA, tmB, tmC, tmCin, p);
   return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ERR_CUDA;
 }
 

@@ -14,6 +14,7 @@ using Diag = DiagBlock<double, NB>;
 
 __global__ void __launch_bounds__(Diag::THREADS) chol_diag64_kernel(const double* A, int64_t lda, int nb, double* dinv,
                                                                     int64_t block_row0, int32_t* status) {
+  kernel_begin();
   Diag::run(A, lda, nb, dinv, nullptr, block_row0, status);
 }
 
@@ -39,7 +40,7 @@ cudaError_t potrf_lower_f64(double* A, int64_t n, int64_t lda, double* dinv, int
     double* Akk = A + k0 * lda + k0;
     double* dk = dinv + step * NB * NB;
     count_launch();
-    chol_diag64_kernel<<<1, Diag::THREADS, Diag::SMEM, stream>>>(Akk, lda, nb, dk, k0, status_dev);
+    launch(chol_diag64_kernel, 1, Diag::THREADS, Diag::SMEM, stream, Akk, lda, nb, dk, k0, status_dev);
     SP_CU(cudaGetLastError());
     const int64_t rem = n - k0 - nb;
     // row r of X (identity right-hand sides) is zero left of column r

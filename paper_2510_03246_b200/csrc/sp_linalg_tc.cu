@@ -26,6 +26,7 @@ using Diag = DiagBlock<float, TB>;
 __global__ void __launch_bounds__(Diag::THREADS) chol_diag128_kernel(const float* A, int64_t lda, int nb, float* dinv,
                                                                      int64_t row0, int32_t* status,
                                                                      const int32_t* skip, int64_t a_bs, int64_t d_bs) {
+  kernel_begin();
   if (skip != nullptr && *skip != 0) return;                  // conditional launch (see SkipScope)
   A += (int64_t)blockIdx.x * a_bs;                            // batched launch: one CTA per system
   dinv += (int64_t)blockIdx.x * d_bs;
@@ -165,6 +166,7 @@ __global__ void __launch_bounds__(RowTile<R>::THREADS) panel_apply_kernel(float*
                                                                  int64_t lds, int64_t s_seg, int write_f32,
                                                                  int32_t* status, PanelNear near,
                                                                  const int32_t* skip, PanelBatch pb) {
+  kernel_begin();
   if (skip != nullptr && *skip != 0) return;
   using Tile = RowTile<R>;
   constexpr int AP = Tile::AP;
@@ -280,8 +282,8 @@ cudaError_t launch_panel_rows(float* X, int64_t ldx, int64_t rows, int nb, const
   });
   if (e != cudaSuccess) return e;
   const bool with_near = TRANS && near.L != nullptr;
-  panel_apply_kernel<TRANS, R><<<dim3((unsigned)ceil_div(rows, R), (unsigned)batch), RowTile<R>::THREADS,
-                                 pa_smem<R>(with_near), stream>>>(X, ldx, rows, nb, dinv, S, lds, s_seg, write_f32 ? 1 : 0, status, near,
+  launch(panel_apply_kernel<TRANS, R>, dim3((unsigned)ceil_div(rows, R), (unsigned)batch), RowTile<R>::THREADS,
+                                 pa_smem<R>(with_near), stream, X, ldx, rows, nb, dinv, S, lds, s_seg, write_f32 ? 1 : 0, status, near,
                                            skip_flag(), pb);
   return cudaGetLastError();
 }
@@ -410,18 +412,21 @@ __global__ void __cluster_dims__(NM_CTAS, 1, 1) __launch_bounds__(NM_THREADS)
     chol_next_diag_kernel(const float* __restrict__ A21, const float* __restrict__ A22, int64_t lda, int nb2,
                           const float* __restrict__ dinv, float* LmT, float* S, int32_t* status,
                           const int32_t* skip) {
+  kernel_begin();
   if (skip != nullptr && *skip != 0) return;
   next_diag_body<0>(A21, A22, lda, nb2, dinv, LmT, S, status);
 }
 __global__ void __launch_bounds__(NM_THREADS)
     chol_next_diag_stage1_kernel(const float* __restrict__ A21, int64_t lda, int nb2, const float* __restrict__ dinv,
                                  float* LmT, int32_t* status, const int32_t* skip) {
+  kernel_begin();
   if (skip != nullptr && *skip != 0) return;
   next_diag_body<1>(A21, nullptr, lda, nb2, dinv, LmT, nullptr, status);
 }
 __global__ void __launch_bounds__(NM_THREADS)
     chol_next_diag_stage2_kernel(const float* __restrict__ A22, int64_t lda, int nb2, float* LmT, float* S,
                                  const int32_t* skip) {
+  kernel_begin();
   if (skip != nullptr && *skip != 0) return;
   next_diag_body<2>(nullptr, A22, lda, nb2, nullptr, LmT, S, nullptr);
 }
@@ -492,7 +497,7 @@ sp_status potrf_lower_tc(float* A, int64_t n, int64_t lda, float* dinv, void* Pv
       if (assist && inner_first && kb > 0) SP_CUDA_OK(cudaStreamWaitEvent(stream, assist->near_done, 0));
       count_launch();
       ProfScope prof(PK_CHOL_DIAG, (double)nb * nb * nb * (2.0 / 3.0), 0.0, stream);
-      chol_diag128_kernel<<<1, Diag::THREADS, Diag::SMEM, stream>>>(from_scratch ? S : A + k0 * lda + k0,
+      launch(chol_diag128_kernel, 1, Diag::THREADS, Diag::SMEM, stream, from_scratch ? S : A + k0 * lda + k0,
                                                                   from_scratch ? (int64_t)TB : lda, nb, dk, k0,
                                                                   status_dev, skip, 0, 0);
       if (cudaGetLastError() != cudaSuccess) return SP_ERR_CUDA;
@@ -520,14 +525,14 @@ sp_status potrf_lower_tc(float* A, int64_t n, int64_t lda, float* dinv, void* Pv
         count_launch();
         ProfScope prof(PK_PANEL_APPLY, 4.0 * TB * TB * TB, 0.0, stream);
         if (!split_lookahead) {
-          chol_next_diag_kernel<<<NM_CTAS, NM_THREADS, NM_SMEM, stream>>>(A + (k0 + nb) * lda + k0,
+          launch(chol_next_diag_kernel, NM_CTAS, NM_THREADS, NM_SMEM, stream, A + (k0 + nb) * lda + k0,
                                                                           A + (k0 + nb) * lda + (k0 + nb), lda, nb2,
                                                                           dk, LmT, S, status_dev, skip);
         } else {
-          chol_next_diag_stage1_kernel<<<NM_CTAS, NM_THREADS, NM_SMEM, stream>>>(A + (k0 + nb) * lda + k0, lda, nb2, dk,
+          launch(chol_next_diag_stage1_kernel, NM_CTAS, NM_THREADS, NM_SMEM, stream, A + (k0 + nb) * lda + k0, lda, nb2, dk,
                                                                                  LmT, status_dev, skip);
           count_launch();
-          chol_next_diag_stage2_kernel<<<NM_CTAS, NM_THREADS, NM_SMEM, stream>>>(A + (k0 + nb) * lda + (k0 + nb), lda,
+          launch(chol_next_diag_stage2_kernel, NM_CTAS, NM_THREADS, NM_SMEM, stream, A + (k0 + nb) * lda + (k0 + nb), lda,
                                                                                  nb2, LmT, S, skip);
         }
         if (cudaGetLastError() != cudaSuccess) return SP_ERR_CUDA;
@@ -847,7 +852,7 @@ sp_status potrf_potrs_tc_batched(float* A, int64_t n, int64_t m, int batch, int6
     const int64_t k0 = kb * TB;
     float* dk = dinv + kb * 2 * TB * TB;
     count_launch();
-    chol_diag128_kernel<<<batch, Diag::THREADS, Diag::SMEM, stream>>>(A + k0 * lda + k0, lda, TB, dk, k0, status_dev, skip,
+    launch(chol_diag128_kernel, batch, Diag::THREADS, Diag::SMEM, stream, A + k0 * lda + k0, lda, TB, dk, k0, status_dev, skip,
                                                                   a_bs, d_bs);
     if (cudaGetLastError() != cudaSuccess) return SP_ERR_CUDA;
     const int64_t rem = n - k0 - TB, prow = rem + m;

@@ -72,6 +72,7 @@ __global__ void __launch_bounds__(kWsWarps * 32, kWsPerSm) wanda_scores_kernel(
     const float* __restrict__ W, int64_t rows, int64_t cols, int64_t ldw, int vec_ok, int kind, int group,
     const float* __restrict__ colsq, int64_t colsq_stride, const double* __restrict__ colabs, double inv_tokens,
     int64_t n_units, float* scores, double* importance, double* part, double* colval, unsigned int* tickets) {
+  kernel_begin();
   __shared__ double red[kWsWarps][kWsCols];
   __shared__ double sm[33];
   __shared__ int s_last;
@@ -244,6 +245,7 @@ template <typename T>
 __global__ void __launch_bounds__(256, 4) weight_stats_partial_kernel(const T* __restrict__ W, int64_t ld,
                                                                       int64_t rows, int64_t cols, int axis,
                                                                       int64_t group, int vec_ok, double* part) {
+  kernel_begin();
   typedef typename StatVec<T>::Raw Raw;
   constexpr int V = StatVec<T>::V;
   __shared__ double sm[33];
@@ -308,6 +310,7 @@ __global__ void __launch_bounds__(256, 4) weight_stats_partial_kernel(const T* _
 // one CTA per block: the parts are added in a fixed order (strided over the threads, then the block tree)
 __global__ void __launch_bounds__(128) weight_stats_finish_kernel(const double* part, int parts, double count,
                                                                   int accumulate, double* stats) {
+  kernel_begin();
   __shared__ double sm[33];
   const int64_t b = blockIdx.x;
   double s[3] = {0.0, 0.0, 0.0};
@@ -327,6 +330,7 @@ __global__ void __launch_bounds__(128) weight_stats_finish_kernel(const double* 
 // (l1 + 0.05 var), from {sum |w|, sum w, sum w^2, count} per head / per matrix.
 __global__ void distribute_importance_kernel(const double* head_stats, int n_heads, const double* fc_stats, int n_fc,
                                              int L, double rho, double gamma, double* I_attn, double* I_mlp) {
+  kernel_begin();
   const int l = blockIdx.x * blockDim.x + threadIdx.x;
   if (l >= L) return;
   const double dl = pow(gamma, (double)(l + 1));
@@ -353,6 +357,7 @@ __global__ void distribute_importance_kernel(const double* head_stats, int n_hea
 // ------------------------------------------------------------------------------------------------ Lemma 1
 __global__ void lemma1_partials_kernel(sp_mat b, sp_mat c, sp_mat dd, sp_mat t, int64_t N, int64_t cols,
                                        int row_blocks, double* part) {
+  kernel_begin();
   const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= cols) return;
   const int64_t rows_per = ceil_div(N, (int64_t)row_blocks);
@@ -400,6 +405,7 @@ __global__ void __launch_bounds__(256, 2) lemma1_partials_vec_kernel(const T* __
                                                                      const T* __restrict__ tt, int64_t ldb,
                                                                      int64_t ldc, int64_t ldd, int64_t ldt, int64_t N,
                                                                      int64_t cols, double* part) {
+  kernel_begin();
   typedef typename L1Vec<T>::Raw Raw;
   constexpr int V = L1Vec<T>::V, CB = 32 * V;
   __shared__ double red[8][CB + 1];
@@ -459,6 +465,7 @@ __global__ void __launch_bounds__(256, 2) lemma1_partials_vec_kernel(const T* __
 // colred[j] = (sum over row blocks of the numerators, of the denominators) of column j
 __global__ void __launch_bounds__(256) lemma1_colred_kernel(const double* __restrict__ part, int row_blocks,
                                                             int64_t cols, double* colred) {
+  kernel_begin();
   const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= cols) return;
   const double2* p2 = reinterpret_cast<const double2*>(part);
@@ -483,6 +490,7 @@ __global__ void __launch_bounds__(1024) lemma1_finish_kernel(const double* part,
                                                              int group, int64_t n_units, float* scores,
                                                              double* importance, double* relaxed, double r_layer,
                                                              double* unit_e) {
+  kernel_begin();
   __shared__ double sm[33];
   double acc_s = 0.0, acc_ie = 0.0;
   for (int64_t u = threadIdx.x; u < n_units; u += blockDim.x) {
@@ -514,6 +522,7 @@ __global__ void __launch_bounds__(1024) lemma1_finish_kernel(const double* part,
 // one warp per row j: cb = <T0[j], W1t[j]>, cc = <T0[j], W10[j]>; s = (cb + cc) / (2 cc)
 __global__ void lemma1_gram_rows_kernel(const float* __restrict__ T0, const float* __restrict__ W1t,
                                         const float* __restrict__ W10, int64_t n, int64_t d, float* scores) {
+  kernel_begin();
   const int64_t j = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (j >= n) return;
@@ -529,6 +538,7 @@ __global__ void lemma1_gram_rows_kernel(const float* __restrict__ T0, const floa
 }
 
 __global__ void __launch_bounds__(1024) mean_scores_kernel(const float* scores, int64_t n, double* importance) {
+  kernel_begin();
   __shared__ double sm[33];
   double acc = 0.0;
   for (int64_t u = threadIdx.x; u < n; u += blockDim.x) acc += (double)scores[u];
@@ -542,6 +552,7 @@ __global__ void __launch_bounds__(1024) mean_scores_kernel(const float* scores, 
 __global__ void __launch_bounds__(1024) allocate_kernel(const double* I, const int64_t* n_units, int L, double rbar,
                                                         double T, const double* T_list, int T_relative, int mode,
                                                         double clip_hi, double* r_out, int64_t* k_out) {
+  kernel_begin();
   __shared__ double sm[33];
   const int t = threadIdx.x;
   r_out += (int64_t)blockIdx.x * L;
@@ -671,6 +682,7 @@ __global__ void __launch_bounds__(1024) topk_select_kernel(const float* __restri
                                                            uint8_t* mask_all, int64_t ld_mask, float* tau_all,
                                                            int32_t* kept_all, int64_t ld_idx, int smem_keys,
                                                            int skip_negative) {
+  kernel_begin();
   extern __shared__ uint32_t s_keys[];
   __shared__ int hist_w[32][256];     // one histogram per warp: adds collide only inside a warp
   __shared__ int hist[256];
@@ -798,6 +810,7 @@ __global__ void __launch_bounds__(1024) topk_select_kernel(const float* __restri
 }
 
 __global__ void __launch_bounds__(1024) mask_to_index_kernel(const uint8_t* mask, int64_t n, int32_t* kept_idx) {
+  kernel_begin();
   __shared__ int warp_tot[32];
   int64_t before = 0;
   for (int64_t base = 0; base < n; base += blockDim.x) {
@@ -813,6 +826,7 @@ __global__ void __launch_bounds__(1024) mask_to_index_kernel(const uint8_t* mask
 // perm = the kept channels in ascending order, then the pruned ones in ascending order; count[0] = kept channels
 __global__ void __launch_bounds__(1024) mask_to_perm_kernel(const uint8_t* mask, int64_t n, int32_t* perm,
                                                             int32_t* count) {
+  kernel_begin();
   __shared__ int warp_tot[32];
   __shared__ int s_kept;
   int kept = 0;
@@ -840,6 +854,7 @@ __global__ void __launch_bounds__(1024) mask_to_perm_kernel(const uint8_t* mask,
 // from, count_old of them); flags[1] = 1 - flags[0]
 __global__ void __launch_bounds__(1024) mask_changed_kernel(const uint8_t* mask, const int32_t* perm,
                                                             const int32_t* count_old, int64_t k, int32_t* flags) {
+  kernel_begin();
   __shared__ int s_bad;
   if (threadIdx.x == 0) s_bad = (int64_t)count_old[0] != k;
   __syncthreads();
@@ -856,6 +871,7 @@ __global__ void __launch_bounds__(1024) mask_changed_kernel(const uint8_t* mask,
 }
 
 __global__ void zero_rows_kernel(const uint8_t* mask, int group, float* W, int64_t rows, int64_t cols, int64_t ld) {
+  kernel_begin();
   const int64_t total = rows * cols;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = e / cols, j = e % cols;
@@ -864,6 +880,7 @@ __global__ void zero_rows_kernel(const uint8_t* mask, int group, float* W, int64
 }
 
 __global__ void zero_cols_kernel(const uint8_t* mask, int group, float* W, int64_t rows, int64_t cols, int64_t ld) {
+  kernel_begin();
   const int64_t total = rows * cols;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = e / cols, j = e % cols;
@@ -874,6 +891,7 @@ __global__ void zero_cols_kernel(const uint8_t* mask, int group, float* W, int64
 template <int W>
 __global__ void __launch_bounds__(kStripThreads) mask_rows_copy_kernel(const uint8_t* mask, const float* src, int64_t lds, float* dst, int64_t ldd,
                                       int64_t rows, int64_t cols) {
+  kernel_begin();
   for_strip<W>(rows, cols, [&](int64_t i, int64_t j, int) {
     dst[i * ldd + j] = mask[i] ? src[i * lds + j] : 0.f;
   });
@@ -936,7 +954,7 @@ cudaError_t wanda_scores(int kind, int group, const float* W, int64_t rows, int6
   cudaError_t e = cudaMemsetAsync(tickets, 0, (size_t)(cg + 1) * sizeof(unsigned int), stream);
   if (e != cudaSuccess) return e;
   count_launch();
-  wanda_scores_kernel<<<dim3((unsigned)cg, (unsigned)rb), kWsWarps * 32, 0, stream>>>(
+  launch(wanda_scores_kernel, dim3((unsigned)cg, (unsigned)rb), kWsWarps * 32, 0, stream, 
       W, rows, cols, ldw, vec_ok, k, group, colsq, colsq_stride, colabs, inv_tokens, n_units, scores, importance, part,
       colval, tickets);
   return cudaGetLastError();
@@ -967,14 +985,14 @@ cudaError_t weight_stats(const void* W, int32_t dt, int64_t ld, int64_t rows, in
   count_launch();
   const dim3 grid((unsigned)n_blocks, (unsigned)parts);
   if (dt == SP_BF16)
-    weight_stats_partial_kernel<__nv_bfloat16><<<grid, 256, 0, stream>>>(reinterpret_cast<const __nv_bfloat16*>(W), ld,
+    launch(weight_stats_partial_kernel<__nv_bfloat16>, grid, 256, 0, stream, reinterpret_cast<const __nv_bfloat16*>(W), ld,
                                                                          rows, cols, axis, group, vec_ok ? 1 : 0,
                                                                          scratch);
   else
-    weight_stats_partial_kernel<float><<<grid, 256, 0, stream>>>(reinterpret_cast<const float*>(W), ld, rows, cols, axis,
+    launch(weight_stats_partial_kernel<float>, grid, 256, 0, stream, reinterpret_cast<const float*>(W), ld, rows, cols, axis,
                                                                  group, vec_ok ? 1 : 0, scratch);
   count_launch();
-  weight_stats_finish_kernel<<<(unsigned)n_blocks, 128, 0, stream>>>(
+  launch(weight_stats_finish_kernel, (unsigned)n_blocks, 128, 0, stream, 
       scratch, parts, (double)block_rows * (double)block_cols, accumulate ? 1 : 0, stats);
   return cudaGetLastError();
 }
@@ -983,7 +1001,7 @@ cudaError_t distribute_importance(const double* head_stats, int n_heads, const d
                                   double rho, double gamma, double* I_attn, double* I_mlp, cudaStream_t stream) {
   if (L <= 0) return cudaSuccess;
   count_launch();
-  distribute_importance_kernel<<<(unsigned)ceil_div((int64_t)L, (int64_t)128), 128, 0, stream>>>(
+  launch(distribute_importance_kernel, (unsigned)ceil_div((int64_t)L, (int64_t)128), 128, 0, stream, 
       head_stats, n_heads, fc_stats, n_fc, L, rho, gamma, I_attn, I_mlp);
   return cudaGetLastError();
 }
@@ -1017,26 +1035,26 @@ cudaError_t lemma1_scores_stream(const sp_mat& b, const sp_mat& c, const sp_mat&
     if (rbv < 1) rbv = 1;
     const dim3 grid((unsigned)cg, (unsigned)rbv);
     if (dt == SP_BF16)
-      lemma1_partials_vec_kernel<__nv_bfloat16><<<grid, 256, 0, stream>>>(
+      launch(lemma1_partials_vec_kernel<__nv_bfloat16>, grid, 256, 0, stream, 
           reinterpret_cast<const __nv_bfloat16*>(b.ptr), reinterpret_cast<const __nv_bfloat16*>(c.ptr),
           reinterpret_cast<const __nv_bfloat16*>(dd.ptr), reinterpret_cast<const __nv_bfloat16*>(t.ptr), b.ld, c.ld,
           dd.ld, t.ld, N, cols, part);
     else
-      lemma1_partials_vec_kernel<float><<<grid, 256, 0, stream>>>(
+      launch(lemma1_partials_vec_kernel<float>, grid, 256, 0, stream, 
           reinterpret_cast<const float*>(b.ptr), reinterpret_cast<const float*>(c.ptr),
           reinterpret_cast<const float*>(dd.ptr), reinterpret_cast<const float*>(t.ptr), b.ld, c.ld, dd.ld, t.ld, N,
           cols, part);
     count_launch();
-    lemma1_colred_kernel<<<(unsigned)ceil_div(cols, (int64_t)256), 256, 0, stream>>>(part, (int)rbv, cols, colred);
+    launch(lemma1_colred_kernel, (unsigned)ceil_div(cols, (int64_t)256), 256, 0, stream, part, (int)rbv, cols, colred);
     count_launch();
-    lemma1_finish_kernel<<<1, 1024, 0, stream>>>(colred, 1, cols, group, n_units, scores, importance, relaxed, r_layer,
+    launch(lemma1_finish_kernel, 1, 1024, 0, stream, colred, 1, cols, group, n_units, scores, importance, relaxed, r_layer,
                                                  unit_e);
     return cudaGetLastError();
   }
-  lemma1_partials_kernel<<<dim3((unsigned)ceil_div(cols, 256), (unsigned)rb), 256, 0, stream>>>(b, c, dd, t, N, cols,
+  launch(lemma1_partials_kernel, dim3((unsigned)ceil_div(cols, 256), (unsigned)rb), 256, 0, stream, b, c, dd, t, N, cols,
                                                                                                rb, part);
   count_launch();
-  lemma1_finish_kernel<<<1, 1024, 0, stream>>>(part, rb, cols, group, n_units, scores, importance, relaxed, r_layer,
+  launch(lemma1_finish_kernel, 1, 1024, 0, stream, part, rb, cols, group, n_units, scores, importance, relaxed, r_layer,
                                                unit_e);
   return cudaGetLastError();
 }
@@ -1047,9 +1065,9 @@ cudaError_t lemma1_scores_gram(const float* T0, const float* W1t, const float* W
   if (n == 0) return cudaSuccess;
   ProfScope prof(PK_SCORES, 0.0, (double)n * (double)d * 12.0, stream);
   count_launch();
-  lemma1_gram_rows_kernel<<<(unsigned)ceil_div(n * 32, 256), 256, 0, stream>>>(T0, W1t, W10, n, d, scores);
+  launch(lemma1_gram_rows_kernel, (unsigned)ceil_div(n * 32, 256), 256, 0, stream, T0, W1t, W10, n, d, scores);
   count_launch();
-  mean_scores_kernel<<<1, 1024, 0, stream>>>(scores, n, importance);
+  launch(mean_scores_kernel, 1, 1024, 0, stream, scores, n, importance);
   return cudaGetLastError();
 }
 
@@ -1057,7 +1075,7 @@ cudaError_t allocate_sparsity(const double* I, const int64_t* n_units, int L, do
                               double clip_hi, double* r_out, int64_t* k_out, cudaStream_t stream) {
   ProfScope prof(PK_ALLOCATE, 0.0, (double)L * 32.0, stream);
   count_launch();
-  allocate_kernel<<<1, 1024, 0, stream>>>(I, n_units, L, rbar, T, nullptr, 0, mode, clip_hi, r_out, k_out);
+  launch(allocate_kernel, 1, 1024, 0, stream, I, n_units, L, rbar, T, nullptr, 0, mode, clip_hi, r_out, k_out);
   return cudaGetLastError();
 }
 
@@ -1066,7 +1084,7 @@ cudaError_t allocate_sparsity_grid(const double* I, const int64_t* n_units, int 
                                    cudaStream_t stream) {
   ProfScope prof(PK_ALLOCATE, 0.0, (double)L * 32.0 * n_T, stream);
   count_launch();
-  allocate_kernel<<<n_T, 1024, 0, stream>>>(I, n_units, L, rbar, 1.0, T_list, T_relative ? 1 : 0, mode, clip_hi, r_out,
+  launch(allocate_kernel, n_T, 1024, 0, stream, I, n_units, L, rbar, 1.0, T_list, T_relative ? 1 : 0, mode, clip_hi, r_out,
                                             k_out);
   return cudaGetLastError();
 }
@@ -1091,12 +1109,13 @@ cudaError_t topk_select_batched(const float* scores, int64_t ld_scores, int64_t 
   const int smem_keys = n <= kMaxSmemKeys ? 1 : 0;
   ProfScope prof(PK_TOPK, 0.0, (double)batch * (double)n * 5.0, stream);
   count_launch();
-  topk_select_kernel<<<(unsigned)batch, 1024, smem_keys ? (size_t)n * sizeof(uint32_t) : 0, stream>>>(
+  launch(topk_select_kernel, (unsigned)batch, 1024, smem_keys ? (size_t)n * sizeof(uint32_t) : 0, stream, 
       scores, ld_scores, n, k_all, k_list, mask, ld_mask, tau, kept_idx, ld_idx, smem_keys, skip_negative ? 1 : 0);
   return cudaGetLastError();
 }
 
 __global__ void fill_i32_kernel(int32_t* x, int n, int32_t v) {
+  kernel_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) x[i] = v;
 }
@@ -1110,6 +1129,7 @@ constexpr int kGselPerBlock = 8192;          // keys per block
 constexpr int kGselState = 260;
 
 __global__ void gsel_init_kernel(int32_t* st, int64_t K, int nblocks) {
+  kernel_begin();
   for (int i = threadIdx.x; i < kGselState + nblocks; i += blockDim.x) st[i] = 0;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -1120,6 +1140,7 @@ __global__ void gsel_init_kernel(int32_t* st, int64_t K, int nblocks) {
 
 __global__ void __launch_bounds__(kGselThreads) gsel_hist_kernel(const float* __restrict__ scores, int64_t n_row,
                                                                  int64_t ld, int64_t total, int pass, int32_t* st) {
+  kernel_begin();
   __shared__ int hist[256];
   __shared__ bool last;
   const int t = threadIdx.x;
@@ -1164,6 +1185,7 @@ __global__ void __launch_bounds__(kGselThreads) gsel_hist_kernel(const float* __
 // per-block counts of keys equal to the threshold key; the last block turns them into exclusive prefixes
 __global__ void __launch_bounds__(kGselThreads) gsel_count_kernel(const float* __restrict__ scores, int64_t n_row,
                                                                   int64_t ld, int64_t total, int32_t* st) {
+  kernel_begin();
   __shared__ int cnt;
   __shared__ bool last;
   const int t = threadIdx.x;
@@ -1201,6 +1223,7 @@ __global__ void __launch_bounds__(kGselThreads) gsel_mask_kernel(const float* __
                                                                  int64_t ld, int64_t ld_mask, int64_t total,
                                                                  const int32_t* st, uint8_t* mask, float* tau,
                                                                  int32_t* counts) {
+  kernel_begin();
   __shared__ int warp_tot[32];
   const int t = threadIdx.x;
   const uint32_t tkey = (uint32_t)st[256];
@@ -1251,6 +1274,7 @@ __global__ void __launch_bounds__(kGselThreads) gsel_mask_kernel(const float* __
 // layers left with fewer than min_keep units keep their own min_keep best: k_fix[l] = min_keep there, -1 elsewhere
 __global__ void gsel_repair_list_kernel(int32_t* counts, int L, int64_t min_keep, int64_t n_row, int64_t* k_fix,
                                         int64_t* counts_out) {
+  kernel_begin();
   const int l = blockIdx.x * blockDim.x + threadIdx.x;
   if (l >= L) return;
   const int64_t mk = min_keep < n_row ? min_keep : n_row;
@@ -1262,6 +1286,7 @@ __global__ void gsel_repair_list_kernel(int32_t* counts, int L, int64_t min_keep
 // counts[l] = kept units of layer l of an L x n mask (rows ld apart); one block per layer
 __global__ void __launch_bounds__(256) mask_row_counts_kernel(const uint8_t* __restrict__ mask, int64_t n, int64_t ld,
                                                               int32_t* __restrict__ counts) {
+  kernel_begin();
   __shared__ int sm[256];
   int c = 0;
   for (int64_t j = threadIdx.x; j < n; j += 256) c += mask[(int64_t)blockIdx.x * ld + j] != 0;
@@ -1298,18 +1323,18 @@ cudaError_t global_select(const float* scores, int64_t ld_scores, int64_t n, int
     e = topk_select(scores, total, K, mask, tau, nullptr, stream);
     if (e != cudaSuccess) return e;
     count_launch();
-    mask_row_counts_kernel<<<L, 256, 0, stream>>>(mask, n, ld_mask, counts);
+    launch(mask_row_counts_kernel, L, 256, 0, stream, mask, n, ld_mask, counts);
   } else if (K <= 0 || K >= total) {      // nothing or everything kept: no threshold to find
     e = cudaMemset2DAsync(mask, (size_t)ld_mask, K > 0 ? 1 : 0, (size_t)n, (size_t)L, stream);
     if (e != cudaSuccess) return e;
     count_launch();
-    gsel_init_kernel<<<1, 256, 0, stream>>>(st, 0, nblocks);
+    launch(gsel_init_kernel, 1, 256, 0, stream, st, 0, nblocks);
     // counts = n or 0 per layer through the repair list below
     e = cudaMemsetAsync(counts, 0, (size_t)L * 4, stream);
     if (e != cudaSuccess) return e;
     if (K > 0) {
       count_launch();
-      fill_i32_kernel<<<(L + 255) / 256, 256, 0, stream>>>(counts, L, (int32_t)n);
+      launch(fill_i32_kernel, (L + 255) / 256, 256, 0, stream, counts, L, (int32_t)n);
     }
     if (tau) {
       e = cudaMemsetAsync(tau, 0xff, sizeof(float), stream);       // NaN: no threshold
@@ -1317,14 +1342,14 @@ cudaError_t global_select(const float* scores, int64_t ld_scores, int64_t n, int
     }
   } else {
     count_launch(7);
-    gsel_init_kernel<<<1, 256, 0, stream>>>(st, K, nblocks);
+    launch(gsel_init_kernel, 1, 256, 0, stream, st, K, nblocks);
     for (int pass = 0; pass < 4; ++pass)
-      gsel_hist_kernel<<<nblocks, kGselThreads, 0, stream>>>(scores, n, ld_scores, total, pass, st);
-    gsel_count_kernel<<<nblocks, kGselThreads, 0, stream>>>(scores, n, ld_scores, total, st);
-    gsel_mask_kernel<<<nblocks, kGselThreads, 0, stream>>>(scores, n, ld_scores, ld_mask, total, st, mask, tau, counts);
+      launch(gsel_hist_kernel, nblocks, kGselThreads, 0, stream, scores, n, ld_scores, total, pass, st);
+    launch(gsel_count_kernel, nblocks, kGselThreads, 0, stream, scores, n, ld_scores, total, st);
+    launch(gsel_mask_kernel, nblocks, kGselThreads, 0, stream, scores, n, ld_scores, ld_mask, total, st, mask, tau, counts);
   }
   count_launch();
-  gsel_repair_list_kernel<<<(L + 255) / 256, 256, 0, stream>>>(counts, L, min_keep, n, k_fix, counts_out);
+  launch(gsel_repair_list_kernel, (L + 255) / 256, 256, 0, stream, counts, L, min_keep, n, k_fix, counts_out);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (min_keep > 0)   // per-layer top-k where the threshold left too few units (layers with k_fix < 0 are skipped)
@@ -1335,7 +1360,7 @@ cudaError_t global_select(const float* scores, int64_t ld_scores, int64_t n, int
 cudaError_t mask_to_index(const uint8_t* mask, int64_t n, int32_t* kept_idx, cudaStream_t stream) {
   if (n == 0) return cudaSuccess;
   count_launch();
-  mask_to_index_kernel<<<1, 1024, 0, stream>>>(mask, n, kept_idx);
+  launch(mask_to_index_kernel, 1, 1024, 0, stream, mask, n, kept_idx);
   return cudaGetLastError();
 }
 
@@ -1343,6 +1368,7 @@ template <int W>
 __global__ void __launch_bounds__(kStripThreads) scale_block_kernel(float* C, int64_t ld, int64_t rows, int64_t cols,
                                                                     const int32_t* f_bits, int power,
                                                                     const int32_t* skip) {
+  kernel_begin();
   if (skip != nullptr && *skip != 0) return;   // conditional launch (see SkipScope)
   const float f = __int_as_float(f_bits[0]);
   const float s = power == 2 ? f * f : f;
@@ -1369,6 +1395,7 @@ __global__ void __launch_bounds__(kStripThreads) scale_block_kernel(float* C, in
 
 // inv[perm[i]] = i
 __global__ void invert_perm_kernel(const int32_t* __restrict__ perm, int64_t n, int32_t* __restrict__ inv) {
+  kernel_begin();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) inv[perm[i]] = (int32_t)i;
 }
@@ -1380,6 +1407,7 @@ __global__ void invert_perm_kernel(const int32_t* __restrict__ perm, int64_t n, 
 // n = 16384: 2.6 -> 0.7 ms; 64 x 64 tiles are 10 % slower).
 __global__ void __launch_bounds__(256) unpermute_gram_kernel(const float* __restrict__ Gp, const int32_t* __restrict__ inv,
                                                              int64_t n, float* __restrict__ G) {
+  kernel_begin();
   constexpr int TS = 32;
   __shared__ float tile[TS][TS + 1];
   __shared__ int pr_s[TS], pc_s[TS];
@@ -1417,12 +1445,14 @@ template <int W>
 __global__ void __launch_bounds__(kStripThreads) unpermute_cols_kernel(const float* __restrict__ Rp,
                                                                        const int32_t* __restrict__ perm, int64_t rows,
                                                                        int64_t n, float* __restrict__ R) {
+  kernel_begin();
   int64_t at[kStripPer];
   strip_index<W>(perm, n, at);
   for_strip<W>(rows, n, [&](int64_t r, int64_t j, int q) { R[r * n + at[q]] = Rp[r * n + j]; });
 }
 
 __global__ void decay_tag_set_kernel(int32_t* tag, int k, float c, int valid, int h_ld, int h_chunk) {
+  kernel_begin();
   tag[1] = valid ? k : -1;
   tag[2] = __float_as_int(c);
   tag[4] = valid ? h_ld : 0;
@@ -1430,6 +1460,7 @@ __global__ void decay_tag_set_kernel(int32_t* tag, int k, float c, int valid, in
 }
 
 __global__ void h_next_ready_kernel(const int32_t* same, const int32_t* tag, int h_ld, int h_chunk, int32_t* ready) {
+  kernel_begin();
   ready[0] = (same[0] != 0 && tag[4] == h_ld && tag[5] == h_chunk && h_ld > 0) ? 1 : 0;
   ready[1] = 1 - ready[0];
 }
@@ -1438,6 +1469,7 @@ template <int W>
 __global__ void __launch_bounds__(kStripThreads) unpermute_rows_kernel(const float* __restrict__ Rp,
                                                                        const int32_t* __restrict__ perm, int64_t n,
                                                                        int64_t cols, float* __restrict__ R) {
+  kernel_begin();
   for_strip<W>(n, cols, [&](int64_t i, int64_t j, int) { R[(int64_t)perm[i] * cols + j] = Rp[i * cols + j]; });
 }
 
@@ -1446,7 +1478,7 @@ cudaError_t scale_block(float* C, int64_t ld, int64_t rows, int64_t cols, const 
   if (rows * cols <= 0) return cudaSuccess;
   count_launch();
   strip_launch(rows, cols, [&](auto w, dim3 grid, dim3 block) {
-    scale_block_kernel<decltype(w)::value><<<grid, block, 0, stream>>>(C, ld, rows, cols, f_bits, power, skip_flag());
+    launch(scale_block_kernel<decltype(w)::value>, grid, block, 0, stream, C, ld, rows, cols, f_bits, power, skip_flag());
   });
   return cudaGetLastError();
 }
@@ -1455,9 +1487,9 @@ cudaError_t unpermute_gram(const float* Gp, const int32_t* perm, int64_t n, floa
                            cudaStream_t stream) {
   if (n <= 0) return cudaSuccess;
   count_launch();
-  invert_perm_kernel<<<(unsigned)ceil_div(n, (int64_t)256), 256, 0, stream>>>(perm, n, inv);
+  launch(invert_perm_kernel, (unsigned)ceil_div(n, (int64_t)256), 256, 0, stream, perm, n, inv);
   count_launch();
-  unpermute_gram_kernel<<<lower_tiles(n, 32), 256, 0, stream>>>(Gp, inv, n, G);
+  launch(unpermute_gram_kernel, lower_tiles(n, 32), 256, 0, stream, Gp, inv, n, G);
   return cudaGetLastError();
 }
 
@@ -1466,7 +1498,7 @@ cudaError_t unpermute_cols(const float* Rp, const int32_t* perm, int64_t rows, i
   if (rows * n <= 0) return cudaSuccess;
   count_launch();
   strip_launch(rows, n, [&](auto w, dim3 grid, dim3 block) {
-    unpermute_cols_kernel<decltype(w)::value><<<grid, block, 0, stream>>>(Rp, perm, rows, n, R);
+    launch(unpermute_cols_kernel<decltype(w)::value>, grid, block, 0, stream, Rp, perm, rows, n, R);
   });
   return cudaGetLastError();
 }
@@ -1474,14 +1506,14 @@ cudaError_t unpermute_cols(const float* Rp, const int32_t* perm, int64_t rows, i
 cudaError_t decay_tag_set(int32_t* tag, int64_t k, float c, bool valid, int64_t h_ld, int64_t h_chunk,
                           cudaStream_t stream) {
   count_launch();
-  decay_tag_set_kernel<<<1, 1, 0, stream>>>(tag, (int)k, c, valid ? 1 : 0, (int)h_ld, (int)h_chunk);
+  launch(decay_tag_set_kernel, 1, 1, 0, stream, tag, (int)k, c, valid ? 1 : 0, (int)h_ld, (int)h_chunk);
   return cudaGetLastError();
 }
 
 cudaError_t h_next_ready(const int32_t* same, const int32_t* tag, int64_t h_ld, int64_t h_chunk, int32_t* ready,
                          cudaStream_t stream) {
   count_launch();
-  h_next_ready_kernel<<<1, 1, 0, stream>>>(same, tag, (int)h_ld, (int)h_chunk, ready);
+  launch(h_next_ready_kernel, 1, 1, 0, stream, same, tag, (int)h_ld, (int)h_chunk, ready);
   return cudaGetLastError();
 }
 
@@ -1490,13 +1522,14 @@ cudaError_t unpermute_rows(const float* Rp, const int32_t* perm, int64_t n, int6
   if (n * cols <= 0) return cudaSuccess;
   count_launch();
   strip_launch(n, cols, [&](auto w, dim3 grid, dim3 block) {
-    unpermute_rows_kernel<decltype(w)::value><<<grid, block, 0, stream>>>(Rp, perm, n, cols, R);
+    launch(unpermute_rows_kernel<decltype(w)::value>, grid, block, 0, stream, Rp, perm, n, cols, R);
   });
   return cudaGetLastError();
 }
 
 __global__ void __launch_bounds__(1024) mask_count_check_kernel(const uint8_t* mask, int64_t n, int64_t k,
                                                                 int32_t* status) {
+  kernel_begin();
   __shared__ int warp_tot[32];
   int kept = 0;
   for (int64_t base = 0; base < n; base += blockDim.x) {
@@ -1511,21 +1544,21 @@ __global__ void __launch_bounds__(1024) mask_count_check_kernel(const uint8_t* m
 cudaError_t mask_count_check(const uint8_t* mask, int64_t n, int64_t k, int32_t* status, cudaStream_t stream) {
   if (status == nullptr) return cudaSuccess;
   count_launch();
-  mask_count_check_kernel<<<1, 1024, 0, stream>>>(mask, n, k, status);
+  launch(mask_count_check_kernel, 1, 1024, 0, stream, mask, n, k, status);
   return cudaGetLastError();
 }
 
 cudaError_t mask_to_perm(const uint8_t* mask, int64_t n, int32_t* perm, int32_t* count, cudaStream_t stream) {
   if (n == 0) return cudaSuccess;
   count_launch();
-  mask_to_perm_kernel<<<1, 1024, 0, stream>>>(mask, n, perm, count);
+  launch(mask_to_perm_kernel, 1, 1024, 0, stream, mask, n, perm, count);
   return cudaGetLastError();
 }
 
 cudaError_t mask_changed(const uint8_t* mask, const int32_t* perm, const int32_t* count_old, int64_t k, int32_t* flags,
                          cudaStream_t stream) {
   count_launch();
-  mask_changed_kernel<<<1, 1024, 0, stream>>>(mask, perm, count_old, k, flags);
+  launch(mask_changed_kernel, 1, 1024, 0, stream, mask, perm, count_old, k, flags);
   return cudaGetLastError();
 }
 
@@ -1534,11 +1567,11 @@ cudaError_t zero_pruned(const uint8_t* mask, int group, float* W_rows, int64_t r
   if (W_rows && r_rows * r_cols > 0) {
     ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
     count_launch();
-    zero_rows_kernel<<<grid_for(r_rows * r_cols, 256), 256, 0, stream>>>(mask, group, W_rows, r_rows, r_cols, r_ld);
+    launch(zero_rows_kernel, grid_for(r_rows * r_cols, 256), 256, 0, stream, mask, group, W_rows, r_rows, r_cols, r_ld);
   }
   if (W_cols && c_rows * c_cols > 0) {
     count_launch();
-    zero_cols_kernel<<<grid_for(c_rows * c_cols, 256), 256, 0, stream>>>(mask, group, W_cols, c_rows, c_cols, c_ld);
+    launch(zero_cols_kernel, grid_for(c_rows * c_cols, 256), 256, 0, stream, mask, group, W_cols, c_rows, c_cols, c_ld);
   }
   return cudaGetLastError();
 }
@@ -1549,7 +1582,7 @@ cudaError_t mask_rows_copy(const uint8_t* mask, const float* src, int64_t lds, f
   ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
   count_launch();
   strip_launch(rows, cols, [&](auto w, dim3 grid, dim3 block) {
-    mask_rows_copy_kernel<decltype(w)::value><<<grid, block, 0, stream>>>(mask, src, lds, dst, ldd, rows, cols);
+    launch(mask_rows_copy_kernel<decltype(w)::value>, grid, block, 0, stream, mask, src, lds, dst, ldd, rows, cols);
   });
   return cudaGetLastError();
 }

@@ -74,6 +74,7 @@ template <int NV>
 __global__ void __launch_bounds__(kRowWarps * 32) softmax_rows_kernel(float* __restrict__ S, int64_t rows, int T,
                                                                       int causal, __nv_bfloat16* __restrict__ Sb,
                                                                       int64_t plane) {
+  kernel_begin();
   const int lane = threadIdx.x & 31;
   const int64_t r = (int64_t)blockIdx.x * kRowWarps + (threadIdx.x >> 5);
   if (r >= rows) return;
@@ -100,6 +101,7 @@ __global__ void __launch_bounds__(256) p_update_kernel(float* __restrict__ P, co
                                                        const float* __restrict__ G1, const float* __restrict__ eta,
                                                        int64_t per_pair, int64_t pairs, float alpha, float beta,
                                                        __nv_bfloat16* __restrict__ Pb, int64_t plane) {
+  kernel_begin();
   struct __align__(4 * V) F { float v[V]; };
   struct __align__(2 * V) H { __nv_bfloat16 v[V]; };
   for (int64_t b = strip_row(); b < pairs; b += strip_rows()) {
@@ -135,6 +137,7 @@ __global__ void __launch_bounds__(kRowWarps * 32) softmax_backward_rows_kernel(f
                                                                                int64_t rows, int T, int causal,
                                                                                float beta,
                                                                                __nv_bfloat16* __restrict__ dSb) {
+  kernel_begin();
   const int lane = threadIdx.x & 31;
   const int64_t r = (int64_t)blockIdx.x * kRowWarps + (threadIdx.x >> 5);
   if (r >= rows) return;
@@ -166,6 +169,7 @@ __global__ void __launch_bounds__(kRowWarps * 32) softmax_backward_rows_kernel(f
 // one block per pair, fixed summation order.  out[b] = sum x^2 (+ sum y^2), b = seq * H + head.
 __global__ void __launch_bounds__(256) pair_sumsq_kernel(const float* __restrict__ x, const float* __restrict__ y,
                                                          int64_t ld, int T, int d_h, int H, double* __restrict__ out) {
+  kernel_begin();
   __shared__ double sm[256];
   const int b = blockIdx.x, seq = b / H, head = b % H;
   const int64_t base = (int64_t)seq * T * ld + (int64_t)head * d_h;
@@ -202,6 +206,7 @@ __global__ void __launch_bounds__(256) pair_sumsq_kernel(const float* __restrict
 // mode 1 (Eq. 87): eta = eta_z / (2 alpha + beta s / d_h).
 __global__ void step_size_kernel(const double* __restrict__ s, int n, int mode, double alpha, double beta, double eta_z,
                                  int d_h, float* __restrict__ eta) {
+  kernel_begin();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= n) return;
   eta[b] = mode == 0 ? (float)(1.0 / (2.0 * (alpha * s[b] + beta)))
@@ -219,6 +224,7 @@ __global__ void __launch_bounds__(256) z_update_kernel(float* __restrict__ Zq, f
                                                        const float* __restrict__ eta, int64_t tokens, int d, int T,
                                                        int d_h, float alpha, __nv_bfloat16* __restrict__ Zqs,
                                                        __nv_bfloat16* __restrict__ Zks, int64_t plane) {
+  kernel_begin();
   struct __align__(4 * V) F { float v[V]; };
   struct __align__(2 * V) B { __nv_bfloat16 v[V]; };
   const int H = d / d_h, c = (int)(blockIdx.x * blockDim.x + threadIdx.x) * V;
@@ -252,6 +258,7 @@ __global__ void __launch_bounds__(256) z_update_kernel(float* __restrict__ Zq, f
 // hi / lo bf16 planes of a dense fp32 tensor of `total` elements: dst[e] = bf16(x), dst[plane + e] = bf16(x - hi).
 __global__ void __launch_bounds__(256) split_planes_kernel(const float* __restrict__ x, int64_t total,
                                                            __nv_bfloat16* __restrict__ dst, int64_t plane) {
+  kernel_begin();
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
     const float v = x[e];
     const __nv_bfloat16 hi = __float2bfloat16_rn(v);
@@ -264,6 +271,7 @@ __global__ void __launch_bounds__(256) split_planes_kernel(const float* __restri
 __global__ void __launch_bounds__(256) split_heads_kernel(const float* __restrict__ P, int64_t n_seq, int64_t H, int64_t per_pair,
                                                           const __grid_constant__ HeadList heads,
                                                           __nv_bfloat16* __restrict__ dst, int64_t plane) {
+  kernel_begin();
   struct __align__(8) B { __nv_bfloat162 v[2]; };
   for (int64_t seq = blockIdx.z; seq < n_seq; seq += gridDim.z) {
     const float* src = P + (seq * H + heads.h[blockIdx.y]) * per_pair;
@@ -285,6 +293,7 @@ __global__ void __launch_bounds__(256) split_heads_kernel(const float* __restric
 __global__ void split_head_cols_kernel(const float* __restrict__ A, int64_t tokens, int64_t d, int d_h,
                                        const __grid_constant__ HeadList heads, __nv_bfloat16* __restrict__ dst, int64_t ld,
                                        int64_t lo_off) {
+  kernel_begin();
   const int per_block = blockDim.x / d_h > 0 ? blockDim.x / d_h : 1;
   const int64_t t0 = (int64_t)blockIdx.x * per_block;
   for (int e = threadIdx.x; e < per_block * d_h; e += blockDim.x) {
@@ -301,6 +310,7 @@ __global__ void split_head_cols_kernel(const float* __restrict__ A, int64_t toke
 
 __global__ void __launch_bounds__(1024) add_ridge_batched_kernel(float* __restrict__ G, int64_t bs, int64_t n, double rho,
                                                                  int rel) {
+  kernel_begin();
   __shared__ double sm[32];
   G += (int64_t)blockIdx.x * bs;
   double s = 0.0;
@@ -322,6 +332,7 @@ __global__ void __launch_bounds__(1024) add_ridge_batched_kernel(float* __restri
 __global__ void __launch_bounds__(256) place_heads_kernel(const float* __restrict__ src, int64_t bs, int64_t d,
                                                           const __grid_constant__ HeadList heads, float* __restrict__ W,
                                                           int64_t ldw) {
+  kernel_begin();
   const float* in = src + (int64_t)blockIdx.y * bs + (int64_t)blockIdx.x * d;
   float* out = W + ((int64_t)heads.h[blockIdx.y] * gridDim.x + blockIdx.x) * ldw;
   for (int64_t c = threadIdx.x; c < d; c += 256) out[c] = in[c];
@@ -329,6 +340,7 @@ __global__ void __launch_bounds__(256) place_heads_kernel(const float* __restric
 
 template <typename T>
 __global__ void set_identity_kernel(T* A, int64_t n, int64_t ld) {
+  kernel_begin();
   const int64_t total = n * n;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = e / n, j = e % n;
@@ -354,7 +366,7 @@ cudaError_t mha_softmax_rows(float* S, int64_t pairs, int T, bool causal, void* 
   count_launch();
   const unsigned grid = (unsigned)ceil_div(rows, (int64_t)kRowWarps);
   const auto run = [&](auto kernel) {
-    kernel<<<grid, kRowWarps * 32, 0, stream>>>(S, rows, T, causal ? 1 : 0, reinterpret_cast<__nv_bfloat16*>(Sb), plane);
+    launch(kernel, grid, kRowWarps * 32, 0, stream, S, rows, T, causal ? 1 : 0, reinterpret_cast<__nv_bfloat16*>(Sb), plane);
   };
   if (T <= 128) run(softmax_rows_kernel<4>);
   else if (T <= 256) run(softmax_rows_kernel<8>);
@@ -380,8 +392,8 @@ cudaError_t mha_p_update(float* P, const float* Phi, const float* G1, const floa
   if (gx * gy > cap) gy = cap / gx > 0 ? cap / gx : 1;
   const dim3 grid((unsigned)gx, (unsigned)gy);
   __nv_bfloat16* pb = reinterpret_cast<__nv_bfloat16*>(Pb);
-  if (vec) p_update_kernel<4><<<grid, block, 0, stream>>>(P, Phi, G1, eta, per_pair, pairs, (float)alpha, (float)beta, pb, plane);
-  else p_update_kernel<1><<<grid, block, 0, stream>>>(P, Phi, G1, eta, per_pair, pairs, (float)alpha, (float)beta, pb, plane);
+  if (vec) launch(p_update_kernel<4>, grid, block, 0, stream, P, Phi, G1, eta, per_pair, pairs, (float)alpha, (float)beta, pb, plane);
+  else launch(p_update_kernel<1>, grid, block, 0, stream, P, Phi, G1, eta, per_pair, pairs, (float)alpha, (float)beta, pb, plane);
   return cudaGetLastError();
 }
 
@@ -393,7 +405,7 @@ cudaError_t mha_softmax_backward_rows(float* S, const float* P, int64_t pairs, i
   count_launch();
   const unsigned grid = (unsigned)ceil_div(rows, (int64_t)kRowWarps);
   const auto run = [&](auto kernel) {
-    kernel<<<grid, kRowWarps * 32, 0, stream>>>(S, P, rows, T, causal ? 1 : 0, (float)beta,
+    launch(kernel, grid, kRowWarps * 32, 0, stream, S, P, rows, T, causal ? 1 : 0, (float)beta,
                                                 reinterpret_cast<__nv_bfloat16*>(dSb));
   };
   if (T <= 128) run(softmax_backward_rows_kernel<4>);
@@ -408,8 +420,8 @@ cudaError_t mha_step_sizes(const float* x, const float* y, int64_t ld, int64_t n
   if (n == 0) return cudaSuccess;
   ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
   count_launch(2);
-  pair_sumsq_kernel<<<n, 256, 0, stream>>>(x, y, ld, T, d_h, H, sums);
-  step_size_kernel<<<(n + 255) / 256, 256, 0, stream>>>(sums, n, mode, alpha, beta, eta_z, d_h, eta);
+  launch(pair_sumsq_kernel, n, 256, 0, stream, x, y, ld, T, d_h, H, sums);
+  launch(step_size_kernel, (n + 255) / 256, 256, 0, stream, sums, n, mode, alpha, beta, eta_z, d_h, eta);
   return cudaGetLastError();
 }
 
@@ -429,7 +441,7 @@ cudaError_t mha_z_update(float* Zq, float* Zk, const float* Gq, const float* Gk,
   int64_t gy = ceil_div((int64_t)sm_count() * 8, gx);
   if (gy > row_blocks) gy = row_blocks;
   const auto run = [&](auto kernel) {
-    kernel<<<dim3((unsigned)gx, (unsigned)gy), block, 0, stream>>>(Zq, Zk, Gq, Gk, Tq, Tk, eta, tokens, d, T, d_h, (float)alpha,
+    launch(kernel, dim3((unsigned)gx, (unsigned)gy), block, 0, stream, Zq, Zk, Gq, Gk, Tq, Tk, eta, tokens, d, T, d_h, (float)alpha,
                                                                  reinterpret_cast<__nv_bfloat16*>(Zqs),
                                                                  reinterpret_cast<__nv_bfloat16*>(Zks), plane);
   };
@@ -442,7 +454,7 @@ template <typename T>
 cudaError_t set_identity(T* A, int64_t n, int64_t ld, cudaStream_t stream) {
   if (n == 0) return cudaSuccess;
   count_launch();
-  set_identity_kernel<<<grid_1d(n * n, 256), 256, 0, stream>>>(A, n, ld);
+  launch(set_identity_kernel<T>, grid_1d(n * n, 256), 256, 0, stream, A, n, ld);
   return cudaGetLastError();
 }
 template cudaError_t set_identity<float>(float*, int64_t, int64_t, cudaStream_t);
@@ -452,7 +464,7 @@ cudaError_t split_planes(const float* x, int64_t total, void* dst, int64_t plane
   if (total == 0) return cudaSuccess;
   ProfScope prof(PK_ELEMENTWISE, 0.0, (double)total * 8.0, stream);
   count_launch();
-  split_planes_kernel<<<grid_1d(total, 256), 256, 0, stream>>>(x, total, reinterpret_cast<__nv_bfloat16*>(dst), plane);
+  launch(split_planes_kernel, grid_1d(total, 256), 256, 0, stream, x, total, reinterpret_cast<__nv_bfloat16*>(dst), plane);
   return cudaGetLastError();
 }
 
@@ -466,7 +478,7 @@ cudaError_t mha_split_heads(const float* P, int64_t n_seq, int64_t H, int64_t pe
   const int64_t cap = ceil_div((int64_t)sm_count() * 32, n_seq * heads.n);
   if (gx > cap) gx = cap;
   const unsigned gz = (unsigned)(n_seq < 65535 ? n_seq : 65535);
-  split_heads_kernel<<<dim3((unsigned)gx, (unsigned)heads.n, gz), 256, 0, stream>>>(
+  launch(split_heads_kernel, dim3((unsigned)gx, (unsigned)heads.n, gz), 256, 0, stream, 
       P, n_seq, H, per_pair, heads, reinterpret_cast<__nv_bfloat16*>(dst), plane);
   return cudaGetLastError();
 }
@@ -477,7 +489,7 @@ cudaError_t mha_split_head_cols(const float* A, int64_t tokens, int64_t d, int64
   ProfScope prof(PK_ELEMENTWISE, 0.0, (double)tokens * heads.n * d_h * 8.0, stream);
   count_launch();
   const int64_t per_block = 256 / d_h > 0 ? 256 / d_h : 1;
-  split_head_cols_kernel<<<dim3((unsigned)ceil_div(tokens, per_block), (unsigned)heads.n), 256, 0, stream>>>(
+  launch(split_head_cols_kernel, dim3((unsigned)ceil_div(tokens, per_block), (unsigned)heads.n), 256, 0, stream, 
       A, tokens, d, (int)d_h, heads, reinterpret_cast<__nv_bfloat16*>(dst), ld, lo_off);
   return cudaGetLastError();
 }
@@ -486,7 +498,7 @@ cudaError_t add_ridge_batched(float* G, int64_t bs, int64_t n, int batch, double
   if (n == 0 || batch == 0) return cudaSuccess;
   ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
   count_launch();
-  add_ridge_batched_kernel<<<(unsigned)batch, 1024, 0, stream>>>(G, bs, n, rho, rel ? 1 : 0);
+  launch(add_ridge_batched_kernel, (unsigned)batch, 1024, 0, stream, G, bs, n, rho, rel ? 1 : 0);
   return cudaGetLastError();
 }
 
@@ -495,7 +507,7 @@ cudaError_t mha_place_heads(const float* src, int64_t bs, int64_t d_h, int64_t d
   if (heads.n == 0 || d_h == 0) return cudaSuccess;
   ProfScope prof(PK_ELEMENTWISE, 0.0, (double)heads.n * d_h * d * 8.0, stream);
   count_launch();
-  place_heads_kernel<<<dim3((unsigned)d_h, (unsigned)heads.n), 256, 0, stream>>>(src, bs, d, heads, W, ldw);
+  launch(place_heads_kernel, dim3((unsigned)d_h, (unsigned)heads.n), 256, 0, stream, src, bs, d, heads, W, ldw);
   return cudaGetLastError();
 }
 

@@ -54,6 +54,11 @@ ProfScope::~ProfScope() {
   if (slot >= 0) cudaEventRecord(g_slots[slot].stop, stream);
 }
 
+bool& overlap_flag() {
+  static thread_local bool on = false;
+  return on;
+}
+
 }  // namespace sp
 
 extern "C" {
