@@ -34,8 +34,8 @@
  *     All other calls, sp_ffn_cache_input_inverse and the precise solves among
  *     them, use the caller's stream alone.  Nothing else persists inside the library.
  *   - Reproducibility: by default a product whose tile count leaves SMs idle is cut along K and its partial
- *     products add up in C in an order that is not fixed, and a factorisation adds updates of its trailing matrix from
- *     two streams (a backward sweep too, for more right-hand sides than one wave of its panels holds); fp32 results
+ *     products add up in C in an order that is not fixed, and a backward sweep with more right-hand sides than one wave of its
+ *     panels holds adds updates from two streams (a factorisation takes its updates in step order); fp32 results
  *     (accumulators, recovered weights, scores) can then differ in their last bits between two runs on equal inputs,
  *     and a mask can differ at scores that tie within that rounding.  sp_set_reproducible(1) switches both off
  *     (process-wide): every sum is then taken in an order fixed by the call's arguments and equal inputs give

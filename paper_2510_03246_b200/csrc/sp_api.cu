@@ -192,8 +192,10 @@ bool make_assist(SolveAssist& a, int prio) {
          cudaEventCreateWithFlags(&a.rest_done[0], cudaEventDisableTiming) == cudaSuccess &&
          cudaEventCreateWithFlags(&a.rest_done[1], cudaEventDisableTiming) == cudaSuccess &&
          cudaEventCreateWithFlags(&a.near_done, cudaEventDisableTiming) == cudaSuccess &&
+         cudaEventCreateWithFlags(&a.next_done, cudaEventDisableTiming) == cudaSuccess &&
          cudaStreamCreateWithPriority(&a.far_stream, cudaStreamNonBlocking, prio) == cudaSuccess &&
          cudaEventCreateWithFlags(&a.far_go, cudaEventDisableTiming) == cudaSuccess &&
+         cudaEventCreateWithFlags(&a.far_first, cudaEventDisableTiming) == cudaSuccess &&
          cudaEventCreateWithFlags(&a.far_done[0], cudaEventDisableTiming) == cudaSuccess &&
          cudaEventCreateWithFlags(&a.far_done[1], cudaEventDisableTiming) == cudaSuccess;
 }

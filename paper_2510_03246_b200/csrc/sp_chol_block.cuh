@@ -25,8 +25,8 @@ __device__ __forceinline__ double recip_sqrt(double x) { return rsqrt(x); }
 //      sub-block comes first, by all warps; the other pieces run beside the next phase A.
 // Every entry receives its updates column by column in ascending order, whatever the blocking.  What bounds the kernel is
 // latency: A (about 120 cycles per column), B and the first piece of C; for 128 columns the other pieces take as long as
-// A.  Measured inside a factorisation: 25 us for 128 columns in fp32, 14 us for 64 in fp64.  (One 4 x 4 block per thread,
-// with two block barriers and all warps' shared update between one 4 x 4 pivot block and the next: 37 and 20 us.)
+// A.  Measured inside a factorisation: 14 us for 64 columns in fp64.  (One 4 x 4 block per thread, with two block barriers and
+// all warps' shared update between one 4 x 4 pivot block and the next: 20 us.)  fp32 takes DiagTiles below.
 template <typename T, int NB>
 struct DiagBlock {
   static constexpr int SB = 32, NS = NB / SB;
@@ -261,10 +261,9 @@ struct DiagBlock {
         for (int v = 0; v < V; ++v) inv[(cs + c + v) * NB + t] = q.v[v];
       }
     };
-    // sub-blocks beyond nb are those of an identity: nothing is eliminated there, their columns of X stay as they are (a
-    // solve for 17 unknowns in fp32: 53 us, 65 through all four).  Two sub-blocks (fp64) are always run: a bound known at
-    // compile time is worth more there (1 % of a fp32-mode layer).
-    const int ns = NS > 2 ? (nb + SB - 1) / SB : NS;
+    // (both sub-blocks are always run, also where the second is that of an identity: a bound known at compile time is worth
+    // more, 1 % of a fp32-mode layer)
+    constexpr int ns = NS;
     for (int s = 0; s < ns; ++s) {
       const int cs = s * SB, ce = cs + SB;
       if (warp == NW - 1) {
@@ -293,6 +292,340 @@ struct DiagBlock {
     }
     if (t >= STORE0)
       for (int cs = (ns - 1) * SB; cs < NB; cs += SB) store_inv(cs);
+  }
+};
+
+// The 128 x 128 diagonal block in fp32, tile by tile: one warp per 32 x 32 tile of the factor's lower triangle (row block rb,
+// column block s) and of X = inv(L)^T (an identity carried along: X L^T = I), 20 in all.  A tile takes its entries less the
+// columns to its left (left-looking), then its own 32 columns four at a time: a tile on the diagonal eliminates them (the
+// serial chain), the others of the column block apply the 4 x 4 inverse C^-1 and the columns it published.  Everything
+// passes through shared memory by column (LT, XT: column k of L and X), groups of four columns signalled by one mbarrier per row
+// block and group, so a tile starts on what is there and no block barrier stands between one column block and the next.
+// Every entry receives its updates column by column in ascending order: the same bits as DiagBlock's.
+// What bounds it: the chain (about 600 cycles per four columns) and, beside it, the registers that shared memory delivers (one
+// per lane and cycle): the columns to the left are taken as 4 x 8 outer products per lane (12 loads for 32 multiply-adds; as
+// broadcasts, 33 for 32, the other tiles' work is twice as long as the chain).  Measured against DiagBlock at 128 columns: 24.6 ->
+// 18.8 us back to back, 30.5 -> 20.3 with cold caches, 27 -> 19 inside a factorisation.
+struct DiagTiles {
+  static constexpr int NB = 128, SB = 32, NS = NB / SB, GS = SB / 4, GROUPS = NB / 4;
+  static constexpr int P = NB + 4;                            // pitch: 16-byte rows, 16 bytes off a multiple of 128
+  static constexpr int TILES = NS * (NS + 1), THREADS = TILES * 32;
+  static constexpr size_t SMEM = ((size_t)2 * NB * P + GROUPS * 16) * sizeof(float) + 2 * NS * GROUPS * 8;
+
+  // Warp -> tile, as hex digits: X (1) or L (0), row block, column block.  Warps w, w + 4, ... share a scheduler: while a
+  // column block is eliminated, its tile on the diagonal, the next one and the tile between them have different ones, and
+  // the others' work is spread over what those leave.
+  static __device__ __forceinline__ int tile_of(int warp) {
+    constexpr int table[TILES] = {0x000, 0x011, 0x022, 0x033, 0x112, 0x032, 0x021, 0x010, 0x113, 0x100,
+                                  0x020, 0x031, 0x103, 0x133, 0x030, 0x101, 0x122, 0x123, 0x102, 0x111};
+    return table[warp];
+  }
+  // waits for a group's barrier, a bounded number of times
+  static __device__ __forceinline__ bool wait(uint32_t bar) {
+    for (int i = 0; i < (1 << 20); ++i) {
+      uint32_t ok;
+      asm volatile(
+          "{\n\t.reg .pred p;\n\t"
+          "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n\t"
+          "selp.u32 %0, 1, 0, p;\n\t}"
+          : "=r"(ok)
+          : "r"(bar)
+          : "memory");
+      if (ok) return true;
+    }
+    return false;
+  }
+  static __device__ __forceinline__ void arrive(uint32_t bar, int lane) {      // by lane 0
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.eq.s32 p, %1, 0;\n\t"
+        "@p mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];\n\t}" ::"r"(bar), "r"(lane)
+        : "memory");
+  }
+  // {a0, a1} += f * {x, y} in one packed instruction
+  static __device__ __forceinline__ void fma2(float& a0, float& a1, float f, float x, float y) {
+    asm("{\n\t.reg .b64 a, b, c;\n\t"
+        "mov.b64 a, {%2, %2};\n\tmov.b64 b, {%3, %4};\n\tmov.b64 c, {%0, %1};\n\t"
+        "fma.rn.f32x2 c, a, b, c;\n\tmov.b64 {%0, %1}, c;\n\t}"
+        : "+f"(a0), "+f"(a1)
+        : "f"(f), "f"(x), "f"(y));
+  }
+  static __device__ __forceinline__ float4 ld(const float* p) { return *reinterpret_cast<const float4*>(p); }
+  // a[c .. c + 3] += f * q
+  static __device__ __forceinline__ void axpy(float (&a)[SB], int c, float f, const float4& q) {
+    fma2(a[c], a[c + 1], f, q.x, q.y);
+    fma2(a[c + 2], a[c + 3], f, q.z, q.w);
+  }
+  // l = m C^-T for a row's entries m of four columns
+  static __device__ __forceinline__ void apply_ci(const float (&m)[4], const float* ci, float (&l)[4]) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      float v = 0.f;
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (q <= k) v = fmaf(m[q], ci[k * 4 + q], v);
+      l[k] = v;
+    }
+  }
+
+  // A: the nb x nb block (lower triangle; rows and columns beyond nb are those of an identity).  inv [NB, NB] receives inv(L),
+  // inv_t its transpose; both dense, zero outside their triangle.
+  static __device__ void run(const float* A, int64_t lda, int nb, float* inv, float* inv_t, int64_t row0, int32_t* status) {
+    extern __shared__ __align__(16) unsigned char diag_smem[];
+    float* LT = reinterpret_cast<float*>(diag_smem);          // LT[k][row]
+    float* XT = LT + NB * P;                                  // XT[k][row]
+    float* CI = XT + NB * P;                                  // C^-1 of every group, row-major
+    const uint32_t bars = (uint32_t)__cvta_generic_to_shared(CI + GROUPS * 16);
+    auto bar = [&](int row_block, int group) { return bars + 8u * (uint32_t)(row_block * GROUPS + group); };
+    const int t = threadIdx.x, lane = t & 31;
+    const int tl = tile_of(t >> 5);
+    const bool mat = (tl >> 8) == 0;
+    const int rb = (tl >> 4) & 15, s = tl & 15;
+    for (int b = t; b < 2 * NS * GROUPS; b += THREADS)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bars + 8u * b) : "memory");
+    __syncthreads();
+    // row blocks and column blocks beyond nb are those of an identity: nothing is eliminated there
+    const int ns = (nb + SB - 1) / SB;
+    const bool live = rb < ns && s < ns;
+    const int i = rb * SB + lane;                             // the lane's row
+    float* own = (mat ? LT : XT) + s * SB * P + rb * SB;      // the tile, [column][row]
+    const float* orow = (mat ? LT : XT) + rb * SB;            // its row block's columns
+    const float* Ls = LT + s * SB;                            // rows of L that belong to its columns
+    const int oid = mat ? rb : NS + rb;                       // row block of the barriers
+    const int first = mat ? 0 : rb;                           // first column block with entries in this row block
+    float a[SB];
+    if (mat) {
+      // whole rows in, turned in the tile's own place
+      const bool vec = lda % 4 == 0 && (reinterpret_cast<uintptr_t>(A) & 15u) == 0;
+      const int c = (lane & 7) * 4, j = s * SB + c;
+      float4 q[8];
+      const float* p = A + (int64_t)(rb * SB + (lane >> 3)) * lda + j;
+      if (vec && nb == NB) {                                  // (all loads in flight at once)
+#pragma unroll
+        for (int u = 0; u < 8; ++u) q[u] = ld(p + (int64_t)(4 * u) * lda);
+      } else {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int gi = rb * SB + u * 4 + (lane >> 3);
+          float v[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) v[e] = (gi < nb && j + e <= gi) ? p[(int64_t)(4 * u) * lda + e] : 0.f;
+          q[u] = make_float4(v[0], v[1], v[2], v[3]);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int gi = rb * SB + u * 4 + (lane >> 3);
+        float v[4] = {q[u].x, q[u].y, q[u].z, q[u].w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) v[e] = j + e > gi ? 0.f : (gi >= nb && j + e == gi) ? 1.f : v[e];
+        q[u] = make_float4(v[0], v[1], v[2], v[3]);
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) *reinterpret_cast<float4*>(own + (u * 4 + (lane >> 3)) * P + c) = q[u];
+      __syncwarp();
+      if (s == 0) {
+#pragma unroll
+        for (int e = 0; e < SB; e += 4) {
+          const float4 u = ld(own + lane * P + e);
+          a[e] = u.x; a[e + 1] = u.y; a[e + 2] = u.z; a[e + 3] = u.w;
+        }
+        __syncwarp();
+      }
+    } else {
+#pragma unroll
+      for (int c = 0; c < SB; ++c) a[c] = rb == s && c == lane ? 1.f : 0.f;
+      if (s > rb) {                                           // the zeros on the other side of the diagonal
+#pragma unroll 4
+        for (int c = 0; c < SB; ++c) {
+          inv[(rb * SB + c) * NB + s * SB + lane] = 0.f;
+          inv_t[(s * SB + c) * NB + rb * SB + lane] = 0.f;
+        }
+      }
+    }
+    bool ok = true;
+    if (live) {
+      if (s > first) {
+        // columns to the left; what the last column block waits for is not needed before the one in front of it is under
+        // way, and the first one's elimination has the schedulers to itself
+        if (s == NS - 1 || (!mat && s == NS - 2)) ok &= wait(bar(1, GS));
+        const int r0 = (lane >> 2) * 4, c0 = (lane & 3) * 8;  // four rows and eight columns per lane
+        float acc[4][8];
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int h = 0; h < 8; h += 4) {
+            const float4 u = mat ? ld(own + (r0 + r) * P + c0 + h) : make_float4(0.f, 0.f, 0.f, 0.f);
+            acc[r][h] = u.x; acc[r][h + 1] = u.y; acc[r][h + 2] = u.z; acc[r][h + 3] = u.w;
+          }
+        for (int g = first * GS; g < s * GS; ++g) {
+          if (oid != s) ok &= wait(bar(oid, g));
+          ok &= wait(bar(s, g));
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const float4 l = ld(orow + (g * 4 + k) * P + r0);
+            const float4 q0 = ld(Ls + (g * 4 + k) * P + c0), q1 = ld(Ls + (g * 4 + k) * P + c0 + 4);
+            const float nl[4] = {-l.x, -l.y, -l.z, -l.w};
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+              fma2(acc[r][0], acc[r][1], nl[r], q0.x, q0.y);
+              fma2(acc[r][2], acc[r][3], nl[r], q0.z, q0.w);
+              fma2(acc[r][4], acc[r][5], nl[r], q1.x, q1.y);
+              fma2(acc[r][6], acc[r][7], nl[r], q1.z, q1.w);
+            }
+          }
+        }
+        // one row per lane from here on
+        __syncwarp();
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+          *reinterpret_cast<float4*>(own + (c0 + c) * P + r0) = make_float4(acc[0][c], acc[1][c], acc[2][c], acc[3][c]);
+        __syncwarp();
+#pragma unroll
+        for (int c = 0; c < SB; ++c) a[c] = own[c * P + lane];
+        __syncwarp();
+      }
+      if (mat && rb == s) {
+        factor(a, own, CI + s * GS * 16, lane, row0 + s * SB, status, bar(s, s * GS));
+      } else {
+#pragma unroll
+        for (int g = 0; g < GS; ++g) {
+          const int j = 4 * g, gg = s * GS + g;
+          ok &= wait(bar(s, gg));
+          float ci[16], l[4];
+#pragma unroll
+          for (int q = 0; q < 16; q += 4) {
+            const float4 u = ld(CI + gg * 16 + q);
+            ci[q] = u.x; ci[q + 1] = u.y; ci[q + 2] = u.z; ci[q + 3] = u.w;
+          }
+          const float mine[4] = {a[j], a[j + 1], a[j + 2], a[j + 3]};
+          apply_ci(mine, ci, l);
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            a[j + k] = l[k];
+            own[(j + k) * P + lane] = l[k];
+          }
+          __syncwarp();
+          arrive(bar(oid, gg), lane);
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int c = j + 4; c < SB; c += 4) axpy(a, c, -l[k], ld(Ls + (s * SB + j + k) * P + c));
+        }
+      }
+    }
+    if (!mat) {
+#pragma unroll
+      for (int c = 0; c < SB; ++c) inv[(s * SB + c) * NB + i] = a[c];
+      if (live) {
+#pragma unroll
+        for (int r = 0; r < SB; r += 4) {
+          const float4 u = ld(own + lane * P + r);            // column s SB + lane, four rows
+          inv_t[(rb * SB + r) * NB + s * SB + lane] = u.x;
+          inv_t[(rb * SB + r + 1) * NB + s * SB + lane] = u.y;
+          inv_t[(rb * SB + r + 2) * NB + s * SB + lane] = u.z;
+          inv_t[(rb * SB + r + 3) * NB + s * SB + lane] = u.w;
+        }
+      } else {
+#pragma unroll 8
+        for (int r = 0; r < SB; ++r) inv_t[(rb * SB + r) * NB + s * SB + lane] = rb == s && r == lane ? 1.f : 0.f;
+      }
+    }
+    if (!ok && lane == 0) report_status(status, SP_ERR_TIMEOUT, (int32_t)row0, 12);
+  }
+
+  // Eliminates a 32 x 32 tile on the diagonal, one row per lane: own[k][row] = L below the 4 x 4 diagonal blocks, CI = their
+  // C^-1, one arrival per group of four columns.  Every lane has the group's 4 x 4 block: its entries before the previous
+  // group's update travel by shuffle while that group is worked on, and the update is repeated on them.
+  static __device__ __forceinline__ void factor(float (&a)[SB], float* own, float* CI, int lane, int64_t row0, int32_t* status,
+                                                uint32_t bar0) {
+    int bad = SB;
+    float m[4][4], nx[4][4], lp[4];
+    auto fetch = [&](int j) {                                 // rows and columns j .. j + 3 as they are now
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (q <= r) nx[r][q] = __shfl_sync(0xffffffffu, a[j + q], j + r);
+    };
+    fetch(0);
+#pragma unroll
+    for (int g = 0; g < GS; ++g) {
+      const int j = 4 * g;
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (q <= r) m[r][q] = nx[r][q];
+      if (g > 0) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float4 u = ld(own + (j - 4 + k) * P + j);
+          const float x[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+          for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+              if (q <= r) m[r][q] = fmaf(-x[r], x[q], m[r][q]);
+        }
+        // off the chain: the previous group's update of this row
+#pragma unroll
+        for (int c = j; c < SB; c += 4)
+#pragma unroll
+          for (int k = 0; k < 4; ++k) axpy(a, c, -lp[k], ld(own + (j - 4 + k) * P + c));
+      }
+      if (g + 1 < GS) fetch(j + 4);
+      float c[4][4], rd[4], ci[16];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        float p = m[k][k];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (q < k) p = fmaf(-c[k][q], c[k][q], p);
+        bad = (p > 0.f || bad < SB) ? bad : j + k;
+        const float r1 = recip_sqrt(p);
+        rd[k] = p > 0.f ? r1 : 1.f;
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+          if (r > k) {
+            float v = m[r][k];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+              if (q < k) v = fmaf(-c[r][q], c[k][q], v);
+            c[r][k] = v * rd[k];
+          }
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        ci[q * 4 + q] = rd[q];
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+          if (r > q) {
+            float v = 0.f;
+#pragma unroll
+            for (int z = 0; z < 4; ++z)
+              if (z >= q && z < r) v = fmaf(c[r][z], ci[z * 4 + q], v);
+            ci[r * 4 + q] = -v * rd[r];
+          } else if (r < q) {
+            ci[r * 4 + q] = 0.f;
+          }
+      }
+      const float mine[4] = {a[j], a[j + 1], a[j + 2], a[j + 3]};
+      apply_ci(mine, ci, lp);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (lane < j + 4) lp[k] = 0.f;
+        own[(j + k) * P + lane] = lp[k];
+      }
+      if (lane == 0) {
+#pragma unroll
+        for (int q = 0; q < 16; q += 4)
+          *reinterpret_cast<float4*>(CI + g * 16 + q) = make_float4(ci[q], ci[q + 1], ci[q + 2], ci[q + 3]);
+      }
+      __syncwarp();
+      arrive(bar0 + 8u * g, lane);
+    }
+    if (bad < SB && lane == 0) report_status(status, SP_ERR_NOT_SPD, (int32_t)(row0 + bad), 0);
   }
 };
 

@@ -19,7 +19,8 @@ namespace {
 
 constexpr int TB = kCholTcNB;          // 128
 
-using Diag = DiagBlock<float, TB>;
+using Diag = DiagTiles;
+static_assert(Diag::NB == TB, "one block");
 
 // Diagonal block: inv(L) and its transpose to dinv[0 : TB*TB] and dinv[TB*TB : 2*TB*TB].  L itself is not written back:
 // the solves use inv(L) of the diagonal blocks and the blocks of L below them only.
@@ -327,13 +328,21 @@ __device__ __forceinline__ void cluster_meet() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+// Where the rows of Lm go: they are the first rows of the panel of this block column, which therefore starts below them
+// and need not wait for this kernel.  (A21 has all 128 columns: only the last block of a matrix is narrower.)
+struct NextRows {
+  __nv_bfloat16* P;      // parts at P[i * ldp + part * seg + c]
+  int64_t ldp, seg;
+  int vec;               // 16-byte aligned rows of A21
+};
+
 // MODE 0: both stages in one launch, the CTAs being one cluster (they meet between the stages);
 // MODE 1 / MODE 2: the stages as two launches of 8 independent CTAs (for use beside persistent GEMM CTAs that hold
 // most SMs, where a cluster of 8 waits for a free group of SMs).
 template <int MODE>
-__device__ __forceinline__ void next_diag_body(const float* __restrict__ A21, const float* __restrict__ A22,
-                                               int64_t lda, int nb2, const float* __restrict__ dinv, float* LmT,
-                                               float* S, int32_t* status) {
+__device__ __forceinline__ void next_diag_body(float* A21, const float* __restrict__ A22, int64_t lda, int nb2,
+                                               const float* __restrict__ dinv, float* LmT, float* S, NextRows out_rows,
+                                               int32_t* status) {
   extern __shared__ __align__(128) float nm_smem[];
   using Tile = RowTile<NM_ROWS>;
   constexpr int AP = Tile::AP;
@@ -380,6 +389,26 @@ __device__ __forceinline__ void next_diag_body(const float* __restrict__ A21, co
     __syncthreads();   // everyone is done with At and Lt
     Tile::store(At, out);                          // own rows, left operand of stage 2
     Tile::store_transposed(LmT + i0, TB, out);     // for the other CTAs
+    // the panel's result for these rows: fp32 in place, bf16 parts
+#pragma unroll
+    for (int q = 0; q < Tile::RT; ++q) {
+      const int i = i0 + ir + q;
+      if (i >= nb2) continue;
+      const float v[4] = {out[q].x, out[q].y, out[q].z, out[q].w};
+      float* dst = A21 + (int64_t)i * lda + c0;
+      if (out_rows.vec) {
+        *reinterpret_cast<float4*>(dst) = out[q];
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) dst[j] = v[j];
+      }
+      __align__(8) __nv_bfloat16 part[3][4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) split3(v[j], part[0][j], part[1][j], part[2][j]);
+#pragma unroll
+      for (int z = 0; z < 3; ++z)
+        *reinterpret_cast<uint2*>(out_rows.P + i * out_rows.ldp + z * out_rows.seg + c0) = *reinterpret_cast<const uint2*>(part[z]);
+    }
     if (MODE == 1) return;
     cluster_meet();
   }
@@ -409,26 +438,26 @@ __device__ __forceinline__ void next_diag_body(const float* __restrict__ A21, co
 }
 
 __global__ void __cluster_dims__(NM_CTAS, 1, 1) __launch_bounds__(NM_THREADS)
-    chol_next_diag_kernel(const float* __restrict__ A21, const float* __restrict__ A22, int64_t lda, int nb2,
-                          const float* __restrict__ dinv, float* LmT, float* S, int32_t* status,
+    chol_next_diag_kernel(float* A21, const float* __restrict__ A22, int64_t lda, int nb2,
+                          const float* __restrict__ dinv, float* LmT, float* S, NextRows out_rows, int32_t* status,
                           const int32_t* skip) {
   kernel_begin();
   if (skip != nullptr && *skip != 0) return;
-  next_diag_body<0>(A21, A22, lda, nb2, dinv, LmT, S, status);
+  next_diag_body<0>(A21, A22, lda, nb2, dinv, LmT, S, out_rows, status);
 }
 __global__ void __launch_bounds__(NM_THREADS)
-    chol_next_diag_stage1_kernel(const float* __restrict__ A21, int64_t lda, int nb2, const float* __restrict__ dinv,
-                                 float* LmT, int32_t* status, const int32_t* skip) {
+    chol_next_diag_stage1_kernel(float* A21, int64_t lda, int nb2, const float* __restrict__ dinv, float* LmT,
+                                 NextRows out_rows, int32_t* status, const int32_t* skip) {
   kernel_begin();
   if (skip != nullptr && *skip != 0) return;
-  next_diag_body<1>(A21, nullptr, lda, nb2, dinv, LmT, nullptr, status);
+  next_diag_body<1>(A21, nullptr, lda, nb2, dinv, LmT, nullptr, out_rows, status);
 }
 __global__ void __launch_bounds__(NM_THREADS)
     chol_next_diag_stage2_kernel(const float* __restrict__ A22, int64_t lda, int nb2, float* LmT, float* S,
                                  const int32_t* skip) {
   kernel_begin();
   if (skip != nullptr && *skip != 0) return;
-  next_diag_body<2>(nullptr, A22, lda, nb2, nullptr, LmT, S, nullptr);
+  next_diag_body<2>(nullptr, A22, lda, nb2, nullptr, LmT, S, NextRows{}, nullptr);
 }
 
 constexpr int kPartA[6] = {0, 0, 1, 0, 2, 1};
@@ -467,9 +496,9 @@ sp_status potrf_lower_tc(float* A, int64_t n, int64_t lda, float* dinv, void* Pv
   float* LmT = S + TB * TB;                  // [128, 128] scratch of the lookahead kernel
   bool rec[2] = {false, false};
   // Far part of a step's trailing update on a stream of its own: it adds into the matrix through the GEMM's atomic TMA
-  // reduction (which needs 16-byte aligned rows and a width that is a multiple of 4), so it commutes with the near
-  // update of the next step, which touches one of its block columns.  What must see it complete waits for its event:
-  // the lookahead kernel of step kb reads block (kb+1, kb+1), last touched by the far update of step kb - 2.
+  // reduction (which needs 16-byte aligned rows and a width that is a multiple of 4).  What must see it complete waits for its
+  // events: the lookahead kernel of step kb reads block (kb+1, kb+1), last touched by the far update of step kb - 2, and
+  // the near update of step kb adds to a block column that the far update of step kb - 1 has among its first two.
   // The far GEMM leaves a few SM pairs to the kernels of the chain, which would otherwise wait for its tiles to end.
   const bool far_apart = assist && assist->far_stream && n % 4 == 0 && lda % 4 == 0 &&
                          (reinterpret_cast<uintptr_t>(A) & 15u) == 0 && !reproducible_mode();
@@ -515,39 +544,47 @@ sp_status potrf_lower_tc(float* A, int64_t n, int64_t lda, float* dinv, void* Pv
       for (int q = 0; q < 2; ++q)
         if (far_rec[q]) SP_CUDA_OK(cudaStreamWaitEvent(stream, assist->far_done[q], 0));
     }
+    // rows of the panel that the lookahead kernel takes: the next diagonal block's
+    const int64_t ahead = assist && rem > 0 && !inner_last ? (rem < TB ? rem : TB) : 0;
     if (assist && rem > 0) {
-      if (!inner_last) {
+      // the panel needs the diagonal block alone (its rows are disjoint from those of the lookahead kernel)
+      SP_CUDA_OK(cudaEventRecord(assist->panel_done, stream));
+      sb = assist->stream;
+      SP_CUDA_OK(cudaStreamWaitEvent(sb, assist->panel_done, 0));
+      if (ahead > 0) {
         // next diagonal block: it reads blocks (kb+1, kb) and (kb+1, kb+1), i.e. the first two block columns of the
         // trailing update of step kb - 1, which that step issues first and signals on their own
         if (kb >= 1) SP_CUDA_OK(cudaStreamWaitEvent(stream, assist->near_done, 0));
         if (far_rec[kb & 1]) SP_CUDA_OK(cudaStreamWaitEvent(stream, assist->far_done[kb & 1], 0));   // far update of step kb - 2
-        const int nb2 = (int)(rem < TB ? rem : TB);
+        const int nb2 = (int)ahead;
+        float* A21 = A + (k0 + nb) * lda + k0;
+        const NextRows rows{P + (k0 + nb) * ldp + k0, ldp, np, lda % 4 == 0 && (reinterpret_cast<uintptr_t>(A) & 15u) == 0};
         count_launch();
         ProfScope prof(PK_PANEL_APPLY, 4.0 * TB * TB * TB, 0.0, stream);
         if (!split_lookahead) {
-          launch(chol_next_diag_kernel, NM_CTAS, NM_THREADS, NM_SMEM, stream, A + (k0 + nb) * lda + k0,
-                                                                          A + (k0 + nb) * lda + (k0 + nb), lda, nb2,
-                                                                          dk, LmT, S, status_dev, skip);
+          launch(chol_next_diag_kernel, NM_CTAS, NM_THREADS, NM_SMEM, stream, A21, A21 + nb, lda, nb2, dk, LmT, S, rows,
+                 status_dev, skip);
         } else {
-          launch(chol_next_diag_stage1_kernel, NM_CTAS, NM_THREADS, NM_SMEM, stream, A + (k0 + nb) * lda + k0, lda, nb2, dk,
-                                                                                 LmT, status_dev, skip);
+          launch(chol_next_diag_stage1_kernel, NM_CTAS, NM_THREADS, NM_SMEM, stream, A21, lda, nb2, dk, LmT, rows,
+                 status_dev, skip);
           count_launch();
-          launch(chol_next_diag_stage2_kernel, NM_CTAS, NM_THREADS, NM_SMEM, stream, A + (k0 + nb) * lda + (k0 + nb), lda,
-                                                                                 nb2, LmT, S, skip);
+          launch(chol_next_diag_stage2_kernel, NM_CTAS, NM_THREADS, NM_SMEM, stream, A21 + nb, lda, nb2, LmT, S, skip);
         }
         if (cudaGetLastError() != cudaSuccess) return SP_ERR_CUDA;
+        SP_CUDA_OK(cudaEventRecord(assist->next_done, stream));
       }
-      // the panel overwrites A21 in place: it starts behind the lookahead kernel
-      SP_CUDA_OK(cudaEventRecord(assist->panel_done, stream));
-      sb = assist->stream;
-      SP_CUDA_OK(cudaStreamWaitEvent(sb, assist->panel_done, 0));
     }
     // L21 = A21 inv(L11)^T, fp32 in place and as bf16 parts in P[k0+nb.., part * np + k0 ..]
-    if (launch_panel_apply<false>(A + (k0 + nb) * lda + k0, lda, prow, nb, dk, P + (k0 + nb) * ldp + k0, ldp, np, true,
+    const int64_t p0 = k0 + nb + ahead;
+    if (launch_panel_apply<false>(A + p0 * lda + k0, lda, prow - ahead, nb, dk, P + p0 * ldp + k0, ldp, np, true,
                                   status_dev, sb) != cudaSuccess)
       return SP_ERR_CUDA;
     if (rem <= 0) break;     // last block: the appended rows are done, nothing is left to update
     if (far_apart && !outer && rem > 2 * TB) SP_CUDA_OK(cudaEventRecord(assist->far_go, sb));   // the panel's parts exist
+    if (ahead > 0) SP_CUDA_OK(cudaStreamWaitEvent(sb, assist->next_done, 0));    // so do the rows of the lookahead kernel
+    // the far update of the step before has added to the columns that this step's near update adds to: every entry receives
+    // its updates in step order, whatever the streams' timing
+    if (kb >= 1 && far_rec[(kb - 1) & 1]) SP_CUDA_OK(cudaStreamWaitEvent(sb, assist->far_first, 0));
     // A22 -= L21 L21^T on the lower triangle
     TcOperand ta{P + (k0 + nb) * ldp, ldp, true}, tb{P + (k0 + nb) * ldp, ldp, true};
     ta.kext = tb.kext = ldp;
@@ -614,21 +651,28 @@ sp_status potrf_lower_tc(float* A, int64_t n, int64_t lda, float* dinv, void* Pv
                              (2.0 * (double)prow * (double)kNear - (double)kNear * (double)kNear) * (double)nb);
       if (st != SP_OK) return st;
       SP_CUDA_OK(cudaEventRecord(assist->near_done, sb));
-      TcOperand fa{P + (k0 + nb + kNear) * ldp, ldp, true}, fb{P + (k0 + nb + kNear) * ldp, ldp, true};
-      fa.kext = fb.kext = ldp;
-      fa.mnext = prow - kNear;
-      fb.mnext = rem - kNear;
-      float* Afar = A22 + kNear * lda + kNear;
-      const double fr = (double)(rem - kNear);
       cudaStream_t sf = sb;
       if (far_apart) {
         sf = assist->far_stream;
         SP_CUDA_OK(cudaStreamWaitEvent(sf, assist->far_go, 0));
       }
-      st = gemm_tc(prow - kNear, rem - kNear, TB, -1.f, fa, fb, 1.f, Operand{Afar, SP_F32, lda, 1},
-                   OutOperand{Afar, SP_F32, lda}, true, status_dev, sf, &sg,
-                   (fr * fr + 2.0 * (double)m_extra * fr) * (double)nb, far_apart ? kFarPairs : 0);
-      if (st != SP_OK) return st;
+      // (first the two block columns that the next step waits for, where the whole takes more than two rounds of tiles)
+      const int64_t fw = rem - kNear;
+      const int64_t cut = far_apart && fw > kNear &&
+                                  ceil_div(fw, (int64_t)256) * ceil_div(prow - kNear, (int64_t)256) > 4 * kFarPairs ? kNear : fw;
+      for (int64_t c0 = 0; c0 < fw; c0 = c0 == 0 ? cut : fw) {
+        const int64_t w = c0 == 0 ? cut : fw - c0, r0 = k0 + nb + kNear + c0, rows_f = prow - kNear - c0;
+        TcOperand fa{P + r0 * ldp, ldp, true}, fb{P + r0 * ldp, ldp, true};
+        fa.kext = fb.kext = ldp;
+        fa.mnext = rows_f;
+        fb.mnext = w;
+        float* Afar = A + r0 * lda + r0;
+        st = gemm_tc(rows_f, w, TB, -1.f, fa, fb, 1.f, Operand{Afar, SP_F32, lda, 1}, OutOperand{Afar, SP_F32, lda}, true,
+                     status_dev, sf, &sg, (double)w * (2.0 * (double)rows_f - (double)w) * (double)nb,
+                     far_apart ? kFarPairs : 0);
+        if (st != SP_OK) return st;
+        if (far_apart && c0 == 0) SP_CUDA_OK(cudaEventRecord(assist->far_first, sf));
+      }
       if (far_apart) {
         SP_CUDA_OK(cudaEventRecord(assist->far_done[kb & 1], sf));
         far_rec[kb & 1] = true;
