@@ -320,9 +320,9 @@ struct DiagTiles {
                                   0x020, 0x031, 0x103, 0x133, 0x030, 0x101, 0x122, 0x123, 0x102, 0x111};
     return table[warp];
   }
-  // waits for a group's barrier, a bounded number of times
+  // waits for a group's barrier, about a second at most
   static __device__ __forceinline__ bool wait(uint32_t bar) {
-    for (int i = 0; i < (1 << 20); ++i) {
+    const auto done = [&] {
       uint32_t ok;
       asm volatile(
           "{\n\t.reg .pred p;\n\t"
@@ -331,8 +331,12 @@ struct DiagTiles {
           : "=r"(ok)
           : "r"(bar)
           : "memory");
-      if (ok) return true;
-    }
+      return ok != 0;
+    };
+    if (done()) return true;
+    const long long t0 = clock64();
+    while (clock64() - t0 < 2000000000ll)
+      if (done()) return true;
     return false;
   }
   static __device__ __forceinline__ void arrive(uint32_t bar, int lane) {      // by lane 0
@@ -448,7 +452,7 @@ struct DiagTiles {
       if (s > first) {
         // columns to the left; what the last column block waits for is not needed before the one in front of it is under
         // way, and the first one's elimination has the schedulers to itself
-        if (s == NS - 1 || (!mat && s == NS - 2)) ok &= wait(bar(1, GS));
+        if (s == NS - 1 || (!mat && s == NS - 2)) ok = ok && wait(bar(1, GS));
         const int r0 = (lane >> 2) * 4, c0 = (lane & 3) * 8;  // four rows and eight columns per lane
         float acc[4][8];
 #pragma unroll
@@ -459,8 +463,8 @@ struct DiagTiles {
             acc[r][h] = u.x; acc[r][h + 1] = u.y; acc[r][h + 2] = u.z; acc[r][h + 3] = u.w;
           }
         for (int g = first * GS; g < s * GS; ++g) {
-          if (oid != s) ok &= wait(bar(oid, g));
-          ok &= wait(bar(s, g));
+          if (oid != s) ok = ok && wait(bar(oid, g));
+          ok = ok && wait(bar(s, g));
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
             const float4 l = ld(orow + (g * 4 + k) * P + r0);
@@ -491,7 +495,7 @@ struct DiagTiles {
 #pragma unroll
         for (int g = 0; g < GS; ++g) {
           const int j = 4 * g, gg = s * GS + g;
-          ok &= wait(bar(s, gg));
+          ok = ok && wait(bar(s, gg));
           float ci[16], l[4];
 #pragma unroll
           for (int q = 0; q < 16; q += 4) {
