@@ -228,17 +228,27 @@ struct DiagBlock {
     constexpr int NW = THREADS / 32;
     // load: one warp per row and 32 V columns, 16 bytes per lane where the rows allow it
     const bool vec = lda % V == 0 && (reinterpret_cast<uintptr_t>(A) & 15u) == 0;
-    constexpr int VPR = NB / V;
+    constexpr int VPR = NB / V, CNT = NB * VPR / THREADS;
+    static_assert(NB * VPR % THREADS == 0, "block / thread mismatch");
+    Vec in[CNT];
+    if (vec && nb == NB) {                                   // (all loads in flight at once; behind a test each they take turns)
 #pragma unroll
-    for (int e = t; e < NB * VPR; e += THREADS) {
-      const int i = e / VPR, c = (e % VPR) * V;
-      Vec q;
-      if (vec && i < nb && c + V <= nb) {
-        q = *reinterpret_cast<const Vec*>(A + (int64_t)i * lda + c);
-      } else {
-#pragma unroll
-        for (int v = 0; v < V; ++v) q.v[v] = (i < nb && c + v <= i) ? A[(int64_t)i * lda + c + v] : (T)0;
+      for (int u = 0; u < CNT; ++u) {
+        const int e = t + u * THREADS;
+        in[u] = *reinterpret_cast<const Vec*>(A + (int64_t)(e / VPR) * lda + (e % VPR) * V);
       }
+    } else {
+#pragma unroll
+      for (int u = 0; u < CNT; ++u) {
+        const int e = t + u * THREADS, i = e / VPR, c = (e % VPR) * V;
+#pragma unroll
+        for (int v = 0; v < V; ++v) in[u].v[v] = (i < nb && c + v <= i) ? A[(int64_t)i * lda + c + v] : (T)0;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < CNT; ++u) {
+      const int e = t + u * THREADS, i = e / VPR, c = (e % VPR) * V;
+      Vec q = in[u];
 #pragma unroll
       for (int v = 0; v < V; ++v) q.v[v] = c + v > i ? (T)0 : (i >= nb && c + v == i) ? (T)1 : q.v[v];
       *reinterpret_cast<Vec*>(M + i * P + c) = q;

@@ -1019,8 +1019,9 @@ sp_status gemm_tc(int64_t M, int64_t N, int64_t K, float alpha, TcOperand A, TcO
     if (best > 1 && p.epi_mode == EPI_TMA_STORE && p.skip != nullptr) best = 1;   // no unconditional clear of C
     if (best > 1) {
       if (p.epi_mode == EPI_TMA_STORE) {
-        if (cudaMemset2DAsync(C.ptr, (size_t)C.ld * 4, 0, (size_t)N * 4, (size_t)M, stream) != cudaSuccess)
-          return SP_ERR_CUDA;
+        const cudaError_t e = C.ld == N ? cudaMemsetAsync(C.ptr, 0, (size_t)M * N * 4, stream)
+                                        : cudaMemset2DAsync(C.ptr, (size_t)C.ld * 4, 0, (size_t)N * 4, (size_t)M, stream);
+        if (e != cudaSuccess) return SP_ERR_CUDA;
         p.epi_mode = EPI_TMA_ADD;
       }
       p.ksplit = best;
