@@ -29,9 +29,7 @@
  *     panels and trailing updates of a factorisation, the z^(1) products) onto a few streams and events that the
  *     library creates once per device and joins back to the caller's stream with events before the call's results are
  *     used (also when a call returns an error after the fork).  That set is shared by all these calls on a device: issue
- *     them from one host thread at a time.  sp_mha_step forks the system of Eq. (86) onto a second such set where no other
- *     host thread's call and no stream capture but the caller's own holds it, and stays on the caller's stream otherwise.
- *     All other calls, sp_ffn_cache_input_inverse and the precise solves among
+ *     them from one host thread at a time.  All other calls, sp_ffn_cache_input_inverse and the precise solves among
  *     them, use the caller's stream alone.  Nothing else persists inside the library.
  *   - Reproducibility: by default a product whose tile count leaves SMs idle is cut along K and its partial
  *     products add up in C in an order that is not fixed, and a backward sweep with more right-hand sides than one wave of its

@@ -200,41 +200,34 @@ struct SideStream {
   cudaEvent_t fork = nullptr, join = nullptr, z1_done = nullptr;
   SolveAssist assist_main{}, assist_side{};   // helpers of the solves on the caller's stream / on `stream`
 };
-bool make_assist(SolveAssist& a, int prio) {
-  return cudaStreamCreateWithPriority(&a.stream, cudaStreamNonBlocking, prio) == cudaSuccess &&
+bool make_assist(SolveAssist& a) {
+  return cudaStreamCreateWithFlags(&a.stream, cudaStreamNonBlocking) == cudaSuccess &&
          cudaEventCreateWithFlags(&a.panel_done, cudaEventDisableTiming) == cudaSuccess &&
          cudaEventCreateWithFlags(&a.rest_done[0], cudaEventDisableTiming) == cudaSuccess &&
          cudaEventCreateWithFlags(&a.rest_done[1], cudaEventDisableTiming) == cudaSuccess &&
          cudaEventCreateWithFlags(&a.near_done, cudaEventDisableTiming) == cudaSuccess &&
          cudaEventCreateWithFlags(&a.next_done, cudaEventDisableTiming) == cudaSuccess &&
-         cudaStreamCreateWithPriority(&a.far_stream, cudaStreamNonBlocking, prio) == cudaSuccess &&
+         cudaStreamCreateWithFlags(&a.far_stream, cudaStreamNonBlocking) == cudaSuccess &&
          cudaEventCreateWithFlags(&a.far_go, cudaEventDisableTiming) == cudaSuccess &&
          cudaEventCreateWithFlags(&a.far_first, cudaEventDisableTiming) == cudaSuccess &&
          cudaEventCreateWithFlags(&a.far_done[0], cudaEventDisableTiming) == cudaSuccess &&
          cudaEventCreateWithFlags(&a.far_done[1], cudaEventDisableTiming) == cudaSuccess;
 }
-constexpr int kMaxSideDevices = 64;
-SideStream* side_stream(int set = 0) {
-  static SideStream tables[2][kMaxSideDevices];
-  static bool failures[2][kMaxSideDevices] = {};
+SideStream* side_stream() {
+  static SideStream table[64];
+  static bool failed[64] = {};
   static std::mutex mu;
   int dev = -1;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxSideDevices) return nullptr;
-  SideStream* table = tables[set];
-  bool* failed = failures[set];
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
   std::lock_guard<std::mutex> guard(mu);
   if (failed[dev]) return nullptr;
   SideStream& ss = table[dev];
   if (!ss.stream) {
-    // the second set carries chains of short kernels beside kernels that fill the GPU: its blocks go first
-    int least = 0, greatest = 0;
-    cudaDeviceGetStreamPriorityRange(&least, &greatest);
-    const int prio = set == 1 ? greatest : 0;
-    if (cudaStreamCreateWithPriority(&ss.stream, cudaStreamNonBlocking, prio) != cudaSuccess ||
+    if (cudaStreamCreateWithFlags(&ss.stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&ss.fork, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&ss.join, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&ss.z1_done, cudaEventDisableTiming) != cudaSuccess ||
-        !make_assist(ss.assist_main, prio) || !make_assist(ss.assist_side, prio)) {
+        !make_assist(ss.assist_main) || !make_assist(ss.assist_side)) {
       failed[dev] = true;
       ss.stream = nullptr;
       return nullptr;
@@ -242,38 +235,6 @@ SideStream* side_stream(int set = 0) {
   }
   return &ss;
 }
-
-// A second set of streams for calls that are not tied to one host thread at a time: held for the duration of the call, and
-// only taken when no other call holds it and no stream capture other than the caller's own has it.  Without it the call
-// stays on the caller's stream.
-class SideLease {
- public:
-  explicit SideLease(cudaStream_t s) {
-    static std::mutex held[kMaxSideDevices];
-    int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxSideDevices) return;
-    std::unique_lock<std::mutex> lock(held[dev], std::try_to_lock);
-    if (!lock.owns_lock()) return;
-    SideStream* set = side_stream(1);
-    if (set == nullptr) return;
-    cudaStreamCaptureStatus mine = cudaStreamCaptureStatusNone;
-    unsigned long long my_id = 0;
-    if (cudaStreamGetCaptureInfo(s, &mine, &my_id) != cudaSuccess || mine == cudaStreamCaptureStatusInvalidated) return;
-    for (cudaStream_t q : {set->stream, set->assist_side.stream, set->assist_side.far_stream}) {
-      cudaStreamCaptureStatus its = cudaStreamCaptureStatusNone;
-      unsigned long long its_id = 0;
-      if (cudaStreamGetCaptureInfo(q, &its, &its_id) != cudaSuccess) return;
-      if (its != cudaStreamCaptureStatusNone && (mine == cudaStreamCaptureStatusNone || its_id != my_id)) return;
-    }
-    lock_ = std::move(lock);
-    side_ = set;
-  }
-  SideStream* get() const { return side_; }
-
- private:
-  std::unique_lock<std::mutex> lock_;
-  SideStream* side_ = nullptr;
-};
 
 // Makes the caller's stream wait for everything queued on the library's
 // streams when a call returns early (an error between a fork and its join), so that no library work is ever left
@@ -539,7 +500,7 @@ sp_status sp_ridge_solve(const float* R, int64_t ldr, const float* G, int64_t ld
   if (!ws || ws_bytes < ridge_ws_bytes(m, n, precise != 0)) return SP_ERR_WORKSPACE;
   if (misaligned(ws, 256)) return SP_ERR_ALIGNMENT;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  const OverlapScope overlap(n <= kOverlapMaxN);
+  const OverlapScope overlap(n <= kOverlapMaxSolve);
   Carver c(ws);
   SolveBufs b = carve_solve(c, n, m, precise ? 8 : 4);
   CU(effective_ridge(G, ldg, n, rho, rho_relative, b.rho, s));
@@ -567,7 +528,7 @@ sp_status sp_linear_refit(const float* R, int64_t ldr, const float* G, int64_t l
   if (!ws || ws_bytes < need) return SP_ERR_WORKSPACE;
   if (misaligned(ws, 256)) return SP_ERR_ALIGNMENT;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  const OverlapScope overlap(n <= kOverlapMaxN);
+  const OverlapScope overlap(n <= kOverlapMaxSolve);
   Carver c(ws);
   SolveBufs b = carve_solve(c, n, m, precise ? 8 : 4);
   int32_t* unit_idx = c.take<int32_t>((size_t)n_units);
@@ -1507,35 +1468,21 @@ static sp_status mha_impl(const sp_mha_module* m, sp_mha_state* st, const sp_mha
     CU(split_bf16(reinterpret_cast<const float*>(m->Wv.ptr), d, nullptr, d, d, dp, p.Wvs, s));
     if (init) CU(split_bf16(reinterpret_cast<const float*>(m->Wo.ptr), d, nullptr, d, d, dp, p.Wos, s));
   }
-  // The system of Eq. (86) needs W_O alone and its result is first used after the gradient steps of Eq. (85): where the
-  // library's second set of streams is free, its chain of short kernels runs beside those.
-  const SideLease lease(init ? nullptr : s);
-  SideStream* side = init ? nullptr : lease.get();
-  JoinOnExit join_guard{side, s};
   if (!init) {
-    cudaStream_t sw = s;
-    const SolveAssist* assist = nullptr;
-    if (side) {
-      CU(cudaEventRecord(side->fork, s));
-      CU(cudaStreamWaitEvent(side->stream, side->fork, 0));
-      sw = side->stream;
-      if (bf16) assist = &side->assist_side;
-    }
     // Eq. (86): a_attn = (W_O^T W_O + I)^-1 (W_O^T ypre + heads); token-major: A_attn = Ypre M1 + Hd Cinv with
     // [M1; Cinv] = [W_O; I] (W_O^T W_O + I)^-1, one regularised solve with 2 d right-hand sides
     MatRef wo{m->Wo.ptr, SP_F32, d}, cf{p.Cf, SP_F32, d};
-    SPCHK(contract(d, d, d, 1.0, wo, false, wo, false, 0.0, cf, cf, true, true, false, status_dev, sw));
-    CU(symmetrize_lower(p.Cf, d, d, sw));
-    CU(cudaMemcpyAsync(p.RW, m->Wo.ptr, (size_t)d * d * sizeof(float), cudaMemcpyDeviceToDevice, sw));
-    CU(set_identity(p.RW + (size_t)d * d, d, d, sw));
-    CU(effective_ridge(nullptr, 0, 1, 1.0, 0, p.sb.rho, sw));
-    if (bf16) SPCHK(ridge_core<float>(p.RW, d, p.Cf, d, 2 * d, d, nullptr, d, p.sb.rho, p.MC, d, p.sb, status_dev, sw, assist));
-    else SPCHK(ridge_core<double>(p.RW, d, p.Cf, d, 2 * d, d, nullptr, d, p.sb.rho, p.MC, d, p.sb, status_dev, sw));
+    SPCHK(contract(d, d, d, 1.0, wo, false, wo, false, 0.0, cf, cf, true, true, false, status_dev, s));
+    CU(symmetrize_lower(p.Cf, d, d, s));
+    CU(cudaMemcpyAsync(p.RW, m->Wo.ptr, (size_t)d * d * sizeof(float), cudaMemcpyDeviceToDevice, s));
+    CU(set_identity(p.RW + (size_t)d * d, d, d, s));
+    CU(effective_ridge(nullptr, 0, 1, 1.0, 0, p.sb.rho, s));
+    if (bf16) SPCHK(ridge_core<float>(p.RW, d, p.Cf, d, 2 * d, d, nullptr, d, p.sb.rho, p.MC, d, p.sb, status_dev, s));
+    else SPCHK(ridge_core<double>(p.RW, d, p.Cf, d, 2 * d, d, nullptr, d, p.sb.rho, p.MC, d, p.sb, status_dev, s));
     if (bf16) {
-      CU(split_bf16(p.MC, d, nullptr, d, d, dp, p.M1s, sw));
-      CU(split_bf16(p.MC + (size_t)d * d, d, nullptr, d, d, dp, p.Cis, sw));
+      CU(split_bf16(p.MC, d, nullptr, d, d, dp, p.M1s, s));
+      CU(split_bf16(p.MC + (size_t)d * d, d, nullptr, d, d, dp, p.Cis, s));
     }
-    if (side) CU(cudaEventRecord(side->z1_done, side->stream));
   }
 
   for (int64_t q0 = 0; q0 < n_seq; q0 += p.sc) {
@@ -1617,7 +1564,6 @@ static sp_status mha_impl(const sp_mha_module* m, sp_mha_state* st, const sp_mha
     }
     // ---- Eq. (86): head outputs Hd = P V, then A_attn = Ypre M1 + Hd Cinv
     {
-      if (side && q0 == 0) CU(cudaStreamWaitEvent(s, side->z1_done, 0));
       BMat hv = bf16 ? tokv(p.Hd, SP_BF16, 2 * dp, 1, 0) : tokv(p.Hd, SP_F32, d, 1, 0);
       SPCHK(bcontract(T, dh, T, 1.0, Pop, true, Vv, false, bf16 ? 3 : 1, kSeg3A, kSeg3B, 0.0, none, hv, bf16 ? dp : 0,
                       nb0, nb1, status_dev, s));
@@ -1669,7 +1615,6 @@ static sp_status mha_impl(const sp_mha_module* m, sp_mha_state* st, const sp_mha
     CU(symmetrize_lower(st->G_X, d, d, s));
     CU(symmetrize_lower(st->G_attn, d, d, s));
   }
-  join_guard.armed = false;
   return SP_OK;
 }
 

@@ -105,7 +105,8 @@ struct OverlapScope {
   ~OverlapScope() { overlap_flag() = saved; }
   OverlapScope(const OverlapScope&) = delete;
 };
-constexpr int64_t kOverlapMaxN = 4608;        // widest system whose solve is launches and gaps for the most part
+constexpr int64_t kOverlapMaxN = 4608;        // widest module whose step is launches and gaps for the most part
+constexpr int64_t kOverlapMaxSolve = 1024;    // the same for a solve of its own
 inline bool may_overlap_launches(cudaStream_t stream) {
   if (!overlap_flag()) return false;
   cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
