@@ -302,8 +302,7 @@ gemm_dmma_kernel(int64_t M, int64_t N, int64_t K, double alpha, const T* A, int6
 // Products of at most 64 values of K with 16-byte aligned fp64 operands: the panels and the next block column's updates of the fp64
 // factorisation and sweeps, links of its chain.  What bounds them is latency, so all of A, B (asynchronous copies) and C (registers)
 // is on its way at once; the form above fetches 16 values of K at a time, each a round trip to memory.  Same instructions in
-// the same order over K: the same bits.  Panels and near updates 6.9 -> 5-6 us, a fp32-mode layer 768 wide 16.18 -> 15.34 ms together
-// with the diagonal blocks' loads.
+// the same order over K: the same bits.  A fp32-mode layer 768 wide: 16.18 -> 15.34 ms together with the diagonal blocks' loads.
 template <bool A_KFAST, bool B_KFAST, int BM>
 struct DmmaShort {
   static constexpr int KMAX = 64, FA = A_KFAST ? KMAX : BM, OA = A_KFAST ? BM : KMAX, FB = B_KFAST ? KMAX : DM_BN,
