@@ -114,11 +114,9 @@ struct SolveBufs {
   double* rho;  // [4] device scalars
   void* P;      // fp32 path: bf16 parts of the Cholesky factor
   void* Xs;     // fp32 path: bf16 parts of one block column of right-hand sides
-  float* scale; // two-part form: scale of the system's rows and columns, row factors of the right-hand sides
-  float* rowf;
 };
 
-SolveBufs carve_solve(Carver& c, int64_t nmax, int64_t mmax, size_t tsize, bool two_part = false) {
+SolveBufs carve_solve(Carver& c, int64_t nmax, int64_t mmax, size_t tsize) {
   SolveBufs b;
   b.rho = c.take<double>(4);
   b.idx = c.take<int32_t>((size_t)nmax);
@@ -127,16 +125,11 @@ SolveBufs carve_solve(Carver& c, int64_t nmax, int64_t mmax, size_t tsize, bool 
   b.dinv = c.take_bytes(dinv_elems(nmax) * tsize);
   b.P = nullptr;
   b.Xs = nullptr;
-  b.scale = b.rowf = nullptr;
   if (tsize == 4) {
     const size_t np = (size_t)chol_tc_pad(nmax);
     b.P = c.take_bytes((np + (size_t)mmax) * 3 * np * 2);
     const size_t rows = (size_t)(nmax > mmax ? nmax : mmax);   // either dimension may be the right-hand-side count
     b.Xs = c.take_bytes((size_t)chol_tc_xs_elems(nmax, (int64_t)rows) * 2);
-    if (two_part) {
-      b.scale = c.take<float>((size_t)nmax);
-      b.rowf = c.take<float>((size_t)std::max(half_rowf_elems(nmax, mmax), half_rowf_elems(mmax, nmax)));
-    }
   }
   return b;
 }
@@ -154,34 +147,27 @@ template <typename T>
 sp_status ridge_core(const float* R, int64_t ldr, const float* G, int64_t ldg, int64_t m, int64_t n_full,
                      const int32_t* idx, int64_t k, const double* rho_dev, float* W, int64_t ldw, SolveBufs& b,
                      int32_t* status, cudaStream_t stream, const SolveAssist* assist = nullptr,
-                     bool split_lookahead = false, const LeadSave* save = nullptr, bool conditional = false,
-                     bool two_part = false) {
+                     bool split_lookahead = false, const LeadSave* save = nullptr, bool conditional = false) {
   const int64_t nn = idx ? k : n_full;
   ProfScope prof(PK_SOLVE, conditional ? 0.0 : (double)nn * nn * nn / 3.0 + 2.0 * (double)m * nn * nn, 0.0, stream);
   T* Gs = reinterpret_cast<T*>(b.Gs);
   T* dinv = reinterpret_cast<T*>(b.dinv);
   T* Rs = Gs + (size_t)nn * nn;     // the right-hand sides sit right below the system matrix, same leading dimension
-  const float* scale = nullptr;
-  if (two_part && b.scale != nullptr) {
-    CU(system_scale(G, ldg, idx, nn, rho_dev, b.scale, stream));
-    scale = b.scale;
-  }
-  if (idx || scale) CU(load_spd_gather<T>(G, ldg, idx, nn, rho_dev, Gs, nn, stream, scale));
+  if (idx) CU(load_spd_gather<T>(G, ldg, idx, nn, rho_dev, Gs, nn, stream));
   else CU(load_spd<T>(G, ldg, nn, rho_dev, Gs, nn, stream));
   if constexpr (sizeof(T) == 4) {
     // the right-hand sides ride through the factorisation as m more rows (their forward substitution); the solve
     // proper is then only the backward sweep
-    const HalfParts half{scale ? b.rowf : nullptr};
-    CU(gather_cols<T>(R, ldr, idx, m, nn, Rs, nn, stream, scale));
-    SPCHK(potrf_lower_tc(Gs, nn, nn, dinv, b.P, status, stream, assist, m, split_lookahead, half));
+    CU(gather_cols<T>(R, ldr, idx, m, nn, Rs, nn, stream));
+    SPCHK(potrf_lower_tc(Gs, nn, nn, dinv, b.P, status, stream, assist, m, split_lookahead));
     if (save) CU(copy_cols_padded(Rs, nn, m, save->k, save->kpad, save->Y, stream));
-    SPCHK(potrs_right_tc(Rs, m, nn, nn, b.P, dinv, b.Xs, status, stream, assist, true, Gs, nn, 0, half));
+    SPCHK(potrs_right_tc(Rs, m, nn, nn, b.P, dinv, b.Xs, status, stream, assist, true, Gs, nn));
   } else {
     CU(gather_cols<T>(R, ldr, idx, m, nn, Rs, nn, stream));
     CU(potrf_lower_f64(Gs, nn, nn, dinv, status, stream, assist, m));
     CU(potrs_backward_f64(Rs, m, nn, nn, Gs, nn, dinv, stream, assist));
   }
-  CU(scatter_cols<T>(Rs, nn, idx, m, nn, n_full, W, ldw, stream, scale));
+  CU(scatter_cols<T>(Rs, nn, idx, m, nn, n_full, W, ldw, stream));
   return SP_OK;
 }
 
@@ -297,7 +283,7 @@ AdmmPlan plan_admm(void* ws, int64_t d, int64_t n, int64_t N, int64_t chunk, int
   const size_t csz = p.bf16 ? 2 : 4;
   Carver c(ws);
   const int64_t nmax = n > d ? n : d;
-  p.sb = carve_solve(c, nmax, nmax == n ? d : n, p.tsize, true);
+  p.sb = carve_solve(c, nmax, nmax == n ? d : n, p.tsize);
   p.sbA = carve_solve(c, d, n, p.tsize);
   p.W1t = c.take<float>((size_t)n * d);
   p.W2t = c.take<float>((size_t)n * d);
@@ -882,15 +868,10 @@ static sp_status admm_step_impl(const sp_ffn_module* m, sp_ffn_state* st, const 
   // millisecond, during which the caller's stream would otherwise sit empty.  (Without a side stream both run on
   // the caller's stream and the order does not matter.)
   CU(effective_ridge(st->G_A, n, n, prm->rho, prm->rho_relative, rho2, s));
-  // The unrestricted recovery, the largest system of a step, takes the two-part form of its products (7168 x 28672: 169 -> 125
-  // ms per step, 2048 x 8192 13.9 -> 12.7; errors of scores and weights against 64 bits as before).  The direct systems of
-  // the kept support and of the a-update stay with three parts: they are a small share, and a change of their rounding alone
-  // moves W1 of a 7168-wide module by 1 % over four iterations, through the sign select (it is 1.5 % from 64 bits either way).
-  const bool two_part = bf16;
   if (skip_scores) {
   } else if (bf16) {
     SPCHK(ridge_core<float>(st->R2, n, st->G_A, n, d, n, reuse ? p.perm : nullptr, n, rho2, p.W2t, n, p.sb, status_dev,
-                            s, side ? &side->assist_main : nullptr, false, reuse ? &lead : nullptr, false, two_part));
+                            s, side ? &side->assist_main : nullptr, false, reuse ? &lead : nullptr));
   } else {
     SPCHK(ridge_core<double>(st->R2, n, st->G_A, n, d, n, nullptr, n, rho2, p.W2t, n, p.sb, status_dev, s,
                              side ? &side->assist_main : nullptr));
@@ -983,8 +964,8 @@ static sp_status admm_step_impl(const sp_ffn_module* m, sp_ffn_state* st, const 
         ProfScope prof(PK_SOLVE, 2.0 * (double)d * k_lead * k_lead, 0.0, s);
         SPCHK(potrs_right_tc(lead.Y, d, k_lead, k_lead, p.sb.P, reinterpret_cast<const float*>(p.sb.dinv), p.sb.Xs,
                              status_dev, s, side ? &side->assist_main : nullptr, true,
-                             reinterpret_cast<const float*>(p.sb.Gs), n, n, HalfParts{p.sb.rowf}));
-        CU(scatter_cols<float>(lead.Y, k_lead, p.sb.idx, d, k, n, st->W2, n, s, p.sb.scale));
+                             reinterpret_cast<const float*>(p.sb.Gs), n, n));
+        CU(scatter_cols<float>(lead.Y, k_lead, p.sb.idx, d, k, n, st->W2, n, s));
       }
       {
         SkipScope skip_if_unchanged(p.reuse_flags + 1);

@@ -201,16 +201,6 @@ __device__ __forceinline__ void strip_index(const int32_t* idx, int64_t cols, in
     at[q] = j < cols ? (idx ? (int64_t)idx[j] : j) : 0;
   }
 }
-// scale[j] (scale == nullptr: 1) of this thread's columns
-template <int W>
-__device__ __forceinline__ void strip_scale(const float* scale, int64_t cols, float (&f)[kStripPer]) {
-  const int64_t c0 = strip_col<W>();
-#pragma unroll
-  for (int q = 0; q < kStripPer; ++q) {
-    const int64_t j = c0 + q * strip_width<W>();
-    f[q] = scale != nullptr && j < cols ? scale[j] : 1.f;
-  }
-}
 #endif
 
 inline size_t dtype_size(int32_t dt) { return dt == SP_BF16 ? 2 : (dt == SP_F64 ? 8 : 4); }
@@ -248,12 +238,6 @@ struct TcOperand {
   bool kmajor;
   int64_t kext = 0;   // extent of the stored matrix along K (0: the K of the call); reads beyond it return zero
   int64_t mnext = 0;  // extent along M (for A) or N (for B) (0: the M / N of the call)
-  bool half = false;  // fp16 elements instead of bf16 (both operands of a product the same)
-};
-// Rows m >= first of a product count f[m - first] times (fp32 C of a call without batch)
-struct TcRowFactor {
-  const float* f = nullptr;
-  int64_t first = 0;
 };
 // K segments: the contraction runs over nseg segments of K indices each; segment s reads A at K offset a_k[s] and
 // M offset a_mn[s], B at K offset b_k[s] and N offset b_mn[s] (elements).  This is how split operands (an fp32 value
@@ -284,7 +268,7 @@ struct TcBatch {
 sp_status gemm_tc(int64_t M, int64_t N, int64_t K, float alpha, TcOperand A, TcOperand B, float beta, Operand Cin,
                   OutOperand C, bool lower_only, int32_t* status_dev, cudaStream_t stream,
                   const TcSegments* segs = nullptr, double alg_flops = -1.0, int max_pairs = 0,
-                  const TcBatch* batch = nullptr, TcRowFactor rows = TcRowFactor{});
+                  const TcBatch* batch = nullptr);
 bool gemm_tc_supported(int64_t M, int64_t N, int64_t K, TcOperand A, TcOperand B);
 
 struct SolveAssist;
@@ -306,15 +290,14 @@ constexpr int kCholNB = 64;
 //   P   : bf16 [chol_tc_pad(n), 3 * chol_tc_pad(n)] — the factor below its diagonal blocks as three bf16 parts
 //   Xs  : chol_tc_xs_elems(n, m) bf16 — the current block columns of the right-hand sides as three bf16 parts
 constexpr int kCholTcNB = 128;
-// Two-level blocking of the factorisation and of the backward sweep: systems of at least kOuterMinN unknowns (kOuterMinHalf in the
-// two-part form, whose products take half the time and meet the traffic of K = 128 updates earlier), outer blocks of
-// kOuterBlocks diagonal blocks.  ADMM step with a two-part system of 8192 unknowns: 13.53 -> 12.69 ms, of 4376: 3.85 -> 3.96.
-constexpr int64_t kOuterMinN = 12288, kOuterMinHalf = 6144;
+// Two-level blocking of the factorisation and of the backward sweep: systems of at least kOuterMinN unknowns, outer blocks
+// of kOuterBlocks diagonal blocks.
+constexpr int64_t kOuterMinN = 12288;
 constexpr int64_t kOuterBlocks = 4;
 int64_t chol_tc_pad(int64_t n);
 // two buffers of one block column, or one of an outer block
 inline int64_t chol_tc_xs_elems(int64_t n, int64_t m) {
-  return m * 3 * kCholTcNB * (n >= kOuterMinHalf ? kOuterBlocks : 2);
+  return m * 3 * kCholTcNB * (n >= kOuterMinN ? kOuterBlocks : 2);
 }
 // Optional second stream (with three events) that carries the part of each step that the next step's first kernel
 // does not wait for: the far part of a solve step's update; the panel and trailing update of a factorisation step.
@@ -329,27 +312,19 @@ struct SolveAssist {
   cudaEvent_t far_go = nullptr, far_done[2] = {nullptr, nullptr};
   cudaEvent_t far_first = nullptr;      // its first two block columns, which the next step's near update adds to, have landed
 };
-// Two-part form of the factor and of the right-hand sides: fp16 hi + lo instead of three bf16 parts (see sp_linalg_tc.cu).
-// rowf: room for half_rowf_elems(n, m) floats.  The system must be scaled to a diagonal in [1, 4) (system_scale).
-struct HalfParts {
-  float* rowf = nullptr;     // nullptr: three bf16 parts
-};
-// factors of the right-hand sides' rows: one set per block column, one of an outer block
-inline int64_t half_rowf_elems(int64_t n, int64_t m) { return (ceil_div(n, (int64_t)kCholTcNB) + 1) * m; }
 // dinv must have room for ceil(n / 128) + 1 pairs of 128 x 128 blocks (the last pair is scratch).
 // m_extra > 0: A has m_extra more rows below row n (same lda), the right-hand sides B of a system X L^T = B; they
 // are carried through the panels and trailing updates and hold X on return (P then needs n + m_extra rows).
 sp_status potrf_lower_tc(float* A, int64_t n, int64_t lda, float* dinv, void* P, int32_t* status_dev,
                          cudaStream_t stream, const SolveAssist* assist = nullptr, int64_t m_extra = 0,
-                         bool split_lookahead = false,    // lookahead kernel as two launches without a cluster
-                         HalfParts half = HalfParts{});
+                         bool split_lookahead = false);   // lookahead kernel as two launches without a cluster
 // forward_done: X already holds the solution of the forward system (it rode along with the factorisation).
 // Lf / ldl (optional): the fp32 factor potrf_lower_tc left in A; with it the backward sweep updates a block column by
 // the one before it inside the panel kernel instead of by a GEMM of its own.
 sp_status potrs_right_tc(float* X, int64_t m, int64_t n, int64_t ldx, const void* P, const float* dinv, void* Xs,
                          int32_t* status_dev, cudaStream_t stream, const SolveAssist* assist = nullptr,
                          bool forward_done = false, const float* Lf = nullptr, int64_t ldl = 0,
-                         int64_t n_factor = 0, HalfParts half = HalfParts{});
+                         int64_t n_factor = 0);
 // n_factor > n: the factor in P / dinv / Lf is that of a larger system of n_factor rows and the solve uses its leading
 // n x n block, which is the factor of the system's leading block (n a multiple of kCholTcNB).
 
@@ -390,27 +365,23 @@ template <typename T>
 cudaError_t load_spd(const float* G, int64_t ldg, int64_t n, const double* rho_dev, T* dst, int64_t ldd,
                      cudaStream_t stream);
 // gathered version: dst[a,b] = G[idx[a], idx[b]] (+rho on diagonal), count read from host k.
-// scale[a] = power of two with scale[a]^2 (G[idx[a], idx[a]] + rho) in [1, 4) (idx == nullptr: identity); 1 where that is not a
-// positive finite number.  load_spd_gather, gather_cols and scatter_cols multiply row / column a by scale[a] (exactly).
-cudaError_t system_scale(const float* G, int64_t ldg, const int32_t* idx, int64_t n, const double* rho_dev, float* scale,
-                         cudaStream_t stream);
 template <typename T>
 cudaError_t load_spd_gather(const float* G, int64_t ldg, const int32_t* idx, int64_t k, const double* rho_dev, T* dst,
-                            int64_t ldd, cudaStream_t stream, const float* scale = nullptr);
+                            int64_t ldd, cudaStream_t stream);
 // dst [rows, kpad] (dense) = the first k columns of src followed by zero columns
 cudaError_t copy_cols_padded(const float* src, int64_t lds, int64_t rows, int64_t k, int64_t kpad, float* dst,
                              cudaStream_t stream);
 // dst[i, a] = (T) src[i, idx[a]]  (idx == nullptr: identity)
 template <typename T>
 cudaError_t gather_cols(const float* src, int64_t lds, const int32_t* idx, int64_t rows, int64_t k, T* dst,
-                        int64_t ldd, cudaStream_t stream, const float* scale = nullptr);
+                        int64_t ldd, cudaStream_t stream);
 // dst[i, :] = src[idx[i], :]
 cudaError_t gather_rows(const float* src, int64_t lds, const int32_t* idx, int64_t rows, int64_t cols, float* dst,
                         int64_t ldd, cudaStream_t stream);
 // dst (fp32, [rows, n]) = 0 ; dst[i, idx[a]] = src[i, a]
 template <typename T>
 cudaError_t scatter_cols(const T* src, int64_t lds, const int32_t* idx, int64_t rows, int64_t k, int64_t n,
-                         float* dst, int64_t ldd, cudaStream_t stream, const float* scale = nullptr);
+                         float* dst, int64_t ldd, cudaStream_t stream);
 // rho_out[0] = rho * trace(G)/n (relative) or rho
 cudaError_t effective_ridge(const float* G, int64_t ldg, int64_t n, double rho, int rel, double* rho_out,
                             cudaStream_t stream);

@@ -143,7 +143,7 @@ constexpr int kSpdTile = 32;
 template <typename T>
 __global__ void __launch_bounds__(256) load_spd_kernel(const float* __restrict__ G, int64_t ldg, const int32_t* idx,
                                                        int64_t n, const double* rho, T* __restrict__ dst, int64_t ldd,
-                                                       const float* __restrict__ scale, const int32_t* skip) {
+                                                       const int32_t* skip) {
   kernel_begin();
   if (skip != nullptr && *skip != 0) return;   // conditional launch (see SkipScope)
   constexpr int TS = kSpdTile;
@@ -178,7 +178,6 @@ __global__ void __launch_bounds__(256) load_spd_kernel(const float* __restrict__
     if (i < n && j <= i) {
       double v = (double)tile[r][tx];
       if (i == j) v += rr;
-      if (scale != nullptr) v *= (double)scale[i] * (double)scale[j];
       dst[i * ldd + j] = (T)v;
     }
   }
@@ -188,15 +187,13 @@ template <int W, typename T>
 __global__ void __launch_bounds__(kStripThreads) gather_cols_kernel(const float* __restrict__ src, int64_t lds,
                                                                     const int32_t* idx, int64_t rows, int64_t k,
                                                                     T* __restrict__ dst, int64_t ldd,
-                                                                    const float* __restrict__ scale, const int32_t* skip) {
+                                                                    const int32_t* skip) {
   kernel_begin();
   if (skip != nullptr && *skip != 0) return;
   int64_t at[kStripPer];
   strip_index<W>(idx, k, at);
-  float f[kStripPer];
-  strip_scale<W>(scale, k, f);
   for_strip<W>(rows, k, [&](int64_t i, int64_t a, int q) {
-    dst[i * ldd + a] = (T)(src[i * lds + at[q]] * f[q]);
+    dst[i * ldd + a] = (T)src[i * lds + at[q]];
   });
 }
 
@@ -213,15 +210,13 @@ template <int W, typename T>
 __global__ void __launch_bounds__(kStripThreads) scatter_cols_kernel(const T* __restrict__ src, int64_t lds,
                                                                      const int32_t* idx, int64_t rows, int64_t k,
                                                                      float* __restrict__ dst, int64_t ldd,
-                                                                     const float* __restrict__ scale, const int32_t* skip) {
+                                                                     const int32_t* skip) {
   kernel_begin();
   if (skip != nullptr && *skip != 0) return;
   int64_t at[kStripPer];
   strip_index<W>(idx, k, at);
-  float f[kStripPer];
-  strip_scale<W>(scale, k, f);
   for_strip<W>(rows, k, [&](int64_t i, int64_t a, int q) {
-    dst[i * ldd + at[q]] = (float)src[i * lds + a] * f[q];
+    dst[i * ldd + at[q]] = (float)src[i * lds + a];
   });
 }
 
@@ -241,23 +236,6 @@ __global__ void __launch_bounds__(kStripThreads) copy_cols_padded_kernel(const f
   for_strip<W>(rows, kpad, [&](int64_t i, int64_t a, int) {
     dst[i * kpad + a] = a < k ? src[i * lds + a] : 0.f;
   });
-}
-
-// scale[a] = 2^-floor(log2(g) / 2), g = G[idx[a], idx[a]] + rho
-__global__ void __launch_bounds__(256) system_scale_kernel(const float* __restrict__ G, int64_t ldg, const int32_t* idx,
-                                                           int64_t n, const double* rho, float* __restrict__ scale) {
-  kernel_begin();
-  const int64_t a = (int64_t)blockIdx.x * 256 + threadIdx.x;
-  if (a >= n) return;
-  const int64_t i = idx ? (int64_t)idx[a] : a;
-  const float g = (float)((double)G[i * ldg + i] + rho[0]);
-  float f = 1.f;
-  if (g > 0.f && g <= 3.0e38f) {
-    int e = (int)((__float_as_uint(g) >> 23) & 255u) - 127;          // (subnormal: as 2^-127)
-    e = e >= 0 ? e / 2 : -((1 - e) / 2);                             // floor(e / 2)
-    f = __uint_as_float((uint32_t)(127 - e) << 23);
-  }
-  scale[a] = f;
 }
 
 __global__ void effective_ridge_kernel(const float* G, int64_t ldg, int64_t n, double rho, int rel, double* out) {
@@ -1205,27 +1183,27 @@ cudaError_t load_spd(const float* G, int64_t ldg, int64_t n, const double* rho_d
   if (n == 0) return cudaSuccess;
   ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
   count_launch();
-  launch(load_spd_kernel<T>, lower_tiles(n, kSpdTile), 256, 0, stream, G, ldg, nullptr, n, rho_dev, dst, ldd, nullptr, skip_flag());
+  launch(load_spd_kernel<T>, lower_tiles(n, kSpdTile), 256, 0, stream, G, ldg, nullptr, n, rho_dev, dst, ldd, skip_flag());
   return cudaGetLastError();
 }
 template <typename T>
 cudaError_t load_spd_gather(const float* G, int64_t ldg, const int32_t* idx, int64_t k, const double* rho_dev, T* dst,
-                            int64_t ldd, cudaStream_t stream, const float* scale) {
+                            int64_t ldd, cudaStream_t stream) {
   if (k == 0) return cudaSuccess;
   ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
   count_launch();
-  launch(load_spd_kernel<T>, lower_tiles(k, kSpdTile), 256, 0, stream, G, ldg, idx, k, rho_dev, dst, ldd, scale, skip_flag());
+  launch(load_spd_kernel<T>, lower_tiles(k, kSpdTile), 256, 0, stream, G, ldg, idx, k, rho_dev, dst, ldd, skip_flag());
   return cudaGetLastError();
 }
 template <typename T>
 cudaError_t gather_cols(const float* src, int64_t lds, const int32_t* idx, int64_t rows, int64_t k, T* dst,
-                        int64_t ldd, cudaStream_t stream, const float* scale) {
+                        int64_t ldd, cudaStream_t stream) {
   if (rows * k == 0) return cudaSuccess;
   ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
   count_launch();
   strip_launch(rows, k, [&](auto w, dim3 grid, dim3 block) {
     launch(gather_cols_kernel<decltype(w)::value, T>, grid, block, 0, stream, 
-        src, lds, idx, rows, k, dst, ldd, scale, skip_flag());
+        src, lds, idx, rows, k, dst, ldd, skip_flag());
   });
   return cudaGetLastError();
 }
@@ -1252,7 +1230,7 @@ cudaError_t gather_rows(const float* src, int64_t lds, const int32_t* idx, int64
 
 template <typename T>
 cudaError_t scatter_cols(const T* src, int64_t lds, const int32_t* idx, int64_t rows, int64_t k, int64_t n,
-                         float* dst, int64_t ldd, cudaStream_t stream, const float* scale) {
+                         float* dst, int64_t ldd, cudaStream_t stream) {
   if (rows * n == 0) return cudaSuccess;
   if (idx) {
     ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
@@ -1265,30 +1243,21 @@ cudaError_t scatter_cols(const T* src, int64_t lds, const int32_t* idx, int64_t 
   count_launch();
   strip_launch(rows, k, [&](auto w, dim3 grid, dim3 block) {
     launch(scatter_cols_kernel<decltype(w)::value, T>, grid, block, 0, stream, 
-        src, lds, idx, rows, k, dst, ldd, scale, skip_flag());
+        src, lds, idx, rows, k, dst, ldd, skip_flag());
   });
   return cudaGetLastError();
 }
 #define SP_INST(T)                                                                                                  \
   template cudaError_t load_spd<T>(const float*, int64_t, int64_t, const double*, T*, int64_t, cudaStream_t);      \
   template cudaError_t load_spd_gather<T>(const float*, int64_t, const int32_t*, int64_t, const double*, T*,       \
-                                          int64_t, cudaStream_t, const float*);                                                   \
+                                          int64_t, cudaStream_t);                                                   \
   template cudaError_t gather_cols<T>(const float*, int64_t, const int32_t*, int64_t, int64_t, T*, int64_t,        \
-                                      cudaStream_t, const float*);                                                  \
+                                      cudaStream_t);                                                                \
   template cudaError_t scatter_cols<T>(const T*, int64_t, const int32_t*, int64_t, int64_t, int64_t, float*,       \
-                                       int64_t, cudaStream_t, const float*);
+                                       int64_t, cudaStream_t);
 SP_INST(float)
 SP_INST(double)
 #undef SP_INST
-
-cudaError_t system_scale(const float* G, int64_t ldg, const int32_t* idx, int64_t n, const double* rho_dev, float* scale,
-                         cudaStream_t stream) {
-  if (n == 0) return cudaSuccess;
-  ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
-  count_launch();
-  launch(system_scale_kernel, (unsigned)ceil_div(n, (int64_t)256), 256, 0, stream, G, ldg, idx, n, rho_dev, scale);
-  return cudaGetLastError();
-}
 
 cudaError_t effective_ridge(const float* G, int64_t ldg, int64_t n, double rho, int rel, double* rho_out,
                             cudaStream_t stream) {

@@ -83,9 +83,6 @@ struct TcParams {
   int8_t a_ord[4], b_ord[4], c_ord[4];
   int64_t c_s0, c_s1, cin_s0, cin_s1;
   int32_t b_shared0;       // one B for all b0
-  int32_t half;            // fp16 operands
-  const float* row_f;      // rows from row_first on count row_f[row - row_first] times
-  int64_t row_first;
   long long wait_budget;   // clock cycles a role may wait on one barrier before it gives up (SP_ERR_TIMEOUT)
   int32_t* status;
   const int32_t* skip;     // conditional launch: every CTA returns at once when *skip != 0 (see SkipScope)
@@ -267,12 +264,12 @@ __device__ __forceinline__ uint64_t make_smem_desc(uint32_t addr, bool kmajor, u
   return d;
 }
 
-// Instruction descriptor of the pair's MMA: 256 x tile_n x 16, bf16 (or fp16) operands, fp32 accumulator.
-__device__ __forceinline__ uint32_t make_instr_desc(bool a_kmajor, bool b_kmajor, int tile_n, bool half) {
+// Instruction descriptor of the pair's MMA: 256 x tile_n x 16, bf16 operands, fp32 accumulator.
+__device__ __forceinline__ uint32_t make_instr_desc(bool a_kmajor, bool b_kmajor, int tile_n) {
   uint32_t d = 0;
   d |= 1u << 4;                          // accumulator format: fp32
-  d |= (half ? 0u : 1u) << 7;            // A format: fp16 or bf16
-  d |= (half ? 0u : 1u) << 10;           // B format: the same
+  d |= 1u << 7;                          // A format: bf16
+  d |= 1u << 10;                         // B format: bf16
   d |= (a_kmajor ? 0u : 1u) << 15;       // A major-ness
   d |= (b_kmajor ? 0u : 1u) << 16;       // B major-ness
   d |= (uint32_t)(tile_n >> 3) << 17;    // N
@@ -456,7 +453,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer (leader CTA only)
     if (lane == 0 && rank == 0) {
-      const uint32_t idesc = make_instr_desc(p.a_kmajor != 0, p.b_kmajor != 0, TN, p.half != 0);
+      const uint32_t idesc = make_instr_desc(p.a_kmajor != 0, p.b_kmajor != 0, TN);
       int s = 0;
       uint32_t ph = 0;
       int acc = 0;
@@ -522,14 +519,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       tile_coords<BATCHED>(p, tile, tm, tn, b0, b1);
       const int64_t c_boff = BATCHED ? (int64_t)b0 * p.c_s0 + (int64_t)b1 * p.c_s1 : 0;
       const int64_t cin_boff = BATCHED ? (int64_t)b0 * p.cin_s0 + (int64_t)b1 * p.cin_s1 : 0;
-      const int64_t row0 = (int64_t)tm * TILE_M + (int64_t)rank * BM + q * 32;   // first global row of this warp
-      float alpha = p.alpha;                  // of this lane's row (not in the batched form)
-      if constexpr (!BATCHED)
-        if (p.row_f != nullptr && row0 + lane >= p.row_first && row0 + lane < p.M) alpha *= p.row_f[row0 + lane - p.row_first];
       // every lane observes the barrier itself; the vote keeps the warp converged for the aligned TMEM loads
       const bool got = mbar_wait(tfull_bar(acc), aph, abort_flag, p.wait_budget);
       if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
       tc_fence_after();
+      const int64_t row0 = (int64_t)tm * TILE_M + (int64_t)rank * BM + q * 32;   // first global row of this warp
       const uint32_t taddr = tmem_base + (uint32_t)(acc * TILE_N) + ((uint32_t)(q * 32) << 16);
       const int rows_here = (p.M - row0 < 32) ? (int)(p.M - row0) : 32;   // may be <= 0 on a ragged last tile
       if (p.epi_mode == EPI_TMA_BF16_CIN) {
@@ -653,8 +647,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           uint8_t* tile = wstg_ptr + buf * 4096 + lane * 128;
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
-            const float4 v = make_float4(alpha * __uint_as_float(r[4 * j]), alpha * __uint_as_float(r[4 * j + 1]),
-                                         alpha * __uint_as_float(r[4 * j + 2]), alpha * __uint_as_float(r[4 * j + 3]));
+            const float4 v = make_float4(p.alpha * __uint_as_float(r[4 * j]), p.alpha * __uint_as_float(r[4 * j + 1]),
+                                         p.alpha * __uint_as_float(r[4 * j + 2]), p.alpha * __uint_as_float(r[4 * j + 3]));
             *reinterpret_cast<float4*>(tile + ((j ^ (lane & 7)) << 4)) = v;
           }
           fence_async_smem();
@@ -701,7 +695,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           tc_ld32(taddr + (uint32_t)c0, r);
           tc_wait_ld();
 #pragma unroll
-          for (int i = 0; i < 32; ++i) stg[lane][i] = alpha * __uint_as_float(r[i]);
+          for (int i = 0; i < 32; ++i) stg[lane][i] = p.alpha * __uint_as_float(r[i]);
           __syncwarp();
           if (gj < p.N) {
             const int64_t c_off = c_boff + row0 * p.c_ld + gj;
@@ -852,7 +846,7 @@ bool gemm_tc_supported(int64_t M, int64_t N, int64_t K, TcOperand A, TcOperand B
 
 sp_status gemm_tc(int64_t M, int64_t N, int64_t K, float alpha, TcOperand A, TcOperand B, float beta, Operand Cin,
                   OutOperand C, bool lower_only, int32_t* status_dev, cudaStream_t stream, const TcSegments* segs,
-                  double alg_flops, int max_pairs, const TcBatch* batch, TcRowFactor rows) {
+                  double alg_flops, int max_pairs, const TcBatch* batch) {
   const bool batched = batch != nullptr;
   if (batched && (batch->nb0 < 1 || batch->nb1 < 1 || batch->a_planes < 1 || batch->b_planes < 1))
     return SP_ERR_INVALID_ARG;
@@ -872,7 +866,6 @@ sp_status gemm_tc(int64_t M, int64_t N, int64_t K, float alpha, TcOperand A, TcO
     if (sg.a_k[i] < 0 || sg.a_mn[i] < 0 || sg.b_k[i] < 0 || sg.b_mn[i] < 0) return SP_ERR_INVALID_ARG;
   }
   if (lower_only && M < N) return SP_ERR_SHAPE;
-  if (A.half != B.half || (rows.f != nullptr && (batched || C.dtype != SP_F32 || rows.first < 0))) return SP_ERR_INVALID_ARG;
   if (beta != 0.f && (Cin.ptr == nullptr || Cin.s1 != 1)) return SP_ERR_INVALID_ARG;
   if (C.dtype != SP_F32 && C.dtype != SP_BF16) return SP_ERR_DTYPE;
   if (beta != 0.f && Cin.dtype != SP_F32 && Cin.dtype != SP_BF16) return SP_ERR_DTYPE;
@@ -924,9 +917,6 @@ sp_status gemm_tc(int64_t M, int64_t N, int64_t K, float alpha, TcOperand A, TcO
   p.cin_s0 = batched ? batch->cin_s0 : 0; p.cin_s1 = batched ? batch->cin_s1 : 0;
 
   p.M = M; p.N = N; p.K = K;
-  p.half = A.half ? 1 : 0;
-  p.row_f = rows.f;
-  p.row_first = rows.first;
   p.alpha = alpha; p.beta = beta;
   p.cin = Cin.ptr; p.cin_dtype = Cin.dtype; p.cin_ld = Cin.s0;
   p.c = C.ptr; p.c_dtype = C.dtype; p.c_ld = C.ld;

@@ -4,16 +4,13 @@
 // activations with a condition number of the order of its size), which a plain bf16 product cannot give.  Every fp32
 // value is therefore held as an exact sum of three bf16 parts (hi + mid + lo, 3 x 8 mantissa bits), and a product
 // of two such operands is taken as the six part products of weight >= 2^-16 (hi.hi, hi.mid, mid.hi, hi.lo, lo.hi,
-// mid.mid), each a K segment of one tcgen05 GEMM with fp32 accumulation.  The dropped terms are below 2^-23.  Systems scaled to
-// a diagonal of about one take two fp16 parts and three products instead (split_half).
+// mid.mid), each a K segment of one tcgen05 GEMM with fp32 accumulation.  The dropped terms are below 2^-23.
 //
 // Blocked right-looking algorithm with 128-wide panels:
 //   diagonal block : one CTA factorises it and forms inv(L11) in the same sweep (sp_chol_block.cuh);
 //   panel          : L21 = A21 inv(L11)^T on the CUDA cores (K = 128), written as fp32 and as the three bf16 parts;
 //   trailing update: A22 -= L21 L21^T (lower triangle) as one six-segment tensor-core GEMM.
 // The triangular solves X L^T = R, W L = X use the same two kernels block column by block column.
-#include <cuda_fp16.h>
-
 #include "sp_chol_block.cuh"
 #include "sp_common.cuh"
 
@@ -43,26 +40,6 @@ __device__ __forceinline__ void split3(float v, __nv_bfloat16& hi, __nv_bfloat16
   mid = __float2bfloat16_rn(r1);
   const float r2 = r1 - __bfloat162float(mid);
   lo = __float2bfloat16_rn(r2);
-}
-
-// Two-part form: x 2^e = hi + lo + (error below 2^-24 |x 2^e|), both fp16.  Rows of the factor are below 2 in a system scaled to a
-// diagonal in [1, 4) (|L_ij| <= sqrt(A_ii)) and take e = kHalfExp; right-hand sides, whose size nothing bounds, take the e that brings
-// the largest entry of the row's block column to [2^kHalfExp, 2^(kHalfExp + 1)); their rows of a product are multiplied by it when
-// they leave the tensor cores (TcRowFactor).  Entries 2^-15 of the largest keep all 22 bits, smaller ones an absolute error
-// of 2^-37 of it.  Three part products (hi.hi, hi.lo, lo.hi; lo.lo is below 2^-24) instead of six, and half as many roundings of
-// the fp32 accumulator, which are what the error consists of.
-constexpr int kHalfExp = 12;
-__device__ __forceinline__ void split_half(float v, float up, __half& hi, __half& lo) {
-  const float x = v * up;
-  hi = __float2half_rn(x);
-  lo = __float2half_rn(x - __half2float(hi));
-}
-// 2^(kHalfExp - floor(log2 m)), limited to +-100; 1 for zero, infinities and NaN
-__device__ __forceinline__ float half_up(float m) {
-  if (!(m > 0.f) || m > 3.0e38f) return 1.f;
-  int e = kHalfExp - ((int)((__float_as_uint(m) >> 23) & 255u) - 127);
-  e = e > 100 ? 100 : e < -100 ? -100 : e;
-  return __uint_as_float((uint32_t)(e + 127) << 23);
 }
 
 // ---- staging of one 128 x 128 fp32 block (64 KiB) into shared memory by bulk asynchronous copies
@@ -178,13 +155,6 @@ struct PanelBatch {
   int64_t x = 0, dinv = 0, s = 0, near_l = 0;    // X (and near.W), dinv, S, near.L
 };
 
-// Two-part form of a panel's result: rows from `first` on are right-hand sides, their 2^(kHalfExp - e) to rowf[row - first].
-struct PanelHalf {
-  int on = 0;
-  float* rowf = nullptr;
-  int64_t first = 0;
-};
-
 // X[i, 0:nb] <- X[i, 0:nb] inv(L)^T (TRANS == false) or X[i, 0:nb] inv(L) (TRANS == true), for `rows` rows.
 // dinv is the pair of TB x TB blocks written by chol_diag128_kernel.  The result is written back in fp32 (write_f32)
 // and as three bf16 parts to S[i * lds + part * s_seg + c] for all TB columns (zero beyond nb).
@@ -196,7 +166,7 @@ __global__ void __launch_bounds__(RowTile<R>::THREADS) panel_apply_kernel(float*
                                                                  const float* __restrict__ dinv, __nv_bfloat16* S,
                                                                  int64_t lds, int64_t s_seg, int write_f32,
                                                                  int32_t* status, PanelNear near,
-                                                                 const int32_t* skip, PanelBatch pb, PanelHalf half) {
+                                                                 const int32_t* skip, PanelBatch pb) {
   kernel_begin();
   if (skip != nullptr && *skip != 0) return;
   using Tile = RowTile<R>;
@@ -280,14 +250,6 @@ __global__ void __launch_bounds__(RowTile<R>::THREADS) panel_apply_kernel(float*
     for (int j = 0; j < 4; ++j)
       if (c0 + j >= nb) v[j] = 0.f;
     out[q] = make_float4(v[0], v[1], v[2], v[3]);
-    float up = (float)(1 << kHalfExp);
-    if (half.on && gi >= half.first) {       // (a warp has whole rows: the condition is uniform over it)
-      float m = fmaxf(fmaxf(fabsf(v[0]), fabsf(v[1])), fmaxf(fabsf(v[2]), fabsf(v[3])));
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-      up = half_up(m);
-      if ((t & 31) == 0 && gi < rows) half.rowf[gi - half.first] = (float)(1 << kHalfExp) / up;
-    }
     if (gi >= rows) continue;
     if (write_f32) {
       float* dst = X + gi * ldx + c0;
@@ -299,14 +261,7 @@ __global__ void __launch_bounds__(RowTile<R>::THREADS) panel_apply_kernel(float*
           if (c0 + j < nb) dst[j] = v[j];
       }
     }
-    if (S && half.on) {
-      __align__(8) __half part[2][4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) split_half(v[j], up, part[0][j], part[1][j]);
-#pragma unroll
-      for (int z = 0; z < 2; ++z)
-        *reinterpret_cast<uint2*>(S + gi * lds + z * s_seg + c0) = *reinterpret_cast<const uint2*>(part[z]);
-    } else if (S) {   // S + gi * lds + part * s_seg + c0 is 8-byte aligned by construction (lds, s_seg multiples of 8)
+    if (S) {   // S + gi * lds + part * s_seg + c0 is 8-byte aligned by construction (lds, s_seg multiples of 8)
       __align__(8) __nv_bfloat16 part[3][4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) split3(v[j], part[0][j], part[1][j], part[2][j]);
@@ -320,7 +275,7 @@ __global__ void __launch_bounds__(RowTile<R>::THREADS) panel_apply_kernel(float*
 template <bool TRANS, int R>
 cudaError_t launch_panel_rows(float* X, int64_t ldx, int64_t rows, int nb, const float* dinv, __nv_bfloat16* S, int64_t lds,
                               int64_t s_seg, bool write_f32, int32_t* status, cudaStream_t stream, PanelNear near,
-                              int batch, PanelBatch pb, PanelHalf half) {
+                              int batch, PanelBatch pb) {
   static PerDeviceOnce attr_once;      // one per instantiation; the attribute belongs to the device's context
   cudaError_t e = attr_once.run([] {
     return cudaFuncSetAttribute(panel_apply_kernel<TRANS, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -330,7 +285,7 @@ cudaError_t launch_panel_rows(float* X, int64_t ldx, int64_t rows, int nb, const
   const bool with_near = TRANS && near.L != nullptr;
   launch(panel_apply_kernel<TRANS, R>, dim3((unsigned)ceil_div(rows, R), (unsigned)batch), RowTile<R>::THREADS,
                                  pa_smem<R>(with_near), stream, X, ldx, rows, nb, dinv, S, lds, s_seg, write_f32 ? 1 : 0, status, near,
-                                           skip_flag(), pb, half);
+                                           skip_flag(), pb);
   return cudaGetLastError();
 }
 
@@ -343,18 +298,17 @@ inline int panel_rows(int64_t rows, int batch, int64_t ctas) {
 template <bool TRANS>
 cudaError_t launch_panel_apply(float* X, int64_t ldx, int64_t rows, int nb, const float* dinv, __nv_bfloat16* S,
                                int64_t lds, int64_t s_seg, bool write_f32, int32_t* status, cudaStream_t stream,
-                               PanelNear near = kNoNear, int batch = 1, PanelBatch pb = PanelBatch{}, int per_cta = 0,
-                               PanelHalf half = PanelHalf{}) {
+                               PanelNear near = kNoNear, int batch = 1, PanelBatch pb = PanelBatch{}, int per_cta = 0) {
   if (rows <= 0) return cudaSuccess;
   count_launch();
   const bool with_near = TRANS && near.L != nullptr;
   ProfScope prof(PK_PANEL_APPLY, (with_near ? 4.0 : 2.0) * (double)rows * TB * TB, 0.0, stream);
   if (per_cta == 0) per_cta = panel_rows(rows, batch, sm_count());
   if (per_cta == 8)
-    return launch_panel_rows<TRANS, 8>(X, ldx, rows, nb, dinv, S, lds, s_seg, write_f32, status, stream, near, batch, pb, half);
+    return launch_panel_rows<TRANS, 8>(X, ldx, rows, nb, dinv, S, lds, s_seg, write_f32, status, stream, near, batch, pb);
   if (per_cta == 16)
-    return launch_panel_rows<TRANS, 16>(X, ldx, rows, nb, dinv, S, lds, s_seg, write_f32, status, stream, near, batch, pb, half);
-  return launch_panel_rows<TRANS, 32>(X, ldx, rows, nb, dinv, S, lds, s_seg, write_f32, status, stream, near, batch, pb, half);
+    return launch_panel_rows<TRANS, 16>(X, ldx, rows, nb, dinv, S, lds, s_seg, write_f32, status, stream, near, batch, pb);
+  return launch_panel_rows<TRANS, 32>(X, ldx, rows, nb, dinv, S, lds, s_seg, write_f32, status, stream, near, batch, pb);
 }
 
 // The six kept part products of two three-part operands: A parts (hi, hi, mid, hi, lo, mid) against B parts
@@ -380,7 +334,6 @@ struct NextRows {
   __nv_bfloat16* P;      // parts at P[i * ldp + part * seg + c]
   int64_t ldp, seg;
   int vec;               // 16-byte aligned rows of A21
-  int half;              // two-part form
 };
 
 // MODE 0: both stages in one launch, the CTAs being one cluster (they meet between the stages);
@@ -449,15 +402,6 @@ __device__ __forceinline__ void next_diag_body(float* A21, const float* __restri
 #pragma unroll
         for (int j = 0; j < 4; ++j) dst[j] = v[j];
       }
-      if (out_rows.half) {
-        __align__(8) __half h[2][4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) split_half(v[j], (float)(1 << kHalfExp), h[0][j], h[1][j]);
-#pragma unroll
-        for (int z = 0; z < 2; ++z)
-          *reinterpret_cast<uint2*>(out_rows.P + i * out_rows.ldp + z * out_rows.seg + c0) = *reinterpret_cast<const uint2*>(h[z]);
-        continue;
-      }
       __align__(8) __nv_bfloat16 part[3][4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) split3(v[j], part[0][j], part[1][j], part[2][j]);
@@ -518,74 +462,15 @@ __global__ void __launch_bounds__(NM_THREADS)
 
 constexpr int kPartA[6] = {0, 0, 1, 0, 2, 1};
 constexpr int kPartB[6] = {0, 1, 0, 2, 0, 1};
-// The first three are those of the two-part form.  A's parts sit ka columns apart and start at a0, B's kb and b0 (along N for
-// b_along_n).
-TcSegments part_products(bool half, int64_t ka, int64_t a0, int64_t kb, int64_t b0, bool b_along_n) {
-  TcSegments sg;
-  sg.nseg = half ? 3 : 6;
-  for (int q = 0; q < sg.nseg; ++q) {
-    sg.a_k[q] = (int32_t)(kPartA[q] * ka + a0);
-    (b_along_n ? sg.b_mn : sg.b_k)[q] = (int32_t)(kPartB[q] * kb + b0);
-  }
-  return sg;
-}
-// C -= (...): both operands of a two-part product carry 2^kHalfExp, which the row factors of right-hand sides allow for
-float minus_one(bool half) { return half ? -1.f / ((float)(1 << kHalfExp) * (float)(1 << kHalfExp)) : -1.f; }
-
-// Two-part form of rows of right-hand sides over the columns of an outer block (up to 512), with one factor per row: what one
-// product over all of them needs.  One warp per row; S at S[row * lds + part * seg + c], zero from `cols` to `width`.
-__global__ void __launch_bounds__(256) split_half_rows_kernel(const float* __restrict__ X, int64_t ldx, int64_t rows, int cols,
-                                                              int width, __nv_bfloat16* S, int64_t lds, int64_t seg,
-                                                              float* __restrict__ rowf, const int32_t* skip) {
-  kernel_begin();
-  if (skip != nullptr && *skip != 0) return;
-  constexpr int PER = kOuterBlocks * TB / 32;
-  const int lane = threadIdx.x & 31;
-  const int64_t r = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-  if (r >= rows) return;
-  float v[PER], m = 0.f;
-#pragma unroll
-  for (int q = 0; q < PER; q += 2)
-#pragma unroll
-    for (int z = 0; z < 2; ++z) {
-      const int c = (q / 2 * 32 + lane) * 2 + z;
-      v[q + z] = c < cols ? X[r * ldx + c] : 0.f;
-      m = fmaxf(m, fabsf(v[q + z]));
-    }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  const float up = half_up(m);
-  if (lane == 0) rowf[r] = (float)(1 << kHalfExp) / up;
-#pragma unroll
-  for (int q = 0; q < PER; q += 2) {
-    const int c = (q / 2 * 32 + lane) * 2;
-    if (c >= width) continue;
-    __half2 hi, lo;
-    split_half(v[q], up, hi.x, lo.x);
-    split_half(v[q + 1], up, hi.y, lo.y);
-    *reinterpret_cast<__half2*>(S + r * lds + c) = hi;
-    *reinterpret_cast<__half2*>(S + r * lds + seg + c) = lo;
-  }
-}
-cudaError_t launch_split_half_rows(const float* X, int64_t ldx, int64_t rows, int64_t cols, int64_t width, __nv_bfloat16* S,
-                                   int64_t lds, int64_t seg, float* rowf, cudaStream_t stream) {
-  if (rows <= 0) return cudaSuccess;
-  count_launch();
-  return launch(split_half_rows_kernel, (unsigned)ceil_div(rows, (int64_t)8), 256, 0, stream, X, ldx, rows, (int)cols,
-                (int)width, S, lds, seg, rowf, skip_flag());
-}
 
 }  // namespace
 
 int64_t chol_tc_pad(int64_t n) { return (n + TB - 1) / TB * TB; }
 
 sp_status potrf_lower_tc(float* A, int64_t n, int64_t lda, float* dinv, void* Pv, int32_t* status_dev,
-                         cudaStream_t stream, const SolveAssist* assist, int64_t m_extra, bool split_lookahead,
-                         HalfParts hp) {
-  __nv_bfloat16* P = reinterpret_cast<__nv_bfloat16*>(Pv);      // (fp16 in the two-part form)
-  const bool half = hp.rowf != nullptr;
-  const int64_t np = chol_tc_pad(n), ldp = (half ? 2 : 3) * np;
-  const float minus = minus_one(half);
+                         cudaStream_t stream, const SolveAssist* assist, int64_t m_extra, bool split_lookahead) {
+  __nv_bfloat16* P = reinterpret_cast<__nv_bfloat16*>(Pv);
+  const int64_t np = chol_tc_pad(n), ldp = 3 * np;
   const int64_t nblk = ceil_div(n, (int64_t)TB);
   const int32_t* skip = skip_flag();
   static PerDeviceOnce attr_once;
@@ -623,7 +508,7 @@ sp_status potrf_lower_tc(float* A, int64_t n, int64_t lda, float* dinv, void* Pv
   // matrix when K is only 128 (n = 28672: 430 GB per factorisation).  With OB > 1 the steps of an outer block of OB
   // diagonal blocks update only the rest of that outer block's columns at once; everything to the right of it gets
   // ONE update per outer block with K = OB * 128, which divides that traffic by OB.
-  const int64_t OB = (assist && n >= (half ? kOuterMinHalf : kOuterMinN)) ? kOuterBlocks : 1;
+  const int64_t OB = (assist && n >= kOuterMinN) ? kOuterBlocks : 1;
   for (int64_t kb = 0; kb < nblk; ++kb) {
     const int64_t k0 = kb * TB;
     const int nb = (int)((n - k0 < TB) ? (n - k0) : TB);
@@ -673,8 +558,7 @@ sp_status potrf_lower_tc(float* A, int64_t n, int64_t lda, float* dinv, void* Pv
         if (far_rec[kb & 1]) SP_CUDA_OK(cudaStreamWaitEvent(stream, assist->far_done[kb & 1], 0));   // far update of step kb - 2
         const int nb2 = (int)ahead;
         float* A21 = A + (k0 + nb) * lda + k0;
-        const NextRows rows{P + (k0 + nb) * ldp + k0, ldp, np, lda % 4 == 0 && (reinterpret_cast<uintptr_t>(A) & 15u) == 0,
-                            half ? 1 : 0};
+        const NextRows rows{P + (k0 + nb) * ldp + k0, ldp, np, lda % 4 == 0 && (reinterpret_cast<uintptr_t>(A) & 15u) == 0};
         count_launch();
         ProfScope prof(PK_PANEL_APPLY, 4.0 * TB * TB * TB, 0.0, stream);
         if (!split_lookahead) {
@@ -692,10 +576,8 @@ sp_status potrf_lower_tc(float* A, int64_t n, int64_t lda, float* dinv, void* Pv
     }
     // L21 = A21 inv(L11)^T, fp32 in place and as bf16 parts in P[k0+nb.., part * np + k0 ..]
     const int64_t p0 = k0 + nb + ahead;
-    float* rowf = hp.rowf + kb * m_extra;      // (two-part form) factors of the right-hand sides' rows for this block column
     if (launch_panel_apply<false>(A + p0 * lda + k0, lda, prow - ahead, nb, dk, P + p0 * ldp + k0, ldp, np, true,
-                                  status_dev, sb, kNoNear, 1, PanelBatch{}, 0,
-                                  PanelHalf{half ? 1 : 0, rowf, rem - ahead}) != cudaSuccess)
+                                  status_dev, sb) != cudaSuccess)
       return SP_ERR_CUDA;
     if (rem <= 0) break;     // last block: the appended rows are done, nothing is left to update
     if (far_apart && !outer && rem > 2 * TB) SP_CUDA_OK(cudaEventRecord(assist->far_go, sb));   // the panel's parts exist
@@ -706,11 +588,14 @@ sp_status potrf_lower_tc(float* A, int64_t n, int64_t lda, float* dinv, void* Pv
     // A22 -= L21 L21^T on the lower triangle
     TcOperand ta{P + (k0 + nb) * ldp, ldp, true}, tb{P + (k0 + nb) * ldp, ldp, true};
     ta.kext = tb.kext = ldp;
-    ta.half = tb.half = half;
     ta.mnext = prow;
     tb.mnext = rem;
-    auto rows_from = [&](const float* f, int64_t first) { return half && m_extra > 0 ? TcRowFactor{f, first} : TcRowFactor{}; };
-    const TcSegments sg = part_products(half, np, k0, np, k0, false);
+    TcSegments sg;
+    sg.nseg = 6;
+    for (int q = 0; q < 6; ++q) {
+      sg.a_k[q] = (int32_t)(kPartA[q] * np + k0);
+      sg.b_k[q] = (int32_t)(kPartB[q] * np + k0);
+    }
     float* A22 = A + (k0 + nb) * lda + (k0 + nb);
     constexpr int64_t kNear = 2 * TB;     // block columns of the update that the next step's chain kernels read
     if (outer) {
@@ -718,10 +603,9 @@ sp_status potrf_lower_tc(float* A, int64_t n, int64_t lda, float* dinv, void* Pv
       const int64_t cols_in = ob_end_col - (k0 + nb);
       if (cols_in > 0) {
         tb.mnext = cols_in;
-        sp_status st = gemm_tc(prow, cols_in, TB, minus, ta, tb, 1.f, Operand{A22, SP_F32, lda, 1},
+        sp_status st = gemm_tc(prow, cols_in, TB, -1.f, ta, tb, 1.f, Operand{A22, SP_F32, lda, 1},
                                OutOperand{A22, SP_F32, lda}, true, status_dev, sb, &sg,
-                               (2.0 * (double)prow * (double)cols_in - (double)cols_in * (double)cols_in) * (double)nb, 0,
-                               nullptr, rows_from(rowf, rem));
+                               (2.0 * (double)prow * (double)cols_in - (double)cols_in * (double)cols_in) * (double)nb);
         if (st != SP_OK) return st;
         SP_CUDA_OK(cudaEventRecord(assist->near_done, sb));
       }
@@ -729,46 +613,42 @@ sp_status potrf_lower_tc(float* A, int64_t n, int64_t lda, float* dinv, void* Pv
       const int64_t cols_out = n - ob_end_col;
       if (inner_last && cols_out > 0) {
         const int64_t o0 = ob_start * TB, kw = ob_end_col - o0, prow_out = cols_out + m_extra;
-        const TcSegments so = part_products(half, np, o0, np, o0, false);
-        float* rowf_o = hp.rowf + nblk * m_extra;
-        if (half && launch_split_half_rows(A + n * lda + o0, lda, m_extra, kw, kw, P + n * ldp + o0, ldp, np, rowf_o, sb) !=
-                        cudaSuccess)
-          return SP_ERR_CUDA;
+        TcSegments so;
+        so.nseg = 6;
+        for (int q = 0; q < 6; ++q) {
+          so.a_k[q] = (int32_t)(kPartA[q] * np + o0);
+          so.b_k[q] = (int32_t)(kPartB[q] * np + o0);
+        }
         float* Aout = A + ob_end_col * lda + ob_end_col;
         const int64_t wn = cols_out < kNear ? cols_out : kNear;
         TcOperand na{P + ob_end_col * ldp, ldp, true}, nbo{P + ob_end_col * ldp, ldp, true};
         na.kext = nbo.kext = ldp;
-        na.half = nbo.half = half;
         na.mnext = prow_out;
         nbo.mnext = wn;
-        sp_status st = gemm_tc(prow_out, wn, kw, minus, na, nbo, 1.f, Operand{Aout, SP_F32, lda, 1},
+        sp_status st = gemm_tc(prow_out, wn, kw, -1.f, na, nbo, 1.f, Operand{Aout, SP_F32, lda, 1},
                                OutOperand{Aout, SP_F32, lda}, true, status_dev, sb, &so,
-                               (2.0 * (double)prow_out * (double)wn - (double)wn * (double)wn) * (double)kw, 0, nullptr,
-                               rows_from(rowf_o, cols_out));
+                               (2.0 * (double)prow_out * (double)wn - (double)wn * (double)wn) * (double)kw);
         if (st != SP_OK) return st;
         SP_CUDA_OK(cudaEventRecord(assist->near_done, sb));
         if (cols_out > wn) {
           TcOperand fa{P + (ob_end_col + wn) * ldp, ldp, true}, fb{P + (ob_end_col + wn) * ldp, ldp, true};
           fa.kext = fb.kext = ldp;
-      fa.half = fb.half = half;
           fa.mnext = prow_out - wn;
           fb.mnext = cols_out - wn;
           float* Afar = Aout + wn * lda + wn;
           const double fr = (double)(cols_out - wn);
-          st = gemm_tc(prow_out - wn, cols_out - wn, kw, minus, fa, fb, 1.f, Operand{Afar, SP_F32, lda, 1},
+          st = gemm_tc(prow_out - wn, cols_out - wn, kw, -1.f, fa, fb, 1.f, Operand{Afar, SP_F32, lda, 1},
                        OutOperand{Afar, SP_F32, lda}, true, status_dev, sb, &so,
-                       (fr * fr + 2.0 * (double)m_extra * fr) * (double)kw, 0, nullptr,
-                       rows_from(rowf_o, cols_out - wn));
+                       (fr * fr + 2.0 * (double)m_extra * fr) * (double)kw);
           if (st != SP_OK) return st;
         }
       }
     } else if (assist && rem > kNear) {
       // two launches: the first two block columns (all rows below), signalled at once, then the rest
       tb.mnext = kNear;
-      sp_status st = gemm_tc(prow, kNear, TB, minus, ta, tb, 1.f, Operand{A22, SP_F32, lda, 1},
+      sp_status st = gemm_tc(prow, kNear, TB, -1.f, ta, tb, 1.f, Operand{A22, SP_F32, lda, 1},
                              OutOperand{A22, SP_F32, lda}, true, status_dev, sb, &sg,
-                             (2.0 * (double)prow * (double)kNear - (double)kNear * (double)kNear) * (double)nb, 0, nullptr,
-                             rows_from(rowf, rem));
+                             (2.0 * (double)prow * (double)kNear - (double)kNear * (double)kNear) * (double)nb);
       if (st != SP_OK) return st;
       SP_CUDA_OK(cudaEventRecord(assist->near_done, sb));
       cudaStream_t sf = sb;
@@ -784,13 +664,12 @@ sp_status potrf_lower_tc(float* A, int64_t n, int64_t lda, float* dinv, void* Pv
         const int64_t w = c0 == 0 ? cut : fw - c0, r0 = k0 + nb + kNear + c0, rows_f = prow - kNear - c0;
         TcOperand fa{P + r0 * ldp, ldp, true}, fb{P + r0 * ldp, ldp, true};
         fa.kext = fb.kext = ldp;
-        fa.half = fb.half = half;
         fa.mnext = rows_f;
         fb.mnext = w;
         float* Afar = A + r0 * lda + r0;
-        st = gemm_tc(rows_f, w, TB, minus, fa, fb, 1.f, Operand{Afar, SP_F32, lda, 1}, OutOperand{Afar, SP_F32, lda}, true,
+        st = gemm_tc(rows_f, w, TB, -1.f, fa, fb, 1.f, Operand{Afar, SP_F32, lda, 1}, OutOperand{Afar, SP_F32, lda}, true,
                      status_dev, sf, &sg, (double)w * (2.0 * (double)rows_f - (double)w) * (double)nb,
-                     far_apart ? kFarPairs : 0, nullptr, rows_from(rowf, fw - c0));
+                     far_apart ? kFarPairs : 0);
         if (st != SP_OK) return st;
         if (far_apart && c0 == 0) SP_CUDA_OK(cudaEventRecord(assist->far_first, sf));
       }
@@ -799,10 +678,9 @@ sp_status potrf_lower_tc(float* A, int64_t n, int64_t lda, float* dinv, void* Pv
         far_rec[kb & 1] = true;
       }
     } else {
-      sp_status st = gemm_tc(prow, rem, TB, minus, ta, tb, 1.f, Operand{A22, SP_F32, lda, 1},
+      sp_status st = gemm_tc(prow, rem, TB, -1.f, ta, tb, 1.f, Operand{A22, SP_F32, lda, 1},
                              OutOperand{A22, SP_F32, lda}, true, status_dev, sb, &sg,
-                             ((double)rem * (double)rem + 2.0 * (double)m_extra * (double)rem) * (double)nb, 0, nullptr,
-                             rows_from(rowf, rem));
+                             ((double)rem * (double)rem + 2.0 * (double)m_extra * (double)rem) * (double)nb);
       if (st != SP_OK) return st;
       if (assist) SP_CUDA_OK(cudaEventRecord(assist->near_done, sb));
     }
@@ -822,16 +700,12 @@ sp_status potrf_lower_tc(float* A, int64_t n, int64_t lda, float* dinv, void* Pv
 
 sp_status potrs_right_tc(float* X, int64_t m, int64_t n, int64_t ldx, const void* Pv, const float* dinv, void* Xsv,
                          int32_t* status_dev, cudaStream_t stream, const SolveAssist* assist, bool forward_done,
-                         const float* Lf, int64_t ldl, int64_t n_factor, HalfParts hp) {
+                         const float* Lf, int64_t ldl, int64_t n_factor) {
   const __nv_bfloat16* P = reinterpret_cast<const __nv_bfloat16*>(Pv);
   __nv_bfloat16* Xs = reinterpret_cast<__nv_bfloat16*>(Xsv);
   if (n_factor > n && n % TB != 0) return SP_ERR_SHAPE;
-  const bool half = hp.rowf != nullptr;
-  if (half && !forward_done) return SP_ERR_UNSUPPORTED;       // (its forward substitution rides with the factorisation)
-  const float minus = minus_one(half);
-  const int64_t parts = half ? 2 : 3;
-  const int64_t np = chol_tc_pad(n_factor > n ? n_factor : n), ldp = parts * np;
-  const int64_t lds = parts * TB;
+  const int64_t np = chol_tc_pad(n_factor > n ? n_factor : n), ldp = 3 * np;
+  const int64_t lds = 3 * TB;
   const int64_t nblk = ceil_div(n, (int64_t)TB);
   // Every step applies the inverse diagonal block to one block column (panel) and then updates the columns still to
   // come.  With an assisting stream the update is cut in two: the next block column, which the next panel needs, stays
@@ -871,7 +745,6 @@ sp_status potrs_right_tc(float* X, int64_t m, int64_t n, int64_t ldx, const void
       const int nb = (int)((n - j0 < TB) ? (n - j0) : TB);
       const float* dj = dinv + jb * 2 * TB * TB;
       __nv_bfloat16* Xcur = Xs + (step & 1) * m * lds;
-      float* rowf = hp.rowf + (step & 1) * m;
       if (assist && rec[step & 1]) SP_CUDA_OK(cudaStreamWaitEvent(stream, assist->rest_done[step & 1], 0));
       // columns still to be updated: [lo, hi)
       const int64_t lo = forward ? j0 + nb : 0, hi = forward ? n : j0;
@@ -885,8 +758,7 @@ sp_status potrs_right_tc(float* X, int64_t m, int64_t n, int64_t ldx, const void
       cudaError_t e = forward ? launch_panel_apply<false>(X + j0, ldx, m, nb, dj, Xcur, lds, TB, true, status_dev, stream)
                               : launch_panel_apply<true>(X + j0, ldx, m, nb, dj, Xcur, lds, TB, true, status_dev, stream,
                                                          pn, 1, PanelBatch{},
-                                                         near_in_panel && assist && runs_beside(j0) ? rows_beside : 0,
-                                                         PanelHalf{half ? 1 : 0, rowf, 0});
+                                                         near_in_panel && assist && runs_beside(j0) ? rows_beside : 0);
       if (e != cudaSuccess) return SP_ERR_CUDA;
       if (hi <= lo) break;
       if (assist) SP_CUDA_OK(cudaEventRecord(assist->panel_done, stream));
@@ -902,25 +774,32 @@ sp_status potrs_right_tc(float* X, int64_t m, int64_t n, int64_t ldx, const void
         const bool on_assist = assist && part == 1;
         cudaStream_t st_run = on_assist ? assist->stream : stream;
         if (on_assist) SP_CUDA_OK(cudaStreamWaitEvent(st_run, assist->panel_done, 0));
+        TcSegments sg;
+        sg.nseg = 6;
         TcOperand tb{nullptr, ldp, forward};
         if (forward) {
           // X[:, c0:c0+w] -= Y_j L[c0:c0+w, j0:j0+nb]^T : B(k, c) = L[c0 + c, j0 + k], K-major rows of P
           tb.ptr = P + c0 * ldp;
           tb.kext = ldp;
           tb.mnext = w;
+          for (int q = 0; q < 6; ++q) {
+            sg.a_k[q] = kPartA[q] * TB;
+            sg.b_k[q] = (int32_t)(kPartB[q] * np + j0);
+          }
         } else {
           // X[:, c0:c0+w] -= W_j L[j0:j0+nb, c0:c0+w] : B(k, c) = L[j0 + k, c0 + c], rows of P, columns (N) contiguous
           tb.ptr = P + j0 * ldp;
           tb.kext = n - j0;      // rows of L that exist; beyond them the tensor map returns zero
           tb.mnext = ldp;
+          for (int q = 0; q < 6; ++q) {
+            sg.a_k[q] = kPartA[q] * TB;
+            sg.b_mn[q] = (int32_t)(kPartB[q] * np + c0);
+          }
         }
-        ta.half = tb.half = half;
-        const TcSegments sg = part_products(half, TB, 0, np, forward ? j0 : c0, !forward);
         float* Xc = X + c0;
-        sp_status stt = gemm_tc(m, w, TB, minus, ta, tb, 1.f, Operand{Xc, SP_F32, ldx, 1}, OutOperand{Xc, SP_F32, ldx},
+        sp_status stt = gemm_tc(m, w, TB, -1.f, ta, tb, 1.f, Operand{Xc, SP_F32, ldx, 1}, OutOperand{Xc, SP_F32, ldx},
                                 false, status_dev, st_run, &sg, 2.0 * (double)m * (double)w * (double)nb,
-                                on_assist && near_in_panel && runs_beside(w) ? (int)beside_pairs : 0, nullptr,
-                                half ? TcRowFactor{rowf, 0} : TcRowFactor{});
+                                on_assist && near_in_panel && runs_beside(w) ? (int)beside_pairs : 0);
         if (stt != SP_OK) return stt;
         if (on_assist) {
           SP_CUDA_OK(cudaEventRecord(assist->rest_done[step & 1], st_run));
@@ -940,21 +819,23 @@ sp_status potrs_right_tc(float* X, int64_t m, int64_t n, int64_t ldx, const void
   // right-hand sides: 0.45 ms for 0.3 TFLOP, 224 times).  The panels of an outer block update the rest of that block
   // only, and everything to its left receives one update per outer block with K = 512.
   auto backward_outer = [&]() -> sp_status {
-    constexpr int64_t OBW = kOuterBlocks * TB;
-    const int64_t ldo = parts * OBW;
+    constexpr int64_t OBW = kOuterBlocks * TB, ldo = 3 * OBW;
     // X[:, c0:c0+w] -= W[:, a0:a0+K of the outer block] L[r0:r0+K, c0:c0+w]
-    auto update = [&](int64_t a0, int64_t r0, int64_t K, int64_t c0, int64_t w, const float* rowf) -> sp_status {
+    auto update = [&](int64_t a0, int64_t r0, int64_t K, int64_t c0, int64_t w) -> sp_status {
       if (w <= 0) return SP_OK;
       TcOperand ta{Xs, ldo, true}, tb{P + r0 * ldp, ldp, false};
       ta.kext = ldo;
       ta.mnext = m;
       tb.kext = n - r0;
       tb.mnext = ldp;
-      ta.half = tb.half = half;
-      const TcSegments sg = part_products(half, OBW, a0, np, c0, true);
-      return gemm_tc(m, w, K, minus, ta, tb, 1.f, Operand{X + c0, SP_F32, ldx, 1}, OutOperand{X + c0, SP_F32, ldx}, false,
-                     status_dev, stream, &sg, 2.0 * (double)m * (double)w * (double)K, 0, nullptr,
-                     half ? TcRowFactor{rowf, 0} : TcRowFactor{});
+      TcSegments sg;
+      sg.nseg = 6;
+      for (int q = 0; q < 6; ++q) {
+        sg.a_k[q] = (int32_t)(kPartA[q] * OBW + a0);
+        sg.b_mn[q] = (int32_t)(kPartB[q] * np + c0);
+      }
+      return gemm_tc(m, w, K, -1.f, ta, tb, 1.f, Operand{X + c0, SP_F32, ldx, 1}, OutOperand{X + c0, SP_F32, ldx}, false,
+                     status_dev, stream, &sg, 2.0 * (double)m * (double)w * (double)K);
     };
     for (int64_t b1 = nblk; b1 > 0;) {
       const int64_t b0 = (b1 - 1) / kOuterBlocks * kOuterBlocks, o0 = b0 * TB;
@@ -963,20 +844,13 @@ sp_status potrs_right_tc(float* X, int64_t m, int64_t n, int64_t ldx, const void
         const int nb = (int)((n - j0 < TB) ? (n - j0) : TB);
         PanelNear pn = kNoNear;
         if (fuse_near && jb + 1 < b1) pn = PanelNear{Lf + p0 * ldl + j0, ldl, X + p0, (int)((n - p0 < TB) ? n - p0 : TB)};
-        float* rowf = hp.rowf + (jb - b0) * m;
         if (launch_panel_apply<true>(X + j0, ldx, m, nb, dinv + jb * 2 * TB * TB, Xs + (j0 - o0), ldo, OBW, true,
-                                     status_dev, stream, pn, 1, PanelBatch{}, 0, PanelHalf{half ? 1 : 0, rowf, 0}) !=
-            cudaSuccess)
+                                     status_dev, stream, pn) != cudaSuccess)
           return SP_ERR_CUDA;
-        sp_status r = update(j0 - o0, j0, TB, o0, j0 - o0 - (fuse_near ? TB : 0), rowf);
+        sp_status r = update(j0 - o0, j0, TB, o0, j0 - o0 - (fuse_near ? TB : 0));
         if (r != SP_OK) return r;
       }
-      const int64_t kw = (b1 - b0) * TB;
-      float* rowf = hp.rowf + kOuterBlocks * m;
-      if (half && o0 > 0 &&
-          launch_split_half_rows(X + o0, ldx, m, n - o0 < kw ? n - o0 : kw, kw, Xs, ldo, OBW, rowf, stream) != cudaSuccess)
-        return SP_ERR_CUDA;
-      sp_status r = update(0, o0, kw, 0, o0, rowf);
+      sp_status r = update(0, o0, (b1 - b0) * TB, 0, o0);
       if (r != SP_OK) return r;
       b1 = b0;
     }
@@ -986,7 +860,7 @@ sp_status potrs_right_tc(float* X, int64_t m, int64_t n, int64_t ldx, const void
     sp_status r = run_sweep(true);    // Y L^T = X, block columns left to right
     if (r != SP_OK) return r;
   }
-  return n >= (half ? kOuterMinHalf : kOuterMinN) ? backward_outer() : run_sweep(false);     // W L = Y, block columns right to left
+  return n >= kOuterMinN ? backward_outer() : run_sweep(false);     // W L = Y, block columns right to left
 #undef SP_CUDA_OK
 }
 
