@@ -88,6 +88,11 @@ __host__ __device__ __forceinline__ size_t align_up(size_t a, size_t b) { return
 // kernels before is touched until they have completed.  Each kernel waits, so the completion of one implies that of all
 // before it, as without the attribute; only launch latency, block start and the set-up ahead of the wait overlap.  Both
 // instructions do nothing in a kernel that was launched plainly.
+// A kernel's life begins while what it reads is still being written, by the library's or by the caller's kernels.  So no kernel
+// has __restrict__ pointers: const and __restrict__ together allow loads on the read-only path, whose contract is that the data
+// does not change during the kernel's whole life, and which the wait need not precede.  Loads through plain pointers stay
+// behind the wait (it clobbers memory) and are coherent, but they stay behind the stores before them too: loads that are to be
+// in flight together stand before the first store of a round (for_strip_move; split_planes 90 -> 140 us where they do not).
 // The attribute is given inside an OverlapScope only, which the entry points open for calls whose kernels are short: their
 // time is launches and gaps (attention step 768 wide, 284 kernels: 2.68 -> 2.42 ms; ADMM step 768 x 3072 2.40 -> 2.28).  Long
 // kernels lose: waiting blocks hold SMs that another stream's kernels could use (ADMM step of 2048 x 8192 on 262144 tokens: 49.3
@@ -183,6 +188,28 @@ __device__ __forceinline__ void for_strip(int64_t rows, int64_t cols, F&& f) {
       const int64_t j = c0 + q * strip_width<W>();
       if (j < cols) f(i, j, q);
     }
+}
+// store(i, j, q, load(i, j, q)) for this thread's rows and columns, the loads of two rows in flight before a store
+template <int W, typename L, typename S>
+__device__ __forceinline__ void for_strip_move(int64_t rows, int64_t cols, L&& load, S&& store) {
+  const int64_t c0 = strip_col<W>(), step = strip_rows<W>();
+  for (int64_t i = strip_row<W>(); i < rows; i += 2 * step) {
+    decltype(load(i, c0, 0)) v[2][kStripPer] = {};
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int q = 0; q < kStripPer; ++q) {
+        const int64_t r = i + h * step, j = c0 + q * strip_width<W>();
+        if (r < rows && j < cols) v[h][q] = load(r, j, q);
+      }
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int q = 0; q < kStripPer; ++q) {
+        const int64_t r = i + h * step, j = c0 + q * strip_width<W>();
+        if (r < rows && j < cols) store(r, j, q, v[h][q]);
+      }
+  }
 }
 // tile (row block y, column block x <= y) of a lower triangle of tiles counted row by row
 __device__ __forceinline__ void lower_tile(unsigned t, unsigned& y, unsigned& x) {

@@ -83,14 +83,16 @@ __device__ __forceinline__ bool pairs_aligned(const float* src, int64_t lds) {
 
 // (kpad is even: a thread takes two columns, so that the bf16 stores are 4 bytes wide)
 template <int W>
-__global__ void __launch_bounds__(kStripThreads) split_bf16_kernel(const float* __restrict__ src, int64_t lds,
-                                                                   const int32_t* __restrict__ row_idx, int64_t rows,
+__global__ void __launch_bounds__(kStripThreads) split_bf16_kernel(const float* src, int64_t lds,
+                                                                   const int32_t* row_idx, int64_t rows,
                                                                    int64_t cols, int64_t kpad,
-                                                                   __nv_bfloat16* __restrict__ dst) {
+                                                                   __nv_bfloat16* dst) {
   kernel_begin();
   const bool vec = pairs_aligned(src, lds);
-  for_strip<W>(rows, kpad / 2, [&](int64_t i, int64_t p, int) {
-    const float2 v = load_pair(src + (row_idx ? (int64_t)row_idx[i] : i) * lds, 2 * p, cols, vec);
+  const auto load = [&](int64_t i, int64_t p, int) {
+    return load_pair(src + (row_idx ? (int64_t)row_idx[i] : i) * lds, 2 * p, cols, vec);
+  };
+  for_strip_move<W>(rows, kpad / 2, load, [&](int64_t i, int64_t p, int, float2 v) {
     const __nv_bfloat162 hi = __floats2bfloat162_rn(v.x, v.y);
     __nv_bfloat162* out = reinterpret_cast<__nv_bfloat162*>(dst + i * 2 * kpad) + p;
     out[0] = hi;
@@ -101,13 +103,13 @@ __global__ void __launch_bounds__(kStripThreads) split_bf16_kernel(const float* 
 // dst[i, part * kpad + j] = part `part` of the three-part bf16 split of src[i, j] (hi + mid + lo = src exactly up to
 // 2^-24); padding columns are zero.
 template <int W>
-__global__ void __launch_bounds__(kStripThreads) split3_bf16_kernel(const float* __restrict__ src, int64_t lds,
+__global__ void __launch_bounds__(kStripThreads) split3_bf16_kernel(const float* src, int64_t lds,
                                                                     int64_t rows, int64_t cols, int64_t kpad,
-                                                                    __nv_bfloat16* __restrict__ dst) {
+                                                                    __nv_bfloat16* dst) {
   kernel_begin();
   const bool vec = pairs_aligned(src, lds);
-  for_strip<W>(rows, kpad / 2, [&](int64_t i, int64_t p, int) {
-    const float2 v = load_pair(src + i * lds, 2 * p, cols, vec);
+  const auto load = [&](int64_t i, int64_t p, int) { return load_pair(src + i * lds, 2 * p, cols, vec); };
+  for_strip_move<W>(rows, kpad / 2, load, [&](int64_t i, int64_t p, int, float2 v) {
     const __nv_bfloat162 hi = __floats2bfloat162_rn(v.x, v.y);
     const float2 r1 = make_float2(v.x - __low2float(hi), v.y - __high2float(hi));
     const __nv_bfloat162 mid = __floats2bfloat162_rn(r1.x, r1.y);
@@ -141,8 +143,8 @@ constexpr int kSpdTile = 32;
 // above the diagonal of G, where it is read as (j, i): those are read with the lanes along i, the others along j, so that
 // either way a warp reads along a row of G (kept channels first, n = 28672: 2.4 -> 1.4 ms).
 template <typename T>
-__global__ void __launch_bounds__(256) load_spd_kernel(const float* __restrict__ G, int64_t ldg, const int32_t* idx,
-                                                       int64_t n, const double* rho, T* __restrict__ dst, int64_t ldd,
+__global__ void __launch_bounds__(256) load_spd_kernel(const float* G, int64_t ldg, const int32_t* idx,
+                                                       int64_t n, const double* rho, T* dst, int64_t ldd,
                                                        const int32_t* skip) {
   kernel_begin();
   if (skip != nullptr && *skip != 0) return;   // conditional launch (see SkipScope)
@@ -184,40 +186,37 @@ __global__ void __launch_bounds__(256) load_spd_kernel(const float* __restrict__
 }
 
 template <int W, typename T>
-__global__ void __launch_bounds__(kStripThreads) gather_cols_kernel(const float* __restrict__ src, int64_t lds,
+__global__ void __launch_bounds__(kStripThreads) gather_cols_kernel(const float* src, int64_t lds,
                                                                     const int32_t* idx, int64_t rows, int64_t k,
-                                                                    T* __restrict__ dst, int64_t ldd,
+                                                                    T* dst, int64_t ldd,
                                                                     const int32_t* skip) {
   kernel_begin();
   if (skip != nullptr && *skip != 0) return;
   int64_t at[kStripPer];
   strip_index<W>(idx, k, at);
-  for_strip<W>(rows, k, [&](int64_t i, int64_t a, int q) {
-    dst[i * ldd + a] = (T)src[i * lds + at[q]];
-  });
+  for_strip_move<W>(rows, k, [&](int64_t i, int64_t, int q) { return src[i * lds + at[q]]; },
+                    [&](int64_t i, int64_t a, int, float v) { dst[i * ldd + a] = (T)v; });
 }
 
 template <int W>
-__global__ void __launch_bounds__(kStripThreads) gather_rows_kernel(const float* __restrict__ src, int64_t lds, const int32_t* __restrict__ idx,
-                                   int64_t rows, int64_t cols, float* __restrict__ dst, int64_t ldd) {
+__global__ void __launch_bounds__(kStripThreads) gather_rows_kernel(const float* src, int64_t lds, const int32_t* idx,
+                                   int64_t rows, int64_t cols, float* dst, int64_t ldd) {
   kernel_begin();
-  for_strip<W>(rows, cols, [&](int64_t i, int64_t j, int) {
-    dst[i * ldd + j] = src[(int64_t)idx[i] * lds + j];
-  });
+  for_strip_move<W>(rows, cols, [&](int64_t i, int64_t j, int) { return src[(int64_t)idx[i] * lds + j]; },
+                    [&](int64_t i, int64_t j, int, float v) { dst[i * ldd + j] = v; });
 }
 
 template <int W, typename T>
-__global__ void __launch_bounds__(kStripThreads) scatter_cols_kernel(const T* __restrict__ src, int64_t lds,
+__global__ void __launch_bounds__(kStripThreads) scatter_cols_kernel(const T* src, int64_t lds,
                                                                      const int32_t* idx, int64_t rows, int64_t k,
-                                                                     float* __restrict__ dst, int64_t ldd,
+                                                                     float* dst, int64_t ldd,
                                                                      const int32_t* skip) {
   kernel_begin();
   if (skip != nullptr && *skip != 0) return;
   int64_t at[kStripPer];
   strip_index<W>(idx, k, at);
-  for_strip<W>(rows, k, [&](int64_t i, int64_t a, int q) {
-    dst[i * ldd + at[q]] = (float)src[i * lds + a];
-  });
+  for_strip_move<W>(rows, k, [&](int64_t i, int64_t a, int) { return src[i * lds + a]; },
+                    [&](int64_t i, int64_t, int q, T v) { dst[i * ldd + at[q]] = (float)v; });
 }
 
 template <int W>
@@ -230,12 +229,11 @@ __global__ void __launch_bounds__(kStripThreads) fill_zero_kernel(float* dst, in
 
 // dst[i, 0:kpad] = src[i, 0:k] followed by zeros
 template <int W>
-__global__ void __launch_bounds__(kStripThreads) copy_cols_padded_kernel(const float* __restrict__ src, int64_t lds, int64_t rows, int64_t k,
-                                        int64_t kpad, float* __restrict__ dst) {
+__global__ void __launch_bounds__(kStripThreads) copy_cols_padded_kernel(const float* src, int64_t lds, int64_t rows, int64_t k,
+                                        int64_t kpad, float* dst) {
   kernel_begin();
-  for_strip<W>(rows, kpad, [&](int64_t i, int64_t a, int) {
-    dst[i * kpad + a] = a < k ? src[i * lds + a] : 0.f;
-  });
+  for_strip_move<W>(rows, kpad, [&](int64_t i, int64_t a, int) { return a < k ? src[i * lds + a] : 0.f; },
+                    [&](int64_t i, int64_t a, int, float v) { dst[i * kpad + a] = v; });
 }
 
 __global__ void effective_ridge_kernel(const float* G, int64_t ldg, int64_t n, double rho, int rel, double* out) {
@@ -254,7 +252,7 @@ __global__ void effective_ridge_kernel(const float* G, int64_t ldg, int64_t n, d
 // channels are cut into groups of 8 consecutive ones: grp_base[g] = number of kept channels before channel 8 g,
 // grp_mask[g] = bit q set when channel 8 g + q is kept.  The kept channels of a group then sit at compact positions
 // grp_base[g], grp_base[g] + 1, ... in channel order.
-__global__ void __launch_bounds__(1024) group_map_kernel(const uint8_t* __restrict__ mask, int64_t n,
+__global__ void __launch_bounds__(1024) group_map_kernel(const uint8_t* mask, int64_t n,
                                                          int32_t* grp_base, uint8_t* grp_mask) {
   kernel_begin();
   __shared__ int warp_tot[32];
@@ -309,11 +307,11 @@ __device__ __forceinline__ void store8(void* base, int32_t dt, int64_t e, const 
 // (fp32) vectors per row.  Columns k..ldh-1 of H are written as zero.
 // lo_off > 0 (bf16 only): H holds two parts side by side, bf16(h) in columns [0, ncols) and bf16(h - bf16(h)) in columns
 // [lo_off, lo_off + ncols), so that a product with H keeps about 16 bits of h (two K segments of the GEMM).
-__global__ void __launch_bounds__(256) prep_h_kernel(const float* __restrict__ Z, const float* __restrict__ U,
-                                                     const float* __restrict__ G, void* __restrict__ H, int32_t hdt,
+__global__ void __launch_bounds__(256) prep_h_kernel(const float* Z, const float* U,
+                                                     const float* G, void* H, int32_t hdt,
                                                      int64_t T, int64_t n,
                                                      int64_t ldh, int64_t ncols, int64_t lo_off, int64_t k,
-                                                     const int32_t* __restrict__ idx, int32_t rows_per_block,
+                                                     const int32_t* idx, int32_t rows_per_block,
                                                      const int32_t* skip) {
   kernel_begin();
   if (skip != nullptr && *skip != 0) return;   // conditional launch (see SkipScope)
@@ -324,30 +322,38 @@ __global__ void __launch_bounds__(256) prep_h_kernel(const float* __restrict__ Z
   for (int q = 0; q < 8; ++q) ch[q] = (p0 + q < k) ? idx[p0 + q] : -1;
   const int64_t r_begin = (int64_t)blockIdx.y * rows_per_block;
   const int64_t r_end = (r_begin + rows_per_block < T) ? r_begin + rows_per_block : T;
-#pragma unroll 2
-  for (int64_t r = r_begin; r < r_end; ++r) {
-    const float* zr = Z + r * n;
-    float h[8];
+  const auto load = [&](const float* M, int64_t r, float (&v)[8]) {
 #pragma unroll
-    for (int q = 0; q < 8; ++q) h[q] = (ch[q] >= 0) ? (G ? zr[ch[q]] : fmaxf(zr[ch[q]], 0.f)) : 0.f;
-    if (G) {           // gated module: phi(z) = g z
-      const float* gr = G + r * n;
-#pragma unroll
-      for (int q = 0; q < 8; ++q)
-        if (ch[q] >= 0) h[q] *= gr[ch[q]];
-    }
-    if (U) {
-      const float* ur = U + r * n;
-#pragma unroll
-      for (int q = 0; q < 8; ++q)
-        if (ch[q] >= 0) h[q] -= ur[ch[q]];
-    }
+    for (int q = 0; q < 8; ++q) v[q] = ch[q] >= 0 ? M[r * n + ch[q]] : 0.f;
+  };
+  const auto store = [&](int64_t r, float (&h)[8]) {
     store8(H, hdt, r * ldh + p0, h);
     if (lo_off > 0) {
 #pragma unroll
       for (int q = 0; q < 8; ++q) h[q] -= __bfloat162float(__float2bfloat16_rn(h[q]));
       store8(H, hdt, r * ldh + lo_off + p0, h);
     }
+  };
+  for (int64_t r = r_begin; r < r_end; r += 2) {       // two rows of loads in flight
+    float h[2][8], g[2][8], u[2][8];
+    const int rows = r + 1 < r_end ? 2 : 1;
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+      if (i < rows) {
+        load(Z, r + i, h[i]);
+        if (G) load(G, r + i, g[i]);
+        if (U) load(U, r + i, u[i]);
+      }
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+      if (i < rows) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          h[i][q] = G ? __fmul_rn(h[i][q], g[i][q]) : fmaxf(h[i][q], 0.f);      // gated module: phi(z) = g z
+          if (U) h[i][q] -= u[i][q];
+        }
+        store(r + i, h[i]);
+      }
   }
 }
 
@@ -427,10 +433,10 @@ __global__ void __launch_bounds__(256, 2) fused_update_kernel(UpdateArgs g) {
   const int64_t r_begin = (int64_t)blockIdx.y * rows_per;
   const int64_t r_end = (r_begin + rows_per < g.T) ? r_begin + rows_per : g.T;
   const float inv_ab = 1.f / (g.alpha + g.beta);
-  float* __restrict__ Zp = g.Z;
-  float* __restrict__ Up = g.U;
-  const float* __restrict__ z1p = g.z1;
-  const float* __restrict__ Dp = g.D;
+  float* Zp = g.Z;
+  float* Up = g.U;
+  const float* z1p = g.z1;
+  const float* Dp = g.D;
   double s_res = 0.0, s_z = 0.0, s_a = 0.0, s_in = 0.0;
   float cs[4] = {0.f, 0.f, 0.f, 0.f};
   // With a transposed A every warp stages kAtRows rows of its 128 channels in shared memory (channel-major) and
@@ -685,9 +691,9 @@ __global__ void __launch_bounds__(256, 2) fused_update_next_kernel(UpdateArgs g)
   const int64_t r_begin = (int64_t)blockIdx.y * rows_per;
   const int64_t r_end = (r_begin + rows_per < g.T) ? r_begin + rows_per : g.T;
   const float inv_ab = 1.f / (g.alpha + g.beta);
-  float* __restrict__ Zp = g.Z;
-  const float* __restrict__ z1p = g.z1;
-  const float* __restrict__ Dp = g.D;
+  float* Zp = g.Z;
+  const float* z1p = g.z1;
+  const float* Dp = g.D;
   double s_res = 0.0, s_z = 0.0, s_a = 0.0, s_in = 0.0;
   float cs[2] = {0.f, 0.f};
   const bool active = c0 < g.n;                                 // n % 4 == 0: a thread's channels exist together
@@ -830,11 +836,11 @@ __global__ void __launch_bounds__(256, 2) fused_update_next_kernel(UpdateArgs g)
 // n % 4 == 0): Ht[p(c), t] = bf16(max(Z[t, c], 0)) for the kept channels c, p(c) = its rank among them — the transposed
 // layout in which the fused update above leaves it.  A thread owns 4 consecutive channels, a warp stages kAtRows rows
 // of its 128 channels in shared memory and writes the kept ones out as 64-byte pieces.
-__global__ void __launch_bounds__(256, 3) gather_ht_kernel(const float* __restrict__ Z, int64_t T, int64_t n, int64_t k,
-                                                           const int32_t* __restrict__ grp_base,
-                                                           const uint8_t* __restrict__ grp_mask,
-                                                           __nv_bfloat16* __restrict__ Ht, int64_t ldt,
-                                                           int32_t row_blocks, const int32_t* __restrict__ skip) {
+__global__ void __launch_bounds__(256, 3) gather_ht_kernel(const float* Z, int64_t T, int64_t n, int64_t k,
+                                                           const int32_t* grp_base,
+                                                           const uint8_t* grp_mask,
+                                                           __nv_bfloat16* Ht, int64_t ldt,
+                                                           int32_t row_blocks, const int32_t* skip) {
   kernel_begin();
   if (skip != nullptr && *skip != 0) return;
   extern __shared__ __align__(16) __nv_bfloat16 zt_tile[];     // [1024][kAtPitch]
@@ -913,7 +919,7 @@ __global__ void __launch_bounds__(256, 3) gather_ht_kernel(const float* __restri
 // A thread owns 4 consecutive channels and walks its rows four at a time (16-byte loads of all four rows in flight
 // before the first store, as in the fused update); |A| is summed in fp32 over the four rows of a round and in fp64
 // across rounds.
-__global__ void __launch_bounds__(256) init_act_kernel(const float* __restrict__ Z, float* gate_io, void* A_out,
+__global__ void __launch_bounds__(256) init_act_kernel(const float* Z, float* gate_io, void* A_out,
                                                        void* Zb_out, int32_t out_dtype, int64_t T, int64_t n,
                                                        double* absA_part, int32_t row_blocks) {
   kernel_begin();
@@ -996,7 +1002,7 @@ __global__ void __launch_bounds__(256) init_act_kernel(const float* __restrict__
 
 // out[j] (+)= sum_r part[r, j]: a block takes 32 columns, its 8 warps take every 8th row block (four loads in flight
 // each), then the 8 partial sums of a column are added in a fixed order.
-__global__ void __launch_bounds__(256) reduce_col_partials_kernel(const double* __restrict__ part, int32_t row_blocks,
+__global__ void __launch_bounds__(256) reduce_col_partials_kernel(const double* part, int32_t row_blocks,
                                                                   int64_t n, double* out, int acc) {
   kernel_begin();
   __shared__ double sm[8][33];
@@ -1038,7 +1044,7 @@ __global__ void reduce_report_kernel(const double* partial, int nblocks, sp_step
 }
 
 // out[0] (+)= scale * sum x^2 over a [rows, cols] fp32 matrix: block partials, then one block adds them in order
-__global__ void __launch_bounds__(256) sumsq_partial_kernel(const float* __restrict__ x, int64_t ld, int64_t rows,
+__global__ void __launch_bounds__(256) sumsq_partial_kernel(const float* x, int64_t ld, int64_t rows,
                                                             int64_t cols, double* part) {
   kernel_begin();
   __shared__ double sm[32];

@@ -163,7 +163,7 @@ struct PanelBatch {
 // (see panel_rows): 768 rows, both products: 10.4 us with 48 CTAs of 16 rows, 15.4 us with 24 of 32.
 template <bool TRANS, int R>
 __global__ void __launch_bounds__(RowTile<R>::THREADS) panel_apply_kernel(float* X, int64_t ldx, int64_t rows, int nb,
-                                                                 const float* __restrict__ dinv, __nv_bfloat16* S,
+                                                                 const float* dinv, __nv_bfloat16* S,
                                                                  int64_t lds, int64_t s_seg, int write_f32,
                                                                  int32_t* status, PanelNear near,
                                                                  const int32_t* skip, PanelBatch pb) {
@@ -340,8 +340,8 @@ struct NextRows {
 // MODE 1 / MODE 2: the stages as two launches of 8 independent CTAs (for use beside persistent GEMM CTAs that hold
 // most SMs, where a cluster of 8 waits for a free group of SMs).
 template <int MODE>
-__device__ __forceinline__ void next_diag_body(float* A21, const float* __restrict__ A22, int64_t lda, int nb2,
-                                               const float* __restrict__ dinv, float* LmT, float* S, NextRows out_rows,
+__device__ __forceinline__ void next_diag_body(float* A21, const float* A22, int64_t lda, int nb2,
+                                               const float* dinv, float* LmT, float* S, NextRows out_rows,
                                                int32_t* status) {
   extern __shared__ __align__(128) float nm_smem[];
   using Tile = RowTile<NM_ROWS>;
@@ -438,22 +438,22 @@ __device__ __forceinline__ void next_diag_body(float* A21, const float* __restri
 }
 
 __global__ void __cluster_dims__(NM_CTAS, 1, 1) __launch_bounds__(NM_THREADS)
-    chol_next_diag_kernel(float* A21, const float* __restrict__ A22, int64_t lda, int nb2,
-                          const float* __restrict__ dinv, float* LmT, float* S, NextRows out_rows, int32_t* status,
+    chol_next_diag_kernel(float* A21, const float* A22, int64_t lda, int nb2,
+                          const float* dinv, float* LmT, float* S, NextRows out_rows, int32_t* status,
                           const int32_t* skip) {
   kernel_begin();
   if (skip != nullptr && *skip != 0) return;
   next_diag_body<0>(A21, A22, lda, nb2, dinv, LmT, S, out_rows, status);
 }
 __global__ void __launch_bounds__(NM_THREADS)
-    chol_next_diag_stage1_kernel(float* A21, int64_t lda, int nb2, const float* __restrict__ dinv, float* LmT,
+    chol_next_diag_stage1_kernel(float* A21, int64_t lda, int nb2, const float* dinv, float* LmT,
                                  NextRows out_rows, int32_t* status, const int32_t* skip) {
   kernel_begin();
   if (skip != nullptr && *skip != 0) return;
   next_diag_body<1>(A21, nullptr, lda, nb2, dinv, LmT, nullptr, out_rows, status);
 }
 __global__ void __launch_bounds__(NM_THREADS)
-    chol_next_diag_stage2_kernel(const float* __restrict__ A22, int64_t lda, int nb2, float* LmT, float* S,
+    chol_next_diag_stage2_kernel(const float* A22, int64_t lda, int nb2, float* LmT, float* S,
                                  const int32_t* skip) {
   kernel_begin();
   if (skip != nullptr && *skip != 0) return;

@@ -69,8 +69,8 @@ __device__ double block_max_bcast(double v, double* smem) {
 constexpr int kWsCols = 128, kWsWarps = 8, kWsUnroll = 8, kWsPerSm = 4;
 
 __global__ void __launch_bounds__(kWsWarps * 32, kWsPerSm) wanda_scores_kernel(
-    const float* __restrict__ W, int64_t rows, int64_t cols, int64_t ldw, int vec_ok, int kind, int group,
-    const float* __restrict__ colsq, int64_t colsq_stride, const double* __restrict__ colabs, double inv_tokens,
+    const float* W, int64_t rows, int64_t cols, int64_t ldw, int vec_ok, int kind, int group,
+    const float* colsq, int64_t colsq_stride, const double* colabs, double inv_tokens,
     int64_t n_units, float* scores, double* importance, double* part, double* colval, unsigned int* tickets) {
   kernel_begin();
   __shared__ double red[kWsWarps][kWsCols];
@@ -242,7 +242,7 @@ __device__ __forceinline__ float stat_scalar(const __nv_bfloat16* p) { return __
 constexpr int kStatInFlight = 8;     // 16-byte loads a thread keeps in flight
 
 template <typename T>
-__global__ void __launch_bounds__(256, 4) weight_stats_partial_kernel(const T* __restrict__ W, int64_t ld,
+__global__ void __launch_bounds__(256, 4) weight_stats_partial_kernel(const T* W, int64_t ld,
                                                                       int64_t rows, int64_t cols, int axis,
                                                                       int64_t group, int vec_ok, double* part) {
   kernel_begin();
@@ -400,9 +400,9 @@ struct L1Vec<__nv_bfloat16> {
 };
 
 template <typename T>
-__global__ void __launch_bounds__(256, 2) lemma1_partials_vec_kernel(const T* __restrict__ b, const T* __restrict__ c,
-                                                                     const T* __restrict__ dd,
-                                                                     const T* __restrict__ tt, int64_t ldb,
+__global__ void __launch_bounds__(256, 2) lemma1_partials_vec_kernel(const T* b, const T* c,
+                                                                     const T* dd,
+                                                                     const T* tt, int64_t ldb,
                                                                      int64_t ldc, int64_t ldd, int64_t ldt, int64_t N,
                                                                      int64_t cols, double* part) {
   kernel_begin();
@@ -463,7 +463,7 @@ __global__ void __launch_bounds__(256, 2) lemma1_partials_vec_kernel(const T* __
 }
 
 // colred[j] = (sum over row blocks of the numerators, of the denominators) of column j
-__global__ void __launch_bounds__(256) lemma1_colred_kernel(const double* __restrict__ part, int row_blocks,
+__global__ void __launch_bounds__(256) lemma1_colred_kernel(const double* part, int row_blocks,
                                                             int64_t cols, double* colred) {
   kernel_begin();
   const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -520,8 +520,8 @@ __global__ void __launch_bounds__(1024) lemma1_finish_kernel(const double* part,
 }
 
 // one warp per row j: cb = <T0[j], W1t[j]>, cc = <T0[j], W10[j]>; s = (cb + cc) / (2 cc)
-__global__ void lemma1_gram_rows_kernel(const float* __restrict__ T0, const float* __restrict__ W1t,
-                                        const float* __restrict__ W10, int64_t n, int64_t d, float* scores) {
+__global__ void lemma1_gram_rows_kernel(const float* T0, const float* W1t,
+                                        const float* W10, int64_t n, int64_t d, float* scores) {
   kernel_begin();
   const int64_t j = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
@@ -677,7 +677,7 @@ __device__ int2 block_excl_scan2(int a, int b, int2* warp_tot, int2* total) {
 // equal scores the lower index first (radix select on order-preserving keys, 8 bits per pass from the top).
 //   scores + b * ld_scores, mask + b * ld_mask, kept_idx + b * ld_idx, tau + b;  k = k_list ? k_list[b] : k_all.
 // The keys are staged once in shared memory when they fit (smem_keys != 0), else re-read from global memory.
-__global__ void __launch_bounds__(1024) topk_select_kernel(const float* __restrict__ scores_all, int64_t ld_scores,
+__global__ void __launch_bounds__(1024) topk_select_kernel(const float* scores_all, int64_t ld_scores,
                                                            int64_t n, int64_t k_all, const int64_t* k_list,
                                                            uint8_t* mask_all, int64_t ld_mask, float* tau_all,
                                                            int32_t* kept_all, int64_t ld_idx, int smem_keys,
@@ -1138,7 +1138,7 @@ __global__ void gsel_init_kernel(int32_t* st, int64_t K, int nblocks) {
   }
 }
 
-__global__ void __launch_bounds__(kGselThreads) gsel_hist_kernel(const float* __restrict__ scores, int64_t n_row,
+__global__ void __launch_bounds__(kGselThreads) gsel_hist_kernel(const float* scores, int64_t n_row,
                                                                  int64_t ld, int64_t total, int pass, int32_t* st) {
   kernel_begin();
   __shared__ int hist[256];
@@ -1183,7 +1183,7 @@ __global__ void __launch_bounds__(kGselThreads) gsel_hist_kernel(const float* __
 }
 
 // per-block counts of keys equal to the threshold key; the last block turns them into exclusive prefixes
-__global__ void __launch_bounds__(kGselThreads) gsel_count_kernel(const float* __restrict__ scores, int64_t n_row,
+__global__ void __launch_bounds__(kGselThreads) gsel_count_kernel(const float* scores, int64_t n_row,
                                                                   int64_t ld, int64_t total, int32_t* st) {
   kernel_begin();
   __shared__ int cnt;
@@ -1219,7 +1219,7 @@ __global__ void __launch_bounds__(kGselThreads) gsel_count_kernel(const float* _
 
 // mask: keys above the threshold key are kept, equal keys in (layer, index) order until the remaining count is used up
 // (a block walks its keys in order: thread t owns a contiguous run).  counts[l] += kept units of layer l.
-__global__ void __launch_bounds__(kGselThreads) gsel_mask_kernel(const float* __restrict__ scores, int64_t n_row,
+__global__ void __launch_bounds__(kGselThreads) gsel_mask_kernel(const float* scores, int64_t n_row,
                                                                  int64_t ld, int64_t ld_mask, int64_t total,
                                                                  const int32_t* st, uint8_t* mask, float* tau,
                                                                  int32_t* counts) {
@@ -1250,22 +1250,30 @@ __global__ void __launch_bounds__(kGselThreads) gsel_mask_kernel(const float* __
   int64_t eq_seen = eq_before_block + base + incl - n_eq;
   int kept_here = 0;
   int64_t cur_layer = i0 < i1 ? i0 / n_row : 0;
-  for (int64_t e = i0; e < i1; ++e) {
-    const int64_t l = e / n_row, j = e % n_row;
-    if (l != cur_layer) {
-      if (kept_here) atomicAdd(&counts[cur_layer], kept_here);
-      kept_here = 0;
-      cur_layer = l;
-    }
-    const float v = scores[l * ld + j];
-    const uint32_t key = score_key(v);
-    const bool is_eq = key == tkey;
-    const bool keep = key > tkey || (is_eq && eq_seen < take_eq);
-    mask[l * ld_mask + j] = (uint8_t)keep;
-    kept_here += keep;
-    if (is_eq) {
-      if (eq_seen == 0 && tau) tau[0] = v != v ? -INFINITY : v;
-      ++eq_seen;
+  for (int64_t e0 = i0; e0 < i1; e0 += 4) {
+    float own[4];                     // (four loads in flight: the loop stores between its entries)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) own[q] = e0 + q < i1 ? scores[((e0 + q) / n_row) * ld + (e0 + q) % n_row] : 0.f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int64_t e = e0 + q;
+      if (e >= i1) break;
+      const int64_t l = e / n_row, j = e % n_row;
+      if (l != cur_layer) {
+        if (kept_here) atomicAdd(&counts[cur_layer], kept_here);
+        kept_here = 0;
+        cur_layer = l;
+      }
+      const float v = own[q];
+      const uint32_t key = score_key(v);
+      const bool is_eq = key == tkey;
+      const bool keep = key > tkey || (is_eq && eq_seen < take_eq);
+      mask[l * ld_mask + j] = (uint8_t)keep;
+      kept_here += keep;
+      if (is_eq) {
+        if (eq_seen == 0 && tau) tau[0] = v != v ? -INFINITY : v;
+        ++eq_seen;
+      }
     }
   }
   if (kept_here) atomicAdd(&counts[cur_layer], kept_here);
@@ -1284,8 +1292,8 @@ __global__ void gsel_repair_list_kernel(int32_t* counts, int L, int64_t min_keep
 }
 
 // counts[l] = kept units of layer l of an L x n mask (rows ld apart); one block per layer
-__global__ void __launch_bounds__(256) mask_row_counts_kernel(const uint8_t* __restrict__ mask, int64_t n, int64_t ld,
-                                                              int32_t* __restrict__ counts) {
+__global__ void __launch_bounds__(256) mask_row_counts_kernel(const uint8_t* mask, int64_t n, int64_t ld,
+                                                              int32_t* counts) {
   kernel_begin();
   __shared__ int sm[256];
   int c = 0;
@@ -1394,7 +1402,7 @@ __global__ void __launch_bounds__(kStripThreads) scale_block_kernel(float* C, in
 }
 
 // inv[perm[i]] = i
-__global__ void invert_perm_kernel(const int32_t* __restrict__ perm, int64_t n, int32_t* __restrict__ inv) {
+__global__ void invert_perm_kernel(const int32_t* perm, int64_t n, int32_t* inv) {
   kernel_begin();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) inv[perm[i]] = (int32_t)i;
@@ -1405,8 +1413,8 @@ __global__ void invert_perm_kernel(const int32_t* __restrict__ perm, int64_t n, 
 // position is the larger are read with the lanes along c, the others along r, so that a warp always reads along a row of
 // Gp and writes along a row of G.  Bound by memory (n = 28672: 9.7 -> 2.1 ms,
 // n = 16384: 2.6 -> 0.7 ms; 64 x 64 tiles are 10 % slower).
-__global__ void __launch_bounds__(256) unpermute_gram_kernel(const float* __restrict__ Gp, const int32_t* __restrict__ inv,
-                                                             int64_t n, float* __restrict__ G) {
+__global__ void __launch_bounds__(256) unpermute_gram_kernel(const float* Gp, const int32_t* inv,
+                                                             int64_t n, float* G) {
   kernel_begin();
   constexpr int TS = 32;
   __shared__ float tile[TS][TS + 1];
@@ -1442,13 +1450,14 @@ __global__ void __launch_bounds__(256) unpermute_gram_kernel(const float* __rest
 }
 
 template <int W>
-__global__ void __launch_bounds__(kStripThreads) unpermute_cols_kernel(const float* __restrict__ Rp,
-                                                                       const int32_t* __restrict__ perm, int64_t rows,
-                                                                       int64_t n, float* __restrict__ R) {
+__global__ void __launch_bounds__(kStripThreads) unpermute_cols_kernel(const float* Rp,
+                                                                       const int32_t* perm, int64_t rows,
+                                                                       int64_t n, float* R) {
   kernel_begin();
   int64_t at[kStripPer];
   strip_index<W>(perm, n, at);
-  for_strip<W>(rows, n, [&](int64_t r, int64_t j, int q) { R[r * n + at[q]] = Rp[r * n + j]; });
+  for_strip_move<W>(rows, n, [&](int64_t r, int64_t j, int) { return Rp[r * n + j]; },
+                    [&](int64_t r, int64_t, int q, float v) { R[r * n + at[q]] = v; });
 }
 
 __global__ void decay_tag_set_kernel(int32_t* tag, int k, float c, int valid, int h_ld, int h_chunk) {
@@ -1466,11 +1475,12 @@ __global__ void h_next_ready_kernel(const int32_t* same, const int32_t* tag, int
 }
 
 template <int W>
-__global__ void __launch_bounds__(kStripThreads) unpermute_rows_kernel(const float* __restrict__ Rp,
-                                                                       const int32_t* __restrict__ perm, int64_t n,
-                                                                       int64_t cols, float* __restrict__ R) {
+__global__ void __launch_bounds__(kStripThreads) unpermute_rows_kernel(const float* Rp,
+                                                                       const int32_t* perm, int64_t n,
+                                                                       int64_t cols, float* R) {
   kernel_begin();
-  for_strip<W>(n, cols, [&](int64_t i, int64_t j, int) { R[(int64_t)perm[i] * cols + j] = Rp[i * cols + j]; });
+  for_strip_move<W>(n, cols, [&](int64_t i, int64_t j, int) { return Rp[i * cols + j]; },
+                    [&](int64_t i, int64_t j, int, float v) { R[(int64_t)perm[i] * cols + j] = v; });
 }
 
 cudaError_t scale_block(float* C, int64_t ld, int64_t rows, int64_t cols, const int32_t* f_bits, int power,

@@ -71,8 +71,8 @@ __device__ __forceinline__ void for_row(int lane, int n, F&& f) {
 // S[row, :] <- softmax over the keys of the row (in place).  rows = pairs * T; row r belongs to query t = r % T; with
 // `causal` keys u > t get probability 0.  Optional bf16 copy.
 template <int NV>
-__global__ void __launch_bounds__(kRowWarps * 32) softmax_rows_kernel(float* __restrict__ S, int64_t rows, int T,
-                                                                      int causal, __nv_bfloat16* __restrict__ Sb,
+__global__ void __launch_bounds__(kRowWarps * 32) softmax_rows_kernel(float* S, int64_t rows, int T,
+                                                                      int causal, __nv_bfloat16* Sb,
                                                                       int64_t plane) {
   kernel_begin();
   const int lane = threadIdx.x & 31;
@@ -97,26 +97,28 @@ __global__ void __launch_bounds__(kRowWarps * 32) softmax_rows_kernel(float* __r
 //   P <- P - eta_b (-2 alpha G1 + 2 beta (P - Phi)),  G1 = R V^T from the preceding product, eta_b per pair.
 // gridDim.y and blockDim.y walk the pairs, a thread takes V neighbouring entries (V = 4: 16-byte accesses).
 template <int V>
-__global__ void __launch_bounds__(256) p_update_kernel(float* __restrict__ P, const float* __restrict__ Phi,
-                                                       const float* __restrict__ G1, const float* __restrict__ eta,
+__global__ void __launch_bounds__(256) p_update_kernel(float* P, const float* Phi, const float* G1, const float* eta,
                                                        int64_t per_pair, int64_t pairs, float alpha, float beta,
-                                                       __nv_bfloat16* __restrict__ Pb, int64_t plane) {
+                                                       __nv_bfloat16* Pb, int64_t plane) {
   kernel_begin();
   struct __align__(4 * V) F { float v[V]; };
   struct __align__(2 * V) H { __nv_bfloat16 v[V]; };
-  for (int64_t b = strip_row(); b < pairs; b += strip_rows()) {
-    const float et = eta[b];
-    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * V; i < per_pair;
-         i += (int64_t)gridDim.x * blockDim.x * V) {
+  struct In { F p, ph, g1; };
+  const int64_t step = strip_rows();
+  for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * V; i < per_pair;
+       i += (int64_t)gridDim.x * blockDim.x * V) {
+    const auto load = [&](int64_t b) {
       const int64_t e = b * per_pair + i;
-      const F p = *reinterpret_cast<const F*>(P + e), ph = *reinterpret_cast<const F*>(Phi + e),
-              g1 = *reinterpret_cast<const F*>(G1 + e);
+      return In{*reinterpret_cast<const F*>(P + e), *reinterpret_cast<const F*>(Phi + e), *reinterpret_cast<const F*>(G1 + e)};
+    };
+    const auto finish = [&](int64_t b, const In& in, float et) {
+      const int64_t e = b * per_pair + i;
       F pn;
       H hi, lo;
 #pragma unroll
       for (int q = 0; q < V; ++q) {
-        const float g = -2.f * alpha * g1.v[q] + 2.f * beta * (p.v[q] - ph.v[q]);
-        pn.v[q] = p.v[q] - et * g;
+        const float g = -2.f * alpha * in.g1.v[q] + 2.f * beta * (in.p.v[q] - in.ph.v[q]);
+        pn.v[q] = in.p.v[q] - et * g;
         hi.v[q] = __float2bfloat16_rn(pn.v[q]);
         lo.v[q] = __float2bfloat16_rn(pn.v[q] - __bfloat162float(hi.v[q]));
       }
@@ -125,6 +127,20 @@ __global__ void __launch_bounds__(256) p_update_kernel(float* __restrict__ P, co
         *reinterpret_cast<H*>(Pb + e) = hi;
         if (plane > 0) *reinterpret_cast<H*>(Pb + plane + e) = lo;
       }
+    };
+    // four pairs at a time: their loads are on their way before the first store
+    for (int64_t b = strip_row(); b < pairs; b += 4 * step) {
+      In x[4];
+      float et[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (b + q * step < pairs) {
+          x[q] = load(b + q * step);
+          et[q] = eta[b + q * step];
+        }
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (b + q * step < pairs) finish(b + q * step, x[q], et[q]);
     }
   }
 }
@@ -132,11 +148,10 @@ __global__ void __launch_bounds__(256) p_update_kernel(float* __restrict__ P, co
 // Softmax and its backward for the softmax term of Eq. (87), one warp per row of logits S:
 //   Phi = softmax(S),  E = Phi - P,  dS = 2 beta Phi (E - sum_u E Phi)  -> as bf16 to dSb, or (dSb == nullptr) in place.
 template <int NV>
-__global__ void __launch_bounds__(kRowWarps * 32) softmax_backward_rows_kernel(float* __restrict__ S,
-                                                                               const float* __restrict__ P,
+__global__ void __launch_bounds__(kRowWarps * 32) softmax_backward_rows_kernel(float* S, const float* P,
                                                                                int64_t rows, int T, int causal,
                                                                                float beta,
-                                                                               __nv_bfloat16* __restrict__ dSb) {
+                                                                               __nv_bfloat16* dSb) {
   kernel_begin();
   const int lane = threadIdx.x & 31;
   const int64_t r = (int64_t)blockIdx.x * kRowWarps + (threadIdx.x >> 5);
@@ -154,21 +169,37 @@ __global__ void __launch_bounds__(kRowWarps * 32) softmax_backward_rows_kernel(f
     dot = fmaf(ph - pu, ph, dot);
   });
   dot = warp_sum(dot);
-  for_row<NV>(lane, T, [&](int u, int i) {
-    float g = 0.f;
-    if (u < lim) {
-      const float ph = v.at(row, lane, i) * inv;
-      g = 2.f * beta * ph * (ph - (NV > 0 ? p[NV > 0 ? i : 0] : prow[u]) - dot);
-    }
+  const auto put = [&](int u, float g) {
     if (dSb) dSb[r * T + u] = __float2bfloat16_rn(g);
     else row[u] = g;
-  });
+  };
+  if constexpr (NV > 0) {
+    for_row<NV>(lane, T, [&](int u, int i) {
+      const float ph = u < lim ? v.at(row, lane, i) * inv : 0.f;
+      put(u, u < lim ? 2.f * beta * ph * (ph - p[i] - dot) : 0.f);
+    });
+  } else {
+    const auto value = [&](int u) {
+      const float ph = __expf(row[u] - v.mx) * inv;
+      return 2.f * beta * ph * (ph - prow[u] - dot);
+    };
+    int u = lane;
+    for (; u + 96 < lim; u += 128) {       // four entries at a time: their loads before the first store
+      float g[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) g[q] = value(u + 32 * q);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) put(u + 32 * q, g[q]);
+    }
+    for (; u < lim; u += 32) put(u, value(u));
+    for (; u < T; u += 32) put(u, 0.f);
+  }
 }
 
 // Sum of squares of the [T, d_h] slice of every (sequence, head) pair of up to two token-major [tokens, d] tensors;
 // one block per pair, fixed summation order.  out[b] = sum x^2 (+ sum y^2), b = seq * H + head.
-__global__ void __launch_bounds__(256) pair_sumsq_kernel(const float* __restrict__ x, const float* __restrict__ y,
-                                                         int64_t ld, int T, int d_h, int H, double* __restrict__ out) {
+__global__ void __launch_bounds__(256) pair_sumsq_kernel(const float* x, const float* y,
+                                                         int64_t ld, int T, int d_h, int H, double* out) {
   kernel_begin();
   __shared__ double sm[256];
   const int b = blockIdx.x, seq = b / H, head = b % H;
@@ -204,8 +235,8 @@ __global__ void __launch_bounds__(256) pair_sumsq_kernel(const float* __restrict
 
 // Step sizes from the sums above: mode 0 (Eq. 85): eta = 1 / (2 (alpha s + beta));
 // mode 1 (Eq. 87): eta = eta_z / (2 alpha + beta s / d_h).
-__global__ void step_size_kernel(const double* __restrict__ s, int n, int mode, double alpha, double beta, double eta_z,
-                                 int d_h, float* __restrict__ eta) {
+__global__ void step_size_kernel(const double* s, int n, int mode, double alpha, double beta, double eta_z,
+                                 int d_h, float* eta) {
   kernel_begin();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= n) return;
@@ -218,12 +249,10 @@ __global__ void step_size_kernel(const double* __restrict__ s, int n, int mode, 
 // optional bf16 hi / lo planes of the new values (operands of the next logits product).  A thread takes V neighbouring
 // columns of one head (V = 4: 16-byte accesses).
 template <int V>
-__global__ void __launch_bounds__(256) z_update_kernel(float* __restrict__ Zq, float* __restrict__ Zk,
-                                                       const float* __restrict__ Gq, const float* __restrict__ Gk,
-                                                       const float* __restrict__ Tq, const float* __restrict__ Tk,
-                                                       const float* __restrict__ eta, int64_t tokens, int d, int T,
-                                                       int d_h, float alpha, __nv_bfloat16* __restrict__ Zqs,
-                                                       __nv_bfloat16* __restrict__ Zks, int64_t plane) {
+__global__ void __launch_bounds__(256) z_update_kernel(float* Zq, float* Zk, const float* Gq, const float* Gk,
+                                                       const float* Tq, const float* Tk, const float* eta, int64_t tokens, int d, int T,
+                                                       int d_h, float alpha, __nv_bfloat16* Zqs,
+                                                       __nv_bfloat16* Zks, int64_t plane) {
   kernel_begin();
   struct __align__(4 * V) F { float v[V]; };
   struct __align__(2 * V) B { __nv_bfloat16 v[V]; };
@@ -233,9 +262,8 @@ __global__ void __launch_bounds__(256) z_update_kernel(float* __restrict__ Zq, f
   for (int64_t tok = strip_row(); tok < tokens; tok += strip_rows()) {
     const int64_t e = tok * d + c;
     const float et = eta[(tok / T) * H + head];
-    const auto step = [&](float* Z, const float* G, const float* Tg, __nv_bfloat16* S) {
-      const F z = *reinterpret_cast<const F*>(Z + e), g = *reinterpret_cast<const F*>(G + e),
-              t = *reinterpret_cast<const F*>(Tg + e);
+    const auto in = [&](const float* p) { return *reinterpret_cast<const F*>(p + e); };
+    const auto step = [&](const F& z, const F& g, const F& t, float* Z, __nv_bfloat16* S) {
       F n;
       B hi, lo;
 #pragma unroll
@@ -250,48 +278,66 @@ __global__ void __launch_bounds__(256) z_update_kernel(float* __restrict__ Zq, f
         *reinterpret_cast<B*>(S + plane + e) = lo;
       }
     };
-    step(Zq, Gq, Tq, Zqs);
-    step(Zk, Gk, Tk, Zks);
+    const F zq = in(Zq), gq = in(Gq), tq = in(Tq), zk = in(Zk), gk = in(Gk), tk = in(Tk);   // (all on their way before a store)
+    step(zq, gq, tq, Zq, Zqs);
+    step(zk, gk, tk, Zk, Zks);
   }
 }
 
 // hi / lo bf16 planes of a dense fp32 tensor of `total` elements: dst[e] = bf16(x), dst[plane + e] = bf16(x - hi).
-__global__ void __launch_bounds__(256) split_planes_kernel(const float* __restrict__ x, int64_t total,
-                                                           __nv_bfloat16* __restrict__ dst, int64_t plane) {
+__global__ void __launch_bounds__(256) split_planes_kernel(const float* x, int64_t total,
+                                                           __nv_bfloat16* dst, int64_t plane) {
   kernel_begin();
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    const float v = x[e];
-    const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-    dst[e] = hi;
-    if (plane > 0) dst[plane + e] = __float2bfloat16_rn(v - __bfloat162float(hi));
+  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t e0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e0 < total; e0 += 4 * step) {
+    float v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] = e0 + q * step < total ? x[e0 + q * step] : 0.f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int64_t e = e0 + q * step;
+      if (e >= total) break;
+      const __nv_bfloat16 hi = __float2bfloat16_rn(v[q]);
+      dst[e] = hi;
+      if (plane > 0) dst[plane + e] = __float2bfloat16_rn(v[q] - __bfloat162float(hi));
+    }
   }
 }
 
 // bf16 hi / lo planes of the selected heads' [T, T] blocks: grid (pieces of a block, slots, sequences), 16-byte reads.
-__global__ void __launch_bounds__(256) split_heads_kernel(const float* __restrict__ P, int64_t n_seq, int64_t H, int64_t per_pair,
+__global__ void __launch_bounds__(256) split_heads_kernel(const float* P, int64_t n_seq, int64_t H, int64_t per_pair,
                                                           const __grid_constant__ HeadList heads,
-                                                          __nv_bfloat16* __restrict__ dst, int64_t plane) {
+                                                          __nv_bfloat16* dst, int64_t plane) {
   kernel_begin();
   struct __align__(8) B { __nv_bfloat162 v[2]; };
   for (int64_t seq = blockIdx.z; seq < n_seq; seq += gridDim.z) {
     const float* src = P + (seq * H + heads.h[blockIdx.y]) * per_pair;
     __nv_bfloat16* out = dst + (seq * gridDim.y + blockIdx.y) * per_pair;
-    for (int64_t e = ((int64_t)blockIdx.x * 256 + threadIdx.x) * 4; e < per_pair; e += (int64_t)gridDim.x * 1024) {
-      const float4 x = *reinterpret_cast<const float4*>(src + e);
-      B hi, lo;
-      hi.v[0] = __floats2bfloat162_rn(x.x, x.y);
-      hi.v[1] = __floats2bfloat162_rn(x.z, x.w);
-      lo.v[0] = __floats2bfloat162_rn(x.x - __low2float(hi.v[0]), x.y - __high2float(hi.v[0]));
-      lo.v[1] = __floats2bfloat162_rn(x.z - __low2float(hi.v[1]), x.w - __high2float(hi.v[1]));
-      *reinterpret_cast<B*>(out + e) = hi;
-      *reinterpret_cast<B*>(out + plane + e) = lo;
+    const int64_t step = (int64_t)gridDim.x * 1024;
+    for (int64_t e0 = ((int64_t)blockIdx.x * 256 + threadIdx.x) * 4; e0 < per_pair; e0 += 4 * step) {
+      float4 x[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (e0 + q * step < per_pair) x[q] = *reinterpret_cast<const float4*>(src + e0 + q * step);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int64_t e = e0 + q * step;
+        if (e >= per_pair) break;
+        B hi, lo;
+        hi.v[0] = __floats2bfloat162_rn(x[q].x, x[q].y);
+        hi.v[1] = __floats2bfloat162_rn(x[q].z, x[q].w);
+        lo.v[0] = __floats2bfloat162_rn(x[q].x - __low2float(hi.v[0]), x[q].y - __high2float(hi.v[0]));
+        lo.v[1] = __floats2bfloat162_rn(x[q].z - __low2float(hi.v[1]), x[q].w - __high2float(hi.v[1]));
+        *reinterpret_cast<B*>(out + e) = hi;
+        *reinterpret_cast<B*>(out + plane + e) = lo;
+      }
     }
   }
 }
 
 // The selected heads' columns of a token-major tensor as hi / lo parts: grid (tokens, slots)
-__global__ void split_head_cols_kernel(const float* __restrict__ A, int64_t tokens, int64_t d, int d_h,
-                                       const __grid_constant__ HeadList heads, __nv_bfloat16* __restrict__ dst, int64_t ld,
+__global__ void split_head_cols_kernel(const float* A, int64_t tokens, int64_t d, int d_h,
+                                       const __grid_constant__ HeadList heads, __nv_bfloat16* dst, int64_t ld,
                                        int64_t lo_off) {
   kernel_begin();
   const int per_block = blockDim.x / d_h > 0 ? blockDim.x / d_h : 1;
@@ -308,7 +354,7 @@ __global__ void split_head_cols_kernel(const float* __restrict__ A, int64_t toke
   }
 }
 
-__global__ void __launch_bounds__(1024) add_ridge_batched_kernel(float* __restrict__ G, int64_t bs, int64_t n, double rho,
+__global__ void __launch_bounds__(1024) add_ridge_batched_kernel(float* G, int64_t bs, int64_t n, double rho,
                                                                  int rel) {
   kernel_begin();
   __shared__ double sm[32];
@@ -329,13 +375,20 @@ __global__ void __launch_bounds__(1024) add_ridge_batched_kernel(float* __restri
   for (int64_t i = threadIdx.x; i < n; i += blockDim.x) G[i * n + i] = (float)((double)G[i * n + i] + r);
 }
 
-__global__ void __launch_bounds__(256) place_heads_kernel(const float* __restrict__ src, int64_t bs, int64_t d,
-                                                          const __grid_constant__ HeadList heads, float* __restrict__ W,
+__global__ void __launch_bounds__(256) place_heads_kernel(const float* src, int64_t bs, int64_t d,
+                                                          const __grid_constant__ HeadList heads, float* W,
                                                           int64_t ldw) {
   kernel_begin();
   const float* in = src + (int64_t)blockIdx.y * bs + (int64_t)blockIdx.x * d;
   float* out = W + ((int64_t)heads.h[blockIdx.y] * gridDim.x + blockIdx.x) * ldw;
-  for (int64_t c = threadIdx.x; c < d; c += 256) out[c] = in[c];
+  for (int64_t c = threadIdx.x; c < d; c += 1024) {
+    float v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] = c + 256 * q < d ? in[c + 256 * q] : 0.f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (c + 256 * q < d) out[c + 256 * q] = v[q];
+  }
 }
 
 template <typename T>
