@@ -192,10 +192,8 @@ bool make_assist(SolveAssist& a) {
          cudaEventCreateWithFlags(&a.rest_done[0], cudaEventDisableTiming) == cudaSuccess &&
          cudaEventCreateWithFlags(&a.rest_done[1], cudaEventDisableTiming) == cudaSuccess &&
          cudaEventCreateWithFlags(&a.near_done, cudaEventDisableTiming) == cudaSuccess &&
-         cudaEventCreateWithFlags(&a.next_done, cudaEventDisableTiming) == cudaSuccess &&
          cudaStreamCreateWithFlags(&a.far_stream, cudaStreamNonBlocking) == cudaSuccess &&
          cudaEventCreateWithFlags(&a.far_go, cudaEventDisableTiming) == cudaSuccess &&
-         cudaEventCreateWithFlags(&a.far_first, cudaEventDisableTiming) == cudaSuccess &&
          cudaEventCreateWithFlags(&a.far_done[0], cudaEventDisableTiming) == cudaSuccess &&
          cudaEventCreateWithFlags(&a.far_done[1], cudaEventDisableTiming) == cudaSuccess;
 }

@@ -328,8 +328,8 @@ __device__ __forceinline__ void cluster_meet() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// Where the rows of Lm go: they are the first rows of the panel of this block column, which therefore starts below them
-// and need not wait for this kernel.  (A21 has all 128 columns: only the last block of a matrix is narrower.)
+// Where the rows of Lm go: they are the first rows of the panel of this block column, whose own kernel therefore starts below
+// them.  (A21 has all 128 columns: only the last block of a matrix is narrower.)
 struct NextRows {
   __nv_bfloat16* P;      // parts at P[i * ldp + part * seg + c]
   int64_t ldp, seg;
@@ -498,7 +498,7 @@ sp_status potrf_lower_tc(float* A, int64_t n, int64_t lda, float* dinv, void* Pv
   // Far part of a step's trailing update on a stream of its own: it adds into the matrix through the GEMM's atomic TMA
   // reduction (which needs 16-byte aligned rows and a width that is a multiple of 4).  What must see it complete waits for its
   // events: the lookahead kernel of step kb reads block (kb+1, kb+1), last touched by the far update of step kb - 2, and
-  // the near update of step kb adds to a block column that the far update of step kb - 1 has among its first two.
+  // the near update of step kb adds to the first block column of the far update of step kb - 1.
   // The far GEMM leaves a few SM pairs to the kernels of the chain, which would otherwise wait for its tiles to end.
   const bool far_apart = assist && assist->far_stream && n % 4 == 0 && lda % 4 == 0 &&
                          (reinterpret_cast<uintptr_t>(A) & 15u) == 0 && !reproducible_mode();
@@ -547,10 +547,6 @@ sp_status potrf_lower_tc(float* A, int64_t n, int64_t lda, float* dinv, void* Pv
     // rows of the panel that the lookahead kernel takes: the next diagonal block's
     const int64_t ahead = assist && rem > 0 && !inner_last ? (rem < TB ? rem : TB) : 0;
     if (assist && rem > 0) {
-      // the panel needs the diagonal block alone (its rows are disjoint from those of the lookahead kernel)
-      SP_CUDA_OK(cudaEventRecord(assist->panel_done, stream));
-      sb = assist->stream;
-      SP_CUDA_OK(cudaStreamWaitEvent(sb, assist->panel_done, 0));
       if (ahead > 0) {
         // next diagonal block: it reads blocks (kb+1, kb) and (kb+1, kb+1), i.e. the first two block columns of the
         // trailing update of step kb - 1, which that step issues first and signals on their own
@@ -571,8 +567,14 @@ sp_status potrf_lower_tc(float* A, int64_t n, int64_t lda, float* dinv, void* Pv
           launch(chol_next_diag_stage2_kernel, NM_CTAS, NM_THREADS, NM_SMEM, stream, A21 + nb, lda, nb2, LmT, S, skip);
         }
         if (cudaGetLastError() != cudaSuccess) return SP_ERR_CUDA;
-        SP_CUDA_OK(cudaEventRecord(assist->next_done, stream));
       }
+      // The panel needs the diagonal block alone, but it starts behind the lookahead kernel: the next diagonal block waits for
+      // that one, and beside it the panel's CTAs would be in its way (its cluster needs eight SMs that have room at once).
+      // Panel behind / beside it: a solve of 4096 unknowns and 1024 right-hand sides 1.71 / 1.86 ms, of 2048 and 4096 1.04 /
+      // 1.17, an ADMM step 2048 x 8192 14.10 / 14.27, 1096 x 4376 and 768 x 3072 equal within 1 %.
+      SP_CUDA_OK(cudaEventRecord(assist->panel_done, stream));
+      sb = assist->stream;
+      SP_CUDA_OK(cudaStreamWaitEvent(sb, assist->panel_done, 0));
     }
     // L21 = A21 inv(L11)^T, fp32 in place and as bf16 parts in P[k0+nb.., part * np + k0 ..]
     const int64_t p0 = k0 + nb + ahead;
@@ -581,10 +583,9 @@ sp_status potrf_lower_tc(float* A, int64_t n, int64_t lda, float* dinv, void* Pv
       return SP_ERR_CUDA;
     if (rem <= 0) break;     // last block: the appended rows are done, nothing is left to update
     if (far_apart && !outer && rem > 2 * TB) SP_CUDA_OK(cudaEventRecord(assist->far_go, sb));   // the panel's parts exist
-    if (ahead > 0) SP_CUDA_OK(cudaStreamWaitEvent(sb, assist->next_done, 0));    // so do the rows of the lookahead kernel
     // the far update of the step before has added to the columns that this step's near update adds to: every entry receives
     // its updates in step order, whatever the streams' timing
-    if (kb >= 1 && far_rec[(kb - 1) & 1]) SP_CUDA_OK(cudaStreamWaitEvent(sb, assist->far_first, 0));
+    if (kb >= 1 && far_rec[(kb - 1) & 1]) SP_CUDA_OK(cudaStreamWaitEvent(sb, assist->far_done[(kb - 1) & 1], 0));
     // A22 -= L21 L21^T on the lower triangle
     TcOperand ta{P + (k0 + nb) * ldp, ldp, true}, tb{P + (k0 + nb) * ldp, ldp, true};
     ta.kext = tb.kext = ldp;
@@ -656,23 +657,17 @@ sp_status potrf_lower_tc(float* A, int64_t n, int64_t lda, float* dinv, void* Pv
         sf = assist->far_stream;
         SP_CUDA_OK(cudaStreamWaitEvent(sf, assist->far_go, 0));
       }
-      // (first the two block columns that the next step waits for, where the whole takes more than two rounds of tiles)
-      const int64_t fw = rem - kNear;
-      const int64_t cut = far_apart && fw > kNear &&
-                                  ceil_div(fw, (int64_t)256) * ceil_div(prow - kNear, (int64_t)256) > 4 * kFarPairs ? kNear : fw;
-      for (int64_t c0 = 0; c0 < fw; c0 = c0 == 0 ? cut : fw) {
-        const int64_t w = c0 == 0 ? cut : fw - c0, r0 = k0 + nb + kNear + c0, rows_f = prow - kNear - c0;
-        TcOperand fa{P + r0 * ldp, ldp, true}, fb{P + r0 * ldp, ldp, true};
-        fa.kext = fb.kext = ldp;
-        fa.mnext = rows_f;
-        fb.mnext = w;
-        float* Afar = A + r0 * lda + r0;
-        st = gemm_tc(rows_f, w, TB, -1.f, fa, fb, 1.f, Operand{Afar, SP_F32, lda, 1}, OutOperand{Afar, SP_F32, lda}, true,
-                     status_dev, sf, &sg, (double)w * (2.0 * (double)rows_f - (double)w) * (double)nb,
-                     far_apart ? kFarPairs : 0);
-        if (st != SP_OK) return st;
-        if (far_apart && c0 == 0) SP_CUDA_OK(cudaEventRecord(assist->far_first, sf));
-      }
+      // (one launch: as two, the block columns that the next near update waits for first, it fills the SMs worse, and a solve of
+      // 8192 unknowns takes 6.35 instead of 6.04 ms)
+      const int64_t fw = rem - kNear, r0 = k0 + nb + kNear, rows_f = prow - kNear;
+      TcOperand fa{P + r0 * ldp, ldp, true}, fb{P + r0 * ldp, ldp, true};
+      fa.kext = fb.kext = ldp;
+      fa.mnext = rows_f;
+      fb.mnext = fw;
+      float* Afar = A + r0 * lda + r0;
+      st = gemm_tc(rows_f, fw, TB, -1.f, fa, fb, 1.f, Operand{Afar, SP_F32, lda, 1}, OutOperand{Afar, SP_F32, lda}, true,
+                   status_dev, sf, &sg, (double)fw * (2.0 * (double)rows_f - (double)fw) * (double)nb, far_apart ? kFarPairs : 0);
+      if (st != SP_OK) return st;
       if (far_apart) {
         SP_CUDA_OK(cudaEventRecord(assist->far_done[kb & 1], sf));
         far_rec[kb & 1] = true;
