@@ -6,7 +6,7 @@ import pytest
 import torch
 
 from oracle import struprune_oracle as O
-from paper_2510_03246_b200 import api, synth
+from paper_2510_03246_b200 import api, pipeline, synth
 from tests._util import TOL, bf16_half_ulp, np64, relerr
 
 pytestmark = pytest.mark.gpu
@@ -258,3 +258,18 @@ def test_mha_value_refit_argument_errors():
     rc = api.lib().sp_mha_value_refit(C.byref(m), C.byref(st), None, 0.1, 1, 0, mod.Wv.data_ptr(), mod.d - 8,
                                       mod.status.data_ptr(), mod._wsbuf.data_ptr(), mod._wsbuf.numel(), None)
     assert rc == 2                                   # SP_ERR_SHAPE: leading dimension below d
+
+
+@pytest.mark.parametrize("d,H", [(256, 4), (2560, 20)])
+def test_recoveries_of_wq_and_wk_are_those_of_each_by_itself(d, H):
+    """One factorisation for both, or (2560 wide, where both together are more right-hand sides than a backward sweep takes in a
+    fixed order) one for each: the same bits as a recovery by itself either way."""
+    X, W = _case(torch.bfloat16, d, H, 16, 2)
+    mod = api.MhaModule(X.to(DEV), *[w.to(DEV) for w in W], n_heads=H, T=16)
+    mod.sp_mha_init(True)
+    ref = [api.sp_ridge_solve(R, mod.G_X, 0.1).clone() for R in (mod.R_Q, mod.R_K)]
+    keep = torch.arange(H, device=DEV) % 2 == 0
+    mod = pipeline.mha_outer_iterations(mod, keep.to(torch.uint8), 1, api.MhaParams(a_steps=1, z_steps=1), rho=0.1, recover_wv=False)
+    rows = keep.repeat_interleave(d // H)
+    for got, want in zip((mod.Wq, mod.Wk), ref):
+        assert torch.equal(got[rows], want[rows]) and torch.all(got[~rows] == 0)
