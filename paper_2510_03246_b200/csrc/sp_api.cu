@@ -845,7 +845,8 @@ static sp_status admm_step_impl(const sp_ffn_module* m, sp_ffn_state* st, const 
   // runs on the side stream while the caller's stream carries the W2 chain.
   SideStream* side = side_stream();
   cudaStream_t sa = side ? side->stream : s;
-  const OverlapScope overlap(std::max(n, d) <= kOverlapMaxN);
+  const bool narrow = std::max(n, d) <= kOverlapMaxN;
+  const OverlapScope overlap(narrow);
   JoinOnExit join_guard{side, s};
   // Reuse of the factorisation for the recovery on the kept support (tensor-core path): the unrestricted system is
   // solved with the channels that the mask kept so far in front.  The leading block of that factor is the factor of
@@ -1044,6 +1045,7 @@ static sp_status admm_step_impl(const sp_ffn_module* m, sp_ffn_state* st, const 
   if (rep_dev && prm->compute_objective && bf16) CU(convert_matrix(st->W2, SP_F32, n, p.W2fb, SP_BF16, n, d, n, s));
 
   // ---- 5b. token pass
+  const OverlapScope overlap_tokens(narrow && p.chunk * n <= kOverlapMaxChunk);
   // Pruned channels (ReLU, no dual variable): a = phi(z) and z_new = c max(z, 0) with c = beta / (alpha + beta), so
   // from the second step with an unchanged mask on their rows of A are c times those of the step before.  The
   // accumulators are therefore built in "kept channels first" order in buffers that persist in the state: the kept
@@ -1279,7 +1281,9 @@ sp_status bcontract(int64_t M, int64_t N, int64_t K, double alpha, BMat A, bool 
   return SP_OK;
 }
 
-constexpr int64_t kOverlapMaxPairs = int64_t(1) << 24;     // T x T entries of a chunk up to which its kernels are short
+// T x T entries of a chunk up to which the attention step's launches carry the attribute (see OverlapScope).  Off / on: 1.6 M entries
+// 1.30 / 1.18 ms a step, 8.4 M 1.31 / 1.26, 16.8 M 2.73 / 2.63, 67 M 4.24 / 4.22 (512 tokens) and 5.08 / 5.23 (1024 tokens), 268 M 9.41 / 9.64.
+constexpr int64_t kOverlapMaxPairs = int64_t(1) << 24;
 
 struct MhaPlan {
   int64_t d, H, T, dh, sc, cap;   // cap = tokens of a full chunk

@@ -94,9 +94,8 @@ __host__ __device__ __forceinline__ size_t align_up(size_t a, size_t b) { return
 // behind the wait (it clobbers memory) and are coherent, but they stay behind the stores before them too: loads that are to be
 // in flight together stand before the first store of a round (for_strip_move; split_planes 90 -> 140 us where they do not).
 // The attribute is given inside an OverlapScope only, which the entry points open for calls whose kernels are short: their
-// time is launches and gaps (attention step 768 wide, 284 kernels: 2.68 -> 2.42 ms; ADMM step 768 x 3072 2.40 -> 2.28).  Long
-// kernels lose: waiting blocks hold SMs that another stream's kernels could use (ADMM step of 2048 x 8192 on 262144 tokens: 49.3
-// -> 51.4 ms).
+// time is launches and gaps (attention step 768 wide, 284 kernels: 2.68 -> 2.42 ms; ADMM step 768 x 3072 2.27 -> 2.11).  Long
+// kernels lose: waiting blocks hold SMs that another stream's kernels could use.
 __device__ __forceinline__ void dependents_may_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_for_predecessors() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void kernel_begin() {
@@ -110,8 +109,18 @@ struct OverlapScope {
   ~OverlapScope() { overlap_flag() = saved; }
   OverlapScope(const OverlapScope&) = delete;
 };
-constexpr int64_t kOverlapMaxN = 4608;        // widest module whose step is launches and gaps for the most part
-constexpr int64_t kOverlapMaxSolve = 1024;    // the same for a solve of its own
+// Weight phase of an ADMM step (and the cached input inverse): modules up to this width.  Its gain falls with the width, whatever the
+// token count: 768 x 3072 on 32768 tokens 3.09 -> 2.88 ms, 1096 x 4376 on 65536 tokens 7.40 -> 7.06, 1280 x 5120 on 8192 tokens
+// 4.78 -> 4.62, 2048 x 8192 on 32768 tokens 14.30 -> 14.06, 3072 x 9216 and 4096 x 11008 less than their runs differ.  Wider
+// modules keep plain launches.
+constexpr int64_t kOverlapMaxN = 4608;
+// Token pass of such a step: chunks of up to this many entries of Z.  Attribute off / on: 6.3 M entries 2.14 / 2.11 ms a step, 12.6 M
+// 2.20 / 2.17, 25 and 33 M equal, 38 M 2.38 / 2.40, 50 M 2.48 / 2.52, 101 M in eight chunks 9.4 / 10.7.
+constexpr int64_t kOverlapMaxChunk = int64_t(1) << 25;
+// Recoveries by themselves (sp_ridge_solve, sp_linear_refit): matrices up to this width, of which a refit solves a part.  On
+// this side 1.05 (1024 unknowns, 2048 right-hand sides: 0.401 -> 0.382 ms) to 1.17 (384 of 768: 0.155 -> 0.132).  Wider ones keep
+// plain launches; that is not a measured line: they ran with the attribute in the passes among which one stood still.
+constexpr int64_t kOverlapMaxSolve = 1024;
 inline bool may_overlap_launches(cudaStream_t stream) {
   if (!overlap_flag()) return false;
   cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
