@@ -23,14 +23,19 @@
  *       fp32 mode: contractions run in fp32 storage with fp64 accumulation; linear systems are factorised in fp64.
  *   - Return value: SP_OK or an error detected on the host before any launch (argument / shape / alignment /
  *     workspace errors).  Numerical failures found on the device (non-positive Cholesky pivot, a bounded wait that
- *     ran out) are written to the caller's `status_dev[4]` = {code, index, aux, 0}; nothing traps or spins forever.
+ *     ran out) are written to the caller's `status_dev[4]` = {code, index, aux, 0}; nothing traps, and no kernel spins on
+ *     memory that another kernel writes.  A kernel's waits for its own copies, matrix instructions and warps have a clock
+ *     budget; those for the other CTAs of its cluster, for tensor memory and for the kernels before it on its stream do not.
  *   - Streams: a call is ordered on the caller's stream, but sp_admm_step, sp_admm_scores, sp_mha_value_refit and
  *     (precise == 0) sp_ridge_solve and sp_linear_refit also fork independent parts (the two weight recoveries, the
  *     panels and trailing updates of a factorisation, the z^(1) products) onto a few streams and events that the
  *     library creates once per device and joins back to the caller's stream with events before the call's results are
  *     used (also when a call returns an error after the fork).  That set is shared by all these calls on a device: issue
  *     them from one host thread at a time.  All other calls, sp_ffn_cache_input_inverse and the precise solves among
- *     them, use the caller's stream alone.  Nothing else persists inside the library.
+ *     them, use the caller's stream alone.  Nothing else persists inside the library.  Calls on small modules launch their
+ *     kernels with programmatic dependent launches (a kernel's blocks may start before its predecessor on the stream
+ *     has ended, and wait for it); on a stream that is being captured all launches are plain ones, so a captured call
+ *     replays without that overlap.
  *   - Reproducibility: by default a product whose tile count leaves SMs idle is cut along K and its partial
  *     products add up in C in an order that is not fixed, and a backward sweep with more right-hand sides than one wave of its
  *     panels holds adds updates from two streams (a factorisation takes its updates in step order); fp32 results

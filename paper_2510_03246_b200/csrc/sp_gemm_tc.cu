@@ -19,10 +19,14 @@
 // leader, MMA issuer (one lane), warps 2..5 = epilogue (each owns the 32 accumulator lanes its warp id maps to).  Two
 // 256-column accumulators are ping-ponged so that the epilogue of tile i overlaps the main loop of tile i+1.
 // Epilogue: the accumulator block of a warp (32 rows x 32 columns) goes through a 128-byte-swizzled shared tile and
-// leaves by a TMA store, or a TMA add-reduction when the call accumulates into C; other cases (bf16 output, a
-// separate Cin, unaligned C) use plain coalesced loads and stores through a padded tile.
-// Every wait is bounded by a clock budget; on expiry the CTA records SP_ERR_TIMEOUT and leaves its loops, and both
-// CTAs still meet at the final cluster barrier before tensor memory is freed.
+// leaves by a TMA store, or a TMA add-reduction when the call accumulates into C; bf16 results, one part or hi and lo
+// parts, by TMA stores as well, with or without a bf16 Cin.  Other cases (another separate Cin, unaligned C) use plain
+// coalesced loads and stores through a padded tile.
+// Every wait of a role for copies, for the tensor core or for another role is bounded by a clock budget; on expiry the CTA
+// records SP_ERR_TIMEOUT and leaves its loops, and both CTAs still meet at the final cluster barrier before tensor memory is
+// freed.  Not bounded, since what they wait for cannot stay away: the two cluster barriers (the CTAs of a pair start together
+// and both reach them on every path), the allocation of tensor memory (the shared memory of a CTA keeps every other CTA of
+// this kernel off its SM, and no other kernel allocates any), and the wait for the kernels before this one.
 #include <cuda.h>
 #include <math.h>
 #include <string.h>

@@ -311,8 +311,6 @@ cudaError_t launch_panel_apply(float* X, int64_t ldx, int64_t rows, int nb, cons
   return launch_panel_rows<TRANS, 32>(X, ldx, rows, nb, dinv, S, lds, s_seg, write_f32, status, stream, near, batch, pb);
 }
 
-// The six kept part products of two three-part operands: A parts (hi, hi, mid, hi, lo, mid) against B parts
-// (hi, mid, hi, lo, hi, mid).
 // ---------------------------------------------------------------------------------------------------------------
 // Lookahead of the factorisation: the NEXT diagonal block, updated with the block column just factored, in one small
 // launch, so that its factorisation does not wait for the full panel and the trailing update:
@@ -324,6 +322,7 @@ constexpr int NM_ROWS = 16, NM_THREADS = RowTile<NM_ROWS>::THREADS, NM_CTAS = TB
 constexpr size_t NM_SMEM = ((size_t)TB * TB + (size_t)TB * RowTile<NM_ROWS>::AP) * sizeof(float) + 16;
 static_assert(NM_CTAS == 8, "one portable cluster covers the block");
 
+// (no time limit: the CTAs of a cluster start together and each reaches the barrier, also after a wait that ran out)
 __device__ __forceinline__ void cluster_meet() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
@@ -460,6 +459,8 @@ __global__ void __launch_bounds__(NM_THREADS)
   next_diag_body<2>(nullptr, A22, lda, nb2, nullptr, LmT, S, NextRows{}, nullptr);
 }
 
+// The six kept part products of two three-part operands: A parts (hi, hi, mid, hi, lo, mid) against B parts
+// (hi, mid, hi, lo, hi, mid).
 constexpr int kPartA[6] = {0, 0, 1, 0, 2, 1};
 constexpr int kPartB[6] = {0, 1, 0, 2, 0, 1};
 
