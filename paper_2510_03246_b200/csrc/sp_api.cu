@@ -114,6 +114,7 @@ struct SolveBufs {
   double* rho;  // [4] device scalars
   void* P;      // fp32 path: bf16 parts of the Cholesky factor
   void* Xs;     // fp32 path: bf16 parts of one block column of right-hand sides
+  SolveOneBufs one;   // fp32 path, solves in one launch: P as above, and its small arrays
 };
 
 SolveBufs carve_solve(Carver& c, int64_t nmax, int64_t mmax, size_t tsize) {
@@ -125,29 +126,35 @@ SolveBufs carve_solve(Carver& c, int64_t nmax, int64_t mmax, size_t tsize) {
   b.dinv = c.take_bytes(dinv_elems(nmax) * tsize);
   b.P = nullptr;
   b.Xs = nullptr;
+  b.one = SolveOneBufs{nullptr, nullptr, nullptr};
   if (tsize == 4) {
     const size_t np = (size_t)chol_tc_pad(nmax);
-    b.P = c.take_bytes((np + (size_t)mmax) * 3 * np * 2);
+    b.P = c.take_bytes((np + (size_t)chol_tc_pad(mmax)) * 3 * np * 2);
     const size_t rows = (size_t)(nmax > mmax ? nmax : mmax);   // either dimension may be the right-hand-side count
     b.Xs = c.take_bytes((size_t)chol_tc_xs_elems(nmax, (int64_t)rows) * 2);
+    b.one.P = b.P;
+    b.one.Y = c.take_bytes((size_t)chol_tc_pad((int64_t)rows) * 3 * kCholTcNB * 2);
+    b.one.flags = c.take<uint32_t>(solve_tc_flag_words(nmax, (int64_t)rows));
   }
   return b;
 }
 
-// Copy of the forward-substituted right-hand sides on the leading k columns of a system (tensor-core path): with it
-// and the factor's leading block the system restricted to its first k unknowns is solved by a backward sweep alone.
+// What a solve leaves for the system restricted to its first k unknowns (tensor-core path): solves in one launch its solution,
+// others a copy of the forward-substituted right-hand sides, with which and the factor's leading block a backward sweep
+// alone solves it.
 struct LeadSave {
   float* Y;       // [m, kpad] dense, columns k..kpad zero
   int64_t k, kpad;
 };
 
 // W[m, n_full] = R[:, idx] (G[idx, idx] + rho I)^-1 scattered back to the idx columns (idx == nullptr: identity).
-// conditional: the call runs under a SkipScope (its work is not counted in the profile's flops).
+// conditional: the call runs under a SkipScope (its work is not counted in the profile's flops).  one_launch: by solve_tc where
+// solve_in_one() says so.
 template <typename T>
 sp_status ridge_core(const float* R, int64_t ldr, const float* G, int64_t ldg, int64_t m, int64_t n_full,
                      const int32_t* idx, int64_t k, const double* rho_dev, float* W, int64_t ldw, SolveBufs& b,
                      int32_t* status, cudaStream_t stream, const SolveAssist* assist = nullptr,
-                     bool split_lookahead = false, const LeadSave* save = nullptr, bool conditional = false) {
+                     bool split_lookahead = false, const LeadSave* save = nullptr, bool conditional = false, bool one_launch = true) {
   const int64_t nn = idx ? k : n_full;
   ProfScope prof(PK_SOLVE, conditional ? 0.0 : (double)nn * nn * nn / 3.0 + 2.0 * (double)m * nn * nn, 0.0, stream);
   T* Gs = reinterpret_cast<T*>(b.Gs);
@@ -159,9 +166,14 @@ sp_status ridge_core(const float* R, int64_t ldr, const float* G, int64_t ldg, i
     // the right-hand sides ride through the factorisation as m more rows (their forward substitution); the solve
     // proper is then only the backward sweep
     CU(gather_cols<T>(R, ldr, idx, m, nn, Rs, nn, stream));
-    SPCHK(potrf_lower_tc(Gs, nn, nn, dinv, b.P, status, stream, assist, m, split_lookahead));
-    if (save) CU(copy_cols_padded(Rs, nn, m, save->k, save->kpad, save->Y, stream));
-    SPCHK(potrs_right_tc(Rs, m, nn, nn, b.P, dinv, b.Xs, status, stream, assist, true, Gs, nn));
+    if (one_launch && solve_in_one(nn)) {
+      SPCHK(solve_tc(Gs, nn, m, nn, Rs, nn, b.one, save ? save->Y : nullptr, save ? save->kpad : 0, save ? save->k : 0, status,
+                     stream));
+    } else {
+      SPCHK(potrf_lower_tc(Gs, nn, nn, dinv, b.P, status, stream, assist, m, split_lookahead));
+      if (save) CU(copy_cols_padded(Rs, nn, m, save->k, save->kpad, save->Y, stream));
+      SPCHK(potrs_right_tc(Rs, m, nn, nn, b.P, dinv, b.Xs, status, stream, assist, true, Gs, nn));
+    }
   } else {
     CU(gather_cols<T>(R, ldr, idx, m, nn, Rs, nn, stream));
     CU(potrf_lower_f64(Gs, nn, nn, dinv, status, stream, assist, m));
@@ -846,6 +858,7 @@ static sp_status admm_step_impl(const sp_ffn_module* m, sp_ffn_state* st, const 
   SideStream* side = side_stream();
   cudaStream_t sa = side ? side->stream : s;
   const bool narrow = std::max(n, d) <= kOverlapMaxN;
+  const bool one = std::max(n, d) <= kSolveOneModule, lead_solved = one && solve_in_one(n);
   const OverlapScope overlap(narrow);
   JoinOnExit join_guard{side, s};
   // Reuse of the factorisation for the recovery on the kept support (tensor-core path): the unrestricted system is
@@ -870,7 +883,7 @@ static sp_status admm_step_impl(const sp_ffn_module* m, sp_ffn_state* st, const 
   if (skip_scores) {
   } else if (bf16) {
     SPCHK(ridge_core<float>(st->R2, n, st->G_A, n, d, n, reuse ? p.perm : nullptr, n, rho2, p.W2t, n, p.sb, status_dev,
-                            s, side ? &side->assist_main : nullptr, false, reuse ? &lead : nullptr));
+                            s, side ? &side->assist_main : nullptr, false, reuse ? &lead : nullptr, false, one));
   } else {
     SPCHK(ridge_core<double>(st->R2, n, st->G_A, n, d, n, nullptr, n, rho2, p.W2t, n, p.sb, status_dev, s,
                              side ? &side->assist_main : nullptr));
@@ -897,7 +910,7 @@ static sp_status admm_step_impl(const sp_ffn_module* m, sp_ffn_state* st, const 
       SPCHK(gemm_tc(n, d, d, 1.f, ta, tb, 0.f, Operand{p.W1t, SP_F32, d, 1}, OutOperand{p.W1t, SP_F32, d}, false,
                     status_dev, sa, &sg, 2.0 * (double)n * d * d));
     } else if (bf16) SPCHK(ridge_core<float>(st->R1, d, st->G_X, d, n, d, nullptr, d, rho1, p.W1t, d, p.sbA, status_dev, sa,
-                                      side ? &side->assist_side : nullptr));
+                                      side ? &side->assist_side : nullptr, false, nullptr, false, one));
     else SPCHK(ridge_core<double>(st->R1, d, st->G_X, d, n, d, nullptr, d, rho1, p.W1t, d, p.sbA, status_dev, sa,
                                       side ? &side->assist_side : nullptr));
   }
@@ -960,20 +973,21 @@ static sp_status admm_step_impl(const sp_ffn_module* m, sp_ffn_state* st, const 
     if (reuse) {
       {
         SkipScope skip_if_changed(p.reuse_flags + 0);
-        ProfScope prof(PK_SOLVE, 2.0 * (double)d * k_lead * k_lead, 0.0, s);
-        SPCHK(potrs_right_tc(lead.Y, d, k_lead, k_lead, p.sb.P, reinterpret_cast<const float*>(p.sb.dinv), p.sb.Xs,
-                             status_dev, s, side ? &side->assist_main : nullptr, true,
-                             reinterpret_cast<const float*>(p.sb.Gs), n, n));
+        ProfScope prof(PK_SOLVE, lead_solved ? 0.0 : 2.0 * (double)d * k_lead * k_lead, 0.0, s);
+        if (!lead_solved)
+          SPCHK(potrs_right_tc(lead.Y, d, k_lead, k_lead, p.sb.P, reinterpret_cast<const float*>(p.sb.dinv), p.sb.Xs,
+                               status_dev, s, side ? &side->assist_main : nullptr, true,
+                               reinterpret_cast<const float*>(p.sb.Gs), n, n));
         CU(scatter_cols<float>(lead.Y, k_lead, p.sb.idx, d, k, n, st->W2, n, s));
       }
       {
         SkipScope skip_if_unchanged(p.reuse_flags + 1);
         SPCHK(ridge_core<float>(st->R2, n, st->G_A, n, d, n, p.sb.idx, k, rho2, st->W2, n, p.sb, status_dev, s,
-                                side ? &side->assist_main : nullptr, z1_ahead, nullptr, true));
+                                side ? &side->assist_main : nullptr, z1_ahead, nullptr, true, one));
       }
     } else if (bf16) {
       SPCHK(ridge_core<float>(st->R2, n, st->G_A, n, d, n, p.sb.idx, k, rho2, st->W2, n, p.sb, status_dev, s,
-                              side ? &side->assist_main : nullptr, z1_ahead));
+                              side ? &side->assist_main : nullptr, z1_ahead, nullptr, false, one));
     } else {
       SPCHK(ridge_core<double>(st->R2, n, st->G_A, n, d, n, p.sb.idx, k, rho2, st->W2, n, p.sb, status_dev, s,
                                side ? &side->assist_main : nullptr));
@@ -1019,10 +1033,14 @@ static sp_status admm_step_impl(const sp_ffn_module* m, sp_ffn_state* st, const 
       // right-hand sides: the rows of W2[:, S]^T as the tensor-core path sees them (bf16-rounded)
       CU(convert_matrix(p.W2b, SP_BF16, kp, p.W2cf, SP_F32, kp, d, k, s));
       CU(transpose_convert<float>(p.W2cf, kp, d, k, Rs, d, s));
-      SPCHK(potrf_lower_tc(Gs, d, d, reinterpret_cast<float*>(p.sb.dinv), p.sb.P, status_dev, s,
-                           side ? &side->assist_main : nullptr, k, z1_ahead));
-      SPCHK(potrs_right_tc(Rs, k, d, d, p.sb.P, reinterpret_cast<float*>(p.sb.dinv), p.sb.Xs, status_dev, s,
-                           side ? &side->assist_main : nullptr, true, Gs, d));
+      if (one && solve_in_one(d)) {
+        SPCHK(solve_tc(Gs, d, k, d, Rs, d, p.sb.one, nullptr, 0, 0, status_dev, s));
+      } else {
+        SPCHK(potrf_lower_tc(Gs, d, d, reinterpret_cast<float*>(p.sb.dinv), p.sb.P, status_dev, s,
+                             side ? &side->assist_main : nullptr, k, z1_ahead));
+        SPCHK(potrs_right_tc(Rs, k, d, d, p.sb.P, reinterpret_cast<float*>(p.sb.dinv), p.sb.Xs, status_dev, s,
+                             side ? &side->assist_main : nullptr, true, Gs, d));
+      }
       if (split_h) {
         CU(split_bf16(Rs, d, nullptr, k, d, dp64, p.Qtb, s));      // only the hi part is used (see the D product)
         qt = MatRef{p.Qtb, SP_BF16, 2 * dp64};

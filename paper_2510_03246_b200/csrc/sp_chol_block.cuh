@@ -331,15 +331,15 @@ struct DiagTiles {
     return table[warp];
   }
   // waits for a group's barrier, about a second at most
-  static __device__ __forceinline__ bool wait(uint32_t bar) {
+  static __device__ __forceinline__ bool wait(uint32_t bar, uint32_t parity) {
     const auto done = [&] {
       uint32_t ok;
       asm volatile(
           "{\n\t.reg .pred p;\n\t"
-          "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n\t"
+          "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
           "selp.u32 %0, 1, 0, p;\n\t}"
           : "=r"(ok)
-          : "r"(bar)
+          : "r"(bar), "r"(parity)
           : "memory");
       return ok != 0;
     };
@@ -382,26 +382,69 @@ struct DiagTiles {
     }
   }
 
+  static constexpr uint32_t BARS = 2 * NS * GROUPS;
+
+  // Where the results go: inv(L) [NB, NB] and its transpose, fp32, dense.  (A tile of X: row rb * 32 + lane in registers, `own` the
+  // same by columns.)
+  struct Dense {
+    float *inv, *inv_t;
+    __device__ __forceinline__ void zeros(int rb, int s, int lane) const {   // the zeros on the other side of the diagonal
+#pragma unroll 4
+      for (int c = 0; c < SB; ++c) {
+        inv[(rb * SB + c) * NB + s * SB + lane] = 0.f;
+        inv_t[(s * SB + c) * NB + rb * SB + lane] = 0.f;
+      }
+    }
+    __device__ __forceinline__ void tile(const float (&a)[SB], const float* own, bool live, int rb, int s, int lane) const {
+#pragma unroll
+      for (int c = 0; c < SB; ++c) inv[(s * SB + c) * NB + rb * SB + lane] = a[c];
+      if (live) {
+#pragma unroll
+        for (int r = 0; r < SB; r += 4) {
+          const float4 u = ld(own + lane * P + r);            // column s SB + lane, four rows
+          inv_t[(rb * SB + r) * NB + s * SB + lane] = u.x;
+          inv_t[(rb * SB + r + 1) * NB + s * SB + lane] = u.y;
+          inv_t[(rb * SB + r + 2) * NB + s * SB + lane] = u.z;
+          inv_t[(rb * SB + r + 3) * NB + s * SB + lane] = u.w;
+        }
+      } else {
+#pragma unroll 8
+        for (int r = 0; r < SB; ++r) inv_t[(rb * SB + r) * NB + s * SB + lane] = rb == s && r == lane ? 1.f : 0.f;
+      }
+    }
+  };
   // A: the nb x nb block (lower triangle; rows and columns beyond nb are those of an identity).  inv [NB, NB] receives inv(L),
   // inv_t its transpose; both dense, zero outside their triangle.
   static __device__ void run(const float* A, int64_t lda, int nb, float* inv, float* inv_t, int64_t row0, int32_t* status) {
     extern __shared__ __align__(16) unsigned char diag_smem[];
-    float* LT = reinterpret_cast<float*>(diag_smem);          // LT[k][row]
+    float* sm = reinterpret_cast<float*>(diag_smem);
+    const uint32_t bars = (uint32_t)__cvta_generic_to_shared(sm + 2 * NB * P + GROUPS * 16);
+    for (uint32_t b = threadIdx.x; b < BARS; b += THREADS)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bars + 8u * b) : "memory");
+    __syncthreads();
+    eliminate<false>(sm, bars, 0, A, lda, nb, Dense{inv, inv_t}, row0, status);
+  }
+  // place of entry (row, col) of a block that is staged in shared memory (STAGED): every tile by rows in its own place
+  static __device__ __forceinline__ int staged_at(int row, int col) {
+    return ((col / SB) * SB + row % SB) * P + (row / SB) * SB + col % SB;
+  }
+
+  // The block comes from A, or (STAGED) sits in sm as staged_at() says: complete, that is zero above the diagonal and an identity
+  // beyond nb.  bars: BARS barriers of one arrival, parity: their phase (a full block completes one of each that is waited for).
+  template <bool STAGED, typename Out>
+  static __device__ __forceinline__ void eliminate(float* sm, uint32_t bars, uint32_t parity, const float* A, int64_t lda, int nb,
+                                                   const Out& out, int64_t row0, int32_t* status) {
+    float* LT = sm;                                           // LT[k][row]
     float* XT = LT + NB * P;                                  // XT[k][row]
     float* CI = XT + NB * P;                                  // C^-1 of every group, row-major
-    const uint32_t bars = (uint32_t)__cvta_generic_to_shared(CI + GROUPS * 16);
     auto bar = [&](int row_block, int group) { return bars + 8u * (uint32_t)(row_block * GROUPS + group); };
     const int t = threadIdx.x, lane = t & 31;
     const int tl = tile_of(t >> 5);
     const bool mat = (tl >> 8) == 0;
     const int rb = (tl >> 4) & 15, s = tl & 15;
-    for (int b = t; b < 2 * NS * GROUPS; b += THREADS)
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bars + 8u * b) : "memory");
-    __syncthreads();
     // row blocks and column blocks beyond nb are those of an identity: nothing is eliminated there
     const int ns = (nb + SB - 1) / SB;
     const bool live = rb < ns && s < ns;
-    const int i = rb * SB + lane;                             // the lane's row
     float* own = (mat ? LT : XT) + s * SB * P + rb * SB;      // the tile, [column][row]
     const float* orow = (mat ? LT : XT) + rb * SB;            // its row block's columns
     const float* Ls = LT + s * SB;                            // rows of L that belong to its columns
@@ -409,34 +452,36 @@ struct DiagTiles {
     const int first = mat ? 0 : rb;                           // first column block with entries in this row block
     float a[SB];
     if (mat) {
-      // whole rows in, turned in the tile's own place
-      const bool vec = lda % 4 == 0 && (reinterpret_cast<uintptr_t>(A) & 15u) == 0;
-      const int c = (lane & 7) * 4, j = s * SB + c;
-      float4 q[8];
-      const float* p = A + (int64_t)(rb * SB + (lane >> 3)) * lda + j;
-      if (vec && nb == NB) {                                  // (all loads in flight at once)
+      if constexpr (!STAGED) {
+        // whole rows in, turned in the tile's own place
+        const bool vec = lda % 4 == 0 && (reinterpret_cast<uintptr_t>(A) & 15u) == 0;
+        const int c = (lane & 7) * 4, j = s * SB + c;
+        float4 q[8];
+        const float* p = A + (int64_t)(rb * SB + (lane >> 3)) * lda + j;
+        if (vec && nb == NB) {                                  // (all loads in flight at once)
 #pragma unroll
-        for (int u = 0; u < 8; ++u) q[u] = ld(p + (int64_t)(4 * u) * lda);
-      } else {
+          for (int u = 0; u < 8; ++u) q[u] = ld(p + (int64_t)(4 * u) * lda);
+        } else {
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            const int gi = rb * SB + u * 4 + (lane >> 3);
+            float v[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) v[e] = (gi < nb && j + e <= gi) ? p[(int64_t)(4 * u) * lda + e] : 0.f;
+            q[u] = make_float4(v[0], v[1], v[2], v[3]);
+          }
+        }
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
           const int gi = rb * SB + u * 4 + (lane >> 3);
-          float v[4];
+          float v[4] = {q[u].x, q[u].y, q[u].z, q[u].w};
 #pragma unroll
-          for (int e = 0; e < 4; ++e) v[e] = (gi < nb && j + e <= gi) ? p[(int64_t)(4 * u) * lda + e] : 0.f;
+          for (int e = 0; e < 4; ++e) v[e] = j + e > gi ? 0.f : (gi >= nb && j + e == gi) ? 1.f : v[e];
           q[u] = make_float4(v[0], v[1], v[2], v[3]);
         }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) *reinterpret_cast<float4*>(own + (u * 4 + (lane >> 3)) * P + c) = q[u];
       }
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int gi = rb * SB + u * 4 + (lane >> 3);
-        float v[4] = {q[u].x, q[u].y, q[u].z, q[u].w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) v[e] = j + e > gi ? 0.f : (gi >= nb && j + e == gi) ? 1.f : v[e];
-        q[u] = make_float4(v[0], v[1], v[2], v[3]);
-      }
-#pragma unroll
-      for (int u = 0; u < 8; ++u) *reinterpret_cast<float4*>(own + (u * 4 + (lane >> 3)) * P + c) = q[u];
       __syncwarp();
       if (s == 0) {
 #pragma unroll
@@ -449,20 +494,14 @@ struct DiagTiles {
     } else {
 #pragma unroll
       for (int c = 0; c < SB; ++c) a[c] = rb == s && c == lane ? 1.f : 0.f;
-      if (s > rb) {                                           // the zeros on the other side of the diagonal
-#pragma unroll 4
-        for (int c = 0; c < SB; ++c) {
-          inv[(rb * SB + c) * NB + s * SB + lane] = 0.f;
-          inv_t[(s * SB + c) * NB + rb * SB + lane] = 0.f;
-        }
-      }
+      if (s > rb) out.zeros(rb, s, lane);
     }
     bool ok = true;
     if (live) {
       if (s > first) {
         // columns to the left; what the last column block waits for is not needed before the one in front of it is under
         // way, and the first one's elimination has the schedulers to itself
-        if (s == NS - 1 || (!mat && s == NS - 2)) ok = ok && wait(bar(1, GS));
+        if (s == NS - 1 || (!mat && s == NS - 2)) ok = ok && wait(bar(1, GS), parity);
         const int r0 = (lane >> 2) * 4, c0 = (lane & 3) * 8;  // four rows and eight columns per lane
         float acc[4][8];
 #pragma unroll
@@ -473,8 +512,8 @@ struct DiagTiles {
             acc[r][h] = u.x; acc[r][h + 1] = u.y; acc[r][h + 2] = u.z; acc[r][h + 3] = u.w;
           }
         for (int g = first * GS; g < s * GS; ++g) {
-          if (oid != s) ok = ok && wait(bar(oid, g));
-          ok = ok && wait(bar(s, g));
+          if (oid != s) ok = ok && wait(bar(oid, g), parity);
+          ok = ok && wait(bar(s, g), parity);
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
             const float4 l = ld(orow + (g * 4 + k) * P + r0);
@@ -505,7 +544,7 @@ struct DiagTiles {
 #pragma unroll
         for (int g = 0; g < GS; ++g) {
           const int j = 4 * g, gg = s * GS + g;
-          ok = ok && wait(bar(s, gg));
+          ok = ok && wait(bar(s, gg), parity);
           float ci[16], l[4];
 #pragma unroll
           for (int q = 0; q < 16; q += 4) {
@@ -528,23 +567,7 @@ struct DiagTiles {
         }
       }
     }
-    if (!mat) {
-#pragma unroll
-      for (int c = 0; c < SB; ++c) inv[(s * SB + c) * NB + i] = a[c];
-      if (live) {
-#pragma unroll
-        for (int r = 0; r < SB; r += 4) {
-          const float4 u = ld(own + lane * P + r);            // column s SB + lane, four rows
-          inv_t[(rb * SB + r) * NB + s * SB + lane] = u.x;
-          inv_t[(rb * SB + r + 1) * NB + s * SB + lane] = u.y;
-          inv_t[(rb * SB + r + 2) * NB + s * SB + lane] = u.z;
-          inv_t[(rb * SB + r + 3) * NB + s * SB + lane] = u.w;
-        }
-      } else {
-#pragma unroll 8
-        for (int r = 0; r < SB; ++r) inv_t[(rb * SB + r) * NB + s * SB + lane] = rb == s && r == lane ? 1.f : 0.f;
-      }
-    }
+    if (!mat) out.tile(a, own, live, rb, s, lane);
     if (!ok && lane == 0) report_status(status, SP_ERR_TIMEOUT, (int32_t)row0, 12);
   }
 

@@ -362,6 +362,27 @@ sp_status potrs_right_tc(float* X, int64_t m, int64_t n, int64_t ldx, const void
 // n_factor > n: the factor in P / dinv / Lf is that of a larger system of n_factor rows and the solve uses its leading
 // n x n block, which is the factor of the system's leading block (n a multiple of kCholTcNB).
 
+// The whole solve W = R G^-1 in one launch (sp_solve_tc.cu), systems that solve_in_one() names.
+//   A: [nn + m, nn] fp32, lower triangle of G and the right-hand sides below it; W [m, nn] may be the latter's place.
+//   lead != nullptr: also the solution [m, lead_k] of the leading lead_k x lead_k system with the leading right-hand sides.
+//   P: bf16 [pad(nn) + pad(m), 3 pad(nn)], Y: bf16 [pad(m), 3 kCholTcNB], flags: solve_tc_flag_words(nn, m) words; pad = chol_tc_pad.
+struct SolveOneBufs {
+  void *P, *Y;
+  uint32_t* flags;
+};
+// One launch against the launches per block column of sp_linalg_tc.cu (unknowns / right-hand sides, us): 384 / 768 126 -> 144, 768 / 768
+// 261 -> 260, 641 / 136 387 -> 261, 1024 / 2048 372 -> 343, 2048 / 4096 1033 -> 788, 4096 / 3302 2306 -> 1651, 5734 / 7168 13319 ->
+// 4310, 8192 / 2048 6022 -> 4392, 9216 / 3072 8974 -> 6908; with two levels of blocks, 12288 / 4096 14735 -> 16072.
+constexpr int64_t kSolveOneMinN = 512, kSolveOneMaxN = kOuterMinN - 1;
+// A step's recoveries: modules up to this width.  The sign select of the z-update turns differences of rounding into differences of
+// the recovered weights; the recoveries of 7168 x 28672 (8192 tokens, five iterations) by the other form's roundings move W1 by
+// 1.3 %, as far as both are from 64 bits (1.5 %).  4096 x 16384 on 4096 tokens: 0.8 %.
+constexpr int64_t kSolveOneModule = 16384;
+inline bool solve_in_one(int64_t n) { return n > kSolveOneMinN && n <= kSolveOneMaxN; }
+size_t solve_tc_flag_words(int64_t n, int64_t m);
+sp_status solve_tc(const float* A, int64_t nn, int64_t m, int64_t lda, float* W, int64_t ldw, const SolveOneBufs& b,
+                   float* lead, int64_t ld_lead, int64_t lead_k, int32_t* status_dev, cudaStream_t stream);
+
 // `batch` independent systems of one size n (a multiple of kCholTcNB) with m right-hand sides each, every step one launch
 // over all of them.  System b: A + b * a_bs = [n + m, n] fp32 (lower triangle of the matrix, then the right-hand sides
 // B of X (L L^T) = B; on return they hold X), dinv + b * d_bs (room as for potrf_lower_tc), P = batch x

@@ -27,11 +27,10 @@
 // freed.  Not bounded, since what they wait for cannot stay away: the two cluster barriers (the CTAs of a pair start together
 // and both reach them on every path), the allocation of tensor memory (the shared memory of a CTA keeps every other CTA of
 // this kernel off its SM, and no other kernel allocates any), and the wait for the kernels before this one.
-#include <cuda.h>
 #include <math.h>
 #include <string.h>
 
-#include "sp_common.cuh"
+#include "sp_tc.cuh"
 
 namespace sp {
 namespace {
@@ -117,86 +116,6 @@ __device__ __forceinline__ void unit_map(const TcParams& p, int u, int num_kb, i
   kb1 = (kb0 + p.kb_per_split < num_kb) ? kb0 + p.kb_per_split : num_kb;
 }
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ uint32_t cluster_ctarank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-// shared::cluster address of the same shared-memory location in CTA `rank` of the cluster
-__device__ __forceinline__ uint32_t map_to_cta(uint32_t addr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-// arrive on a barrier given by its shared::cluster address (own CTA or the peer)
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster_addr) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster_addr) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// Bounded wait.  Returns false when the budget ran out or another role of this CTA already gave up.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, long long budget) {
-  if (mbar_try(bar, parity)) return true;
-  // (a try_wait may itself suspend the thread for a while, so the clock is read after every unsuccessful try)
-  const long long t0 = clock64();
-  while (!mbar_try(bar, parity)) {
-    if (*abort_flag) return false;
-    if (clock64() - t0 > budget) {
-      *abort_flag = 1;
-      return false;
-    }
-  }
-  return true;
-}
-
-// Load of one box into this CTA's shared memory; the bytes complete on the barrier `bar_cluster_addr`, which is the
-// pair leader's (cta_group::2 form: the barrier may live in the peer CTA).
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int32_t c0, int32_t c1,
-                                            uint32_t bar_cluster_addr) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-      ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(bar_cluster_addr)
-      : "memory");
-}
-// plain one-CTA load (epilogue: a block of Cin into this warp's shared tile, completing on this CTA's barrier)
-__device__ __forceinline__ void tma_load_2d_local(uint32_t dst, const CUtensorMap* map, int32_t c0, int32_t c1,
-                                                  uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-      ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(bar)
-      : "memory");
-}
-__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, int32_t c0, int32_t c1, uint32_t src) {
-  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];"
-               ::"l"(map), "r"(c0), "r"(c1), "r"(src)
-               : "memory");
-}
-__device__ __forceinline__ void tma_reduce_add_2d(const CUtensorMap* map, int32_t c0, int32_t c1, uint32_t src) {
-  asm volatile("cp.reduce.async.bulk.tensor.2d.global.shared::cta.add.tile.bulk_group [%0, {%1, %2}], [%3];"
-               ::"l"(map), "r"(c0), "r"(c1), "r"(src)
-               : "memory");
-}
 // five-dimensional forms for batched launches
 __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* map, const Coord5& c,
                                             uint32_t bar_cluster_addr) {
@@ -215,59 +134,6 @@ __device__ __forceinline__ void tma_reduce_add_5d(const CUtensorMap* map, const 
                ::"l"(map), "r"(c.x[0]), "r"(c.x[1]), "r"(c.x[2]), "r"(c.x[3]), "r"(c.x[4]), "r"(src)
                : "memory");
 }
-__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void bulk_wait_read_1() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-// The MMAs issued so far by this thread arrive on the barrier at this shared-memory offset in BOTH CTAs of the pair.
-__device__ __forceinline__ void tc_commit_pair(uint32_t bar) {
-  const uint16_t mask = 3;
-  asm volatile(
-      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-      ::"r"(bar), "h"(mask)
-      : "memory");
-}
-__device__ __forceinline__ void tc_mma_bf16_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                                 uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-__device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t* r) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr)
-      : "memory");
-}
-__device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-
-// Shared-memory matrix descriptor of a 128-byte-swizzled operand tile.
-//   K-major : rows of 64 bf16 (128 B); 8-row groups 1024 B apart (stride byte offset); leading offset unused (1).
-//   MN-major: 64-element (128 B) runs along MN, one per K index; 8-K-index groups 1024 B apart (stride offset);
-//             consecutive 64-element MN blocks `mn_block_bytes` apart (leading offset).
-__device__ __forceinline__ uint64_t make_smem_desc(uint32_t addr, bool kmajor, uint32_t mn_block_bytes) {
-  uint64_t d = 0;
-  d |= (uint64_t)((addr & 0x3ffffu) >> 4);
-  const uint32_t lbo = kmajor ? 1u : (mn_block_bytes >> 4);
-  d |= (uint64_t)(lbo & 0x3fffu) << 16;
-  d |= (uint64_t)((1024u >> 4) & 0x3fffu) << 32;
-  d |= (uint64_t)1 << 46;  // descriptor version of this architecture
-  d |= (uint64_t)2 << 61;  // 128-byte swizzle
-  return d;
-}
-
 // Instruction descriptor of the pair's MMA: 256 x tile_n x 16, bf16 operands, fp32 accumulator.
 __device__ __forceinline__ uint32_t make_instr_desc(bool a_kmajor, bool b_kmajor, int tile_n) {
   uint32_t d = 0;
@@ -762,13 +628,15 @@ EncodeTiledFn encode_fn() {
   return fn;
 }
 
+}  // namespace
+
 // Tensor map of a row-major matrix [outer, inner] with leading dimension ld (elements), 128-byte swizzle.
 //   bf16 operand, K-major : inner = K, outer = rows, box = {64, 128} (B of the narrow tile: {64, 64})
 //   bf16 operand, MN-major: inner = rows, outer = K, box = {64, 64}
 //   fp32 output C         : inner = N, outer = M, box = {32, 32}
 //   bf16 C / Cin          : inner = N, outer = M, box = {32, 32}, 64-byte swizzle
 bool make_map(CUtensorMap* map, bool f32, const void* ptr, int64_t inner, int64_t outer, int64_t ld, int box_inner,
-              int box_outer, bool swizzle64 = false) {
+              int box_outer, bool swizzle64) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return false;
   cuuint64_t dims[2] = {(cuuint64_t)inner, (cuuint64_t)outer};
@@ -781,8 +649,6 @@ bool make_map(CUtensorMap* map, bool f32, const void* ptr, int64_t inner, int64_
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
 }
-
-}  // namespace
 
 namespace {
 // Five-dimensional tensor map of a batched operand.  Roles: inner (contiguous) dimension, outer dimension (stride ld),
