@@ -888,27 +888,35 @@ static sp_status admm_step_impl(const sp_ffn_module* m, sp_ffn_state* st, const 
     SPCHK(ridge_core<double>(st->R2, n, st->G_A, n, d, n, nullptr, n, rho2, p.W2t, n, p.sb, status_dev, s,
                              side ? &side->assist_main : nullptr));
   }
-  const bool need_w1 = !scores_only || prm->score_kind == SP_SCORE_LEMMA1;   // only the Lemma-1 score reads W1~
+  // With the cached inverse of the constant system W1~ = R1 Ginv is one product, both operands as three bf16 parts, the six part
+  // products of weight >= 2^-16 as K segments (Ginv is symmetric, so its rows serve as the K-major B operand).  Only the kept
+  // rows are wanted, unless the Lemma-1 score reads W1~: they are formed once the mask is there (below).  (All rows beside the
+  // recovery of W2~ take the tensor cores from it: 7168 x 28672 with 20 % kept 167 -> 152 ms a step, gated 4096 x 11008 with 30 %
+  // 13.6 -> 12.2; 768 x 3072 equal.)
+  const bool lemma1 = !skip_scores && prm->score_kind == SP_SCORE_LEMMA1;
+  const bool w1_product = bf16 && st->G_X_inv != nullptr, w1_kept = w1_product && !scores_only && !lemma1;
+  const int64_t dp3 = split_kpad(d);
+  auto w1_rows = [&](const int32_t* rows_idx, int64_t rows) -> sp_status {
+    CU(split3_bf16(st->R1, d, rows_idx, rows, d, dp3, p.R1p, sa));
+    TcOperand ta{p.R1p, 3 * dp3, true}, tb{p.Gip, 3 * dp3, true};
+    ta.kext = tb.kext = 3 * dp3;
+    TcSegments sg;
+    sg.nseg = 6;
+    static const int pa[6] = {0, 0, 1, 0, 2, 1}, pb[6] = {0, 1, 0, 2, 0, 1};
+    for (int q = 0; q < 6; ++q) {
+      sg.a_k[q] = (int32_t)(pa[q] * dp3);
+      sg.b_k[q] = (int32_t)(pb[q] * dp3);
+    }
+    ProfScope prof(PK_SOLVE, 2.0 * (double)rows * d * d, 0.0, sa);
+    return gemm_tc(rows, d, d, 1.f, ta, tb, 0.f, Operand{p.W1t, SP_F32, d, 1}, OutOperand{p.W1t, SP_F32, d}, false, status_dev,
+                   sa, &sg, 2.0 * (double)rows * d * d);
+  };
+  const bool need_w1 = !scores_only || lemma1;               // only the Lemma-1 score reads W1~
   if (need_w1) {
     CU(effective_ridge(st->G_X, d, d, prm->rho, prm->rho_relative, rho1, sa));
-    if (bf16 && st->G_X_inv) {
-      // cached inverse of the constant system: W1~ = R1 Ginv, both operands as three bf16 parts, the six part products
-      // of weight >= 2^-16 as K segments (Ginv is symmetric, so its rows serve as the K-major B operand)
-      const int64_t dp3 = split_kpad(d);
-      CU(split3_bf16(st->R1, d, n, d, dp3, p.R1p, sa));
-      CU(split3_bf16(st->G_X_inv, d, d, d, dp3, p.Gip, sa));
-      TcOperand ta{p.R1p, 3 * dp3, true}, tb{p.Gip, 3 * dp3, true};
-      ta.kext = tb.kext = 3 * dp3;
-      TcSegments sg;
-      sg.nseg = 6;
-      static const int pa[6] = {0, 0, 1, 0, 2, 1}, pb[6] = {0, 1, 0, 2, 0, 1};
-      for (int q = 0; q < 6; ++q) {
-        sg.a_k[q] = (int32_t)(pa[q] * dp3);
-        sg.b_k[q] = (int32_t)(pb[q] * dp3);
-      }
-      ProfScope prof(PK_SOLVE, 2.0 * (double)n * d * d, 0.0, sa);
-      SPCHK(gemm_tc(n, d, d, 1.f, ta, tb, 0.f, Operand{p.W1t, SP_F32, d, 1}, OutOperand{p.W1t, SP_F32, d}, false,
-                    status_dev, sa, &sg, 2.0 * (double)n * d * d));
+    if (w1_product) {
+      CU(split3_bf16(st->G_X_inv, d, nullptr, d, d, dp3, p.Gip, sa));
+      if (!w1_kept) SPCHK(w1_rows(nullptr, n));
     } else if (bf16) SPCHK(ridge_core<float>(st->R1, d, st->G_X, d, n, d, nullptr, d, rho1, p.W1t, d, p.sbA, status_dev, sa,
                                       side ? &side->assist_side : nullptr, false, nullptr, false, one));
     else SPCHK(ridge_core<double>(st->R1, d, st->G_X, d, n, d, nullptr, d, rho1, p.W1t, d, p.sbA, status_dev, sa,
@@ -919,7 +927,7 @@ static sp_status admm_step_impl(const sp_ffn_module* m, sp_ffn_state* st, const 
 
   // ---- 2. unit scores and layer importance
   if (skip_scores) {
-  } else if (prm->score_kind == SP_SCORE_LEMMA1) {
+  } else if (lemma1) {
     if (!joined) { CU(cudaStreamWaitEvent(s, side->join, 0)); joined = true; }   // this score reads W1~
     // b = W1~ X, c = d = t = z^pre = W1_0 X, written through G_X:  T0 = W1_0 G_X
     MatRef w10{m->W1_0.ptr, SP_F32, m->W1_0.ld}, gx{st->G_X, SP_F32, d}, t0{p.T0, SP_F32, d};
@@ -946,8 +954,22 @@ static sp_status admm_step_impl(const sp_ffn_module* m, sp_ffn_state* st, const 
   if (reuse) CU(mask_changed(st->mask, p.perm, p.reuse_flags + 2, k, p.reuse_flags, s));
 
   // ---- 4. masked weights: W1 = diag(M) W1~ ; W2 = recovery on the kept support (or M (.) W2~)
-  if (!joined) { CU(cudaStreamWaitEvent(s, side->join, 0)); joined = true; }
-  CU(mask_rows_copy(st->mask, p.W1t, d, st->W1, d, n, d, s));
+  // (the kept rows of W1~ on the side stream, beside what follows; without it both are the caller's)
+  if (w1_kept) {
+    if (side) {
+      CU(cudaEventRecord(side->fork, s));
+      CU(cudaStreamWaitEvent(sa, side->fork, 0));
+    }
+    SPCHK(w1_rows(p.sb.idx, k));
+    CU(place_rows(st->mask, p.sb.idx, k, p.W1t, d, st->W1, d, n, d, sa));
+    if (side) CU(cudaEventRecord(side->join, sa));
+    joined = side == nullptr;
+  } else {
+    if (!joined) { CU(cudaStreamWaitEvent(s, side->join, 0)); joined = true; }
+    CU(mask_rows_copy(st->mask, p.W1t, d, st->W1, d, n, d, s));
+  }
+  const float* w1_src = w1_kept ? p.W1t : st->W1;             // rows of the kept channels: by themselves, or to be gathered
+  const int32_t* w1_idx = w1_kept ? nullptr : p.sb.idx;
   // z1 = X W1[S, :]^T needs only the mask and W1: when the workspace has room for z1 of all tokens, these products
   // run on the side stream, on a subset of the SMs, while the caller's stream carries the recovery of W2 on the kept
   // support and the operands of the a-update (chains of short kernels that cannot fill the GPU).
@@ -956,7 +978,7 @@ static sp_status admm_step_impl(const sp_ffn_module* m, sp_ffn_state* st, const 
   if (z1_ahead) {
     CU(cudaEventRecord(side->fork, s));
     CU(cudaStreamWaitEvent(side->stream, side->fork, 0));
-    CU(split_bf16(st->W1, d, p.sb.idx, k, d, split_kpad(d), p.W1b, side->stream));
+    CU(split_bf16(w1_src, d, w1_idx, k, d, split_kpad(d), p.W1b, side->stream));
     const size_t esz_x = 2;
     for (int64_t t0 = 0; t0 < N; t0 += p.chunk) {
       const int64_t Tc = (N - t0 < p.chunk) ? N - t0 : p.chunk;
@@ -1013,7 +1035,10 @@ static sp_status admm_step_impl(const sp_ffn_module* m, sp_ffn_state* st, const 
   CU(gather_cols<float>(st->W2, n, idx, d, k, p.W2cf, kp, s));
   MatRef w1{nullptr, SP_F32, d}, w2{p.W2cf, SP_F32, kp}, qt{p.Qt, SP_F32, d};
   if (bf16) {
-    if (!z1_ahead) CU(split_bf16(st->W1, d, idx, k, d, split_kpad(d), p.W1b, s));
+    if (!z1_ahead) {
+      if (!joined) { CU(cudaStreamWaitEvent(s, side->join, 0)); joined = true; }
+      CU(split_bf16(w1_src, d, w1_idx, k, d, split_kpad(d), p.W1b, s));
+    }
     CU(convert_matrix(p.W2cf, SP_F32, kp, p.W2b, SP_BF16, kp, d, k, s));
     w2 = MatRef{p.W2b, SP_BF16, kp};
     if (split_h) CU(split_bf16(p.W2cf, kp, nullptr, d, k, kp64, p.W2sb, s));

@@ -400,8 +400,9 @@ cudaError_t symmetrize_lower(float* G, int64_t n, int64_t ld, cudaStream_t strea
 cudaError_t split_bf16(const float* src, int64_t lds, const int32_t* row_idx, int64_t rows, int64_t cols, int64_t kpad,
                        void* dst, cudaStream_t stream);
 // dst [rows, 3 * kpad] bf16: the hi, mid and lo parts of src side by side (an fp32 value as an exact sum of three bf16)
-cudaError_t split3_bf16(const float* src, int64_t lds, int64_t rows, int64_t cols, int64_t kpad, void* dst,
-                        cudaStream_t stream);
+// row_idx as above
+cudaError_t split3_bf16(const float* src, int64_t lds, const int32_t* row_idx, int64_t rows, int64_t cols, int64_t kpad,
+                        void* dst, cudaStream_t stream);
 // dst[j, i] = (TD) src[i, j]
 template <typename TD>
 cudaError_t transpose_convert(const float* src, int64_t lds, int64_t rows, int64_t cols, TD* dst, int64_t ldd,
@@ -614,6 +615,9 @@ cudaError_t mask_changed(const uint8_t* mask, const int32_t* perm, const int32_t
 cudaError_t zero_pruned(const uint8_t* mask, int group, float* W_rows, int64_t r_rows, int64_t r_cols, int64_t r_ld,
                         float* W_cols, int64_t c_rows, int64_t c_cols, int64_t c_ld, cudaStream_t stream);
 // dst[i,:] = mask[i] ? src[i,:] : 0
+// dst[idx[p], :] = src[p, :] for the k kept rows, zero rows where the mask is zero
+cudaError_t place_rows(const uint8_t* mask, const int32_t* idx, int64_t k, const float* src, int64_t lds, float* dst, int64_t ldd,
+                       int64_t rows, int64_t cols, cudaStream_t stream);
 cudaError_t mask_rows_copy(const uint8_t* mask, const float* src, int64_t lds, float* dst, int64_t ldd, int64_t rows,
                            int64_t cols, cudaStream_t stream);
 

@@ -103,12 +103,12 @@ __global__ void __launch_bounds__(kStripThreads) split_bf16_kernel(const float* 
 // dst[i, part * kpad + j] = part `part` of the three-part bf16 split of src[i, j] (hi + mid + lo = src exactly up to
 // 2^-24); padding columns are zero.
 template <int W>
-__global__ void __launch_bounds__(kStripThreads) split3_bf16_kernel(const float* src, int64_t lds,
+__global__ void __launch_bounds__(kStripThreads) split3_bf16_kernel(const float* src, int64_t lds, const int32_t* row_idx,
                                                                     int64_t rows, int64_t cols, int64_t kpad,
                                                                     __nv_bfloat16* dst) {
   kernel_begin();
   const bool vec = pairs_aligned(src, lds);
-  const auto load = [&](int64_t i, int64_t p, int) { return load_pair(src + i * lds, 2 * p, cols, vec); };
+  const auto load = [&](int64_t i, int64_t p, int) { return load_pair(src + (row_idx ? (int64_t)row_idx[i] : i) * lds, 2 * p, cols, vec); };
   for_strip_move<W>(rows, kpad / 2, load, [&](int64_t i, int64_t p, int, float2 v) {
     const __nv_bfloat162 hi = __floats2bfloat162_rn(v.x, v.y);
     const float2 r1 = make_float2(v.x - __low2float(hi), v.y - __high2float(hi));
@@ -1150,14 +1150,14 @@ template cudaError_t transpose_convert<double>(const float*, int64_t, int64_t, i
 template cudaError_t transpose_convert<__nv_bfloat16>(const float*, int64_t, int64_t, int64_t, __nv_bfloat16*,
                                                       int64_t, cudaStream_t);
 
-cudaError_t split3_bf16(const float* src, int64_t lds, int64_t rows, int64_t cols, int64_t kpad, void* dst,
-                        cudaStream_t stream) {
+cudaError_t split3_bf16(const float* src, int64_t lds, const int32_t* row_idx, int64_t rows, int64_t cols, int64_t kpad,
+                        void* dst, cudaStream_t stream) {
   if (rows * kpad == 0) return cudaSuccess;
   ProfScope prof(PK_ELEMENTWISE, 0.0, (double)rows * cols * 10.0, stream);
   count_launch();
   strip_launch(rows, kpad / 2, [&](auto w, dim3 grid, dim3 block) {
     launch(split3_bf16_kernel<decltype(w)::value>, grid, block, 0, stream, 
-        src, lds, rows, cols, kpad, reinterpret_cast<__nv_bfloat16*>(dst));
+        src, lds, row_idx, rows, cols, kpad, reinterpret_cast<__nv_bfloat16*>(dst));
   });
   return cudaGetLastError();
 }

@@ -897,6 +897,20 @@ __global__ void __launch_bounds__(kStripThreads) mask_rows_copy_kernel(const uin
   });
 }
 
+// dst[idx[p], :] = src[p, :] for the k kept rows, zero rows elsewhere
+template <int W>
+__global__ void __launch_bounds__(kStripThreads) place_rows_kernel(const uint8_t* mask, const int32_t* idx, int64_t k, const float* src,
+                                                                   int64_t lds, float* dst, int64_t ldd, int64_t rows, int64_t cols) {
+  kernel_begin();
+  for_strip<W>(rows, cols, [&](int64_t i, int64_t j, int) {
+    if (!mask[i]) dst[i * ldd + j] = 0.f;
+    if (i < k) {
+      const int64_t r = idx[i];
+      if (r >= 0 && r < rows) dst[r * ldd + j] = src[i * lds + j];     // (a mask with fewer kept rows leaves the list short)
+    }
+  });
+}
+
 inline int grid_for(int64_t total, int threads) {
   int64_t b = ceil_div(total, (int64_t)threads);
   if (b > 148 * 16) b = 148 * 16;
@@ -1593,6 +1607,17 @@ cudaError_t mask_rows_copy(const uint8_t* mask, const float* src, int64_t lds, f
   count_launch();
   strip_launch(rows, cols, [&](auto w, dim3 grid, dim3 block) {
     launch(mask_rows_copy_kernel<decltype(w)::value>, grid, block, 0, stream, mask, src, lds, dst, ldd, rows, cols);
+  });
+  return cudaGetLastError();
+}
+
+cudaError_t place_rows(const uint8_t* mask, const int32_t* idx, int64_t k, const float* src, int64_t lds, float* dst, int64_t ldd,
+                       int64_t rows, int64_t cols, cudaStream_t stream) {
+  if (rows * cols == 0) return cudaSuccess;
+  ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
+  count_launch();
+  strip_launch(rows, cols, [&](auto w, dim3 grid, dim3 block) {
+    launch(place_rows_kernel<decltype(w)::value>, grid, block, 0, stream, mask, idx, k, src, lds, dst, ldd, rows, cols);
   });
   return cudaGetLastError();
 }
