@@ -126,13 +126,14 @@ SolveBufs carve_solve(Carver& c, int64_t nmax, int64_t mmax, size_t tsize) {
   b.dinv = c.take_bytes(dinv_elems(nmax) * tsize);
   b.P = nullptr;
   b.Xs = nullptr;
-  b.one = SolveOneBufs{nullptr, nullptr, nullptr};
+  b.one = SolveOneBufs{nullptr, nullptr, nullptr, nullptr};
   if (tsize == 4) {
     const size_t np = (size_t)chol_tc_pad(nmax);
     b.P = c.take_bytes((np + (size_t)chol_tc_pad(mmax)) * 3 * np * 2);
     const size_t rows = (size_t)(nmax > mmax ? nmax : mmax);   // either dimension may be the right-hand-side count
     b.Xs = c.take_bytes((size_t)chol_tc_xs_elems(nmax, (int64_t)rows) * 2);
     b.one.P = b.P;
+    b.one.pre = reinterpret_cast<float*>(b.dinv);      // (the other form's inverse diagonal blocks)
     b.one.Y = c.take_bytes((size_t)chol_tc_pad((int64_t)rows) * 3 * kCholTcNB * 2);
     b.one.flags = c.take<uint32_t>(solve_tc_flag_words(nmax, (int64_t)rows));
   }

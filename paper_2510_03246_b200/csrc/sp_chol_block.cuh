@@ -422,23 +422,23 @@ struct DiagTiles {
     for (uint32_t b = threadIdx.x; b < BARS; b += THREADS)
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bars + 8u * b) : "memory");
     __syncthreads();
-    eliminate<false>(sm, bars, 0, A, lda, nb, Dense{inv, inv_t}, row0, status);
+    eliminate<false>(threadIdx.x, sm, bars, 0, A, lda, nb, Dense{inv, inv_t}, row0, status);
   }
   // place of entry (row, col) of a block that is staged in shared memory (STAGED): every tile by rows in its own place
   static __device__ __forceinline__ int staged_at(int row, int col) {
     return ((col / SB) * SB + row % SB) * P + (row / SB) * SB + col % SB;
   }
 
-  // The block comes from A, or (STAGED) sits in sm as staged_at() says: complete, that is zero above the diagonal and an identity
+  // t: the thread.  The block comes from A, or (STAGED) sits in sm as staged_at() says: complete, that is zero above the diagonal and an identity
   // beyond nb.  bars: BARS barriers of one arrival, parity: their phase (a full block completes one of each that is waited for).
   template <bool STAGED, typename Out>
-  static __device__ __forceinline__ void eliminate(float* sm, uint32_t bars, uint32_t parity, const float* A, int64_t lda, int nb,
+  static __device__ __forceinline__ void eliminate(int t, float* sm, uint32_t bars, uint32_t parity, const float* A, int64_t lda, int nb,
                                                    const Out& out, int64_t row0, int32_t* status) {
     float* LT = sm;                                           // LT[k][row]
     float* XT = LT + NB * P;                                  // XT[k][row]
     float* CI = XT + NB * P;                                  // C^-1 of every group, row-major
     auto bar = [&](int row_block, int group) { return bars + 8u * (uint32_t)(row_block * GROUPS + group); };
-    const int t = threadIdx.x, lane = t & 31;
+    const int lane = t & 31;
     const int tl = tile_of(t >> 5);
     const bool mat = (tl >> 8) == 0;
     const int rb = (tl >> 4) & 15, s = tl & 15;

@@ -368,12 +368,14 @@ sp_status potrs_right_tc(float* X, int64_t m, int64_t n, int64_t ldx, const void
 //   P: bf16 [pad(nn) + pad(m), 3 pad(nn)], Y: bf16 [pad(m), 3 kCholTcNB], flags: solve_tc_flag_words(nn, m) words; pad = chol_tc_pad.
 struct SolveOneBufs {
   void *P, *Y;
+  float* pre;         // 2 ceil(nn / kCholTcNB) blocks of kCholTcNB^2
   uint32_t* flags;
 };
-// One launch against the launches per block column of sp_linalg_tc.cu (unknowns / right-hand sides, us): 384 / 768 126 -> 144, 768 / 768
-// 261 -> 260, 641 / 136 387 -> 261, 1024 / 2048 372 -> 343, 2048 / 4096 1033 -> 788, 4096 / 3302 2306 -> 1651, 5734 / 7168 13319 ->
-// 4310, 8192 / 2048 6022 -> 4392, 9216 / 3072 8974 -> 6908; with two levels of blocks, 12288 / 4096 14735 -> 16072.
-constexpr int64_t kSolveOneMinN = 512, kSolveOneMaxN = kOuterMinN - 1;
+// One launch against the launches per block column of sp_linalg_tc.cu (unknowns / right-hand sides, us): 128 / 128 41 -> 58, 256 / 256 78 ->
+// 87, 257 / 100 156 -> 103, 384 / 768 129 -> 115, 768 / 768 261 -> 194, 1024 / 2048 372 -> 248, 3072 / 768 1164 -> 716, 4096 / 3302
+// 2306 -> 1237, 8192 / 2048 6022 -> 4262; 5734 / 7168 13319 -> 4310 and 9216 / 3072 8974 -> 6908 when the chain was 20 % slower; with
+// two levels of blocks 12288 / 4096 14735 -> 16072.
+constexpr int64_t kSolveOneMinN = 256, kSolveOneMaxN = kOuterMinN - 1;
 // A step's recoveries: modules up to this width.  The sign select of the z-update turns differences of rounding into differences of
 // the recovered weights; the recoveries of 7168 x 28672 (8192 tokens, five iterations) by the other form's roundings move W1 by
 // 1.3 %, as far as both are from 64 bits (1.5 %).  4096 x 16384 on 4096 tokens: 0.8 %.

@@ -7,14 +7,22 @@
 //   r >= nblk: the forward-substituted right-hand sides Y.
 // A tile is one task of one thread block.  It takes its entry of [G; I; R] less sum_k tile(r, k) L(j, k)^T over the k that exist to
 // its left (left-looking: the running value stays in registers, nothing is read back and rewritten), and
-//   D(j)    : factorises the block on the diagonal and inverts the factor (DiagTiles): X(j, j);
+//   the chain: factorises the blocks on the diagonal and inverts the factor (DiagTiles): X(j, j), then the tile below it and its
+//             part of the next diagonal block's sum, all in one thread block (their sums over k < j come from other blocks, PRE);
 //   T(r, j) : multiplies by X(j, j) = inv(L_jj)^T;
 //   W(r, j) : sum_k Y(r, k) X(j, k)^T over k >= j, the result (last, when all columns are there).
-// So there is no backward sweep, a serial chain of its own, and what follows a diagonal block (its column's next tile, the next
-// block's last update) waits for flags of its own tiles, not for launches.
+// So there is no backward sweep, a serial chain of its own, and what follows a diagonal block waits for flags of its own tiles, not for
+// launches.
 //
-// Tasks are taken by a counter in an order in which every task comes after those it reads.  A block that waits therefore waits for
-// a task that a running block has: any number of resident blocks makes progress, beside whatever else runs on the GPU.
+// What bounds it: up to about 6000 unknowns the chain, 28 us per 128 unknowns (elimination 16, X and the tile below it into operand
+// form 2, their product 2.2, its result into operand form 1, the diagonal block's update 2.2; as one task per diagonal block, handed on
+// through memory, 36); above, the loads of the products (192 KB per two tiles' product, 1.6 us, as much as the tensor core takes for
+// operands of 128 rows).  3072 unknowns and 768 right-hand sides: 1164 us as launches per block column, 1015 with a task per
+// diagonal block, 716.
+//
+// Tasks are taken by a counter in an order in which every task comes after those it reads (the chain, first, runs beside them).  A block
+// that waits therefore waits for a task that a running block has: two resident blocks make progress, beside whatever else runs on
+// the GPU, and a wait that runs out ends the launch with a status.
 //
 // Every product of two tiles is the six part products of weight >= 2^-16, hi.hi in one accumulator of 128 columns of tensor memory
 // and the five small ones in a second: the tensor core truncates its sums, so what is added one after the other to a sum of full
@@ -37,8 +45,11 @@ constexpr uint32_t BOX = 64 * TB * 2;                     // 64 columns of 128 r
 constexpr uint32_t OPER = 3 * BOX;                        // the three parts of 64 columns: 48 KB
 constexpr uint32_t SLOT = 2 * OPER;                       // both operands of a half chunk (64 of K)
 constexpr uint32_t DATA = 2 * SLOT;
-constexpr uint32_t NBARS = 10;
-constexpr size_t SMEM = DATA + 1024 /*alignment*/ + (NBARS + Diag::BARS) * 8 + 4 * TB * sizeof(float) /*row maxima*/;
+constexpr uint32_t PRE_BYTES = TB * TB * 4;
+constexpr uint32_t PRE_AT = (uint32_t)(Diag::SMEM - Diag::BARS * 8);   // chain block: a tile's sum, behind DiagTiles' arrays
+constexpr uint32_t AREA = PRE_AT + PRE_BYTES > DATA ? PRE_AT + PRE_BYTES : DATA;
+constexpr uint32_t NBARS = 11;
+constexpr size_t SMEM = AREA + 1024 /*alignment*/ + (NBARS + Diag::BARS) * 8 + 4 * TB * sizeof(float) /*row maxima*/;
 static_assert(Diag::SMEM - Diag::BARS * 8 <= DATA, "the diagonal block's arrays lie over the operand slots");
 constexpr uint32_t TMEM_COLS = 4 * TB;                    // two pairs of accumulators in turn
 constexpr long long WAIT_BUDGET = 4000000000LL;           // about two seconds
@@ -56,6 +67,7 @@ struct SolveParams {
   float* lead;                 // optional [m, .]: the solution of the leading lead_k x lead_k system
   int64_t ld_lead;
   int lead_k;
+  float* pre;                  // [2 nblk][128][128]: what the chain block takes over of a column (see TASK_PRE)
   uint32_t* flags;
   int32_t* status;
   const int32_t* skip;
@@ -122,44 +134,69 @@ __device__ __forceinline__ void split3x2(float x, float y, uint32_t (&o)[3]) {
   o[2] = *reinterpret_cast<uint32_t*>(&l);
 }
 
-// X(j, j) of DiagTiles as parts: D points at its first element
-struct PartsOut {
-  __nv_bfloat16* D;
-  int64_t ldp, np;
-  __device__ __forceinline__ void row(int i, int col, const float (&a)[32], bool zero) const {
-#pragma unroll
-    for (int c = 0; c < 32; c += 8) {
-      uint32_t o[4][3];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) split3x2(zero ? 0.f : a[c + 2 * e], zero ? 0.f : a[c + 2 * e + 1], o[e]);
-#pragma unroll
-      for (int z = 0; z < 3; ++z)
-        *reinterpret_cast<uint4*>(D + i * ldp + z * np + col + c) = make_uint4(o[0][z], o[1][z], o[2][z], o[3][z]);
-    }
-  }
-  __device__ __forceinline__ void zeros(int rb, int s, int lane) const {
-#pragma unroll
-    for (int c = 0; c < 32; c += 8)
-#pragma unroll
-      for (int z = 0; z < 3; ++z)
-        *reinterpret_cast<uint4*>(D + (s * 32 + lane) * ldp + z * np + rb * 32 + c) = make_uint4(0, 0, 0, 0);
-  }
-  __device__ __forceinline__ void tile(const float (&a)[32], const float*, bool, int rb, int s, int lane) const {
-    row(rb * 32 + lane, s * 32, a, false);
-  }
+// X(j, j) of DiagTiles is read where it lies in shared memory
+struct NoOut {
+  __device__ __forceinline__ void zeros(int, int, int) const {}
+  __device__ __forceinline__ void tile(const float (&)[32], const float*, bool, int, int, int) const {}
 };
+// 32 values of a row, from chunk u0 (8 columns) of its box on, as three parts in the layout of the operands: rows of 64 columns,
+// 128-byte swizzle, the parts a box apart
+__device__ __forceinline__ void put_parts(uint8_t* box, int row, int u0, const float (&v)[32]) {
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    uint32_t o[4][3];
+#pragma unroll
+    for (int w = 0; w < 4; ++w) split3x2(v[8 * u + 2 * w], v[8 * u + 2 * w + 1], o[w]);
+    uint8_t* at = box + row * 128 + (((u0 + u) ^ (row & 7)) << 4);
+#pragma unroll
+    for (int z = 0; z < 3; ++z) *reinterpret_cast<uint4*>(at + z * BOX) = make_uint4(o[0][z], o[1][z], o[2][z], o[3][z]);
+  }
+}
+// place of chunk q (4 columns) of row i in a tile's sum handed to the chain block: no bank conflicts for a row per lane
+__device__ __forceinline__ int pre_at(int i, int q) { return i * TB + ((q ^ (i & 31)) << 2); }
+// all of an operand area (two halves of 64 columns, three parts) to memory; one thread, up to the point where the area may be written again
+__device__ __forceinline__ void store_tile(const CUtensorMap* map, int part_cols, int col, int row, uint32_t src) {
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+#pragma unroll
+    for (int z = 0; z < 3; ++z) tma_store_2d(map, z * part_cols + col + h * 64, row, src + h * OPER + z * BOX);
+  bulk_commit();
+  asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+}
+// The six products of one pair of 16-wide slices, at the descriptors of their hi parts (a box apart: the other parts): hi.hi into d, the small
+// ones into d + TB; later = 0 for the first slice of a sum.
+__device__ __forceinline__ void mma_slice(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t later) {
+  mma(d, a, b, idesc, later);
+#pragma unroll
+  for (int s = 1; s < 6; ++s)
+    mma(d + TB, a + part_a(s) * (BOX >> 4), b + part_b(s) * (BOX >> 4), idesc, s > 1 ? 1u : later);
+}
+// the tile whose last product is multiplied by X(j, j): A (K-major) at a, X at b (rows of K, columns contiguous)
+__device__ __forceinline__ void mma_by_x(uint32_t d, uint32_t a, uint32_t b) {
+  const uint64_t bd = make_smem_desc(b, false, OPER);
+#pragma unroll 1
+  for (int k = 0; k < 8; ++k)
+    mma_slice(d, make_smem_desc(a + (k >> 2) * OPER + (k & 3) * 32, true, 0), bd + k * (16 * 128 >> 4), instr_desc(false), k > 0 ? 1u : 0u);
+}
+// half h (64 of K) of the product of two tiles
+__device__ __forceinline__ void mma_half(uint32_t d, uint32_t a, uint32_t b, int h) {
+  const uint64_t ad = make_smem_desc(a, true, 0), bd = make_smem_desc(b, true, 0);
+#pragma unroll 1
+  for (int k = 0; k < 4; ++k) mma_slice(d, ad + k * 2, bd + k * 2, instr_desc(true), h > 0 || k > 0 ? 1u : 0u);
+}
 
-enum TaskKind : int { TASK_D = 0, TASK_T = 1, TASK_W = 2 };
+enum TaskKind : int { TASK_CHAIN = 0, TASK_T = 1, TASK_W = 2, TASK_PRE = 3 };
 struct Task {
   int kind, R, j;       // row block (in rows of P), column block
   int k0, k1;           // tiles to the left (W: of the sum)
   int lead;             // W: k of the leading system's last block (-1: none)
+  int pre;              // PRE: its place
 };
-// D(0); then column by column: the tile below the diagonal and the next diagonal block first (the chain), the factor's other
-// tiles, the right-hand sides, X.  nblk + mb tasks a column (one less in the last), then the W, longest sums first.
+// The chain; then column by column: what it takes over of the tile below the diagonal and of the next diagonal block (their sums over
+// k < j), the factor's other tiles, the right-hand sides, X.  nblk + mb tasks a column (one less in the last), then the W, longest sums first.
 __device__ __forceinline__ Task task_of(const SolveParams& p, int t) {
   Task q;
-  q.lead = -1;
+  q.lead = q.pre = -1;
   const int C = p.nblk + p.mb, cols = p.nblk * C;
   if (t >= cols) {
     const int u = t - cols;
@@ -175,19 +212,107 @@ __device__ __forceinline__ Task task_of(const SolveParams& p, int t) {
   q.j = t == 0 ? 0 : (t - 1) / C;
   const int idx = t == 0 ? 0 : (t - 1) % C, below = p.nblk - 1 - q.j, rest = below > 0 ? idx - (below + 1) : idx;
   if (t == 0) {
-    q.kind = TASK_D;
+    q.kind = TASK_CHAIN;
     q.R = 0;
   } else if (rest >= 0) {
     q.R = rest < p.mb ? p.nblk + rest : rest - p.mb;
-  } else if (idx == 1) {
-    q.kind = TASK_D;
-    q.R = ++q.j;
   } else {
-    q.R = q.j + (idx == 0 ? 1 : idx);
+    q.R = q.j + (idx <= 1 ? 1 : idx);
+    if (idx <= 1) {
+      q.kind = TASK_PRE;
+      q.pre = 2 * q.j + idx;
+    }
   }
   q.k0 = q.R < q.j ? q.R : 0;
   q.k1 = q.j;
+  if (q.kind == TASK_PRE && idx == 1) q.j = q.R;      // the diagonal block (j + 1, j + 1), also over k < j
   return q;
+}
+
+__device__ __forceinline__ float ld_shared(uint32_t at) {
+  float v;
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(at) : "memory");
+  return v;
+}
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  mbar_expect_tx(bar, bytes);
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
+               : "memory");
+}
+// A thread's place: of the epilogue's threads (warps from EPI0 on) row i, columns 32 g .. + 31 of a tile.  Volatile: formed where it is called.
+__device__ __noinline__ void eliminate_block(uint32_t off, uint32_t bars, int j, int nb, int32_t* status) {
+  extern __shared__ uint8_t smem_raw[];
+  int t;
+  asm volatile("mov.u32 %0, %%tid.x;" : "=r"(t));
+  Diag::eliminate<true>(t, reinterpret_cast<float*>(smem_raw + off), bars, (uint32_t)j & 1u, nullptr, 0, nb, NoOut{}, (int64_t)j * TB, status);
+}
+struct Place {
+  int warp, lane, g, i;
+  uint32_t data, tmem;
+  uint8_t* ptr;
+};
+__device__ __forceinline__ Place place(uint8_t* smem, const volatile uint32_t* s_tmem) {
+  Place q;
+  int t;
+  uint32_t zero;
+  asm volatile("mov.u32 %0, %%tid.x;" : "=r"(t));
+  asm volatile("mov.u32 %0, 0;" : "=r"(zero));
+  q.warp = t >> 5;
+  q.lane = t & 31;
+  q.g = (q.warp - EPI0) >> 2;
+  q.i = (q.warp & 3) * 32 + q.lane;
+  const uint32_t raw = smem_u32(smem), up = (raw + zero + 1023u) & ~1023u;
+  q.data = up;
+  q.ptr = smem + (up - raw);
+  q.tmem = *s_tmem;
+  return q;
+}
+// waits for the product of two tiles (both its accumulators at `at` and at + TB): f(c, value) for the thread's 32 columns
+template <typename F>
+__device__ __forceinline__ bool read_sum(uint32_t tfull, uint32_t tempty, uint32_t parity, uint32_t at, int lane,
+                                         volatile int* abort_flag, long long budget, F&& f) {
+  const bool there = __all_sync(0xffffffffu, mbar_wait(tfull, parity, abort_flag, budget));
+  tc_fence_after();
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    uint32_t hi[16], lo[16];
+    tc_ld16(at + h * 16, hi);
+    tc_ld16(at + TB + h * 16, lo);
+    tc_wait_ld();
+#pragma unroll
+    for (int c = 0; c < 16; ++c) f(h * 16 + c, __uint_as_float(hi[c]) + __uint_as_float(lo[c]));
+  }
+  tc_fence_before();
+  __syncwarp();
+  if (lane == 0) arrive(tempty);
+  return there;
+}
+// until a flag is set
+__device__ __forceinline__ bool wait_flag(const uint32_t* f, volatile int* abort_flag, long long budget) {
+  const long long t0 = clock64();
+  while (ld_acquire(f) == 0u) {
+    if (*abort_flag != 0 || clock64() - t0 > budget) {
+      *abort_flag = 1;
+      return false;
+    }
+  }
+  return true;
+}
+// a block on the diagonal, where DiagTiles expects its tiles: zero above the diagonal, an identity beyond nb
+__device__ __forceinline__ void stage_block(const Place& at, const float (&v)[32], int nb) {
+  if (at.g > (at.warp & 3)) return;
+  float* dst = reinterpret_cast<float*>(at.ptr) + Diag::staged_at(at.i, at.g * 32);
+#pragma unroll
+  for (int c = 0; c < 32; c += 4) {
+    float u[4];
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+      const int col = at.g * 32 + c + w;
+      u[w] = col > at.i ? 0.f : at.i >= nb ? (col == at.i ? 1.f : 0.f) : v[c + w];
+    }
+    *reinterpret_cast<float4*>(dst + c) = make_float4(u[0], u[1], u[2], u[3]);
+  }
 }
 
 __global__ void __launch_bounds__(THREADS, 1)
@@ -200,15 +325,16 @@ solve_tc_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
   extern __shared__ uint8_t smem_raw[];
   __shared__ uint32_t s_tmem;
   __shared__ int s_abort, s_ticket[2];
-  const uint32_t raw = smem_u32(smem_raw), data = (raw + 1023u) & ~1023u, bars = data + DATA;
+  const uint32_t raw = smem_u32(smem_raw), data = (raw + 1023u) & ~1023u, bars = data + AREA;
   uint8_t* const data_ptr = smem_raw + (data - raw);
   auto full = [&](int h) { return bars + 8u * h; };              // a half chunk has landed
   auto empty = [&](int h) { return bars + 8u * (2 + h); };       // its products have read it
   auto tfull = [&](int b) { return bars + 8u * (4 + b); };       // an accumulator is complete
   auto tempty = [&](int b) { return bars + 8u * (6 + b); };      // and read
   const uint32_t xfull = bars + 8u * 8, aready = bars + 8u * 9;  // X(j, j) has landed; the left operand is written
+  const uint32_t xfree = bars + 8u * 10;                         // chain: X(j, j) has left (barriers in this order there too)
   const uint32_t dbars = bars + 8u * NBARS;
-  float* const row_max = reinterpret_cast<float*>(data_ptr + DATA + (NBARS + Diag::BARS) * 8);   // [4][128]
+  float* const row_max = reinterpret_cast<float*>(data_ptr + AREA + (NBARS + Diag::BARS) * 8);   // [4][128]
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   volatile int* abort_flag = &s_abort;
   if (threadIdx.x == 0) {
@@ -220,6 +346,7 @@ solve_tc_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
       mbar_init(tempty(h), EPI_WARPS);
     }
     mbar_init(xfull, 1);
+    mbar_init(xfree, 1);
     mbar_init(aready, EPI_WARPS);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_smem();
@@ -237,10 +364,136 @@ solve_tc_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
   wait_for_predecessors();
 
   uint32_t* const flags = p.flags + kFlags0;
+  uint32_t* const pre_flags = flags + (int64_t)p.nblk * (p.nblk + p.mb);
   const int total = p.nblk * (p.nblk + 2 * p.mb), np = p.nblk * TB;
-  uint32_t kc = 0, cc = 0, xc = 0, dc = 0;   // chunks, accumulators, final products and diagonal blocks so far (the same in every role)
+  // chunks, accumulators, written operands, loads of X(j, j) so far (the same in every role)
+  uint32_t kc = 0, cc = 0, xc = 0, fc = 0;
+  // epilogue threads: row i, columns 32 g .. + 31 of a tile
+  const int g = (warp - EPI0) >> 2, i = (warp & 3) * 32 + lane;
+  const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(g * 32);
+  // the next product of two tiles: f(c, value) for this thread's 32 columns
+  auto sum_of = [&](uint32_t cl, auto&& f) {
+    return read_sum(tfull(cl & 1u), tempty(cl & 1u), (cl >> 1) & 1u, taddr + (cl & 1u) * 2 * TB, lane, abort_flag, p.budget, f);
+  };
   if (threadIdx.x == 0) s_ticket[0] = (int)atomicAdd(p.flags, 1u);
   __syncthreads();
+  if (s_ticket[0] == 0) {
+    // ------------------------------------------------------------------ the chain: all diagonal blocks, one after the other
+    // Areas: X(j, j) lies where DiagTiles worked, the tile below it in the second slot; its sum comes in behind DiagTiles' arrays.  The
+    // elimination takes nearly all registers, and what is spilled goes to the second-level cache, since shared memory has taken
+    // the first (40 us a block with 500 bytes spilled inside it, 30 with 130).  So it is a call of its own, and everything but j
+    // is formed anew behind it (Place).
+    Place at = place(smem_raw, &s_tmem);
+    if (at.warp >= EPI0) {
+      float v[32];
+#pragma unroll
+      for (int c = 0; c < 32; ++c) {
+        const int col = at.g * 32 + c;
+        v[c] = at.i < p.nn && col <= at.i && col < p.nn ? p.A[(int64_t)at.i * p.lda + col] : 0.f;
+      }
+      stage_block(at, v, p.nn < TB ? p.nn : TB);
+    }
+    for (int j = 0; j < p.nblk; ++j) {
+      __syncthreads();
+      if (*abort_flag != 0) break;
+      {
+        const int nb = p.nn - j * TB < TB ? p.nn - j * TB : TB;
+eliminate_block(at.data - smem_u32(smem_raw), at.data + AREA + 8u * NBARS, j, nb, p.status);
+      }
+      at = place(smem_raw, &s_tmem);
+      const bool more = j + 1 < p.nblk;
+      const uint32_t par = (uint32_t)j & 1u, bars_j = at.data + AREA;
+      const uint32_t tfull0 = bars_j + 8u * 4, tempty0 = bars_j + 8u * 6, xfull_j = bars_j + 8u * 8, aready_j = bars_j + 8u * 9,
+                     xfree_j = bars_j + 8u * 10;
+      uint32_t* const flags_j = p.flags + kFlags0;
+      uint32_t* const pre_j = flags_j + (int64_t)p.nblk * (p.nblk + p.mb) + 2 * j;
+      const float* const sums = p.pre + (int64_t)(2 * j) * (TB * TB);
+      if (at.warp == 0 && more && at.lane == 0 && wait_flag(pre_j, abort_flag, p.budget)) {     // (its tile of L is done first)
+        asm volatile("fence.proxy.async;" ::: "memory");
+        bulk_load(at.data + PRE_AT, sums, PRE_BYTES, xfull_j);
+      }
+      __syncwarp();
+      __syncthreads();                       // X is complete
+      __syncwarp();
+      if (at.warp >= EPI0) {
+        float v[32];
+        const int ns = (p.nn - j * TB + 31) / 32;
+        if (at.g >= (at.warp & 3) && at.g < ns) {
+          const uint32_t col = at.data + 4u * (uint32_t)((TB + at.g * 32) * Diag::P + at.i);
+#pragma unroll
+          for (int c = 0; c < 32; ++c) v[c] = ld_shared(col + 4u * c * Diag::P);
+        } else {
+          const int one = at.g >= ns ? at.i - at.g * 32 : -1;    // beyond the matrix: an identity
+#pragma unroll
+          for (int c = 0; c < 32; ++c) v[c] = c == one ? 1.f : 0.f;
+        }
+        epi_sync();                          // and read
+        put_parts(at.ptr + (at.g >> 1) * OPER, at.i, (at.g & 1) * 4, v);
+        if (more) {
+          mbar_wait(xfull_j, par, abort_flag, p.budget);
+          const float* src = reinterpret_cast<const float*>(at.ptr + PRE_AT);
+#pragma unroll
+          for (int c = 0; c < 32; c += 4) {
+            const float4 u = *reinterpret_cast<const float4*>(src + pre_at(at.i, at.g * 8 + c / 4));
+            v[c] = u.x; v[c + 1] = u.y; v[c + 2] = u.z; v[c + 3] = u.w;
+          }
+          epi_sync();                        // the sum lies where the operand is written
+          put_parts(at.ptr + SLOT + (at.g >> 1) * OPER, at.i, (at.g & 1) * 4, v);
+        }
+      }
+      fence_async_smem();
+      __syncthreads();
+      if (*abort_flag != 0) break;
+      if (at.warp == 1 && more && at.lane == 0) {
+        bool ok = mbar_wait(tempty0, par ^ 1u, abort_flag, p.budget);
+        if (ok) {
+          tc_fence_after();
+          mma_by_x(at.tmem, at.data + SLOT, at.data);
+          commit(tfull0);
+          ok = mbar_wait(tempty0 + 8u, par ^ 1u, abort_flag, p.budget) && mbar_wait(aready_j, par, abort_flag, p.budget);
+          if (ok) {
+            tc_fence_after();
+#pragma unroll 1
+            for (int h = 0; h < 2; ++h) mma_half(at.tmem + 2 * TB, at.data + SLOT + h * OPER, at.data + SLOT + h * OPER, h);
+            commit(tfull0 + 8u);
+          }
+        }
+      } else if (at.warp == 2 && at.lane == 0) {
+        store_tile(&tmP, np, j * TB, j * TB, at.data);
+        arrive(xfree_j);
+        bulk_wait_all();
+        publish(flags_j + (int64_t)j * p.nblk + j);
+      } else if (at.warp == 3 && more && at.lane == 0) {
+        if (mbar_wait(aready_j, par, abort_flag, p.budget)) {
+          store_tile(&tmP, np, j * TB, (j + 1) * TB, at.data + SLOT);
+          bulk_wait_all();
+          publish(flags_j + (int64_t)(j + 1) * p.nblk + j);
+        }
+      } else if (at.warp >= EPI0 && more) {
+        const uint32_t taddr_j = at.tmem + ((uint32_t)((at.warp & 3) * 32) << 16) + (uint32_t)(at.g * 32);
+        float d[32];
+        const bool ok = read_sum(tfull0, tempty0, par, taddr_j, at.lane, abort_flag, p.budget, [&](int c, float u) { d[c] = u; });
+        put_parts(at.ptr + SLOT + (at.g >> 1) * OPER, at.i, (at.g & 1) * 4, d);
+        fence_async_smem();
+        __syncwarp();
+        if (ok && at.lane == 0) arrive(aready_j);
+        // the sum of the next diagonal block, while its last product is formed
+        wait_flag(pre_j + 1, abort_flag, p.budget);
+        __syncwarp();
+        const float4* src = reinterpret_cast<const float4*>(sums + TB * TB) + (at.warp - EPI0) * 32 + at.lane;
+#pragma unroll
+        for (int c = 0; c < 32; c += 4) {
+          const float4 u = src[c / 4 * (EPI_WARPS * 32)];
+          d[c] = u.x; d[c + 1] = u.y; d[c + 2] = u.z; d[c + 3] = u.w;
+        }
+        read_sum(tfull0 + 8u, tempty0 + 8u, par, taddr_j + 2 * TB, at.lane, abort_flag, p.budget, [&](int c, float u) { d[c] -= u; });
+        mbar_wait(xfree_j, par, abort_flag, p.budget);
+        stage_block(at, d, p.nn - (j + 1) * TB < TB ? p.nn - (j + 1) * TB : TB);
+      }
+      __syncwarp();
+    }
+    __syncthreads();
+  } else
   for (int turn = 0;; turn ^= 1) {
     const int ticket = s_ticket[turn];
     int* const next_ticket = &s_ticket[turn ^ 1];      // written while others may still read the first
@@ -250,13 +503,13 @@ solve_tc_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
     const int nq = tk.k1 - tk.k0 + (tk.lead >= 0 ? 1 : 0);
     const int masked = tk.lead >= 0 ? tk.lead - tk.k0 : -1;       // the chunk that reads the masked copy
     auto k_of = [&](int q) { return tk.k0 + (masked >= 0 && q > masked ? q - 1 : q); };
-    const int Brow = tk.kind == TASK_W ? tk.j : tk.kind == TASK_D ? tk.R : tk.j;
+    const bool same = tk.R == tk.j;      // both operands are the same tiles
     bool ok = true;
 
     if (warp == 0) {
       // ------------------------------------------------------------------ loads
       const uint32_t* fa = flags + (int64_t)tk.R * p.nblk;
-      const uint32_t* fb = flags + (int64_t)Brow * p.nblk;
+      const uint32_t* fb = flags + (int64_t)tk.j * p.nblk;
       // until tile k of both rows is there (lane l looks at k + l); known: how far the look reached
       int known = tk.k0;
       auto wait_tiles = [&](int k, int k1, bool both) {
@@ -283,18 +536,18 @@ solve_tc_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
       uint32_t kl = kc;
       for (int q = 0; q < nq && ok; ++q, ++kl) {
         const int k = k_of(q);
-        ok = wait_tiles(k, tk.k1, tk.kind != TASK_D);
+        ok = wait_tiles(k, tk.k1, !same);
         if (ok && lane == 0) {
           for (int h = 0; h < 2 && ok; ++h) {
             if (!mbar_wait(empty(h), (kl & 1u) ^ 1u, abort_flag, p.budget)) { ok = false; break; }
-            mbar_expect_tx(full(h), tk.kind == TASK_D ? OPER : SLOT);
+            mbar_expect_tx(full(h), same ? OPER : SLOT);
             const uint32_t dst = data + h * SLOT;
 #pragma unroll
             for (int z = 0; z < 3; ++z) {
               const int col = k * TB + h * 64;
               if (q == masked) tma_load_2d_local(dst + z * BOX, &tmY, z * TB + h * 64, (tk.R - p.nblk) * TB, full(h));
               else tma_load_2d_local(dst + z * BOX, &tmP, z * np + col, tk.R * TB, full(h));
-              if (tk.kind != TASK_D) tma_load_2d_local(dst + OPER + z * BOX, &tmP, z * np + col, Brow * TB, full(h));
+              if (!same) tma_load_2d_local(dst + OPER + z * BOX, &tmP, z * np + col, tk.j * TB, full(h));
             }
           }
         }
@@ -320,7 +573,6 @@ solve_tc_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
     } else if (warp == 1) {
       // ------------------------------------------------------------------ products
       if (lane == 0) {
-        const uint32_t idesc = instr_desc(true);
         uint32_t kl = kc, cl = cc;
         for (int q = 0; q < nq && ok; ++q, ++kl, ++cl) {
           const uint32_t d = tmem + (cl & 1u) * 2 * TB;
@@ -329,40 +581,26 @@ solve_tc_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
             ok = mbar_wait(full(h), kl & 1u, abort_flag, p.budget);
             if (!ok) break;
             tc_fence_after();
-            const uint32_t a = data + h * SLOT, b = tk.kind == TASK_D ? a : a + OPER;
-#pragma unroll
-            for (int s = 0; s < 6; ++s)
-#pragma unroll
-              for (int k = 0; k < 4; ++k)
-                mma(s > 0 ? d + TB : d, make_smem_desc(a + part_a(s) * BOX + k * 32, true, 0),
-                    make_smem_desc(b + part_b(s) * BOX + k * 32, true, 0), idesc, h > 0 || s > 1 || k > 0 ? 1u : 0u);
+            const uint32_t a = data + h * SLOT;
+            mma_half(d, a, same ? a : a + OPER, h);
             commit(empty(h));
           }
           if (ok) commit(tfull(cl & 1u));
         }
         if (tk.kind == TASK_T && ok) {
-          const uint32_t d = tmem + (cl & 1u) * 2 * TB, idx = instr_desc(false);
+          const uint32_t d = tmem + (cl & 1u) * 2 * TB;
           ok = mbar_wait(tempty(cl & 1u), ((cl >> 1) & 1u) ^ 1u, abort_flag, p.budget) &&
-               mbar_wait(aready, xc & 1u, abort_flag, p.budget) && mbar_wait(xfull, xc & 1u, abort_flag, p.budget);
+               mbar_wait(aready, xc & 1u, abort_flag, p.budget) && mbar_wait(xfull, fc & 1u, abort_flag, p.budget);
           if (ok) {
             tc_fence_after();
-#pragma unroll 1
-            for (int s = 0; s < 6; ++s) {
-              const int pa = part_a(s), pb = part_b(s);
-#pragma unroll
-              for (int k = 0; k < 8; ++k)
-                mma(s > 0 ? d + TB : d, make_smem_desc(data + (k >> 2) * OPER + pa * BOX + (k & 3) * 32, true, 0),
-                    make_smem_desc(data + SLOT + pb * BOX + k * 16 * 128, false, OPER), idx, s > 1 || k > 0 ? 1u : 0u);
-            }
+            mma_by_x(d, data, data + SLOT);
             commit(tfull(cl & 1u));
           }
         }
-        if (tk.kind != TASK_D) *next_ticket = (int)atomicAdd(p.flags, 1u);
+        *next_ticket = (int)atomicAdd(p.flags, 1u);
       }
     } else if (warp >= EPI0) {
       // ------------------------------------------------------------------ the running value, and what leaves
-      const int e = warp - EPI0, g = e >> 2, i = (warp & 3) * 32 + lane;   // row i, columns 32 g .. + 31 of the tile
-      const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(g * 32);
       const int col0 = tk.j * TB + g * 32;
       float s[32];
       {
@@ -382,69 +620,18 @@ solve_tc_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
           for (int c = 0; c < 32; ++c) s[c] = c < n_col ? src[c] : 0.f;
         }
       }
-      // the next product of two tiles: this thread's 32 values
-      auto sum_of = [&](uint32_t cl, float (&v)[32]) {
-        const bool there = mbar_wait(tfull(cl & 1u), (cl >> 1) & 1u, abort_flag, p.budget);
-        if (!__all_sync(0xffffffffu, there)) return false;
-        tc_fence_after();
-        const uint32_t at = taddr + (cl & 1u) * 2 * TB;
-        uint32_t hi[32];
-        tc_ld32(at, hi);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          uint32_t lo[16];
-          tc_ld16(at + TB + h * 16, lo);
-          tc_wait_ld();
-#pragma unroll
-          for (int c = 0; c < 16; ++c) v[h * 16 + c] = __uint_as_float(hi[h * 16 + c]) + __uint_as_float(lo[c]);
-        }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) arrive(tempty(cl & 1u));
-        return true;
-      };
       uint32_t cl = cc;
       for (int q = 0; q < nq && ok; ++q, ++cl) {
-        float r[32];
-        ok = sum_of(cl, r);
-        if (!ok) break;
-        if (q == masked) {
+        if (q != masked) {
+          ok = sum_of(cl, [&](int c, float v) { s[c] -= v; });
+        } else {
           // the leading system's solution ends here
           const int64_t row = (int64_t)(tk.R - p.nblk) * TB + i;
-          if (row < p.m) {
-            float* dst = p.lead + row * p.ld_lead + col0;
-#pragma unroll
-            for (int c = 0; c < 32; ++c)
-              if (col0 + c < p.lead_k) dst[c] = r[c] - s[c];
-          }
-        } else {
-#pragma unroll
-          for (int c = 0; c < 32; ++c) s[c] -= r[c];
+          float* dst = p.lead + row * p.ld_lead + col0;
+          const int n_out = row < p.m ? p.lead_k - col0 : 0;
+          ok = sum_of(cl, [&](int c, float v) { if (c < n_out) dst[c] = v - s[c]; });
         }
       }
-      // the three parts of this thread's values as a K-major operand in the first slot (also the layout in which they leave)
-      const uint32_t box_row = (uint32_t)(g >> 1) * OPER + (uint32_t)i * 128u;
-      auto put = [&](float (&v)[32]) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          uint32_t o[4][3];
-#pragma unroll
-          for (int w = 0; w < 4; ++w) split3x2(v[8 * u + 2 * w], v[8 * u + 2 * w + 1], o[w]);
-          const uint32_t at = box_row + ((((uint32_t)(g & 1) * 4u + u) ^ (uint32_t)(i & 7)) << 4);
-#pragma unroll
-          for (int z = 0; z < 3; ++z)
-            *reinterpret_cast<uint4*>(data_ptr + at + z * BOX) = make_uint4(o[0][z], o[1][z], o[2][z], o[3][z]);
-        }
-        fence_async_smem();
-      };
-      auto leave = [&](const CUtensorMap* map, int part_cols, int col, int row) {     // one thread
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-          for (int z = 0; z < 3; ++z) tma_store_2d(map, z * part_cols + col + h * 64, row, data + h * OPER + z * BOX);
-        bulk_commit();
-        bulk_wait_all();
-      };
       if (tk.kind == TASK_T) {
         // Rows of tiny values are brought to the order of one by a power of two: below 2^-110 the low parts would be cut off.
         float top = 0.f, back = 1.f;
@@ -461,28 +648,35 @@ solve_tc_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
             for (int c = 0; c < 32; ++c) s[c] *= up;
           }
         }
+        uint8_t* const box = data_ptr + (g >> 1) * OPER;
         if (ok) {
-          put(s);
+          put_parts(box, i, (g & 1) * 4, s);
+          fence_async_smem();
           __syncwarp();
           if (lane == 0) arrive(aready);
-          ok = sum_of(cl, s);
-#pragma unroll
-          for (int c = 0; c < 32; ++c) s[c] *= back;
+          ok = sum_of(cl, [&](int c, float v) { s[c] = v * back; });
         }
-        if (ok) put(s);
+        if (ok) {
+          put_parts(box, i, (g & 1) * 4, s);
+          fence_async_smem();
+        }
         epi_sync();
-        const bool all = *abort_flag == 0;
-        if (all && threadIdx.x == EPI0 * 32) leave(&tmP, np, tk.j * TB, tk.R * TB);
+        const bool one = threadIdx.x == EPI0 * 32 && *abort_flag == 0;
+        if (one) store_tile(&tmP, np, tk.j * TB, tk.R * TB, data);
         if (p.lead != nullptr && tk.R >= p.nblk && tk.j == (p.lead_k - 1) / TB) {
           // copy of the right-hand sides' last block of the leading system, zero beyond it
           epi_sync();
 #pragma unroll
           for (int c = 0; c < 32; ++c) s[c] = col0 + c < p.lead_k ? s[c] : 0.f;
-          put(s);
+          put_parts(box, i, (g & 1) * 4, s);
+          fence_async_smem();
           epi_sync();
-          if (all && threadIdx.x == EPI0 * 32) leave(&tmY, TB, 0, (tk.R - p.nblk) * TB);
+          if (one) store_tile(&tmY, TB, 0, (tk.R - p.nblk) * TB, data);
         }
-        if (all && threadIdx.x == EPI0 * 32) publish(flags + (int64_t)tk.R * p.nblk + tk.j);
+        if (one) {
+          bulk_wait_all();
+          publish(flags + (int64_t)tk.R * p.nblk + tk.j);
+        }
       } else if (tk.kind == TASK_W) {
         const int64_t row = (int64_t)(tk.R - p.nblk) * TB + i;
         if (ok && row < p.m) {
@@ -497,37 +691,24 @@ solve_tc_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
               if (col0 + c < p.nn) dst[c] = -s[c];
           }
         }
-      } else if (g <= (warp & 3)) {
-        // the block on the diagonal, where DiagTiles expects its tiles
-        const int nb = p.nn - tk.j * TB < TB ? p.nn - tk.j * TB : TB;
-        float* dst = reinterpret_cast<float*>(data_ptr) + Diag::staged_at(i, g * 32);
+      } else {
+        // for the chain block
+        // (a diagonal block thread by thread, as it is read; the tile below one for a copy to shared memory)
+        float* dst = p.pre + (int64_t)tk.pre * (TB * TB);
 #pragma unroll
-        for (int c = 0; c < 32; ++c) {
-          const int col = g * 32 + c;
-          s[c] = col > i ? 0.f : i >= nb ? (col == i ? 1.f : 0.f) : s[c];
+        for (int c = 0; c < 32; c += 4) {
+          const int at = same ? (c / 4 * (EPI_WARPS * 32) + threadIdx.x - EPI0 * 32) * 4 : pre_at(i, g * 8 + c / 4);
+          *reinterpret_cast<float4*>(dst + at) = make_float4(s[c], s[c + 1], s[c + 2], s[c + 3]);
         }
-#pragma unroll
-        for (int c = 0; c < 32; c += 4) *reinterpret_cast<float4*>(dst + c) = make_float4(s[c], s[c + 1], s[c + 2], s[c + 3]);
+        epi_sync();
+        if (threadIdx.x == EPI0 * 32 && *abort_flag == 0) publish(pre_flags + tk.pre);
       }
     }
     __syncwarp();            // (the block's barriers count whole warps)
     kc += (uint32_t)nq;
     cc += (uint32_t)nq + (tk.kind == TASK_T ? 1u : 0u);
     xc += tk.kind == TASK_T ? 1u : 0u;
-    if (tk.kind == TASK_D) {
-      __syncthreads();
-      if (*abort_flag == 0) {                    // (set before the barrier only: the same for every thread)
-        const int nb = p.nn - tk.j * TB < TB ? p.nn - tk.j * TB : TB;
-        const PartsOut out{p.P + (int64_t)tk.j * TB * p.ldp + tk.j * TB, p.ldp, np};
-        Diag::eliminate<true>(reinterpret_cast<float*>(data_ptr), dbars, dc & 1u, nullptr, 0, nb, out, (int64_t)tk.j * TB, p.status);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-          publish(flags + (int64_t)tk.j * p.nblk + tk.j);
-          *next_ticket = (int)atomicAdd(p.flags, 1u);
-        }
-        ++dc;                                    // (a narrower block is the last one: nothing waits on its barriers again)
-      }
-    }
+    fc += tk.kind == TASK_T ? 1u : 0u;
     fence_async_smem();
     __syncthreads();
     if (*abort_flag != 0) break;
@@ -550,7 +731,7 @@ solve_tc_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
 
 size_t solve_tc_flag_words(int64_t n, int64_t m) {
   const size_t nblk = (size_t)ceil_div(n, (int64_t)TB), mb = (size_t)ceil_div(m, (int64_t)TB);
-  return kFlags0 + nblk * (nblk + mb);
+  return kFlags0 + nblk * (nblk + mb) + 2 * nblk;
 }
 
 sp_status solve_tc(const float* A, int64_t nn, int64_t m, int64_t lda, float* W, int64_t ldw, const SolveOneBufs& b,
@@ -572,6 +753,7 @@ sp_status solve_tc(const float* A, int64_t nn, int64_t m, int64_t lda, float* W,
   p.lead = lead;
   p.ld_lead = ld_lead;
   p.lead_k = (int)lead_k;
+  p.pre = b.pre;
   p.flags = b.flags;
   p.status = status_dev;
   p.skip = skip_flag();
