@@ -1669,11 +1669,12 @@ struct ValueRefitPlan {
   void* R;      // bf16 mode: per head of the group [cap, 2 dq]: regressors (d columns) beside the head's Aattn (d_h columns),
                 // hi | lo; fp32 mode: regressors of one head, [cap, d]
   float* G;     // per kept head [d + d_h, d]: sum over sequences of R^T R (lower triangle) and, below it, of Aattn_i^T R
-  // the heads' systems solved together, in place in G (bf16 mode, d a multiple of the solver's block): see
-  // potrf_potrs_tc_batched
-  bool batched;
+  // the heads' systems solved together, in place in G (bf16 mode): solve_tc, or, for d a multiple of the solver's block that is not
+  // for it, potrf_potrs_tc_batched
+  bool batched, one;    // one: in one launch (solve_tc)
   float* dinv_all;
   void *P_all, *Xs_all;
+  uint32_t* flags_all;
   size_t bytes;
 };
 
@@ -1701,13 +1702,17 @@ ValueRefitPlan plan_value_refit(void* ws, int64_t d, int64_t H, int64_t T, int64
   }
   p.R = c.take_bytes(p.bf16 ? (size_t)p.hg * p.cap * 2 * p.dq * 2 : (size_t)p.cap * d * 4);
   p.G = c.take<float>((size_t)H * (d + p.dh) * d);
-  p.batched = p.bf16 && d % kCholTcNB == 0;
+  p.one = p.bf16 && solve_in_one(d);
+  p.batched = p.one || (p.bf16 && d % kCholTcNB == 0);
   p.dinv_all = nullptr;
   p.P_all = p.Xs_all = nullptr;
+  p.flags_all = nullptr;
   if (p.batched) {
+    const size_t np = (size_t)chol_tc_pad(d);
     p.dinv_all = c.take<float>((size_t)H * dinv_elems(d));
-    p.P_all = c.take_bytes((size_t)H * (d + p.dh) * 3 * d * 2);
+    p.P_all = c.take_bytes((size_t)H * (np + (size_t)chol_tc_pad(p.dh)) * 3 * np * 2);
     p.Xs_all = c.take_bytes((size_t)H * 2 * p.dh * 3 * kCholTcNB * 2);
+    p.flags_all = c.take<uint32_t>((size_t)H * solve_tc_flag_words(d, p.dh));
   }
   p.bytes = align_up(c.off, 256);
   return p;
@@ -1842,8 +1847,15 @@ sp_status sp_mha_value_refit(const sp_mha_module* m, const sp_mha_state* st, con
     CU(add_ridge_batched(p.G, g_bs, d, (int)nk, rho, rho_relative != 0, s));
     {
       ProfScope prof(PK_SOLVE, (double)nk * ((double)d * d * d / 3.0 + 2.0 * (double)dh * d * d), 0.0, s);
-      SPCHK(potrf_potrs_tc_batched(p.G, d, dh, (int)nk, g_bs, p.dinv_all, (int64_t)dinv_elems(d), p.P_all, p.Xs_all,
-                                   status_dev, s));
+      // (an attention step 2048 wide, 16 kept heads: 14.7 ms with a launch per step over all systems, 14.05 in one launch; 768 wide, 6
+      // heads: 2.43 and 2.28)
+      if (p.one) {
+        const SolveOneBufs one{p.P_all, nullptr, p.dinv_all, p.flags_all};
+        SPCHK(solve_tc(p.G, d, dh, d, p.G + (size_t)d * d, d, one, nullptr, 0, 0, status_dev, s, (int)nk, g_bs));
+      } else {
+        SPCHK(potrf_potrs_tc_batched(p.G, d, dh, (int)nk, g_bs, p.dinv_all, (int64_t)dinv_elems(d), p.P_all, p.Xs_all,
+                                     status_dev, s));
+      }
     }
     for (int64_t i0 = 0; i0 < nk; i0 += kMaxHeadGroup)
       CU(mha_place_heads(p.G + (size_t)i0 * g_bs + (size_t)d * d, g_bs, dh, d,

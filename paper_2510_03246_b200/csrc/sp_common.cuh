@@ -366,6 +366,7 @@ sp_status potrs_right_tc(float* X, int64_t m, int64_t n, int64_t ldx, const void
 //   A: [nn + m, nn] fp32, lower triangle of G and the right-hand sides below it; W [m, nn] may be the latter's place.
 //   lead != nullptr: also the solution [m, lead_k] of the leading lead_k x lead_k system with the leading right-hand sides.
 //   P: bf16 [pad(nn) + pad(m), 3 pad(nn)], Y: bf16 [pad(m), 3 kCholTcNB], flags: solve_tc_flag_words(nn, m) words; pad = chol_tc_pad.
+//   batch > 1: that many systems, A and W a_bs elements apart, the other arrays one system's behind the other's (no lead).
 struct SolveOneBufs {
   void *P, *Y;
   float* pre;         // 2 ceil(nn / kCholTcNB) blocks of kCholTcNB^2
@@ -383,7 +384,8 @@ constexpr int64_t kSolveOneModule = 16384;
 inline bool solve_in_one(int64_t n) { return n > kSolveOneMinN && n <= kSolveOneMaxN; }
 size_t solve_tc_flag_words(int64_t n, int64_t m);
 sp_status solve_tc(const float* A, int64_t nn, int64_t m, int64_t lda, float* W, int64_t ldw, const SolveOneBufs& b,
-                   float* lead, int64_t ld_lead, int64_t lead_k, int32_t* status_dev, cudaStream_t stream);
+                   float* lead, int64_t ld_lead, int64_t lead_k, int32_t* status_dev, cudaStream_t stream, int batch = 1,
+                   int64_t a_bs = 0);
 
 // `batch` independent systems of one size n (a multiple of kCholTcNB) with m right-hand sides each, every step one launch
 // over all of them.  System b: A + b * a_bs = [n + m, n] fp32 (lower triangle of the matrix, then the right-hand sides

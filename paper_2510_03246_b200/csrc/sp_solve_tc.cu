@@ -59,7 +59,7 @@ constexpr int kFlags0 = 32;                               // flags[0]: the task 
 struct SolveParams {
   const float* A;              // [nn + m, nn] fp32: lower triangle of the system, right-hand sides below
   int64_t lda;
-  int nn, m, nblk, mb;
+  int nn, m, nblk, mb, group;
   __nv_bfloat16* P;
   int64_t ldp;                 // 3 np
   float* W;                    // [m, nn], may be the right-hand sides' own place
@@ -72,6 +72,8 @@ struct SolveParams {
   int32_t* status;
   const int32_t* skip;
   long long budget;
+  int64_t a_bs;                // distance of the systems' A (and W), systems = gridDim.y; the rest lies one system behind the other
+  int rows, flag_words;        // rows of P and words of flags of a system
 };
 
 __device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
@@ -185,15 +187,17 @@ __device__ __forceinline__ void mma_half(uint32_t d, uint32_t a, uint32_t b, int
   for (int k = 0; k < 4; ++k) mma_slice(d, ad + k * 2, bd + k * 2, instr_desc(true), h > 0 || k > 0 ? 1u : 0u);
 }
 
-enum TaskKind : int { TASK_CHAIN = 0, TASK_T = 1, TASK_W = 2, TASK_PRE = 3 };
+enum TaskKind : int { TASK_T = 0, TASK_W = 1, TASK_PRE = 2 };
 struct Task {
   int kind, R, j;       // row block (in rows of P), column block
   int k0, k1;           // tiles to the left (W: of the sum)
   int lead;             // W: k of the leading system's last block (-1: none)
   int pre;              // PRE: its place
 };
-// The chain; then column by column: what it takes over of the tile below the diagonal and of the next diagonal block (their sums over
-// k < j), the factor's other tiles, the right-hand sides, X.  nblk + mb tasks a column (one less in the last), then the W, longest sums first.
+// The chain; then groups of p.group columns.  A group begins with the tiles that its own columns need: what the chain takes over of the
+// tile below a diagonal block and of the next diagonal block (their sums over k < j), and the factor's tiles down to the first row
+// behind the group; then row by row the group's tiles of the rows below, of the right-hand sides and of X.  nblk + mb tasks a
+// column (one less in the last), then the W, longest sums first.
 __device__ __forceinline__ Task task_of(const SolveParams& p, int t) {
   Task q;
   q.lead = q.pre = -1;
@@ -208,24 +212,40 @@ __device__ __forceinline__ Task task_of(const SolveParams& p, int t) {
     if (p.lead != nullptr && q.j * TB < p.lead_k) q.lead = (p.lead_k - 1) / TB;
     return q;
   }
+  // (t > 0: the chain is not a task of this kind)
+  const int j0 = (t - 1) / (p.group * C) * p.group, n_col = p.nblk - j0 < p.group ? p.nblk - j0 : p.group;
+  const int last = j0 + p.group < p.nblk - 1 ? j0 + p.group : p.nblk - 1;     // last row of the first part
+  int idx = t - 1 - j0 * C;
   q.kind = TASK_T;
-  q.j = t == 0 ? 0 : (t - 1) / C;
-  const int idx = t == 0 ? 0 : (t - 1) % C, below = p.nblk - 1 - q.j, rest = below > 0 ? idx - (below + 1) : idx;
-  if (t == 0) {
-    q.kind = TASK_CHAIN;
-    q.R = 0;
-  } else if (rest >= 0) {
-    q.R = rest < p.mb ? p.nblk + rest : rest - p.mb;
-  } else {
-    q.R = q.j + (idx <= 1 ? 1 : idx);
-    if (idx <= 1) {
-      q.kind = TASK_PRE;
-      q.pre = 2 * q.j + idx;
+  q.R = -1;
+  for (int j = j0; j < j0 + n_col && q.R < 0; ++j) {
+    const int pre = j + 1 < p.nblk ? 2 : 0, count = pre + (last - j - 1 > 0 ? last - j - 1 : 0);
+    if (idx < count) {
+      q.j = j;
+      q.R = idx < pre ? j + 1 : j + 2 + idx - pre;
+      if (idx < pre) {
+        q.kind = TASK_PRE;
+        q.pre = 2 * j + idx;
+      }
+    } else {
+      idx -= count;
+    }
+  }
+  if (q.R < 0) {
+    const int below = p.nblk - 1 - last, rows = below + p.mb + j0;
+    if (idx < rows * n_col) {
+      const int r = idx / n_col;
+      q.j = j0 + idx % n_col;
+      q.R = r < below ? last + 1 + r : r < below + p.mb ? p.nblk + r - below : r - below - p.mb;
+    } else {                                             // X within the group
+      idx -= rows * n_col;
+      for (q.j = j0 + 1; idx >= q.j - j0; ++q.j) idx -= q.j - j0;
+      q.R = j0 + idx;
     }
   }
   q.k0 = q.R < q.j ? q.R : 0;
   q.k1 = q.j;
-  if (q.kind == TASK_PRE && idx == 1) q.j = q.R;      // the diagonal block (j + 1, j + 1), also over k < j
+  if (q.kind == TASK_PRE && (q.pre & 1) != 0) q.j = q.R;  // the diagonal block (j + 1, j + 1), also over k < j
   return q;
 }
 
@@ -315,6 +335,8 @@ __device__ __forceinline__ void stage_block(const Place& at, const float (&v)[32
   }
 }
 
+// BATCH: gridDim.y systems.  (One system has a form of its own: registers are short.)
+template <bool BATCH>
 __global__ void __launch_bounds__(THREADS, 1)
 solve_tc_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CUtensorMap tmY, const SolveParams p) {
   dependents_may_launch();
@@ -323,6 +345,7 @@ solve_tc_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
     if (*p.skip != 0) return;
   }
   extern __shared__ uint8_t smem_raw[];
+  const int system = BATCH ? (int)blockIdx.y : 0;
   __shared__ uint32_t s_tmem;
   __shared__ int s_abort, s_ticket[2];
   const uint32_t raw = smem_u32(smem_raw), data = (raw + 1023u) & ~1023u, bars = data + AREA;
@@ -363,7 +386,8 @@ solve_tc_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
   const uint32_t tmem = s_tmem;
   wait_for_predecessors();
 
-  uint32_t* const flags = p.flags + kFlags0;
+  uint32_t* const ticket_of = p.flags + (int64_t)system * p.flag_words;
+  uint32_t* const flags = ticket_of + kFlags0;
   uint32_t* const pre_flags = flags + (int64_t)p.nblk * (p.nblk + p.mb);
   const int total = p.nblk * (p.nblk + 2 * p.mb), np = p.nblk * TB;
   // chunks, accumulators, written operands, loads of X(j, j) so far (the same in every role)
@@ -375,7 +399,7 @@ solve_tc_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
   auto sum_of = [&](uint32_t cl, auto&& f) {
     return read_sum(tfull(cl & 1u), tempty(cl & 1u), (cl >> 1) & 1u, taddr + (cl & 1u) * 2 * TB, lane, abort_flag, p.budget, f);
   };
-  if (threadIdx.x == 0) s_ticket[0] = (int)atomicAdd(p.flags, 1u);
+  if (threadIdx.x == 0) s_ticket[0] = (int)atomicAdd(ticket_of, 1u);
   __syncthreads();
   if (s_ticket[0] == 0) {
     // ------------------------------------------------------------------ the chain: all diagonal blocks, one after the other
@@ -389,7 +413,7 @@ solve_tc_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
 #pragma unroll
       for (int c = 0; c < 32; ++c) {
         const int col = at.g * 32 + c;
-        v[c] = at.i < p.nn && col <= at.i && col < p.nn ? p.A[(int64_t)at.i * p.lda + col] : 0.f;
+        v[c] = at.i < p.nn && col <= at.i && col < p.nn ? p.A[(int64_t)system * p.a_bs + (int64_t)at.i * p.lda + col] : 0.f;
       }
       stage_block(at, v, p.nn < TB ? p.nn : TB);
     }
@@ -405,9 +429,10 @@ eliminate_block(at.data - smem_u32(smem_raw), at.data + AREA + 8u * NBARS, j, nb
       const uint32_t par = (uint32_t)j & 1u, bars_j = at.data + AREA;
       const uint32_t tfull0 = bars_j + 8u * 4, tempty0 = bars_j + 8u * 6, xfull_j = bars_j + 8u * 8, aready_j = bars_j + 8u * 9,
                      xfree_j = bars_j + 8u * 10;
-      uint32_t* const flags_j = p.flags + kFlags0;
+      uint32_t* const flags_j = p.flags + (int64_t)system * p.flag_words + kFlags0;
       uint32_t* const pre_j = flags_j + (int64_t)p.nblk * (p.nblk + p.mb) + 2 * j;
-      const float* const sums = p.pre + (int64_t)(2 * j) * (TB * TB);
+      const float* const sums = p.pre + (int64_t)(2 * (system * p.nblk + j)) * (TB * TB);
+      const int row0 = system * p.rows;
       if (at.warp == 0 && more && at.lane == 0 && wait_flag(pre_j, abort_flag, p.budget)) {     // (its tile of L is done first)
         asm volatile("fence.proxy.async;" ::: "memory");
         bulk_load(at.data + PRE_AT, sums, PRE_BYTES, xfull_j);
@@ -459,13 +484,13 @@ eliminate_block(at.data - smem_u32(smem_raw), at.data + AREA + 8u * NBARS, j, nb
           }
         }
       } else if (at.warp == 2 && at.lane == 0) {
-        store_tile(&tmP, np, j * TB, j * TB, at.data);
+        store_tile(&tmP, np, j * TB, row0 + j * TB, at.data);
         arrive(xfree_j);
         bulk_wait_all();
         publish(flags_j + (int64_t)j * p.nblk + j);
       } else if (at.warp == 3 && more && at.lane == 0) {
         if (mbar_wait(aready_j, par, abort_flag, p.budget)) {
-          store_tile(&tmP, np, j * TB, (j + 1) * TB, at.data + SLOT);
+          store_tile(&tmP, np, j * TB, row0 + (j + 1) * TB, at.data + SLOT);
           bulk_wait_all();
           publish(flags_j + (int64_t)(j + 1) * p.nblk + j);
         }
@@ -504,6 +529,7 @@ eliminate_block(at.data - smem_u32(smem_raw), at.data + AREA + 8u * NBARS, j, nb
     const int masked = tk.lead >= 0 ? tk.lead - tk.k0 : -1;       // the chunk that reads the masked copy
     auto k_of = [&](int q) { return tk.k0 + (masked >= 0 && q > masked ? q - 1 : q); };
     const bool same = tk.R == tk.j;      // both operands are the same tiles
+    const int row0 = system * p.rows;
     bool ok = true;
 
     if (warp == 0) {
@@ -546,8 +572,8 @@ eliminate_block(at.data - smem_u32(smem_raw), at.data + AREA + 8u * NBARS, j, nb
             for (int z = 0; z < 3; ++z) {
               const int col = k * TB + h * 64;
               if (q == masked) tma_load_2d_local(dst + z * BOX, &tmY, z * TB + h * 64, (tk.R - p.nblk) * TB, full(h));
-              else tma_load_2d_local(dst + z * BOX, &tmP, z * np + col, tk.R * TB, full(h));
-              if (!same) tma_load_2d_local(dst + OPER + z * BOX, &tmP, z * np + col, tk.j * TB, full(h));
+              else tma_load_2d_local(dst + z * BOX, &tmP, z * np + col, row0 + tk.R * TB, full(h));
+              if (!same) tma_load_2d_local(dst + OPER + z * BOX, &tmP, z * np + col, row0 + tk.j * TB, full(h));
             }
           }
         }
@@ -566,7 +592,7 @@ eliminate_block(at.data - smem_u32(smem_raw), at.data + AREA + 8u * NBARS, j, nb
             for (int h = 0; h < 2; ++h)
 #pragma unroll
               for (int z = 0; z < 3; ++z)
-                tma_load_2d_local(data + SLOT + h * OPER + z * BOX, &tmP, z * np + tk.j * TB + h * 64, tk.j * TB, xfull);
+                tma_load_2d_local(data + SLOT + h * OPER + z * BOX, &tmP, z * np + tk.j * TB + h * 64, row0 + tk.j * TB, xfull);
           }
         }
       }
@@ -597,7 +623,7 @@ eliminate_block(at.data - smem_u32(smem_raw), at.data + AREA + 8u * NBARS, j, nb
             commit(tfull(cl & 1u));
           }
         }
-        *next_ticket = (int)atomicAdd(p.flags, 1u);
+        *next_ticket = (int)atomicAdd(ticket_of, 1u);
       }
     } else if (warp >= EPI0) {
       // ------------------------------------------------------------------ the running value, and what leaves
@@ -607,7 +633,7 @@ eliminate_block(at.data - smem_u32(smem_raw), at.data + AREA + 8u * NBARS, j, nb
         const int64_t row = tk.R < p.nblk ? (int64_t)tk.R * TB + i : (int64_t)p.nn + (int64_t)(tk.R - p.nblk) * TB + i;
         const bool have = tk.kind != TASK_W && tk.R >= tk.j &&
                           (tk.R < p.nblk ? row < p.nn : row < (int64_t)p.nn + p.m);
-        const float* src = p.A + row * p.lda + col0;
+        const float* src = p.A + (int64_t)system * p.a_bs + row * p.lda + col0;
         const int n_col = have ? (p.nn - col0 < 32 ? p.nn - col0 : 32) : 0;
         if (n_col == 32 && p.lda % 4 == 0) {
 #pragma unroll
@@ -662,7 +688,7 @@ eliminate_block(at.data - smem_u32(smem_raw), at.data + AREA + 8u * NBARS, j, nb
         }
         epi_sync();
         const bool one = threadIdx.x == EPI0 * 32 && *abort_flag == 0;
-        if (one) store_tile(&tmP, np, tk.j * TB, tk.R * TB, data);
+        if (one) store_tile(&tmP, np, tk.j * TB, row0 + tk.R * TB, data);
         if (p.lead != nullptr && tk.R >= p.nblk && tk.j == (p.lead_k - 1) / TB) {
           // copy of the right-hand sides' last block of the leading system, zero beyond it
           epi_sync();
@@ -680,7 +706,7 @@ eliminate_block(at.data - smem_u32(smem_raw), at.data + AREA + 8u * NBARS, j, nb
       } else if (tk.kind == TASK_W) {
         const int64_t row = (int64_t)(tk.R - p.nblk) * TB + i;
         if (ok && row < p.m) {
-          float* dst = p.W + row * p.ldw + col0;
+          float* dst = p.W + (int64_t)system * p.a_bs + row * p.ldw + col0;
           if (col0 + 32 <= p.nn && p.ldw % 4 == 0) {
 #pragma unroll
             for (int c = 0; c < 32; c += 4)
@@ -694,7 +720,7 @@ eliminate_block(at.data - smem_u32(smem_raw), at.data + AREA + 8u * NBARS, j, nb
       } else {
         // for the chain block
         // (a diagonal block thread by thread, as it is read; the tile below one for a copy to shared memory)
-        float* dst = p.pre + (int64_t)tk.pre * (TB * TB);
+        float* dst = p.pre + (int64_t)(2 * system * p.nblk + tk.pre) * (TB * TB);
 #pragma unroll
         for (int c = 0; c < 32; c += 4) {
           const int at = same ? (c / 4 * (EPI_WARPS * 32) + threadIdx.x - EPI0 * 32) * 4 : pre_at(i, g * 8 + c / 4);
@@ -735,8 +761,8 @@ size_t solve_tc_flag_words(int64_t n, int64_t m) {
 }
 
 sp_status solve_tc(const float* A, int64_t nn, int64_t m, int64_t lda, float* W, int64_t ldw, const SolveOneBufs& b,
-                   float* lead, int64_t ld_lead, int64_t lead_k, int32_t* status_dev, cudaStream_t stream) {
-  if (!solve_in_one(nn) || m < 1 || m > (1 << 24)) return SP_ERR_SHAPE;
+                   float* lead, int64_t ld_lead, int64_t lead_k, int32_t* status_dev, cudaStream_t stream, int batch, int64_t a_bs) {
+  if (!solve_in_one(nn) || m < 1 || m > (1 << 24) || batch < 1 || batch > 65535 || (batch > 1 && lead != nullptr)) return SP_ERR_SHAPE;
   SolveParams p;
   memset(&p, 0, sizeof(p));
   p.A = A;
@@ -745,6 +771,10 @@ sp_status solve_tc(const float* A, int64_t nn, int64_t m, int64_t lda, float* W,
   p.m = (int)m;
   p.nblk = (int)ceil_div(nn, (int64_t)TB);
   p.mb = (int)ceil_div(m, (int64_t)TB);
+  // Columns that are worked on together: a row's tiles are then read for all of them at about the same time, once from memory.  1 / 2 / 4
+  // columns, ms: 4096 unknowns, 3302 right-hand sides 1.25 / 1.24 / 1.31, 6553 / 4096 3.85 / 3.68 / 3.77, 8192 / 2048 4.41 / 4.09 /
+  // 3.96, 11000 / 2048 9.09 / 8.32 / 8.37; smaller ones, whose parts the second-level cache holds, equal.
+  p.group = p.nblk >= 60 ? 4 : p.nblk >= 40 ? 2 : 1;
   const int64_t np = (int64_t)p.nblk * TB, rows = np + (int64_t)p.mb * TB;
   p.P = reinterpret_cast<__nv_bfloat16*>(b.P);
   p.ldp = 3 * np;
@@ -757,19 +787,26 @@ sp_status solve_tc(const float* A, int64_t nn, int64_t m, int64_t lda, float* W,
   p.flags = b.flags;
   p.status = status_dev;
   p.skip = skip_flag();
+  p.a_bs = a_bs;
+  p.rows = (int)rows;
+  p.flag_words = (int)solve_tc_flag_words(nn, m);
+  if (rows * batch > 0x7fffffff) return SP_ERR_SHAPE;
   p.budget = wait_budget_cycles() > 0 ? wait_budget_cycles() : WAIT_BUDGET;
   CUtensorMap tmP, tmY;
-  if (!make_map(&tmP, false, b.P, 3 * np, rows, 3 * np, 64, TB) ||
-      !make_map(&tmY, false, b.Y, 3 * TB, (int64_t)p.mb * TB, 3 * TB, 64, TB))
+  if (!make_map(&tmP, false, b.P, 3 * np, rows * batch, 3 * np, 64, TB) ||
+      !make_map(&tmY, false, lead ? b.Y : b.P, 3 * TB, (int64_t)p.mb * TB, 3 * TB, 64, TB))      // (read for `lead` alone)
     return SP_ERR_CUDA;
   static PerDeviceOnce attr_once;
-  if (attr_once.run([] { return cudaFuncSetAttribute(solve_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM); }) !=
-      cudaSuccess)
+  if (attr_once.run([] {
+        const cudaError_t e = cudaFuncSetAttribute(solve_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
+        return e != cudaSuccess ? e : cudaFuncSetAttribute(solve_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
+      }) != cudaSuccess)
     return SP_ERR_CUDA;
-  if (cudaMemsetAsync(b.flags, 0, solve_tc_flag_words(nn, m) * sizeof(uint32_t), stream) != cudaSuccess) return SP_ERR_CUDA;
-  const int64_t tasks = (int64_t)p.nblk * (p.nblk + 2 * p.mb), sms = sm_count();
+  if (cudaMemsetAsync(b.flags, 0, (size_t)p.flag_words * batch * sizeof(uint32_t), stream) != cudaSuccess) return SP_ERR_CUDA;
+  // (a system has two blocks at least: the chain waits for sums of the others)
+  const int64_t tasks = (int64_t)p.nblk * (p.nblk + 2 * p.mb), share = sm_count() / batch, blocks = share > 2 ? share : 2;
   count_launch();
-  launch(solve_tc_kernel, (unsigned)(tasks < sms ? tasks : sms), THREADS, SMEM, stream, tmP, tmY, p);
+  launch(batch > 1 ? solve_tc_kernel<true> : solve_tc_kernel<false>, dim3((unsigned)(tasks < blocks ? tasks : blocks), (unsigned)batch), THREADS, SMEM, stream, tmP, tmY, p);
   return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ERR_CUDA;
 }
 
