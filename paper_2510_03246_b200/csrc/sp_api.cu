@@ -122,7 +122,13 @@ SolveBufs carve_solve(Carver& c, int64_t nmax, int64_t mmax, size_t tsize) {
   b.rho = c.take<double>(4);
   b.idx = c.take<int32_t>((size_t)nmax);
   // the system matrix and, right behind its nn x nn elements, the right-hand sides (one [nn + m, nn] array)
-  b.Gs = c.take_bytes((size_t)(nmax + mmax) * nmax * tsize);
+  // (fp64: and, for systems that are solved with the inverse of their factor, as many elements for that and the result)
+  size_t elems = (size_t)(nmax + mmax) * nmax;
+  if (tsize == 8) {
+    const size_t inv = (size_t)(nmax < kInverseMaxN ? nmax : kInverseMaxN);
+    elems = std::max(elems, 2 * inv * (inv + (size_t)std::max(nmax, mmax)));
+  }
+  b.Gs = c.take_bytes(elems * tsize);
   b.dinv = c.take_bytes(dinv_elems(nmax) * tsize);
   b.P = nullptr;
   b.Xs = nullptr;
@@ -177,8 +183,14 @@ sp_status ridge_core(const float* R, int64_t ldr, const float* G, int64_t ldg, i
     }
   } else {
     CU(gather_cols<T>(R, ldr, idx, m, nn, Rs, nn, stream));
-    CU(potrf_lower_f64(Gs, nn, nn, dinv, status, stream, assist, m));
-    CU(potrs_backward_f64(Rs, m, nn, nn, Gs, nn, dinv, stream, assist));
+    if (nn <= kInverseMaxN) {
+      T* X = Rs + (size_t)(m + nn) * nn;
+      CU(solve_inverse_f64(Gs, nn, m, dinv, X, status, stream, assist));
+      Rs = X;
+    } else {
+      CU(potrf_lower_f64(Gs, nn, nn, dinv, status, stream, assist, m));
+      CU(potrs_backward_f64(Rs, m, nn, nn, Gs, nn, dinv, stream, assist));
+    }
   }
   CU(scatter_cols<T>(Rs, nn, idx, m, nn, n_full, W, ldw, stream));
   return SP_OK;
@@ -816,9 +828,9 @@ sp_status sp_ffn_cache_input_inverse(const sp_ffn_module* m, sp_ffn_state* st, d
   // instead of 5.4 ms, once per module, but two calls on two streams queue there and an open capture may hold it.)
   CU(load_spd<double>(st->G_X, d, d, b.rho, Gs, d, s));
   CU(set_identity(X, d, d, s));
-  CU(potrf_lower_f64(Gs, d, d, reinterpret_cast<double*>(b.dinv), status_dev, s, nullptr, d, true));
+  CU(potrf_lower_f64(Gs, d, d, reinterpret_cast<double*>(b.dinv), status_dev, s, nullptr, 0, true));
   CU(gemm_simt(d, d, d, 1.0, Operand{X, SP_F64, d, 1}, Operand{X, SP_F64, 1, d}, 0.0, Operand{st->G_X_inv, SP_F32, d, 1},
-               OutOperand{st->G_X_inv, SP_F32, d}, true, true, s, true));
+               OutOperand{st->G_X_inv, SP_F32, d}, true, true, s, kTriBoth));
   CU(symmetrize_lower(st->G_X_inv, d, d, s));
   return SP_OK;
 }
@@ -1080,8 +1092,14 @@ static sp_status admm_step_impl(const sp_ffn_module* m, sp_ffn_state* st, const 
       CU(load_spd<double>(p.Cf, d, d, gam, Gs, d, s));
       CU(transpose_convert<double>(p.W2cf, kp, d, k, Rs, d, s));
       const SolveAssist* assist = side ? &side->assist_main : nullptr;
-      CU(potrf_lower_f64(Gs, d, d, reinterpret_cast<double*>(p.sb.dinv), status_dev, s, assist, k));
-      CU(potrs_backward_f64(Rs, k, d, d, Gs, d, reinterpret_cast<double*>(p.sb.dinv), s, assist));
+      if (d <= kInverseMaxN) {
+        double* X = Rs + (size_t)(k + d) * d;
+        CU(solve_inverse_f64(Gs, d, k, reinterpret_cast<double*>(p.sb.dinv), X, status_dev, s, assist));
+        Rs = X;
+      } else {
+        CU(potrf_lower_f64(Gs, d, d, reinterpret_cast<double*>(p.sb.dinv), status_dev, s, assist, k));
+        CU(potrs_backward_f64(Rs, k, d, d, Gs, d, reinterpret_cast<double*>(p.sb.dinv), s, assist));
+      }
       CU(convert_matrix(Rs, SP_F64, d, p.Qt, SP_F32, d, k, d, s));
     }
   }

@@ -259,10 +259,11 @@ struct OutOperand {
 
 // C[M,N] (row-major) = alpha * sum_k A(i,k) B(k,j) + beta * Cin[i,j].  Cin may alias C or be another matrix of
 // another dtype; beta == 0 never reads Cin.  lower_only skips tiles that lie strictly above the diagonal.
-// acc64: accumulate in fp64 (else fp32).  k_tri: A(i, k) = 0 for k < i and B(k, j) = 0 for k < j, so that a tile may
+// acc64: accumulate in fp64 (else fp32).  k_tri: B(k, j) = 0 for k < j and (kTriBoth) A(i, k) = 0 for k < i, so that a tile may
 // start its sum there (honoured where it pays; the stored zeros are read otherwise).
+constexpr int kTriBoth = 1, kTriColumns = 2;
 cudaError_t gemm_simt(int64_t M, int64_t N, int64_t K, double alpha, Operand A, Operand B, double beta,
-                      Operand Cin, OutOperand C, bool lower_only, bool acc64, cudaStream_t stream, bool k_tri = false);
+                      Operand Cin, OutOperand C, bool lower_only, bool acc64, cudaStream_t stream, int k_tri = 0);
 
 // tcgen05 path: bf16 operands, fp32 accumulation in tensor memory.
 //   a_kmajor: A is stored [M, K] row-major (K contiguous) ; else [K, M] row-major (M contiguous).
@@ -312,10 +313,16 @@ struct SolveAssist;
 //   potrf_lower_f64: in-place lower Cholesky of the n x n matrix A (ld lda); the strict upper triangle and the diagonal
 //   blocks of the factor are not written; dinv: ceil(n / kCholNB) inverse diagonal blocks [kCholNB, kCholNB].
 //   m_extra > 0: A has m_extra more rows below row n, right-hand sides B of X L^T = B that ride along and hold X on
-//   return.  extra_is_identity: B is the identity (m_extra == n), so that X is upper triangular and a step touches
-//   only the rows that are no longer zero.
+//   return.  identity: n more rows below those hold an identity, whose X = L^-T is upper triangular; a step touches only its
+//   rows that are no longer zero.
 cudaError_t potrf_lower_f64(double* A, int64_t n, int64_t lda, double* dinv, int32_t* status_dev, cudaStream_t stream,
-                            const SolveAssist* assist, int64_t m_extra, bool extra_is_identity = false);
+                            const SolveAssist* assist, int64_t m_extra, bool identity = false);
+// W[m, n] = B L^-T L^-1 with the factor of the n x n matrix A, the right-hand sides B below it and, below those, room for n more
+// rows (all dense, leading dimension n).
+cudaError_t solve_inverse_f64(double* A, int64_t n, int64_t m, double* dinv, double* W, int32_t* status_dev, cudaStream_t stream,
+                              const SolveAssist* assist);
+// Systems of up to this many unknowns (the identity costs n^3 / 3 operations, which pay while the chain leaves the fp64 pipe idle).
+constexpr int64_t kInverseMaxN = 4096;
 // X[m,n] <- X L^-1 (backward sweep with the factor of potrf_lower_f64).
 cudaError_t potrs_backward_f64(double* X, int64_t m, int64_t n, int64_t ldx, const double* L, int64_t ldl,
                                const double* dinv, cudaStream_t stream, const SolveAssist* assist);

@@ -215,9 +215,9 @@ gemm_dmma_kernel(int64_t M, int64_t N, int64_t K, double alpha, const T* A, int6
 #pragma unroll
       for (int q = 0; q < 4; ++q) acc[i][j][q] = 0.0;
 
-  // k_tri: both operands are zero for K indices below their own M / N index (upper-triangular rows)
+  // k_tri: both operands (kTriBoth) or B (kTriColumns) are zero for K indices below their own M / N index (upper-triangular rows)
   int64_t k0 = 0;
-  if (k_tri) k0 = (row0 > col0 ? row0 : col0) / DM_BK * DM_BK;
+  if (k_tri) k0 = (k_tri == kTriBoth && row0 > col0 ? row0 : col0) / DM_BK * DM_BK;
   SlabA fa;
   SlabB fb;
   fa.fetch(A, lda, va, row0, k0, M, K);
@@ -440,13 +440,13 @@ cudaError_t launch_dmma_short(int64_t M, int64_t N, int64_t K, double alpha, con
 
 template <typename T, int BM>
 void launch_dmma(int64_t M, int64_t N, int64_t K, double alpha, const Operand& A, const Operand& B, double beta,
-                 const Operand& Cin, const OutOperand& C, bool lower_only, bool k_tri, cudaStream_t stream) {
+                 const Operand& Cin, const OutOperand& C, bool lower_only, int tri, cudaStream_t stream) {
   const dim3 grid((unsigned)ceil_div(N, DM_BN), (unsigned)ceil_div(M, BM));
   const bool ak = A.s1 == 1, bk = B.s0 == 1;
   const int64_t lda = ak ? A.s0 : A.s1, ldb = bk ? B.s1 : B.s0;
   const T* a = reinterpret_cast<const T*>(A.ptr);
   const T* b = reinterpret_cast<const T*>(B.ptr);
-  const int lo = lower_only ? 1 : 0, tri = k_tri ? 1 : 0;
+  const int lo = lower_only ? 1 : 0;
   if (ak && bk) launch(gemm_dmma_kernel<T, true, true, BM>, grid, DM_THREADS, 0, stream, M, N, K, alpha, a, lda, b, ldb, beta, Cin, C, lo, tri);
   else if (ak) launch(gemm_dmma_kernel<T, true, false, BM>, grid, DM_THREADS, 0, stream, M, N, K, alpha, a, lda, b, ldb, beta, Cin, C, lo, tri);
   else if (bk) launch(gemm_dmma_kernel<T, false, true, BM>, grid, DM_THREADS, 0, stream, M, N, K, alpha, a, lda, b, ldb, beta, Cin, C, lo, tri);
@@ -456,7 +456,7 @@ void launch_dmma(int64_t M, int64_t N, int64_t K, double alpha, const Operand& A
 }  // namespace
 
 cudaError_t gemm_simt(int64_t M, int64_t N, int64_t K, double alpha, Operand A, Operand B, double beta, Operand Cin,
-                      OutOperand C, bool lower_only, bool acc64, cudaStream_t stream, bool k_tri) {
+                      OutOperand C, bool lower_only, bool acc64, cudaStream_t stream, int k_tri) {
   if (M <= 0 || N <= 0) return cudaSuccess;
   count_launch();
   ProfScope prof(PK_GEMM_SIMT, (lower_only ? 1.0 : 2.0) * (double)M * (double)N * (double)K, 0.0, stream);
