@@ -1309,10 +1309,11 @@ struct BMat {
 
 // C_b = alpha * sum over segments A_b[plane pa] B_b[plane pb] + beta * Cin_b for all nb0 x nb1 pairs.
 // bf16 operands: one batched tensor-core launch.  fp32 operands (fp32 mode): plane 0 holds the full value, the
-// segments collapse to one product per pair with fp64 accumulation.
+// segments collapse to one product per pair with fp64 accumulation.  lower: tiles above the diagonal are left out; k_tri: see TcBatch
+// (the zeros are read in fp32 mode).
 sp_status bcontract(int64_t M, int64_t N, int64_t K, double alpha, BMat A, bool a_kmajor, BMat B, bool b_kmajor,
                     int nseg, const int* pa, const int* pb, double beta, BMat Cin, BMat C, int64_t c_lo_off, int nb0,
-                    int nb1, int32_t* status, cudaStream_t s) {
+                    int nb1, int32_t* status, cudaStream_t s, bool lower = false, int32_t k_tri = 0) {
   if (M <= 0 || N <= 0 || nb0 <= 0 || nb1 <= 0) return SP_OK;
   if (A.dt == SP_BF16 && B.dt == SP_BF16) {
     TcOperand ta{A.ptr, A.ld, a_kmajor}, tb{B.ptr, B.ld, b_kmajor};
@@ -1326,7 +1327,8 @@ sp_status bcontract(int64_t M, int64_t N, int64_t K, double alpha, BMat A, bool 
     bt.a_planes = A.planes; bt.a_plane = A.plane; bt.b_planes = B.planes; bt.b_plane = B.plane;
     OutOperand out{const_cast<void*>(C.ptr), C.dt, C.ld};
     out.lo_off = c_lo_off;
-    return gemm_tc(M, N, K, (float)alpha, ta, tb, (float)beta, Operand{Cin.ptr, Cin.dt, Cin.ld, 1}, out, false, status,
+    bt.k_tri = k_tri;
+    return gemm_tc(M, N, K, (float)alpha, ta, tb, (float)beta, Operand{Cin.ptr, Cin.dt, Cin.ld, 1}, out, lower, status,
                    s, &sg, 2.0 * (double)M * N * K * nb0 * nb1, 0, &bt);
   }
   for (int b1 = 0; b1 < nb1; ++b1)
@@ -1338,7 +1340,7 @@ sp_status bcontract(int64_t M, int64_t N, int64_t K, double alpha, BMat A, bool 
       Operand b{at(B), B.dt, b_kmajor ? 1 : B.ld, b_kmajor ? B.ld : 1};
       Operand cin{Cin.ptr ? at(Cin) : nullptr, Cin.dt, Cin.ld, 1};
       OutOperand out{const_cast<uint8_t*>(at(C)), C.dt, C.ld};
-      CU(gemm_simt(M, N, K, alpha, a, b, beta, cin, out, false, true, s));
+      CU(gemm_simt(M, N, K, alpha, a, b, beta, cin, out, lower, true, s));
     }
   return SP_OK;
 }
@@ -1568,7 +1570,7 @@ static sp_status mha_impl(const sp_mha_module* m, sp_mha_state* st, const sp_mha
 
     // logits S = Zq_i Zk_i^T / sqrt(d_h) and Phi = softmax(S)
     SPCHK(bcontract(T, T, dh, inv_sqrt, Zqv, true, Zkv, true, bf16 ? 3 : 1, kSeg3A, kSeg3B, 0.0, none, ttv(p.S, SP_F32), 0,
-                    nb0, nb1, status_dev, s));
+                    nb0, nb1, status_dev, s, causal));
     if (init) {
       // forward definition: P = softmax(S), heads = P V, Ypre = heads W_O^T
       CU(mha_softmax_rows(p.S, pairs, (int)T, causal, p.Pb, pplane, s));
@@ -1640,16 +1642,17 @@ static sp_status mha_impl(const sp_mha_module* m, sp_mha_state* st, const sp_mha
     // ---- Eq. (87): joint gradient steps on (Zq, Zk) through the softmax
     for (int it = 0; it < prm->z_steps; ++it) {
       SPCHK(bcontract(T, T, dh, inv_sqrt, Zqv, true, Zkv, true, bf16 ? 3 : 1, kSeg3A, kSeg3B, 0.0, none,
-                      ttv(p.G, SP_F32), 0, nb0, nb1, status_dev, s));
-      CU(mha_softmax_backward_rows(p.G, P, pairs, (int)T, causal, prm->beta, p.Pb, s));
+                      ttv(p.G, SP_F32), 0, nb0, nb1, status_dev, s, causal));
+      const bool tri = causal && bf16;
+      CU(mha_softmax_backward_rows(p.G, P, pairs, (int)T, causal, tri ? (int)kTcTileRows : (int)T, prm->beta, p.Pb, s));
       const BMat dS = bf16 ? ttv(p.Pb, SP_BF16) : ttv(p.G, SP_F32);
       // gq = dS Zk_i / sqrt(d_h), gk = dS^T Zq_i / sqrt(d_h) (hi parts of the operands)
       BMat Zk1 = Zkv, Zq1 = Zqv;
       Zk1.planes = Zq1.planes = 1;
       SPCHK(bcontract(T, dh, T, inv_sqrt, dS, true, Zk1, false, 1, kSegHH, kSegHH, 0.0, none, tokv(p.Gq, SP_F32, d, 1, 0),
-                      0, nb0, nb1, status_dev, s));
+                      0, nb0, nb1, status_dev, s, false, tri ? kTriALower : 0));
       SPCHK(bcontract(T, dh, T, inv_sqrt, dS, false, Zq1, false, 1, kSegHH, kSegHH, 0.0, none, tokv(p.Gk, SP_F32, d, 1, 0),
-                      0, nb0, nb1, status_dev, s));
+                      0, nb0, nb1, status_dev, s, false, tri ? kTriAUpper : 0));
       CU(mha_step_sizes(Zq, Zk, d, nq, (int)T, (int)dh, (int)H, 1, prm->alpha, prm->beta, prm->eta_z, p.sums, p.eta_z, s));
       CU(mha_z_update(Zq, Zk, p.Gq, p.Gk, p.Tq, p.Tk, p.eta_z, Tc, (int)d, (int)T, (int)dh, prm->alpha,
                       bf16 ? p.Zqs : nullptr, bf16 ? p.Zks : nullptr, plane, s));

@@ -292,14 +292,18 @@ struct TcSegments {
 // per-sequence products of an attention module (head = a column slice of a token-major tensor, sequence = a row range)
 // are issued together.  A and B may also consist of several planes (e.g. the hi and lo parts of a split operand, each
 // a whole tensor, x_plane elements apart); a K segment then names the plane it reads.  Every stride times the element
-// size must be a multiple of 16 bytes.  Not available together with lower_only or a cut along K.
+// size must be a multiple of 16 bytes.  Not available together with a cut along K.
 struct TcBatch {
   int32_t nb0 = 1, nb1 = 1;
   int64_t a_s0 = 0, a_s1 = 0, b_s0 = 0, b_s1 = 0, c_s0 = 0, c_s1 = 0, cin_s0 = 0, cin_s1 = 0;
   int32_t a_planes = 1, b_planes = 1;
   int64_t a_plane = 0, b_plane = 0;
   bool b_shared0 = false;       // B is the same for all nb0 products (b_s0 unused)
+  // one segment: A(i, k) is zero for k in later (kTriALower) or earlier (kTriAUpper) blocks of kTcTileRows than i's, and not read there
+  int32_t k_tri = 0;
 };
+constexpr int32_t kTriALower = 1, kTriAUpper = 2;
+constexpr int64_t kTcTileRows = 256;
 // K is the extent of ONE segment.  alg_flops >= 0 overrides the flop count recorded for profiling.  max_pairs > 0
 // limits the launch to that many CTA pairs (SM pairs), leaving the other SMs to kernels of another stream.
 sp_status gemm_tc(int64_t M, int64_t N, int64_t K, float alpha, TcOperand A, TcOperand B, float beta, Operand Cin,
@@ -531,8 +535,9 @@ cudaError_t mha_softmax_rows(float* S, int64_t pairs, int T, bool causal, void* 
 // P <- P - eta_pair (-2 alpha G1 + 2 beta (P - Phi)); Pb: optional bf16 copy of the new P (hi / lo planes as above)
 cudaError_t mha_p_update(float* P, const float* Phi, const float* G1, const float* eta, int64_t pairs, int T,
                          double alpha, double beta, void* Pb, int64_t plane, cudaStream_t stream);
-// dS = 2 beta Phi (E - rowsum(E Phi)), Phi = softmax(S), E = Phi - P, as bf16 to dSb or (dSb == nullptr) in place of S
-cudaError_t mha_softmax_backward_rows(float* S, const float* P, int64_t pairs, int T, bool causal, double beta,
+// dS = 2 beta Phi (E - rowsum(E Phi)), Phi = softmax(S), E = Phi - P, as bf16 to dSb or (dSb == nullptr) in place of S;
+// causal: zero for keys u > query t, written up to the end of the query's block of `tail` keys
+cudaError_t mha_softmax_backward_rows(float* S, const float* P, int64_t pairs, int T, bool causal, int tail, double beta,
                                       void* dSb, cudaStream_t stream);
 // per-pair step sizes from the squared norms of the [T, d_h] slices of x (and y): mode 0: 1 / (2 (alpha s + beta)),
 // mode 1: eta_z / (2 alpha + beta s / d_h); sums: n_seq * H doubles of scratch

@@ -38,6 +38,7 @@ namespace {
 constexpr int BM = 128;            // rows of A (and of the accumulator) per CTA
 constexpr int BNH = 128;           // columns of B loaded per CTA (half of the pair's tile)
 constexpr int TILE_M = 2 * BM;     // tile of the CTA pair
+static_assert(TILE_M == kTcTileRows, "blocks of TcBatch::k_tri");
 constexpr int TILE_N = 2 * BNH;
 constexpr int kNarrowN = 128;      // columns of the narrow tile
 constexpr int kMinCutKb = 32;      // a range of K that a tile may be cut into has at least this many k-blocks
@@ -86,6 +87,7 @@ struct TcParams {
   int8_t a_ord[4], b_ord[4], c_ord[4];
   int64_t c_s0, c_s1, cin_s0, cin_s1;
   int32_t b_shared0;       // one B for all b0
+  int32_t k_tri;           // see TcBatch
   long long wait_budget;   // clock cycles a role may wait on one barrier before it gives up (SP_ERR_TIMEOUT)
   int32_t* status;
   const int32_t* skip;     // conditional launch: every CTA returns at once when *skip != 0 (see SkipScope)
@@ -188,6 +190,11 @@ __device__ __forceinline__ void tile_coords(const TcParams& p, int t, int& tm, i
   }
 }
 
+// k-blocks of a tile of rows whose other blocks of A are zero
+__device__ __forceinline__ void tri_range(const TcParams& p, int tm, int& kb0, int& kb1) {
+  if (p.k_tri == kTriALower) kb1 = min(kb1, (tm + 1) * (TILE_M / BK));
+  if (p.k_tri == kTriAUpper) kb0 = max(kb0, tm * (TILE_M / BK));
+}
 __device__ __forceinline__ void tc_commit_local(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
@@ -268,6 +275,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         int tm, tn, tile, kb0, kb1, b0, b1;
         unit_map(p, u, num_kb, tile, kb0, kb1);
         tile_coords<BATCHED>(p, tile, tm, tn, b0, b1);
+        if constexpr (BATCHED) tri_range(p, tm, kb0, kb1);
         for (int kb = kb0; kb < kb1; ++kb) {
           if (!mbar_wait(empty_bar(s), ph ^ 1u, abort_flag, p.wait_budget)) { ok = false; break; }
           // the leader's barrier collects the bytes of both CTAs' loads of this stage
@@ -336,6 +344,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const uint32_t d_tmem = tmem_base + (uint32_t)(acc * TILE_N);
         int tile, kb0, kb1;
         unit_map(p, u, num_kb, tile, kb0, kb1);
+        if constexpr (BATCHED) {
+          if (p.k_tri != 0) {
+            int tm, tn, b0, b1;
+            tile_coords<true>(p, tile, tm, tn, b0, b1);
+            tri_range(p, tm, kb0, kb1);
+          }
+        }
         for (int kb = kb0; kb < kb1; ++kb) {
           if (!mbar_wait(full_bar(s), ph, abort_flag, p.wait_budget)) { ok = false; break; }
           tc_fence_after();
@@ -761,6 +776,9 @@ sp_status gemm_tc(int64_t M, int64_t N, int64_t K, float alpha, TcOperand A, TcO
     const TcBatch& bt = *batch;
     const int b_nb0 = bt.b_shared0 ? 1 : bt.nb0;
     p.b_shared0 = bt.b_shared0 ? 1 : 0;
+    // (square: every tile of rows has blocks left)
+    if (bt.k_tri != 0 && (sg.nseg != 1 || M != K)) return SP_ERR_INVALID_ARG;
+    p.k_tri = bt.k_tri;
     for (int i = 0; i < sg.nseg; ++i)
       if (sg.a_p[i] < 0 || sg.a_p[i] >= bt.a_planes || sg.b_p[i] < 0 || sg.b_p[i] >= bt.b_planes)
         return SP_ERR_INVALID_ARG;

@@ -147,9 +147,10 @@ __global__ void __launch_bounds__(256) p_update_kernel(float* P, const float* Ph
 
 // Softmax and its backward for the softmax term of Eq. (87), one warp per row of logits S:
 //   Phi = softmax(S),  E = Phi - P,  dS = 2 beta Phi (E - sum_u E Phi)  -> as bf16 to dSb, or (dSb == nullptr) in place.
+// Beyond the causal limit zeros are written up to the end of the row's block of `tail` keys.
 template <int NV>
 __global__ void __launch_bounds__(kRowWarps * 32) softmax_backward_rows_kernel(float* S, const float* P,
-                                                                               int64_t rows, int T, int causal,
+                                                                               int64_t rows, int T, int causal, int tail,
                                                                                float beta,
                                                                                __nv_bfloat16* dSb) {
   kernel_begin();
@@ -173,8 +174,9 @@ __global__ void __launch_bounds__(kRowWarps * 32) softmax_backward_rows_kernel(f
     if (dSb) dSb[r * T + u] = __float2bfloat16_rn(g);
     else row[u] = g;
   };
+  const int end = causal && tail < T ? min(T, ((lim - 1) / tail + 1) * tail) : T;
   if constexpr (NV > 0) {
-    for_row<NV>(lane, T, [&](int u, int i) {
+    for_row<NV>(lane, end, [&](int u, int i) {
       const float ph = u < lim ? v.at(row, lane, i) * inv : 0.f;
       put(u, u < lim ? 2.f * beta * ph * (ph - p[i] - dot) : 0.f);
     });
@@ -192,7 +194,7 @@ __global__ void __launch_bounds__(kRowWarps * 32) softmax_backward_rows_kernel(f
       for (int q = 0; q < 4; ++q) put(u + 32 * q, g[q]);
     }
     for (; u < lim; u += 32) put(u, value(u));
-    for (; u < T; u += 32) put(u, 0.f);
+    for (; u < end; u += 32) put(u, 0.f);
   }
 }
 
@@ -450,7 +452,7 @@ cudaError_t mha_p_update(float* P, const float* Phi, const float* G1, const floa
   return cudaGetLastError();
 }
 
-cudaError_t mha_softmax_backward_rows(float* S, const float* P, int64_t pairs, int T, bool causal, double beta,
+cudaError_t mha_softmax_backward_rows(float* S, const float* P, int64_t pairs, int T, bool causal, int tail, double beta,
                                       void* dSb, cudaStream_t stream) {
   const int64_t rows = pairs * T;
   if (rows == 0) return cudaSuccess;
@@ -458,7 +460,7 @@ cudaError_t mha_softmax_backward_rows(float* S, const float* P, int64_t pairs, i
   count_launch();
   const unsigned grid = (unsigned)ceil_div(rows, (int64_t)kRowWarps);
   const auto run = [&](auto kernel) {
-    launch(kernel, grid, kRowWarps * 32, 0, stream, S, P, rows, T, causal ? 1 : 0, (float)beta,
+    launch(kernel, grid, kRowWarps * 32, 0, stream, S, P, rows, T, causal ? 1 : 0, tail, (float)beta,
                                                 reinterpret_cast<__nv_bfloat16*>(dSb));
   };
   if (T <= 128) run(softmax_backward_rows_kernel<4>);
