@@ -824,8 +824,8 @@ sp_status sp_ffn_cache_input_inverse(const sp_ffn_module* m, sp_ffn_state* st, d
   ProfScope prof(PK_SOLVE, (double)d * d * d, 0.0, s);
   double* Gs = reinterpret_cast<double*>(b.Gs);
   double* X = Gs + (size_t)d * d;
-  // On the caller's stream alone, like the precise solves.  (With far updates on an assisting stream d = 4096 takes 4.6
-  // instead of 5.4 ms, once per module, but two calls on two streams queue there and an open capture may hold it.)
+  // On the caller's stream alone, like the precise solves: on an assisting stream two calls on two streams would queue, and an open
+  // capture might hold it.
   CU(load_spd<double>(st->G_X, d, d, b.rho, Gs, d, s));
   CU(set_identity(X, d, d, s));
   CU(potrf_lower_f64(Gs, d, d, reinterpret_cast<double*>(b.dinv), status_dev, s, nullptr, 0, true));

@@ -2,7 +2,7 @@
 // mode and for the cached inverse of the input system.  The O(n^3) and O(m n^2) work is GEMMs on the diagonal-block
 // inverses; only the 64 x 64 diagonal factorisation runs in a single thread block.  What bounds it: up to n of a few
 // thousand the chain diagonal block -> panel -> next block column (about 33 us per 64 columns), above that the fp64 pipe.
-// The inverse of a 4096-wide input system takes 5.4 ms (36 ms with scalar fp64 products and a solve for 4096 columns).
+// The inverse of a 4096-wide input system takes 4.7 ms (36 ms with scalar fp64 products and a solve for 4096 columns).
 #include "sp_chol_block.cuh"
 #include "sp_common.cuh"
 
@@ -10,6 +10,9 @@ namespace sp {
 namespace {
 
 constexpr int NB = kCholNB;
+// Two-level updates on one stream: inverse of an input system, us: 768 wide 319 -> 332, 1024 549 -> 501, 2048 1481 -> 1339, 4096 5357 ->
+// 4682.
+constexpr int64_t kOuterMinF64 = 1024;
 using Diag = DiagBlock<double, NB>;
 
 __global__ void __launch_bounds__(Diag::THREADS) chol_diag64_kernel(const double* A, int64_t lda, int nb, double* dinv,
@@ -36,6 +39,8 @@ cudaError_t potrf_lower_f64(double* A, int64_t n, int64_t lda, double* dinv, int
     return cudaFuncSetAttribute(chol_diag64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Diag::SMEM);
   }));
   const bool apart = assist && assist->far_stream && (m_extra > 0 || identity);
+  constexpr int64_t OUTER = 4 * NB;
+  const bool two_level = !assist && n >= kOuterMinF64;
   int last = -1;      // event of the far update still in flight
   for (int64_t k0 = 0, step = 0; k0 < n; k0 += NB, ++step) {
     const int nb = (int)((n - k0 < NB) ? (n - k0) : NB);
@@ -52,6 +57,20 @@ cudaError_t potrf_lower_f64(double* A, int64_t n, int64_t lda, double* dinv, int
     // rows and finishes reading them before it writes.
     if (rows > 0)
       SP_CU(gemm_simt(rows, nb, nb, 1.0, op(A21, lda, 1), op(dk, 1, NB), 0.0, op(A21, lda, 1), out(A21, lda), false, true, stream));
+    // one stream, wide matrix: the rest of an outer block's columns now, everything to its right once per outer block, with K four times as
+    // long (a quarter of the passes over the matrix)
+    if (two_level) {
+      const int64_t o0 = k0 / OUTER * OUTER, end = o0 + OUTER < n ? o0 + OUTER : n;
+      if (rem <= 0) break;
+      double* A22 = A21 + nb;
+      if (end > k0 + nb)
+        SP_CU(gemm_simt(rows, end - k0 - nb, nb, -1.0, op(A21, lda, 1), op(A21, 1, lda), 1.0, op(A22, lda, 1), out(A22, lda), true,
+                        true, stream));
+      else
+        SP_CU(gemm_simt(rows, rem, end - o0, -1.0, op(A + end * lda + o0, lda, 1), op(A + end * lda + o0, 1, lda), 1.0,
+                        op(A22, lda, 1), out(A22, lda), true, true, stream));
+      continue;
+    }
     const int64_t wn = (assist && rem > NB) ? NB : rem;      // columns of the near update
     if (wn < rem || apart) SP_CU(cudaEventRecord(assist->panel_done, stream));
     if (apart) {
