@@ -514,8 +514,8 @@ sp_status sp_gemm(int32_t transA, int32_t transB, int64_t M, int64_t N, int64_t 
                   int32_t* status_dev, void* stream);
 sp_status sp_symmetrize(float* G, int64_t n, int64_t ldg, void* stream);
 
-/* sp_set_wait_budget(cycles): every barrier wait inside the tensor-core GEMM kernel is bounded by a clock budget
- * (about two seconds by default); a wait that outlasts it makes the kernel record SP_ERR_TIMEOUT in status_dev, drain
+/* sp_set_wait_budget(cycles): every barrier wait inside the tensor-core GEMM kernel and every wait of a one-launch solve is bounded by
+ * a clock budget (about two and 16 seconds by default); a wait that outlasts it makes the kernel record SP_ERR_TIMEOUT in status_dev, drain
  * its copies and tensor-core work in flight, free its tensor memory and return, leaving C incomplete.  This call
  * changes the budget process-wide (0 restores the default).  It exists for diagnosis and for testing the time-out
  * path: with a budget of a few cycles an ordinary wait for a long K loop already runs out. */

@@ -52,7 +52,8 @@ constexpr uint32_t NBARS = 11;
 constexpr size_t SMEM = AREA + 1024 /*alignment*/ + (NBARS + Diag::BARS) * 8 + 4 * TB * sizeof(float) /*row maxima*/;
 static_assert(Diag::SMEM - Diag::BARS * 8 <= DATA, "the diagonal block's arrays lie over the operand slots");
 constexpr uint32_t TMEM_COLS = 4 * TB;                    // two pairs of accumulators in turn
-constexpr long long WAIT_BUDGET = 4000000000LL;           // about two seconds
+// about 16 seconds: a block may wait for others of its launch that have no room yet beside another stream's long kernels
+constexpr long long WAIT_BUDGET = 32000000000LL;
 constexpr long long DRAIN = 200000000LL;
 constexpr int kFlags0 = 32;                               // flags[0]: the task counter
 

@@ -212,15 +212,6 @@ def prune_attention_heads(H: torch.Tensor, Ypre: torch.Tensor, W_O: torch.Tensor
     return mask, W_new, scores
 
 
-def _recover_together(d: int, precise: bool, device) -> bool:
-    """W_Q and W_K have one system matrix: one factorisation with the rows of both below it takes two thirds of the time of
-    two (2048 wide 1.17 against 1.78 ms, 2560 wide 1.65 against 2.48, 5120 wide 6.8 against 8.8).  But a backward sweep takes its
-    updates in a fixed order only up to one wave of its panels, 32 right-hand sides per SM (148 SMs: 4736); between half a wave
-    and a whole one each recovery by itself keeps that order and both together would not, so there they are solved apart."""
-    wave = 32 * torch.cuda.get_device_properties(device).multi_processor_count
-    return precise or 2 * d <= wave or d > wave
-
-
 def mha_outer_iterations(mod: api.MhaModule, head_mask: torch.Tensor, iters: int, params: api.MhaParams | None = None,
                          rho: float = 0.1, rho_relative: bool = True, recover_wv: bool = True):
     """Outer loop of Algorithm 2's SparseLLM2 for one attention module with a fixed head mask (u8 [n_heads], from the
@@ -239,14 +230,10 @@ def mha_outer_iterations(mod: api.MhaModule, head_mask: torch.Tensor, iters: int
     unit_scores = head_mask.to(torch.float32)
     api.sp_apply_mask(unit_scores, k_heads, group=d_head, W_rows=mod.Wv)
     precise = mod.X.dtype == torch.float32          # fp32 mode: fp64 factorisations
-    together = _recover_together(mod.d, precise, mod.X.device)
     for _ in range(iters):
-        if together:
-            Wqk = api.sp_ridge_solve(torch.cat((mod.R_Q, mod.R_K)), mod.G_X, rho, rho_relative, precise)
-            Wq, Wk = Wqk[:mod.d], Wqk[mod.d:]
-        else:
-            Wq = api.sp_ridge_solve(mod.R_Q, mod.G_X, rho, rho_relative, precise)
-            Wk = api.sp_ridge_solve(mod.R_K, mod.G_X, rho, rho_relative, precise)
+        # one system matrix: one factorisation with the rows of both below it (2048 wide 0.58 against 1.03 ms)
+        Wqk = api.sp_ridge_solve(torch.cat((mod.R_Q, mod.R_K)), mod.G_X, rho, rho_relative, precise)
+        Wq, Wk = Wqk[:mod.d], Wqk[mod.d:]
         api.sp_apply_mask(unit_scores, k_heads, group=d_head, W_rows=Wq)
         api.sp_apply_mask(unit_scores, k_heads, group=d_head, W_rows=Wk)
         Wo = api.sp_linear_refit(mod.R_O, mod.G_attn, head_mask, k_heads, rho, group=d_head, precise=precise,
