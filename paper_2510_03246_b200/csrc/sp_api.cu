@@ -1868,9 +1868,9 @@ sp_status sp_mha_value_refit(const sp_mha_module* m, const sp_mha_state* st, con
     CU(add_ridge_batched(p.G, g_bs, d, (int)nk, rho, rho_relative != 0, s));
     {
       ProfScope prof(PK_SOLVE, (double)nk * ((double)d * d * d / 3.0 + 2.0 * (double)dh * d * d), 0.0, s);
-      // (an attention step 2048 wide, 16 kept heads: 14.7 ms with a launch per step over all systems, 14.05 in one launch; 768 wide, 6
-      // heads: 2.43 and 2.28)
-      if (p.one) {
+      // one launch while a system has six thread blocks (an attention step 2048 wide, 16 kept heads: 14.7 -> 14.05 ms; the whole call with
+      // 8192 tokens twice, 18 / 24 / 28 / 32 kept heads: 10.44 -> 10.24, 13.30 -> 13.27, equal, 17.4 -> 17.4..18.0)
+      if (p.one && (d % kCholTcNB != 0 || nk * 6 <= sm_count())) {
         const SolveOneBufs one{p.P_all, nullptr, p.dinv_all, p.flags_all};
         SPCHK(solve_tc(p.G, d, dh, d, p.G + (size_t)d * d, d, one, nullptr, 0, 0, status_dev, s, (int)nk, g_bs));
       } else {
