@@ -878,7 +878,8 @@ static sp_status admm_step_impl(const sp_ffn_module* m, sp_ffn_state* st, const 
   // solved with the channels that the mask kept so far in front.  The leading block of that factor is the factor of
   // the restricted system of those channels, and the leading columns of the forward-substituted right-hand sides are
   // its forward substitution.  When the new top-k selects the same channels (a device flag, no host round trip), the
-  // restricted recovery is one backward sweep; otherwise the restricted system is factorised as usual.  The kernels
+  // restricted recovery is one backward sweep (or there already: a one-launch solve forms it with the unrestricted one);
+  // otherwise the restricted system is factorised as usual.  The kernels
   // of both branches are always queued and return at once when their branch is not taken.
   const bool skip_scores = prm->skip_scores != 0;   // fixed mask: W2~ and the scores serve nothing
   const int64_t k_lead = chol_tc_pad(k);

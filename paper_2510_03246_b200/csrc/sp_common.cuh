@@ -109,7 +109,8 @@ struct OverlapScope {
   ~OverlapScope() { overlap_flag() = saved; }
   OverlapScope(const OverlapScope&) = delete;
 };
-// Weight phase of an ADMM step (and the cached input inverse): modules up to this width.  Its gain falls with the width, whatever the
+// Weight phase of an ADMM step (and the cached input inverse): modules up to this width.  (Measured with recoveries by launches per block
+// column; most of them are one launch now.)  Its gain falls with the width, whatever the
 // token count: 768 x 3072 on 32768 tokens 3.09 -> 2.88 ms, 1096 x 4376 on 65536 tokens 7.40 -> 7.06, 1280 x 5120 on 8192 tokens
 // 4.78 -> 4.62, 2048 x 8192 on 32768 tokens 14.30 -> 14.06, 3072 x 9216 and 4096 x 11008 less than their runs differ.  Wider
 // modules keep plain launches.

@@ -6,6 +6,9 @@
 // of two such operands is taken as the six part products of weight >= 2^-16 (hi.hi, hi.mid, mid.hi, hi.lo, lo.hi,
 // mid.mid), each a K segment of one tcgen05 GEMM with fp32 accumulation.  The dropped terms are below 2^-23.
 //
+// Systems that solve_in_one() names are solved in one launch instead (sp_solve_tc.cu); this form serves smaller and wider ones, the
+// widest modules, and many systems at a time.
+//
 // Blocked right-looking algorithm with 128-wide panels:
 //   diagonal block : one CTA factorises it and forms inv(L11) in the same sweep (sp_chol_block.cuh);
 //   panel          : L21 = A21 inv(L11)^T on the CUDA cores (K = 128), written as fp32 and as the three bf16 parts;

@@ -16,8 +16,8 @@
 //
 // What bounds it: up to about 6000 unknowns the chain, 28 us per 128 unknowns (elimination 16, X and the tile below it into operand
 // form 2, their product 2.2, its result into operand form 1, the diagonal block's update 2.2; as one task per diagonal block, handed on
-// through memory, 36); above, the loads of the products (192 KB per two tiles' product, 1.6 us, as much as the tensor core takes for
-// operands of 128 rows).  3072 unknowns and 768 right-hand sides: 1164 us as launches per block column, 1015 with a task per
+// through memory, 36); above, the loads of the products (192 KB per two tiles' product; 3.8 us at 8192 unknowns, where the tensor core
+// takes 1.6.  Four slots of half the depth, with rows of 64 bytes, are slower: 3.96 -> 4.44 ms).  3072 unknowns and 768 right-hand sides: 1164 us as launches per block column, 1015 with a task per
 // diagonal block, 716.
 //
 // Tasks are taken by a counter in an order in which every task comes after those it reads (the chain, first, runs beside them).  A block
