@@ -101,6 +101,9 @@ __device__ __forceinline__ bool epi_any(bool v) {
       : "memory");
   return r != 0;
 }
+// Block barrier: whether any wait of the block has run out, one answer for all threads.  (Read by each for itself behind a plain
+// barrier, the flag may be set by a warp that is ahead, and the block's warps would end up at different barriers.)
+__device__ __forceinline__ bool given_up(volatile int* abort_flag) { return __syncthreads_or(*abort_flag) != 0; }
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 512;" ::: "memory"); }
 __device__ __forceinline__ void arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
@@ -419,12 +422,8 @@ solve_tc_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
       stage_block(at, v, p.nn < TB ? p.nn : TB);
     }
     for (int j = 0; j < p.nblk; ++j) {
-      __syncthreads();
-      if (*abort_flag != 0) break;
-      {
-        const int nb = p.nn - j * TB < TB ? p.nn - j * TB : TB;
-eliminate_block(at.data - smem_u32(smem_raw), at.data + AREA + 8u * NBARS, j, nb, p.status);
-      }
+      if (given_up(abort_flag)) break;
+      eliminate_block(at.data - smem_u32(smem_raw), at.data + AREA + 8u * NBARS, j, p.nn - j * TB < TB ? p.nn - j * TB : TB, p.status);
       at = place(smem_raw, &s_tmem);
       const bool more = j + 1 < p.nblk;
       const uint32_t par = (uint32_t)j & 1u, bars_j = at.data + AREA;
@@ -468,8 +467,7 @@ eliminate_block(at.data - smem_u32(smem_raw), at.data + AREA + 8u * NBARS, j, nb
         }
       }
       fence_async_smem();
-      __syncthreads();
-      if (*abort_flag != 0) break;
+      if (given_up(abort_flag)) break;
       if (at.warp == 1 && more && at.lane == 0) {
         bool ok = mbar_wait(tempty0, par ^ 1u, abort_flag, p.budget);
         if (ok) {
@@ -737,8 +735,7 @@ eliminate_block(at.data - smem_u32(smem_raw), at.data + AREA + 8u * NBARS, j, nb
     xc += tk.kind == TASK_T ? 1u : 0u;
     fc += tk.kind == TASK_T ? 1u : 0u;
     fence_async_smem();
-    __syncthreads();
-    if (*abort_flag != 0) break;
+    if (given_up(abort_flag)) break;
   }
   if (*abort_flag != 0) {
     // a wait ran out: copies and products in flight get time to end before shared and tensor memory are released

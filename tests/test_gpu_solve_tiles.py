@@ -48,3 +48,25 @@ def test_solution_on_the_kept_support_comes_with_the_factor(n, k):
     assert torch.equal(W != 0, mod.W2 != 0)
     # two solves of one system: fp32 roundings magnified by its condition number, at most 1 + n / rho
     assert float((W - mod.W2).norm() / W.norm()) <= 10 * (1 + n / 0.1) * 2.0 ** -24
+
+
+@pytest.mark.parametrize("n,m,budget", [(1024, 300, 1), (2304, 128, 20000)])
+def test_waits_that_run_out_end_the_solve(n, m, budget):
+    """With a budget of a few cycles ordinary waits run out (nothing is withheld): the solve reports SP_ERR_TIMEOUT and returns, and the
+    next one is the same as the one before."""
+    G, R = _system(n, m, n)
+    status = torch.zeros(4, dtype=torch.int32, device=DEV)
+    W = api.sp_ridge_solve(R, G, 1e-3, rho_relative=False)
+    torch.cuda.synchronize()
+    assert api.lib().sp_set_wait_budget(budget) == 0
+    try:
+        for _ in range(4):
+            status.zero_()
+            api.sp_ridge_solve(R, G, 1e-3, rho_relative=False, status=status)
+            torch.cuda.synchronize()
+            assert status.tolist()[0] == 7 and status.tolist()[2] == 13
+    finally:
+        api.lib().sp_set_wait_budget(0)
+    status.zero_()
+    assert torch.equal(W, api.sp_ridge_solve(R, G, 1e-3, rho_relative=False, status=status))
+    assert status.tolist() == [0, 0, 0, 0]
