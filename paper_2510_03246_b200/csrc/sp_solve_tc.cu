@@ -555,6 +555,7 @@ solve_tc_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
           }
           __nanosleep(20);
         }
+        __syncwarp();        // lane 0 loads what other lanes have acquired: a vote orders no memory
         asm volatile("fence.proxy.async;" ::: "memory");
         return true;
       };

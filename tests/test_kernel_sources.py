@@ -30,3 +30,12 @@ def test_no_loads_on_the_read_only_path():
         code = re.sub(r"//[^\n]*", "", path.read_text())
         for what in (r"__restrict__", r"\b__ldg\s*\(", r"ld\.global\.nc"):
             assert not re.search(what, code), f"{path.name}: {re.search(what, code).group(0)}"
+
+
+def test_flags_acquired_by_other_lanes_are_ordered_before_the_loads():
+    """The loader of the one-launch solve looks at 32 tiles' flags, a lane each, and lane 0 then issues the loads: between the
+    acquires and the proxy fence in front of the loads stands a warp barrier (a vote orders no memory)."""
+    text = re.sub(r"//[^\n]*", "", (CSRC / "sp_solve_tc.cu").read_text())
+    wait = text[text.index("auto wait_tiles"):text.index("uint32_t kl = kc;")]
+    after = wait[wait.rindex("__ballot_sync"):]
+    assert re.search(r"__syncwarp\(\);\s*asm volatile\(\"fence\.proxy\.async", after)
