@@ -821,6 +821,10 @@ __global__ void __launch_bounds__(1024) mask_to_index_kernel(const uint8_t* mask
     if (keep) kept_idx[before + rank] = (int32_t)i;
     before += tot;
   }
+  // the rest: the last kept unit once more (unit 0 of an empty mask), so that a list taken for longer than the mask says holds units
+  __syncthreads();
+  const int32_t last = before > 0 ? kept_idx[before - 1] : 0;
+  for (int64_t i = before + threadIdx.x; i < n; i += blockDim.x) kept_idx[i] = last;
 }
 
 // perm = the kept channels in ascending order, then the pruned ones in ascending order; count[0] = kept channels
@@ -906,7 +910,7 @@ __global__ void __launch_bounds__(kStripThreads) place_rows_kernel(const uint8_t
     if (!mask[i]) dst[i * ldd + j] = 0.f;
     if (i < k) {
       const int64_t r = idx[i];
-      if (r >= 0 && r < rows) dst[r * ldd + j] = src[i * lds + j];     // (a mask with fewer kept rows leaves the list short)
+      if (mask[r]) dst[r * ldd + j] = src[i * lds + j];     // (the list of an empty mask names a pruned row)
     }
   });
 }
