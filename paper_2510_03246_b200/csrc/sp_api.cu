@@ -1045,7 +1045,7 @@ static sp_status admm_step_impl(const sp_ffn_module* m, sp_ffn_state* st, const 
   const bool split_h = bf16 && m->act == SP_ACT_SWIGLU;
   const int64_t kp64 = split_kpad(k), dp64 = split_kpad(d);
   if (split_h && dp64 != d) CU(cudaMemsetAsync(p.E, 0, (size_t)p.chunk * 2 * dp64 * 2, s));   // padding columns stay zero
-  CU(build_group_map(st->mask, n, p.grp_base, p.grp_mask, s));
+  CU(build_group_map(st->mask, n, k, p.grp_base, p.grp_mask, s));
   CU(gather_cols<float>(st->W2, n, idx, d, k, p.W2cf, kp, s));
   MatRef w1{nullptr, SP_F32, d}, w2{p.W2cf, SP_F32, kp}, qt{p.Qt, SP_F32, d};
   if (bf16) {

@@ -489,8 +489,8 @@ struct UpdateArgs {
   void* Ht_out = nullptr;
   const int32_t* zt_pruned_flag = nullptr;
 };
-// grp_base / grp_mask of a u8 mask over n channels (see sp_elementwise.cu)
-cudaError_t build_group_map(const uint8_t* mask, int64_t n, int32_t* grp_base, uint8_t* grp_mask, cudaStream_t stream);
+// grp_base / grp_mask of a u8 mask over n channels, the first k that it keeps (see sp_elementwise.cu)
+cudaError_t build_group_map(const uint8_t* mask, int64_t n, int64_t k, int32_t* grp_base, uint8_t* grp_mask, cudaStream_t stream);
 // H[T, ldh] (compact on the k kept channels idx[0..k), ldh a multiple of 8) = storage(phi(Z) - U);
 // phi(z) = gate * z when gate != nullptr, else ReLU.
 // lo_off > 0 (bf16 storage, a multiple of 8, 2 * lo_off <= ldh): H is split into bf16 hi and lo parts, the hi part in

@@ -252,7 +252,8 @@ __global__ void effective_ridge_kernel(const float* G, int64_t ldg, int64_t n, d
 // channels are cut into groups of 8 consecutive ones: grp_base[g] = number of kept channels before channel 8 g,
 // grp_mask[g] = bit q set when channel 8 g + q is kept.  The kept channels of a group then sit at compact positions
 // grp_base[g], grp_base[g] + 1, ... in channel order.
-__global__ void __launch_bounds__(1024) group_map_kernel(const uint8_t* mask, int64_t n,
+// A mask that keeps more than k channels (reported elsewhere): those beyond the k-th count as pruned, there is no column for them.
+__global__ void __launch_bounds__(1024) group_map_kernel(const uint8_t* mask, int64_t n, int64_t k,
                                                          int32_t* grp_base, uint8_t* grp_mask) {
   kernel_begin();
   __shared__ int warp_tot[32];
@@ -279,7 +280,9 @@ __global__ void __launch_bounds__(1024) group_map_kernel(const uint8_t* mask, in
     int before = s_before;
     for (int i = 0; i < w; ++i) before += warp_tot[i];
     if (g < groups) {
-      grp_base[g] = before + v - cnt;
+      const int first = before + v - cnt;
+      for (int over = first + cnt - (int)k; over > 0 && bits != 0; --over) bits &= ~(1u << (31 - __clz(bits)));
+      grp_base[g] = first < k ? first : (int)k;
       grp_mask[g] = (uint8_t)bits;
     }
     __syncthreads();
@@ -1273,11 +1276,11 @@ cudaError_t effective_ridge(const float* G, int64_t ldg, int64_t n, double rho, 
   return cudaGetLastError();
 }
 
-cudaError_t build_group_map(const uint8_t* mask, int64_t n, int32_t* grp_base, uint8_t* grp_mask, cudaStream_t stream) {
+cudaError_t build_group_map(const uint8_t* mask, int64_t n, int64_t k, int32_t* grp_base, uint8_t* grp_mask, cudaStream_t stream) {
   if (n == 0) return cudaSuccess;
   ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
   count_launch();
-  launch(group_map_kernel, 1, 1024, 0, stream, mask, n, grp_base, grp_mask);
+  launch(group_map_kernel, 1, 1024, 0, stream, mask, n, k, grp_base, grp_mask);
   return cudaGetLastError();
 }
 

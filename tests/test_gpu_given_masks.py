@@ -56,3 +56,27 @@ def test_step_on_fewer_units_than_announced(kept):
     # the inverse rounded to fp32, six part products without terms below 2^-23: a few roundings per term, at random over d terms
     bound = 8 * d ** 0.5 * 2.0 ** -24 * (R1.abs() @ torch.linalg.inv(G + 0.1 * G.diagonal().mean() * torch.eye(d, device=DEV, dtype=torch.float64)).abs())
     assert bool(((mod.W1.double() - ref).abs() <= bound)[keep].all())
+
+
+@pytest.mark.parametrize("kept", [302, 315, 520])
+@pytest.mark.parametrize("act", ["relu", "gated", "dual"])
+@pytest.mark.parametrize("overlap", [False, True])
+def test_step_on_more_units_than_announced(kept, act, overlap):
+    """The units beyond the announced number have no column among the kept ones' products: they are updated like pruned ones."""
+    d, n, N, k = 136, 520, 768, 301
+    g = torch.Generator(device=DEV).manual_seed(kept)
+    rand = lambda *s: torch.randn(*s, generator=g, device=DEV)
+    mod = api.FfnModule(rand(N, d).bfloat16(), rand(n, d) * 0.1, rand(d, n) * 0.1, dual_mode=act == "dual", overlap_k=k if overlap else 0,
+                        Wg_0=rand(n, d) * 0.1 if act == "gated" else None)
+    mod.sp_ffn_init()
+    mod.mask.zero_()
+    mod.mask[torch.randperm(n, generator=g, device=DEV)[:kept]] = 1
+    beyond = torch.nonzero(mod.mask).flatten()[k:]
+    z = mod.Z.clone()
+    mod._workspace(0).fill_(0x7f)
+    mod.sp_admm_step(api.AdmmParams(k_keep=k, rho=0.1, reselect_mask=False, skip_scores=True, dual_mode=act == "dual"))
+    assert mod.status.tolist()[:2] == [2, kept]      # SP_ERR_SHAPE, units kept
+    # z1 = 0 and a = phi(z) there; one product, one sum and one quotient of fp32
+    want = torch.where(z < 0, 0.0, z / 2) if act != "gated" else mod.Gate.square() * z / (mod.Gate.square() + 1)
+    assert float((mod.Z - want).abs()[:, beyond].max()) <= 4 * 2.0 ** -24 * float(z.abs().max())
+    assert torch.isfinite(mod.Z).all() and torch.isfinite(mod.W1).all()
