@@ -975,7 +975,7 @@ static sp_status admm_step_impl(const sp_ffn_module* m, sp_ffn_state* st, const 
       CU(cudaStreamWaitEvent(sa, side->fork, 0));
     }
     SPCHK(w1_rows(p.sb.idx, k));
-    CU(place_rows(st->mask, p.sb.idx, k, p.W1t, d, st->W1, d, n, d, sa));
+    CU(place_rows(st->mask, p.sb.idx, k, p.W1t, d, st->R1, st->G_X_inv, st->W1, d, n, d, sa));
     if (side) CU(cudaEventRecord(side->join, sa));
     joined = side == nullptr;
   } else {

@@ -631,10 +631,11 @@ cudaError_t mask_changed(const uint8_t* mask, const int32_t* perm, const int32_t
                          cudaStream_t stream);
 cudaError_t zero_pruned(const uint8_t* mask, int group, float* W_rows, int64_t r_rows, int64_t r_cols, int64_t r_ld,
                         float* W_cols, int64_t c_rows, int64_t c_cols, int64_t c_ld, cudaStream_t stream);
+// dst[idx[p], :] = src[p, :] for the k >= 1 listed rows (ascending), zero rows where the mask is zero; rows that it keeps beyond the list:
+// R[i, :] M (R [rows, cols], M [cols, cols])
+cudaError_t place_rows(const uint8_t* mask, const int32_t* idx, int64_t k, const float* src, int64_t lds, const float* R, const float* M,
+                       float* dst, int64_t ldd, int64_t rows, int64_t cols, cudaStream_t stream);
 // dst[i,:] = mask[i] ? src[i,:] : 0
-// dst[idx[p], :] = src[p, :] for the k kept rows, zero rows where the mask is zero
-cudaError_t place_rows(const uint8_t* mask, const int32_t* idx, int64_t k, const float* src, int64_t lds, float* dst, int64_t ldd,
-                       int64_t rows, int64_t cols, cudaStream_t stream);
 cudaError_t mask_rows_copy(const uint8_t* mask, const float* src, int64_t lds, float* dst, int64_t ldd, int64_t rows,
                            int64_t cols, cudaStream_t stream);
 

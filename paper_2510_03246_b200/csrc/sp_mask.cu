@@ -901,10 +901,12 @@ __global__ void __launch_bounds__(kStripThreads) mask_rows_copy_kernel(const uin
   });
 }
 
-// dst[idx[p], :] = src[p, :] for the k kept rows, zero rows elsewhere
+// dst[idx[p], :] = src[p, :] for the k listed rows, zero rows where the mask is zero.  Rows that a mask keeps beyond the list (its count
+// is reported elsewhere) are formed here, row by row: R[i, :] M.
 template <int W>
 __global__ void __launch_bounds__(kStripThreads) place_rows_kernel(const uint8_t* mask, const int32_t* idx, int64_t k, const float* src,
-                                                                   int64_t lds, float* dst, int64_t ldd, int64_t rows, int64_t cols) {
+                                                                   int64_t lds, const float* R, const float* M, float* dst, int64_t ldd,
+                                                                   int64_t rows, int64_t cols) {
   kernel_begin();
   for_strip<W>(rows, cols, [&](int64_t i, int64_t j, int) {
     if (!mask[i]) dst[i * ldd + j] = 0.f;
@@ -912,6 +914,15 @@ __global__ void __launch_bounds__(kStripThreads) place_rows_kernel(const uint8_t
       const int64_t r = idx[i];
       if (mask[r]) dst[r * ldd + j] = src[i * lds + j];     // (the list of an empty mask names a pruned row)
     }
+  });
+  // (behind the last listed row: as a rule a few pruned ones)
+  const int64_t first = (int64_t)idx[k - 1] + 1;
+  for_strip<W>(rows - first, cols, [&](int64_t t, int64_t j, int) {
+    const int64_t i = first + t;
+    if (!mask[i]) return;
+    double v = 0.0;
+    for (int64_t c = 0; c < cols; ++c) v += (double)R[i * cols + c] * (double)M[c * cols + j];
+    dst[i * ldd + j] = (float)v;
   });
 }
 
@@ -1615,13 +1626,13 @@ cudaError_t mask_rows_copy(const uint8_t* mask, const float* src, int64_t lds, f
   return cudaGetLastError();
 }
 
-cudaError_t place_rows(const uint8_t* mask, const int32_t* idx, int64_t k, const float* src, int64_t lds, float* dst, int64_t ldd,
-                       int64_t rows, int64_t cols, cudaStream_t stream) {
-  if (rows * cols == 0) return cudaSuccess;
+cudaError_t place_rows(const uint8_t* mask, const int32_t* idx, int64_t k, const float* src, int64_t lds, const float* R, const float* M,
+                       float* dst, int64_t ldd, int64_t rows, int64_t cols, cudaStream_t stream) {
+  if (rows * cols == 0 || k < 1) return cudaSuccess;
   ProfScope prof(PK_ELEMENTWISE, 0.0, 0.0, stream);
   count_launch();
   strip_launch(rows, cols, [&](auto w, dim3 grid, dim3 block) {
-    launch(place_rows_kernel<decltype(w)::value>, grid, block, 0, stream, mask, idx, k, src, lds, dst, ldd, rows, cols);
+    launch(place_rows_kernel<decltype(w)::value>, grid, block, 0, stream, mask, idx, k, src, lds, R, M, dst, ldd, rows, cols);
   });
   return cudaGetLastError();
 }

@@ -34,8 +34,8 @@ def test_refit_on_fewer_units_than_announced(units, group, k, kept, precise):
     assert torch.all(W[:, ~(cols | first)] == 0)
 
 
-@pytest.mark.parametrize("kept", [0, 100, 300])
-def test_step_on_fewer_units_than_announced(kept):
+@pytest.mark.parametrize("kept", [0, 100, 300, 301, 302, 520])
+def test_w1_of_a_mask_of_another_size(kept):
     """W1 is R1 (G_X + rho I)^-1 on the units that the mask keeps and zero elsewhere."""
     d, n, N, k = 136, 520, 768, 301
     g = torch.Generator(device=DEV).manual_seed(kept)
@@ -48,13 +48,14 @@ def test_step_on_fewer_units_than_announced(kept):
     mod._workspace(0).fill_(0x7f)
     mod.W1.fill_(7.0)
     mod.sp_admm_step(api.AdmmParams(k_keep=k, rho=0.1, reselect_mask=False, skip_scores=True))
-    assert mod.status.tolist()[:2] == [2, kept]      # SP_ERR_SHAPE, units kept
+    assert mod.status.tolist()[:2] == ([2, kept] if kept != k else [0, 0])      # SP_ERR_SHAPE, units kept
     G = G.tril() + G.tril(-1).T
-    ref = R1 @ torch.linalg.inv(G + 0.1 * G.diagonal().mean() * torch.eye(d, device=DEV, dtype=torch.float64))
+    inv = torch.linalg.inv(G + 0.1 * G.diagonal().mean() * torch.eye(d, device=DEV, dtype=torch.float64))
+    ref = R1 @ inv
     keep = mod.mask.bool()
     assert torch.all(mod.W1[~keep] == 0)
     # the inverse rounded to fp32, six part products without terms below 2^-23: a few roundings per term, at random over d terms
-    bound = 8 * d ** 0.5 * 2.0 ** -24 * (R1.abs() @ torch.linalg.inv(G + 0.1 * G.diagonal().mean() * torch.eye(d, device=DEV, dtype=torch.float64)).abs())
+    bound = 8 * d ** 0.5 * 2.0 ** -24 * (R1.abs() @ inv.abs())
     assert bool(((mod.W1.double() - ref).abs() <= bound)[keep].all())
 
 
