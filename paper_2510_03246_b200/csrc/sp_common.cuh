@@ -381,7 +381,7 @@ sp_status potrs_right_tc(float* X, int64_t m, int64_t n, int64_t ldx, const void
 //   batch > 1: that many systems, A and W a_bs elements apart, the other arrays one system's behind the other's (no lead).
 struct SolveOneBufs {
   void *P, *Y;
-  float* pre;         // 2 ceil(nn / kCholTcNB) blocks of kCholTcNB^2
+  float* pre;         // 2 ceil(nn / kCholTcNB) blocks of kCholTcNB^2, and behind those of all systems ceil(nn / kCholTcNB) times kCholTcNB
   uint32_t* flags;
 };
 // One launch against the launches per block column of sp_linalg_tc.cu (unknowns / right-hand sides, us): 128 / 128 41 -> 58, 256 / 256 78 ->

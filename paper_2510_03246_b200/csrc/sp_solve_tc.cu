@@ -49,7 +49,9 @@ constexpr uint32_t PRE_BYTES = TB * TB * 4;
 constexpr uint32_t PRE_AT = (uint32_t)(Diag::SMEM - Diag::BARS * 8);   // chain block: a tile's sum, behind DiagTiles' arrays
 constexpr uint32_t AREA = PRE_AT + PRE_BYTES > DATA ? PRE_AT + PRE_BYTES : DATA;
 constexpr uint32_t NBARS = 11;
-constexpr size_t SMEM = AREA + 1024 /*alignment*/ + (NBARS + Diag::BARS) * 8 + 4 * TB * sizeof(float) /*row maxima*/;
+// [4][128] floats: maxima of a tile's rows; chain block: the rows' factors of the tile that PRE_AT holds
+constexpr uint32_t ROW_MAX_AT = (AREA + (NBARS + Diag::BARS) * 8 + 15) / 16 * 16;
+constexpr size_t SMEM = ROW_MAX_AT + 4 * TB * sizeof(float) + 1024 /*alignment*/;
 static_assert(Diag::SMEM - Diag::BARS * 8 <= DATA, "the diagonal block's arrays lie over the operand slots");
 constexpr uint32_t TMEM_COLS = 4 * TB;                    // two pairs of accumulators in turn
 // about 16 seconds: a block may wait for others of its launch that have no room yet beside another stream's long kernels
@@ -69,6 +71,7 @@ struct SolveParams {
   int64_t ld_lead;
   int lead_k;
   float* pre;                  // [2 nblk][128][128]: what the chain block takes over of a column (see TASK_PRE)
+  float* pre_back;             // [nblk][128]: factors of the rows of the tile below a diagonal block (see scale_tiny_row)
   uint32_t* flags;
   int32_t* status;
   const int32_t* skip;
@@ -105,6 +108,27 @@ __device__ __forceinline__ bool epi_any(bool v) {
 // barrier, the flag may be set by a warp that is ahead, and the block's warps would end up at different barriers.)
 __device__ __forceinline__ bool given_up(volatile int* abort_flag) { return __syncthreads_or(*abort_flag) != 0; }
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 512;" ::: "memory"); }
+// Rows of tiny values are brought to the order of one by a power of two before they are split: below 2^-110 the low parts would be cut
+// off.  row_part_max: of a thread's 32 columns of a row; where that is tiny() in any thread of the epilogue, all of them call
+// scale_tiny_row (thread of row i, columns 32 g .. + 31): the factor that takes the row's product back.
+__device__ __forceinline__ bool tiny(float top) { return top > 0.f && top < 0x1p-80f; }
+__device__ __forceinline__ float row_part_max(const float (&v)[32]) {
+  float top = 0.f;
+#pragma unroll
+  for (int c = 0; c < 32; ++c) top = fmaxf(top, fabsf(v[c]));
+  return top;
+}
+__device__ __forceinline__ float scale_tiny_row(float (&v)[32], float top, float* row_max, int g, int i) {
+  row_max[g * kCholTcNB + i] = top;
+  epi_sync();
+#pragma unroll
+  for (int q = 0; q < 4; ++q) top = fmaxf(top, row_max[q * kCholTcNB + i]);
+  if (!tiny(top)) return 1.f;
+  const float up = top < 0x1p-104f ? 0x1p104f : 0x1p80f;
+#pragma unroll
+  for (int c = 0; c < 32; ++c) v[c] *= up;
+  return 1.f / up;
+}
 __device__ __forceinline__ void arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
@@ -259,7 +283,6 @@ __device__ __forceinline__ float ld_shared(uint32_t at) {
   return v;
 }
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-  mbar_expect_tx(bar, bytes);
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
                : "memory");
@@ -361,7 +384,7 @@ solve_tc_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
   const uint32_t xfull = bars + 8u * 8, aready = bars + 8u * 9;  // X(j, j) has landed; the left operand is written
   const uint32_t xfree = bars + 8u * 10;                         // chain: X(j, j) has left (barriers in this order there too)
   const uint32_t dbars = bars + 8u * NBARS;
-  float* const row_max = reinterpret_cast<float*>(data_ptr + AREA + (NBARS + Diag::BARS) * 8);   // [4][128]
+  float* const row_max = reinterpret_cast<float*>(data_ptr + ROW_MAX_AT);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   volatile int* abort_flag = &s_abort;
   if (threadIdx.x == 0) {
@@ -435,7 +458,9 @@ solve_tc_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
       const int row0 = system * p.rows;
       if (at.warp == 0 && more && at.lane == 0 && wait_flag(pre_j, abort_flag, p.budget)) {     // (its tile of L is done first)
         asm volatile("fence.proxy.async;" ::: "memory");
+        mbar_expect_tx(xfull_j, PRE_BYTES + TB * 4);
         bulk_load(at.data + PRE_AT, sums, PRE_BYTES, xfull_j);
+        bulk_load(at.data + ROW_MAX_AT, p.pre_back + (int64_t)(system * p.nblk + j) * TB, TB * 4, xfull_j);
       }
       __syncwarp();
       __syncthreads();                       // X is complete
@@ -497,6 +522,11 @@ solve_tc_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
         const uint32_t taddr_j = at.tmem + ((uint32_t)((at.warp & 3) * 32) << 16) + (uint32_t)(at.g * 32);
         float d[32];
         const bool ok = read_sum(tfull0, tempty0, par, taddr_j, at.lane, abort_flag, p.budget, [&](int c, float u) { d[c] = u; });
+        const float back = ld_shared(at.data + ROW_MAX_AT + 4u * (uint32_t)at.i);
+        if (back != 1.f) {
+#pragma unroll
+          for (int c = 0; c < 32; ++c) d[c] *= back;
+        }
         put_parts(at.ptr + SLOT + (at.g >> 1) * OPER, at.i, (at.g & 1) * 4, d);
         fence_async_smem();
         __syncwarp();
@@ -659,21 +689,8 @@ solve_tc_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
         }
       }
       if (tk.kind == TASK_T) {
-        // Rows of tiny values are brought to the order of one by a power of two: below 2^-110 the low parts would be cut off.
-        float top = 0.f, back = 1.f;
-#pragma unroll
-        for (int c = 0; c < 32; ++c) top = fmaxf(top, fabsf(s[c]));
-        if (epi_any(top > 0.f && top < 0x1p-80f)) {
-          row_max[g * TB + i] = top;
-          epi_sync();
-          top = fmaxf(fmaxf(row_max[i], row_max[TB + i]), fmaxf(row_max[2 * TB + i], row_max[3 * TB + i]));
-          if (top > 0.f && top < 0x1p-80f) {
-            const float up = top < 0x1p-104f ? 0x1p104f : 0x1p80f;
-            back = 1.f / up;
-#pragma unroll
-            for (int c = 0; c < 32; ++c) s[c] *= up;
-          }
-        }
+        const float top = row_part_max(s);
+        const float back = epi_any(tiny(top)) ? scale_tiny_row(s, top, row_max, g, i) : 1.f;
         uint8_t* const box = data_ptr + (g >> 1) * OPER;
         if (ok) {
           put_parts(box, i, (g & 1) * 4, s);
@@ -718,15 +735,26 @@ solve_tc_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
           }
         }
       } else {
-        // for the chain block
-        // (a diagonal block thread by thread, as it is read; the tile below one for a copy to shared memory)
+        // for the chain block (a diagonal block thread by thread, as it is read; the tile below one for a copy to shared memory, and what
+        // its rows were divided by: as a rule one, and known behind the barrier that the flag needs anyway)
         float* dst = p.pre + (int64_t)(2 * system * p.nblk + tk.pre) * (TB * TB);
+        const auto put = [&] {
 #pragma unroll
-        for (int c = 0; c < 32; c += 4) {
-          const int at = same ? (c / 4 * (EPI_WARPS * 32) + threadIdx.x - EPI0 * 32) * 4 : pre_at(i, g * 8 + c / 4);
-          *reinterpret_cast<float4*>(dst + at) = make_float4(s[c], s[c + 1], s[c + 2], s[c + 3]);
+          for (int c = 0; c < 32; c += 4) {
+            const int at = same ? (c / 4 * (EPI_WARPS * 32) + threadIdx.x - EPI0 * 32) * 4 : pre_at(i, g * 8 + c / 4);
+            *reinterpret_cast<float4*>(dst + at) = make_float4(s[c], s[c + 1], s[c + 2], s[c + 3]);
+          }
+        };
+        float* const back = p.pre_back + (int64_t)(system * p.nblk + tk.j) * TB + i;
+        put();
+        if (!same && g == 0) *back = 1.f;
+        const float top = row_part_max(s);
+        if (epi_any(!same && tiny(top))) {
+          const float f = scale_tiny_row(s, top, row_max, g, i);
+          put();
+          if (g == 0) *back = f;
+          epi_sync();
         }
-        epi_sync();
         if (threadIdx.x == EPI0 * 32 && *abort_flag == 0) publish(pre_flags + tk.pre);
       }
     }
@@ -783,6 +811,7 @@ sp_status solve_tc(const float* A, int64_t nn, int64_t m, int64_t lda, float* W,
   p.ld_lead = ld_lead;
   p.lead_k = (int)lead_k;
   p.pre = b.pre;
+  p.pre_back = b.pre + (size_t)batch * 2 * p.nblk * TB * TB;
   p.flags = b.flags;
   p.status = status_dev;
   p.skip = skip_flag();

@@ -50,6 +50,18 @@ def test_solution_on_the_kept_support_comes_with_the_factor(n, k):
     assert float((W - mod.W2).norm() / W.norm()) <= 10 * (1 + n / 0.1) * 2.0 ** -24
 
 
+@pytest.mark.parametrize("n,m", [(300, 40), (1024, 129), (1153, 64)])
+@pytest.mark.parametrize("scale", [-112, -116])
+def test_systems_of_tiny_entries(n, m, scale):
+    """G and R times 2^scale have the solution of G and R, with the same bound: no part of an operand is cut off."""
+    G, R = _system(n, m, n + m)
+    c = 2.0 ** scale
+    W = api.sp_ridge_solve(R * c, G * c, 1e-3 * c, rho_relative=False)
+    G64 = G.double().tril() + G.double().tril(-1).T + 1e-3 * torch.eye(n, device=DEV, dtype=torch.float64)
+    ref = torch.cholesky_solve(R.double().T, torch.linalg.cholesky(G64)).T
+    assert float((W.double() - ref).norm() / ref.norm()) <= max(10.0, n ** 0.5) * 34 * 2.0 ** -24
+
+
 @pytest.mark.parametrize("n,m,budget", [(1024, 300, 1), (2304, 128, 20000)])
 def test_waits_that_run_out_end_the_solve(n, m, budget):
     """With a budget of a few cycles ordinary waits run out (nothing is withheld): the solve reports SP_ERR_TIMEOUT and returns, and the
