@@ -117,16 +117,16 @@ struct SolveBufs {
   SolveOneBufs one;   // fp32 path, solves in one launch: P as above, and its small arrays
 };
 
-SolveBufs carve_solve(Carver& c, int64_t nmax, int64_t mmax, size_t tsize) {
+// in_step: solves inside a step (fp64: assisted, and either dimension may be the right-hand sides').
+SolveBufs carve_solve(Carver& c, int64_t nmax, int64_t mmax, size_t tsize, bool in_step = false) {
   SolveBufs b;
   b.rho = c.take<double>(4);
   b.idx = c.take<int32_t>((size_t)nmax);
   // the system matrix and, right behind its nn x nn elements, the right-hand sides (one [nn + m, nn] array)
-  // (fp64: and, for systems that are solved with the inverse of their factor, as many elements for that and the result)
   size_t elems = (size_t)(nmax + mmax) * nmax;
   if (tsize == 8) {
-    const size_t inv = (size_t)(nmax < kInverseMaxN ? nmax : kInverseMaxN);
-    elems = std::max(elems, 2 * inv * (inv + (size_t)std::max(nmax, mmax)));
+    elems = solve_f64_elems(nmax, mmax, in_step);
+    if (in_step) elems = std::max(elems, solve_f64_elems(mmax, nmax, true));
   }
   b.Gs = c.take_bytes(elems * tsize);
   b.dinv = c.take_bytes(dinv_elems(nmax) * tsize);
@@ -183,7 +183,7 @@ sp_status ridge_core(const float* R, int64_t ldr, const float* G, int64_t ldg, i
     }
   } else {
     CU(gather_cols<T>(R, ldr, idx, m, nn, Rs, nn, stream));
-    if (nn <= kInverseMaxN) {
+    if (inverse_f64(nn, m, assist != nullptr)) {
       T* X = Rs + (size_t)(m + nn) * nn;
       CU(solve_inverse_f64(Gs, nn, m, dinv, X, status, stream, assist));
       Rs = X;
@@ -306,8 +306,8 @@ AdmmPlan plan_admm(void* ws, int64_t d, int64_t n, int64_t N, int64_t chunk, int
   const size_t csz = p.bf16 ? 2 : 4;
   Carver c(ws);
   const int64_t nmax = n > d ? n : d;
-  p.sb = carve_solve(c, nmax, nmax == n ? d : n, p.tsize);
-  p.sbA = carve_solve(c, d, n, p.tsize);
+  p.sb = carve_solve(c, nmax, nmax == n ? d : n, p.tsize, true);
+  p.sbA = carve_solve(c, d, n, p.tsize, true);
   p.W1t = c.take<float>((size_t)n * d);
   p.W2t = c.take<float>((size_t)n * d);
   p.Qt = c.take<float>((size_t)n * d);
@@ -1093,7 +1093,7 @@ static sp_status admm_step_impl(const sp_ffn_module* m, sp_ffn_state* st, const 
       CU(load_spd<double>(p.Cf, d, d, gam, Gs, d, s));
       CU(transpose_convert<double>(p.W2cf, kp, d, k, Rs, d, s));
       const SolveAssist* assist = side ? &side->assist_main : nullptr;
-      if (d <= kInverseMaxN) {
+      if (inverse_f64(d, k, assist != nullptr)) {
         double* X = Rs + (size_t)(k + d) * d;
         CU(solve_inverse_f64(Gs, d, k, reinterpret_cast<double*>(p.sb.dinv), X, status_dev, s, assist));
         Rs = X;

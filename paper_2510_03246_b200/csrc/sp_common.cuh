@@ -315,6 +315,7 @@ bool gemm_tc_supported(int64_t M, int64_t N, int64_t K, TcOperand A, TcOperand B
 
 struct SolveAssist;
 // fp64 factorisation and solves (sp_linalg.cu), block columns of kCholNB.
+constexpr int kCholNB = 64;
 //   potrf_lower_f64: in-place lower Cholesky of the n x n matrix A (ld lda); the strict upper triangle and the diagonal
 //   blocks of the factor are not written; dinv: ceil(n / kCholNB) inverse diagonal blocks [kCholNB, kCholNB].
 //   m_extra > 0: A has m_extra more rows below row n, right-hand sides B of X L^T = B that ride along and hold X on
@@ -326,12 +327,26 @@ cudaError_t potrf_lower_f64(double* A, int64_t n, int64_t lda, double* dinv, int
 // rows (all dense, leading dimension n).
 cudaError_t solve_inverse_f64(double* A, int64_t n, int64_t m, double* dinv, double* W, int32_t* status_dev, cudaStream_t stream,
                               const SolveAssist* assist);
-// Systems of up to this many unknowns (the identity costs n^3 / 3 operations, which pay while the chain leaves the fp64 pipe idle).
-constexpr int64_t kInverseMaxN = 4096;
+// Which systems (n unknowns, m right-hand sides) are solved that way: more than one diagonal block (one has no chain: 64 / 256 33 us by the
+// sweep, 45 with the identity; 65 / 65 72 -> 60), up to 4096 unknowns (the identity costs n^3 / 3 operations, which pay while the chain
+// leaves the fp64 pipe idle).  Inside a step it runs beside the chain (assisted; fp32 mode, a step of 128 x 512 0.64 -> 0.56 ms, 768 x 3072
+// 5.8 -> 4.9, 1024 x 4096 10.0 -> 9.0).  On one stream its rows are the chain's own: for wide systems only with right-hand sides enough
+// that the sweep would cost more.  Sweep / identity, us: 1024 / 256 536 / 482, 2560 / 16 1780 / 1712, 3072 / 16 2264 / 2326, 3072 / 768 3024 /
+// 2830, 3584 / 448 3406 / 3503, 3584 / 896 4011 / 3849, 4096 / 1024 5136 / 5290, 4096 / 2048 6742 / 6440, 4096 / 16384 29889 / 22979.
+constexpr int64_t kInverseMaxN = 4096, kInverseAloneN = 3072;
+inline bool inverse_f64(int64_t n, int64_t m, bool assisted) {
+  return n > kCholNB && n <= kInverseMaxN && (assisted || 2 * m >= 3 * (n - kInverseAloneN));
+}
+// fp64 elements of a solve's system, right-hand sides, identity and result, for up to n unknowns and m right-hand sides
+inline size_t solve_f64_elems(int64_t n, int64_t m, bool assisted) {
+  const int64_t most = assisted ? kInverseMaxN : kInverseAloneN + 2 * m / 3;
+  const int64_t inv = n < most ? n : most < kInverseMaxN ? most : kInverseMaxN;
+  const size_t sweep = (size_t)(n + m) * n, inverse = inv > kCholNB ? 2 * (size_t)(inv + m) * inv : 0;
+  return sweep > inverse ? sweep : inverse;
+}
 // X[m,n] <- X L^-1 (backward sweep with the factor of potrf_lower_f64).
 cudaError_t potrs_backward_f64(double* X, int64_t m, int64_t n, int64_t ldx, const double* L, int64_t ldl,
                                const double* dinv, cudaStream_t stream, const SolveAssist* assist);
-constexpr int kCholNB = 64;
 
 // fp32 factorisation / solves with tensor-core trailing updates (sp_linalg_tc.cu).  Panels are kCholTcNB wide.
 //   dinv: ceil(n / kCholTcNB) blocks of 2 * kCholTcNB^2 floats (inverse diagonal blocks and their transposes)

@@ -48,6 +48,13 @@ def test_workspace_queries(lib):
     w32 = api.workspace_bytes(api.SP_WS_RIDGE_SOLVE, 64, 128, 0, 0, api.SP_F32)
     assert w64 >= 8 * 128 * 128 and w32 >= 4 * 128 * 128 + 6 * 128 * 128
     assert api.workspace_bytes(99, 1, 1, 1) == 0
+    # fp64 solves: the system and its right-hand sides, twice where the inverse of the factor is formed, and little else
+    for n, m, inverse in ((64, 4096, False), (1024, 256, True), (3072, 8, True), (4096, 16, False), (4096, 1024, False),
+                          (4096, 4096, True), (5000, 4096, False)):
+        elems = (n + m) * n * (2 if inverse else 1)
+        got = api.workspace_bytes(api.SP_WS_RIDGE_SOLVE, m, n, 0, 0, api.SP_F64)
+        smaller = 2 * (3072 + 2 * m // 3 + m) * (3072 + 2 * m // 3) if n > 3072 else 0     # a refit's system may be narrower
+        assert 8 * elems <= got <= 8 * max(elems, smaller) + 8 * 256 * (n + 256) + 65536, (n, m)
 
 
 def test_host_side_validation_without_gpu(lib):

@@ -105,6 +105,29 @@ def test_precise_ridge_solve_at_block_edges(n, m):
     assert torch.equal(got, again)      # no result depends on the order of the two streams
 
 
+@pytest.mark.parametrize("n,m,k", [(64, 200, 64), (65, 200, 64), (3073, 1, 3073), (3073, 2, 3073), (3400, 491, 3400), (3400, 492, 3400),
+                                   (3600, 400, 3300), (4097, 1600, 4096)])
+def test_precise_solves_by_sweep_and_by_inverse(n, m, k):
+    """Both sides of the lines between a backward sweep and the inverse of the factor; a refit narrower than the system whose
+    workspace it has (k units of n kept), right up to that workspace's end."""
+    api = _api()
+    G = _spd(n, n)
+    g = torch.Generator(device="cuda").manual_seed(m)
+    R = torch.randn(m, n, generator=g, device="cuda")
+    keep = torch.sort(torch.randperm(n, generator=g, device="cuda")[:k]).values
+    mask = torch.zeros(n, dtype=torch.uint8, device="cuda")
+    mask[keep] = 1
+    rho = 0.01 * float(G.double().diagonal().mean())
+    need = api.workspace_bytes(api.SP_WS_LINEAR_REFIT, m, n, 0, 0, api.SP_F64)
+    buf = torch.full((need + 4096,), 0x5a, dtype=torch.uint8, device="cuda")
+    got = api.sp_linear_refit(R, G, mask, k, rho, precise=True, ws=buf[:need])
+    H = G[keep][:, keep].double() + rho * torch.eye(k, device="cuda", dtype=torch.float64)
+    want = torch.linalg.solve(H, R[:, keep].double().T).T
+    # fp64 throughout (condition number below 1e5: 1e-10 of the largest entry), stored as fp32 (2^-24)
+    assert float((got[:, keep].double() - want).abs().max() / want.abs().max()) < 1.2e-7
+    assert torch.all(got[:, mask == 0] == 0) and torch.all(buf[need:] == 0x5a)
+
+
 @pytest.mark.parametrize("n,m", [(1, 3), (31, 40), (33, 8), (96, 129), (127, 64), (128, 200), (129, 7), (385, 96), (1000, 300)])
 def test_tensor_core_ridge_solve_at_block_edges(n, m):
     """Diagonal blocks of 128 eliminated in sub-blocks of 32, panels of a few rows."""
