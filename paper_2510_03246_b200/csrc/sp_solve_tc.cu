@@ -789,7 +789,8 @@ size_t solve_tc_flag_words(int64_t n, int64_t m) {
 
 sp_status solve_tc(const float* A, int64_t nn, int64_t m, int64_t lda, float* W, int64_t ldw, const SolveOneBufs& b,
                    float* lead, int64_t ld_lead, int64_t lead_k, int32_t* status_dev, cudaStream_t stream, int batch, int64_t a_bs) {
-  if (!solve_in_one(nn) || m < 1 || m > (1 << 24) || batch < 1 || batch > 65535 || (batch > 1 && lead != nullptr)) return SP_ERR_SHAPE;
+  // (2^27 right-hand sides have parts of 300 GB at least; up to there rows, tasks and flags are counted in 32 bits)
+  if (!solve_in_one(nn) || m < 1 || m > (1 << 27) || batch < 1 || batch > 65535 || (batch > 1 && lead != nullptr)) return SP_ERR_SHAPE;
   SolveParams p;
   memset(&p, 0, sizeof(p));
   p.A = A;
