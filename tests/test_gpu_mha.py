@@ -226,6 +226,9 @@ def test_mha_value_refit_matches_oracle(dtype, d, H, T, n_seq, chunk, causal):
     (64, 4, 1032, 2, 2, (0, 1, 3)),      # 2064 tokens in a chunk: the Gram products in two ranges, 16 tokens in the second
     (128, 16, 16, 5, 2, (1, 2, 7, 15)),  # batched systems, heads not in a row, a last chunk of one sequence
     (256, 2, 40, 3, 0, (1,)),            # one head, one sequence per chunk
+    # many systems in one launch, the last block of 128 partly filled: many thread blocks a system, two, and two with more blocks
+    # than SMs
+    (320, 5, 40, 3, 2, (0, 1, 3, 4)), (416, 52, 16, 6, 2, tuple(range(52))), (608, 76, 16, 6, 3, tuple(range(76))),
 ])
 def test_mha_value_refit_of_some_heads(d, H, T, n_seq, chunk, kept):
     """The kept heads' products in groups, packed from their places among all heads: against the oracle from the same P, Aattn, X."""
@@ -262,8 +265,8 @@ def test_mha_value_refit_argument_errors():
 
 @pytest.mark.parametrize("d,H", [(256, 4), (2560, 20)])
 def test_recoveries_of_wq_and_wk_are_those_of_each_by_itself(d, H):
-    """One factorisation for both, or (2560 wide, where both together are more right-hand sides than a backward sweep takes in a
-    fixed order) one for each: the same bits as a recovery by itself either way."""
+    """One solve for both, launches per block column (256 wide) or one launch: the same bits as a recovery by itself, since no sum of
+    a solve depends on the right-hand sides beside its own."""
     X, W = _case(torch.bfloat16, d, H, 16, 2)
     mod = api.MhaModule(X.to(DEV), *[w.to(DEV) for w in W], n_heads=H, T=16)
     mod.sp_mha_init(True)

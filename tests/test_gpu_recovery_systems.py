@@ -67,8 +67,7 @@ def test_products_of_the_factor_keep_all_bits_of_fp32(scores_only):
     mod.sp_ffn_init()
     mod.G_A.copy_(G)
     mod.R2.copy_(R)
-    # whole pairs are kept; with the kept channels in front the two of a pair are still two blocks of 128 apart (the block next to a
-    # diagonal one is updated on the CUDA cores)
+    # whole pairs are kept; with the kept channels in front the two of a pair are still two blocks of 128 apart
     keep = torch.arange(n, device=DEV) % 2 == 0
     mod.mask.copy_(keep)
     prm = api.AdmmParams(rho=2.0 ** -60, rho_relative=False, k_keep=n // 2, reselect_mask=False)

@@ -1,5 +1,5 @@
-"""Regularised solves in one launch: sizes around the tiles of 128, few and many right-hand sides, the widest system, against 64
-bits."""
+"""Regularised solves in one launch (257 to 12287 unknowns; sizes below are the other form's, at the line between them): sizes around the
+tiles of 128, few and many right-hand sides, columns in groups of one, two and four, the widest system, against 64 bits."""
 import pytest
 import torch
 
@@ -17,7 +17,7 @@ def _system(n, m, seed):
 
 
 @pytest.mark.parametrize("n,m", [(1, 1), (256, 129), (257, 1), (383, 128), (640, 127), (767, 300), (1024, 129), (1153, 130), (2304, 40),
-                                 (12287, 3)])
+                                 (5100, 300), (5340, 129), (7680, 300), (8069, 513), (12287, 3)])
 def test_solve_around_the_tiles(n, m):
     G, R = _system(n, m, n + m)
     status = torch.zeros(4, dtype=torch.int32, device=DEV)
@@ -30,7 +30,7 @@ def test_solve_around_the_tiles(n, m):
     assert torch.equal(W, api.sp_ridge_solve(R, G, 1e-3, rho_relative=False))       # a fixed order, whatever the timing
 
 
-@pytest.mark.parametrize("n,k", [(256, 128), (264, 64), (600, 128), (768, 385), (1160, 577)])
+@pytest.mark.parametrize("n,k", [(256, 128), (264, 64), (600, 128), (768, 385), (1160, 577), (5240, 1901), (7928, 3137)])
 def test_solution_on_the_kept_support_comes_with_the_factor(n, k):
     """The second of two steps whose mask stays takes the restricted solution from the unrestricted solve: the same as the solve of
     the restricted system by itself."""
