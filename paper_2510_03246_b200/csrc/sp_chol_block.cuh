@@ -429,8 +429,9 @@ struct DiagTiles {
     return ((col / SB) * SB + row % SB) * P + (row / SB) * SB + col % SB;
   }
 
-  // t: the thread.  The block comes from A, or (STAGED) sits in sm as staged_at() says: complete, that is zero above the diagonal and an identity
-  // beyond nb.  bars: BARS barriers of one arrival, parity: their phase (a full block completes one of each that is waited for).
+  // t: the thread.  The block comes from A, or (STAGED) sits in sm as staged_at() says: complete, that is zero above the diagonal
+  // and an identity beyond nb.  bars: BARS barriers of one arrival, parity: their phase (a full block completes one of each that is
+  // waited for).
   template <bool STAGED, typename Out>
   static __device__ __forceinline__ void eliminate(int t, float* sm, uint32_t bars, uint32_t parity, const float* A, int64_t lda, int nb,
                                                    const Out& out, int64_t row0, int32_t* status) {

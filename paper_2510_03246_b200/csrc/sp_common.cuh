@@ -109,18 +109,18 @@ struct OverlapScope {
   ~OverlapScope() { overlap_flag() = saved; }
   OverlapScope(const OverlapScope&) = delete;
 };
-// Weight phase of an ADMM step (and the cached input inverse): modules up to this width.  (Measured with recoveries by launches per block
-// column; most of them are one launch now.)  Its gain falls with the width, whatever the
-// token count: 768 x 3072 on 32768 tokens 3.09 -> 2.88 ms, 1096 x 4376 on 65536 tokens 7.40 -> 7.06, 1280 x 5120 on 8192 tokens
-// 4.78 -> 4.62, 2048 x 8192 on 32768 tokens 14.30 -> 14.06, 3072 x 9216 and 4096 x 11008 less than their runs differ.  Wider
-// modules keep plain launches.
+// Weight phase of an ADMM step (and the cached input inverse): modules up to this width.  Attribute off / on, ms a step: 768 x 3072 on 2048
+// tokens 1.320 / 1.265, on 32768 tokens 2.014 / 1.999, 1096 x 4376 on 9973 tokens 2.535 / 2.508, on 65536 tokens equal.  Wider
+// modules keep plain launches: with recoveries by launches per block column 2048 x 8192 on 32768 tokens gained 1.7 % and 3072 x 9216 less
+// than its runs differ; most recoveries are one launch now, and the line was not measured again.
 constexpr int64_t kOverlapMaxN = 4608;
 // Token pass of such a step: chunks of up to this many entries of Z.  Attribute off / on: 6.3 M entries 2.14 / 2.11 ms a step, 12.6 M
 // 2.20 / 2.17, 25 and 33 M equal, 38 M 2.38 / 2.40, 50 M 2.48 / 2.52, 101 M in eight chunks 9.4 / 10.7.
 constexpr int64_t kOverlapMaxChunk = int64_t(1) << 25;
-// Recoveries by themselves (sp_ridge_solve, sp_linear_refit): matrices up to this width, of which a refit solves a part.  On
-// this side 1.05 (1024 unknowns, 2048 right-hand sides: 0.401 -> 0.382 ms) to 1.17 (384 of 768: 0.155 -> 0.132).  Wider ones keep
-// plain launches; that is not a measured line: they ran with the attribute in the passes among which one stood still.
+// Recoveries by themselves (sp_ridge_solve, sp_linear_refit): matrices up to this width, of which a refit solves a part.  Attribute
+// off / on, us: 128 unknowns, 128 right-hand sides 49 / 36, 256 / 256 92 / 77, 128 of 256 62 / 42, 384 of 768 132 / 119, 768 / 768 196 / 192,
+// 1024 / 2048 254 / 248.  Wider ones keep plain launches; that is not a measured line: they ran with the attribute in the passes among
+// which one stood still.
 constexpr int64_t kOverlapMaxSolve = 1024;
 inline bool may_overlap_launches(cudaStream_t stream) {
   if (!overlap_flag()) return false;
@@ -399,14 +399,16 @@ struct SolveOneBufs {
   float* pre;         // 2 ceil(nn / kCholTcNB) blocks of kCholTcNB^2, and behind those of all systems ceil(nn / kCholTcNB) times kCholTcNB
   uint32_t* flags;
 };
-// One launch against the launches per block column of sp_linalg_tc.cu (unknowns / right-hand sides, us): 128 / 128 41 -> 58, 256 / 256 78 ->
-// 87, 257 / 100 156 -> 103, 384 / 768 129 -> 115, 768 / 768 261 -> 194, 1024 / 2048 372 -> 248, 3072 / 768 1164 -> 716, 4096 / 3302
-// 2306 -> 1237, 8192 / 2048 6022 -> 4262; 5734 / 7168 13319 -> 4310 and 9216 / 3072 8974 -> 6908 when the chain was 20 % slower; with
-// two levels of blocks 12288 / 4096 14735 -> 16072.
+// Launches per block column (sp_linalg_tc.cu) against one launch, unknowns / right-hand sides, us: 128 / 128 41 -> 59, 256 / 256 78 -> 86,
+// 257 / 100 154 -> 104, 384 / 768 129 -> 116, 768 / 768 265 -> 194, 1024 / 2048 374 -> 250, 2048 / 4096 1036 -> 587, 3072 / 768 1183 -> 728,
+// 4096 / 3302 2312 -> 1270, 5734 / 7168 13410 -> 3920, 8192 / 2048 6055 -> 3990, 9216 / 3072 8970 -> 6230; with two levels of blocks
+// 12288 / 4096 14740 -> 14510.
 constexpr int64_t kSolveOneMinN = 256, kSolveOneMaxN = kOuterMinN - 1;
-// A step's recoveries: modules up to this width.  The sign select of the z-update turns differences of rounding into differences of
-// the recovered weights; the recoveries of 7168 x 28672 (8192 tokens, five iterations) by the other form's roundings move W1 by
-// 1.3 %, as far as both are from 64 bits (1.5 %).  4096 x 16384 on 4096 tokens: 0.8 %.
+// A step's recoveries: modules up to this width.  Not for speed and not for accuracy: the sign select of the z-update turns differences of
+// rounding into differences of the recovered weights, and beyond it a step by this form differs from one by the other form's roundings by
+// about a percent of W1, the size of its distance from 64 bits, which is the same for both.  n x n / 4 on 8192 tokens, 20 % kept, five
+// iterations: W1 moves by 0.83 / 0.88 / 0.96 / 1.03 % for n = 18432 / 20480 / 24576 / 28672 (16384 on 4096 tokens: 0.8), is
+// 1.25 / 1.30 / 1.39 / 1.45 % from 64 bits either way (W2: 0.48 .. 0.58 and 0.95 .. 1.03 %), and a step takes 46.2 / 59.2 / 97.6 / 149.0 against 43.4 / 57.1 / 95.4 / 143.1 ms.
 constexpr int64_t kSolveOneModule = 16384;
 inline bool solve_in_one(int64_t n) { return n > kSolveOneMinN && n <= kSolveOneMaxN; }
 size_t solve_tc_flag_words(int64_t n, int64_t m);

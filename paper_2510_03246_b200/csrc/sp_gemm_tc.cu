@@ -25,8 +25,8 @@
 // Every wait of a role for copies, for the tensor core or for another role is bounded by a clock budget; on expiry the CTA
 // records SP_ERR_TIMEOUT and leaves its loops, and both CTAs still meet at the final cluster barrier before tensor memory is
 // freed.  Not bounded, since what they wait for cannot stay away: the two cluster barriers (the CTAs of a pair start together
-// and both reach them on every path), the allocation of tensor memory (the shared memory of a CTA keeps every other CTA of
-// this kernel off its SM, and no other kernel allocates any), and the wait for the kernels before this one.
+// and both reach them on every path), the allocation of tensor memory (the shared memory of a CTA, 225 KB here and 208 KB in
+// solve_tc_kernel, keeps every other CTA that allocates any off its SM), and the wait for the kernels before this one.
 #include <math.h>
 #include <string.h>
 

@@ -17,8 +17,8 @@
 // What bounds it: up to about 6000 unknowns the chain, 28 us per 128 unknowns (elimination 16, X and the tile below it into operand
 // form 2, their product 2.2, its result into operand form 1, the diagonal block's update 2.2; as one task per diagonal block, handed on
 // through memory, 36); above, the loads of the products (192 KB per two tiles' product; 3.8 us at 8192 unknowns, where the tensor core
-// takes 1.6.  Four slots of half the depth, with rows of 64 bytes, are slower: 3.96 -> 4.44 ms).  3072 unknowns and 768 right-hand sides: 1164 us as launches per block column, 1015 with a task per
-// diagonal block, 716.
+// takes 1.6.  Four slots of half the depth, with rows of 64 bytes, are slower: 3.96 -> 4.44 ms).  3072 unknowns and 768 right-hand
+// sides: 1183 us as launches per block column, 1015 with a task per diagonal block, 728.
 //
 // Tasks are taken by a counter in an order in which every task comes after those it reads (the chain, first, runs beside them).  A block
 // that waits therefore waits for a task that a running block has: two resident blocks make progress, beside whatever else runs on
@@ -63,8 +63,7 @@ struct SolveParams {
   const float* A;              // [nn + m, nn] fp32: lower triangle of the system, right-hand sides below
   int64_t lda;
   int nn, m, nblk, mb, group;
-  __nv_bfloat16* P;
-  int64_t ldp;                 // 3 np
+  __nv_bfloat16* P;            // pitch 3 np
   float* W;                    // [m, nn], may be the right-hand sides' own place
   int64_t ldw;
   float* lead;                 // optional [m, .]: the solution of the leading lead_k x lead_k system
@@ -206,7 +205,8 @@ __device__ __forceinline__ void mma_by_x(uint32_t d, uint32_t a, uint32_t b) {
   const uint64_t bd = make_smem_desc(b, false, OPER);
 #pragma unroll 1
   for (int k = 0; k < 8; ++k)
-    mma_slice(d, make_smem_desc(a + (k >> 2) * OPER + (k & 3) * 32, true, 0), bd + k * (16 * 128 >> 4), instr_desc(false), k > 0 ? 1u : 0u);
+    mma_slice(d, make_smem_desc(a + (k >> 2) * OPER + (k & 3) * 32, true, 0), bd + k * (16 * 128 >> 4), instr_desc(false),
+              k > 0 ? 1u : 0u);
 }
 // half h (64 of K) of the product of two tiles
 __device__ __forceinline__ void mma_half(uint32_t d, uint32_t a, uint32_t b, int h) {
@@ -287,13 +287,16 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
                ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
                : "memory");
 }
-// A thread's place: of the epilogue's threads (warps from EPI0 on) row i, columns 32 g .. + 31 of a tile.  Volatile: formed where it is called.
+// (a call of its own: see the chain)
 __device__ __noinline__ void eliminate_block(uint32_t off, uint32_t bars, int j, int nb, int32_t* status) {
   extern __shared__ uint8_t smem_raw[];
   int t;
   asm volatile("mov.u32 %0, %%tid.x;" : "=r"(t));
-  Diag::eliminate<true>(t, reinterpret_cast<float*>(smem_raw + off), bars, (uint32_t)j & 1u, nullptr, 0, nb, NoOut{}, (int64_t)j * TB, status);
+  Diag::eliminate<true>(t, reinterpret_cast<float*>(smem_raw + off), bars, (uint32_t)j & 1u, nullptr, 0, nb, NoOut{}, (int64_t)j * TB,
+                        status);
 }
+// A thread's place: of the epilogue's threads (warps from EPI0 on) row i, columns 32 g .. + 31 of a tile.  Volatile: formed where it is
+// called.
 struct Place {
   int warp, lane, g, i;
   uint32_t data, tmem;
@@ -446,7 +449,8 @@ solve_tc_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
     }
     for (int j = 0; j < p.nblk; ++j) {
       if (given_up(abort_flag)) break;
-      eliminate_block(at.data - smem_u32(smem_raw), at.data + AREA + 8u * NBARS, j, p.nn - j * TB < TB ? p.nn - j * TB : TB, p.status);
+      const int nb = p.nn - j * TB < TB ? p.nn - j * TB : TB;
+      eliminate_block(at.data - smem_u32(smem_raw), at.data + AREA + 8u * NBARS, j, nb, p.status);
       at = place(smem_raw, &s_tmem);
       const bool more = j + 1 < p.nblk;
       const uint32_t par = (uint32_t)j & 1u, bars_j = at.data + AREA;
@@ -805,7 +809,6 @@ sp_status solve_tc(const float* A, int64_t nn, int64_t m, int64_t lda, float* W,
   p.group = p.nblk >= 60 ? 4 : p.nblk >= 40 ? 2 : 1;
   const int64_t np = (int64_t)p.nblk * TB, rows = np + (int64_t)p.mb * TB;
   p.P = reinterpret_cast<__nv_bfloat16*>(b.P);
-  p.ldp = 3 * np;
   p.W = W;
   p.ldw = ldw;
   p.lead = lead;
@@ -835,7 +838,8 @@ sp_status solve_tc(const float* A, int64_t nn, int64_t m, int64_t lda, float* W,
   // (a system has two blocks at least: the chain waits for sums of the others)
   const int64_t tasks = (int64_t)p.nblk * (p.nblk + 2 * p.mb), share = sm_count() / batch, blocks = share > 2 ? share : 2;
   count_launch();
-  launch(batch > 1 ? solve_tc_kernel<true> : solve_tc_kernel<false>, dim3((unsigned)(tasks < blocks ? tasks : blocks), (unsigned)batch), THREADS, SMEM, stream, tmP, tmY, p);
+  launch(batch > 1 ? solve_tc_kernel<true> : solve_tc_kernel<false>, dim3((unsigned)(tasks < blocks ? tasks : blocks), (unsigned)batch),
+         THREADS, SMEM, stream, tmP, tmY, p);
   return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ERR_CUDA;
 }
 
