@@ -908,6 +908,7 @@ __global__ void __launch_bounds__(kStripThreads) place_rows_kernel(const uint8_t
                                                                    int64_t lds, const float* R, const float* M, float* dst, int64_t ldd,
                                                                    int64_t rows, int64_t cols) {
   kernel_begin();
+  const int64_t first = (int64_t)idx[k - 1] + 1;            // (read ahead of the stores)
   for_strip<W>(rows, cols, [&](int64_t i, int64_t j, int) {
     if (!mask[i]) dst[i * ldd + j] = 0.f;
     if (i < k) {
@@ -916,14 +917,14 @@ __global__ void __launch_bounds__(kStripThreads) place_rows_kernel(const uint8_t
     }
   });
   // (behind the last listed row: as a rule a few pruned ones)
-  const int64_t first = (int64_t)idx[k - 1] + 1;
-  for_strip<W>(rows - first, cols, [&](int64_t t, int64_t j, int) {
-    const int64_t i = first + t;
-    if (!mask[i]) return;
-    double v = 0.0;
-    for (int64_t c = 0; c < cols; ++c) v += (double)R[i * cols + c] * (double)M[c * cols + j];
-    dst[i * ldd + j] = (float)v;
-  });
+  for (int64_t i = first + strip_row<W>(); i < rows; i += strip_rows<W>()) {
+    if (!mask[i]) continue;
+    for (int64_t j = strip_col<W>(), q = 0; q < kStripPer && j < cols; ++q, j += strip_width<W>()) {
+      double v = 0.0;
+      for (int64_t c = 0; c < cols; ++c) v += (double)R[i * cols + c] * (double)M[c * cols + j];
+      dst[i * ldd + j] = (float)v;
+    }
+  }
 }
 
 inline int grid_for(int64_t total, int threads) {
