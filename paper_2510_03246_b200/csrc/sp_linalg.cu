@@ -31,7 +31,9 @@ inline OutOperand out(double* p, int64_t ld) { return OutOperand{p, SP_F64, ld};
 // A step's chain is diagonal block -> panel -> update of the next block column ("near"); the rest of the trailing update
 // ("far") runs on the assisting stream and is only waited for by the near update of the next step, which writes the
 // first of its columns.  The rows below the matrix (right-hand sides, identity) are no part of the chain: they follow on a third
-// stream, a panel and an update a step.
+// stream, a panel and an update a step, behind the near update.  (Behind the panel, like the far update, their blocks and the near update's
+// compete for the SMs, and which of the streams goes first differs from process to process: two fp32-mode iterations of 768 x 3072 14.42 ms
+// in one half of the processes, 15.56 in the other, 50 instead of 39 us for each of the first blocks of the 3072-wide system; now 14.63 in all.)
 cudaError_t potrf_lower_f64(double* A, int64_t n, int64_t lda, double* dinv, int32_t* status_dev, cudaStream_t stream,
                             const SolveAssist* assist, int64_t m_extra, bool identity) {
   static PerDeviceOnce attr_once;
@@ -71,23 +73,31 @@ cudaError_t potrf_lower_f64(double* A, int64_t n, int64_t lda, double* dinv, int
                         op(A22, lda, 1), out(A22, lda), true, true, stream));
       continue;
     }
-    const int64_t wn = (assist && rem > NB) ? NB : rem;      // columns of the near update
-    if (wn < rem || apart) SP_CU(cudaEventRecord(assist->panel_done, stream));
-    if (apart) {
+    const auto rows_below = [&]() -> cudaError_t {
       cudaStream_t sx = assist->far_stream;
       double* E = A + n * lda + k0;
-      SP_CU(cudaStreamWaitEvent(sx, assist->panel_done, 0));
+      SP_CU(cudaEventRecord(assist->near_done, stream));
+      SP_CU(cudaStreamWaitEvent(sx, assist->near_done, 0));
       SP_CU(gemm_simt(extra, nb, nb, 1.0, op(E, lda, 1), op(dk, 1, NB), 0.0, op(E, lda, 1), out(E, lda), false, true, sx));
       if (rem > 0)
         SP_CU(gemm_simt(extra, rem, nb, -1.0, op(E, lda, 1), op(A21, 1, lda), 1.0, op(E + nb, lda, 1), out(E + nb, lda), false,
                         true, sx));
+      return cudaSuccess;
+    };
+    if (rem <= 0) {
+      if (apart) SP_CU(rows_below());
+      break;
     }
-    if (rem <= 0) break;
+    const int64_t wn = (assist && rem > NB) ? NB : rem;      // columns of the near update
     double* A22 = A21 + nb;
-    if (wn < rem) SP_CU(cudaStreamWaitEvent(assist->stream, assist->panel_done, 0));
+    if (wn < rem) {
+      SP_CU(cudaEventRecord(assist->panel_done, stream));
+      SP_CU(cudaStreamWaitEvent(assist->stream, assist->panel_done, 0));
+    }
     if (last >= 0) SP_CU(cudaStreamWaitEvent(stream, assist->rest_done[last], 0));
     SP_CU(gemm_simt(rows, wn, nb, -1.0, op(A21, lda, 1), op(A21, 1, lda), 1.0, op(A22, lda, 1), out(A22, lda), true,
                     true, stream));
+    if (apart) SP_CU(rows_below());
     last = -1;
     if (wn < rem) {
       double* L2 = A21 + wn * lda;
