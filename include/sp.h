@@ -494,7 +494,8 @@ size_t sp_mha_value_refit_workspace_bytes(int64_t d, int64_t n_heads, int64_t T,
  *                    rho_eff as in sp_admm_params.  G is read from its lower triangle and left unchanged.
  * sp_linear_refit  — recovery on a kept support of column groups: W[:, S] = R[:, S](G[S,S] + rho_eff I)^-1,
  *                    other columns zero (Algorithm 2, "importance + recovery solver"; used for W2 and for W_O heads).
- *                    mask: u8 [n_units] with exactly k_keep ones (k_keep is a host value).  The ridge is that of the
+ *                    mask: u8 [n_units] with exactly k_keep ones (k_keep is a host value; another number of ones is not
+ *                    noticed, and W is then no solution, but nothing is accessed out of range).  The ridge is that of the
  *                    FULL system: rho_eff = rho * trace(G)/dim(G) when rho_relative != 0 (computed on the device),
  *                    else rho.
  * sp_gemm          — C[M,N] = alpha * opA(A) opB(B) + beta * C, opX(X) = X or X^T; test and utility entry.
