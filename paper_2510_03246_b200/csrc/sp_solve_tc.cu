@@ -57,7 +57,7 @@ constexpr uint32_t TMEM_COLS = 4 * TB;                    // two pairs of accumu
 // about 16 seconds: a block may wait for others of its launch that have no room yet beside another stream's long kernels
 constexpr long long WAIT_BUDGET = 32000000000LL;
 constexpr long long DRAIN = 200000000LL;
-constexpr int kFlags0 = 32;                               // flags[0]: the task counter
+constexpr int kFlags0 = 32;                               // flags[0]: the task counter; [1] of the first system: blocks that have come
 
 struct SolveParams {
   const float* A;              // [nn + m, nn] fp32: lower triangle of the system, right-hand sides below
@@ -375,8 +375,8 @@ solve_tc_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
     if (*p.skip != 0) return;
   }
   extern __shared__ uint8_t smem_raw[];
-  const int system = BATCH ? (int)blockIdx.y : 0;
   __shared__ uint32_t s_tmem;
+  __shared__ volatile int s_system;
   __shared__ int s_abort, s_ticket[2];
   const uint32_t raw = smem_u32(smem_raw), data = (raw + 1023u) & ~1023u, bars = data + AREA;
   uint8_t* const data_ptr = smem_raw + (data - raw);
@@ -416,7 +416,14 @@ solve_tc_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
   const uint32_t tmem = s_tmem;
   wait_for_predecessors();
 
-  uint32_t* const ticket_of = p.flags + (int64_t)system * p.flag_words;
+  // The system, in the order in which blocks come, which need not be that of their numbers: all blocks of a system are there before the
+  // next one's first, so two running blocks are enough here too.  (In shared memory: registers are short.)
+  if constexpr (BATCH) {
+    if (threadIdx.x == 0) s_system = (int)(atomicAdd(p.flags + 1, 1u) / gridDim.x);
+    __syncthreads();
+  }
+  const auto system = [&] { return BATCH ? (int)s_system : 0; };
+  uint32_t* const ticket_of = p.flags + (int64_t)system() * p.flag_words;
   uint32_t* const flags = ticket_of + kFlags0;
   uint32_t* const pre_flags = flags + (int64_t)p.nblk * (p.nblk + p.mb);
   const int total = p.nblk * (p.nblk + 2 * p.mb), np = p.nblk * TB;
@@ -443,7 +450,7 @@ solve_tc_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
 #pragma unroll
       for (int c = 0; c < 32; ++c) {
         const int col = at.g * 32 + c;
-        v[c] = at.i < p.nn && col <= at.i && col < p.nn ? p.A[(int64_t)system * p.a_bs + (int64_t)at.i * p.lda + col] : 0.f;
+        v[c] = at.i < p.nn && col <= at.i && col < p.nn ? p.A[(int64_t)system() * p.a_bs + (int64_t)at.i * p.lda + col] : 0.f;
       }
       stage_block(at, v, p.nn < TB ? p.nn : TB);
     }
@@ -456,15 +463,15 @@ solve_tc_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
       const uint32_t par = (uint32_t)j & 1u, bars_j = at.data + AREA;
       const uint32_t tfull0 = bars_j + 8u * 4, tempty0 = bars_j + 8u * 6, xfull_j = bars_j + 8u * 8, aready_j = bars_j + 8u * 9,
                      xfree_j = bars_j + 8u * 10;
-      uint32_t* const flags_j = p.flags + (int64_t)system * p.flag_words + kFlags0;
+      uint32_t* const flags_j = p.flags + (int64_t)system() * p.flag_words + kFlags0;
       uint32_t* const pre_j = flags_j + (int64_t)p.nblk * (p.nblk + p.mb) + 2 * j;
-      const float* const sums = p.pre + (int64_t)(2 * (system * p.nblk + j)) * (TB * TB);
-      const int row0 = system * p.rows;
+      const float* const sums = p.pre + (int64_t)(2 * (system() * p.nblk + j)) * (TB * TB);
+      const int row0 = system() * p.rows;
       if (at.warp == 0 && more && at.lane == 0 && wait_flag(pre_j, abort_flag, p.budget)) {     // (its tile of L is done first)
         asm volatile("fence.proxy.async;" ::: "memory");
         mbar_expect_tx(xfull_j, PRE_BYTES + TB * 4);
         bulk_load(at.data + PRE_AT, sums, PRE_BYTES, xfull_j);
-        bulk_load(at.data + ROW_MAX_AT, p.pre_back + (int64_t)(system * p.nblk + j) * TB, TB * 4, xfull_j);
+        bulk_load(at.data + ROW_MAX_AT, p.pre_back + (int64_t)(system() * p.nblk + j) * TB, TB * 4, xfull_j);
       }
       __syncwarp();
       __syncthreads();                       // X is complete
@@ -562,7 +569,7 @@ solve_tc_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
     const int masked = tk.lead >= 0 ? tk.lead - tk.k0 : -1;       // the chunk that reads the masked copy
     auto k_of = [&](int q) { return tk.k0 + (masked >= 0 && q > masked ? q - 1 : q); };
     const bool same = tk.R == tk.j;      // both operands are the same tiles
-    const int row0 = system * p.rows;
+    const int row0 = system() * p.rows;
     bool ok = true;
 
     if (warp == 0) {
@@ -667,7 +674,7 @@ solve_tc_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
         const int64_t row = tk.R < p.nblk ? (int64_t)tk.R * TB + i : (int64_t)p.nn + (int64_t)(tk.R - p.nblk) * TB + i;
         const bool have = tk.kind != TASK_W && tk.R >= tk.j &&
                           (tk.R < p.nblk ? row < p.nn : row < (int64_t)p.nn + p.m);
-        const float* src = p.A + (int64_t)system * p.a_bs + row * p.lda + col0;
+        const float* src = p.A + (int64_t)system() * p.a_bs + row * p.lda + col0;
         const int n_col = have ? (p.nn - col0 < 32 ? p.nn - col0 : 32) : 0;
         if (n_col == 32 && p.lda % 4 == 0) {
 #pragma unroll
@@ -727,7 +734,7 @@ solve_tc_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
       } else if (tk.kind == TASK_W) {
         const int64_t row = (int64_t)(tk.R - p.nblk) * TB + i;
         if (ok && row < p.m) {
-          float* dst = p.W + (int64_t)system * p.a_bs + row * p.ldw + col0;
+          float* dst = p.W + (int64_t)system() * p.a_bs + row * p.ldw + col0;
           if (col0 + 32 <= p.nn && p.ldw % 4 == 0) {
 #pragma unroll
             for (int c = 0; c < 32; c += 4)
@@ -741,7 +748,7 @@ solve_tc_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
       } else {
         // for the chain block (a diagonal block thread by thread, as it is read; the tile below one for a copy to shared memory, and what
         // its rows were divided by: as a rule one, and known behind the barrier that the flag needs anyway)
-        float* dst = p.pre + (int64_t)(2 * system * p.nblk + tk.pre) * (TB * TB);
+        float* dst = p.pre + (int64_t)(2 * system() * p.nblk + tk.pre) * (TB * TB);
         const auto put = [&] {
 #pragma unroll
           for (int c = 0; c < 32; c += 4) {
@@ -749,7 +756,7 @@ solve_tc_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__
             *reinterpret_cast<float4*>(dst + at) = make_float4(s[c], s[c + 1], s[c + 2], s[c + 3]);
           }
         };
-        float* const back = p.pre_back + (int64_t)(system * p.nblk + tk.j) * TB + i;
+        float* const back = p.pre_back + (int64_t)(system() * p.nblk + tk.j) * TB + i;
         put();
         if (!same && g == 0) *back = 1.f;
         const float top = row_part_max(s);
